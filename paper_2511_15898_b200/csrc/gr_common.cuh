@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <stdint.h>
 #include "gr.h"
 
@@ -52,6 +53,38 @@ template <class T> using RawPtr = T*;       // (an alias, so that "GR_PTR(double
 #define GR_CHECK_FLAG (nullptr)
 #define GR_CHECK_FLAG_INIT do { } while (0)
 #define GR_CHECK_VALUE (0)
+#endif
+
+// Vector loads and stores through these pointers (the address is aligned to the vector).  The bounds-checked build takes
+// the elements one by one, each checked.
+#ifdef GR_CHECK
+template <class P> __device__ inline float4 ld_f4(const P& p) { return make_float4(p[0], p[1], p[2], p[3]); }
+template <class P> __device__ inline float2 ld_f2(const P& p) { return make_float2(p[0], p[1]); }
+template <class P> __device__ inline double2 ld_d2(const P& p) { return make_double2(p[0], p[1]); }
+template <class P> __device__ inline uint2 ld_u2(const P& p) { return make_uint2(p[0], p[1]); }
+template <class P> __device__ inline void st_f4(const P& p, float4 v) { p[0] = v.x; p[1] = v.y; p[2] = v.z; p[3] = v.w; }
+template <class P> __device__ inline void st_f2(const P& p, float2 v) { p[0] = v.x; p[1] = v.y; }
+template <class P> __device__ inline void st_d2(const P& p, double2 v) { p[0] = v.x; p[1] = v.y; }
+template <class P> __device__ inline uint4 ld_h8(const P& p) {
+    uint32_t w[4];
+    for (int z = 0; z < 4; z++) w[z] = (uint32_t)__half_as_ushort(p[2 * z]) | ((uint32_t)__half_as_ushort(p[2 * z + 1]) << 16);
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+template <class P> __device__ inline void st_h2(const P& p, uint32_t v) {
+    p[0] = __ushort_as_half((unsigned short)(v & 0xffffu)); p[1] = __ushort_as_half((unsigned short)(v >> 16));
+}
+template <class P> __device__ inline void st_h8(const P& p, uint4 v) { st_h2(p, v.x); st_h2(p + 2, v.y); st_h2(p + 4, v.z); st_h2(p + 6, v.w); }
+#else
+__device__ __forceinline__ float4 ld_f4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float2 ld_f2(const float* p) { return *reinterpret_cast<const float2*>(p); }
+__device__ __forceinline__ double2 ld_d2(const double* p) { return *reinterpret_cast<const double2*>(p); }
+__device__ __forceinline__ uint2 ld_u2(const uint32_t* p) { return *reinterpret_cast<const uint2*>(p); }
+__device__ __forceinline__ void st_f4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ void st_f2(float* p, float2 v) { *reinterpret_cast<float2*>(p) = v; }
+__device__ __forceinline__ void st_d2(double* p, double2 v) { *reinterpret_cast<double2*>(p) = v; }
+__device__ __forceinline__ uint4 ld_h8(const __half* p) { return *reinterpret_cast<const uint4*>(p); }
+__device__ __forceinline__ void st_h2(__half* p, uint32_t v) { *reinterpret_cast<uint32_t*>(p) = v; }
+__device__ __forceinline__ void st_h8(__half* p, uint4 v) { *reinterpret_cast<uint4*>(p) = v; }
 #endif
 
 constexpr int kMaxSupport = GR_MAX_SUPPORT;   // largest support the convex programs are solved on
@@ -179,6 +212,12 @@ __device__ inline float fkey_inv(uint32_t k) {
 __device__ inline unsigned long long ckey(float v, int id) {
     return ((unsigned long long)fkey(v) << 32) | (unsigned long long)(0xffffffffu - (uint32_t)id);
 }
+
+// fp64 functions kept out of line: the solve kernels call them from many places, and a small batch runs most of their code
+// exactly once per SM, so what it waits for is instruction fetches.
+static __device__ __noinline__ double m_exp(double x) { return exp(x); }
+static __device__ __noinline__ double m_log(double x) { return log(x); }
+static __device__ __noinline__ double m_div(double a, double b) { return a / b; }
 
 constexpr int kMaxDevices = 64;               // per-device caches of the host code (function attributes, streams)
 

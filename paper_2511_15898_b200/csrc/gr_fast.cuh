@@ -1,894 +1,1291 @@
-// Fast per-instance solve for supports up to 128 tokens and n <= 16: one CTA per instance, 96 threads and four
-// CTAs per SM for supports up to 64, 128 threads and one CTA per SM above.
+// Fast per-instance solve for supports up to 128 tokens and n <= 16: one CTA per instance.
 //
-// Same mathematics as the robust kernel (gr_solve.cu): the gradient of the convex functions
+// Same mathematics as the general kernel (gr_solve.cu): the gradient of the convex functions
 // of the inner system / of an outer block (Thm "Inner Convex Solver", Thm "Outer Convex Solver")
 // is the one-dimensional integral
-//   g_i = w_i int e^{-t slack} x_i(t) n! [lambda^n] P(lambda; t) h_i(lambda; t) dt,
-// and Newton's method on alpha = log w uses its exact Hessian.  Organised for throughput:
-//   - one warp per quadrature node, one lane per token (up to four tokens per lane on the larger supports):
-//     every power series lives in registers;
-//   - the product P = e^{lambda h} prod_j f_j over the tokens is not multiplied out:
-//     d/dlambda log f_j = x_j d_j (1 + (1 - x_j) h_j), so the log-derivative S of P is a SUM over
-//     tokens (a warp reduction) and P follows from P' = S P.  In fp64 this is accurate to
-//     ~1e-12 for n <= 16 and degrades beyond (larger n takes the robust kernel);
-//   - h_j(lambda) = H(d_j lambda; x_j) with H(mu; x) = (e^mu - 1) / (1 + x (e^mu - 1)), whose
-//     coefficients obey a recurrence with compile-time constants 1/c!;
-//   - the Hessian's off-diagonal part  - sum_q c_q t_q (w x)_i (w x)_l n! [lambda^n] P h_i h_l  is a
-//     dense contraction over (node, series index); it only steers the iteration, so it is
-//     taken on every second node (trapezoid step doubled) and accumulated in fp32 from operands
-//     staged in shared memory; the gradient itself stays fp64 on every node;
-//   - the iteration starts from a mean-field point (each token against the expected weight
-//     of the other drafted tokens, with a bound on what a single huge competitor can add).
+//   g_i = w_i int e^{-t slack} x_i(t) n! [lambda^n] P(lambda; t) h_i(lambda; t) dt,   x_i = e^{-t w_i},
+// and Newton's method on alpha = log w uses its exact Hessian.  How the work is laid out:
+//   - the power series are scaled, lambda -> sigma lambda with sigma^n = n!, so that n! disappears and every
+//     coefficient is of order one (fp32 can hold them);
+//   - h(mu; x) = (e^mu - 1) / (1 + x (e^mu - 1)) obeys h' = 1 + (1 - 2x) h - x (1 - x) h^2 (the logistic curve's
+//     Riccati equation), which gives its coefficients stably at every x; up to eight of them come from the closed
+//     polynomials in x (1 - x) that the equation generates (the cumulants of a Bernoulli variable);
+//   - the product P = e^{lambda h} prod_j f_j is not multiplied out: d/dlambda log f_j = x_j d_j (1 + (1 - x_j) h_j), so
+//     the log-derivative S of P is a SUM over the tokens and P follows from P' = S P;
+//   - S: one thread per (quadrature node, share of the tokens), no reduction across lanes but the shares' sums;
+//     P: one thread per node;  g: one thread per token, walking the nodes (no reduction at all);
+//   - the Hessian's off-diagonal part  - sum_q c_q t_q (w x)_i (w x)_l n! [lambda^n] P h_i h_l  is a dense contraction over
+//     (node, series index): operands staged in shared memory in fp16, MMAs, fp32 accumulators in registers from the first node to
+//     the end of the factorisation.  The tokens are ordered by draft mass, so that the lower triangle pairs the series
+//     P h of the heavier token (all terms positive) with the h of the lighter one, and nothing cancels;
+//   - the iteration runs in fp32 as long as the residual is far above fp32's noise; the last evaluations, the only ones
+//     that can end it, are fp64 on the full quadrature grid and reuse the last factorisation (a Newton step with a
+//     Hessian from a point 1e-4 away contracts as well as one with a fresh one).
 #pragma once
 #include "gr_prep.cuh"
 #include "gr_verify.cuh"
 
-// The translation unit that includes this file chooses the padded support size: 64 (96-thread CTAs, four per
-// SM) or 128 (256-thread CTAs, one per SM: its shared memory admits no second CTA, so the one CTA brings two warps
-// per scheduler itself), and a namespace of its own for the instantiation.
-#ifndef GR_FAST_MP
-#define GR_FAST_MP 64
-#define GR_FAST_NS fast64
-#endif
-
 namespace gr {
-namespace GR_FAST_NS {
+namespace fast {
 
-constexpr int kMP = GR_FAST_MP;       // padded support size of these kernels
-constexpr int kRL = kMP / 32;         // rows (or tokens) per lane when a warp covers the whole support
-constexpr int kFT = kMP == 64 ? 96 : 256;   // threads per CTA (at least kMP - 8: one thread per panel row)
-constexpr int kFCtas = kMP == 64 ? 4 : 1;   // CTAs per SM the kernels are compiled for
-constexpr int kFW = kFT / 32;         // warps per CTA
-constexpr int kJC = kMP == 64 ? 6 : 4;      // Hessian nodes staged per chunk
-constexpr double kFTEnd = 25.0;       // quadrature range constants, identical to the robust kernel's
+constexpr double kFTEnd = 25.0;       // quadrature range constants, identical to the general kernel's
 constexpr double kFDrop = 1.0;
 constexpr double kFTail = 3.0;
 constexpr int kFMaxNodes = 128;
-constexpr int kMS = kMP + 8;          // row stride of the staged operands (floats): conflict-free MMA fragment loads
-constexpr int kJS = kMP + 1;          // row stride of the contraction accumulator / Hessian (floats)
+constexpr int kQC = 32;               // quadrature nodes handled together
 constexpr double kFAlphaClamp = 80.0;
 constexpr double kFStepClamp = 3.0;
+constexpr double kFCoarse = 1.0e-2;        // above this residual the trapezoid step is doubled
 constexpr double kFPredictStep = 1.0;      // largest |delta alpha| after which the stop on a predicted residual is allowed
 constexpr double kFPredictSafety = 10.0;   // the prediction s2 must be this many times below the tolerance
 constexpr double kFRatioSafety = 3.0;      // the predicted residual rho * r must be this many times below the tolerance
-constexpr double kFTrustPivot = 0.02;       // smallest relative pivot at which a predicted stop is allowed
+constexpr double kFTrustPivot = 0.02;      // smallest relative pivot at which a predicted stop is allowed
 constexpr double kFPredictBound = 3.0;     // reported norm after such a stop: kFPredictBound * s2
-constexpr int kFSweeps = 5;           // fixed-point sweeps of the starting point
+constexpr double kFLowLeave = 3.0e-5;      // predicted residual at which the iteration goes over to fp64
+constexpr double kFLowFloor = 1.0e-4;      // below this residual a failure to improve is taken for fp32's noise
+constexpr double kFChordBase = 0.02;       // contraction assumed of a step with the Hessian of a point a distance 0 away
+constexpr int kFCgMax = 16;                // conjugate-gradient iterations before the factorisation takes over
+constexpr float kFCgTol = 2.0e-4f;         // and their relative residual
+constexpr float kFScaleJump = 0.5f;        // distance of the common scale from which its curve is inverted exactly
+constexpr int kFSweeps = 5;                // fixed-point sweeps of the starting point
 
-struct FastLayout {
-    int KP;
-    int d, tg, p, r, key, psi, Dr, alpha, alpha_prev, delta, w, g, g2, col, gw, g2w, tq, cq, scal, uni;
-    int jacc_bytes_off, ints, total_bytes, uni_doubles;
-    __host__ __device__ FastLayout(int KP_, int NT) : KP(KP_) {
-        int o = 0;
-        d = o; o += KP; tg = o; o += KP; p = o; o += KP; r = o; o += KP; key = o; o += KP;
-        psi = o; o += KP + 4; Dr = o; o += KP + 4;
-        alpha = o; o += KP; alpha_prev = o; o += KP; delta = o; o += KP; w = o; o += KP; g = o; o += KP;
-        g2 = o; o += KP; col = o; o += kMP;
-        gw = o; o += kFW * KP; g2w = o; o += kFW * KP;
-        tq = o; o += kFMaxNodes; cq = o; o += kFMaxNodes;
-        scal = o; o += 48;
-        uni = o;
-        // union: staging of the Hessian operands (two float arrays [kJC * NT][kMS]) / vectors of the Newton step
-        const int stage_doubles = (2 * kJC * NT * kMS * 4 + 7) / 8;
-        const int jmat_doubles = 2 * (kMP + 4) + 2 * kMP;    // (floats, so twice what is needed) pivot row / column buffers
-        uni_doubles = stage_doubles > jmat_doubles ? stage_doubles : jmat_doubles;
-        o += uni_doubles;
-        jacc_bytes_off = o * 8;                       // float [kMP][kMP] accumulator of the contraction
-        o += (kMP * (kMP + 1) + 1) / 2;
-        ints = o * 8;
-        total_bytes = ints + KP * 4 * 4 + 64;
+// Compile-time geometry.  NT: series length (>= n), MP: padded support size, T: threads, JC: Hessian nodes staged
+// together, CTAS: CTAs per SM the registers are held to.
+template <int NT_, int MP_, int T_, int JC_, int CTAS_>
+struct Cfg {
+    static constexpr int NT = NT_, MP = MP_, T = T_, JC = JC_, kCtas = CTAS_;
+    static constexpr int kNG = T / MP;            // copies of the token threads (they share the nodes out among them)
+    static constexpr int kW = T / 32, kTW = MP / 32;
+    static constexpr int kRow = NT + 4;           // row stride of the product series (16-byte aligned rows in fp32 and fp64)
+        static constexpr int kTS = MP + 4;            // token stride of the staged operands: conflict-free fragment loads
+    static constexpr int kPanels = MP / 8;
+    static constexpr int kPr = MP / 32;           // pairs of 16-row tiles (a, MP / 16 - 1 - a): equal work per pair
+    static constexpr int kS = kW / kPr;           // warps that share a pair's column tiles
+    static constexpr int kNA = (MP / 16 + kS - 1) / kS, kNB = (MP / 8 + kS - 1) / kS;
+    static constexpr int kPack = NT >= 16 ? 1 : 16 / NT;   // Hessian nodes that fill one MMA depth of 16
+    static constexpr int kKS = JC / kPack;        // MMA steps per staged chunk
+    static_assert(T % MP == 0 && kW % kPr == 0 && kS * kNB <= MP / 8 && T >= kQC && JC % kPack == 0, "geometry");
+    // shared memory, byte offsets
+    static constexpr int oD = 0, oRhs = oD + MP * 8, oDr = oRhs + MP * 8, oWd = oDr + (MP + 4) * 8, oDsd = oWd + MP * 8;
+    static constexpr int oRed = oDsd + MP * 8, oScal = oRed + 64 * 8, oTq = oScal + 16 * 8, oCq = oTq + kQC * 8, oKq = oCq + kQC * 8;
+    static constexpr int oPP = oKq + kQC * 4, oSP = oPP + kQC * kRow * 8;
+    static constexpr int oWf = oSP + T * (NT + 2) * 8, oDsf = oWf + MP * 4, oE = oDsf + MP * 4;
+    static constexpr int oDg = oE + (NT <= 8 ? MP * 32 : 0), oYv = oDg + MP * 4, oDl = oYv + MP * 4;
+    static constexpr int oLd = oDl + MP * 4;                     // factored 8 x 8 diagonal blocks
+    static constexpr int oBlk = oLd + kPanels * 64 * 4, oOrd = oBlk + MP * 4, oTr = oOrd + MP * 4;
+    static constexpr int oU = (oTr + MP * 4 + 15) & ~15;           // union: staging / factor / start table / preparation
+    static constexpr int kStage = kKS * 4 * kTS * 8;               // bytes of one staged operand
+    static constexpr int kLFloats = 8 * (MP * kPanels - 4 * kPanels * (kPanels - 1));
+    static constexpr int kNS = MP + 8;                             // row stride of the scaled Hessian (halves): conflict-free rows
+    static constexpr int kPi = MP * kNS * 2;
+    static constexpr int kPrep = MP * 8 * 3 + (MP + 4) * 8 + MP * 8;
+    static constexpr int kU0 = 2 * kStage > kLFloats * 4 ? 2 * kStage : kLFloats * 4;
+    static constexpr int kU1 = kPi > kPrep ? kPi : kPrep;
+    static constexpr int kU2 = kU0 > kU1 ? kU0 : kU1;
+    static constexpr int kU = kU2 > kVerifyScratchBytes ? kU2 : kVerifyScratchBytes;
+    static constexpr int kBytes = oU + kU;
+};
+
+extern __shared__ __align__(16) unsigned char smem_raw[];
+
+// four (fp32) or two (fp64) consecutive elements; the other type's version is never called
+template <class P> __device__ __forceinline__ void ld_vec(const P& p, float* o) { const float4 v = ld_f4(p); o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w; }
+template <class P> __device__ __forceinline__ void ld_vec(const P& p, double* o) { const double2 v = ld_d2(p); o[0] = v.x; o[1] = v.y; }
+template <class P> __device__ __forceinline__ void st_vec(const P& p, const float* o) { st_f4(p, make_float4(o[0], o[1], o[2], o[3])); }
+template <class P> __device__ __forceinline__ void st_vec(const P& p, const double* o) { st_d2(p, make_double2(o[0], o[1])); }
+
+// Every array of the layout.  The base is the kernel's dynamic shared memory, so the addresses are constants wherever this
+// is constructed (functions that are kept out of line build it for themselves).
+template <class C>
+struct FSm {
+    GR_PTR(double) d, rhs, Dr, wd, dsd, red, scal;
+    GR_PTR(float) wf, E, dg, yv, dl, Ld, Lp;
+    GR_PTR(uint32_t) AS, HS;       // staged operands: half2 elements [step][4][token][2]
+    GR_PTR(float) kq;
+    GR_PTR(__half) pi;              // start: presence probabilities; later the scaled Hessian (row stride kNS)
+    GR_PTR(int) blk, ord, trunc;
+    char* base;
+    int* flag;
+    __device__ __forceinline__ explicit FSm(int* ck) {
+        char* const sb = reinterpret_cast<char*>(smem_raw);
+        base = sb; flag = ck;
+        d = GR_MKPTR(double, reinterpret_cast<double*>(sb + C::oD), C::MP, ck);
+        rhs = GR_MKPTR(double, reinterpret_cast<double*>(sb + C::oRhs), C::MP, ck);
+        Dr = GR_MKPTR(double, reinterpret_cast<double*>(sb + C::oDr), C::MP + 4, ck);
+        wd = GR_MKPTR(double, reinterpret_cast<double*>(sb + C::oWd), C::MP, ck);
+        dsd = GR_MKPTR(double, reinterpret_cast<double*>(sb + C::oDsd), C::MP, ck);
+        red = GR_MKPTR(double, reinterpret_cast<double*>(sb + C::oRed), 64, ck);
+        scal = GR_MKPTR(double, reinterpret_cast<double*>(sb + C::oScal), 16, ck);
+        wf = GR_MKPTR(float, reinterpret_cast<float*>(sb + C::oWf), C::MP, ck);
+        E = GR_MKPTR(float, reinterpret_cast<float*>(sb + C::oE), C::MP * 8, ck);
+        dg = GR_MKPTR(float, reinterpret_cast<float*>(sb + C::oDg), C::MP, ck);
+        yv = GR_MKPTR(float, reinterpret_cast<float*>(sb + C::oYv), C::MP, ck);
+        dl = GR_MKPTR(float, reinterpret_cast<float*>(sb + C::oDl), C::MP, ck);
+        Ld = GR_MKPTR(float, reinterpret_cast<float*>(sb + C::oLd), C::kPanels * 64, ck);
+        blk = GR_MKPTR(int, reinterpret_cast<int*>(sb + C::oBlk), C::MP, ck);
+        ord = GR_MKPTR(int, reinterpret_cast<int*>(sb + C::oOrd), C::MP, ck);
+        trunc = GR_MKPTR(int, reinterpret_cast<int*>(sb + C::oTr), C::MP, ck);
+        AS = GR_MKPTR(uint32_t, reinterpret_cast<uint32_t*>(sb + C::oU), C::kStage / 4, ck);
+        HS = GR_MKPTR(uint32_t, reinterpret_cast<uint32_t*>(sb + C::oU + C::kStage), C::kStage / 4, ck);
+        kq = GR_MKPTR(float, reinterpret_cast<float*>(sb + C::oKq), kQC, ck);
+        Lp = GR_MKPTR(float, reinterpret_cast<float*>(sb + C::oU), C::kLFloats, ck);
+        pi = GR_MKPTR(__half, reinterpret_cast<__half*>(sb + C::oU), C::MP * C::kNS, ck);
     }
 };
-static inline int fast_smem_bytes(int KP, int NT) { return FastLayout(KP, NT).total_bytes; }
+enum { SC_FAIL = 0, SC_PIVOT = 1, SC_OUT = 4 };
 
-struct FSm {
-    GR_PTR(double) d, tg, p, r, key, psi, Dr, alpha, alpha_prev, delta, w, g, g2, col, gw, g2w, tq, cq, scal, J;
-    GR_PTR(float) AS, HS, Jacc;
-    GR_PTR(int) id, blk, itmp, trunc;
-    int KP;
+// Arrays whose element type is the precision of the evaluation.
+template <class C, typename R>
+struct RSm {
+    GR_PTR(R) tq, cq, PP, SP, w, ds;
+    __device__ explicit RSm(const FSm<C>& sm) {
+        tq = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oTq), kQC, sm.flag);
+        cq = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oCq), kQC, sm.flag);
+        PP = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oPP), kQC * C::kRow, sm.flag);
+        SP = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oSP), C::T * (C::NT + 2) * (8 / (int)sizeof(R)), sm.flag);
+        const int ow = sizeof(R) == 4 ? C::oWf : C::oWd, od = sizeof(R) == 4 ? C::oDsf : C::oDsd;
+        w = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + ow), C::MP, sm.flag);
+        ds = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + od), C::MP, sm.flag);
+    }
 };
-enum { SC_Q = 0, SC_FAIL = 1, SC_RED = 8, SC_GRID = 24 };   // (SC_RED: one slot per warp; 16..23: preparation outputs;
-                                                            //  SC_GRID: two slots per warp)
 
 __device__ __forceinline__ double ipow(double x, int n) {
     double r = 1.0;
+#pragma unroll 1
     while (n > 0) { if (n & 1) r *= x; x *= x; n >>= 1; }
     return r;
 }
 
-// exp(-y) for y >= 0 (fp64): range reduction by ln 2 and a degree-13 Taylor polynomial on |r| <= ln2/2
-// (truncation below 1e-17 relative); results below 2^-1000 are flushed to zero.
+// exp(-y) for y >= 0 (fp64): Cody and Waite's range reduction by a two-part ln 2 and a degree-13 Taylor polynomial on
+// |r| <= ln2/2 (truncation below 1e-17 relative), summed in pairs and fours (Estrin's scheme: a third of Horner's chain,
+// which is what a warp alone on its scheduler waits for); results below 2^-1000 are flushed to zero.
 __device__ __forceinline__ double exp_neg(double y)
 {
     const double t = -y;
     const double kf = rint(t * 1.4426950408889634);
-    if (kf < -1000.0) return 0.0;
     double r = fma(-kf, 6.93147180369123816490e-01, t);
     r = fma(-kf, 1.90821492927058770002e-10, r);
-    double p = 1.6059043836821613e-10;                 // 1/13!
-    p = fma(p, r, 2.08767569878681e-09);               // 1/12!
-    p = fma(p, r, 2.505210838544172e-08);              // 1/11!
-    p = fma(p, r, 2.755731922398589e-07);              // 1/10!
-    p = fma(p, r, 2.7557319223985893e-06);             // 1/9!
-    p = fma(p, r, 2.48015873015873e-05);               // 1/8!
-    p = fma(p, r, 1.984126984126984e-04);              // 1/7!
-    p = fma(p, r, 1.388888888888889e-03);              // 1/6!
-    p = fma(p, r, 8.333333333333333e-03);              // 1/5!
-    p = fma(p, r, 4.1666666666666664e-02);             // 1/4!
-    p = fma(p, r, 1.6666666666666666e-01);             // 1/3!
-    p = fma(p, r, 0.5);
-    p = fma(p, r, 1.0);
-    p = fma(p, r, 1.0);
+    const double r2 = r * r, r4 = r2 * r2;
+    const double a0 = 1.0 + r, a1 = fma(r, 1.6666666666666666e-01, 0.5);                    // 1/2!, 1/3!
+    const double a2 = fma(r, 8.333333333333333e-03, 4.1666666666666664e-02);                // 1/4!, 1/5!
+    const double a3 = fma(r, 1.984126984126984e-04, 1.388888888888889e-03);                 // 1/6!, 1/7!
+    const double a4 = fma(r, 2.7557319223985893e-06, 2.48015873015873e-05);                 // 1/8!, 1/9!
+    const double a5 = fma(r, 2.505210838544172e-08, 2.755731922398589e-07);                 // 1/10!, 1/11!
+    const double a6 = fma(r, 1.6059043836821613e-10, 2.08767569878681e-09);                 // 1/12!, 1/13!
+    const double b0 = fma(r2, a1, a0), b1 = fma(r2, a3, a2), b2 = fma(r2, a5, a4);
+    const double p = fma(r4, fma(r4, fma(r4, a6, b2), b1), b0);
     const int k = (int)kf;
-    return __hiloint2double(__double2hiint(p) + (k << 20), __double2loint(p));
+    return kf < -1000.0 ? 0.0 : __hiloint2double(__double2hiint(p) + (k << 20), __double2loint(p));
 }
+__device__ __forceinline__ float ex2_approx(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+template <typename R> struct Rx;
+template <> struct Rx<double> {
+    static __device__ __forceinline__ double expneg(double y) { return exp_neg(y); }
+    static __device__ __forceinline__ double ex(double x) { return m_exp(x); }
+    static __device__ __forceinline__ double lg(double x) { return m_log(x); }
+};
+template <> struct Rx<float> {
+    static __device__ __forceinline__ float expneg(float y) { return ex2_approx(y * -1.4426950408889634f); }
+    static __device__ __forceinline__ float ex(float x) { return ex2_approx(x * 1.4426950408889634f); }
+    static __device__ __forceinline__ float lg(float x) { return __logf(x); }
+};
 
-__device__ __forceinline__ constexpr double inv_fact(int c) {
-    double f = 1.0;
-    for (int i = 2; i <= c; i++) f *= (double)i;
-    return 1.0 / f;
-}
-
-// hh[c], c = 1..NT: coefficients of (e^mu - 1) / (1 + x (e^mu - 1)) in mu.  Column-oriented so that the
-// dependent chain is two operations per coefficient.
-template <int NT>
-__device__ __forceinline__ void unit_h_series(double x, double* hh)
+// h[c], c = 1 .. N (N <= 8): coefficients of h(mu; x), from u = 1 - 2x and p = x (1 - x)
+// (closed forms of the Riccati recurrence below).
+template <int N, typename R>
+__device__ __forceinline__ void unit_series(R u, R p, R* h)
 {
-    double acc[NT + 1];
-#pragma unroll
-    for (int c = 1; c <= NT; c++) acc[c] = 0.0;
-    hh[1] = 1.0;
-#pragma unroll
-    for (int k = 1; k < NT; k++) {
-#pragma unroll
-        for (int c = k + 1; c <= NT; c++) acc[c] = fma(inv_fact(c - k), hh[k], acc[c]);
-        hh[k + 1] = fma(-x, acc[k + 1], inv_fact(k + 1));
-    }
+    h[1] = R(1);
+    if (N >= 2) h[2] = u * R(0.5);
+    if (N >= 3) h[3] = R(1.0 / 6) - p;
+    if (N >= 4) h[4] = u * fma(p, R(-0.5), R(1.0 / 24));
+    if (N >= 5) h[5] = fma(p, p - R(0.25), R(1.0 / 120));
+    if (N >= 6) h[6] = u * fma(p, fma(p, R(0.5), R(-1.0 / 12)), R(1.0 / 720));
+    if (N >= 7) h[7] = fma(p, fma(p, R(1.0 / 3) - p, R(-1.0 / 40)), R(1.0 / 5040));
+    if (N >= 8) h[8] = u * fma(p, fma(p, fma(p, R(-0.5), R(1.0 / 8)), R(-1.0 / 160)), R(1.0 / 40320));
 }
-
-__device__ __forceinline__ double warp_sum_d(double v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// Sum of NT-entry vectors over the 32 lanes, result in every lane.  Recursive halving: at each of the
-// first log2(NT) levels a lane keeps half of its entries and hands the other half to its partner, so the
-// exchange costs NT - 1 + (5 - log2 NT) shuffles instead of 5 NT; an all-gather of NT shuffles follows.
-template <int NT>
-__device__ __forceinline__ void warp_allreduce_series(double* S, int lane)
+// h[c], c = 1 .. N: coefficients of h(ds lambda; x) in lambda by the Riccati recurrence
+//   (c + 1) h_{c+1} = ds (1 - 2x) h_c - ds x (1 - x) sum_{a=1}^{c-1} h_a h_{c-a},   h_1 = ds.
+template <int N, typename R>
+__device__ __forceinline__ void riccati_series(R ds, R du, R dp, R* h)
 {
-    static_assert(NT == 4 || NT == 8 || NT == 16, "series length");
-    int cnt = NT, o = 16;
+    h[1] = ds;
+    const R m2 = R(-2) * dp;
 #pragma unroll
-    for (int lvl = 0; lvl < (NT == 16 ? 4 : (NT == 8 ? 3 : 2)); lvl++) {
-        const int half = cnt >> 1;
-        const bool up = (lane & o) != 0;
+    for (int c = 1; c < N; c++) {
+        R a = R(0);
 #pragma unroll
-        for (int c = 0; c < NT / 2; c++) {
-            if (c < half) {
-                const double keep = up ? S[c + half] : S[c];
-                const double send = up ? S[c] : S[c + half];
-                S[c] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-            }
-        }
-        cnt = half; o >>= 1;
-    }
-    double v = S[0];
-    for (; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    // lane bits (4, 3[, 2[, 1]]) say which entry the lane holds
-#pragma unroll
-    for (int c = 0; c < NT; c++) {
-        const int src = (NT == 16) ? ((((c >> 3) & 1) << 4) | (((c >> 2) & 1) << 3) | (((c >> 1) & 1) << 2) | ((c & 1) << 1))
-                      : (NT == 8) ? ((((c >> 2) & 1) << 4) | (((c >> 1) & 1) << 3) | ((c & 1) << 2))
-                                  : ((((c >> 1) & 1) << 4) | ((c & 1) << 3));
-        S[c] = __shfl_sync(0xffffffffu, v, src);
+        for (int k = 1; 2 * k < c; k++) a = fma(h[k], h[c - k], a);
+        if (c % 2 == 0) a = fma(R(0.5) * h[c / 2], h[c / 2], a);
+        h[c + 1] = fma(m2, a, du * h[c]) * R(1.0 / (c + 1));
     }
 }
 
-// tf32 rounding of a staged operand (the contraction runs on the tensor cores: it is the one dense
-// contraction of the path, and it only steers Newton's method)
-__device__ __forceinline__ float to_tf32(float x) {
-    uint32_t u;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(u) : "f"(x));
-    return __uint_as_float(u);
-}
-
-// Series of length 16 cancel too strongly for one tf32 product (a dominant draft token makes the terms of
-// sum_kappa A[n - kappa] h[kappa] alternate at ~1e3 times their sum): their operands are staged in full fp32 and
-// split into two tf32 parts when the fragments are loaded (three MMAs per tile step, error ~1e-6 per term).
-template <int NT>
-__device__ __forceinline__ float stage_round(float x) { return NT > 8 ? x : to_tf32(x); }
-
-__device__ __forceinline__ void mma_tf32(float& c0, float& c1, float& c2, float& c3, uint32_t a0, uint32_t a1,
-                                         uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
+__device__ __forceinline__ void mma_tf32(float* c, const float* a, const float* b)
 {
     asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(c0), "+f"(c1), "+f"(c2), "+f"(c3)
-                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(__float_as_uint(a[0])), "r"(__float_as_uint(a[1])), "r"(__float_as_uint(a[2])),
+                   "r"(__float_as_uint(a[3])), "r"(__float_as_uint(b[0])), "r"(__float_as_uint(b[1])));
 }
 
-// One chunk of the Hessian contraction: Jacc[i][l] += sum over the staged rows kk of AS[kk][i] HS[kk][l] for the
-// 16 x 8 tiles that touch the lower triangle, as m16n8k8 tf32 MMAs with fp32 accumulation.  K8 = staged rows,
-// a multiple of 8.  The lower tiles are dealt round-robin to the warps.
-template <bool kSplit>
-__device__ __forceinline__ void hess_chunk(const FSm& sm, int K8, int m)
+__device__ __forceinline__ void mma_f16(float* c, const uint32_t* a, const uint32_t* b)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int gid = lane >> 2, tig = lane & 3;
-    // tile (mi, ni), ni <= 2 mi + 1, has the running number mi (mi + 1) + ni
-    for (int t = warp; t < (kMP / 16) * (kMP / 16 + 1); t += kFW) {
-        int mi = 0;
-        while ((mi + 1) * (mi + 2) <= t) mi++;
-        const int ni = t - mi * (mi + 1);
-        const int i0 = 16 * mi, l0 = 8 * ni;
-        if (i0 >= m || l0 >= m) continue;
-        float c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f;
-        for (int k0 = 0; k0 < K8; k0 += 8) {
-            GR_PTR(const float) Ap = sm.AS + ((k0 + tig) * kMS + i0 + gid);
-            GR_PTR(const float) Bp = sm.HS + ((k0 + tig) * kMS + l0 + gid);
-            const float fa[4] = {Ap[0], Ap[8], Ap[4 * kMS], Ap[4 * kMS + 8]};
-            const float fb[2] = {Bp[0], Bp[4 * kMS]};
-            if (kSplit) {
-                uint32_t ah[4], al[4], bh[2], bl[2];
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+__device__ __forceinline__ uint32_t pack_half(float a, float b) {
+    const __half2 h = __floats2half2_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// ---- reductions over the token threads (the first kTW warps; the other copies' values are ignored); every thread
+// gets the result.  Two scratch areas in turn (`par`): one barrier each.  Out of line for the sake of code size.
+// (maximum of a, or its sum with `add`; sum of b)
+template <class C>
+__device__ __noinline__ double2 tok_max_sum_fn(double a, double b, bool add, int par, int* flag)
+{
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) {
+        const double t = __shfl_xor_sync(0xffffffffu, a, o);
+        a = add ? a + t : fmax(a, t);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    GR_PTR(double) r = GR_MKPTR(double, reinterpret_cast<double*>(smem_raw + C::oRed), 64, flag) + 32 * par;
+    const int w = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0 && w < C::kTW) { r[2 * w] = a; r[2 * w + 1] = b; }
+    __syncthreads();
+    a = r[0]; b = r[1];
+#pragma unroll
+    for (int i = 1; i < C::kTW; i++) { a = add ? a + r[2 * i] : fmax(a, r[2 * i]); b += r[2 * i + 1]; }
+    return make_double2(a, b);
+}
+template <class C>
+__device__ __forceinline__ void tok_max_sum(const FSm<C>& sm, double& a, double& b, int& par)
+{
+    const double2 t = tok_max_sum_fn<C>(a, b, false, par, sm.flag);
+    par ^= 1;
+    a = t.x; b = t.y;
+}
+template <class C>
+__device__ __forceinline__ double tok_sum(const FSm<C>& sm, double v, int& par)
+{
+    const double2 t = tok_max_sum_fn<C>(0.0, v, false, par, sm.flag);
+    par ^= 1;
+    return t.y;
+}
+// largest and smallest of the tokens' log-weights (fp32: they only place the quadrature grid)
+template <class C>
+__device__ __forceinline__ void tok_range(const FSm<C>& sm, float v, bool on, float& hi, float& lo, int& par)
+{
+    const unsigned a = __reduce_max_sync(0xffffffffu, on ? fkey(v) : 0u), b = __reduce_max_sync(0xffffffffu, on ? fkey(-v) : 0u);
+    GR_PTR(double) r = sm.red + 32 * par;
+    par ^= 1;
+    const int w = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0 && w < C::kTW) r[w] = __hiloint2double((int)a, (int)b);
+    __syncthreads();
+    unsigned ka = 0u, kb = 0u;
+#pragma unroll
+    for (int i = 0; i < C::kTW; i++) { const double t = r[i]; ka = max(ka, (unsigned)__double2hiint(t)); kb = max(kb, (unsigned)__double2loint(t)); }
+    hi = fkey_inv(ka); lo = -fkey_inv(kb);
+}
+
+// Accumulator fragments of the tiles a warp owns: row tiles a and b of its pair, column tiles cs, cs + kS, ...
+template <class C>
+struct Frags { float A[C::kNA][4], B[C::kNB][4]; };
+
+// Adds the staged operands (ksteps MMA depths of 16) to the fragments.  Straight-line: every tile of the pair, those above
+// the diagonal included, so that the loads of a step go out together.  (An m16n8k16 fp16 MMA takes the tensor pipe as long
+// as an m16n8k8 tf32 one, 8 cycles, and carries the same mantissa.)
+template <class C>
+__device__ __forceinline__ void hess_mma(const FSm<C>& sm, Frags<C>& fr, int ksteps)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gid = lane >> 2, tig = lane & 3;
+    const int ra = warp % C::kPr, rb = C::MP / 16 - 1 - ra, cs = warp / C::kPr;
+#pragma unroll 1
+    for (int ks = 0; ks < ksteps; ks++) {
+        GR_PTR(const uint32_t) Ap = sm.AS + 2 * ((ks * 4 + tig) * C::kTS + gid);
+        GR_PTR(const uint32_t) Hp = sm.HS + 2 * ((ks * 4 + tig) * C::kTS + gid);
+        uint2 hv[C::kNB];
+#pragma unroll
+        for (int s = 0; s < C::kNB; s++) hv[s] = ld_u2(Hp + 16 * (cs + s * C::kS));
+        const uint2 a0 = ld_u2(Ap + 32 * ra), a1 = ld_u2(Ap + 32 * ra + 16), b0 = ld_u2(Ap + 32 * rb), b1 = ld_u2(Ap + 32 * rb + 16);
+        const uint32_t fa[4] = {a0.x, a1.x, a0.y, a1.y}, fb[4] = {b0.x, b1.x, b0.y, b1.y};
+#pragma unroll
+        for (int s = 0; s < C::kNB; s++) {
+            const uint32_t bb[2] = {hv[s].x, hv[s].y};
+            if (s < C::kNA) mma_f16(fr.A[s < C::kNA ? s : 0], fa, bb);
+            mma_f16(fr.B[s], fb, bb);
+        }
+    }
+}
+
+// Gradient g and the Hessian's diagonal part g2 at the weights in shared memory (this thread's in w_own), in fp64; or in
+// fp32 with kJac, which adds the Hessian's contraction (fragments fr) from every jstride-th node: the off-diagonal entries
+// times z_i z_l, z = rhs^(-1/2) (z_own is this thread's), which keeps the fp16 operands of order one.
+//   amax, amin  extreme log-weights;  hs = sigma * (draft mass above the block)
+// Every token thread (all copies) gets g and g2.
+template <class C, typename R, bool kJac>
+__device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, double hs, int slack, double qstep_d, int jstride,
+                                            float amax, float amin, double w_own, double ds_own, float z_own, double& g_out,
+                                            double& g2_out, Frags<C>& fr)
+{
+    static_assert(!kJac || sizeof(R) == 4, "the contraction's operands are fp32");
+    constexpr int NT = C::NT, T = C::T;
+    const RSm<C, R> rs(sm);
+    const int tid = threadIdx.x, i = tid % C::MP, ng = tid / C::MP;
+    const R qstep = (R)qstep_d;
+    // (where the grid lies does not matter to its accuracy: fp32)
+    const float wmax = Rx<float>::ex(amax), wmin = Rx<float>::ex(amin);
+    const float f_hi = Rx<float>::lg((float)kFTEnd / (slack ? 1.f + wmin : wmin));
+    const float f_0 = -Rx<float>::lg((slack ? 1.f : 0.f) + wmax) - (float)kFDrop;
+    int Q = (int)ceilf((f_hi - (f_0 - (float)kFTail)) / (float)qstep_d) + 1;
+    if (Q > kFMaxNodes) Q = kFMaxNodes;
+    const R s_hi = (R)f_hi, s0 = (R)f_0;
+    const R wi = (R)w_own, dsi = (R)ds_own;
+    R dp[NT <= 8 ? NT + 1 : 1];
+    if (NT <= 8) {
+        dp[0] = R(1);
+#pragma unroll
+        for (int c = 1; c <= (NT <= 8 ? NT : 0); c++) dp[c] = dp[c - 1] * dsi;
+    }
+    R g = R(0), g2 = R(0);
+    if (kJac) {
+#pragma unroll
+        for (int s = 0; s < C::kNA; s++) { fr.A[s][0] = fr.A[s][1] = fr.A[s][2] = fr.A[s][3] = 0.f; }
+#pragma unroll
+        for (int s = 0; s < C::kNB; s++) { fr.B[s][0] = fr.B[s][1] = fr.B[s][2] = fr.B[s][3] = 0.f; }
+    }
+    const bool live = kJac || (i & ~31) < m;       // (the contraction's operands are staged for every slot: zeros beyond m)
+#pragma unroll 1
+    for (int q0 = 0; q0 < Q; q0 += kQC) {
+        const int nq = min(kQC, Q - q0);
+        // ---- S: this thread's share of the tokens at its node (16 or 32 node slots)
+        const bool narrow = nq <= 16;
+        const int q = tid & (narrow ? 15 : 31), G = T / (narrow ? 16 : 32), grp = tid / (narrow ? 16 : 32);
+        constexpr int kSS = sizeof(R) == 4 ? NT + 4 : NT + 2;      // row stride of the shares: conflict-free vector access
+        {
+            const R s = s_hi - qstep * (R)(q0 + q);
+            const R e = Rx<R>::expneg(s - s0);
+            const R t = Rx<R>::expneg(e - s);
+            if (tid < nq) {
+                const R c0 = qstep * (R(1) + e) * t * (slack ? Rx<R>::expneg(t) : R(1));
+                rs.tq[q] = t; rs.cq[q] = c0;
+                if (kJac) sm.kq[q] = sqrtf((float)((R)jstride * c0 * t));
+            }
+            R S[NT];
+#pragma unroll
+            for (int c = 0; c < NT; c++) S[c] = R(0);
+            if (q < nq) {
+#pragma unroll 2
+                for (int j = grp; j < m; j += G) {
+                    const R x = Rx<R>::expneg(t * rs.w[j]);
+                    const R d = rs.ds[j];
+                    const R u = fma(R(-2), x, R(1)), p = fma(-x, x, x);
+                    S[0] = fma(x, d, S[0]);
+                    R h[NT + 1];
+                    if (NT <= 8) {
+                        unit_series<NT - 1, R>(u, p, h);
+                        R pe[8];                           // p ds^(c+1)
+                        if (sizeof(R) == 4) {
+                            const float4 e0 = ld_f4(sm.E + 8 * j), e1 = NT > 4 ? ld_f4(sm.E + 8 * j + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+                            const float ev[8] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
+#pragma unroll
+                            for (int c = 1; c < 8; c++) pe[c] = p * (R)ev[c];
+                        } else {
+                            const R d2 = d * d, d4 = d2 * d2, pd = p * d;
+                            pe[1] = p * d2; pe[2] = pd * d2; pe[3] = p * d4; pe[4] = pd * d4;
+                            pe[5] = pe[1] * d4; pe[6] = pe[2] * d4; pe[7] = pe[3] * d4;
+                        }
+#pragma unroll
+                        for (int c = 1; c < NT; c++) S[c] = fma(pe[c & 7], h[c], S[c]);
+                    } else {
+                        const R pd = p * d;
+                        riccati_series<NT - 1, R>(d, d * u, pd, h);
+#pragma unroll
+                        for (int c = 1; c < NT; c++) S[c] = fma(pd, h[c], S[c]);
+                    }
+                }
+            }
+            if (narrow) {
+#pragma unroll
+                for (int c = 0; c < NT; c++) S[c] += __shfl_xor_sync(0xffffffffu, S[c], 16);
+            }
+            if (q < nq && (!narrow || (tid & 16) == 0)) {
+                GR_PTR(R) row = rs.SP + ((tid >> 5) * 32 + q) * kSS;
+#pragma unroll
+                for (int c = 0; c < NT; c += 16 / (int)sizeof(R)) st_vec(row + c, S + c);
+            }
+        }
+        __syncthreads();
+        // ---- P: one thread per node.  PP[j] = P[n - 1 - j], so that PP[c - 1] pairs with h[c] in [lambda^n] P h
+        if (tid < nq) {
+            R S[NT], P[NT + 1], acc[NT + 1];
+#pragma unroll
+            for (int c = 0; c < NT; c++) S[c] = R(0);
+#pragma unroll 2
+            for (int k = 0; k < C::kW; k++) {
+                GR_PTR(const R) row = rs.SP + (k * 32 + tid) * kSS;
+#pragma unroll
+                for (int c = 0; c < NT; c += 16 / (int)sizeof(R)) {
+                    R v[16 / sizeof(R)];
+                    ld_vec(row + c, v);
+#pragma unroll
+                    for (int z = 0; z < 16 / (int)sizeof(R); z++) S[c + z] += v[z];
+                }
+            }
+            S[0] += (R)hs;
+            P[0] = R(1);
+#pragma unroll
+            for (int c = 1; c <= NT; c++) acc[c] = R(0);
+#pragma unroll
+            for (int k = 0; k < NT - 1; k++) {
+#pragma unroll
+                for (int c = k + 1; c < NT; c++) acc[c] = fma(S[c - 1 - k], P[k], acc[c]);
+                P[k + 1] = acc[k + 1] * R(1.0 / (k + 1));
+            }
+            GR_PTR(R) row = rs.PP + tid * C::kRow;
+#pragma unroll
+            for (int e = 0; e < NT; e++) {
+                // (entries at and beyond n are zero)
+                if (e < n) row[n - 1 - e] = P[e]; else row[e] = R(0);
+            }
+        }
+        __syncthreads();
+        // ---- g: one thread per token; with kJac the operands of the contraction for every jstride-th node
+        const int span = kJac ? jstride * C::JC : nq;
+        const int step = kJac ? jstride : 1;
+#pragma unroll 1
+        for (int qa = 0; qa < nq; qa += span) {
+            const int qb = min(nq, qa + span);
+            const int nst = kJac ? (qb - qa + jstride - 1) / jstride : 0;
+            auto node = [&](int q2, bool stage, int slot) {
+                const R t = rs.tq[q2], c0 = rs.cq[q2];
+                const R x = Rx<R>::expneg(t * wi);
+                const R u = fma(R(-2), x, R(1)), p = fma(-x, x, x);
+                R h[NT + 1];
+                if (NT <= 8) {
+                    unit_series<NT, R>(u, p, h);
+#pragma unroll
+                    for (int c = 1; c <= NT; c++) h[c] *= dp[NT <= 8 ? c : 0];
+                } else {
+                    riccati_series<NT, R>(dsi, dsi * u, dsi * p, h);
+                }
+                R pr[NT];
+                R v0 = R(0), v1 = R(0);
+#pragma unroll
+                for (int c = 0; c < NT; c += 16 / (int)sizeof(R)) ld_vec(rs.PP + q2 * C::kRow + c, pr + c);
+#pragma unroll
+                for (int c = 0; c < NT; c += 2) { v0 = fma(pr[c], h[c + 1], v0); v1 = fma(pr[c + 1], h[c + 2], v1); }
+                const R ux = wi * x;
+                const R gi = c0 * ux * (v0 + v1);
+                g += gi;
+                g2 = fma(gi * t, wi, g2);
+                if (stage) {
+                    // A = P h (series), paired as sum_kappa A[n - kappa] h_l[kappa], kappa = 1 .. n - 1; both sides carry the
+                    // square root of the node's weight and of the token's scale
+                    const float uz = sm.kq[q2] * (float)ux * z_own;
+                    // (pair z of the node's series indices: element (z & 3) of its MMA depth, half (z >> 2) of the fragment)
+                    const int o = (slot / C::kPack) * 8 * C::kTS + 2 * i;
+                    const int sub = slot % C::kPack;
+#pragma unroll
+                    for (int z = 0; z < NT / 2; z++) {
+                        float a[2];
+#pragma unroll
+                        for (int y = 0; y < 2; y++) {
+                            const int kap = 2 * z + y + 1;
+                            float v = 0.f;
+#pragma unroll
+                            for (int c = 1; c <= NT - kap; c++) v = fmaf((float)h[c], (float)pr[kap + c - 1], v);
+                            a[y] = v;
+                        }
+                        const int f = sub * (NT / 2) + z, at = o + (f & 3) * 2 * C::kTS + (f >> 2);
+                        sm.AS[at] = pack_half(uz * a[0], uz * a[1]);
+                        sm.HS[at] = pack_half(uz * (float)h[2 * z + 1], z == NT / 2 - 1 ? 0.f : uz * (float)h[2 * z + 2]);
+                    }
+                }
+            };
+            if (live) {
+                if (kJac) {
+#pragma unroll 2
+                    for (int z = ng; z < nst; z += C::kNG) node(qa + z * step, true, z);
+                    if (jstride == 2) {
+#pragma unroll 2
+                        for (int z = qa + 1 + 2 * ng; z < qb; z += 2 * C::kNG) node(z, false, 0);
+                    }
+                } else {
+#pragma unroll 2
+                    for (int z = ng; z < nq; z += C::kNG) node(z, false, 0);
+                }
+            }
+            if (kJac) {
+                // unused slots of the last MMA depth
+                if (C::kPack > 1 && nst % C::kPack != 0) {
+                    for (int e = nst * (NT / 2) + tid / C::MP; e < (nst + C::kPack - 1) / C::kPack * 8; e += C::kNG) {
+                        const int at = (e >> 3) * 8 * C::kTS + 2 * i + (e & 3) * 2 * C::kTS + ((e & 7) >> 2);
+                        sm.AS[at] = 0u; sm.HS[at] = 0u;
+                    }
+                }
+                __syncthreads();
+                hess_mma<C>(sm, fr, (nst + C::kPack - 1) / C::kPack);
+                __syncthreads();
+            }
+        }
+        if (!kJac) __syncthreads();
+    }
+    double gd = (double)g, g2d = (double)g2;
+    if (C::kNG > 1) {
+        // sum over the copies, in the same order everywhere
+        GR_PTR(double) gs = GR_MKPTR(double, reinterpret_cast<double*>(sm.base + C::oSP), C::T * (C::NT + 2), sm.flag);
+        gs[2 * tid] = gd; gs[2 * tid + 1] = g2d;
+        __syncthreads();
+        gd = 0.0; g2d = 0.0;
+#pragma unroll
+        for (int k = 0; k < C::kNG; k++) { gd += gs[2 * (k * C::MP + i)]; g2d += gs[2 * (k * C::MP + i) + 1]; }
+        __syncthreads();
+    }
+    g_out = gd; g2_out = g2d;
+}
+
+// The fp64 evaluation, kept out of line (it is called once or twice per system, and its registers stay its own).
+template <class C>
+__device__ __noinline__ double2 eval_fp64(int m, int n, double hs, int slack, double qstep, float amax, float amin, double w_own,
+                                          double ds_own, int* flag)
+{
+    const FSm<C> sm(flag);
+    Frags<C> none;
+    double2 r;
+    eval_system<C, double, false>(sm, m, n, hs, slack, qstep, 1, amax, amin, w_own, ds_own, 0.f, r.x, r.y, none);
+    return r;
+}
+
+// Float index of row r (>= 8 j) of the j-th 8-column panel.  Within a factored row column c sits at panel_pos(c), so that
+// the columns t and t + 4 an MMA fragment needs are adjacent.
+template <class C>
+__device__ __forceinline__ int panel_row(int j, int r) { return 8 * (C::MP * j - 4 * j * (j - 1)) + (r - 8 * j) * 8; }
+__device__ __forceinline__ int panel_pos(int c) { return c < 4 ? 2 * c : 2 * c - 7; }
+__device__ __forceinline__ float fast_rsqrt(float x) { float y; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+// fp32 value as two tf32 parts (the tensor core drops the low bits of the second)
+__device__ __forceinline__ void split_tf32(float x, float& hi, float& lo) {
+    hi = __uint_as_float(__float_as_uint(x) & 0xffffe000u);
+    lo = x - hi;
+}
+
+// Factorisation H = L L^T (fp32) out of the fragments, which hold the contraction: off-diagonal add - fr times sm.wf of row and
+// column, diagonal in sm.dg; the forward substitution of sm.yv is carried along (result in sm.dl).  L stays in shared memory for later
+// right-hand sides.  The matrix never leaves the fragments as a whole: each 8-column panel is written to shared memory,
+// every thread factors the 8 x 8 diagonal block in registers (redundantly: no exchange), one thread per row solves the
+// panel below it, and the fragments take the rank-8 update (operands split into two tf32 parts, ~fp32 products).  The
+// eight threads of the block's own rows solve for unit vectors instead: they get the inverse of the block's factor,
+// which turns the substitutions' 8 x 8 solves into independent dot products (sm.Ld: row i holds column i of the inverse).
+// SC_FAIL / SC_PIVOT receive whether a pivot was not positive and the smallest relative pivot.
+template <class C>
+__device__ __forceinline__ void factor(const FSm<C>& sm, Frags<C>& fr, int m, float add)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tig = lane & 3;
+    const int ra = warp % C::kPr, rb = C::MP / 16 - 1 - ra, cs = warp / C::kPr;
+    const int m16 = (m + 15) & ~15;
+    // matrix out of the contraction (identity beyond m)
+    auto entry = [&](float f, int row, int col) {
+        return row == col ? sm.dg[row] : (row < m && col < m ? add - f * sm.wf[row] * sm.wf[col] : 0.f);
+    };
+#pragma unroll
+    for (int s = 0; s < C::kNB; s++) {
+        const int ni = cs + s * C::kS;
+#pragma unroll
+        for (int z = 0; z < 4; z++) {
+            const int col = 8 * ni + 2 * tig + (z & 1), r = gid + 8 * (z >> 1);
+            if (s < C::kNA) fr.A[s < C::kNA ? s : 0][z] = entry(fr.A[s < C::kNA ? s : 0][z], 16 * ra + r, col);
+            fr.B[s][z] = entry(fr.B[s][z], 16 * rb + r, col);
+        }
+    }
+    bool bad = false;
+    float pmin = 1.f;
+    const int npan = (m + 7) >> 3;
+#pragma unroll 1
+    for (int j = 0; j < npan; j++) {
+        // the panel's columns out of the fragments
+        auto put = [&](int rt, const float* v) {
+            GR_PTR(float) p = sm.Lp + panel_row<C>(j, 16 * rt + gid) + 2 * tig;
+            if (2 * rt >= j) st_f2(p, make_float2(v[0], v[1]));
+            st_f2(p + 64, make_float2(v[2], v[3]));               // (eight rows further)
+        };
+#pragma unroll
+        for (int s = 0; s < C::kNB; s++) {
+            if (cs + s * C::kS == j) {
+                if (s < C::kNA && 2 * ra + 1 >= j) put(ra, fr.A[s < C::kNA ? s : 0]);
+                if (2 * rb + 1 >= j && 16 * rb < m16) put(rb, fr.B[s]);
+            }
+        }
+        __syncthreads();
+        const int r = 8 * j + tid;
+        if (r < m16) {
+            float Lb[8][8], yb[8], v[8];
+            {
+                GR_PTR(const float) p = sm.Lp + panel_row<C>(j, 8 * j);
+                GR_PTR(const float) yp = sm.yv + 8 * j;
+                GR_PTR(const float) q = sm.Lp + panel_row<C>(j, r);
+#pragma unroll
+                for (int c = 0; c < 8; c++) {
+                    const float4 lo = ld_f4(p + 8 * c);
+                    Lb[c][0] = lo.x; Lb[c][1] = lo.y; Lb[c][2] = lo.z; Lb[c][3] = lo.w;
+                    if (c >= 4) { const float4 hi = ld_f4(p + 8 * c + 4); Lb[c][4] = hi.x; Lb[c][5] = hi.y; Lb[c][6] = hi.z; Lb[c][7] = hi.w; }
+                }
+                const float4 y0 = ld_f4(yp), y1 = ld_f4(yp + 4), q0 = ld_f4(q), q1 = ld_f4(q + 4);
+                yb[0] = y0.x; yb[1] = y0.y; yb[2] = y0.z; yb[3] = y0.w; yb[4] = y1.x; yb[5] = y1.y; yb[6] = y1.z; yb[7] = y1.w;
+                v[0] = q0.x; v[1] = q0.y; v[2] = q0.z; v[3] = q0.w; v[4] = q1.x; v[5] = q1.y; v[6] = q1.z; v[7] = q1.w;
+            }
+            float yi = sm.yv[r];
+            if (tid < 8) {
+#pragma unroll
+                for (int c = 0; c < 8; c++) v[c] = tid == c ? 1.f : 0.f;
+                yi = 0.f;
+            }
+            float piv = 1.f;
+#pragma unroll
+            for (int c = 0; c < 8; c++) {
+                const float dv = Lb[c][c];
+                bad = bad || !(dv > 0.f);
+                if (tid == c) piv = dv;
+                const float di = fast_rsqrt(dv);
+#pragma unroll
+                for (int r2 = c + 1; r2 < 8; r2++) Lb[r2][c] *= di;
+                yb[c] *= di;
+                const float lc = v[c] * di;
+                v[c] = lc;
+#pragma unroll
+                for (int c3 = c + 1; c3 < 8; c3++) {
+#pragma unroll
+                    for (int r2 = c3; r2 < 8; r2++) Lb[r2][c3] = fmaf(-Lb[r2][c], Lb[c3][c], Lb[r2][c3]);
+                    v[c3] = fmaf(-lc, Lb[c3][c], v[c3]);
+                    yb[c3] = fmaf(-Lb[c3][c], yb[c], yb[c3]);
+                }
+                yi = fmaf(-lc, yb[c], yi);
+            }
+            if (tid < 8) {
+                // column tid of the inverse factor; the finished right-hand side
+                float yo = 0.f;
+#pragma unroll
+                for (int c = 0; c < 8; c++) if (tid == c) yo = yb[c];
+                GR_PTR(float) p = sm.Ld + j * 64 + tid * 8;
+                st_f4(p, make_float4(v[0], v[1], v[2], v[3]));
+                st_f4(p + 4, make_float4(v[4], v[5], v[6], v[7]));
+                sm.dl[r] = yo;
+                pmin = fminf(pmin, __fdividef(piv, sm.dg[r]));
+            } else {
+                sm.yv[r] = yi;
+                GR_PTR(float) p = sm.Lp + panel_row<C>(j, r);
+                st_f4(p, make_float4(v[0], v[4], v[1], v[5]));
+                st_f4(p + 4, make_float4(v[2], v[6], v[3], v[7]));
+            }
+        }
+        __syncthreads();
+        // rank-8 update of the tiles to the right (loads first; rows of the diagonal block itself only reach entries above
+        // the diagonal)
+        const bool onA = 2 * ra + 1 > j && 16 * ra < m, onB = 2 * rb + 1 > j && 16 * rb < m;
+        if (onA || onB) {
+            float fa[4], fb[4];
+            float2 cv[C::kNB];
+            auto load_rows = [&](int rt, float* f) {
+                GR_PTR(const float) p = sm.Lp + panel_row<C>(j, max(16 * rt, 8 * j) + gid) + 2 * tig;
+                const float2 f0 = ld_f2(p), f1 = ld_f2(p + 64);
+                f[0] = -f0.x; f[1] = -f1.x; f[2] = -f0.y; f[3] = -f1.y;
+            };
+#pragma unroll
+            for (int s = 0; s < C::kNB; s++)
+                cv[s] = ld_f2(sm.Lp + panel_row<C>(j, 8 * max(cs + s * C::kS, j) + gid) + 2 * tig);
+            load_rows(ra, fa);
+            load_rows(rb, fb);
+            {
+                float al[4], bl[4], ah[4], bh[4];
+#pragma unroll
+                for (int z = 0; z < 4; z++) { split_tf32(fa[z], ah[z], al[z]); split_tf32(fb[z], bh[z], bl[z]); }
+#pragma unroll
+                for (int s = 0; s < C::kNB; s++) {
+                    const int ni = cs + s * C::kS;
+                    if (ni > j && 8 * ni < m) {
+                        float ch[2], cl[2];
+                        split_tf32(cv[s].x, ch[0], cl[0]); split_tf32(cv[s].y, ch[1], cl[1]);
+                        if (s < C::kNA && onA) {
+                            float* x = fr.A[s < C::kNA ? s : 0];
+                            mma_tf32(x, al, ch); mma_tf32(x, ah, cl); mma_tf32(x, ah, ch);
+                        }
+                        if (onB) { mma_tf32(fr.B[s], bl, ch); mma_tf32(fr.B[s], bh, cl); mma_tf32(fr.B[s], bh, ch); }
+                    }
+                }
+            }
+        }
+        // (the next panel goes to an area of its own: no barrier here)
+    }
+    if (tid < 32) {
+        pmin = fminf(pmin, __shfl_xor_sync(0xffffffffu, pmin, 4));
+        pmin = fminf(pmin, __shfl_xor_sync(0xffffffffu, pmin, 2));
+        pmin = fminf(pmin, __shfl_xor_sync(0xffffffffu, pmin, 1));
+        if (tid == 0) { sm.scal[SC_FAIL] = bad ? 1.0 : 0.0; sm.scal[SC_PIVOT] = (double)pmin; }
+    }
+}
+
+// Backward substitution L^T x = sm.dl, in place, warp 0: eight unknowns at a time from the last panel up.
+template <class C>
+__device__ __noinline__ void backward_subst(int m, int* flag)
+{
+    const FSm<C> sm(flag);
+    constexpr int kU = C::MP / 32;
+    const int lane = threadIdx.x, e = lane & 7;
+    if (lane >= 32) return;
+    __syncwarp();
+    float y[kU];
+#pragma unroll
+    for (int u = 0; u < kU; u++) y[u] = lane + 32 * u < m ? sm.dl[lane + 32 * u] : 0.f;
+    __syncwarp();
+#pragma unroll 1
+    for (int j = (m - 1) >> 3; j >= 0; j--) {
+        // x = (inverse of the diagonal block)^T y: lane e of every octet forms x_e = sum_c Ld[e][c] y_c
+        float li[8], l[kU][8];
+        {
+            GR_PTR(const float) p = sm.Ld + 64 * j + 8 * e;
+            const float4 lo = ld_f4(p), hi = ld_f4(p + 4);
+            li[0] = lo.x; li[1] = lo.y; li[2] = lo.z; li[3] = lo.w; li[4] = hi.x; li[5] = hi.y; li[6] = hi.z; li[7] = hi.w;
+        }
+#pragma unroll
+        for (int u = 0; u < kU; u++) {
+            // rows 8 j .. 8 j + 7 of this lane's column (rows of its own diagonal block are not used)
+            const int c = lane + 32 * u, pj = min(c >> 3, j);
+            GR_PTR(const float) p = sm.Lp + panel_row<C>(pj, 8 * j) + panel_pos(c & 7);
+#pragma unroll
+            for (int z = 0; z < 8; z++) l[u][z] = p[8 * z];
+        }
+        float src = y[0];
+#pragma unroll
+        for (int u = 1; u < kU; u++) if ((8 * j) >> 5 == u) src = y[u];
+        float x0 = 0.f, x1 = 0.f;
+#pragma unroll
+        for (int c = 0; c < 8; c += 2) {
+            x0 = fmaf(li[c], __shfl_sync(0xffffffffu, src, (8 * j + c) & 31), x0);
+            x1 = fmaf(li[c + 1], __shfl_sync(0xffffffffu, src, (8 * j + c + 1) & 31), x1);
+        }
+        const float x = x0 + x1;
+        if (lane < 8) sm.dl[8 * j + lane] = x;
+        float a[kU], b[kU];
+#pragma unroll
+        for (int u = 0; u < kU; u++) { a[u] = 0.f; b[u] = 0.f; }
+#pragma unroll
+        for (int c = 0; c < 8; c += 2) {
+            const float xa = __shfl_sync(0xffffffffu, x, c), xb = __shfl_sync(0xffffffffu, x, c + 1);
+#pragma unroll
+            for (int u = 0; u < kU; u++) { a[u] = fmaf(l[u][c], xa, a[u]); b[u] = fmaf(l[u][c + 1], xb, b[u]); }
+        }
+#pragma unroll
+        for (int u = 0; u < kU; u++) if (lane + 32 * u < 8 * j) y[u] -= a[u] + b[u];
+    }
+}
+
+// Right-hand side of the Newton system.  Along its own coordinate a token's flow behaves like a logistic curve
+// g_i = c sigma(alpha_i - kappa): linear in w_i while the token is light, saturating at the flow c of the tuples it can win
+// at all once it is heavy.  The curve through the current value and slope (H_ii = g_i (1 - g_i / c) gives c = g_i^2 / g2_i)
+// is inverted exactly: H_ii (logit(rhs_i / c) - logit(g_i / c)) replaces rhs_i - g_i.  Near the solution the two agree to
+// first order; far from it a token close to saturation is placed at once, and a light one gets the multiplicative
+// update log(rhs_i / g_i).  A target at or beyond the saturation level says that the curve is off: plain residual.
+__device__ __forceinline__ float newton_rhs(double g, double g2, double r)
+{
+    const float gf = (float)g, diff = (float)(r - g), hii = (float)(g - g2);
+    const float room = 1.f - __fdividef((float)r * __fdividef((float)g2, gf), gf);
+    const float arg = fmaxf(__fdividef(diff, gf * fmaxf(room, 1e-3f)), -0.999999f);
+    return room > 1e-3f ? hii * (fabsf(arg) < 0.01f ? arg * fmaf(arg, fmaf(arg, 1.f / 3.f, -0.5f), 1.f) : __logf(1.f + arg)) : diff;
+}
+
+// fp32 evaluation at one point and what the Newton step needs from it, out of line (its registers, fragments included, stay
+// its own).  Default: the Hessian scaled to unit diagonal, I - N with N_il = H_il / sqrt(H_ii H_ll), N in half precision
+// (its error, 2^-11, is that of the contraction's operands) for cg_solve below; sm.dg receives 1 / sqrt(H_ii).
+// With `chol` a Cholesky factorisation instead, for systems conjugate gradients do not get through.  `given`: the gradient
+// and the diagonal part come from the caller, in fp64.
+template <class C>
+__device__ __noinline__ double2 eval_hessian(int m, int n, double hs, int slack, double qstep, int jstride, float amax, float amin,
+                                             double w_own, double ds_own, double rhs, bool given, bool chol, double2 gg, int* flag)
+{
+    const FSm<C> sm(flag);
+    const int tid = threadIdx.x, i = tid % C::MP, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tig = lane & 3;
+    Frags<C> fr;
+    double g, g2;
+    const float zr = i < m ? (float)rhs : 1.f, zi = rsqrtf(zr);
+    eval_system<C, float, true>(sm, m, n, hs, slack, qstep, jstride, amax, amin, w_own, ds_own, i < m ? zi : 0.f, g, g2, fr);
+    if (given) { g = gg.x; g2 = gg.y; }
+    if (chol) {
+        // an outer block's function is constant along (1,...,1): that direction is pinned with 1/m everywhere
+        const float add = slack ? 0.f : 1.f / (float)m;
+        if (tid < C::MP) {
+            sm.yv[i] = i < m ? newton_rhs(g, g2, rhs) : 0.f;
+            sm.dg[i] = i < m ? (float)(g - g2) + add : 1.f;
+            sm.wf[i] = zr * zi;                                // undoes the operands' scale
+        }
+        __syncthreads();
+        factor<C>(sm, fr, m, add);
+    } else {
+        // (a diagonal that is not positive gives NaN, which the solve reports)
+        if (tid < C::MP) {
+            const float rd = i < m ? rsqrtf((float)(g - g2)) : 1.f;
+            sm.dg[i] = rd;
+            sm.wf[i] = zr * zi * rd;
+        }
+        __syncthreads();
+        const int ra = warp % C::kPr, rb = C::MP / 16 - 1 - ra, cs = warp / C::kPr;
+        GR_PTR(__half) N = sm.pi;
+        // the lower triangle (and what the diagonal tiles hold beyond it) out of the fragments ...
+        auto put = [&](const float* v, int rt, int ni) {
+            const int c0 = 8 * ni + 2 * tig, r0 = 16 * rt + gid;
+            const float2 sc = ld_f2(sm.wf + c0);
+            const float s0 = sm.wf[r0], s1 = sm.wf[r0 + 8];
+            GR_PTR(__half) q = N + r0 * C::kNS + c0;
+            st_h2(q, pack_half(v[0] * s0 * sc.x, v[1] * s0 * sc.y));
+            st_h2(q + 8 * C::kNS, pack_half(v[2] * s1 * sc.x, v[3] * s1 * sc.y));           // (eight rows further)
+        };
+#pragma unroll
+        for (int s = 0; s < C::kNB; s++) {
+            const int ni = cs + s * C::kS;
+            if (s < C::kNA && ni <= 2 * ra + 1) put(fr.A[s < C::kNA ? s : 0], ra, ni);
+            if (ni <= 2 * rb + 1) put(fr.B[s], rb, ni);
+        }
+        __syncthreads();
+        // ... and every row's upper part out of its column (eight entries at a time; what other threads rewrite meanwhile in
+        // the lower triangle does not change)
+#pragma unroll 2
+        for (int c = tid / C::MP; c < C::MP / 8; c += C::kNG) {
+            GR_PTR(__half) own = N + i * C::kNS + 8 * c;
+            const uint4 o = ld_h8(own);
+            const uint32_t ov[4] = {o.x, o.y, o.z, o.w};
+            uint32_t nv[4];
+#pragma unroll
+            for (int z = 0; z < 4; z++) {
+                const int l = 8 * c + 2 * z;
+                const uint32_t t0 = __half_as_ushort(N[l * C::kNS + i]), t1 = __half_as_ushort(N[(l + 1) * C::kNS + i]);
+                const uint32_t e0 = l == i ? 0u : (l > i ? t0 : (ov[z] & 0xffffu));
+                const uint32_t e1 = l + 1 == i ? 0u : (l + 1 > i ? t1 : (ov[z] >> 16));
+                nv[z] = e0 | (e1 << 16);
+            }
+            st_h8(own, make_uint4(nv[0], nv[1], nv[2], nv[3]));
+        }
+        __syncthreads();
+    }
+    double2 r; r.x = g; r.y = g2;
+    return r;
+}
+
+// sums of up to three values over the token threads
+template <class C, int K>
+__device__ __forceinline__ void tok_sums(const FSm<C>& sm, float* v, int& par)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int k = 0; k < K; k++) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    }
+    if (C::T == 32) return;
+    GR_PTR(float) r = GR_PCAST(float, sm.red + 32 * par);
+    par ^= 1;
+    if ((threadIdx.x & 31) == 0 && (threadIdx.x >> 5) < C::kTW)
+        st_f4(r + 4 * (threadIdx.x >> 5), make_float4(v[0], K > 1 ? v[K > 1 ? 1 : 0] : 0.f, K > 2 ? v[K > 2 ? 2 : 0] : 0.f, 0.f));
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < C::kTW; w++) {
+        const float4 t = ld_f4(r + 4 * w);
+        const float tv[3] = {t.x, t.y, t.z};
+#pragma unroll
+        for (int k = 0; k < K; k++) v[k] = w == 0 ? tv[k] : v[k] + tv[k];
+    }
+}
+
+// Newton step by conjugate gradients on the scaled Hessian: this thread's component of the step, or NaN when the residual
+// did not fall by `rtol` in kFCgMax iterations.  Off the heavy-weight regime the scaled Hessian has all its eigenvalues
+// within 0.8 - 1.5 but one, so four or five iterations give four digits: 2 k cycles against 18 k for a 50 x 50
+// factorisation with its substitutions.  One thread per row, the row in registers; one reduction per iteration
+// (Chronopoulos and Gear's form).
+// The one eigenvalue is the common scale of the weights, the direction (1,...,1): H 1 = s, s_i = g2_i / w_i the rate at
+// which token i takes mass from the slack, tiny when the acceptance is close to one.  s is known exactly, so the diagonal
+// is set from the row sums, s_i + sum_l |H_il| (whatever the rounding of the off-diagonal part, the matrix then has the
+// right action on that direction), and the direction itself is deflated: the iteration works on
+// (I - s 1^T / sum s) H, and the step gets `shift`, the caller's answer for the common scale, less s . y / sum s.
+// (kap = -1 / sum s, lin = sum rhs / sum s.)
+// An outer block (slack == 0) has s = 0: the matrix is singular along the direction, e e^T / (e . e) is added, e = sqrt(H_ii)
+// (kap = 1 / (e . e), lin = 0).
+template <class C>
+__device__ __noinline__ float cg_solve(int m, int slack, float rhs, float s_own, float kap, float lin, float shift, float rtol,
+                                       int* flag)
+{
+    constexpr int kCol = C::MP / C::kNG;                        // columns of this copy
+    const FSm<C> sm(flag);
+    const int tid = threadIdx.x, i = tid % C::MP, ng = tid / C::MP;
+    int par = 0;
+    const float sd = sm.dg[i];
+    float row[kCol];
+    {
+        GR_PTR(const __half) np = sm.pi + i * C::kNS + ng * kCol;
+#pragma unroll
+        for (int c = 0; c < kCol; c += 8) {
+            const uint4 v = ld_h8(np + c);
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int z = 0; z < 4; z++) {
+                const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[z]));
+                row[c + 2 * z] = f.x; row[c + 2 * z + 1] = f.y;
+            }
+        }
+    }
+    const bool on = i < m;
+    GR_PTR(float) part = GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oSP), C::T, flag);
+    // N times the vector in `vec` (the caller has written its own entry)
+    auto times_n = [&](GR_PTR(float) vec) {
+        __syncthreads();
+        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll
+        for (int c = 0; c < kCol; c += 4) {
+            const float4 v = ld_f4(vec + ng * kCol + c);
+            a0 = fmaf(row[c], v.x, a0); a1 = fmaf(row[c + 1], v.y, a1); a2 = fmaf(row[c + 2], v.z, a2); a3 = fmaf(row[c + 3], v.w, a3);
+        }
+        float nv = (a0 + a1) + (a2 + a3);
+        if (C::kNG > 1) {
+            part[tid] = nv;
+            __syncthreads();
+            nv = 0.f;
+#pragma unroll
+            for (int k = 0; k < C::kNG; k++) nv += part[k * C::MP + i];
+        }
+        return nv;
+    };
+    // diagonal from the row sums; v: the deflated (slack) or added (outer block) direction, kap its factor
+    const float sdi = on ? __fdividef(1.f, sd) : 0.f;
+    if (ng == 0) sm.yv[i] = sdi;
+    const float nrow = times_n(sm.yv);
+    const float si = on && slack ? s_own : 0.f;
+    const float diag = on ? sd * fmaf(si, sd, nrow) : 1.f;
+    const float v = slack ? si * sd : sdi;
+    float r = on ? rhs * sd : 0.f, x = 0.f, p = 0.f, s = 0.f;
+    r = fmaf(-lin, v, r);
+    float gam_old = 0.f, al_old = 0.f, goal = 0.f;
+    bool done = false;
+#pragma unroll 1
+    for (int it = 0; it <= kFCgMax; it++) {
+        GR_PTR(float) vec = (it & 1) ? sm.yv : sm.dl;            // two buffers in turn
+        if (ng == 0) vec[i] = r;
+        float w = fmaf(diag, r, -times_n(vec));
+        float d[3] = {r * r, r * w, v * r};
+        tok_sums<C, 3>(sm, d, par);
+        w = fmaf(v, kap * d[2], w);
+        d[1] = fmaf(d[2] * d[2], kap, d[1]);
+        const float gam = d[0];
+        if (it == 0) goal = gam * rtol * rtol;
+        if (gam <= goal) { done = true; break; }
+        const float beta = it == 0 ? 0.f : __fdividef(gam, gam_old);
+        const float al = __fdividef(gam, it == 0 ? d[1] : d[1] - beta * __fdividef(gam, al_old));
+        p = fmaf(beta, p, r); s = fmaf(beta, s, w);
+        x = fmaf(al, p, x); r = fmaf(-al, s, r);
+        gam_old = gam; al_old = al;
+    }
+    float y = x * sd;
+    if (slack) {
+        float sy[1] = {si * y};
+        tok_sums<C, 1>(sm, sy, par);
+        y += shift + kap * sy[0];
+    }
+    __syncthreads();
+    // (not positive definite, NaN or slow: NaN)
+    return done ? y : __int_as_float(0x7fc00000);
+}
+
+// One system: m tokens at support positions ord[0 .. m) (draft mass ascending), draft mass above the block.
+struct System { int m, slack; double hmass; };
+
+// Starting point (log-weight of this thread's token): token i wins the share w_i / (slack + w_i + S_i) of the tuples that contain it, S_i = the
+// weight it is up against.  A competitor j, present with probability pi_ij = Pr[i and j drafted] / Pr[i drafted],
+// adds to S_i the weight e_j for which 1 / (A + e_j) = (1 - pi_ij) / A + pi_ij / (A + w_j), A = slack + w_i + S_i:
+// e_j = A pi_ij / (A / w_j + 1 - pi_ij).  For w_j << A this is the mean-field value pi_ij w_j; a huge w_j counts for
+// A pi_ij / (1 - pi_ij) only (token i simply loses the tuples that contain j).  fp32: it is a starting point.
+template <class C>
+__device__ __noinline__ double start_point(int m, int slack, int n, double d_i, double rhs_i, double Tm,
+                                           int* flag)
+{
+    const FSm<C> sm(flag);
+    const int tid = threadIdx.x, i = tid % C::MP, ng = tid / C::MP;
+    const bool on = i < m, lead = ng == 0;
+    int par = 0;
+    // masses relative to the system's total: token avoided / a pair avoided, (1 - d_i / T)^n and (1 - (d_i + d_j) / T)^n
+    const double iT = m_div(1.0, Tm);
+    const float fn = (float)n, rel = (float)(d_i * iT);
+    const double col_d = on ? ipow(fmax(1.0 - d_i * iT, 0.0), n) : 0.0;
+    const float col = (float)col_d, ci = on ? (float)(1.0 - col_d) : 1.f, ic = __fdividef(1.f, ci);   // ci: Pr[token i drafted]
+    const float rho = on ? fminf((float)(rhs_i * ipow(iT, n)) * ic, 0.999f) : 0.5f;
+    const float odds = __fdividef(rho, 1.f - rho);
+    float wi = slack ? odds : (on ? __fdividef((float)rhs_i, (float)d_i) : 1.f);
+    // a rarely drafted token: Pr[j drafted | i drafted] tends to 1 - (1 - d_j / T)^(n - 1)
+    const bool rare = ci < 0.02f;
+    const float pres = 1.f - (rel < 1.f ? __fdividef(col, 1.f - rel) : 0.f);
+    RSm<C, float> rf(sm);
+    GR_PTR(float) tab = rf.SP;
+    if (lead) { st_f4(tab + 4 * i, make_float4(rel, col, pres, 0.f)); sm.wf[i] = __fdividef(1.f, wi); }
+    __syncthreads();
+    // (eight columns at a time: their chains overlap; columns beyond m hold 0)
+    GR_PTR(__half) prow = sm.pi + i * C::kNS;
+    const int nc = (m + 7) >> 3;
+    if ((i & ~31) < m) {
+#pragma unroll 1
+        for (int c = ng; c < nc; c += C::kNG) {
+            uint32_t pk[4];
+#pragma unroll
+            for (int z = 0; z < 4; z++) {
+                float pv[2];
+#pragma unroll
+                for (int y = 0; y < 2; y++) {
+                    const int j = 8 * c + 2 * z + y;
+                    const float4 tj = ld_f4(tab + 4 * j);
+                    const float both = ex2_approx(fn * __log2f(fmaxf(1.f - rel - tj.x, 0.f)));
+                    const float pij = rare ? tj.z : (1.f - col - tj.y + both) * ic;
+                    pv[y] = (j == i || j >= m) ? 0.f : fminf(fmaxf(pij, 0.f), 1.f);
+                }
+                const __half2 h = __floats2half2_rn(pv[0], pv[1]);
+                pk[z] = *reinterpret_cast<const uint32_t*>(&h);
+            }
+            st_h8(prow + 8 * c, make_uint4(pk[0], pk[1], pk[2], pk[3]));
+        }
+    }
+    __syncthreads();
+    float A = (slack ? 1.f : 0.f) + wi;
+    GR_PTR(float) part = GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oSP), C::T, sm.flag);
+#pragma unroll 1
+    for (int sweep = 0; sweep < kFSweeps; sweep++) {
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        if ((i & ~31) < m) {
+#pragma unroll 2
+            for (int c = ng; c < nc; c += C::kNG) {
+                const uint4 pk = ld_h8(prow + 8 * c);
+                const float4 w0 = ld_f4(sm.wf + 8 * c), w1 = ld_f4(sm.wf + 8 * c + 4);
+                const uint32_t u[4] = {pk.x, pk.y, pk.z, pk.w};
+                const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
 #pragma unroll
                 for (int z = 0; z < 4; z++) {
-                    const float hi = to_tf32(fa[z]);
-                    ah[z] = __float_as_uint(hi); al[z] = __float_as_uint(to_tf32(fa[z] - hi));
-                }
-#pragma unroll
-                for (int z = 0; z < 2; z++) {
-                    const float hi = to_tf32(fb[z]);
-                    bh[z] = __float_as_uint(hi); bl[z] = __float_as_uint(to_tf32(fb[z] - hi));
-                }
-                mma_tf32(c0, c1, c2, c3, al[0], al[1], al[2], al[3], bh[0], bh[1]);
-                mma_tf32(c0, c1, c2, c3, ah[0], ah[1], ah[2], ah[3], bl[0], bl[1]);
-                mma_tf32(c0, c1, c2, c3, ah[0], ah[1], ah[2], ah[3], bh[0], bh[1]);
-            } else {
-                mma_tf32(c0, c1, c2, c3, __float_as_uint(fa[0]), __float_as_uint(fa[1]), __float_as_uint(fa[2]),
-                         __float_as_uint(fa[3]), __float_as_uint(fb[0]), __float_as_uint(fb[1]));
-            }
-        }
-        GR_PTR(float) J0 = sm.Jacc + ((i0 + gid) * kJS + l0 + 2 * tig);
-        J0[0] += c0; J0[1] += c1;
-        J0[8 * kJS] += c2; J0[8 * kJS + 1] += c3;
-    }
-}
-
-// g (always), and with want_jac the diagonal part g2 and the contraction Jacc, at the weights in sm.w.
-// The contraction takes every jstride-th node (weights scaled by jstride).
-// Node abscissae / weights are in sm.tq / sm.cq, their number in sm.scal[SC_Q].
-template <int NT, int TPL>
-__device__ void fast_eval(const FSm& sm, int m, int n, GR_PTR(const double) d, double hmass, bool want_jac, int jstride)
-{
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, KP = sm.KP;
-    const int Q = (int)sm.scal[SC_Q];
-    double wr[TPL], dr[TPL], gacc[TPL], g2acc[TPL];
-#pragma unroll
-    for (int tt = 0; tt < TPL; tt++) {
-        const int j = lane + 32 * tt;
-        wr[tt] = j < m ? sm.w[j] : 0.0;
-        dr[tt] = j < m ? d[j] : 0.0;
-        gacc[tt] = 0.0; g2acc[tt] = 0.0;
-    }
-    if (want_jac) {
-        for (int e = tid; e < kMP * kJS; e += kFT) sm.Jacc[e] = 0.f;
-    }
-    const int span = jstride * kJC;      // nodes per chunk: every jstride-th one is a Hessian node
-    for (int q0 = 0; q0 < Q; q0 += span) {
-        const int q1 = min(Q, q0 + span);
-        for (int q = q0 + warp; q < q1; q += kFW) {
-            const double t = sm.tq[q];
-            double S[NT];
-#pragma unroll
-            for (int c = 0; c < NT; c++) S[c] = 0.0;
-            double xk[TPL];
-#pragma unroll
-            for (int tt = 0; tt < TPL; tt++) {
-                const double x = exp_neg(t * wr[tt]);
-                xk[tt] = x;
-                double hh[NT + 1];
-                unit_h_series<NT>(x, hh);
-                // h[c] = d^c hh[c];  S[0] += x d,  S[c] += x (1 - x) d h[c]
-                const double dd = dr[tt];
-                S[0] = fma(x, dd, S[0]);
-                double pw = x * (1.0 - x) * dd;
-#pragma unroll
-                for (int c = 1; c < NT; c++) {
-                    pw *= dd;
-                    S[c] = fma(pw, hh[c], S[c]);
-                }
-            }
-            // log-derivative of the product: sum over the tokens (all lanes end with the totals)
-            warp_allreduce_series<NT>(S, lane);
-            S[0] += hmass;
-            // P' = S P, column-oriented
-            double P[NT + 1], acc[NT + 1];
-            P[0] = 1.0;
-#pragma unroll
-            for (int c = 1; c <= NT; c++) acc[c] = 0.0;
-#pragma unroll
-            for (int k = 0; k < NT; k++) {
-#pragma unroll
-                for (int c = k + 1; c <= NT; c++) acc[c] = fma(S[c - 1 - k], P[k], acc[c]);
-                P[k + 1] = acc[k + 1] * (1.0 / (double)(k + 1));
-            }
-            // R[c] = P[n - c]: the coefficient that pairs with h[c] in [lambda^n] P h
-            // (for n < NT: the reversed series moved down by NT - n places, one conditional move per bit)
-            double R[NT + 1];
-#pragma unroll
-            for (int c = 1; c <= NT; c++) R[c] = P[NT - c];
-            if (n != NT) {
-                const int sh = NT - n;
-#pragma unroll
-                for (int bit = NT / 2; bit >= 1; bit >>= 1) {
-                    if (sh & bit) {
-#pragma unroll
-                        for (int c = 1; c <= NT; c++) R[c] = (c + bit <= NT) ? R[c + bit] : 0.0;
-                    }
-                }
-            }
-            const double cq = sm.cq[q];
-            const bool jnode = want_jac && ((q - q0) % jstride == 0);
-            const int slot = (q - q0) / jstride;
-#pragma unroll
-            for (int tt = 0; tt < TPL; tt++) {
-                double hh[NT + 1], hd[NT + 1];
-                unit_h_series<NT>(xk[tt], hh);
-                const double dd = dr[tt];
-                double pw = 1.0, val = 0.0;
-#pragma unroll
-                for (int c = 1; c <= NT; c++) {
-                    pw *= dd;
-                    hd[c] = pw * hh[c];                 // h[c] = d^c hh[c]
-                    val = fma(R[c], hd[c], val);
-                }
-                const double u = wr[tt] * xk[tt];
-                const double gi = cq * u * val;
-                gacc[tt] += gi;
-                g2acc[tt] = fma(gi * t, wr[tt], g2acc[tt]);
-                if (jnode) {
-                    // A = P h (series), paired as  sum_kappa A[n - kappa] h_l[kappa],  kappa = 1..n-1.
-                    // Staged scaled: AS = 2 c_q t u A[n - kappa] (the 2: every second node), HS = u h[kappa].
-                    // Row kappa - 1 of the node's slot holds the pair (A[n - kappa], h[kappa]); rows n - 1 .. NT - 1
-                    // are zero (they pad the contraction length to a multiple of the MMA depth).
-                    const int j = lane + 32 * tt;
-                    const double sa = (double)jstride * cq * t * u;
-                    GR_PTR(float) as = sm.AS + (slot * NT * kMS + j);
-                    GR_PTR(float) hs = sm.HS + (slot * NT * kMS + j);
-                    if (n == NT) {
-                        // full series length: fixed rows, each A consumed as soon as it is formed
-#pragma unroll
-                        for (int kap = 1; kap < NT; kap++) {
-                            double a = 0.0;              // A[NT - kap] = sum_c h[c] P[NT - kap - c]
-#pragma unroll
-                            for (int c = 1; c <= NT - kap; c++) a = fma(hd[c], P[NT - kap - c], a);
-                            as[(kap - 1) * kMS] = stage_round<NT>((float)(sa * a));
-                            hs[(kap - 1) * kMS] = stage_round<NT>((float)(u * hd[kap]));
-                            if (TPL == 1) { as[(kap - 1) * kMS + 32] = 0.f; hs[(kap - 1) * kMS + 32] = 0.f; }
-                        }
-                        as[(NT - 1) * kMS] = 0.f; hs[(NT - 1) * kMS] = 0.f;
-                        if (TPL == 1) { as[(NT - 1) * kMS + 32] = 0.f; hs[(NT - 1) * kMS + 32] = 0.f; }
-                    } else {
-#pragma unroll
-                        for (int e2 = 1; e2 < NT; e2++) {
-                            double a = 0.0;              // A[e2] = sum_{c=1..e2} h[c] P[e2 - c]
-#pragma unroll
-                            for (int c = 1; c <= e2; c++) a = fma(hd[c], P[e2 - c], a);
-                            if (e2 < n) as[(n - e2 - 1) * kMS] = stage_round<NT>((float)(sa * a));
-                        }
-#pragma unroll
-                        for (int kap = 1; kap <= NT; kap++) {
-                            const bool live = kap < n;
-                            if (!live) as[(kap - 1) * kMS] = 0.f;
-                            hs[(kap - 1) * kMS] = live ? stage_round<NT>((float)(u * hd[kap])) : 0.f;
-                            if (TPL == 1) { as[(kap - 1) * kMS + 32] = 0.f; hs[(kap - 1) * kMS + 32] = 0.f; }
-                        }
-                    }
+                    const float2 pv = __half22float2(*reinterpret_cast<const __half2*>(&u[z]));
+                    acc[z] += __fdividef(pv.x, fmaf(A, wv[2 * z], 1.f - pv.x));
+                    acc[z] += __fdividef(pv.y, fmaf(A, wv[2 * z + 1], 1.f - pv.y));
                 }
             }
         }
-        if (want_jac) {
-            const int nstaged = (q1 - q0 + jstride - 1) / jstride;
-            int K8 = nstaged * NT;
-            if (K8 & 7) {
-                // NT = 4 with an odd number of staged nodes: one more all-zero slot completes the MMA depth
-                for (int e = tid; e < NT * kMS; e += kFT) { sm.AS[K8 * kMS + e] = 0.f; sm.HS[K8 * kMS + e] = 0.f; }
-                K8 += NT;
-            }
+        float Si = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+        if (C::kNG > 1) {
+            part[tid] = Si;
             __syncthreads();
-            hess_chunk<(NT > 8)>(sm, K8, m);
-            __syncthreads();
+            Si = 0.f;
+#pragma unroll
+            for (int k = 0; k < C::kNG; k++) Si += part[k * C::MP + i];
         }
-    }
-#pragma unroll
-    for (int tt = 0; tt < TPL; tt++) {
-        const int j = lane + 32 * tt;
-        if (j < m) { sm.gw[warp * KP + j] = gacc[tt]; sm.g2w[warp * KP + j] = g2acc[tt]; }
-    }
-    __syncthreads();
-    if (tid < m) {
-        double a = 0.0, b2 = 0.0;
-#pragma unroll
-        for (int w2 = 0; w2 < kFW; w2++) { a += sm.gw[w2 * KP + tid]; b2 += sm.g2w[w2 * KP + tid]; }
-        sm.g[tid] = a; sm.g2[tid] = b2;
-    }
-    __syncthreads();
-}
-
-// w = exp(alpha), its range, and the quadrature grid for it.
-static __device__ void fast_grid(const FSm& sm, int m, int n, int slack, double qstep)
-{
-    const int tid = threadIdx.x;
-    GR_PTR(double) red = sm.scal + SC_GRID;
-    double a = 0.0;
-    if (tid < m) { a = sm.alpha[tid]; sm.w[tid] = exp(a); }
-    // extreme alphas in one pass (they give the extreme weights)
-    double hi = tid < m ? a : -1.0e300, lo = tid < m ? -a : -1.0e300;
-    for (int o = 16; o > 0; o >>= 1) {
-        hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-        lo = fmax(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-    }
-    __syncthreads();
-    if ((tid & 31) == 0) { red[2 * (tid >> 5)] = hi; red[2 * (tid >> 5) + 1] = lo; }
-    __syncthreads();
-    hi = red[0]; lo = red[1];
-#pragma unroll
-    for (int i = 1; i < kFW; i++) { hi = fmax(hi, red[2 * i]); lo = fmax(lo, red[2 * i + 1]); }
-    lo = -lo;
-    const double wmax = exp(hi), wmin = exp(lo);
-    const double rate = slack ? 1.0 + wmin : wmin;
-    const double s_hi = log(kFTEnd / rate);
-    const double s0 = -log((slack ? 1.0 : 0.0) + wmax) - kFDrop;
-    int Q = (int)ceil((s_hi - (s0 - kFTail)) / qstep) + 1;
-    if (Q > kFMaxNodes) Q = kFMaxNodes;
-    double nfact = 1.0;
-    for (int c = 2; c <= n; c++) nfact *= (double)c;
-    for (int q = tid; q < Q; q += kFT) {
-        const double s = s_hi - qstep * (double)q;
-        const double e = exp(-(s - s0));
-        const double t = exp(s - e);
-        sm.tq[q] = t;
-        sm.cq[q] = qstep * (1.0 + e) * t * (slack ? exp(-t) : 1.0) * nfact;
-    }
-    if (tid == 0) sm.scal[SC_Q] = (double)Q;
-    __syncthreads();
-}
-
-// Newton step: fp32 Cholesky of the Hessian in place in the contraction accumulator (row stride kJS),
-// with the forward substitution carried along and the backward substitution on warp 0.  The step only
-// steers the iteration (the fp64 gradient decides convergence) and the Hessian was accumulated in fp32.
-// Matrix: off-diagonal -Jacc (lower triangle), diagonal g - g2, plus `add` everywhere.  Writes the step
-// into sm.delta; sets SC_FAIL when a pivot is not positive.
-static __device__ void fast_newton_step(const FSm& sm, int m, GR_PTR(const double) rhs, double add)
-{
-    const int tid = threadIdx.x;
-    GR_PTR(float) Jm = sm.Jacc;
-    GR_PTR(float) yv = GR_PCAST(float, sm.J);          // [kMP] working right-hand side
-    GR_PTR(float) yf = yv + kMP;                       // [kMP] forward-substituted right-hand side, then the solution
-    GR_PTR(float) dg = yf + kMP;                       // [kMP] diagonal of the factor
-    const float addf = (float)add;
-    for (int e = tid; e < m * kMP; e += kFT) {
-        const int i = e / kMP, l = e & (kMP - 1);
-        if (l < i) Jm[i * kJS + l] = addf - Jm[i * kJS + l];
-    }
-    if (tid < m) {
-        Jm[tid * kJS + tid] = (float)(sm.g[tid] - sm.g2[tid]) + addf;
-        // Right-hand side.  Along its own coordinate a token's flow behaves like a logistic curve
-        // g_i = c sigma(alpha_i - kappa): linear in w_i while the token is light, saturating at the flow c of the
-        // tuples it can win at all once it is heavy.  The curve through the current value and slope
-        // (H_ii = g_i (1 - g_i / c)  gives  c = g_i^2 / g2_i)  is inverted exactly:  H_ii (logit(rhs_i / c) -
-        // logit(g_i / c))  replaces  rhs_i - g_i.  Near the solution the two agree to first order; far from it a
-        // token close to saturation (weight in the thousands) is placed at once, where the plain residual moves
-        // its weight by a factor e per step, and a light token gets the multiplicative update log(rhs_i / g_i).
-        const double gi = sm.g[tid], g2i = sm.g2[tid], ri = rhs[tid];
-        // (a target at or beyond the saturation level this curve predicts says that the curve is off: the plain
-        // residual is used for that token; without this a single token of weight ~1e5 crawled for 40 steps)
-        const double room = 1.0 - ri * g2i / (gi * gi);
-        const double arg = fmax((ri - gi) / (gi * fmax(room, 1e-3)), -1.0 + 1e-12);
-        yv[tid] = (float)(room > 1e-3 ? (gi - g2i) * log1p(arg) : ri - gi);
-    }
-    __syncthreads();
-    bool bad = false;
-    // Blocked right-looking factorisation in panels of eight columns: every thread factors the 8 x 8 diagonal block
-    // in registers (redundantly: no exchange needed), one thread per row solves the panel below it and carries the
-    // forward substitution along, and the rest of the matrix takes the panel's rank-8 update on the tensor cores.
-    for (int j0 = 0; j0 < m; j0 += 8) {
-        const int nb = min(8, m - j0);
-        float Lb[8][8], yb[8], dinv[8];
-#pragma unroll
-        for (int c = 0; c < 8; c++) {
-#pragma unroll
-            for (int c2 = 0; c2 <= c; c2++) Lb[c][c2] = (c < nb) ? Jm[(j0 + c) * kJS + j0 + c2] : (c == c2 ? 1.f : 0.f);
-            yb[c] = (c < nb) ? yv[j0 + c] : 0.f;
-        }
-#pragma unroll
-        for (int c = 0; c < 8; c++) {
-            const float dv = Lb[c][c];
-            if (!(dv > 0.f)) bad = true;
-            dinv[c] = rsqrtf(dv);
-            Lb[c][c] = dv * dinv[c];
-            yb[c] *= dinv[c];
-#pragma unroll
-            for (int r2 = c + 1; r2 < 8; r2++) Lb[r2][c] *= dinv[c];
-#pragma unroll
-            for (int r2 = c + 1; r2 < 8; r2++) {
-#pragma unroll
-                for (int c3 = c + 1; c3 <= r2; c3++) Lb[r2][c3] = fmaf(-Lb[r2][c], Lb[c3][c], Lb[r2][c3]);
-                yb[r2] = fmaf(-Lb[r2][c], yb[c], yb[r2]);
-            }
-        }
-        if (bad) break;
-        // panel below the block: one row per thread (it touches no entry of the block itself)
-        const int i1 = j0 + nb + tid;
-        if (i1 < m) {
-            float v[8];
-#pragma unroll
-            for (int c = 0; c < 8; c++) v[c] = (c < nb) ? Jm[i1 * kJS + j0 + c] : 0.f;
-            float yi = yv[i1];
-#pragma unroll
-            for (int c = 0; c < 8; c++) {
-                const float lc = v[c] * dinv[c];
-#pragma unroll
-                for (int c3 = c + 1; c3 < 8; c3++) v[c3] = fmaf(-lc, Lb[c3][c], v[c3]);
-                yi = fmaf(-lc, yb[c], yi);
-                if (c < nb) Jm[i1 * kJS + j0 + c] = lc;
-            }
-            yv[i1] = yi;
+        Si *= A;
+        if (on) {
+            wi = odds * (slack ? 1.f + Si : fmaxf(Si, 1e-30f));
+            A = (slack ? 1.f : 0.f) + wi + Si;
         }
         __syncthreads();
-        // every thread has read the block by now: one of them stores its factor
-        if (tid == kFT - 1) {
-#pragma unroll
-            for (int c = 0; c < 8; c++) {
-                if (c < nb) {
-                    dg[j0 + c] = Lb[c][c]; yf[j0 + c] = yb[c];
-#pragma unroll
-                    for (int c2 = 0; c2 < c; c2++) Jm[(j0 + c) * kJS + j0 + c2] = Lb[c][c2];
-                }
-            }
-        }
-        // trailing update  J[i][l] -= sum_c L[i][c] L[l][c],  j0 + 8 <= l <= i:  m16n8k8 MMAs on the 16 x 8 tiles of
-        // the lower triangle, operands split into two tf32 parts (~fp32 products)
-        const int t0 = j0 + 8;
-        if (t0 < m) {
-            const int lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tig = lane & 3;
-            // tile t of the lower triangle: row mi of 16-row tiles holds tiles mi (mi + 1) .. (mi + 1)(mi + 2) - 1
-            // (2 mi + 2 of them); each warp takes every kFW-th tile and finds (mi, ni) from t directly
-            const int nmt = (m - t0 + 15) >> 4;
-            for (int t = warp; t < nmt * (nmt + 1); t += kFW) {
-                int mi = (int)((sqrtf((float)(4 * t + 1)) - 1.f) * 0.5f);
-                while (mi * (mi + 1) > t) mi--;
-                while ((mi + 1) * (mi + 2) <= t) mi++;
-                const int ni = t - mi * (mi + 1);
-                {
-                    if (t0 + 8 * ni >= m) continue;
-                    const int ra = t0 + 16 * mi + gid, rb = ra + 8, l0 = t0 + 8 * ni, cb = l0 + gid;
-                    const bool oa = ra < m, ob = rb < m, oc = cb < m;
-                    const float fa[4] = {oa ? -Jm[ra * kJS + j0 + tig] : 0.f, ob ? -Jm[rb * kJS + j0 + tig] : 0.f,
-                                         oa ? -Jm[ra * kJS + j0 + tig + 4] : 0.f, ob ? -Jm[rb * kJS + j0 + tig + 4] : 0.f};
-                    const float fb[2] = {oc ? Jm[cb * kJS + j0 + tig] : 0.f, oc ? Jm[cb * kJS + j0 + tig + 4] : 0.f};
-                    GR_PTR(float) C0 = Jm + (ra * kJS + l0 + 2 * tig);
-                    GR_PTR(float) C1 = Jm + (rb * kJS + l0 + 2 * tig);
-                    float c0 = oa ? C0[0] : 0.f, c1 = oa ? C0[1] : 0.f, c2 = ob ? C1[0] : 0.f, c3 = ob ? C1[1] : 0.f;
-                    uint32_t ah[4], al[4], bh[2], bl[2];
-#pragma unroll
-                    for (int z = 0; z < 4; z++) {
-                        const float hi = to_tf32(fa[z]);
-                        ah[z] = __float_as_uint(hi); al[z] = __float_as_uint(to_tf32(fa[z] - hi));
-                    }
-#pragma unroll
-                    for (int z = 0; z < 2; z++) {
-                        const float hi = to_tf32(fb[z]);
-                        bh[z] = __float_as_uint(hi); bl[z] = __float_as_uint(to_tf32(fb[z] - hi));
-                    }
-                    // three independent accumulations (the small cross terms apart), summed afterwards
-                    float e0 = 0.f, e1 = 0.f, e2 = 0.f, e3 = 0.f, f0 = 0.f, f1 = 0.f, f2 = 0.f, f3 = 0.f;
-                    mma_tf32(e0, e1, e2, e3, al[0], al[1], al[2], al[3], bh[0], bh[1]);
-                    mma_tf32(f0, f1, f2, f3, ah[0], ah[1], ah[2], ah[3], bl[0], bl[1]);
-                    mma_tf32(c0, c1, c2, c3, ah[0], ah[1], ah[2], ah[3], bh[0], bh[1]);
-                    if (oa) { C0[0] = c0 + (e0 + f0); C0[1] = c1 + (e1 + f1); }
-                    if (ob) { C1[0] = c2 + (e2 + f2); C1[1] = c3 + (e3 + f3); }
-                }
-            }
-        }
+        if (lead && on) sm.wf[i] = __fdividef(1.f, wi);
         __syncthreads();
     }
-    if (bad) {
-        if (tid == 0) sm.scal[SC_FAIL] = 1.0;
-        __syncthreads();
-        return;
-    }
-    // backward substitution L^T x = y on warp 0, column-oriented with the right-hand side in registers (lane l holds
-    // entries l, l + 32, ...): unknown e is finished by its owner, broadcast, and taken out of the entries above it.
-    // One multiply, one shuffle and one FMA per unknown on the critical path; row e of L is fetched one step ahead.
-    if (tid < 32 && kRL == 2) {
-        // (two entries per lane, written out: the general form below compiles to slower code for them)
-        const int lane = tid;
-        float y0 = lane < m ? yf[lane] : 0.f, y1 = lane + 32 < m ? yf[lane + 32] : 0.f;
-        const float r0 = lane < m ? 1.f / dg[lane] : 0.f, r1 = lane + 32 < m ? 1.f / dg[lane + 32] : 0.f;
-        float a0n = Jm[(m - 1) * kJS + lane], a1n = Jm[(m - 1) * kJS + lane + 32];
-        for (int e = m - 1; e >= 0; e--) {
-            const float a0 = a0n, a1 = a1n;
-            if (e > 0) { a0n = Jm[(e - 1) * kJS + lane]; a1n = Jm[(e - 1) * kJS + lane + 32]; }
-            const float xe = __shfl_sync(0xffffffffu, (e & 32) ? y1 * r1 : y0 * r0, e & 31);
-            if (lane == (e & 31)) {
-                if (e & 32) y1 = xe; else y0 = xe;
-            }
-            if (lane < e) y0 = fmaf(-a0, xe, y0);
-            if (lane + 32 < e) y1 = fmaf(-a1, xe, y1);
-        }
-        if (lane < m) yf[lane] = y0;
-        if (lane + 32 < m) yf[lane + 32] = y1;
-    }
-    if (kRL != 2) {
-        // Wider supports: blocked, eight unknowns at a time from the last panel down.  Every thread keeps its own entry
-        // of the right-hand side in a register; the block's eight entries go through shared memory (two buffers in
-        // turn, one barrier per block), every thread solves the 8 x 8 triangle redundantly and takes the block's
-        // unknowns out of its own entry.  About 350 cycles per block, where the one-warp form above spent over 400
-        // per unknown at four entries per lane.
-        float yl = tid < m ? yf[tid] : 0.f;
-        int buf = 0;
-        for (int j0 = ((m - 1) >> 3) << 3; j0 >= 0; j0 -= 8) {
-            const int nb = min(8, m - j0);
-            GR_PTR(float) yb = yv + 8 * buf;
-            if (tid >= j0 && tid < j0 + nb) yb[tid - j0] = yl;
-            __syncthreads();
-            float x[8];
-#pragma unroll
-            for (int c = 7; c >= 0; c--) {
-                float v = 0.f;
-                if (c < nb) {
-                    v = yb[c];
-#pragma unroll
-                    for (int c2 = 7; c2 > c; c2--)
-                        if (c2 < nb) v = fmaf(-Jm[(j0 + c2) * kJS + j0 + c], x[c2], v);
-                    v = v / dg[j0 + c];
-                }
-                x[c] = v;
-            }
-            if (tid < j0) {
-#pragma unroll
-                for (int c = 0; c < 8; c++)
-                    if (c < nb) yl = fmaf(-Jm[(j0 + c) * kJS + tid], x[c], yl);
-            }
-            if (tid == kFT - 1) {
-#pragma unroll
-                for (int c = 0; c < 8; c++)
-                    if (c < nb) yf[j0 + c] = x[c];
-            }
-            buf ^= 1;
-        }
-    }
-    __syncthreads();
-    if (tid < m) sm.delta[tid] = (double)yf[tid];
-    __syncthreads();
-}
-
-// Smallest pivot of the last factorisation relative to the diagonal entry it came from: how much of the diagonal the
-// elimination left (near 1 for a well-conditioned system; 1e-3 and below where the fp32 system is close to singular
-// and its solution no longer a Newton step).  Reads the factor's diagonal where fast_newton_step left it.
-static __device__ double fast_relative_pivot(const FSm& sm, int m, double add)
-{
-    const int tid = threadIdx.x;
-    GR_PTR(float) dg = GR_PCAST(float, sm.J) + 2 * kMP;
-    const double rp = tid < m ? (double)dg[tid] * (double)dg[tid] / (sm.g[tid] - sm.g2[tid] + add) : 1.0;
-    return -block_reduce_max(-rp, sm.scal + SC_RED);
-}
-
-// Newton iteration for one system.  On return sm.w holds exp(alpha) at the last evaluated point.
-template <int NT, int TPL>
-__device__ int fast_system(const FSm& sm, int m, int n, GR_PTR(const double) d, GR_PTR(const double) rhs, double hmass,
-                           int slack, double tol, int max_iters, double qstep, double* gnorm, int* iters)
-{
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    GR_PTR(double) red = sm.scal + SC_RED;
-    // ---- mean-field starting point: token i wins the share w_i / (slack + w_i + S_i) of the tuples that
-    //      contain it, S_i = expected weight of the other drafted tokens given that i was drafted
-    const double T = hmass + block_reduce_sum(tid < m ? d[tid] : 0.0, red);
-    const double Tn = ipow(T, n);
-    double ci = 1.0, rho = 0.5, wi = 1.0;
-    if (tid < m) {
-        sm.col[tid] = ipow(fmax(T - d[tid], 0.0), n);        // mass of tuples avoiding token tid
-        ci = Tn - sm.col[tid];
-        rho = fmin(rhs[tid] / ci, 1.0 - 1e-3);
-        wi = slack ? rho / (1.0 - rho) : rhs[tid] / d[tid];
-    }
+    double alpha = on ? (double)__logf(wi) : 0.0;
     if (!slack) {
-        const double ml = block_reduce_sum(tid < m ? log(wi) : 0.0, red) / (double)m;
-        wi *= exp(-ml);
+        const double mean = tok_sum<C>(sm, on ? alpha : 0.0, par) / (double)m;
+        if (on) alpha -= mean;
     }
-    if (tid < m) sm.w[tid] = wi;
-    __syncthreads();
-    // Pr[i and j drafted, all drafts inside] once, in the (still unused) contraction accumulator
-    for (int e = tid; e < m * kMP; e += kFT) {
-        const int i = e / kMP, j = e - i * kMP;
-        if (j < m) {
-            const double pij = Tn - sm.col[i] - sm.col[j] + ipow(fmax(T - d[i] - d[j], 0.0), n);
-            sm.Jacc[i * kJS + j] = (i == j) ? 0.f : (float)pij;
-        }
-    }
-    __syncthreads();
-    // Sweeps of  w_i = rho_i / (1 - rho_i) * (slack + S_i),  S_i = the weight token i is up against.  A competitor j,
-    // present with probability pi_ij = Pr[i and j drafted] / Pr[i drafted], adds to S_i the weight e_j for which
-    // 1 / (A + e_j) = (1 - pi_ij) / A + pi_ij / (A + w_j),  A = slack + w_i + S_i:  e_j = A pi_ij w_j / (A + w_j (1 - pi_ij)).
-    // For w_j << A this is the mean-field value pi_ij w_j; a huge w_j counts for A pi_ij / (1 - pi_ij) only (token i
-    // simply loses the tuples that contain j), which keeps the start sane when a few weights are in the thousands.
-    // fp32: it is a starting point.
-    if (tid < m) { sm.g2[tid] = 1.0 / ci; sm.g[tid] = (slack ? 1.0 : 0.0) + wi; }
-    __syncthreads();
-    GR_PTR(float) part = sm.AS;                       // [kFW][kMP] partial sums (the staging area is idle here)
-    for (int sweep = 0; sweep < kFSweeps; sweep++) {
-        // lane = rows lane, lane + 32, ...; warp = a contiguous share of the columns: no shuffles, independent sums
-        {
-            const int chunk = (m + kFW - 1) / kFW;
-            const int jlo = warp * chunk, jhi = min(m, jlo + chunk);
-            float Ar[kRL], cr[kRL], sa[kRL], sb[kRL];
-            GR_PTR(const float) row[kRL];
-#pragma unroll
-            for (int u = 0; u < kRL; u++) {
-                const int r = lane + 32 * u;
-                const bool on = r < m;
-                Ar[u] = on ? (float)sm.g[r] : 1.f; cr[u] = on ? (float)sm.g2[r] : 0.f;
-                row[u] = sm.Jacc + ((on ? r : 0) * kJS);
-                sa[u] = 0.f; sb[u] = 0.f;
-            }
-            int j = jlo;
-            for (; j + 1 < jhi; j += 2) {
-                const float wa = (float)sm.w[j], wb = (float)sm.w[j + 1];
-#pragma unroll
-                for (int u = 0; u < kRL; u++) {
-                    const float pa = fminf(row[u][j] * cr[u], 1.f), pb = fminf(row[u][j + 1] * cr[u], 1.f);
-                    sa[u] += __fdividef(Ar[u] * pa * wa, Ar[u] + wa * (1.f - pa));
-                    sb[u] += __fdividef(Ar[u] * pb * wb, Ar[u] + wb * (1.f - pb));
-                }
-            }
-            if (j < jhi) {
-                const float wa = (float)sm.w[j];
-#pragma unroll
-                for (int u = 0; u < kRL; u++) {
-                    const float pa = fminf(row[u][j] * cr[u], 1.f);
-                    sa[u] += __fdividef(Ar[u] * pa * wa, Ar[u] + wa * (1.f - pa));
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kRL; u++) part[warp * kMP + lane + 32 * u] = sa[u] + sb[u];
-        }
-        __syncthreads();
-        double Si = 0.0;
-        if (tid < m) {
-#pragma unroll
-            for (int w2 = 0; w2 < kFW; w2++) Si += (double)part[w2 * kMP + tid];
-            wi = rho / (1.0 - rho) * (slack ? 1.0 + Si : fmax(Si, 1e-300));
-        }
-        double scale = 1.0;
-        if (!slack) {
-            const double ml = block_reduce_sum(tid < m ? log(wi) : 0.0, red) / (double)m;
-            scale = exp(-ml);
-            wi *= scale;
-        }
-        __syncthreads();
-        if (tid < m) { sm.w[tid] = wi; sm.g[tid] = (slack ? 1.0 : 0.0) + wi + scale * Si; }
-        __syncthreads();
-    }
-    if (tid < m) {
-        sm.alpha[tid] = fmin(fmax(log(wi), -kFAlphaClamp), kFAlphaClamp);
-    }
-    __syncthreads();
+    return fmin(fmax(alpha, -kFAlphaClamp), kFAlphaClamp);
+}
 
-    int status = GR_NOT_CONVERGED, it = 0;
-    double rn = 0.0, rprev = 1.0e300, lam = 1.0;
-    bool was_coarse = true;
-    bool full_grid_only = false;         // set once a factorisation has failed
-    int stalls = 0;
-    bool predicted = false;              // the norm returned is a prediction, not an evaluation                      // times a step could not be made to reduce the residual at any length tried
+// Newton iteration for one system.  Returns the status; w_out = exp(alpha) of this thread's token at the last accepted point.
+template <class C>
+__device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, int n, double sigma, double tol, int max_iters,
+                                           double qstep, double* gnorm, int* iters, double* w_out)
+{
+    const int tid = threadIdx.x, i = tid % C::MP;
+    const int m = sy.m, slack = sy.slack;
+    const bool on = i < m, lead = tid < C::MP;
+    int par = 0;
+    const int pos = on ? sm.ord[i] : 0;
+    const double rhs_i = on ? sm.rhs[pos] : 0.0, d_i = on ? sm.d[pos] : 0.0, ds_i = d_i * sigma;
+    double dmax = d_i, Tm = d_i;
+    tok_max_sum<C>(sm, dmax, Tm, par);
+    Tm += sy.hmass;
+    // mass of the tuples the system serves, and the slack's share of it at the solution
+    const double Tn = ipow(Tm, n);
+    const float t0 = slack ? (float)(Tn - tok_sum<C>(sm, rhs_i, par)) : 0.f;
+    const double hs = sy.hmass * sigma;
+
+    double alpha = start_point<C>(m, slack, n, d_i, rhs_i, Tm, sm.flag);
+    // scaled draft masses (and at short series their powers) for the evaluations
+    if (lead) {
+        sm.dsd[i] = ds_i;
+        RSm<C, float> rs(sm);
+        rs.ds[i] = (float)ds_i;
+        if (C::NT <= 8) {
+            float pw = (float)ds_i;
+            const float f = pw;
+#pragma unroll
+            for (int c = 0; c < 8; c++) { sm.E[8 * i + c] = pw; pw *= f; }
+        }
+    }
+
+    double alpha_prev = alpha, delta = 0.0, g = 0.0, g2 = 0.0;
+    int status = GR_NOT_CONVERGED, it = 0, stalls = 0, was_kind = -1;
+    double rn = 0.0, rprev = 1.0e300, lam = 1.0, dist = 0.0;
+    // Three modes.  Low: gradient and Hessian in fp32, conjugate gradients.  Chord: fp64 gradient, the last Hessian.  High:
+    // fp64 gradient, fp32 Hessian of the same point, with `chol` a Cholesky factorisation.  A single token that dominates a
+    // long series (its terms would cancel in fp32) starts in the last mode.
+    enum { kLow, kChord, kHigh };
+    int mode = (C::NT <= 8 || dmax < 0.6 * Tm) ? kLow : kHigh;
+    bool full_grid = false, predicted = false, chol = false;
+#pragma unroll 1
     for (; it < max_iters; it++) {
-        // far from the solution the trapezoid step is doubled (quadrature error ~4e-6, far below the gradient
-        // norm there): half the nodes, every one of them a Hessian node.  Convergence is only ever declared on
-        // the full grid.
-        const bool coarse = rprev > 1.0e-2 && !full_grid_only;
-        fast_grid(sm, m, n, slack, coarse ? 2.0 * qstep : qstep);
-        // Hessian nodes: every second one on the full grid, every one on the doubled step (taking every second one
-        // there too kept all eight warps of the wide kernel busy and saved 8 % on one shape, but a Hessian from six or
-        // seven nodes cost others one to three more evaluations, and a 128-token, n = 16 shape seven times its time)
-        fast_eval<NT, TPL>(sm, m, n, d, hmass, true, coarse ? 1 : 2);
-        rn = block_reduce_sum(tid < m ? fabs(sm.g[tid] - rhs[tid]) : 0.0, red);
-        if (rn <= tol && !coarse) { status = GR_OK; it++; break; }
-        // (a residual on the full grid is not compared with the coarse grid's: they differ by the coarse quadrature error)
-        const bool comparable = coarse == was_coarse;
-        was_coarse = coarse;
-        if (comparable && !(rn < rprev) && lam > 1.0 / 64.0 && it > 0) {
-            // the last step did not reduce the gradient norm: retry it at half length
-            lam *= 0.5;
-            if (tid < m) sm.alpha[tid] = sm.alpha_prev[tid] + lam * sm.delta[tid];
-            __syncthreads();
-            continue;
-        }
-        // A step that did not reduce the residual even at 1/64 of its length: the fp32 Newton system has reached its
-        // accuracy for this instance (weights of 1e5 and more).  The second time the instance is handed to the fp64
-        // kernel, which starts from the last accepted point, instead of spending the rest of the evaluation budget.
-        if (comparable && !(rn < rprev) && it > 0 && ++stalls >= 2) {
-            if (tid < m) sm.alpha[tid] = sm.alpha_prev[tid];
-            __syncthreads();
-            break;
-        }
-        // contraction of the last full step (same grid on both sides)
-        const double rho = (comparable && !coarse && it > 0 && lam == 1.0) ? rn / rprev : 1.0e300;
-        rprev = rn; lam = 1.0;
-        if (tid < m) sm.alpha_prev[tid] = sm.alpha[tid];
-        if (tid == 0) sm.scal[SC_FAIL] = 0.0;
-        // Newton step with the Hessian (off-diagonal from the contraction, diagonal g - g2); an outer block's
-        // function is constant along (1,...,1): pin that direction with 1/m everywhere
-        fast_newton_step(sm, m, rhs, slack ? 0.0 : 1.0 / (double)m);
-        const bool fail = sm.scal[SC_FAIL] != 0.0;
-        // (a Hessian from the doubled step that is not positive definite in fp32: with the full grid's diagonal the
-        // factorisation usually goes through, where proportional fitting would crawl down to the switch at 1e-2)
-        if (fail) full_grid_only = true;
-        if (fail) {
-            // proportional-fitting step  alpha += log(rhs / g)
-            if (tid < m) sm.delta[tid] = log(rhs[tid] / sm.g[tid]);
-            __syncthreads();
-        }
-        double dl = tid < m ? sm.delta[tid] : 0.0;
-        if (!(dl == dl)) dl = 0.0;
-        if (!slack) dl -= block_reduce_sum(tid < m ? dl : 0.0, red) / (double)m;
-        const double dm = block_reduce_max(tid < m ? fabs(dl) : 0.0, red);
-        // a full Newton step below 1e-11 in alpha: the weights cannot be improved at this quadrature accuracy
-        if (!fail && dm < 1.0e-11) { status = GR_OK; it++; break; }
-        if (dm > kFStepClamp) dl *= kFStepClamp / dm;
-        // second-order size of the step, sum_i g_i delta_i^2: what a full Newton step in alpha = log w leaves behind
-        // (each flow g_i is a sum of terms exponential in alpha over positive normalisers, so the part of g the
-        // linear model misses is of the order of g_i delta_i^2 per token)
-        const double s2 = block_reduce_sum(tid < m ? sm.g[tid] * dl * dl : 0.0, red);
-        if (tid < m) {
-            sm.delta[tid] = dl;
-            sm.alpha[tid] = fmin(fmax(sm.alpha[tid] + dl, -kFAlphaClamp), kFAlphaClamp);
-        }
-        __syncthreads();
-        // Stop on a predicted residual, without another evaluation, after a step from a point evaluated on the full
-        // grid.  Two forms.  (i) The step is small: the residual it leaves is bounded by a small multiple of s2
-        // (measured on every benchmark shape and at target temperatures down to 0.3, 2300 full-grid steps: next residual
-        // <= 8.5 s2 + the quadrature floor of ~3e-9, median 0.15 s2); with 10 s2 below the tolerance the step is taken,
-        // and the reported norm is 3 s2.  (ii) The last full step on this grid contracted the residual by rho < 0.1:
-        // the next one is taken to contract no worse (Newton's contraction improves as it converges, and where it
-        // converges only linearly, by 0.03 - 0.06 per step on systems with a small pivot, this is what happens), so
-        // 3 rho r_k below the tolerance stops; the reported norm is rho r_k.  This form serves tolerances near the
-        // quadrature floor, where s2 is too coarse.
-        // Neither is trusted when the factorisation cancelled all but a few percent of some diagonal entry: with
-        // weights of 1e5 and more the fp32 system stops producing Newton steps, the residual stays where it is while
-        // the steps, and with them s2, shrink; every such case measured had a relative pivot below 4e-3, every other
-        // above 3e-2.
-        const bool by_step = !coarse && dm <= kFPredictStep && kFPredictSafety * s2 < tol;
-        const bool by_ratio = rho < 0.1 && dm <= kFStepClamp && kFRatioSafety * rho * rn < tol;
-        if (!fail && (by_step || by_ratio)
-            && fast_relative_pivot(sm, m, slack ? 0.0 : 1.0 / (double)m) > kFTrustPivot) {
-            if (tid < m) sm.w[tid] = exp(sm.alpha[tid]);
-            __syncthreads();
-            rn = by_step ? kFPredictBound * s2 : rho * rn;
+        // far from the solution the trapezoid step is doubled (quadrature error ~4e-6, far below the gradient norm
+        // there): half the nodes, every one of them a Hessian node.  Convergence is only declared on the full grid.
+        const bool coarse = rprev > kFCoarse && !full_grid && mode != kChord;
+        const int kind = 2 * mode + (coarse ? 1 : 0);
+        const double w_i = !on ? 0.0 : (mode == kLow ? (double)__expf((float)alpha) : m_exp(alpha));
+        if (lead) { sm.wd[i] = w_i; sm.wf[i] = (float)w_i; }
+        float amax, amin;
+        tok_range<C>(sm, (float)alpha, on, amax, amin, par);
+        const double qs = coarse ? 2.0 * qstep : qstep;
+        double2 gg = make_double2(0.0, 0.0);
+        if (mode != kLow) gg = eval_fp64<C>(m, n, hs, slack, qs, amax, amin, w_i, ds_i, sm.flag);
+        if (mode != kChord)
+            gg = eval_hessian<C>(m, n, hs, slack, qs, coarse ? 1 : 2, amax, amin, w_i, ds_i, rhs_i, mode == kHigh, chol, gg, sm.flag);
+        g = gg.x; g2 = gg.y;
+        const double2 rg = tok_max_sum_fn<C>(on ? g : 0.0, on ? fabs(g - rhs_i) : 0.0, true, par, sm.flag);
+        par ^= 1;
+        rn = rg.y;
+        // (residuals are only compared within one grid and one precision)
+        const bool comparable = kind == was_kind && it > 0;
+        was_kind = kind;
+        // Stop on an evaluated residual.  (An fp32 evaluation on the full grid is good to ~1e-6: enough to see a tolerance
+        // of 1e-4 and more met.  Between half the tolerance and the tolerance one more step, which costs a tenth of an
+        // evaluation, leaves a residual far below it, unless steps have stopped helping.)
+        if (rn <= tol && !coarse && (mode != kLow || tol >= 1.0e-4) && (rn <= 0.5 * tol || (comparable && rn > 0.5 * rprev))) {
             status = GR_OK; it++;
-            predicted = true;
             break;
         }
+        bool high = false;               // the same point again with an fp64 gradient on the full grid
+        if (mode == kChord) {
+            // the reused Hessian no longer serves: one of its own from here on
+            high = !(rn <= 1.0e-3) || (comparable && !(rn < 0.3 * rprev));
+        } else if (comparable && !(rn < rprev)) {
+            if (mode == kLow && rn < kFLowFloor) high = true;          // at the noise of fp32
+            else if (lam > 1.0 / 64.0) {
+                // the last step did not reduce the gradient norm: retry it at half length
+                lam *= 0.5;
+                alpha = alpha_prev + lam * delta;
+                continue;
+            } else if (mode == kLow) {
+                high = true; alpha = alpha_prev;
+            } else {
+                // A step that did not reduce the residual even at 1/64 of its length: the fp32 Newton system has reached
+                // its accuracy for this instance.  Conjugate gradients give way to the factorisation; the second time there
+                // the instance is handed to the general kernel, which starts from the last accepted point.
+                if (chol && ++stalls >= 2) { alpha = alpha_prev; break; }
+                chol = true;
+            }
+        }
+        if (high) { mode = kHigh; full_grid = true; rprev = 1.0e300; lam = 1.0; was_kind = -1; continue; }
+        // contraction of the last full step (same grid and precision on both sides)
+        const double rho = (comparable && !coarse && lam == 1.0) ? rn / rprev : 1.0e300;
+        rprev = rn; lam = 1.0;
+        alpha_prev = alpha;
+        // Newton step
+        double dl;
+        bool fail = false;
+        float pivot = 1.f;
+        double jump = 0.0;               // part of the step that is a common shift, not subject to the clamp
+        if (!chol) {
+            // The common scale of the weights.  The slack's share g0 = T^n - sum g is, along that scale, a falling logistic
+            // curve whose slope is sum s; where its target t0 is far below (acceptance close to one), the curve is inverted
+            // exactly, as the tokens' own curves are in newton_rhs: a Newton step would move the scale by one at most.
+            const float b = on ? newton_rhs(g, g2, rhs_i) : 0.f, s_i = on ? __fdividef((float)g2, (float)w_i) : 0.f;
+            float shift = 0.f;
+            float sums[3] = {b, slack ? s_i : 0.f, on ? (float)(g - g2) : 0.f};
+            tok_sums<C, 3>(sm, sums, par);
+            const float lin = slack ? __fdividef(sums[0], sums[1]) : 0.f;
+            if (slack) {
+                const float g0 = (float)(Tn - rg.x);
+                shift = lin;
+                pivot = __fdividef(sums[1], sums[2]);               // of the order of the smallest relative pivot
+                if (t0 > 0.f && g0 > sums[1] && g0 > 1.0e-5f) {
+                    // saturation level c0 from value and slope:  slope = g0 (1 - g0 / c0)
+                    const float inv = __fdividef(g0 - sums[1], g0 * g0);              // 1 / c0
+                    const float q = __fdividef(g0 * (1.f - t0 * inv), t0 * (1.f - g0 * inv));
+                    const float far = q > 0.f ? __logf(q) : 0.f;
+                    if (far > kFScaleJump) { shift = fminf(far, 16.f); jump = (double)shift; }
+                }
+            }
+            const float step = cg_solve<C>(m, slack, b, s_i, slack ? -__fdividef(1.f, sums[1]) : __fdividef(1.f, sums[2]), lin, shift, kFCgTol, sm.flag);
+
+            // (NaN for every thread or none: the iteration's scalars are common)
+            if (__syncthreads_or(!(step == step))) {
+                // badly conditioned: the same point again with an fp64 gradient and a factorisation
+                mode = kHigh; chol = true; full_grid = true; rprev = 1.0e300; was_kind = -1;
+                continue;
+            }
+            dl = (double)step;
+        } else {
+            backward_subst<C>(m, sm.flag);
+            __syncthreads();
+            fail = sm.scal[SC_FAIL] != 0.0;
+            pivot = (float)sm.scal[SC_PIVOT];
+            dl = on ? (double)sm.dl[i] : 0.0;
+            // proportional-fitting step  alpha += log(rhs / g)  (and the full grid from here on)
+            if (fail) { full_grid = true; dl = on ? m_log(rhs_i / g) : 0.0; }
+        }
+        if (!(dl == dl)) dl = 0.0;
+        if (!slack) {
+            const double mean = tok_sum<C>(sm, dl, par) / (double)m;
+            if (on) dl -= mean;
+        }
+        double dm = on ? fabs(dl - jump) : 0.0, s2 = on ? g * dl * dl : 0.0;
+        tok_max_sum<C>(sm, dm, s2, par);
+        // a full Newton step below 1e-11 in alpha: the weights cannot be improved at this quadrature accuracy
+        if (!fail && mode != kLow && dm < 1.0e-11) { status = GR_OK; it++; break; }
+        if (dm > kFStepClamp && on) dl = jump + (dl - jump) * (kFStepClamp / dm);
+        delta = dl;
+        alpha = fmin(fmax(alpha + dl, -kFAlphaClamp), kFAlphaClamp);
+        // Stop on a predicted residual, without another evaluation, after a step from a point evaluated in fp64 on the
+        // full grid.  s2 = sum_i g_i delta_i^2 is what a full Newton step in alpha = log w leaves behind (each flow is a
+        // sum of terms exponential in alpha over positive normalisers; measured on every benchmark shape and at target
+        // temperatures down to 0.3, 2300 full-grid steps: next residual <= 8.5 s2 + the quadrature floor of ~3e-9, median
+        // 0.15 s2).  (i) By the step: 10 s2 below the tolerance.  (ii) With a reused Hessian a linear term comes on top: the
+        // distance to the point it was formed at, plus the accuracy it was formed with.  (iii) By the ratio: the last full
+        // step on this grid contracted the residual by rho < 0.1 and the next one is taken to contract no worse.
+        // None is trusted when the factorisation cancelled all but a few percent of some diagonal entry: with weights of
+        // 1e5 and more the fp32 system stops producing Newton steps, the residual stays where it is while the steps, and
+        // with them s2, shrink; every such case measured had a relative pivot below 4e-3, every other above 3e-2.
+        const bool trusted = !fail && pivot > (float)kFTrustPivot;
+        if (mode == kLow) {
+            // the next point is close enough: fp64 from here on, with this factorisation
+            if (kFPredictBound * s2 < kFLowLeave && dm + jump <= 0.1) { mode = trusted ? kChord : kHigh; full_grid = true; dist = dm; }
+        } else if (trusted && !coarse) {
+            const double lin = mode == kChord ? (kFChordBase + 2.0 * dist) * rn : 0.0;
+            const bool by_step = dm + jump <= kFPredictStep && kFPredictSafety * s2 + 3.0 * lin < tol;
+            const bool by_ratio = rho < 0.1 && dm <= kFStepClamp && kFRatioSafety * rho * rn < tol;
+            if (by_step || by_ratio) {
+                rn = by_step ? kFPredictBound * s2 + lin : rho * rn;
+                status = GR_OK; it++;
+                predicted = true;
+                break;
+            }
+            if (mode == kChord) dist += dm;
+        }
     }
-    if (status != GR_OK) {
-        // not converged here: leave the last accepted point (the fp64 kernel's starting point)
-        __syncthreads();
-        if (tid < m) sm.w[tid] = exp(status == GR_NOT_CONVERGED ? sm.alpha_prev[tid] : sm.alpha[tid]);
-        __syncthreads();
-    }
+    // (not converged here: the last accepted point, the general kernel's starting point)
+    *w_out = on ? m_exp(status == GR_OK ? alpha : alpha_prev) : 0.0;
     *gnorm = rn;
     *iters = it | (predicted ? kItersPredicted : 0);
     return status;
 }
 
-template <int NT, int TPL>
-__global__ void __launch_bounds__(kFT, kFCtas)
+template <class C>
+__global__ void __launch_bounds__(C::T, C::kCtas)
 fast_solve_kernel(const char* __restrict__ ws, char* __restrict__ params, int pstride, int kcap, int V, int n, int topk,
-                  double temp_t, double temp_d, double tol, int max_iters, double qstep, double tau,
+                  double temp_t, double temp_d, double tol, int max_iters, double qstep, double tau, double sigma,
                   float* __restrict__ alpha_out, int* __restrict__ status_out, FusedArgs fa)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_sel;
     GR_CHECK_FLAG_DECL;
     GR_CHECK_FLAG_INIT;
@@ -902,142 +1299,127 @@ fast_solve_kernel(const char* __restrict__ ws, char* __restrict__ params, int ps
         if (tid == 0) write_no_rule(pv.h, n, wv.h->bad != 0, alpha_out, status_out, b);
         if (fused) {
             __syncthreads();
-            fused_draw(fa, pv.h, b, n, smem_raw, GR_CHECK_FLAG);
+            fused_draw(fa, pv.h, b, n, smem_raw + C::oU, GR_CHECK_FLAG);
         }
         return;
     }
-    const int KP = kcap;
-    FastLayout L(KP, NT);
-    double* base = reinterpret_cast<double*>(smem_raw);
-    FSm sm;
+    constexpr int MP = C::MP;
     int* const ck = GR_CHECK_FLAG;
-    (void)ck;
-    sm.d = GR_MKPTR(double, base + L.d, KP, ck); sm.tg = GR_MKPTR(double, base + L.tg, KP, ck);
-    sm.p = GR_MKPTR(double, base + L.p, KP, ck); sm.r = GR_MKPTR(double, base + L.r, KP, ck);
-    sm.key = GR_MKPTR(double, base + L.key, KP, ck);
-    sm.psi = GR_MKPTR(double, base + L.psi, KP + 4, ck); sm.Dr = GR_MKPTR(double, base + L.Dr, KP + 4, ck);
-    sm.alpha = GR_MKPTR(double, base + L.alpha, KP, ck); sm.alpha_prev = GR_MKPTR(double, base + L.alpha_prev, KP, ck);
-    sm.delta = GR_MKPTR(double, base + L.delta, KP, ck); sm.w = GR_MKPTR(double, base + L.w, KP, ck);
-    sm.g = GR_MKPTR(double, base + L.g, KP, ck); sm.g2 = GR_MKPTR(double, base + L.g2, KP, ck);
-    sm.col = GR_MKPTR(double, base + L.col, kMP, ck);
-    sm.gw = GR_MKPTR(double, base + L.gw, kFW * KP, ck); sm.g2w = GR_MKPTR(double, base + L.g2w, kFW * KP, ck);
-    sm.tq = GR_MKPTR(double, base + L.tq, kFMaxNodes, ck); sm.cq = GR_MKPTR(double, base + L.cq, kFMaxNodes, ck);
-    sm.scal = GR_MKPTR(double, base + L.scal, 48, ck);
-    sm.J = GR_MKPTR(double, base + L.uni, L.uni_doubles, ck);
-    sm.AS = GR_MKPTR(float, reinterpret_cast<float*>(base + L.uni), kJC * NT * kMS, ck);
-    sm.HS = GR_MKPTR(float, reinterpret_cast<float*>(base + L.uni) + kJC * NT * kMS, kJC * NT * kMS, ck);
-    sm.Jacc = GR_MKPTR(float, reinterpret_cast<float*>(smem_raw + L.jacc_bytes_off), kMP * kJS, ck);
-    int* ib = reinterpret_cast<int*>(smem_raw + L.ints);
-    sm.id = GR_MKPTR(int, ib, KP, ck); sm.blk = GR_MKPTR(int, ib + KP, KP, ck);
-    sm.itmp = GR_MKPTR(int, ib + 2 * KP, KP, ck); sm.trunc = GR_MKPTR(int, ib + 3 * KP, KP, ck);
-    sm.KP = KP;
+    const FSm<C> sm(ck);
+    char* const sb = sm.base;
+
+    // ---- distributions, ratio order, H*, residuals, blocks (arrays the solve does not need live in the union area)
     PrepSm ps;
-    ps.d = sm.d; ps.tg = sm.tg; ps.p = sm.p; ps.r = sm.r; ps.key = sm.key; ps.psi = sm.psi; ps.Dr = sm.Dr;
-    ps.id = sm.id; ps.blk = sm.blk; ps.itmp = sm.itmp; ps.red = sm.scal + SC_RED; ps.out3 = sm.scal + 16;
+    double* const ub = reinterpret_cast<double*>(sb + C::oU);
+    ps.d = sm.d; ps.p = sm.rhs; ps.Dr = sm.Dr;
+    ps.tg = GR_MKPTR(double, ub, MP, ck); ps.r = GR_MKPTR(double, ub + MP, MP, ck);
+    ps.key = GR_MKPTR(double, ub + 2 * MP, MP, ck); ps.psi = GR_MKPTR(double, ub + 3 * MP, MP + 4, ck);
+    int* const ui = reinterpret_cast<int*>(ub + 4 * MP + 4);
+    ps.id = GR_MKPTR(int, ui, MP, ck); ps.itmp = GR_MKPTR(int, ui + MP, MP, ck);
+    ps.blk = sm.blk; ps.red = sm.red; ps.out3 = sm.scal + SC_OUT;
     const PrepResult pr = prep_instance(ps, wv, pv.h, V, n, topk, temp_t, temp_d);
     const int k = pr.k, jstar = pr.jstar;
-
-    int status = GR_OK, iters_total = 0;
-    double gnorm_total = 0.0;
     // Truncated variant (Algorithm 1 with an error threshold): every system is solved on its truncation set alone,
-    // to gradient norm 5 tau; the other tokens keep weight 0.  The gathered arrays reuse what the preparation no
-    // longer needs.
+    // to gradient norm 5 tau; the other tokens keep weight 0.
     const bool trunc = tau > 0.0;
     if (trunc) {
-        truncation_sets(ps, sm.trunc, sm.itmp, k, jstar, n, tau);
+        truncation_sets(ps, sm.trunc, ps.itmp, k, jstar, n, tau);
         tol = 5.0 * tau;
     }
-    GR_PTR(double) dT = sm.key; GR_PTR(double) rT = sm.psi; GR_PTR(int) tmap = sm.itmp;
-    if (tid < k) pv.w[tid] = trunc ? 0.0 : 1.0;
     // with the drafted tuple at hand only the system it selects is solved
-    const int sel = fused ? selected_system(fa.draft + (size_t)b * n, n, k, jstar, sm.id, sm.blk, &s_sel) : -2;
-    bool skipped = false;
-    if (jstar > 0 && sel >= 0) skipped = true;
-    if (jstar > 0 && sel < 0) {
-        double gn = 0.0; int it = 0;
-        if (!trunc) {
-            const int st = fast_system<NT, TPL>(sm, jstar, n, sm.d, sm.tg, 0.0, 1, tol, max_iters, qstep, &gn, &it);
-            if (st != GR_OK) status = kNeedFallback;
-            if (tid < jstar) pv.w[tid] = sm.w[tid];
-        } else {
-            const int mT = gather_truncated(sm.trunc, 0, jstar, sm.d, sm.tg, dT, rT, tmap, &s_sel);
-            if (mT > 0) {
-                const int st = fast_system<NT, TPL>(sm, mT, n, dT, rT, 0.0, 1, tol, max_iters, qstep, &gn, &it);
-                if (st != GR_OK) status = kNeedFallback;
-                if (tid < mT) pv.w[tmap[tid]] = sm.w[tid];
-            }
-        }
-        gnorm_total += gn; iters_total = add_iters(iters_total, it);
-        __syncthreads();
+    const int sel = fused ? selected_system(fa.draft + (size_t)b * n, n, k, jstar, ps.id, sm.blk, &s_sel) : -2;
+    // the rule's arrays, except the weights of the systems solved below
+    for (int j = tid; j < kcap; j += C::T) {
+        const bool in = j < k;
+        pv.id[j] = in ? ps.id[j] : -1;
+        pv.blk[j] = in ? sm.blk[j] : -2;
+        pv.r[j] = in ? ps.r[j] : 0.0;
+        pv.p[j] = in ? sm.rhs[j] : 0.0;
+        pv.w[j] = in && !trunc ? 1.0 : 0.0;
     }
-    int lo = jstar;
+    __syncthreads();
+
+    // ---- the systems: the inner one on H*, then every outer block with two or more tokens
+    int status = GR_OK, iters_total = 0;
+    double gnorm_total = 0.0;
+    bool skipped = false;
+    int lo = 0;
+#pragma unroll 1
     while (lo < k && status == GR_OK) {
-        int hi = lo;
+        const bool inner = lo < jstar;
+        int hi;
         const int bk = sm.blk[lo];
-        while (hi + 1 < k && sm.blk[hi + 1] == bk) hi++;
-        const int m = hi - lo + 1;
-        const bool wanted = sel == -2 || sel == bk;
-        if (!trunc) {
-            if (m >= 2 && !wanted) skipped = true;
-            if (m >= 2 && wanted) {
-                double gn; int it;
-                const int st = fast_system<NT, TPL>(sm, m, n, sm.d + lo, sm.p + lo, sm.Dr[lo], 0, tol, max_iters, qstep,
-                                                    &gn, &it);
-                if (st != GR_OK) status = kNeedFallback;
-                gnorm_total += gn; iters_total = add_iters(iters_total, it);
-                if (tid < m) pv.w[lo + tid] = sm.w[tid];
-                __syncthreads();
-            }
-        } else {
+        if (inner) hi = jstar;
+        else { hi = lo + 1; while (hi < k && sm.blk[hi] == bk) hi++; }
+        const bool wanted = sel == -2 || (inner ? sel < 0 : sel == bk);
+        if (tid < MP) sm.wf[tid] = tid < k ? (float)sm.d[tid] : 0.f;
+        __syncthreads();
+        // tokens of the system in ascending draft mass (positions break ties; fp32 is enough to order them)
+        const int pos = lo + tid;
+        const bool in = tid < MP && pos < hi && (!trunc || sm.trunc[pos] != 0);
+        const float dv = in ? sm.wf[pos] : 0.f;
+        double hm = inner ? 0.0 : sm.Dr[lo];
+        if (trunc && !inner) {
             // tuples counted: those inside (H* u T)^n, so the mass above the block is drf(H*) plus the T-part of the
             // higher-ratio outer blocks
-            double hT = sm.Dr[jstar];
-            for (int j = jstar; j < lo; j++) hT += sm.trunc[j] ? sm.d[j] : 0.0;
-            const int mT = gather_truncated(sm.trunc, lo, hi + 1, sm.d, sm.p, dT, rT, tmap, &s_sel);
-            if (mT == 1 && tid == 0) pv.w[tmap[0]] = 1.0;
-            if (mT >= 2 && !wanted) skipped = true;
-            if (mT >= 2 && wanted) {
-                double gn; int it;
-                const int st = fast_system<NT, TPL>(sm, mT, n, dT, rT, hT, 0, tol, max_iters, qstep, &gn, &it);
-                if (st != GR_OK) status = kNeedFallback;
-                gnorm_total += gn; iters_total = add_iters(iters_total, it);
-                if (tid < mT) pv.w[tmap[tid]] = sm.w[tid];
-            }
-            __syncthreads();
+            hm = sm.Dr[jstar];
+            for (int j = jstar; j < lo; j++) hm += sm.trunc[j] ? sm.d[j] : 0.0;
         }
-        lo = hi + 1;
+        if (in) {
+            int rank = 0;
+#pragma unroll 4
+            for (int j = lo; j < hi; j++) {
+                const float dj = sm.wf[j];
+                rank += ((!trunc || sm.trunc[j] != 0) && (dj < dv || (dj == dv && j < pos))) ? 1 : 0;
+            }
+            sm.ord[rank] = pos;
+        }
+        const int m = __syncthreads_count(in);
+        if (trunc && !inner && m == 1 && in) pv.w[pos] = 1.0;
+        const bool solve = inner ? m > 0 : m >= 2;
+        // (a skipped inner system always leaves the rule partial)
+        if (!wanted && (solve || inner)) skipped = true;
+        if (solve && wanted) {
+            System sy;
+            sy.m = m; sy.slack = inner ? 1 : 0; sy.hmass = hm;
+            double gn, w; int it;
+            const int st = fast_system<C>(sm, sy, n, sigma, tol, max_iters, qstep, &gn, &it, &w);
+            if (st != GR_OK) status = kNeedFallback;
+            gnorm_total += gn; iters_total = add_iters(iters_total, it);
+            if (tid < m) pv.w[sm.ord[tid]] = w;
+        }
+        __syncthreads();
+        lo = hi;
     }
     if (status == GR_OK && skipped) status = GR_PARTIAL_RULE;
-    write_rule(ps, pv, KP, pr, n, status, gnorm_total, iters_total, alpha_out, status_out, b, GR_CHECK_FLAG,
-               wv.h->check);
+    write_rule_header(pv, pr, n, status, gnorm_total, iters_total, alpha_out, status_out, b, GR_CHECK_FLAG, wv.h->check);
     if (fused && status != kNeedFallback) {
         __syncthreads();                       // the rule this CTA wrote is visible to its first warp
-        fused_draw(fa, pv.h, b, n, smem_raw + L.uni * 8, GR_CHECK_FLAG);
+        fused_draw(fa, pv.h, b, n, smem_raw + C::oU, GR_CHECK_FLAG);
     }
 }
 
-template <int NT, int TPL>
+template <class C>
 int launch_fast_t(const char* ws, char* params, int pstride, int kcap, int V, int n, int topk, double temp_t,
-                         double temp_d, double tol, int max_iters, double qstep, double tau, int batch, float* alpha_out,
-                         int* status_out, FusedArgs fa, cudaStream_t st)
+                  double temp_d, double tol, int max_iters, double qstep, double tau, int batch, float* alpha_out,
+                  int* status_out, FusedArgs fa, cudaStream_t st)
 {
-    const int smem = fast_smem_bytes(kcap, NT);
     // function attributes belong to the device: set once per device
     static bool configured[kMaxDevices] = {false};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return GR_E_LAUNCH; }
     if (!configured[dev]) {
-        if (cudaFuncSetAttribute(fast_solve_kernel<NT, TPL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kMP == 64 ? 96 * 1024 : 200 * 1024) != cudaSuccess)
+        if (cudaFuncSetAttribute(fast_solve_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kBytes) != cudaSuccess)
             return GR_E_LAUNCH;
-        // the CTAs are small: ask for the largest shared-memory carve-out so that kFCtas of them fit on an SM
-        if (cudaFuncSetAttribute(fast_solve_kernel<NT, TPL>, cudaFuncAttributePreferredSharedMemoryCarveout,
+        // the CTAs are small: ask for the largest shared-memory carve-out so that many of them fit on an SM
+        if (cudaFuncSetAttribute(fast_solve_kernel<C>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  cudaSharedmemCarveoutMaxShared) != cudaSuccess)
             return GR_E_LAUNCH;
         configured[dev] = true;
     }
-    fast_solve_kernel<NT, TPL><<<batch, kFT, smem, st>>>(ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol,
-                                                         max_iters, qstep, tau, alpha_out, status_out, fa);
+    const double sigma = exp(lgamma((double)n + 1.0) / (double)n);       // sigma^n = n!
+    fast_solve_kernel<C><<<batch, C::T, C::kBytes, st>>>(ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol,
+                                                         max_iters, qstep, tau, sigma, alpha_out, status_out, fa);
     return GR_OK;
 }
 
@@ -1047,11 +1429,8 @@ int launch_fast_t(const char* ws, char* params, int pstride, int kcap, int V, in
         double tol, int max_iters, double qstep, double tau, int batch, float *alpha_out, int *status_out,       \
         FusedArgs fa, cudaStream_t st
 #define GR_FAST_PASS ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol, max_iters, qstep, tau, batch, alpha_out, status_out, fa, st
-#define GR_FAST_INSTANTIATE(NT)                                                                \
-    int launch_fast_n##NT(GR_FAST_ARGS) {                                                       \
-        return kcap <= 32 * (kRL - 1) ? launch_fast_t<NT, kRL - 1>(GR_FAST_PASS)                    \
-                                      : launch_fast_t<NT, kRL>(GR_FAST_PASS);                       \
-    }
+#define GR_FAST_INSTANTIATE(NAME, NT, MP, T, JC, CTAS)                                                            \
+    int launch_fast_##NAME(GR_FAST_ARGS) { return launch_fast_t<Cfg<NT, MP, T, JC, CTAS>>(GR_FAST_PASS); }
 
-}  // namespace GR_FAST_NS
+}  // namespace fast
 }  // namespace gr

@@ -1,8 +1,9 @@
-// Fast solve kernels for series length 4 (draft counts up to 4), supports up to 64 tokens.
+// Fast solve kernels for series length 4 (draft counts up to 4).
 #include "gr_fast.cuh"
 
 namespace gr {
-namespace GR_FAST_NS {
-GR_FAST_INSTANTIATE(4)
-}
+namespace fast {
+GR_FAST_INSTANTIATE(n4_m32, 4, 32, 64, 8, 8)
+GR_FAST_INSTANTIATE(n4_m64, 4, 64, 64, 8, 7)
+}  // namespace fast
 }  // namespace gr

@@ -1,8 +1,10 @@
-// Fast solve kernels for series length 8 (draft counts up to 8), supports up to 64 tokens.
+// Fast solve kernels for series length 8 (draft counts up to 8).
 #include "gr_fast.cuh"
 
 namespace gr {
-namespace GR_FAST_NS {
-GR_FAST_INSTANTIATE(8)
-}
+namespace fast {
+GR_FAST_INSTANTIATE(n8_m32, 8, 32, 64, 8, 8)
+GR_FAST_INSTANTIATE(n8_m64, 8, 64, 128, 6, 4)
+GR_FAST_INSTANTIATE(n8_m128, 8, 128, 128, 4, 3)
+}  // namespace fast
 }  // namespace gr

@@ -9,23 +9,27 @@ namespace gr {
 constexpr int kNeedFallback = 100;   // internal status: the fast kernel asks the robust kernel to redo the instance
 
 // CTA-wide reductions; `scratch` needs one double per warp.  Every thread gets the result.
-__device__ inline double block_reduce_max(double v, GR_PTR(double) scratch) {
+static __device__ __noinline__ double block_reduce_max(double v, GR_PTR(double) scratch) {
+#pragma unroll 1
     for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
     const int nw = blockDim.x >> 5;
     __syncthreads();
     if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = v;
     __syncthreads();
     double r = scratch[0];
+#pragma unroll 1
     for (int i = 1; i < nw; i++) r = fmax(r, scratch[i]);
     return r;
 }
-__device__ inline double block_reduce_sum(double v, GR_PTR(double) scratch) {
+static __device__ __noinline__ double block_reduce_sum(double v, GR_PTR(double) scratch) {
+#pragma unroll 1
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     const int nw = blockDim.x >> 5;
     __syncthreads();
     if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = v;
     __syncthreads();
     double r = 0.0;
+#pragma unroll 1
     for (int i = 0; i < nw; i++) r += scratch[i];
     return r;
 }
@@ -34,7 +38,7 @@ __device__ inline double block_reduce_sum(double v, GR_PTR(double) scratch) {
 struct PrepSm {
     GR_PTR(double) d, tg, p, r, key, psi, Dr;
     GR_PTR(int) id, blk, itmp;
-    GR_PTR(double) red;     // one double per warp of reduction scratch
+    GR_PTR(double) red;     // two doubles per warp of reduction scratch
     GR_PTR(double) out3;    // 3 doubles: jstar, nblocks, alpha*
 };
 struct PrepResult { int k, jstar, nblocks; double alpha_star, lse_t; };
@@ -64,47 +68,57 @@ __device__ inline void write_no_rule(Header* h, int n, bool bad, float* alpha_ou
     status_out[b] = h->status;
 }
 
-// Everything before the convex minimisation.  Every thread of the CTA calls it.
+// Everything before the convex minimisation.  Every thread of the CTA calls it; the block has at least as many threads
+// as the support has tokens.  Bound by latency (a chain of short steps on at most 128 numbers), so every step but the
+// in-order prefix sums is one position per thread with warp scans and ballots.
 __device__ inline PrepResult prep_instance(const PrepSm& sm, const WsView& wv, Header* hdr, int V, int n, int topk,
                                            double temp_t, double temp_d)
 {
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     const int kfull = (topk <= 0 || topk >= V) ? V : topk;
     const int k = wv.h->count;
+    const int kw = (k + 31) >> 5;                 // warps that hold tokens
+    const bool on = tid < k;
     double lse_t = wv.h->lse_t;
     // ---- distributions on the support (App. A; App. N): fp64 from the fp32 / bf16 logits
     double a_i = 0.0, b_i = 0.0;
     int my_id = 0;
-    if (tid < k) {
+    if (on) {
         my_id = wv.id[tid];
-        a_i = (double)wv.tl[tid] / temp_t;
-        b_i = (double)wv.dl[tid] / temp_d;
+        a_i = m_div((double)wv.tl[tid], temp_t);
+        b_i = m_div((double)wv.dl[tid], temp_d);
+        sm.key[tid] = b_i - a_i; sm.itmp[tid] = my_id;
     }
-    const double bmax = block_reduce_max(tid < k ? b_i : -1.0e300, sm.red);
-    const double bsum = block_reduce_sum(tid < k ? exp(b_i - bmax) : 0.0, sm.red);
-    const double lse_d = bmax + log(bsum);
+    const double bmax = block_reduce_max(on ? b_i : -1.0e300, sm.red);
+    const double eb = on ? m_exp(b_i - bmax) : 0.0;
+    const double bsum = block_reduce_sum(eb, sm.red);
+    double tg_i;
     if (kfull == V) {
         // the support is the whole vocabulary: normalise the target in fp64 over these same entries, so that
         // it sums to one to rounding (the streaming kernel's fp32 sum is only good to ~1e-7, which would
         // leave the outermost block's flows inconsistent with the mass of the tuples that feed them)
-        const double amax = block_reduce_max(tid < k ? a_i : -1.0e300, sm.red);
-        const double asum = block_reduce_sum(tid < k ? exp(a_i - amax) : 0.0, sm.red);
-        lse_t = amax + log(asum);
+        const double amax = block_reduce_max(on ? a_i : -1.0e300, sm.red);
+        const double ea = on ? m_exp(a_i - amax) : 0.0;
+        const double asum = block_reduce_sum(ea, sm.red);
+        lse_t = amax + m_log(asum);
+        tg_i = m_div(ea, asum);
         if (tid == 0) hdr->lse_t = lse_t;
+    } else {
+        tg_i = on ? m_exp(a_i - lse_t) : 0.0;
     }
     // ---- ratio order: decreasing log-ratio key, equal keys by smaller id (Sec. 5.1)
-    if (tid < k) { sm.key[tid] = b_i - a_i; sm.itmp[tid] = my_id; }
-    __syncthreads();
-    if (tid < k) {
-        const double ky = sm.key[tid];
+    // (the reductions above made the keys visible)
+    if (on) {
+        const double ky = b_i - a_i;
         int rank = 0;
+#pragma unroll 4
         for (int j = 0; j < k; j++) {
             const double kj = sm.key[j];
             rank += (kj > ky || (kj == ky && sm.itmp[j] < my_id)) ? 1 : 0;
         }
         sm.id[rank] = my_id;
-        sm.tg[rank] = exp(a_i - lse_t);
-        sm.d[rank] = exp(b_i - lse_d);
+        sm.tg[rank] = tg_i;
+        sm.d[rank] = m_div(eb, bsum);
     }
     __syncthreads();
     // ---- prefix sums in order, psi along the chain, H* and alpha* (Eq. "subset-select")
@@ -131,42 +145,63 @@ __device__ inline PrepResult prep_instance(const PrepSm& sm, const WsView& wv, H
         }
     }
     __syncthreads();
-    for (int j = 1 + tid; j <= k; j += blockDim.x) {
-        const double base = sm.Dr[j];
-        double pw = 1.0, sq = base;
+    // thread `pos` owns psi[pos + 1]
+    double v = 1.0e300;
+    if (on) {
+        double pw = 1.0, sq = sm.Dr[tid + 1];
+#pragma unroll 1
         for (int e = n; e > 0; e >>= 1) { if (e & 1) pw *= sq; sq *= sq; }
-        sm.psi[j] = sm.psi[j] - pw;
+        v = sm.psi[tid + 1] - pw;
+        sm.psi[tid + 1] = v;
+    }
+    // minimum of psi over the positions from this one up (inclusive of psi[pos + 1]): a suffix scan, exact in any order
+    double suf = v;
+#pragma unroll 1
+    for (int o = 1; o < 32; o <<= 1) {
+        const double t = __shfl_down_sync(0xffffffffu, suf, o);
+        if (lane + o < 32) suf = fmin(suf, t);
     }
     __syncthreads();
-    // first strict minimum of psi (H* = the prefix up to it), every thread for itself
-    int jstar = 0; double best = 0.0;
-    for (int j = 1; j <= k; j++) {
-        const double v = sm.psi[j];
-        if (v < best) { best = v; jstar = j; }
+    if (lane == 0) sm.red[warp] = suf;
+    __syncthreads();
+    double best = 0.0;                            // psi of the empty prefix
+#pragma unroll 1
+    for (int w2 = 0; w2 < kw; w2++) {
+        const double t = sm.red[w2];
+        best = fmin(best, t);
+        if (w2 > warp) suf = fmin(suf, t);
     }
+    // first strict minimum of psi (H* = the prefix up to it)
+    __syncthreads();
+    {
+        const unsigned hit = __ballot_sync(0xffffffffu, on && best < 0.0 && v == best);
+        if (lane == 0) sm.red[warp] = hit ? (double)(warp * 32 + __ffs(hit)) : 0.0;
+    }
+    __syncthreads();
+    int jstar = 0;
+#pragma unroll 1
+    for (int w2 = kw - 1; w2 >= 0; w2--) { const double t = sm.red[w2]; if (t > 0.0) jstar = (int)t; }
     // ---- outer residuals by cumulative minima along the increasing-ratio chain; blocks end at
-    //      every new strict minimum (Sec. 6.1, Thm "polymatroid", Lemma "q-convex").  One position per thread:
-    //      the running minimum that reaches a position is the minimum of psi over the positions above it
-    //      (exact in any order), and its block number counts the strict minima above it.
-    for (int pos = tid; pos < k; pos += blockDim.x) {
-        if (pos < jstar) {
-            sm.p[pos] = sm.tg[pos]; sm.r[pos] = 0.0; sm.blk[pos] = -1;
+    //      every new strict minimum (Sec. 6.1, Thm "polymatroid", Lemma "q-convex").  `suf` is the running minimum
+    //      that reaches this position; its block number counts the strict minima above it.
+    const bool outer = on && tid >= jstar;
+    const double c = on ? sm.psi[tid] : 0.0;
+    const unsigned recs = __ballot_sync(0xffffffffu, outer && c < suf);
+    if (lane == 0) sm.red[nw + warp] = (double)__popc(recs);
+    __syncthreads();
+    if (on) {
+        if (!outer) {
+            sm.p[tid] = sm.tg[tid]; sm.r[tid] = 0.0; sm.blk[tid] = -1;
         } else {
-            double m_prev = sm.psi[k];
-            int blk = 0;
-            for (int j = k - 1; j > pos; j--) {
-                const double c = sm.psi[j];
-                if (c < m_prev) { m_prev = c; blk++; }
-            }
-            const double c = sm.psi[pos];
-            const double rr = c < m_prev ? m_prev - c : 0.0;
-            sm.r[pos] = rr;
-            sm.p[pos] = sm.tg[pos] - rr;
-            sm.blk[pos] = blk;
-            if (pos == jstar) {
-                // the lowest position of the chain closes the last block: it is open unless this position is a record
-                sm.out3[1] = (double)(blk + 1);
-            }
+            int blk = __popc(recs & ~((2u << lane) - 1u));
+#pragma unroll 1
+            for (int w2 = warp + 1; w2 < kw; w2++) blk += (int)sm.red[nw + w2];
+            const double rr = c < suf ? suf - c : 0.0;
+            sm.r[tid] = rr;
+            sm.p[tid] = sm.tg[tid] - rr;
+            sm.blk[tid] = blk;
+            // the lowest position of the chain closes the last block: it is open unless this position is a record
+            if (tid == jstar) sm.out3[1] = (double)(blk + 1);
         }
     }
     if (tid == 0) {
@@ -176,8 +211,7 @@ __device__ inline PrepResult prep_instance(const PrepSm& sm, const WsView& wv, H
     }
     __syncthreads();
     PrepResult pr;
-    pr.k = k; pr.jstar = (int)sm.out3[0]; pr.nblocks = (int)sm.out3[1]; pr.alpha_star = sm.out3[2]; pr.lse_t = lse_t;
-    __syncthreads();
+    pr.k = k; pr.jstar = jstar; pr.nblocks = (int)sm.out3[1]; pr.alpha_star = 1.0 + best; pr.lse_t = lse_t;
     return pr;
 }
 
@@ -197,6 +231,7 @@ __device__ inline void truncation_sets(const PrepSm& sm, GR_PTR(int) in_T, GR_PT
         const double dv = sm.d[tid];
         const int iv = sm.id[tid];
         int rank = 0;
+#pragma unroll 1
         for (int j = lo; j < hi; j++) {
             const double dj = sm.d[j];
             rank += (dj > dv || (dj == dv && sm.id[j] < iv)) ? 1 : 0;
@@ -207,10 +242,12 @@ __device__ inline void truncation_sets(const PrepSm& sm, GR_PTR(int) in_T, GR_PT
     __syncthreads();
     if (tid == 0) {
         double D = 0.0;
+#pragma unroll 1
         for (int j = 0; j < jstar; j++) D += sm.d[j];
         auto powi = [](double x, int e) { double r = 1.0; while (e > 0) { if (e & 1) r *= x; x *= x; e >>= 1; } return r; };
         const double Dn = powi(D, n);
         double c = 0.0, gam = Dn;
+#pragma unroll 1
         for (int q = 0; q < jstar && gam > tau; q++) {
             const int pos = scratch[q];
             c += sm.d[pos]; in_T[pos] = 1;
@@ -218,6 +255,7 @@ __device__ inline void truncation_sets(const PrepSm& sm, GR_PTR(int) in_T, GR_PT
         }
         c = D;
         double eps = 1.0 - Dn;
+#pragma unroll 1
         for (int q = jstar; q < k && eps > tau; q++) {
             const int pos = scratch[q];
             c += sm.d[pos]; in_T[pos] = 1;
@@ -244,9 +282,28 @@ __device__ inline int gather_truncated(GR_PTR(const int) in_T, int lo, int hi, G
     return *count;
 }
 
-// Rule arrays (except w, which the solvers write as they go) and the header.
+// The header of a solved instance and the per-instance outputs, by thread 0, after the CTA has written the rule's arrays.
 // `check_flag` / `check_before`: the bounds-checked build's per-CTA flag and what the streaming kernel reported for
 // the row (nullptr / 0 otherwise): a skipped access turns the status into GR_CHECK_FAILED.
+__device__ inline void write_rule_header(const ParamView& pv, const PrepResult& pr, int n, int status, double gnorm,
+                                         int iters, float* alpha_out, int* status_out, long long b,
+                                         const int* check_flag, int check_before)
+{
+    if (threadIdx.x == 0) {
+        if (check_before || (check_flag && *check_flag)) status = GR_CHECK_FAILED;
+        Header* h = pv.h;
+        h->n = n; h->k = pr.k; h->jstar = pr.jstar; h->nblocks = pr.nblocks; h->status = status;
+        h->alpha_star = pr.alpha_star;
+        h->resid_total = 1.0 - pr.alpha_star;
+        h->gnorm = gnorm; h->iters = iters;
+        __threadfence();
+        h->magic = kMagic;
+        alpha_out[b] = (float)pr.alpha_star;
+        status_out[b] = status == kNeedFallback ? GR_NOT_CONVERGED : status;
+    }
+}
+
+// Rule arrays (except w, which the solvers write as they go) and the header.
 __device__ inline void write_rule(const PrepSm& sm, const ParamView& pv, int KP, const PrepResult& pr, int n,
                                   int status, double gnorm, int iters, float* alpha_out, int* status_out, long long b,
                                   const int* check_flag = nullptr, int check_before = 0)
@@ -261,18 +318,7 @@ __device__ inline void write_rule(const PrepSm& sm, const ParamView& pv, int KP,
         if (!in) pv.w[j] = 0.0;
     }
     __syncthreads();
-    if (tid == 0) {
-        if (check_before || (check_flag && *check_flag)) status = GR_CHECK_FAILED;
-        Header* h = pv.h;
-        h->n = n; h->k = pr.k; h->jstar = pr.jstar; h->nblocks = pr.nblocks; h->status = status;
-        h->alpha_star = pr.alpha_star;
-        h->resid_total = 1.0 - pr.alpha_star;
-        h->gnorm = gnorm; h->iters = iters;
-        __threadfence();
-        h->magic = kMagic;
-        alpha_out[b] = (float)pr.alpha_star;
-        status_out[b] = status == kNeedFallback ? GR_NOT_CONVERGED : status;
-    }
+    write_rule_header(pv, pr, n, status, gnorm, iters, alpha_out, status_out, b, check_flag, check_before);
 }
 
 }  // namespace gr

@@ -257,7 +257,7 @@ __device__ inline int selected_system(const int* draft_row, int n, int k, int js
 
 // Draw of instance b by warp 0 of a solve kernel's CTA, after the rule (or the no-rule header) was written and the
 // CTA synchronised.
-__device__ inline void fused_draw(const FusedArgs& fa, const Header* h, long long b, int n, void* scratch,
+static __device__ __noinline__ void fused_draw(const FusedArgs& fa, const Header* h, long long b, int n, void* scratch,
                                   int* check_flag = nullptr)
 {
     if (threadIdx.x >= 32) return;
