@@ -16,14 +16,22 @@ int launch_fast_n8_m128(GR_FAST_ARGS);
 int launch_fast_n16_m32(GR_FAST_ARGS);
 int launch_fast_n16_m64(GR_FAST_ARGS);
 int launch_fast_n16_m128(GR_FAST_ARGS);
+int launch_fast_c24_m32(GR_FAST_ARGS);
+int launch_fast_c24_m64(GR_FAST_ARGS);
+int launch_fast_c24_m128(GR_FAST_ARGS);
 }
 
 // Returns 1 when no fast variant covers the shape (the caller then runs the general kernel on everything);
 // after a return of 0 the caller runs the general kernel on the instances this one flagged (normally none).
 int launch_fast(GR_FAST_ARGS)
 {
-    if (kcap <= 0 || kcap > 128 || n > 16 || n < 2) return 1;
+    if (kcap <= 0 || kcap > 128 || n < 2) return 1;
 #define GR_FAST_PASS ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol, max_iters, qstep, tau, batch, alpha_out, status_out, fa, st
+    if (n > 16) {
+        if (kcap <= 32) return fast::launch_fast_c24_m32(GR_FAST_PASS);
+        if (kcap <= 64) return fast::launch_fast_c24_m64(GR_FAST_PASS);
+        return fast::launch_fast_c24_m128(GR_FAST_PASS);
+    }
     if (kcap <= 32) {
         if (n <= 4) return fast::launch_fast_n4_m32(GR_FAST_PASS);
         if (n <= 8) return fast::launch_fast_n8_m32(GR_FAST_PASS);

@@ -1,4 +1,4 @@
-// Fast per-instance solve for supports up to 128 tokens and n <= 16: one CTA per instance.
+// Fast per-instance solve for supports up to 128 tokens and n = 2 .. 32: one CTA per instance.
 //
 // Same mathematics as the general kernel (gr_solve.cu): the gradient of the convex functions
 // of the inner system / of an outer block (Thm "Inner Convex Solver", Thm "Outer Convex Solver")
@@ -18,6 +18,9 @@
 //     (node, series index): operands staged in shared memory in fp16, MMAs, fp32 accumulators in registers from the first node to
 //     the end of the factorisation.  The tokens are ordered by draft mass, so that the lower triangle pairs the series
 //     P h of the heavier token (all terms positive) with the h of the lighter one, and nothing cancels;
+//   - above 16 drafts the series give way to samples on a circle (eval_contour): the factors f_j are entire functions of
+//     lambda, so [lambda^n] is a mean over a few points of |lambda| = 0.8 n (conjugate pairs, 16 to 24 of them), exact to
+//     1e-11 and free of the cancellation that a dominant token brings into the division e / f as series;
 //   - the iteration runs in fp32 as long as the residual is far above fp32's noise; the last evaluations, the only ones
 //     that can end it, are fp64 on the full quadrature grid and reuse the last factorisation (a Newton step with a
 //     Hessian from a point 1e-4 away contracts as well as one with a fresh one).
@@ -54,32 +57,43 @@ constexpr int kFSweeps = 5;                // fixed-point sweeps of the starting
 template <int NT_, int MP_, int T_, int JC_, int CTAS_>
 struct Cfg {
     static constexpr int NT = NT_, MP = MP_, T = T_, JC = JC_, kCtas = CTAS_;
+    static constexpr bool kContour = NT > 16;     // samples on a circle instead of series (NT: largest number of them)
     static constexpr int kNG = T / MP;            // copies of the token threads (they share the nodes out among them)
     static constexpr int kW = T / 32, kTW = MP / 32;
     static constexpr int kRow = NT + 4;           // row stride of the product series (16-byte aligned rows in fp32 and fp64)
-        static constexpr int kTS = MP + 4;            // token stride of the staged operands: conflict-free fragment loads
+    static constexpr int kTS = MP + 4;            // token stride of the staged operands: conflict-free fragment loads
     static constexpr int kPanels = MP / 8;
     static constexpr int kPr = MP / 32;           // pairs of 16-row tiles (a, MP / 16 - 1 - a): equal work per pair
     static constexpr int kS = kW / kPr;           // warps that share a pair's column tiles
     static constexpr int kNA = (MP / 16 + kS - 1) / kS, kNB = (MP / 8 + kS - 1) / kS;
     static constexpr int kPack = NT >= 16 ? 1 : 16 / NT;   // Hessian nodes that fill one MMA depth of 16
-    static constexpr int kKS = JC / kPack;        // MMA steps per staged chunk
+    static constexpr int kKS = kContour ? (JC * NT + 7) / 8 : JC / kPack;   // MMA steps per staged chunk
     static_assert(T % MP == 0 && kW % kPr == 0 && kS * kNB <= MP / 8 && T >= kQC && JC % kPack == 0, "geometry");
     // shared memory, byte offsets
     static constexpr int oD = 0, oRhs = oD + MP * 8, oDr = oRhs + MP * 8, oWd = oDr + (MP + 4) * 8, oDsd = oWd + MP * 8;
     static constexpr int oRed = oDsd + MP * 8, oScal = oRed + 64 * 8, oTq = oScal + 16 * 8, oCq = oTq + kQC * 8, oKq = oCq + kQC * 8;
-    static constexpr int oPP = oKq + kQC * 4, oSP = oPP + kQC * kRow * 8;
-    static constexpr int oWf = oSP + T * (NT + 2) * 8, oDsf = oWf + MP * 4, oE = oDsf + MP * 4;
+    // (contour: x of every token and node in SP, samples of the product in PP, their square roots behind them (only the fp32
+    // evaluation, which leaves half of PP free, has them), tables of e^(lambda d) - 1
+    // in fp64 and fp32, and the samples' weights)
+    static constexpr int kXS = kQC + 1;
+    static constexpr int kPPBytes = kContour ? NT * kQC * 16 : kQC * kRow * 8;
+    static constexpr int kSPMin = T * 16 > MP * 16 ? T * 16 : MP * 16;
+    static constexpr int kSPBytes = !kContour ? T * (NT + 2) * 8 : (MP * kXS * 8 > kSPMin ? MP * kXS * 8 : kSPMin);
+    static constexpr int oPP = oKq + kQC * 4, oSP = oPP + kPPBytes, oSQ = oPP + NT * kQC * 8;
+    static constexpr int oEd = oSP + kSPBytes, oEs = oEd + (kContour ? NT * MP * 16 : 0);
+    static constexpr int oCd = oEs + (kContour ? NT * MP * 8 : 0);
+    static constexpr int oWf = oCd + (kContour ? NT * 16 : 0), oDsf = oWf + MP * 4, oE = oDsf + MP * 4;
     static constexpr int oDg = oE + (NT <= 8 ? MP * 32 : 0), oYv = oDg + MP * 4, oDl = oYv + MP * 4;
     static constexpr int oLd = oDl + MP * 4;                     // factored 8 x 8 diagonal blocks
     static constexpr int oBlk = oLd + kPanels * 64 * 4, oOrd = oBlk + MP * 4, oTr = oOrd + MP * 4;
     static constexpr int oU = (oTr + MP * 4 + 15) & ~15;           // union: staging / factor / start table / preparation
-    static constexpr int kStage = kKS * 4 * kTS * 8;               // bytes of one staged operand
+    static constexpr int kStage = kKS * 4 * kTS * 8;               // bytes of one staged operand (contour: the only one)
     static constexpr int kLFloats = 8 * (MP * kPanels - 4 * kPanels * (kPanels - 1));
     static constexpr int kNS = MP + 8;                             // row stride of the scaled Hessian (halves): conflict-free rows
     static constexpr int kPi = MP * kNS * 2;
     static constexpr int kPrep = MP * 8 * 3 + (MP + 4) * 8 + MP * 8;
-    static constexpr int kU0 = 2 * kStage > kLFloats * 4 ? 2 * kStage : kLFloats * 4;
+    static constexpr int kOps = kContour ? 1 : 2;
+    static constexpr int kU0 = kOps * kStage > kLFloats * 4 ? kOps * kStage : kLFloats * 4;
     static constexpr int kU1 = kPi > kPrep ? kPi : kPrep;
     static constexpr int kU2 = kU0 > kU1 ? kU0 : kU1;
     static constexpr int kU = kU2 > kVerifyScratchBytes ? kU2 : kVerifyScratchBytes;
@@ -126,13 +140,21 @@ struct FSm {
         ord = GR_MKPTR(int, reinterpret_cast<int*>(sb + C::oOrd), C::MP, ck);
         trunc = GR_MKPTR(int, reinterpret_cast<int*>(sb + C::oTr), C::MP, ck);
         AS = GR_MKPTR(uint32_t, reinterpret_cast<uint32_t*>(sb + C::oU), C::kStage / 4, ck);
-        HS = GR_MKPTR(uint32_t, reinterpret_cast<uint32_t*>(sb + C::oU + C::kStage), C::kStage / 4, ck);
+        HS = GR_MKPTR(uint32_t, reinterpret_cast<uint32_t*>(sb + C::oU + (C::kOps - 1) * C::kStage), C::kStage / 4, ck);
         kq = GR_MKPTR(float, reinterpret_cast<float*>(sb + C::oKq), kQC, ck);
         Lp = GR_MKPTR(float, reinterpret_cast<float*>(sb + C::oU), C::kLFloats, ck);
         pi = GR_MKPTR(__half, reinterpret_cast<__half*>(sb + C::oU), C::MP * C::kNS, ck);
     }
 };
-enum { SC_FAIL = 0, SC_PIVOT = 1, SC_OUT = 4 };
+enum { SC_FAIL = 0, SC_PIVOT = 1, SC_NP = 2, SC_OUT = 4 };
+
+// The circle of the contour kernels: `np` conjugate pairs of points r e^(i theta), angles theta and n theta (mod 2 pi),
+// factor 2 n! / (N r^n) of the mean.
+constexpr int kMaxPoints = 24;
+struct Circle { int np; double r, factor; double ct[kMaxPoints], st[kMaxPoints], nth[kMaxPoints]; };
+struct NoCircle {};
+template <bool> struct CircleOf { typedef NoCircle type; };
+template <> struct CircleOf<true> { typedef Circle type; };
 
 // Arrays whose element type is the precision of the evaluation.
 template <class C, typename R>
@@ -141,8 +163,8 @@ struct RSm {
     __device__ explicit RSm(const FSm<C>& sm) {
         tq = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oTq), kQC, sm.flag);
         cq = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oCq), kQC, sm.flag);
-        PP = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oPP), kQC * C::kRow, sm.flag);
-        SP = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oSP), C::T * (C::NT + 2) * (8 / (int)sizeof(R)), sm.flag);
+        PP = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oPP), C::kPPBytes / (int)sizeof(R), sm.flag);
+        SP = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oSP), C::kSPBytes / (int)sizeof(R), sm.flag);
         const int ow = sizeof(R) == 4 ? C::oWf : C::oWd, od = sizeof(R) == 4 ? C::oDsf : C::oDsd;
         w = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + ow), C::MP, sm.flag);
         ds = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + od), C::MP, sm.flag);
@@ -310,6 +332,11 @@ __device__ __forceinline__ void hess_mma(const FSm<C>& sm, Frags<C>& fr, int kst
         uint2 hv[C::kNB];
 #pragma unroll
         for (int s = 0; s < C::kNB; s++) hv[s] = ld_u2(Hp + 16 * (cs + s * C::kS));
+        if (C::kContour) {
+            // Re(a b) = Re a Re b - Im a Im b
+#pragma unroll
+            for (int s = 0; s < C::kNB; s++) { hv[s].x ^= 0x80000000u; hv[s].y ^= 0x80000000u; }
+        }
         const uint2 a0 = ld_u2(Ap + 32 * ra), a1 = ld_u2(Ap + 32 * ra + 16), b0 = ld_u2(Ap + 32 * rb), b1 = ld_u2(Ap + 32 * rb + 16);
         const uint32_t fa[4] = {a0.x, a1.x, a0.y, a1.y}, fb[4] = {b0.x, b1.x, b0.y, b1.y};
 #pragma unroll
@@ -319,6 +346,209 @@ __device__ __forceinline__ void hess_mma(const FSm<C>& sm, Frags<C>& fr, int kst
             mma_f16(fr.B[s], fb, bb);
         }
     }
+}
+
+// Quadrature grid in the log-time variable for log-weights in [amin, amax]: number of nodes, upper end, start of the
+// lower-tail compression.  (Where the grid lies does not matter to its accuracy: fp32.)
+__device__ __forceinline__ int quad_grid(float amax, float amin, int slack, float qstep, float& s_hi, float& s0)
+{
+    const float wmax = Rx<float>::ex(amax), wmin = Rx<float>::ex(amin);
+    s_hi = Rx<float>::lg((float)kFTEnd / (slack ? 1.f + wmin : wmin));
+    s0 = -Rx<float>::lg((slack ? 1.f : 0.f) + wmax) - (float)kFDrop;
+    const int Q = (int)ceilf((s_hi - (s0 - (float)kFTail)) / qstep) + 1;
+    return Q > kFMaxNodes ? kFMaxNodes : Q;
+}
+
+// Sum of (g, g2) over the copies of the token threads, in the same order everywhere.
+template <class C>
+__device__ __forceinline__ void sum_copies(const FSm<C>& sm, double& g, double& g2)
+{
+    if (C::kNG > 1) {
+        const int tid = threadIdx.x, i = tid % C::MP;
+        GR_PTR(double) gs = GR_MKPTR(double, reinterpret_cast<double*>(sm.base + C::oSP), C::kSPBytes / 8, sm.flag);
+        gs[2 * tid] = g; gs[2 * tid + 1] = g2;
+        __syncthreads();
+        g = 0.0; g2 = 0.0;
+#pragma unroll
+        for (int k = 0; k < C::kNG; k++) { g += gs[2 * (k * C::MP + i)]; g2 += gs[2 * (k * C::MP + i) + 1]; }
+        __syncthreads();
+    }
+}
+
+// Arrays of the contour kernels; complex numbers are pairs of R.
+template <class C, typename R>
+struct CSm {
+    GR_PTR(R) tq, cq, X, P, E, c, w;
+    GR_PTR(float) sq;
+    __device__ explicit CSm(const FSm<C>& sm) {
+        constexpr int k = (int)sizeof(R);
+        tq = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oTq), kQC, sm.flag);
+        cq = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oCq), kQC, sm.flag);
+        X = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oSP), C::MP * C::kXS, sm.flag);
+        P = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oPP), 2 * C::NT * kQC, sm.flag);
+        E = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + (k == 4 ? C::oEs : C::oEd)), 2 * C::NT * C::MP, sm.flag);
+        w = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + (k == 4 ? C::oWf : C::oWd)), C::MP, sm.flag);
+        sq = GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oSQ), 2 * C::NT * kQC, sm.flag);
+    }
+};
+template <class P> __device__ __forceinline__ void ld_c(const P& p, float& a, float& b) { const float2 v = ld_f2(p); a = v.x; b = v.y; }
+template <class P> __device__ __forceinline__ void ld_c(const P& p, double& a, double& b) { const double2 v = ld_d2(p); a = v.x; b = v.y; }
+template <class P> __device__ __forceinline__ void st_c(const P& p, float a, float b) { st_f2(p, make_float2(a, b)); }
+template <class P> __device__ __forceinline__ void st_c(const P& p, double a, double b) { st_d2(p, make_double2(a, b)); }
+
+// Tables of a system for the contour: e^(lambda_p d_j) - 1 for every point and token, and the points' weights
+// 2 n! / (N r^n) e^(-i n theta_p) e^(lambda_p h) T^n, with the masses relative to the system's total T.
+template <class C>
+__device__ __noinline__ void contour_tables(const Circle& ci, int m, double rel, double hrel, double Tn, int* flag)
+{
+    const FSm<C> sm(flag);
+    const CSm<C, double> cd(sm);
+    const CSm<C, float> cf(sm);
+    GR_PTR(double) cw = GR_MKPTR(double, reinterpret_cast<double*>(sm.base + C::oCd), 2 * C::NT, flag);
+    const int tid = threadIdx.x, i = tid % C::MP;
+    for (int p = tid / C::MP; p < ci.np; p += C::kNG) {
+        double sn = 0.0, cs = 1.0, e = 1.0;
+        if (i < m) { sincos(ci.r * ci.st[p] * rel, &sn, &cs); e = m_exp(ci.r * ci.ct[p] * rel); }
+        const double re = e * cs - 1.0, im = e * sn;
+        st_d2(cd.E + 2 * (p * C::MP + i), make_double2(re, im));
+        st_f2(cf.E + 2 * (p * C::MP + i), make_float2((float)re, (float)im));
+    }
+    if (tid < ci.np) {
+        double sn, cs;
+        sincos(ci.r * ci.st[tid] * hrel - ci.nth[tid], &sn, &cs);
+        const double e = m_exp(ci.r * ci.ct[tid] * hrel) * ci.factor * Tn;
+        st_d2(cw + 2 * tid, make_double2(e * cs, e * sn));
+    }
+    if (tid == 0) sm.scal[SC_NP] = (double)ci.np;
+}
+
+__device__ __forceinline__ float recip(float x) { return __fdividef(1.f, x); }
+__device__ __forceinline__ double recip(double x) { return __drcp_rn(x); }
+
+// As eval_system (same arguments and results), with [lambda^n] taken as a mean over points of a circle:
+//   M = sum_p c_p prod_j f_pj,  dM/dx_i = sum_p Re(P_p h_pi),  d2M/dx_i dx_l = sum_p Re(P_p h_pi h_pl),
+//   f_pj = 1 + x_j E_pj,  h = E / f,  E_pj = e^(lambda_p d_j) - 1 (tables).
+// The rounded f that went into the product is the one that is divided out again, so a factor close to zero does no harm.
+// For the Hessian sqrt(P_p) h_pi is staged, once, as (Re, Im) half pairs: products of two such are of order one, whatever
+// the token's mass.  Errors against 96 points and fp64 throughout, n = 17 to 32, largest mass 0.12 to 0.6: flows 1e-11 in
+// fp64, 1e-7 in fp32; scaled Hessian 2e-5 from 11-bit operands.
+template <class C, typename R, bool kJac>
+__device__ __forceinline__ void eval_contour(const FSm<C>& sm, int m, int slack, double qstep_d, int jstride, float amax,
+                                             float amin, double w_own, float z_own, double& g_out, double& g2_out, Frags<C>& fr)
+{
+    constexpr int T = C::T;
+    const CSm<C, R> cs(sm);
+    GR_PTR(double) cw = GR_MKPTR(double, reinterpret_cast<double*>(sm.base + C::oCd), 2 * C::NT, sm.flag);
+    const int tid = threadIdx.x, i = tid % C::MP, ng = tid / C::MP;
+    const int np = (int)sm.scal[SC_NP];
+    const R qstep = (R)qstep_d, wi = (R)w_own;
+    float s_hi, s0;
+    const int Q = quad_grid(amax, amin, slack, (float)qstep_d, s_hi, s0);
+    R g = R(0), g2 = R(0);
+    if (kJac) {
+#pragma unroll
+        for (int s = 0; s < C::kNA; s++) { fr.A[s][0] = fr.A[s][1] = fr.A[s][2] = fr.A[s][3] = 0.f; }
+#pragma unroll
+        for (int s = 0; s < C::kNB; s++) { fr.B[s][0] = fr.B[s][1] = fr.B[s][2] = fr.B[s][3] = 0.f; }
+    }
+    const bool live = kJac || (i & ~31) < m;
+#pragma unroll 1
+    for (int q0 = 0; q0 < Q; q0 += kQC) {
+        const int nq = min(kQC, Q - q0);
+        const int slots = nq <= 16 ? 16 : 32;
+        const int q = tid & (slots - 1), G = T / slots, grp = tid / slots;
+        // ---- x of every token at this thread's node
+        const R s = (R)s_hi - qstep * (R)(q0 + q);
+        const R e = Rx<R>::expneg(s - (R)s0);
+        const R t = Rx<R>::expneg(e - s);
+        if (tid < nq) {
+            const R c0 = qstep * (R(1) + e) * t * (slack ? Rx<R>::expneg(t) : R(1));
+            cs.tq[q] = t; cs.cq[q] = c0;
+            if (kJac) sm.kq[q] = sqrtf((float)((R)jstride * c0 * t));
+        }
+#pragma unroll 2
+        for (int j = grp; j < m; j += G) cs.X[j * C::kXS + q] = Rx<R>::expneg(t * cs.w[j]);
+        __syncthreads();
+        // ---- product of the factors, one thread per (node, point)
+        if (q < nq) {
+#pragma unroll 1
+            for (int p = grp; p < np; p += G) {
+                R a = (R)cw[2 * p], b = (R)cw[2 * p + 1];
+#pragma unroll 4
+                for (int j = 0; j < m; j++) {
+                    const R x = cs.X[j * C::kXS + q];
+                    R er, ei;
+                    ld_c(cs.E + 2 * (p * C::MP + j), er, ei);
+                    const R fx = fma(x, er, R(1)), fy = x * ei;
+                    const R a2 = fma(a, fx, -(b * fy));
+                    b = fma(a, fy, b * fx);
+                    a = a2;
+                }
+                st_c(cs.P + 2 * (p * kQC + q), a, b);
+                if (kJac) {
+                    // square root, either branch: only products of two of them are used
+                    const float af = (float)a, bf = (float)b, mag = sqrtf(fmaf(af, af, bf * bf));
+                    const float u = sqrtf(0.5f * (mag + fabsf(af))), v = u > 0.f ? __fdividef(0.5f * bf, u) : 0.f;
+                    st_c(cs.sq + 2 * (p * kQC + q), af >= 0.f ? u : fabsf(v), af >= 0.f ? v : copysignf(u, bf));
+                }
+            }
+        }
+        __syncthreads();
+        // ---- g: one thread per token; with kJac the operands of the contraction for every jstride-th node
+        const int span = kJac ? jstride * C::JC : nq;
+#pragma unroll 1
+        for (int qa = 0; qa < nq; qa += span) {
+            const int qb = min(nq, qa + span);
+            const int nst = kJac ? (qb - qa + jstride - 1) / jstride : 0;
+            if (live) {
+#pragma unroll 1
+                for (int q2 = qa + ng; q2 < qb; q2 += C::kNG) {
+                    const R t2 = cs.tq[q2], c0 = cs.cq[q2];
+                    const R x = i < m ? cs.X[i * C::kXS + q2] : R(0);
+                    const R ux = wi * x;
+                    const bool stage = kJac && (jstride == 1 || ((q2 - qa) & 1) == 0);
+                    const float uz = stage ? sm.kq[q2] * (float)ux * z_own : 0.f;
+                    const int f0 = stage ? (q2 - qa) / jstride * np : 0;
+                    R v0 = R(0), v1 = R(0);
+#pragma unroll 4
+                    for (int p = 0; p < np; p++) {
+                        R er, ei, pr, pi;
+                        ld_c(cs.E + 2 * (p * C::MP + i), er, ei);
+                        ld_c(cs.P + 2 * (p * kQC + q2), pr, pi);
+                        const R fx = fma(x, er, R(1)), fy = x * ei;
+                        const R inv = recip(fma(fx, fx, fy * fy));
+                        // h = E conj(f) / |f|^2
+                        const R ix = fx * inv, iy = fy * inv;
+                        const R hr = fma(er, ix, ei * iy), hi = fma(ei, ix, -(er * iy));
+                        v0 = fma(pr, hr, v0); v1 = fma(-pi, hi, v1);
+                        if (kJac && stage) {
+                            float sr, si;
+                            ld_c(cs.sq + 2 * (p * kQC + q2), sr, si);
+                            const float a = uz * (float)hr, b = uz * (float)hi;
+                            const int f = f0 + p;
+                            sm.AS[((f >> 3) * 4 + (f & 3)) * 2 * C::kTS + 2 * i + ((f >> 2) & 1)] =
+                                pack_half(fmaf(sr, a, -(si * b)), fmaf(sr, b, si * a));
+                        }
+                    }
+                    const R gi = c0 * ux * (v0 + v1);
+                    g += gi;
+                    g2 = fma(gi * t2, wi, g2);
+                }
+            }
+            if (kJac) {
+                // unused slots of the last MMA depth
+                const int tot = nst * np;
+                for (int f = tot + ng; f < ((tot + 7) & ~7); f += C::kNG)
+                    sm.AS[((f >> 3) * 4 + (f & 3)) * 2 * C::kTS + 2 * i + ((f >> 2) & 1)] = 0u;
+                __syncthreads();
+                hess_mma<C>(sm, fr, (tot + 7) >> 3);
+                __syncthreads();
+            }
+        }
+        if (!kJac) __syncthreads();
+    }
+    g_out = (double)g; g2_out = (double)g2;
+    sum_copies<C>(sm, g_out, g2_out);
 }
 
 // Gradient g and the Hessian's diagonal part g2 at the weights in shared memory (this thread's in w_own), in fp64; or in
@@ -336,13 +566,8 @@ __device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, doub
     const RSm<C, R> rs(sm);
     const int tid = threadIdx.x, i = tid % C::MP, ng = tid / C::MP;
     const R qstep = (R)qstep_d;
-    // (where the grid lies does not matter to its accuracy: fp32)
-    const float wmax = Rx<float>::ex(amax), wmin = Rx<float>::ex(amin);
-    const float f_hi = Rx<float>::lg((float)kFTEnd / (slack ? 1.f + wmin : wmin));
-    const float f_0 = -Rx<float>::lg((slack ? 1.f : 0.f) + wmax) - (float)kFDrop;
-    int Q = (int)ceilf((f_hi - (f_0 - (float)kFTail)) / (float)qstep_d) + 1;
-    if (Q > kFMaxNodes) Q = kFMaxNodes;
-    const R s_hi = (R)f_hi, s0 = (R)f_0;
+    float s_hi, s0;
+    const int Q = quad_grid(amax, amin, slack, (float)qstep_d, s_hi, s0);
     const R wi = (R)w_own, dsi = (R)ds_own;
     R dp[NT <= 8 ? NT + 1 : 1];
     if (NT <= 8) {
@@ -366,8 +591,8 @@ __device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, doub
         const int q = tid & (narrow ? 15 : 31), G = T / (narrow ? 16 : 32), grp = tid / (narrow ? 16 : 32);
         constexpr int kSS = sizeof(R) == 4 ? NT + 4 : NT + 2;      // row stride of the shares: conflict-free vector access
         {
-            const R s = s_hi - qstep * (R)(q0 + q);
-            const R e = Rx<R>::expneg(s - s0);
+            const R s = (R)s_hi - qstep * (R)(q0 + q);
+            const R e = Rx<R>::expneg(s - (R)s0);
             const R t = Rx<R>::expneg(e - s);
             if (tid < nq) {
                 const R c0 = qstep * (R(1) + e) * t * (slack ? Rx<R>::expneg(t) : R(1));
@@ -534,18 +759,8 @@ __device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, doub
         }
         if (!kJac) __syncthreads();
     }
-    double gd = (double)g, g2d = (double)g2;
-    if (C::kNG > 1) {
-        // sum over the copies, in the same order everywhere
-        GR_PTR(double) gs = GR_MKPTR(double, reinterpret_cast<double*>(sm.base + C::oSP), C::T * (C::NT + 2), sm.flag);
-        gs[2 * tid] = gd; gs[2 * tid + 1] = g2d;
-        __syncthreads();
-        gd = 0.0; g2d = 0.0;
-#pragma unroll
-        for (int k = 0; k < C::kNG; k++) { gd += gs[2 * (k * C::MP + i)]; g2d += gs[2 * (k * C::MP + i) + 1]; }
-        __syncthreads();
-    }
-    g_out = gd; g2_out = g2d;
+    g_out = (double)g; g2_out = (double)g2;
+    sum_copies<C>(sm, g_out, g2_out);
 }
 
 // The fp64 evaluation, kept out of line (it is called once or twice per system, and its registers stay its own).
@@ -556,7 +771,8 @@ __device__ __noinline__ double2 eval_fp64(int m, int n, double hs, int slack, do
     const FSm<C> sm(flag);
     Frags<C> none;
     double2 r;
-    eval_system<C, double, false>(sm, m, n, hs, slack, qstep, 1, amax, amin, w_own, ds_own, 0.f, r.x, r.y, none);
+    if constexpr (C::kContour) eval_contour<C, double, false>(sm, m, slack, qstep, 1, amax, amin, w_own, 0.f, r.x, r.y, none);
+    else eval_system<C, double, false>(sm, m, n, hs, slack, qstep, 1, amax, amin, w_own, ds_own, 0.f, r.x, r.y, none);
     return r;
 }
 
@@ -809,7 +1025,8 @@ __device__ __noinline__ double2 eval_hessian(int m, int n, double hs, int slack,
     Frags<C> fr;
     double g, g2;
     const float zr = i < m ? (float)rhs : 1.f, zi = rsqrtf(zr);
-    eval_system<C, float, true>(sm, m, n, hs, slack, qstep, jstride, amax, amin, w_own, ds_own, i < m ? zi : 0.f, g, g2, fr);
+    if constexpr (C::kContour) eval_contour<C, float, true>(sm, m, slack, qstep, jstride, amax, amin, w_own, i < m ? zi : 0.f, g, g2, fr);
+    else eval_system<C, float, true>(sm, m, n, hs, slack, qstep, jstride, amax, amin, w_own, ds_own, i < m ? zi : 0.f, g, g2, fr);
     if (given) { g = gg.x; g2 = gg.y; }
     if (chol) {
         // an outer block's function is constant along (1,...,1): that direction is pinned with 1/m everywhere
@@ -1095,7 +1312,8 @@ __device__ __noinline__ double start_point(int m, int slack, int n, double d_i, 
 
 // Newton iteration for one system.  Returns the status; w_out = exp(alpha) of this thread's token at the last accepted point.
 template <class C>
-__device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, int n, double sigma, double tol, int max_iters,
+__device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, const typename CircleOf<C::kContour>::type& circle,
+                                           int n, double sigma, double tol, int max_iters,
                                            double qstep, double* gnorm, int* iters, double* w_out)
 {
     const int tid = threadIdx.x, i = tid % C::MP;
@@ -1114,7 +1332,10 @@ __device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, i
 
     double alpha = start_point<C>(m, slack, n, d_i, rhs_i, Tm, sm.flag);
     // scaled draft masses (and at short series their powers) for the evaluations
-    if (lead) {
+    if constexpr (C::kContour) {
+        const double iT = m_div(1.0, Tm);
+        contour_tables<C>(circle, m, d_i * iT, sy.hmass * iT, Tn, sm.flag);
+    } else if (lead) {
         sm.dsd[i] = ds_i;
         RSm<C, float> rs(sm);
         rs.ds[i] = (float)ds_i;
@@ -1133,7 +1354,7 @@ __device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, i
     // fp64 gradient, fp32 Hessian of the same point, with `chol` a Cholesky factorisation.  A single token that dominates a
     // long series (its terms would cancel in fp32) starts in the last mode.
     enum { kLow, kChord, kHigh };
-    int mode = (C::NT <= 8 || dmax < 0.6 * Tm) ? kLow : kHigh;
+    int mode = (C::NT <= 8 || C::kContour || dmax < 0.6 * Tm) ? kLow : kHigh;
     bool full_grid = false, predicted = false, chol = false;
 #pragma unroll 1
     for (; it < max_iters; it++) {
@@ -1284,7 +1505,8 @@ template <class C>
 __global__ void __launch_bounds__(C::T, C::kCtas)
 fast_solve_kernel(const char* __restrict__ ws, char* __restrict__ params, int pstride, int kcap, int V, int n, int topk,
                   double temp_t, double temp_d, double tol, int max_iters, double qstep, double tau, double sigma,
-                  float* __restrict__ alpha_out, int* __restrict__ status_out, FusedArgs fa)
+                  float* __restrict__ alpha_out, int* __restrict__ status_out, FusedArgs fa,
+                  const __grid_constant__ typename CircleOf<C::kContour>::type circle)
 {
     __shared__ int s_sel;
     GR_CHECK_FLAG_DECL;
@@ -1383,7 +1605,7 @@ fast_solve_kernel(const char* __restrict__ ws, char* __restrict__ params, int ps
             System sy;
             sy.m = m; sy.slack = inner ? 1 : 0; sy.hmass = hm;
             double gn, w; int it;
-            const int st = fast_system<C>(sm, sy, n, sigma, tol, max_iters, qstep, &gn, &it, &w);
+            const int st = fast_system<C>(sm, sy, circle, n, sigma, tol, max_iters, qstep, &gn, &it, &w);
             if (st != GR_OK) status = kNeedFallback;
             gnorm_total += gn; iters_total = add_iters(iters_total, it);
             if (tid < m) pv.w[sm.ord[tid]] = w;
@@ -1418,8 +1640,21 @@ int launch_fast_t(const char* ws, char* params, int pstride, int kcap, int V, in
         configured[dev] = true;
     }
     const double sigma = exp(lgamma((double)n + 1.0) / (double)n);       // sigma^n = n!
+    typename CircleOf<C::kContour>::type circle;
+    if constexpr (C::kContour) {
+        // N points, a multiple of eight and at least n + 12: what is folded onto [lambda^n] from [lambda^(n + N)] is below
+        // 1e-11 of it at this radius, and the mean loses one digit only (the saddle lies at |lambda| = n)
+        const int N = 8 * ((n + 12 + 7) / 8);
+        circle.np = N / 2;
+        circle.r = 0.8 * (double)n;
+        circle.factor = 2.0 / (double)N * exp(lgamma((double)n + 1.0) - (double)n * log(circle.r));
+        for (int p = 0; p < circle.np; p++) {
+            const double th = ((double)p + 0.5) * 2.0 * 3.14159265358979323846 / (double)N;
+            circle.ct[p] = cos(th); circle.st[p] = sin(th); circle.nth[p] = fmod((double)n * th, 2.0 * 3.14159265358979323846);
+        }
+    }
     fast_solve_kernel<C><<<batch, C::T, C::kBytes, st>>>(ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol,
-                                                         max_iters, qstep, tau, sigma, alpha_out, status_out, fa);
+                                                         max_iters, qstep, tau, sigma, alpha_out, status_out, fa, circle);
     return GR_OK;
 }
 

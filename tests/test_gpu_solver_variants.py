@@ -1,0 +1,29 @@
+"""The solve kernels at the sizes where a variant can go wrong: supports around the padded sizes (32, 64, 128) and the
+16-row tiles, draft counts at both ends of every series length and number of circle points.  Every instance against the
+oracle: structure, optimal acceptance and the gradient norm at the GPU's weights."""
+import pytest
+import torch
+
+import paper_2511_15898_b200 as G
+from paper_2511_15898_b200 import workloads as W
+from paper_2511_15898_b200.build import build_library
+from tests import parity as P
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build_library()
+    G.load_library()
+
+
+@pytest.mark.parametrize("n", [2, 4, 5, 8, 9, 16, 17, 20, 21, 28, 29, 32])
+@pytest.mark.parametrize("topk", [2, 16, 17, 32, 33, 64, 65, 128])
+def test_draft_counts_and_supports_at_the_edges(n, topk):
+    wl = W.config3(batch=3, device="cuda", seed=9000 + 40 * topk + n, V=2000, n=n, topk=topk)
+    rep = P.certify(wl)
+    print(rep.summary())
+    assert rep.n_status_ok == rep.n_inst and rep.n_struct_mismatch == 0, (rep.summary(), rep.details[:5])
+    assert rep.alpha_err <= 1e-6 and rep.cert_solver_max <= 3.2e-7, rep.summary()
+    assert rep.n_underreported == 0 and rep.n_evaluated_off == 0, (rep.summary(), rep.details[:5])
