@@ -15,6 +15,8 @@ alpha_kernel(const char* __restrict__ ws, int V, int topk, double temp_t, double
     __shared__ double s_key[kMaxSupport], s_tg[kMaxSupport], s_d[kMaxSupport], s_Tg[kMaxSupport + 1], s_Dr[kMaxSupport + 1];
     __shared__ int s_id[kMaxSupport];
     __shared__ double s_red[32];
+    pdl_wait();
+    pdl_trigger();
     const int tid = threadIdx.x;
     const long long b = blockIdx.x;
     const WsView wv = view_ws(ws, b);
@@ -88,7 +90,7 @@ void launch_alpha(const char* ws, int V, int topk, double temp_t, double temp_d,
     NList nl;
     nl.count = n_count;
     for (int i = 0; i < GR_MAX_ALPHA_N; i++) nl.n[i] = i < n_count ? n_list[i] : 1;
-    alpha_kernel<<<batch, kAlphaThreads, 0, st>>>(ws, V, topk, temp_t, temp_d, nl, alpha_out, status_out);
+    launch_pdl(alpha_kernel, batch, kAlphaThreads, 0, st, ws, V, topk, temp_t, temp_d, nl, alpha_out, status_out);
 }
 
 }  // namespace gr

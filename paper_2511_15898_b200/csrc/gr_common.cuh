@@ -219,6 +219,23 @@ static __device__ __noinline__ double m_exp(double x) { return exp(x); }
 static __device__ __noinline__ double m_log(double x) { return log(x); }
 static __device__ __noinline__ double m_div(double a, double b) { return a / b; }
 
+// Programmatic dependent launch.  Every kernel of a call is launched with launch_pdl and begins with these two: it may be
+// scheduled, and its CTAs take the places that its predecessor's last wave leaves, before the predecessor has ended, but it
+// touches no memory until the predecessor has completed (which, by the same rule, had waited for its own).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = st; cfg.attrs = &at; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 constexpr int kMaxDevices = 64;               // per-device caches of the host code (function attributes, streams)
 
 }  // namespace gr

@@ -1509,6 +1509,8 @@ fast_solve_kernel(const char* __restrict__ ws, char* __restrict__ params, int ps
                   const __grid_constant__ typename CircleOf<C::kContour>::type circle)
 {
     __shared__ int s_sel;
+    pdl_wait();
+    pdl_trigger();
     GR_CHECK_FLAG_DECL;
     GR_CHECK_FLAG_INIT;
     const bool fused = fa.draft != nullptr;
@@ -1653,8 +1655,8 @@ int launch_fast_t(const char* ws, char* params, int pstride, int kcap, int V, in
             circle.ct[p] = cos(th); circle.st[p] = sin(th); circle.nth[p] = fmod((double)n * th, 2.0 * 3.14159265358979323846);
         }
     }
-    fast_solve_kernel<C><<<batch, C::T, C::kBytes, st>>>(ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol,
-                                                         max_iters, qstep, tau, sigma, alpha_out, status_out, fa, circle);
+    launch_pdl(fast_solve_kernel<C>, batch, C::T, C::kBytes, st, ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol,
+               max_iters, qstep, tau, sigma, alpha_out, status_out, fa, circle);
     return GR_OK;
 }
 

@@ -75,6 +75,8 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, int
                     int out_stride, int out_off, int* __restrict__ status_out)
 {
     extern __shared__ __align__(16) unsigned char bk_smem[];
+    pdl_wait();
+    pdl_trigger();
     GR_CHECK_FLAG_DECL;
     GR_CHECK_FLAG_INIT;
     unsigned long long* const bt_raw = reinterpret_cast<unsigned long long*>(bk_smem);
@@ -269,6 +271,8 @@ fullsort_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, i
     __shared__ double s_a[kFsThreads / 32], s_b[kFsThreads / 32];
     __shared__ double s_carry[2];
     __shared__ double s_min[kFsThreads / 32];
+    pdl_wait();
+    pdl_trigger();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long b = blockIdx.x;
     const WsHeader* wh = reinterpret_cast<const WsHeader*>(ws + (size_t)b * ws_stride());
@@ -443,22 +447,22 @@ void launch_fullsort(const void* q, const void* p, int dtype, int V, int n, doub
     }
     const size_t sstride = (size_t)next_pow2(V) * 12;
     if (dtype == GR_F32)
-        bucket_alpha_kernel<float><<<batch, kBkThreads, kBkSmemBytes, st>>>((const float*)q, (const float*)p, V, n, temp_t,
+        launch_pdl(bucket_alpha_kernel<float>, batch, kBkThreads, kBkSmemBytes, st, (const float*)q, (const float*)p, V, n, temp_t,
                                                                             temp_d, ws, scratch, sstride, params, pstride,
                                                                             force_sort, alpha_out, out_stride, out_off,
                                                                             status_out);
     else
-        bucket_alpha_kernel<__nv_bfloat16><<<batch, kBkThreads, kBkSmemBytes, st>>>((const __nv_bfloat16*)q,
+        launch_pdl(bucket_alpha_kernel<__nv_bfloat16>, batch, kBkThreads, kBkSmemBytes, st, (const __nv_bfloat16*)q,
                                                                                     (const __nv_bfloat16*)p, V, n, temp_t,
                                                                                     temp_d, ws, scratch, sstride, params,
                                                                                     pstride, force_sort, alpha_out, out_stride,
                                                                                     out_off, status_out);
     if (dtype == GR_F32)
-        fullsort_alpha_kernel<float><<<batch, kFsThreads, kFsSmemBytes, st>>>((const float*)q, (const float*)p, V, n, temp_t,
+        launch_pdl(fullsort_alpha_kernel<float>, batch, kFsThreads, kFsSmemBytes, st, (const float*)q, (const float*)p, V, n, temp_t,
                                                                    temp_d, ws, scratch, params, pstride, alpha_out,
                                                                    out_stride, out_off);
     else
-        fullsort_alpha_kernel<__nv_bfloat16><<<batch, kFsThreads, kFsSmemBytes, st>>>((const __nv_bfloat16*)q,
+        launch_pdl(fullsort_alpha_kernel<__nv_bfloat16>, batch, kFsThreads, kFsSmemBytes, st, (const __nv_bfloat16*)q,
                                                                            (const __nv_bfloat16*)p, V, n, temp_t,
                                                                            temp_d, ws, scratch, params, pstride,
                                                                            alpha_out, out_stride, out_off);

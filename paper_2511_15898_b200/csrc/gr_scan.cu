@@ -176,6 +176,8 @@ scan_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, int ksel, f
     __shared__ float2 s_chunk_raw[kMaxChunks];
     __shared__ float s_dm[kScanWarps], s_ds[kScanWarps];
     __shared__ int s_hist_raw[256];
+    pdl_wait();
+    pdl_trigger();
     GR_CHECK_FLAG_DECL;
     GR_CHECK_FLAG_INIT;
     GR_PTR(unsigned long long) s_keys = GR_MKPTR(unsigned long long, s_keys_raw, kCandCap, GR_CHECK_FLAG);
@@ -428,21 +430,20 @@ void launch_scan(const void* q, const void* p, int dtype, int V, int ksel, bool 
 {
     const double log2e = 1.4426950408889634;
     float sc_t = (float)(log2e / temp_t), sc_d = (float)(log2e / temp_d);
-    dim3 grid(batch), block(kScanThreads);
     if (dtype == GR_F32) {
         if (full_large)
-            scan_kernel<float, true><<<grid, block, 0, st>>>((const float*)q, (const float*)p, V, ksel, sc_t, sc_d,
+            launch_pdl(scan_kernel<float, true>, batch, kScanThreads, 0, st, (const float*)q, (const float*)p, V, ksel, sc_t, sc_d,
                                                                temp_t, temp_d, ws, params, pstride, kcap);
         else
-            scan_kernel<float, false><<<grid, block, 0, st>>>((const float*)q, (const float*)p, V, ksel, sc_t, sc_d,
+            launch_pdl(scan_kernel<float, false>, batch, kScanThreads, 0, st, (const float*)q, (const float*)p, V, ksel, sc_t, sc_d,
                                                                 temp_t, temp_d, ws, params, pstride, kcap);
     } else {
         if (full_large)
-            scan_kernel<__nv_bfloat16, true><<<grid, block, 0, st>>>((const __nv_bfloat16*)q, (const __nv_bfloat16*)p,
+            launch_pdl(scan_kernel<__nv_bfloat16, true>, batch, kScanThreads, 0, st, (const __nv_bfloat16*)q, (const __nv_bfloat16*)p,
                                                                        V, ksel, sc_t, sc_d, temp_t, temp_d, ws, params,
                                                                        pstride, kcap);
         else
-            scan_kernel<__nv_bfloat16, false><<<grid, block, 0, st>>>((const __nv_bfloat16*)q, (const __nv_bfloat16*)p,
+            launch_pdl(scan_kernel<__nv_bfloat16, false>, batch, kScanThreads, 0, st, (const __nv_bfloat16*)q, (const __nv_bfloat16*)p,
                                                                         V, ksel, sc_t, sc_d, temp_t, temp_d, ws, params,
                                                                         pstride, kcap);
     }

@@ -28,6 +28,7 @@ constexpr double kTEnd = 25.0;      // integrand below exp(-kTEnd) at the upper 
 constexpr double kDrop = 1.0;       // the lower-tail compression starts this far below the fastest transition
 constexpr double kTail = 3.0;       // and the grid extends this far below that
 constexpr int kMaxNodes = 512;
+constexpr int kFlaggedGrid = 148;  // CTAs of the pass that looks for flagged instances: one per SM
 constexpr double kAlphaClamp = 80.0;
 constexpr double kStepClamp = 3.0;
 
@@ -560,8 +561,8 @@ __device__ int solve_system(const Sm& sm, int m, GR_PTR(const double) d, GR_PTR(
     return status;
 }
 
-__global__ void __launch_bounds__(kSolveThreads)
-solve_kernel(const char* __restrict__ ws, char* __restrict__ params, int pstride, int kcap, int V, int n, int topk,
+// One instance, by the whole CTA.
+__device__ void solve_instance(long long b, const char* __restrict__ ws, char* __restrict__ params, int pstride, int kcap, int V, int n, int topk,
              double temp_t, double temp_d, double tol, int max_iters, double qstep, double tau, int Qt, int only_flagged,
              float* __restrict__ alpha_out, int* __restrict__ status_out, FusedArgs fa)
 {
@@ -571,12 +572,9 @@ solve_kernel(const char* __restrict__ ws, char* __restrict__ params, int pstride
     GR_CHECK_FLAG_INIT;
     const bool fused = fa.draft != nullptr;
     const int tid = threadIdx.x;
-    const long long b = blockIdx.x;
     char* pb = params + (size_t)b * pstride;
     ParamView pv = view_params(pb, kcap, V, GR_CHECK_FLAG);
     const WsView wv = view_ws(ws, b, GR_CHECK_FLAG);
-    // second pass after the fast kernel: only the instances it flagged are redone
-    if (only_flagged && !(pv.h->magic == kMagic && pv.h->status == kNeedFallback)) return;
     if (kcap == 0 || wv.h->bad != 0 || wv.h->count <= 0) {
         // no rule: whole-vocabulary support beyond the capacity, or unusable logits
         if (tid == 0) write_no_rule(pv.h, n, wv.h->bad != 0, alpha_out, status_out, b);
@@ -711,6 +709,40 @@ solve_kernel(const char* __restrict__ ws, char* __restrict__ params, int pstride
     }
 }
 
+// only_flagged: the second pass after the fast kernel, which redoes the instances that one gave up (normally none).  A grid
+// of one wave looks them up, one instance per thread, and does those it finds one after the other.
+__global__ void __launch_bounds__(kSolveThreads)
+solve_kernel(const char* __restrict__ ws, char* __restrict__ params, int pstride, int kcap, int V, int n, int topk,
+             double temp_t, double temp_d, double tol, int max_iters, double qstep, double tau, int Qt, int only_flagged,
+             int batch, float* __restrict__ alpha_out, int* __restrict__ status_out, FusedArgs fa)
+{
+    __shared__ int s_list[kSolveThreads], s_count;
+    pdl_wait();
+    pdl_trigger();
+    if (!only_flagged) {
+        solve_instance(blockIdx.x, ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol, max_iters, qstep, tau, Qt, 0,
+                       alpha_out, status_out, fa);
+        return;
+    }
+    for (long long b0 = blockIdx.x; b0 < batch; b0 += (long long)gridDim.x * kSolveThreads) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_count = 0;
+        __syncthreads();
+        const long long b = b0 + (long long)threadIdx.x * gridDim.x;
+        if (b < batch) {
+            const Header* h = reinterpret_cast<const Header*>(params + (size_t)b * pstride);
+            if (h->magic == kMagic && h->status == kNeedFallback) s_list[atomicAdd(&s_count, 1)] = (int)b;
+        }
+        __syncthreads();
+        const int count = s_count;
+        for (int i = 0; i < count; i++) {
+            solve_instance(s_list[i], ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol, max_iters, qstep, tau, Qt, 1,
+                           alpha_out, status_out, fa);
+            __syncthreads();
+        }
+    }
+}
+
 int launch_solve(const char* ws, char* params, int pstride, int kcap, int V, int n, int topk, double temp_t,
                  double temp_d, double tol, int max_iters, double qstep, double tau, int batch, int only_flagged,
                  float* alpha_out, int* status_out, FusedArgs fa, cudaStream_t st)
@@ -733,8 +765,9 @@ int launch_solve(const char* ws, char* params, int pstride, int kcap, int V, int
             return GR_E_LAUNCH;
         configured[dev] = true;
     }
-    solve_kernel<<<batch, kSolveThreads, smem, st>>>(ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol,
-                                                     max_iters, qstep, tau, Qt, only_flagged, alpha_out, status_out, fa);
+    const int grid = only_flagged && batch > kFlaggedGrid ? kFlaggedGrid : batch;
+    launch_pdl(solve_kernel, grid, kSolveThreads, smem, st, ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol,
+               max_iters, qstep, tau, Qt, only_flagged, batch, alpha_out, status_out, fa);
     return GR_OK;
 }
 

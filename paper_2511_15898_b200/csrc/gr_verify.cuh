@@ -1,6 +1,6 @@
 // Slice of the transport for the drafted tuple and the accept / resample draw
-// (Eq. "cases", Eq. "approx-c", "normalized" in Algorithm 1; App. A steps 3-4), as warp-level
-// device code: one warp serves one instance.  Used by the stand-alone verify kernel and by the
+// (Eq. "cases", Eq. "approx-c", "normalized" in Algorithm 1; App. A steps 3-4), as CTA-level
+// device code: one CTA serves one instance.  Used by the stand-alone verify kernel and by the
 // solve kernels when they are given the drafted tokens (fused solve + verify).
 #pragma once
 #include "gr_common.cuh"
@@ -16,164 +16,161 @@ struct FusedArgs {
     int* vstatus;              // [batch]
 };
 
-// Shared-memory scratch of one verifying warp.
+// Shared-memory scratch of one verifying CTA.
 struct VerifyScratch {
-    GR_PTR(int) l_id; GR_PTR(double) l_r; GR_PTR(int) s_id; GR_PTR(double) s_p;       // kMaxSupport entries each
-    int* flag;                                              // bounds-checked build: where skipped accesses are reported
+    GR_PTR(double) res;        // residuals of one chunk of the target row, in id order
+    GR_PTR(double) p;          // support: flow,
+    GR_PTR(double) red;        // one double per warp; [32]: mass before the selected chunk
+    GR_PTR(int) id;            // id,
+    GR_PTR(int) chunk;         // chunk of the target row that holds it
+    GR_PTR(int) tok;           // drafted tokens and their positions in the ratio order
+    GR_PTR(int) pos;
+    GR_PTR(int) dec;           // token, accepted, status, whether to resample; two search results
+    int* flag;                 // bounds-checked build: where skipped accesses are reported
 };
-constexpr int kVerifyScratchBytes = kMaxSupport * 24;
+constexpr int kChunkSpan = kChunk + 8;           // longest chunk: the first one also holds the row's unaligned head
+constexpr int kVerifyScratchBytes = (kChunkSpan + kMaxSupport + 34) * 8 + (2 * kMaxSupport + 2 * kMaxDrafts + 8) * 4;
 // base: 8-byte aligned, kVerifyScratchBytes long
 __device__ inline VerifyScratch verify_scratch(void* base, int* flag = nullptr) {
     VerifyScratch v;
-    double* lr = reinterpret_cast<double*>(base);
-    int* li = reinterpret_cast<int*>(lr + 2 * kMaxSupport);
-    v.l_r = GR_MKPTR(double, lr, kMaxSupport, flag);
-    v.s_p = GR_MKPTR(double, lr + kMaxSupport, kMaxSupport, flag);
-    v.l_id = GR_MKPTR(int, li, kMaxSupport, flag);
-    v.s_id = GR_MKPTR(int, li + kMaxSupport, kMaxSupport, flag);
+    double* d = reinterpret_cast<double*>(base);
+    v.res = GR_MKPTR(double, d, kChunkSpan, flag); d += kChunkSpan;
+    v.p = GR_MKPTR(double, d, kMaxSupport, flag); d += kMaxSupport;
+    v.red = GR_MKPTR(double, d, 34, flag); d += 34;
+    int* t = reinterpret_cast<int*>(d);
+    v.id = GR_MKPTR(int, t, kMaxSupport, flag); t += kMaxSupport;
+    v.chunk = GR_MKPTR(int, t, kMaxSupport, flag); t += kMaxSupport;
+    v.tok = GR_MKPTR(int, t, kMaxDrafts, flag); t += kMaxDrafts;
+    v.pos = GR_MKPTR(int, t, kMaxDrafts, flag); t += kMaxDrafts;
+    v.dec = GR_MKPTR(int, t, 8, flag);
     v.flag = flag;
     return v;
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll 1
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 __device__ __forceinline__ double warp_incl_scan(double v, int lane) {
+#pragma unroll 1
     for (int o = 1; o < 32; o <<= 1) {
         double t = __shfl_up_sync(0xffffffffu, v, o);
         if (lane >= o) v += t;
     }
     return v;
 }
-
-// Inverse CDF of the resample distribution in ascending id order at `frac` of its total.
-// Residual of id i: the outer residual r_i on support ids (0 on H*), tgt_i elsewhere.
-// Two levels: per-chunk masses from the scan kernel's table minus the flow p_i of the
-// support ids in the chunk, then an exact fp64 pass over the one chunk selected.
-__device__ inline int resample_draw(const Header* h, const ParamView& pv, int k, double frac, int lane,
-                             GR_PTR(int) l_id, GR_PTR(double) l_r, GR_PTR(int) s_id, GR_PTR(double) s_p)
+// Inclusive prefix over the CTA's threads, *total gets the sum.  (One barrier before the slots may be reused.)
+static __device__ __noinline__ double block_incl_scan(double v, GR_PTR(double) red, double* total)
 {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    v = warp_incl_scan(v, lane);
+    __syncthreads();
+    if (lane == 31) red[warp] = v;
+    __syncthreads();
+    double off = 0.0, tot = 0.0;
+#pragma unroll 1
+    for (int w = 0; w < nw; w++) { const double t = red[w]; if (w < warp) off += t; tot += t; }
+    *total = tot;
+    return v + off;
+}
+
+// Inverse CDF of the resample distribution in ascending id order at `frac` of its total, by the whole CTA.
+// Residual of id i: the outer residual r_i on support ids (0 on H*), tgt_i elsewhere.
+// Two levels: per-chunk masses from the scan kernel's table minus the flow p_i of the support ids in the chunk (one
+// chunk per thread), then an exact fp64 pass over the one chunk selected (its residuals in shared memory, a run of
+// consecutive ids per thread).  Bound by the latency of three dependent reads; with one warp per instance the two
+// passes took 25 us, as they do here 4.
+__device__ inline int resample_draw(const Header* h, const ParamView& pv, int k, double frac, const VerifyScratch& vs)
+{
+    const int tid = threadIdx.x, bd = blockDim.x;
     const int nch = h->nch, head = h->head, V = h->V, dtype = h->dtype;
     const double T = (double)h->temp_target, lse = h->lse_t;
     const void* row = h->q_row;
-    // The total residual mass is known in closed form (1 - alpha*, or 1 when the target itself is sampled), so
-    // one pass over the chunk masses finds the chunk.  The support's (id, flow) pairs are staged in shared memory.
-    for (int j = lane; j < k; j += 32) { s_id[j] = pv.id[j]; s_p[j] = pv.p[j]; }
-    __syncwarp();
+    // the total residual mass is known in closed form (1 - alpha*, or 1 when the target itself is sampled)
     const double thr = frac * (k > 0 ? h->resid_total : 1.0);
-    int sel = -1; double before = 0.0, run = 0.0;
-    int last_pos_chunk = -1;
-    for (int c0 = 0; c0 < nch && sel < 0; c0 += 32) {
-        const int c = c0 + lane;
+    if (tid == 0) { vs.dec[4] = 0x7fffffff; vs.dec[5] = -1; }
+    double run = 0.0;
+    int sel = 0x7fffffff;
+#pragma unroll 1
+    for (int c0 = 0; c0 < nch; c0 += bd) {
+        const int c = c0 + tid;
         double R = 0.0;
         if (c < nch) {
             const float2 ms = pv.chunk[c];
-            R = (double)ms.y * exp((double)ms.x / T - lse);
-            const int cb = chunk_begin(c, head), ce = chunk_end(c, head, nch, V);
-            for (int j = 0; j < k; j++) { const int id = s_id[j]; if (id >= cb && id < ce) R -= s_p[j]; }
+            R = (double)ms.y * m_exp(m_div((double)ms.x, T) - lse);
+#pragma unroll 4
+            for (int j = 0; j < k; j++) if (vs.chunk[j] == c) R -= vs.p[j];
             if (R < 0.0) R = 0.0;
         }
-        const double inc = warp_incl_scan(R, lane) + run;
-        const unsigned hit = __ballot_sync(0xffffffffu, c < nch && inc > thr);
-        const unsigned pos = __ballot_sync(0xffffffffu, c < nch && R > 0.0);
-        if (pos) last_pos_chunk = c0 + 31 - __clz(pos);
-        if (hit) {
-            const int l = __ffs(hit) - 1;
-            sel = c0 + l;
-            before = __shfl_sync(0xffffffffu, inc - R, l);
-        }
-        run = __shfl_sync(0xffffffffu, inc, 31);
+        double tot;
+        const double inc = block_incl_scan(R, vs.red, &tot) + run;
+        if (c < nch && inc > thr) atomicMin(&vs.dec[4], c);
+        if (c < nch && R > 0.0) atomicMax(&vs.dec[5], c);
+        __syncthreads();
+        sel = vs.dec[4];
+        if (sel == c) vs.red[32] = inc - R;
+        run += tot;
+        if (sel != 0x7fffffff) break;
     }
-    if (sel < 0) { sel = last_pos_chunk; before = -1.0; }   // rounding left the threshold above the total
+    __syncthreads();
+    double want = 1.0e300;                      // (rounding left the threshold above the total: the last id of positive mass)
+    if (sel != 0x7fffffff) want = thr - vs.red[32];
+    else sel = vs.dec[5];
     if (sel < 0) return -1;
-    // support ids inside the selected chunk
-    const int cb = chunk_begin(sel, head), ce = chunk_end(sel, head, nch, V);
-    int nl = 0;
-    for (int j0 = 0; j0 < k; j0 += 32) {
-        const int j = j0 + lane;
-        const int id = j < k ? pv.id[j] : -1;
-        const bool in = id >= cb && id < ce;
-        const unsigned mk = __ballot_sync(0xffffffffu, in);
-        if (in) { const int s = nl + __popc(mk & ((1u << lane) - 1u)); l_id[s] = id; l_r[s] = pv.r[j]; }
-        nl += __popc(mk);
+    // ---- exact pass over the chunk in id order
+    const int cb = chunk_begin(sel, head), len = chunk_end(sel, head, nch, V) - cb;
+#pragma unroll 4
+    for (int e = tid; e < len; e += bd) vs.res[e] = m_exp(m_div((double)load_logit_dyn(row, dtype, cb + e), T) - lse);
+    __syncthreads();
+    for (int j = tid; j < k; j += bd) if (vs.chunk[j] == sel) vs.res[vs.id[j] - cb] = pv.r[j];
+    if (tid == 0) { vs.dec[4] = 0x7fffffff; vs.dec[5] = -1; }
+    __syncthreads();
+    const int per = ((len + bd - 1) / bd) | 1;              // (odd: no bank conflicts)
+    const int e0 = min(tid * per, len), e1 = min(e0 + per, len);
+    double sum = 0.0;
+    int lastp = -1;
+#pragma unroll 1
+    for (int e = e0; e < e1; e++) { const double r = vs.res[e]; sum += r; if (r > 0.0) lastp = e; }
+    double tot;
+    const double inc = block_incl_scan(sum, vs.red, &tot);
+    double acc = inc - sum;
+    int hit = 0x7fffffff;
+    if (inc > want) {
+#pragma unroll 1
+        for (int e = e0; e < e1; e++) { acc += vs.res[e]; if (acc > want) { hit = e; break; } }
+        if (hit == 0x7fffffff && e1 > e0) hit = e1 - 1;     // (the run's sum and its walk round differently)
     }
-    __syncwarp();
-    // exact pass over the chunk in id order, 32 consecutive ids at a time (one per lane): the first id whose running
-    // total exceeds the threshold; the last id of positive residual when rounding left the threshold above the total
-    const double want = before < 0.0 ? 1.0e300 : thr - before;
-    double run2 = 0.0;
-    int token = -1, lastp = -1;
-    constexpr int kRows = 8;                 // rows of 32 ids whose logits are fetched together
-    for (int g0 = cb; g0 < ce && token < 0; g0 += 32 * kRows) {
-        float lg[kRows];
-#pragma unroll
-        for (int q = 0; q < kRows; q++) {
-            const int i = g0 + 32 * q + lane;
-            lg[q] = i < ce ? load_logit_dyn(row, dtype, i) : 0.f;
-        }
-#pragma unroll
-        for (int q = 0; q < kRows; q++) {
-            const int r0 = g0 + 32 * q;
-            if (r0 < ce && token < 0) {
-                const int i = r0 + lane;
-                const bool in = i < ce;
-                double res = 0.0;
-                if (in) {
-                    res = exp((double)lg[q] / T - lse);
-                    for (int s2 = 0; s2 < nl; s2++) if (l_id[s2] == i) res = l_r[s2];
-                }
-                const double inc = warp_incl_scan(res, lane) + run2;
-                const unsigned hit = __ballot_sync(0xffffffffu, in && inc > want);
-                const unsigned posl = __ballot_sync(0xffffffffu, in && res > 0.0);
-                if (posl) lastp = r0 + 31 - __clz(posl);
-                if (hit) token = r0 + __ffs(hit) - 1;
-                run2 = __shfl_sync(0xffffffffu, inc, 31);
-            }
-        }
-    }
-    return token >= 0 ? token : lastp;
+    if (hit != 0x7fffffff) atomicMin(&vs.dec[4], hit);
+    if (lastp >= 0) atomicMax(&vs.dec[5], lastp);
+    __syncthreads();
+    const int found = vs.dec[4], last = vs.dec[5];
+    return found != 0x7fffffff ? cb + found : (last >= 0 ? cb + last : -1);
 }
-
 
 // One lane's share of the slice pi(.|omega) (Eq. "cases", Eq. "approx-c", "normalized" in Algorithm 1): lane s < n
 // holds drafted token s.  uniq: first occurrence of its token; pi: its probability (0 for repeats and for tokens
 // outside the serving system); inner: every drafted token lies in H*; rho: mass of the resample segment.
 struct SliceLane { bool uniq, inner; double pi, rho; };
 
-// Slice of a solved instance (k > 0) for the drafted tuple, one warp; `tok` is this lane's drafted token (lanes >= n: any).
-// Returns GR_OK, or GR_DRAFT_OUT_OF_SUPPORT when a drafted token is not in the support.
-__device__ inline int slice_instance(const Header* h, const ParamView& pv, int tok, int lane, SliceLane& sl)
+// Slice of a solved instance (k > 0) for the drafted tuple, one warp; `pos` is the position of this lane's drafted token in
+// the ratio order (lanes >= n: any).  Returns GR_OK, or GR_DRAFT_OUT_OF_SUPPORT when a drafted token is not in the support.
+__device__ inline int slice_instance(const Header* h, const ParamView& pv, int pos, int lane, SliceLane& sl)
 {
-    const int n = h->n, k = h->k, jstar = h->jstar;
+    const int n = h->n, jstar = h->jstar;
     sl.uniq = false; sl.inner = false; sl.pi = 0.0; sl.rho = 0.0;
-    // position of every drafted token in the ratio order
-    int pos = -1;
-    for (int s = 0; s < n; s++) {
-        const int ts = __shfl_sync(0xffffffffu, tok, s);
-        int found = -1;
-        for (int j0 = 0; j0 < k; j0 += 32) {
-            const int j = j0 + lane;
-            const unsigned mk = __ballot_sync(0xffffffffu, j < k && pv.id[j] == ts);
-            if (mk) found = j0 + __ffs(mk) - 1;
-        }
-        if (lane == s) pos = found;
-    }
     const bool missing = __any_sync(0xffffffffu, lane < n && pos < 0);
     if (missing) return GR_DRAFT_OUT_OF_SUPPORT;
     // distinct tokens in order of first occurrence; the lowest-ratio position met
-    bool uniq = lane < n;
-    int maxpos = lane < n ? pos : -1;
-    for (int s = 0; s < n; s++) {
-        const int ps = __shfl_sync(0xffffffffu, pos, s);
-        if (lane > s && lane < n && pos == ps) uniq = false;
-    }
-    for (int o = 16; o > 0; o >>= 1) maxpos = max(maxpos, __shfl_xor_sync(0xffffffffu, maxpos, o));
+    const unsigned same = __match_any_sync(0xffffffffu, lane < n ? pos : -1 - lane);
+    const bool uniq = lane < n && __ffs(same) - 1 == lane;
+    const int maxpos = __reduce_max_sync(0xffffffffu, lane < n ? pos : -1);
     const bool inner = maxpos < jstar;
     double wv = 0.0;
+    bool served = false;
     if (uniq) {
-        if (inner) wv = pv.w[pos];
-        else wv = (pv.blk[pos] == pv.blk[maxpos]) ? pv.w[pos] : 0.0;
+        served = inner || pv.blk[pos] == pv.blk[maxpos];
+        if (served) wv = pv.w[pos];
     }
     const double W = warp_sum(wv) + (inner ? 1.0 : 0.0);
     sl.uniq = uniq; sl.inner = inner;
@@ -181,7 +178,6 @@ __device__ inline int slice_instance(const Header* h, const ParamView& pv, int t
         sl.pi = wv / W;
     } else {
         // (truncated variant) every served token carries weight 0: they share the tuple equally
-        const bool served = uniq && pv.blk[pos] == pv.blk[maxpos];
         const int cnt = __popc(__ballot_sync(0xffffffffu, served));
         sl.pi = served ? 1.0 / (double)cnt : 0.0;
     }
@@ -189,12 +185,31 @@ __device__ inline int slice_instance(const Header* h, const ParamView& pv, int t
     return GR_OK;
 }
 
-// The whole verification of one instance by one warp.  `h` is the instance's header (already checked to carry
-// the magic number); a rule marked partial is accepted only from the kernel that solved it for these drafts.
-__device__ inline void verify_instance(const Header* h, const int* draft_row, const float* uni_row, int lane,
-                                       const VerifyScratch& vs, bool allow_partial, int& token, int& accepted,
-                                       int& status)
+// Support and drafted tokens into the scratch, and where each drafted token sits in the ratio order (-1: nowhere).
+__device__ inline void locate_drafts(const Header* h, const ParamView& pv, const int* draft_row, const VerifyScratch& vs)
 {
+    const int tid = threadIdx.x, bd = blockDim.x, k = h->k, n = h->n, nch = h->nch, head = h->head;
+    if (tid < kMaxDrafts) { vs.tok[tid] = tid < n ? draft_row[tid] : -1; vs.pos[tid] = -1; }
+    for (int j = tid; j < k; j += bd) {
+        const int id = pv.id[j];
+        vs.id[j] = id; vs.p[j] = pv.p[j]; vs.chunk[j] = chunk_of(id, head, nch);
+    }
+    __syncthreads();
+    for (int j = tid; j < k; j += bd) {
+        const int id = vs.id[j];
+#pragma unroll 4
+        for (int s = 0; s < n; s++) if (vs.tok[s] == id) vs.pos[s] = j;
+    }
+    __syncthreads();
+}
+
+// The whole verification of one instance by one CTA (at least two warps).  `h` is the instance's header (already checked
+// to carry the magic number); a rule marked partial is accepted only from the kernel that solved it for these drafts.
+// Every thread gets the result.
+__device__ inline void verify_instance(const Header* h, const int* draft_row, const float* uni_row, const VerifyScratch& vs,
+                                       bool allow_partial, int& token, int& accepted, int& status)
+{
+    const int lane = threadIdx.x & 31;
     token = -1; accepted = 0;
     status = h->status;
     if (status == GR_BAD_LOGITS) return;
@@ -203,33 +218,39 @@ __device__ inline void verify_instance(const Header* h, const int* draft_row, co
         status = GR_OK;
     }
     ParamView pv = view_params((void*)h, h->kcap, h->V, vs.flag);
-    const int n = h->n, k = h->k;
+    const int k = h->k;
     const double u0 = (double)uni_row[0], u1 = (double)uni_row[1];
-    const int tok = lane < n ? draft_row[lane] : -1;
+    locate_drafts(h, pv, draft_row, vs);
     if (k == 0) {
         // no rule was solved: emit a sample of the target distribution itself
-        token = resample_draw(h, pv, 0, u1, lane, vs.l_id, vs.l_r, vs.s_id, vs.s_p);
-        accepted = __any_sync(0xffffffffu, lane < n && tok == token) ? 1 : 0;
-        if (token < 0) accepted = 0;
+        token = resample_draw(h, pv, 0, u1, vs);
+        if (token >= 0) {
+            for (int s = 0; s < h->n; s++) if (vs.tok[s] == token) accepted = 1;
+        }
         return;
     }
-    SliceLane sl;
-    if (slice_instance(h, pv, tok, lane, sl) != GR_OK) { status = GR_DRAFT_OUT_OF_SUPPORT; return; }
-    const bool uniq = sl.uniq, inner = sl.inner;
-    const double pi = sl.pi;
-    const double cum = warp_incl_scan(pi, lane);
-    const unsigned hit = __ballot_sync(0xffffffffu, uniq && cum > u0);
-    if (hit) {
-        token = __shfl_sync(0xffffffffu, tok, __ffs(hit) - 1);
-        accepted = 1;
-    } else if (!inner) {
-        const unsigned posm = __ballot_sync(0xffffffffu, uniq && pi > 0.0);
-        token = __shfl_sync(0xffffffffu, tok, 31 - __clz(posm));
-        accepted = 1;
-    } else {
-        token = resample_draw(h, pv, k, u1, lane, vs.l_id, vs.l_r, vs.s_id, vs.s_p);
-        accepted = 0;
+    if (threadIdx.x < 32) {
+        const int tok = vs.tok[lane];
+        SliceLane sl;
+        int tk = -1, ac = 0, again = 0;
+        const int st = slice_instance(h, pv, vs.pos[lane], lane, sl);
+        if (st == GR_OK) {
+            const double cum = warp_incl_scan(sl.pi, lane);
+            const unsigned hit = __ballot_sync(0xffffffffu, sl.uniq && cum > u0);
+            const unsigned posm = __ballot_sync(0xffffffffu, sl.uniq && sl.pi > 0.0);
+            if (hit || !sl.inner) {
+                tk = __shfl_sync(0xffffffffu, tok, hit ? __ffs(hit) - 1 : 31 - __clz(posm));
+                ac = 1;
+            } else {
+                again = 1;
+            }
+        }
+        if (lane == 0) { vs.dec[0] = tk; vs.dec[1] = ac; vs.dec[2] = st; vs.dec[3] = again; }
     }
+    __syncthreads();
+    if (vs.dec[2] != GR_OK) { status = vs.dec[2]; return; }
+    token = vs.dec[0]; accepted = vs.dec[1];
+    if (vs.dec[3]) token = resample_draw(h, pv, k, u1, vs);
 }
 
 // Which system the drafted tuple selects (Eq. "cases"): -1 the inner system (every drafted token in H*), b >= 0 the
@@ -255,18 +276,15 @@ __device__ inline int selected_system(const int* draft_row, int n, int k, int js
     return maxpos < jstar ? -1 : sblk[maxpos];
 }
 
-// Draw of instance b by warp 0 of a solve kernel's CTA, after the rule (or the no-rule header) was written and the
-// CTA synchronised.
+// Draw of instance b by a solve kernel's CTA, after the rule (or the no-rule header) was written and the CTA synchronised.
 static __device__ __noinline__ void fused_draw(const FusedArgs& fa, const Header* h, long long b, int n, void* scratch,
-                                  int* check_flag = nullptr)
+                                               int* check_flag = nullptr)
 {
-    if (threadIdx.x >= 32) return;
-    const int lane = threadIdx.x;
     int token, accepted, status;
-    verify_instance(h, fa.draft + (size_t)b * n, fa.uni + 2 * (size_t)b, lane, verify_scratch(scratch, check_flag), true,
-                    token, accepted, status);
+    verify_instance(h, fa.draft + (size_t)b * n, fa.uni + 2 * (size_t)b, verify_scratch(scratch, check_flag), true, token,
+                    accepted, status);
     if (check_flag && *check_flag) status = GR_CHECK_FAILED;
-    if (lane == 0) {
+    if (threadIdx.x == 0) {
         fa.out_token[b] = token;
         fa.out_acc[b] = (unsigned char)accepted;
         fa.vstatus[b] = status;
