@@ -50,6 +50,8 @@ constexpr double kFChordBase = 0.02;       // contraction assumed of a step with
 constexpr int kFCgMax = 16;                // conjugate-gradient iterations before the factorisation takes over
 constexpr float kFCgTol = 2.0e-4f;         // and their relative residual
 constexpr float kFScaleJump = 0.5f;        // distance of the common scale from which its curve is inverted exactly
+constexpr float kFSmallSlack = 1.0e-4f;     // share of the mass below which Tn - sum g is mostly rounding in fp32
+constexpr float kFLeastSlack = 1.0e-9f;     // and the least share aimed at (the quadrature's floor)
 constexpr int kFSweeps = 5;                // fixed-point sweeps of the starting point
 
 // Compile-time geometry.  NT: series length (>= n), MP: padded support size, T: threads, JC: Hessian nodes staged
@@ -1403,7 +1405,11 @@ __device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, c
                 // its accuracy for this instance.  Conjugate gradients give way to the factorisation; the second time there
                 // the instance is handed to the general kernel, which starts from the last accepted point.
                 if (chol && ++stalls >= 2) { alpha = alpha_prev; break; }
-                chol = true;
+                if (!chol) {
+                    // (the last accepted point once more: this one has no factorisation)
+                    chol = true; alpha = alpha_prev; rprev = 1.0e300; lam = 1.0; was_kind = -1;
+                    continue;
+                }
             }
         }
         if (high) { mode = kHigh; full_grid = true; rprev = 1.0e300; lam = 1.0; was_kind = -1; continue; }
@@ -1426,14 +1432,19 @@ __device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, c
             tok_sums<C, 3>(sm, sums, par);
             const float lin = slack ? __fdividef(sums[0], sums[1]) : 0.f;
             if (slack) {
-                const float g0 = (float)(Tn - rg.x);
+                const float g0 = (float)(Tn - rg.x), slope = sums[1];
                 shift = lin;
-                pivot = __fdividef(sums[1], sums[2]);               // of the order of the smallest relative pivot
-                if (t0 > 0.f && g0 > sums[1] && g0 > 1.0e-5f) {
+                pivot = __fdividef(slope, sums[2]);                 // of the order of the smallest relative pivot
+                float far = 0.f;
+                if (g0 < kFSmallSlack * (float)Tn) {
+                    // too small a difference for fp32; the slope, a sum of positive terms, is the share itself there
+                    far = __logf(__fdividef(fmaxf(slope, 1.0e-30f), fmaxf(t0, kFLeastSlack * (float)Tn)));
+                    if (mode == kLow || fabsf(far) > kFScaleJump) { shift = fminf(fmaxf(far, -16.f), 16.f); jump = (double)shift; }
+                } else if (t0 > 0.f && g0 > slope) {
                     // saturation level c0 from value and slope:  slope = g0 (1 - g0 / c0)
-                    const float inv = __fdividef(g0 - sums[1], g0 * g0);              // 1 / c0
+                    const float inv = __fdividef(g0 - slope, g0 * g0);                // 1 / c0
                     const float q = __fdividef(g0 * (1.f - t0 * inv), t0 * (1.f - g0 * inv));
-                    const float far = q > 0.f ? __logf(q) : 0.f;
+                    far = q > 0.f ? __logf(q) : 0.f;
                     if (far > kFScaleJump) { shift = fminf(far, 16.f); jump = (double)shift; }
                 }
             }
@@ -1454,8 +1465,9 @@ __device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, c
             dl = on ? (double)sm.dl[i] : 0.0;
             // proportional-fitting step  alpha += log(rhs / g)  (and the full grid from here on)
             if (fail) { full_grid = true; dl = on ? m_log(rhs_i / g) : 0.0; }
+            // (no usable step: the general kernel's)
+            if (__syncthreads_or(!(fabs(dl) < 1.0e300))) break;
         }
-        if (!(dl == dl)) dl = 0.0;
         if (!slack) {
             const double mean = tok_sum<C>(sm, dl, par) / (double)m;
             if (on) dl -= mean;
@@ -1463,7 +1475,7 @@ __device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, c
         double dm = on ? fabs(dl - jump) : 0.0, s2 = on ? g * dl * dl : 0.0;
         tok_max_sum<C>(sm, dm, s2, par);
         // a full Newton step below 1e-11 in alpha: the weights cannot be improved at this quadrature accuracy
-        if (!fail && mode != kLow && dm < 1.0e-11) { status = GR_OK; it++; break; }
+        if (!fail && mode != kLow && dm + fabs(jump) < 1.0e-11) { status = GR_OK; it++; break; }
         if (dm > kFStepClamp && on) dl = jump + (dl - jump) * (kFStepClamp / dm);
         delta = dl;
         alpha = fmin(fmax(alpha + dl, -kFAlphaClamp), kFAlphaClamp);
@@ -1480,10 +1492,10 @@ __device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, c
         const bool trusted = !fail && pivot > (float)kFTrustPivot;
         if (mode == kLow) {
             // the next point is close enough: fp64 from here on, with this factorisation
-            if (kFPredictBound * s2 < kFLowLeave && dm + jump <= 0.1) { mode = trusted ? kChord : kHigh; full_grid = true; dist = dm; }
+            if (kFPredictBound * s2 < kFLowLeave && dm + fabs(jump) <= 0.1) { mode = trusted ? kChord : kHigh; full_grid = true; dist = dm; }
         } else if (trusted && !coarse) {
             const double lin = mode == kChord ? (kFChordBase + 2.0 * dist) * rn : 0.0;
-            const bool by_step = dm + jump <= kFPredictStep && kFPredictSafety * s2 + 3.0 * lin < tol;
+            const bool by_step = dm + fabs(jump) <= kFPredictStep && kFPredictSafety * s2 + 3.0 * lin < tol;
             const bool by_ratio = rho < 0.1 && dm <= kFStepClamp && kFRatioSafety * rho * rn < tol;
             if (by_step || by_ratio) {
                 rn = by_step ? kFPredictBound * s2 + lin : rho * rn;

@@ -522,7 +522,8 @@ __device__ int solve_system(const Sm& sm, int m, GR_PTR(const double) d, GR_PTR(
             if (tid < m) sm.delta[tid] = log(rhs[tid] / sm.g[tid]);
             __syncthreads();
         }
-        double dm = block_reduce_max(tid < m ? fabs(sm.delta[tid]) : 0.0, red);
+        // (a component that is not a number counts as infinite: fmax would drop it)
+        double dm = block_reduce_max(tid < m ? (sm.delta[tid] == sm.delta[tid] ? fabs(sm.delta[tid]) : 1.0e300) : 0.0, red);
         if (!(dm < 1.0e300)) dm = 1.0e300;
         // a full Newton step below 1e-11 in alpha: the weights cannot be improved at this quadrature accuracy
         if (!fail && dm < 1.0e-11) { status = GR_OK; it++; break; }
