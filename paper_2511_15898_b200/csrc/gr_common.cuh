@@ -5,6 +5,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <stdint.h>
+#include <type_traits>
 #include "gr.h"
 
 namespace gr {
@@ -155,7 +156,7 @@ __host__ __device__ inline ParamView view_params(void* base, int kcap, int V = 1
 // Workspace of one instance (written by the scan kernel, read by the solve kernel).
 struct __align__(16) WsHeader {
     double lse_t;        // log sum exp of target logits / temp_target
-    double lse_d;        // same for the whole draft row (only when the support is the whole vocabulary)
+    double lse_d;        // (unused)
     int count;           // entries that follow (the support, k of them)
     int bad;             // 1 when a non-finite logit was met
     int check;           // bounds-checked build: the streaming kernel skipped an out-of-range access on this row
@@ -219,21 +220,51 @@ static __device__ __noinline__ double m_exp(double x) { return exp(x); }
 static __device__ __noinline__ double m_log(double x) { return log(x); }
 static __device__ __noinline__ double m_div(double a, double b) { return a / b; }
 
+// exp(-y) for y >= 0 (fp64): Cody and Waite's range reduction by a two-part ln 2 and a degree-13 Taylor polynomial on
+// |r| <= ln2/2 (truncation below 1e-17 relative), summed in pairs and fours (Estrin's scheme: a third of Horner's chain,
+// which is what a warp alone on its scheduler waits for); results below 2^-1000 are flushed to zero.
+__device__ __forceinline__ double exp_neg(double y)
+{
+    const double t = -y;
+    const double kf = rint(t * 1.4426950408889634);
+    double r = fma(-kf, 6.93147180369123816490e-01, t);
+    r = fma(-kf, 1.90821492927058770002e-10, r);
+    const double r2 = r * r, r4 = r2 * r2;
+    const double a0 = 1.0 + r, a1 = fma(r, 1.6666666666666666e-01, 0.5);                    // 1/2!, 1/3!
+    const double a2 = fma(r, 8.333333333333333e-03, 4.1666666666666664e-02);                // 1/4!, 1/5!
+    const double a3 = fma(r, 1.984126984126984e-04, 1.388888888888889e-03);                 // 1/6!, 1/7!
+    const double a4 = fma(r, 2.7557319223985893e-06, 2.48015873015873e-05);                 // 1/8!, 1/9!
+    const double a5 = fma(r, 2.505210838544172e-08, 2.755731922398589e-07);                 // 1/10!, 1/11!
+    const double a6 = fma(r, 1.6059043836821613e-10, 2.08767569878681e-09);                 // 1/12!, 1/13!
+    const double b0 = fma(r2, a1, a0), b1 = fma(r2, a3, a2), b2 = fma(r2, a5, a4);
+    const double p = fma(r4, fma(r4, fma(r4, a6, b2), b1), b0);
+    const int k = (int)kf;
+    return kf < -1000.0 ? 0.0 : __hiloint2double(__double2hiint(p) + (k << 20), __double2loint(p));
+}
+
 // Programmatic dependent launch.  Every kernel of a call is launched with launch_pdl and begins with these two: it may be
 // scheduled, and its CTAs take the places that its predecessor's last wave leaves, before the predecessor has ended, but it
 // touches no memory until the predecessor has completed (which, by the same rule, had waited for its own).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class... P>
+inline cudaError_t launch_pdl_cluster(int cluster, void (*kernel)(P...), int grid, int block, int smem, cudaStream_t st,
+                                      std::remove_const_t<P>... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = st; cfg.attrs = at; cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 template <class... P, class... A>
 inline cudaError_t launch_pdl(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t st, A... args)
 {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at = {};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = st; cfg.attrs = &at; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    return launch_pdl_cluster<P...>(1, kernel, grid, block, smem, st, static_cast<P>(args)...);
 }
 
 constexpr int kMaxDevices = 64;               // per-device caches of the host code (function attributes, streams)

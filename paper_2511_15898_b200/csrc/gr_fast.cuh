@@ -180,27 +180,6 @@ __device__ __forceinline__ double ipow(double x, int n) {
     return r;
 }
 
-// exp(-y) for y >= 0 (fp64): Cody and Waite's range reduction by a two-part ln 2 and a degree-13 Taylor polynomial on
-// |r| <= ln2/2 (truncation below 1e-17 relative), summed in pairs and fours (Estrin's scheme: a third of Horner's chain,
-// which is what a warp alone on its scheduler waits for); results below 2^-1000 are flushed to zero.
-__device__ __forceinline__ double exp_neg(double y)
-{
-    const double t = -y;
-    const double kf = rint(t * 1.4426950408889634);
-    double r = fma(-kf, 6.93147180369123816490e-01, t);
-    r = fma(-kf, 1.90821492927058770002e-10, r);
-    const double r2 = r * r, r4 = r2 * r2;
-    const double a0 = 1.0 + r, a1 = fma(r, 1.6666666666666666e-01, 0.5);                    // 1/2!, 1/3!
-    const double a2 = fma(r, 8.333333333333333e-03, 4.1666666666666664e-02);                // 1/4!, 1/5!
-    const double a3 = fma(r, 1.984126984126984e-04, 1.388888888888889e-03);                 // 1/6!, 1/7!
-    const double a4 = fma(r, 2.7557319223985893e-06, 2.48015873015873e-05);                 // 1/8!, 1/9!
-    const double a5 = fma(r, 2.505210838544172e-08, 2.755731922398589e-07);                 // 1/10!, 1/11!
-    const double a6 = fma(r, 1.6059043836821613e-10, 2.08767569878681e-09);                 // 1/12!, 1/13!
-    const double b0 = fma(r2, a1, a0), b1 = fma(r2, a3, a2), b2 = fma(r2, a5, a4);
-    const double p = fma(r4, fma(r4, fma(r4, a6, b2), b1), b0);
-    const int k = (int)kf;
-    return kf < -1000.0 ? 0.0 : __hiloint2double(__double2hiint(p) + (k << 20), __double2loint(p));
-}
 __device__ __forceinline__ float ex2_approx(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 template <typename R> struct Rx;
 template <> struct Rx<double> {

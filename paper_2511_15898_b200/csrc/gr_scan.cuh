@@ -1,0 +1,528 @@
+// Streaming pass over the two logit rows of an instance, as CTA-level device code: by a kernel of its own (one CTA or one
+// cluster per row) or by the solve kernel's CTA before it solves the row.
+//
+// In a single read of the rows it produces
+//   - the log-sum-exp of the target row at temp_target and, per 1024-element chunk,
+//     the (max, sum exp2) pair the resample draw later uses as a two-level CDF
+//     (distributions from logits: App. A, first paragraph);
+//   - the draft support: the `ksel` largest draft logits, equal logits resolved in
+//     favour of the smaller id (top-k reduction of the problem, App. N), together
+//     with the target logits at those ids.
+//
+// One warp takes a chunk, in batches of U 128-bit vectors of each row per lane, all of them loaded before the first is used;
+// differences and scalings as packed pairs.
+//
+// Selection without a second pass: a threshold tau that is provably not above the ksel-th largest draft logit is derived
+// from running maxima of disjoint groups of elements (each of the ksel largest group maxima is a distinct element, so the
+// ksel-th largest of them bounds the answer from below), refined whenever the part read has grown fourfold; elements >= tau are
+// appended to a shared candidate list and the exact answer is taken from the list at the end.  If the list ever
+// overflows (adversarially ordered rows) an exact multi-pass radix selection over the row replaces it.
+#pragma once
+#include "gr_common.cuh"
+
+namespace gr {
+
+constexpr int kMaxChunks = 2049;     // V <= 2^21
+constexpr int kMaxCluster = 8;
+constexpr int kRankAll = 128;        // candidates that are ranked as they are; more go through a last threshold first
+
+// Arguments common to every row.
+struct ScanArgs {
+    const void* q; const void* p;    // logits
+    int dtype, V, ksel;
+    float sc_t, sc_d;                // log2(e) / temperature
+    double temp_t, temp_d;
+    char* ws; char* params;          // workspace records; params block or nullptr (the caller wants the records only)
+    int pstride, kcap;
+};
+
+// Shared memory.  NTHR threads, CAP candidates, CH chunk entries.
+template <int NTHR, int CAP, int CH>
+struct __align__(16) ScanShared {
+    static constexpr int kThr = NTHR, kCap = CAP, kCh = CH;
+    unsigned long long keys[CAP];    // candidates (value, id), then composite keys
+    float2 chunk[CH];
+    double lse[1], part[NTHR / 32], top;
+    unsigned long long prefix;
+    unsigned int gkey[NTHR];
+    int hist[256];
+    int need, cnt, bad, kept;
+    float tau;
+    // cluster-split rows (used in the leading CTA): what the others found
+    int part_cnt[kMaxCluster], part_bad[kMaxCluster];
+};
+
+template <typename T> struct VecTraits;
+template <> struct VecTraits<float> {
+    static constexpr int N = 4;
+    // the two packed pairs of a 16-byte vector, i = 0, 1
+    __device__ static unsigned long long pair(const ulonglong2& v, int i) { return i == 0 ? v.x : v.y; }
+    static constexpr int kPairs = 2;
+};
+template <> struct VecTraits<__nv_bfloat16> {
+    static constexpr int N = 8;
+    __device__ static unsigned long long pair(const ulonglong2& v, int i) {
+        const unsigned int w = (unsigned int)((i < 2 ? v.x : v.y) >> (32 * (i & 1)));
+        return ((unsigned long long)(w & 0xffff0000u) << 32) | (unsigned long long)(w << 16);
+    }
+    static constexpr int kPairs = 4;
+};
+__device__ __forceinline__ float f_lo(unsigned long long v) { return __uint_as_float((unsigned int)v); }
+__device__ __forceinline__ float f_hi(unsigned long long v) { return __uint_as_float((unsigned int)(v >> 32)); }
+__device__ __forceinline__ unsigned long long f_pack(float lo, float hi) {
+    return ((unsigned long long)__float_as_uint(hi) << 32) | __float_as_uint(lo);
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float warp_max(float x) { return fkey_inv(__reduce_max_sync(0xffffffffu, fkey(x))); }
+// (max, sum) of two parts of a sum of exp2((x - max) sc); an empty part is (-inf, 0)
+__device__ __forceinline__ void osm_merge(float& m, float& s, float mo, float so, float sc) {
+    const float mn = fmaxf(m, mo);
+    const float a = (m == mn) ? s : s * ex2((m - mn) * sc);
+    const float b = (mo == mn) ? so : so * ex2((mo - mn) * sc);
+    s = a + b; m = mn;
+}
+__device__ __forceinline__ ulonglong2 ldg_stream(const void* p) {
+    ulonglong2 v;
+    asm volatile("ld.global.cs.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p));
+    return v;
+}
+
+// Address of a shared-memory object in the CTA of rank `rank` of this cluster.
+__device__ __forceinline__ unsigned int cluster_addr(const void* p, unsigned int rank) {
+    unsigned int r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((unsigned int)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_cluster(unsigned int addr, unsigned int v) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster(unsigned int addr, unsigned long long v) {
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// The `need`-th largest of the threads' running maxima (16 leading key bits, rounded down); never below the old threshold.
+// (512 threads: 16 counting barriers, 0.3 us; one warp searching 512 values in shared memory took three times that.)
+template <class SS>
+__device__ __forceinline__ void refine_tau(SS& sh, float mx, int need)
+{
+    const unsigned int key = fkey(mx);
+    unsigned int res = 0;
+#pragma unroll 1
+    for (int bit = 31; bit >= 16; bit--) {
+        const unsigned int t = res | (1u << bit);
+        if (__syncthreads_count(key >= t) >= need) res = t;
+    }
+    if (threadIdx.x == 0) sh.tau = fmaxf(sh.tau, fkey_inv(res));
+    __syncthreads();
+}
+
+template <class SS>
+__device__ __forceinline__ void push_candidate(SS& sh, float val, int id, float tau) {
+    if (val >= tau) {
+        const int slot = atomicAdd(&sh.cnt, 1);
+        if (slot < SS::kCap) {
+            reinterpret_cast<float*>(sh.keys)[slot] = val;
+            reinterpret_cast<int*>(sh.keys)[SS::kCap + slot] = id;
+        }
+    }
+}
+
+// Exact selection of the ksel largest composite keys among this CTA's chunks by eight 8-bit radix passes over them (slow
+// path, taken only when the candidate list overflowed).
+template <typename T, class SS>
+__device__ __noinline__ void exact_select_slow(SS& sh, const T* prow, int V, int head, int nch, int first, int stride, int ksel)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) { sh.prefix = 0ull; sh.need = ksel; }
+    __syncthreads();
+#pragma unroll 1
+    for (int pass = 0; pass < 9; pass++) {
+        // (the ninth pass collects)
+        const int shift = 56 - 8 * pass;
+        if (pass < 8) for (int i = tid; i < 256; i += SS::kThr) sh.hist[i] = 0;
+        if (pass == 8 && tid == 0) sh.cnt = 0;
+        __syncthreads();
+        const unsigned long long prefix = sh.prefix;
+        for (int c = first + warp; c < nch; c += stride) {
+            const int e1 = chunk_end(c, head, nch, V);
+            for (int i = chunk_begin(c, head) + lane; i < e1; i += 32) {
+                const float v = load_logit<T>(prow, i);
+                const unsigned long long key = ckey(v, i);
+                if (pass == 8) {
+                    if (key >= prefix) push_candidate(sh, v, i, -INFINITY);
+                } else if (pass == 0 || (key >> (shift + 8)) == (prefix >> (shift + 8))) {
+                    atomicAdd(&sh.hist[(int)((key >> shift) & 255ull)], 1);
+                }
+            }
+        }
+        __syncthreads();
+        if (pass < 8 && tid == 0) {
+            int need = sh.need, acc = 0, bin = 255;
+            for (; bin > 0; bin--) {
+                if (acc + sh.hist[bin] >= need) break;
+                acc += sh.hist[bin];
+            }
+            sh.need = need - acc;
+            sh.prefix = prefix | ((unsigned long long)bin << shift);
+        }
+        __syncthreads();
+    }
+}
+
+// The nsel largest of the M composite keys in sh.keys, handed to `take(rank, key)`.
+template <class SS, class F>
+__device__ __forceinline__ void rank_select(SS& sh, int M, int nsel, F take)
+{
+#pragma unroll 1
+    for (int e = threadIdx.x; e < M; e += SS::kThr) {
+        const unsigned long long me = sh.keys[e];
+        int rank = 0;
+#pragma unroll 4
+        for (int j = 0; j < M; j++) rank += (sh.keys[j] > me) ? 1 : 0;
+        if (rank < nsel) take(rank, me);
+    }
+}
+
+// Terms of the row's log-sum-exp, in fp64 from the chunk table (so that the chunk masses sum to one): a chunk per thread.
+template <class SS>
+__device__ __forceinline__ void lse_terms(SS& sh, int nch, double temp_t)
+{
+    const int tid = threadIdx.x, lane = tid & 31;
+    float mf = -INFINITY;
+    for (int c = lane; c < nch; c += 32) mf = fmaxf(mf, sh.chunk[c].x);
+    const double top = (double)warp_max(mf);
+    double acc = 0.0;
+#pragma unroll 1
+    for (int c = tid; c < nch; c += SS::kThr) acc += (double)sh.chunk[c].y * exp_neg((top - (double)sh.chunk[c].x) / temp_t);
+    if ((tid & ~31) < nch) {
+#pragma unroll 1
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    }
+    if (lane == 0) sh.part[tid >> 5] = acc;
+    if (tid == 0) sh.top = top;
+}
+
+// Row b, by this CTA (cn == 1) or by the cn CTAs of its cluster, of which this is number cr and number 0 writes the results.
+// kFull: the support is the whole vocabulary and exceeds kMaxSupport; no support is selected (the draft row is read for
+// unusable logits only).
+template <typename T, bool kFull, int kInFlight, class SS>
+__device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b, int cr, int cn, int* check)
+{
+    using VT = VecTraits<T>;
+    constexpr int N = VT::N;
+    constexpr int S = kChunk / (32 * N);   // vectors per lane and chunk
+    constexpr int U = kInFlight < S ? kInFlight : S, NB = S / U;   // vectors of each row in flight, batches
+    constexpr int W = SS::kThr / 32;
+    static_assert(S % U == 0, "a chunk is a whole number of batches");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int V = A.V, ksel = A.ksel;
+    const T* qrow = (const T*)A.q + (size_t)b * V;
+    const T* prow = (const T*)A.p + (size_t)b * V;
+    const int head = row_head(A.q, b, V, (int)sizeof(T));
+    const int nch = num_chunks(V, head);
+    const int first = cr * W, stride = cn * W;           // this CTA's chunks: first + warp, + stride, ...
+    const bool take_all = !kFull && V <= SS::kCap;       // every element is a candidate
+    const bool use_tau = !kFull && !take_all;
+    if (tid == 0) { sh.cnt = 0; sh.bad = 0; sh.tau = -INFINITY; }
+    if (cn > 1) cluster_barrier(); else __syncthreads();
+
+    float g0 = -INFINITY;                  // running maximum of this thread's draft logits
+    unsigned long long chk = 0ull;         // plain sums (two packed): any NaN / inf makes them non-finite
+    const float sc_t = A.sc_t;
+    const unsigned long long sc2 = f_pack(sc_t, sc_t);
+    const int rounds = (nch + stride - 1) / stride;
+    const int vec_end = head + ((V - head) / N) * N, tail = V - vec_end;
+
+#pragma unroll 1
+    for (int r = 0; r < rounds; r++) {
+        const int c = first + r * stride + warp;
+        const bool cvalid = c < nch;
+        const bool whole = cvalid && head + (c + 1) * kChunk <= vec_end;
+        // target: this lane's (max, sum exp2) of the chunk, vector by vector; the elements before the first and behind the
+        // last vector come first.  (The order of these fp32 sums is part of the results: it decides the last bit of the
+        // chunk masses, and with 10^5 ids a resampled token can hang on that.)
+        float cm = -INFINITY, cs = 0.f;
+#pragma unroll 1
+        for (int nb = 0; nb < NB; nb++) {
+            const int base = head + c * kChunk + (nb * U * 32 + lane) * N;
+            const bool sample = use_tau && r == 0 && nb == 0;
+            const float tau = sample ? INFINITY : (use_tau ? *((volatile float*)&sh.tau) : -INFINITY);
+            ulonglong2 qv[U], pv[U];
+            if (cvalid) {
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    const int i0 = base + u * 32 * N;
+                    bool ok = whole || i0 + N <= vec_end;
+#ifdef GR_CHECK
+                    if (ok && (i0 < 0 || i0 + N > V || ((size_t)(qrow + i0) & 15) || ((size_t)(prow + i0) & 15))) { if (check) *check = 1; ok = false; }
+#endif
+                    if (ok) { qv[u] = ldg_stream(qrow + i0); pv[u] = ldg_stream(prow + i0); }
+                }
+                auto scalar = [&](int i) {
+                    const float x = load_logit<T>(qrow, i), v = load_logit<T>(prow, i);
+                    const float mn = fmaxf(cm, x);
+                    cs = fmaf(cs, ex2((cm - mn) * sc_t), ex2((x - mn) * sc_t));
+                    cm = mn;
+                    chk = add2(chk, f_pack(x, v));
+                    g0 = fmaxf(g0, v);
+                    if (!kFull) push_candidate(sh, v, i, tau);
+                };
+                if (nb == 0) {
+                    if (c == 0 && lane < head) scalar(lane);
+                    if (c == nch - 1 && lane < tail) scalar(vec_end + lane);
+                }
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    if (whole || base + u * 32 * N + N <= vec_end) {
+                        unsigned long long x[VT::kPairs];
+                        float vm = -INFINITY;
+#pragma unroll
+                        for (int i = 0; i < VT::kPairs; i++) {
+                            x[i] = VT::pair(qv[u], i);
+                            vm = fmaxf(vm, fmaxf(f_lo(x[i]), f_hi(x[i])));
+                            chk = add2(chk, x[i]);
+                        }
+                        const float mn = fmaxf(cm, vm);
+                        // (a factor of exactly one where the maximum stands)
+                        const float keep = cm == mn ? 1.f : ex2((cm - mn) * sc_t);
+                        const unsigned long long nm = f_pack(-mn, -mn);
+#pragma unroll
+                        for (int i = 0; i < VT::kPairs; i++) {
+                            const unsigned long long y = mul2(add2(x[i], nm), sc2);
+                            const float e0 = ex2(f_lo(y)), e1 = ex2(f_hi(y));
+                            cs = i == 0 ? fmaf(cs, keep, e0) : cs + e0;
+                            cs += e1;
+                        }
+                        cm = mn;
+                    }
+                }
+                // draft
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    if (whole || base + u * 32 * N + N <= vec_end) {
+                        float vm = -INFINITY;
+#pragma unroll
+                        for (int i = 0; i < VT::kPairs; i++) {
+                            const unsigned long long x = VT::pair(pv[u], i);
+                            vm = fmaxf(vm, fmaxf(f_lo(x), f_hi(x)));
+                            chk = add2(chk, x);
+                        }
+                        g0 = fmaxf(g0, vm);
+                        if (!kFull && vm >= tau) {
+#pragma unroll
+                            for (int i = 0; i < VT::kPairs; i++) {
+                                const unsigned long long x = VT::pair(pv[u], i);
+                                push_candidate(sh, f_lo(x), base + u * 32 * N + 2 * i, tau);
+                                push_candidate(sh, f_hi(x), base + u * 32 * N + 2 * i + 1, tau);
+                            }
+                        }
+                    }
+                }
+            }
+            if (sample) {
+                // the first batch had no threshold: it gives one, and its draft logits, still in registers, are tested now
+                refine_tau(sh, g0, ksel);
+                if (cvalid) {
+                    const float t1 = *((volatile float*)&sh.tau);
+#pragma unroll
+                    for (int u = 0; u < U; u++) {
+                        if (whole || base + u * 32 * N + N <= vec_end) {
+#pragma unroll
+                            for (int i = 0; i < VT::kPairs; i++) {
+                                const unsigned long long x = VT::pair(pv[u], i);
+                                if (fmaxf(f_lo(x), f_hi(x)) >= t1) {
+                                    push_candidate(sh, f_lo(x), base + u * 32 * N + 2 * i, t1);
+                                    push_candidate(sh, f_hi(x), base + u * 32 * N + 2 * i + 1, t1);
+                                }
+                            }
+                        }
+                    }
+                    if (c == 0 && lane < head) push_candidate(sh, load_logit<T>(prow, lane), lane, t1);
+                    if (c == nch - 1 && lane < tail) push_candidate(sh, load_logit<T>(prow, vec_end + lane), vec_end + lane, t1);
+                }
+            }
+        }
+        if (cvalid) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float mo = __shfl_xor_sync(0xffffffffu, cm, o), so = __shfl_xor_sync(0xffffffffu, cs, o);
+                osm_merge(cm, cs, mo, so, sc_t);
+            }
+            if (lane == 0) sh.chunk[c] = make_float2(cm, cs);
+        }
+        // a better threshold whenever the part read has grown fourfold (k = 50 of 512 groups: some 60 candidates in a first
+        // part, 180 more per fourfold)
+        if (use_tau && r + 1 < rounds && (r & (r + 1)) == 0 && ((r + 1) & 0x55555555)) refine_tau(sh, g0, ksel);
+    }
+    // non-finite inputs
+    {
+        const bool badl = !(fabsf(f_lo(chk)) <= 3.0e38f) || !(fabsf(f_hi(chk)) <= 3.0e38f);
+        if (__any_sync(0xffffffffu, badl) && lane == 0) atomicOr(&sh.bad, 1);
+    }
+    // ---- candidates: a last threshold from the whole part, then composite keys of those that pass it
+    __syncthreads();
+    if (cn == 1) lse_terms(sh, nch, A.temp_t);
+    if (use_tau && sh.cnt > kRankAll) refine_tau(sh, g0, ksel);
+    int M = 0, nsel = 0;
+    if (!kFull) {
+        nsel = ksel < V ? ksel : V;
+        if (sh.cnt > SS::kCap) exact_select_slow<T>(sh, prow, V, head, nch, first, stride, nsel);
+        M = min(sh.cnt, SS::kCap);
+        constexpr int kPer = SS::kCap / SS::kThr;
+        const float tau = use_tau ? sh.tau : -INFINITY;
+        unsigned long long kk[kPer];
+#pragma unroll
+        for (int u = 0; u < kPer; u++) {
+            const int e = tid + u * SS::kThr;
+            kk[u] = 0ull;
+            if (e < M) {
+                const float v = reinterpret_cast<const float*>(sh.keys)[e];
+                if (v >= tau) kk[u] = ckey(v, reinterpret_cast<const int*>(sh.keys)[SS::kCap + e]);
+            }
+        }
+        if (tid == 0) sh.kept = 0;
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kPer; u++) {
+            const bool on = kk[u] != 0ull;
+            const unsigned mk = __ballot_sync(0xffffffffu, on);
+            int at = 0;
+            if (mk != 0 && lane == 0) at = atomicAdd(&sh.kept, __popc(mk));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(mk & ((1u << lane) - 1u));
+            if (on) sh.keys[at] = kk[u];
+        }
+        __syncthreads();
+        M = sh.kept;
+    }
+    if (cn > 1) {
+        // ---- the other CTAs' parts to the first one: chunk entries, status, and each one's own nsel largest keys
+        const unsigned int lead_chunk = cluster_addr(&sh.chunk[0], 0), lead_keys = cluster_addr(&sh.keys[0], 0);
+        if (cr > 0) {
+            for (int c = first + warp; c < nch; c += stride) {
+                if (lane == 0) {
+                    const float2 t = sh.chunk[c];
+                    st_cluster(lead_chunk + 8u * (unsigned)c, f_pack(t.x, t.y));
+                }
+            }
+        }
+        const int keep = min(M, nsel);
+        // (the leader's list is overwritten only after it has taken its own largest: a barrier on both sides)
+        if (tid == 0) { st_cluster(cluster_addr(&sh.part_cnt[cr], 0), (unsigned int)keep); st_cluster(cluster_addr(&sh.part_bad[cr], 0), (unsigned int)sh.bad); }
+        unsigned long long own = 0ull;
+        int own_rank = -1;
+        // keep <= kMaxSupport <= kThr candidates survive in one CTA; a thread may hold several of the M, so survivors go
+        // through the upper half of the key array
+        unsigned long long* stage = sh.keys + SS::kCap - kMaxSupport;
+        const bool overlap = M > SS::kCap - kMaxSupport;
+        if (!overlap) rank_select(sh, M, keep, [&](int rank, unsigned long long key) { stage[rank] = key; });
+        __syncthreads();
+        if (!overlap && tid < keep) { own = stage[tid]; own_rank = tid; }
+        if (overlap) {
+            // (a list this full comes from rows of ties only: one thread per key, ranks counted from global order)
+            for (int e = tid; e < M; e += SS::kThr) {
+                const unsigned long long me = sh.keys[e];
+                int rank = 0;
+                for (int j = 0; j < M; j++) rank += (sh.keys[j] > me) ? 1 : 0;
+                if (rank < keep) sh.gkey[rank] = (unsigned int)e;
+            }
+            __syncthreads();
+            if (tid < keep) { own = sh.keys[sh.gkey[tid]]; own_rank = tid; }
+        }
+        cluster_barrier();
+        if (own_rank >= 0) st_cluster(lead_keys + 8u * (unsigned)(cr * kMaxSupport + own_rank), own);
+        cluster_barrier();
+        if (cr > 0) return;
+        // compact the parts
+        unsigned long long kk[kMaxCluster * kMaxSupport / SS::kThr];
+#pragma unroll
+        for (int u = 0; u < kMaxCluster * kMaxSupport / SS::kThr; u++) {
+            const int e = tid + u * SS::kThr, part = e / kMaxSupport, at = e % kMaxSupport;
+            kk[u] = (part < cn && at < sh.part_cnt[part]) ? sh.keys[e] : 0ull;
+        }
+        if (tid == 0) {
+            sh.kept = 0;
+            for (int i = 1; i < cn; i++) sh.bad |= sh.part_bad[i];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kMaxCluster * kMaxSupport / SS::kThr; u++) {
+            if (kk[u] != 0ull) sh.keys[atomicAdd(&sh.kept, 1)] = kk[u];
+        }
+        __syncthreads();
+        M = sh.kept;
+    }
+
+    // ---- row totals (the terms are in shared memory since a barrier at least)
+    if (cn > 1) lse_terms(sh, nch, A.temp_t);
+    if (cn > 1 || kFull) __syncthreads();
+    if (tid == SS::kThr - 1) {
+        double acc = sh.part[0];
+#pragma unroll
+        for (int w = 1; w < W; w++) acc += sh.part[w];
+        sh.lse[0] = sh.top / A.temp_t + m_log(acc);
+        if (!isfinite(sh.lse[0])) sh.bad = 1;
+    }
+    // ---- exact support out of the candidates
+    char* wsb = A.ws + (size_t)b * ws_stride();
+    if (!kFull) {
+        int* w_id_raw = reinterpret_cast<int*>(wsb + sizeof(WsHeader));
+        float* w_dl_raw = reinterpret_cast<float*>(w_id_raw + kMaxSupport);
+        GR_PTR(int) w_id = GR_MKPTR(int, w_id_raw, kMaxSupport, check);
+        GR_PTR(float) w_dl = GR_MKPTR(float, w_dl_raw, kMaxSupport, check);
+        GR_PTR(float) w_tl = GR_MKPTR(float, w_dl_raw + kMaxSupport, kMaxSupport, check);
+        if (M < nsel) nsel = M;   // cannot happen for finite rows; keeps the writes in range
+        rank_select(sh, M, nsel, [&](int rank, unsigned long long key) {
+            int id = (int)(0xffffffffu - (unsigned int)key);
+#ifdef GR_CHECK
+            if (id < 0 || id >= V) { if (check) *check = 1; id = 0; }
+#endif
+            w_id[rank] = id;
+            w_dl[rank] = fkey_inv((unsigned int)(key >> 32));
+            w_tl[rank] = load_logit<T>(qrow, id);
+        });
+    }
+    __syncthreads();
+    // ---- outputs: workspace header, chunk table and the header fields owned by this pass
+    if (tid == 0) {
+        WsHeader* wh = reinterpret_cast<WsHeader*>(wsb);
+        wh->lse_t = sh.lse[0];
+        wh->lse_d = 0.0;
+        wh->count = nsel;
+        wh->bad = sh.bad;
+        wh->check = check ? *check : 0;
+    }
+    if (A.params == nullptr) return;
+    char* pb = A.params + (size_t)b * A.pstride;
+    ParamView pv = view_params(pb, A.kcap, V, check);
+    for (int c = tid; c < nch; c += SS::kThr) pv.chunk[c] = sh.chunk[c];
+    if (tid == 0) {
+        Header* h = pv.h;
+        h->magic = 0;            // completed by the solve
+        h->V = V; h->nch = nch; h->head = head;
+        h->q_row = qrow;
+        h->dtype = sizeof(T) == 2 ? GR_BF16 : GR_F32;
+        h->lse_t = sh.lse[0];
+        h->temp_target = (float)A.temp_t;
+        h->kcap = A.kcap; h->stride = A.pstride;
+    }
+}
+
+}  // namespace gr

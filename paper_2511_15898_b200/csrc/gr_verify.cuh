@@ -80,12 +80,12 @@ static __device__ __noinline__ double block_incl_scan(double v, GR_PTR(double) r
 // Two levels: per-chunk masses from the scan kernel's table minus the flow p_i of the support ids in the chunk (one
 // chunk per thread), then an exact fp64 pass over the one chunk selected (its residuals in shared memory, a run of
 // consecutive ids per thread).  Bound by the latency of three dependent reads; with one warp per instance the two
-// passes took 25 us, as they do here 4.
+// passes took 25 us.
 __device__ inline int resample_draw(const Header* h, const ParamView& pv, int k, double frac, const VerifyScratch& vs)
 {
     const int tid = threadIdx.x, bd = blockDim.x;
     const int nch = h->nch, head = h->head, V = h->V, dtype = h->dtype;
-    const double T = (double)h->temp_target, lse = h->lse_t;
+    const double rT = m_div(1.0, (double)h->temp_target), lse = h->lse_t;
     const void* row = h->q_row;
     // the total residual mass is known in closed form (1 - alpha*, or 1 when the target itself is sampled)
     const double thr = frac * (k > 0 ? h->resid_total : 1.0);
@@ -95,14 +95,21 @@ __device__ inline int resample_draw(const Header* h, const ParamView& pv, int k,
 #pragma unroll 1
     for (int c0 = 0; c0 < nch; c0 += bd) {
         const int c = c0 + tid;
+        // flows of the support ids per chunk, as integers (2^-62 units: the sums do not depend on the order of the atomics)
+        GR_PTR(unsigned long long) sub = GR_PCAST(unsigned long long, vs.res);
+        sub[tid] = 0ull;
+        __syncthreads();
+        for (int j = tid; j < k; j += bd) {
+            const int at = vs.chunk[j] - c0;
+            if (at >= 0 && at < bd) atomicAdd(&sub[at], (unsigned long long)__double2ll_rn(vs.p[j] * 4611686018427387904.0));
+        }
         double R = 0.0;
         if (c < nch) {
             const float2 ms = pv.chunk[c];
-            R = (double)ms.y * m_exp(m_div((double)ms.x, T) - lse);
-#pragma unroll 4
-            for (int j = 0; j < k; j++) if (vs.chunk[j] == c) R -= vs.p[j];
-            if (R < 0.0) R = 0.0;
+            R = (double)ms.y * m_exp((double)ms.x * rT - lse);
         }
+        __syncthreads();
+        if (c < nch) R = fmax(R - (double)(long long)sub[tid] * (1.0 / 4611686018427387904.0), 0.0);
         double tot;
         const double inc = block_incl_scan(R, vs.red, &tot) + run;
         if (c < nch && inc > thr) atomicMin(&vs.dec[4], c);
@@ -121,7 +128,7 @@ __device__ inline int resample_draw(const Header* h, const ParamView& pv, int k,
     // ---- exact pass over the chunk in id order
     const int cb = chunk_begin(sel, head), len = chunk_end(sel, head, nch, V) - cb;
 #pragma unroll 4
-    for (int e = tid; e < len; e += bd) vs.res[e] = m_exp(m_div((double)load_logit_dyn(row, dtype, cb + e), T) - lse);
+    for (int e = tid; e < len; e += bd) vs.res[e] = exp_neg(lse - (double)load_logit_dyn(row, dtype, cb + e) * rT);
     __syncthreads();
     for (int j = tid; j < k; j += bd) if (vs.chunk[j] == sel) vs.res[vs.id[j] - cb] = pv.r[j];
     if (tid == 0) { vs.dec[4] = 0x7fffffff; vs.dec[5] = -1; }
