@@ -163,6 +163,9 @@ struct __align__(16) WsHeader {
     int pad;
 };
 // then: int id[kMaxSupport]; float dl[kMaxSupport]; float tl[kMaxSupport];
+// Of a whole-vocabulary row the streaming pass keeps, where the support would be: the draft row's maximum and the range of
+// the log-ratio draft / target (fp32, in units of log 2; it only places buckets).
+struct FullRow { float pmax, kmax, kmin, qmax; };
 __host__ __device__ inline int ws_stride() { return (int)sizeof(WsHeader) + kMaxSupport * 12; }
 
 // alignment head of row b: elements before the first 16-byte boundary

@@ -7,7 +7,8 @@
 // bucket_alpha_kernel finds that minimum without sorting the row: the log-ratio keys are binned into 4096 equal
 // buckets (a monotone map, so the bucket order is the ratio order), the bucket masses give psi exactly at every
 // bucket boundary, and a lower bound on psi inside a bucket (the ratios inside it span one bucket width) leaves
-// only the few buckets next to the minimum to be ordered exactly, in shared memory.  Three passes over the row.
+// only the few buckets next to the minimum to be ordered exactly, in shared memory.  One pass over the row (its maxima and
+// the range of the keys come from the streaming pass) and one over the 2-byte bucket numbers it leaves behind.
 // A row whose candidate buckets do not fit is handed to fullsort_alpha_kernel: one CTA per instance sorts (key, id)
 // pairs of the row in global scratch with a bitonic network, then scans tgt and drf along the order.
 // The network's passes with a compare distance below the tile size (4096 pairs, 48 KB) run on tiles staged in
@@ -37,36 +38,84 @@ constexpr int kBkThreads = 1024;
 constexpr int kBkBuckets = 4096;
 constexpr int kBkPer = kBkBuckets / kBkThreads;   // buckets per thread in the scan over buckets
 constexpr int kBkMaxCand = 4096;                  // elements of candidate buckets held in shared memory
-constexpr int kBkMaxPerBucket = 256;              // largest candidate bucket ordered in shared memory
-constexpr double kBkScale = 4398046511104.0;      // 2^42: masses are summed as integers (exact, order-free)
-constexpr int kBkSmemBytes = kBkBuckets * (8 + 8 + 4 + 4) + kBkMaxCand * (8 + 4 + 4);
+constexpr int kBkTab = 32, kBkCopies = 16;        // 2^(42 + j / 32), a copy for every lane of a half-warp
+constexpr int kBkSmemBytes = kBkBuckets * (4 * 4 + 4 + 4) + kBkMaxCand * (8 + 4 + 4 + 4 + 4) + kBkTab * kBkCopies * 8;
 
-__device__ inline unsigned long long mass_fixed(double x, double mx) { return (unsigned long long)llrint(exp(x - mx) * kBkScale); }
+// exp(-y) in units of 2^-42, rounded to an integer (masses are summed as integers: exact, order-free).  y >= 0.
+// 2^(k/32) from a table times a degree-5 Taylor polynomial on |r| <= ln2/64 (2e-15 relative, a hundredth of the unit):
+// ten fp64 operations, where exp and llrint took about forty.
+__device__ __forceinline__ unsigned long long mass_fixed(double y, GR_PTR(const double) tab)
+{
+    const double magic = 6755399441055744.0;                                   // 1.5 * 2^52
+    y = __hiloint2double(min(__double2hiint(y), 0x40468000), __double2loint(y));   // (at 45 and beyond it rounds to nothing)
+    const double m = fma(y, -46.16624130844682, magic);                        // 32 / ln 2
+    const int k = __double2loint(m);
+    const double r = fma(magic - m, 0.021660849392498290, -y);                 // ln 2 / 32
+    double p = fma(r, 8.333333333333333e-03, 4.1666666666666664e-02);
+    p = fma(r, p, 1.6666666666666666e-01);
+    p = fma(r, p, 0.5);
+    p = fma(r, p, 1.0);
+    p = fma(r, p, 1.0);
+    const double v = p * tab[(k & (kBkTab - 1)) * kBkCopies];                  // (tab: this lane's copy)
+    const double u = __hiloint2double(__double2hiint(v) + (k & ~(kBkTab - 1)) * 32768, __double2loint(v)) + 4503599627370496.0;   // 2^52
+    return (unsigned long long)__double_as_longlong(u) - 0x4330000000000000ull;
+}
 
-// Exclusive prefix over the CTA of one 64-bit integer per thread; *total gets the sum.  s_w: kBkThreads / 32 slots.
+// 64-bit sum in shared memory out of native 32-bit atomics: the carry out of the low word is rare
+__device__ __forceinline__ void add_mass(GR_PTR(unsigned) lo, GR_PTR(unsigned) hi, int c, unsigned long long v)
+{
+    const unsigned l = (unsigned)v, old = atomicAdd(&lo[c], l);
+    const unsigned h = (unsigned)(v >> 32) + (old + l < l ? 1u : 0u);
+    if (h != 0u) atomicAdd(&hi[c], h);
+}
+
+// x^n by squaring
+__device__ __forceinline__ double power(double x, int n)
+{
+    double r = 1.0;
+    for (; n > 0; n >>= 1) { if (n & 1) r *= x; x *= x; }
+    return r;
+}
+
+// Exclusive prefix over the CTA of one 64-bit integer per thread; *total gets the sum.  s_w: a slot per warp (32 of them).
 __device__ inline unsigned long long block_exscan_u64(unsigned long long v, unsigned long long* s_w,
                                                       unsigned long long* total)
 {
+    static_assert(kBkThreads == 1024, "one slot per lane");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned long long inc = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long t = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += t;
-    }
+    auto warp_scan = [&](unsigned long long x) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long t = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += t;
+        }
+        return x;
+    };
+    const unsigned long long inc = warp_scan(v);
     __syncthreads();
     if (lane == 31) s_w[warp] = inc;
     __syncthreads();
-    unsigned long long off = 0, tot = 0;
-    for (int w2 = 0; w2 < kBkThreads / 32; w2++) {
-        const unsigned long long x = s_w[w2];
-        if (w2 < warp) off += x;
-        tot += x;
-    }
-    *total = tot;
-    return off + inc - v;
+    const unsigned long long all = warp_scan(s_w[lane]);
+    const unsigned long long off = __shfl_sync(0xffffffffu, all, (warp + 31) & 31);
+    *total = __shfl_sync(0xffffffffu, all, 31);
+    return (warp > 0 ? off : 0ull) + inc - v;
+}
+// Minimum over the CTA, for every thread (s_r: a slot per warp; a barrier before its next use is the caller's).
+__device__ inline double block_min(double v, double* s_r)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if ((threadIdx.x & 31) == 0) s_r[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = s_r[threadIdx.x & 31];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
 }
 
 // flag[0] of the instance's scratch region: 1 when fullsort_alpha_kernel has to do the row, else 0.
+// 512 rows of 50257 in fp32: about 150 us (three passes with exp, 64-bit shared atomics and counts: 408).  Bound by the fp64 pipe (28
+// operations per id) and the shared atomics, not by the 206 MB it reads.
 template <typename T>
 __global__ void __launch_bounds__(kBkThreads)
 bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, int n, double temp_t, double temp_d,
@@ -79,26 +128,33 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, int
     pdl_trigger();
     GR_CHECK_FLAG_DECL;
     GR_CHECK_FLAG_INIT;
-    unsigned long long* const bt_raw = reinterpret_cast<unsigned long long*>(bk_smem);
-    int* const cnt_raw = reinterpret_cast<int*>(bt_raw + 2 * kBkBuckets);
-    double* const ckey_raw = reinterpret_cast<double*>(cnt_raw + 2 * kBkBuckets);
-    int* const cid_raw = reinterpret_cast<int*>(ckey_raw + kBkMaxCand);
-    GR_PTR(unsigned long long) bt = GR_MKPTR(unsigned long long, bt_raw, kBkBuckets, GR_CHECK_FLAG);   // target mass, then exclusive prefix
-    GR_PTR(unsigned long long) bd = GR_MKPTR(unsigned long long, bt_raw + kBkBuckets, kBkBuckets, GR_CHECK_FLAG);   // draft mass, ditto
-    GR_PTR(int) cnt = GR_MKPTR(int, cnt_raw, kBkBuckets, GR_CHECK_FLAG);            // elements per bucket / fill cursor
-    GR_PTR(int) seg = GR_MKPTR(int, cnt_raw + kBkBuckets, kBkBuckets, GR_CHECK_FLAG);   // start of a candidate's segment, -1
+    double* const ckey_raw = reinterpret_cast<double*>(bk_smem);
+    double* const tab_raw = ckey_raw + kBkMaxCand;
+    unsigned* const w_raw = reinterpret_cast<unsigned*>(tab_raw + kBkTab * kBkCopies);
+    int* const i_raw = reinterpret_cast<int*>(w_raw + 4 * kBkBuckets);
     GR_PTR(double) ckey = GR_MKPTR(double, ckey_raw, kBkMaxCand, GR_CHECK_FLAG);    // candidate elements: key,
-    GR_PTR(int) cid = GR_MKPTR(int, cid_raw, kBkMaxCand, GR_CHECK_FLAG);            // id,
-    GR_PTR(int) sid = GR_MKPTR(int, cid_raw + kBkMaxCand, kBkMaxCand, GR_CHECK_FLAG);   // ids in order
-    __shared__ double s_r[4][kBkThreads / 32];
+    GR_PTR(double) tab_all = GR_MKPTR(double, tab_raw, kBkTab * kBkCopies, GR_CHECK_FLAG);
+    GR_PTR(const double) tab = tab_all + (threadIdx.x & (kBkCopies - 1));
+    // target and draft mass of a bucket, then the exclusive prefix (low and high words)
+    GR_PTR(unsigned) tl = GR_MKPTR(unsigned, w_raw, kBkBuckets, GR_CHECK_FLAG), th = GR_MKPTR(unsigned, w_raw + kBkBuckets, kBkBuckets, GR_CHECK_FLAG);
+    GR_PTR(unsigned) dl = GR_MKPTR(unsigned, w_raw + 2 * kBkBuckets, kBkBuckets, GR_CHECK_FLAG), dh = GR_MKPTR(unsigned, w_raw + 3 * kBkBuckets, kBkBuckets, GR_CHECK_FLAG);
+    GR_PTR(int) cnt = GR_MKPTR(int, i_raw, kBkBuckets, GR_CHECK_FLAG);              // elements of a candidate bucket / fill cursor
+    GR_PTR(int) seg = GR_MKPTR(int, i_raw + kBkBuckets, kBkBuckets, GR_CHECK_FLAG); // start of a candidate's segment; -1: none
+    GR_PTR(int) cid = GR_MKPTR(int, i_raw + 2 * kBkBuckets, kBkMaxCand, GR_CHECK_FLAG);                      // id,
+    GR_PTR(int) sid = GR_MKPTR(int, i_raw + 2 * kBkBuckets + kBkMaxCand, kBkMaxCand, GR_CHECK_FLAG);         // ids in order,
+    GR_PTR(int) lid = GR_MKPTR(int, i_raw + 2 * kBkBuckets + 2 * kBkMaxCand, kBkMaxCand, GR_CHECK_FLAG);     // ids and
+    GR_PTR(int) lbk = GR_MKPTR(int, i_raw + 2 * kBkBuckets + 3 * kBkMaxCand, kBkMaxCand, GR_CHECK_FLAG);     // buckets as found
+    __shared__ double s_r[kBkThreads / 32];
     __shared__ unsigned long long s_w[kBkThreads / 32];
-    __shared__ int s_nelem, s_fallback;
+    __shared__ int s_nelem, s_found, s_fallback, s_lo, s_hi;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long b = blockIdx.x;
-    const WsHeader* wh = reinterpret_cast<const WsHeader*>(ws + (size_t)b * ws_stride());
+    const char* const rec = ws + (size_t)b * ws_stride();
+    const WsHeader* wh = reinterpret_cast<const WsHeader*>(rec);
     // (no params block and a status array when called for the optimal acceptance alone)
     Header* hdr = params ? reinterpret_cast<Header*>(params + (size_t)b * pstride) : nullptr;
-    int* flag = reinterpret_cast<int*>(scratch + (size_t)b * scratch_stride);
+    char* const scr = scratch + (size_t)b * scratch_stride;
+    int* flag = reinterpret_cast<int*>(scr);
     if (tid == 0 && status_out) status_out[b] = wh->bad != 0 ? GR_BAD_LOGITS : GR_OK;
     if (wh->bad != 0 || force_sort) {
         if (tid == 0) {
@@ -109,85 +165,140 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, int
     }
     const T* qrow = q + (size_t)b * V;
     const T* prow = p + (size_t)b * V;
+    const FullRow fr = *reinterpret_cast<const FullRow*>(rec + sizeof(WsHeader));
     // (scaled logits as products with the reciprocal temperatures: one rounding away from the quotients the sort
     // uses, which moves alpha* by ~1e-16; every pass here forms them the same way)
     const double rt = 1.0 / temp_t, rd = 1.0 / temp_d;
-    // ---- pass 1: maxima of both scaled rows, range of the key d - a
-    double mt = -1.0e300, md = -1.0e300, kmax = -1.0e300, kmin = 1.0e300;
-#pragma unroll 4
-    for (int i = tid; i < V; i += kBkThreads) {
-        const double a = (double)load_logit<T>(qrow, i) * rt, d = (double)load_logit<T>(prow, i) * rd;
-        mt = fmax(mt, a); md = fmax(md, d); kmax = fmax(kmax, d - a); kmin = fmin(kmin, d - a);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        mt = fmax(mt, __shfl_xor_sync(0xffffffffu, mt, o)); md = fmax(md, __shfl_xor_sync(0xffffffffu, md, o));
-        kmax = fmax(kmax, __shfl_xor_sync(0xffffffffu, kmax, o)); kmin = fmin(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
-    }
-    if (lane == 0) { s_r[0][warp] = mt; s_r[1][warp] = md; s_r[2][warp] = kmax; s_r[3][warp] = kmin; }
-    for (int c = tid; c < kBkBuckets; c += kBkThreads) { bt[c] = 0ull; bd[c] = 0ull; cnt[c] = 0; seg[c] = -1; }
-    if (tid == 0) { s_nelem = 0; s_fallback = 0; }
-    __syncthreads();
-    for (int w2 = 0; w2 < kBkThreads / 32; w2++) {
-        mt = fmax(mt, s_r[0][w2]); md = fmax(md, s_r[1][w2]); kmax = fmax(kmax, s_r[2][w2]); kmin = fmin(kmin, s_r[3][w2]);
-    }
-    // bucket of a key: floor((kmax - key) * invw), a non-decreasing function of kmax - key in floating point, so
-    // every element of a lower bucket comes before every element of a higher one in the ratio order
-    const double span = kmax - kmin;
+    const double mt = (double)fr.qmax * rt, md = (double)fr.pmax * rd;
+    // bucket of a key d - a: floor((kmax - key) * invw), clamped: a non-decreasing function of kmax - key in floating
+    // point, so every element of a lower bucket comes before every element of a higher one in the ratio order.  (kmax
+    // and kmin are fp32 values: a key may lie outside.)
+    const double ln2 = 0.6931471805599453;
+    const double kmax = (double)fr.kmax * ln2, span = kmax - (double)fr.kmin * ln2;
     const double invw = span > 0.0 ? (double)kBkBuckets / (span * (1.0 + 1e-9)) : 0.0;
-    // ---- pass 2: bucket masses (integers: the sums do not depend on the order of the atomics)
-#pragma unroll 4
-    for (int i = tid; i < V; i += kBkThreads) {
-        const double a = (double)load_logit<T>(qrow, i) * rt, d = (double)load_logit<T>(prow, i) * rd;
-        const int c = min(kBkBuckets - 1, (int)((kmax - (d - a)) * invw));
-        atomicAdd(&bt[c], mass_fixed(a, mt));
-        atomicAdd(&bd[c], mass_fixed(d, md));
-        atomicAdd(&cnt[c], 1);
+    for (int c = tid; c < kBkBuckets; c += kBkThreads) { tl[c] = 0u; th[c] = 0u; dl[c] = 0u; dh[c] = 0u; cnt[c] = 0; seg[c] = -1; }
+    for (int e = tid; e < kBkTab * kBkCopies; e += kBkThreads) tab_all[e] = exp2(42.0 + (double)(e / kBkCopies) / kBkTab);
+    if (tid == 0) { s_nelem = 0; s_found = 0; s_fallback = 0; s_lo = kBkBuckets; s_hi = -1; }
+    __syncthreads();
+    // ---- the row: bucket masses (integers: the sums do not depend on the order of the atomics), bucket numbers to scratch
+    // (number of id i at code[i + shift], so that a vector of logits has its numbers in one aligned store)
+    constexpr int N = 16 / (int)sizeof(T);
+    const int head = row_head(q, b, V, (int)sizeof(T)), shift = (N - head % N) % N;
+    unsigned short* const code_raw = reinterpret_cast<unsigned short*>(scr + 16);
+    GR_PTR(unsigned short) code = GR_MKPTR(unsigned short, code_raw, V + 16, GR_CHECK_FLAG);
+    auto key_of = [&](float x, float v) { return (double)v * rd - (double)x * rt; };
+    auto element = [&](float x, float v) {
+        const double a = (double)x * rt, d = (double)v * rd;
+        const double t = __dadd_rd((kmax - (d - a)) * invw, 6755399441055744.0);
+        const int c = min(max(__double2loint(t), 0), kBkBuckets - 1);
+        add_mass(tl, th, c, mass_fixed(mt - a, tab));
+        add_mass(dl, dh, c, mass_fixed(md - d, tab));
+        return c;
+    };
+    const int nvec = (V - head) / N, tail0 = head + nvec * N;
+    if (tid < head) code[tid + shift] = (unsigned short)element(load_logit<T>(qrow, tid), load_logit<T>(prow, tid));
+    if (tid < V - tail0) code[tail0 + tid + shift] = (unsigned short)element(load_logit<T>(qrow, tail0 + tid), load_logit<T>(prow, tail0 + tid));
+    const uint4* const qv = reinterpret_cast<const uint4*>(qrow + head);
+    const uint4* const pv = reinterpret_cast<const uint4*>(prow + head);
+    uint4 xq = make_uint4(0u, 0u, 0u, 0u), xp = xq;
+    if (tid < nvec) { xq = __ldcs(qv + tid); xp = __ldcs(pv + tid); }
+#pragma unroll 1
+    for (int e = tid; e < nvec; e += kBkThreads) {
+        const uint4 cq = xq, cp = xp;
+        if (e + kBkThreads < nvec) { xq = __ldcs(qv + e + kBkThreads); xp = __ldcs(pv + e + kBkThreads); }
+        const unsigned wq[4] = {cq.x, cq.y, cq.z, cq.w}, wp[4] = {cp.x, cp.y, cp.z, cp.w};
+        unsigned out[N / 2];
+#pragma unroll
+        for (int z = 0; z < N; z += 2) {
+            float x0, x1, v0, v1;
+            if (N == 4) {
+                x0 = __uint_as_float(wq[z & 3]); x1 = __uint_as_float(wq[(z + 1) & 3]);
+                v0 = __uint_as_float(wp[z & 3]); v1 = __uint_as_float(wp[(z + 1) & 3]);
+            } else {
+                x0 = __uint_as_float(wq[z / 2] << 16); x1 = __uint_as_float(wq[z / 2] & 0xffff0000u);
+                v0 = __uint_as_float(wp[z / 2] << 16); v1 = __uint_as_float(wp[z / 2] & 0xffff0000u);
+            }
+            const int c0 = element(x0, v0), c1 = element(x1, v1);
+            out[z / 2] = (unsigned)c0 | ((unsigned)c1 << 16);
+        }
+        const int at = head + e * N + shift;                       // a multiple of N; at + N <= V + N
+#ifdef GR_CHECK
+        if (at < 0 || at + N > V + 16) { s_check_flag = 1; continue; }
+#endif
+        if (N == 4) *reinterpret_cast<uint2*>(code_raw + at) = make_uint2(out[0], out[1]);
+        else *reinterpret_cast<uint4*>(code_raw + at) = make_uint4(out[0], out[1], out[N / 2 - 2], out[N / 2 - 1]);
     }
     __syncthreads();
     // ---- prefixes over the buckets, psi at every boundary, lower bound inside every bucket
     unsigned long long mT[kBkPer], mD[kBkPer], sT = 0, sD = 0;
 #pragma unroll
-    for (int u = 0; u < kBkPer; u++) { mT[u] = bt[tid * kBkPer + u]; mD[u] = bd[tid * kBkPer + u]; sT += mT[u]; sD += mD[u]; }
+    for (int u = 0; u < kBkPer; u++) {
+        const int c = tid * kBkPer + u;
+        mT[u] = ((unsigned long long)th[c] << 32) | tl[c]; mD[u] = ((unsigned long long)dh[c] << 32) | dl[c];
+        sT += mT[u]; sD += mD[u];
+    }
     unsigned long long totT, totD;
     unsigned long long pT = block_exscan_u64(sT, s_w, &totT);
     unsigned long long pD = block_exscan_u64(sD, s_w, &totD);
     const double iT = 1.0 / (double)totT, iD = 1.0 / (double)totD;
     // tgt_i / drf_i = exp(-key_i) * rscale
     const double rscale = exp(md - mt) * ((double)totD / (double)totT);
+    const double slack = (double)(V + 1) * iT + 1e-14;
     double lb[kBkPer], best = 0.0;                          // psi of the empty prefix
 #pragma unroll
     for (int u = 0; u < kBkPer; u++) {
         const int c = tid * kBkPer + u;
-        bt[c] = pT; bd[c] = pD;
+        tl[c] = (unsigned)pT; th[c] = (unsigned)(pT >> 32); dl[c] = (unsigned)pD; dh[c] = (unsigned)(pD >> 32);
         const double T0 = (double)pT * iT, D0 = (double)pD * iD;
         pT += mT[u]; pD += mD[u];
         const double T1 = (double)pT * iT, D1 = (double)pD * iD;
-        const double dn = pow(D1, (double)n);
-        if (cnt[c] > 0) best = fmin(best, T1 - dn);
-        // Inside the bucket every ratio tgt / drf is at least rho (its keys are at most kmax - c w), so a prefix that
-        // ends inside it has  psi >= T0 + rho (D - D0) - D^n,  concave in D: its minimum over [D0, D1] is at an end.
-        // At D0 that is the previous boundary's psi; at D1 it is the bound below.  The slack covers the rounding of
-        // the masses to integers (one unit each).
+        const double dn = power(D1, n);
+        best = fmin(best, T1 - dn);
+        // Inside the bucket every ratio tgt / drf is at least rho (its keys are at most kmax - c w; the first bucket has no
+        // such limit), so a prefix that ends inside it has  psi >= T0 + rho (D - D0) - D^n,  concave in D: its minimum
+        // over [D0, D1] is at an end.  At D0 that is the previous boundary's psi; at D1 it is the bound below.  The slack
+        // covers the rounding of the masses to integers (one unit per id).
         const double khi = kmax - (invw > 0.0 ? (double)c / invw * (1.0 - 1e-12) : 0.0);
-        const double rho = exp(-khi) * rscale * (1.0 - 1e-9);
-        lb[u] = T0 + rho * (D1 - D0) - dn - ((double)(cnt[c] + 1) * iT + 1e-14);
+        const double rho = c == 0 ? 0.0 : exp(-khi) * rscale * (1.0 - 1e-9);
+        lb[u] = mT[u] + mD[u] == 0ull ? 1.0 : T0 + rho * (D1 - D0) - dn - slack;
     }
-    for (int o = 16; o > 0; o >>= 1) best = fmin(best, __shfl_xor_sync(0xffffffffu, best, o));
-    __syncthreads();
-    if (lane == 0) s_r[0][warp] = best;
-    __syncthreads();
-    for (int w2 = 0; w2 < kBkThreads / 32; w2++) best = fmin(best, s_r[0][w2]);
+    best = block_min(best, s_r);
     // ---- candidate buckets: those whose interior could hold a smaller psi
 #pragma unroll
     for (int u = 0; u < kBkPer; u++) {
-        const int c = tid * kBkPer + u, L = cnt[c];
-        if (L >= 2 && lb[u] < best) {
-            if (L > kBkMaxPerBucket) s_fallback = 1;
-            else {
-                const int off = atomicAdd(&s_nelem, L);
-                if (off + L > kBkMaxCand) s_fallback = 1;
-                else { seg[c] = off; cnt[c] = 0; }
+        const int c = tid * kBkPer + u;
+        if (lb[u] < best) { seg[c] = 0; atomicMin(&s_lo, c); atomicMax(&s_hi, c); }
+    }
+    __syncthreads();
+    const int lo = s_lo, hi = s_hi;
+    // ---- their elements, found by the bucket numbers
+    if (hi >= lo) {
+        const int ncode = V + shift;
+#pragma unroll 2
+        for (int e = tid; e < (ncode + 7) / 8; e += kBkThreads) {
+            const uint4 w = *reinterpret_cast<const uint4*>(code_raw + 8 * e);     // (16-byte aligned; within the region)
+            const unsigned ww[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+            for (int z = 0; z < 8; z++) {
+                const int c = (int)((ww[z / 2] >> (16 * (z & 1))) & 0xffffu), i = 8 * e + z - shift;
+                if (c >= lo && c <= hi && i >= 0 && i < V && seg[c] >= 0) {
+                    const int at = atomicAdd(&s_found, 1);
+                    if (at < kBkMaxCand) { lid[at] = i; lbk[at] = c; }
+                    atomicAdd(&cnt[c], 1);
+                }
             }
+        }
+    }
+    __syncthreads();
+    const int found = s_found;
+#pragma unroll
+    for (int u = 0; u < kBkPer; u++) {
+        const int c = tid * kBkPer + u;
+        if (seg[c] >= 0) {
+            const int L = cnt[c];
+            if (found > kBkMaxCand) s_fallback = 1;
+            else if (L >= 2) { seg[c] = atomicAdd(&s_nelem, L); cnt[c] = 0; }
+            else seg[c] = -1;
         }
     }
     __syncthreads();
@@ -195,61 +306,64 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, int
         if (tid == 0) flag[0] = 1;
         return;
     }
-    // ---- pass 3: the candidates' elements, each bucket into its own segment
+    // ---- each bucket into its own segment, ordered by (key descending, id ascending) by counting
     if (s_nelem > 0) {
-#pragma unroll 4
-        for (int i = tid; i < V; i += kBkThreads) {
-            const double a = (double)load_logit<T>(qrow, i) * rt, d = (double)load_logit<T>(prow, i) * rd;
-            const int c = min(kBkBuckets - 1, (int)((kmax - (d - a)) * invw));
-            if (seg[c] >= 0) {
-                const int pos = seg[c] + atomicAdd(&cnt[c], 1);
-                ckey[pos] = d - a; cid[pos] = i;
+        constexpr int kOwn = kBkMaxCand / kBkThreads;
+        int pos[kOwn];
+#pragma unroll
+        for (int u = 0; u < kOwn; u++) {
+            const int e = tid + u * kBkThreads;
+            pos[u] = -1;
+            if (e < found) {
+                const int c = lbk[e], i = lid[e];
+                if (seg[c] >= 0) {
+                    pos[u] = seg[c] + atomicAdd(&cnt[c], 1);
+                    ckey[pos[u]] = key_of(load_logit<T>(qrow, i), load_logit<T>(prow, i)); cid[pos[u]] = i;
+                }
             }
         }
-    }
-    __syncthreads();
-    // ---- one warp per candidate bucket: order by (key descending, id ascending) by counting, then walk the prefixes
-    if (s_nelem > 0) {
-        for (int c = warp; c < kBkBuckets; c += kBkThreads / 32) {
-            const int off = seg[c];
-            if (off < 0) continue;
-            const int L = cnt[c];
-            for (int e = lane; e < L; e += 32) {
-                const double ke = ckey[off + e];
-                const int ie = cid[off + e];
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kOwn; u++) {
+            if (pos[u] >= 0) {
+                const int c = lbk[tid + u * kBkThreads], off = seg[c], L = cnt[c];
+                const double ke = ckey[pos[u]];
+                const int ie = cid[pos[u]];
                 int rank = 0;
-                for (int j = 0; j < L; j++) {
-                    const double kj = ckey[off + j];
-                    const int ij = cid[off + j];
-                    rank += (kj > ke || (kj == ke && ij < ie)) ? 1 : 0;
+                for (int j = off; j < off + L; j++) {
+                    const double kj = ckey[j];
+                    rank += (kj > ke || (kj == ke && cid[j] < ie)) ? 1 : 0;
                 }
                 sid[off + rank] = ie;
             }
-            __syncwarp();
-            unsigned long long cT = bt[c], cD = bd[c];
+        }
+        __syncthreads();
+    }
+    // ---- one warp per candidate bucket walks the prefixes
+    if (s_nelem > 0) {
+        for (int c = lo + warp; c <= hi; c += kBkThreads / 32) {
+            const int off = seg[c];
+            if (off < 0) continue;
+            const int L = cnt[c];
+            unsigned long long cT = ((unsigned long long)th[c] << 32) | tl[c], cD = ((unsigned long long)dh[c] << 32) | dl[c];
             for (int base = 0; base < L; base += 32) {
                 unsigned long long tf = 0, df = 0;
                 if (base + lane < L) {
                     const int id = sid[off + base + lane];
-                    tf = mass_fixed((double)load_logit<T>(qrow, id) * rt, mt);
-                    df = mass_fixed((double)load_logit<T>(prow, id) * rd, md);
+                    tf = mass_fixed(mt - (double)load_logit<T>(qrow, id) * rt, tab);
+                    df = mass_fixed(md - (double)load_logit<T>(prow, id) * rd, tab);
                 }
                 for (int o = 1; o < 32; o <<= 1) {
                     const unsigned long long t2 = __shfl_up_sync(0xffffffffu, tf, o), d2 = __shfl_up_sync(0xffffffffu, df, o);
                     if (lane >= o) { tf += t2; df += d2; }
                 }
                 if (base + lane < L)
-                    best = fmin(best, (double)(cT + tf) * iT - pow((double)(cD + df) * iD, (double)n));
+                    best = fmin(best, (double)(cT + tf) * iT - power((double)(cD + df) * iD, n));
                 cT += __shfl_sync(0xffffffffu, tf, 31); cD += __shfl_sync(0xffffffffu, df, 31);
             }
         }
-        for (int o = 16; o > 0; o >>= 1) best = fmin(best, __shfl_xor_sync(0xffffffffu, best, o));
-        __syncthreads();
-        if (lane == 0) s_r[0][warp] = best;
-        __syncthreads();
-        for (int w2 = 0; w2 < kBkThreads / 32; w2++) best = fmin(best, s_r[0][w2]);
+        best = block_min(best, s_r);
     }
-    __syncthreads();
     if (tid == 0) {
         flag[0] = 0;
         if (hdr) { hdr->alpha_star = 1.0 + best; hdr->resid_total = -best; }
@@ -266,7 +380,7 @@ template <typename T>
 __global__ void __launch_bounds__(kFsThreads)
 fullsort_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, int n, double temp_t, double temp_d,
                       const char* __restrict__ ws, char* __restrict__ scratch, char* __restrict__ params, int pstride,
-                      float* __restrict__ alpha_out, int out_stride, int out_off)
+                      int batch, float* __restrict__ alpha_out, int out_stride, int out_off)
 {
     __shared__ double s_a[kFsThreads / 32], s_b[kFsThreads / 32];
     __shared__ double s_carry[2];
@@ -274,10 +388,12 @@ fullsort_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, i
     pdl_wait();
     pdl_trigger();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long b = blockIdx.x;
+    // (normally no row is left to it: a grid of one wave looks)
+#pragma unroll 1
+    for (long long b = blockIdx.x; b < batch; b += gridDim.x) {
     const WsHeader* wh = reinterpret_cast<const WsHeader*>(ws + (size_t)b * ws_stride());
     Header* hdr = params ? reinterpret_cast<Header*>(params + (size_t)b * pstride) : nullptr;
-    if (wh->bad != 0) return;                       // header / status already say GR_BAD_LOGITS
+    if (wh->bad != 0) continue;                     // header / status already say GR_BAD_LOGITS
     const T* qrow = q + (size_t)b * V;
     const T* prow = p + (size_t)b * V;
     const int VP = next_pow2(V);
@@ -285,7 +401,7 @@ fullsort_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, i
     // the first word of the region says whether bucket_alpha_kernel left this row to the sort
     const int todo = reinterpret_cast<const int*>(key)[0];
     __syncthreads();
-    if (todo == 0) return;
+    if (todo == 0) continue;
     int* idx = reinterpret_cast<int*>(key + VP);
     for (int i = tid; i < VP; i += kFsThreads) {
         if (i < V) {
@@ -424,6 +540,8 @@ fullsort_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, i
         if (hdr) { hdr->alpha_star = 1.0 + best; hdr->resid_total = -best; }
         alpha_out[(size_t)b * out_stride + out_off] = (float)(1.0 + best);
     }
+    __syncthreads();
+    }
 }
 
 void launch_fullsort(const void* q, const void* p, int dtype, int V, int n, double temp_t, double temp_d, int batch,
@@ -445,7 +563,8 @@ void launch_fullsort(const void* q, const void* p, int dtype, int V, int n, doub
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, kBkSmemBytes) == cudaSuccess;
         if (dev >= 0 && ok) configured[dev] = true;
     }
-    const size_t sstride = (size_t)next_pow2(V) * 12;
+    const size_t sstride = (size_t)next_pow2(V) * 12;       // (room for V + 16 bucket numbers behind the flag: V > GR_MAX_SUPPORT)
+    const int sort_grid = batch < 148 ? batch : 148;
     if (dtype == GR_F32)
         launch_pdl(bucket_alpha_kernel<float>, batch, kBkThreads, kBkSmemBytes, st, (const float*)q, (const float*)p, V, n, temp_t,
                                                                             temp_d, ws, scratch, sstride, params, pstride,
@@ -458,14 +577,14 @@ void launch_fullsort(const void* q, const void* p, int dtype, int V, int n, doub
                                                                                     pstride, force_sort, alpha_out, out_stride,
                                                                                     out_off, status_out);
     if (dtype == GR_F32)
-        launch_pdl(fullsort_alpha_kernel<float>, batch, kFsThreads, kFsSmemBytes, st, (const float*)q, (const float*)p, V, n, temp_t,
-                                                                   temp_d, ws, scratch, params, pstride, alpha_out,
+        launch_pdl(fullsort_alpha_kernel<float>, sort_grid, kFsThreads, kFsSmemBytes, st, (const float*)q, (const float*)p, V, n, temp_t,
+                                                                   temp_d, ws, scratch, params, pstride, batch, alpha_out,
                                                                    out_stride, out_off);
     else
-        launch_pdl(fullsort_alpha_kernel<__nv_bfloat16>, batch, kFsThreads, kFsSmemBytes, st, (const __nv_bfloat16*)q,
+        launch_pdl(fullsort_alpha_kernel<__nv_bfloat16>, sort_grid, kFsThreads, kFsSmemBytes, st, (const __nv_bfloat16*)q,
                                                                            (const __nv_bfloat16*)p, V, n, temp_t,
                                                                            temp_d, ws, scratch, params, pstride,
-                                                                           alpha_out, out_stride, out_off);
+                                                                           batch, alpha_out, out_stride, out_off);
 }
 
 }  // namespace gr

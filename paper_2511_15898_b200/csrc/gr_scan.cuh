@@ -242,12 +242,19 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
     const bool take_all = !kFull && V <= SS::kCap;       // every element is a candidate
     const bool use_tau = !kFull && !take_all;
     if (tid == 0) { sh.cnt = 0; sh.bad = 0; sh.tau = -INFINITY; }
+    if (kFull && tid < 3) sh.hist[tid] = 0;
     if (cn > 1) cluster_barrier(); else __syncthreads();
 
     float g0 = -INFINITY;                  // running maximum of this thread's draft logits
     unsigned long long chk = 0ull;         // plain sums (two packed): any NaN / inf makes them non-finite
     const float sc_t = A.sc_t;
     const unsigned long long sc2 = f_pack(sc_t, sc_t);
+    float kmax = -INFINITY, kmin = INFINITY;                // range of the log-ratios draft / target (kFull)
+    auto ratio_range = [&](unsigned long long x, unsigned long long v) {
+        const unsigned long long m = mul2(x, f_pack(-sc_t, -sc_t));
+        const float k0 = fmaf(f_lo(v), A.sc_d, f_lo(m)), k1 = fmaf(f_hi(v), A.sc_d, f_hi(m));
+        kmax = fmaxf(kmax, fmaxf(k0, k1)); kmin = fminf(kmin, fminf(k0, k1));
+    };
     const int rounds = (nch + stride - 1) / stride;
     const int vec_end = head + ((V - head) / N) * N, tail = V - vec_end;
 
@@ -283,6 +290,7 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
                     cm = mn;
                     chk = add2(chk, f_pack(x, v));
                     g0 = fmaxf(g0, v);
+                    if (kFull) ratio_range(f_pack(x, x), f_pack(v, v));
                     if (!kFull) push_candidate(sh, v, i, tau);
                 };
                 if (nb == 0) {
@@ -326,6 +334,10 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
                             chk = add2(chk, x);
                         }
                         g0 = fmaxf(g0, vm);
+                        if (kFull) {
+#pragma unroll
+                            for (int i = 0; i < VT::kPairs; i++) ratio_range(VT::pair(qv[u], i), VT::pair(pv[u], i));
+                        }
                         if (!kFull && vm >= tau) {
 #pragma unroll
                             for (int i = 0; i < VT::kPairs; i++) {
@@ -470,6 +482,13 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
         M = sh.kept;
     }
 
+    if (kFull) {
+        // (sh.hist is zero)
+        const unsigned a = __reduce_max_sync(0xffffffffu, fkey(g0)), k1 = __reduce_max_sync(0xffffffffu, fkey(kmax));
+        const unsigned k0 = __reduce_max_sync(0xffffffffu, fkey(-kmin));
+        unsigned* const top = reinterpret_cast<unsigned*>(sh.hist);
+        if (lane == 0) { atomicMax(&top[0], a); atomicMax(&top[1], k1); atomicMax(&top[2], k0); }
+    }
     // ---- row totals (the terms are in shared memory since a barrier at least)
     if (cn > 1) lse_terms(sh, nch, A.temp_t);
     if (cn > 1 || kFull) __syncthreads();
@@ -508,6 +527,12 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
         wh->count = nsel;
         wh->bad = sh.bad;
         wh->check = check ? *check : 0;
+        if (kFull) {
+            const unsigned* const top = reinterpret_cast<const unsigned*>(sh.hist);
+            FullRow fr;
+            fr.pmax = fkey_inv(top[0]); fr.kmax = fkey_inv(top[1]); fr.kmin = -fkey_inv(top[2]); fr.qmax = (float)sh.top;
+            *reinterpret_cast<FullRow*>(wsb + sizeof(WsHeader)) = fr;
+        }
     }
     if (A.params == nullptr) return;
     char* pb = A.params + (size_t)b * A.pstride;
