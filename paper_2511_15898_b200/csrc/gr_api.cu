@@ -103,9 +103,8 @@ static int solve_impl(const void* q_logits, const void* p_logits, int dtype, int
         // no rule is solved for this shape, but the optimal acceptance still is (bucketed search for the minimum of
         // psi, or with force_robust a sort of the whole row and a prefix scan)
         char* scratch = (char*)workspace + (size_t)gr::ws_stride() * (size_t)batch;
-        gr::launch_fullsort(q_logits, p_logits, dtype, V, n, (double)temp_target, (double)temp_draft, batch,
-                            (const char*)workspace, scratch, (char*)params, pstride, force_robust, alpha_star, 1, 0,
-                            nullptr, st);
+        gr::launch_fullsort(q_logits, p_logits, dtype, V, &n, 1, (double)temp_target, (double)temp_draft, batch,
+                            (const char*)workspace, scratch, (char*)params, pstride, force_robust, alpha_star, nullptr, st);
     }
     if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return GR_E_LAUNCH; }
     return GR_OK;
@@ -153,13 +152,12 @@ int gr_alpha_star(const void* q_logits, const void* p_logits, int dtype, int V, 
     gr::NvtxRange whole("gr_alpha_star");
     if (kcap == 0) {
         // untruncated draft on a large vocabulary: the streaming pass for the row statistics, then the bucketed
-        // search for min psi once per draft count (rows it cannot separate take the sort)
+        // search for min psi for all draft counts (rows it cannot separate take the sort)
         gr::launch_scan(q_logits, p_logits, dtype, V, kfull, true, (double)temp_target, (double)temp_draft, batch,
                         (char*)workspace, nullptr, 0, kcap, st);
         char* scratch = (char*)workspace + (size_t)gr::ws_stride() * (size_t)batch;
-        for (int j = 0; j < n_count; j++)
-            gr::launch_fullsort(q_logits, p_logits, dtype, V, n_list[j], (double)temp_target, (double)temp_draft, batch,
-                                (const char*)workspace, scratch, nullptr, 0, 0, alpha_star, n_count, j, status, st);
+        gr::launch_fullsort(q_logits, p_logits, dtype, V, n_list, n_count, (double)temp_target, (double)temp_draft, batch,
+                            (const char*)workspace, scratch, nullptr, 0, 0, alpha_star, status, st);
         if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return GR_E_LAUNCH; }
         return GR_OK;
     }

@@ -69,6 +69,9 @@ __device__ __forceinline__ void add_mass(GR_PTR(unsigned) lo, GR_PTR(unsigned) h
     if (h != 0u) atomicAdd(&hi[c], h);
 }
 
+// Draft counts of one call: everything but the last step is common to them.
+struct NList { int count; int n[GR_MAX_ALPHA_N]; };
+
 // x^n by squaring
 __device__ __forceinline__ double power(double x, int n)
 {
@@ -113,15 +116,15 @@ __device__ inline double block_min(double v, double* s_r)
     return v;
 }
 
-// flag[0] of the instance's scratch region: 1 when fullsort_alpha_kernel has to do the row, else 0.
+// flag[0] of the instance's scratch region: bit j set when fullsort_alpha_kernel has to do the row for the j-th draft count.
 // 512 rows of 50257 in fp32: about 150 us (three passes with exp, 64-bit shared atomics and counts: 408).  Bound by the fp64 pipe (28
 // operations per id) and the shared atomics, not by the 206 MB it reads.
 template <typename T>
 __global__ void __launch_bounds__(kBkThreads)
-bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, int n, double temp_t, double temp_d,
+bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, const __grid_constant__ NList nl, double temp_t, double temp_d,
                     const char* __restrict__ ws, char* __restrict__ scratch, size_t scratch_stride,
                     char* __restrict__ params, int pstride, int force_sort, float* __restrict__ alpha_out,
-                    int out_stride, int out_off, int* __restrict__ status_out)
+                    int* __restrict__ status_out)
 {
     extern __shared__ __align__(16) unsigned char bk_smem[];
     pdl_wait();
@@ -158,8 +161,9 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, int
     if (tid == 0 && status_out) status_out[b] = wh->bad != 0 ? GR_BAD_LOGITS : GR_OK;
     if (wh->bad != 0 || force_sort) {
         if (tid == 0) {
-            flag[0] = 1;                            // (a bad row returns at once there too)
-            if (wh->bad != 0 && status_out) alpha_out[(size_t)b * out_stride + out_off] = nanf("");
+            flag[0] = (1 << nl.count) - 1;          // (a bad row returns at once there too)
+            if (wh->bad != 0 && status_out)
+                for (int j = 0; j < nl.count; j++) alpha_out[(size_t)b * nl.count + j] = nanf("");
         }
         return;
     }
@@ -238,20 +242,37 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, int
         sT += mT[u]; sD += mD[u];
     }
     unsigned long long totT, totD;
-    unsigned long long pT = block_exscan_u64(sT, s_w, &totT);
-    unsigned long long pD = block_exscan_u64(sD, s_w, &totD);
+    {
+        unsigned long long t = block_exscan_u64(sT, s_w, &totT), d = block_exscan_u64(sD, s_w, &totD);
+#pragma unroll
+        for (int u = 0; u < kBkPer; u++) {
+            const int c = tid * kBkPer + u;
+            tl[c] = (unsigned)t; th[c] = (unsigned)(t >> 32); dl[c] = (unsigned)d; dh[c] = (unsigned)(d >> 32);
+            t += mT[u]; d += mD[u];
+        }
+    }
     const double iT = 1.0 / (double)totT, iD = 1.0 / (double)totD;
     // tgt_i / drf_i = exp(-key_i) * rscale
     const double rscale = exp(md - mt) * ((double)totD / (double)totT);
     const double slack = (double)(V + 1) * iT + 1e-14;
+    __syncthreads();
+    int todo = 0;                                           // draft counts left to the sort
+#pragma unroll 1
+    for (int ni = 0; ni < nl.count; ni++) {
+    const int n = nl.n[ni];
     double lb[kBkPer], best = 0.0;                          // psi of the empty prefix
+    // (the masses are read back as prefixes: holding them in registers across this loop spilled, 10 % of the kernel)
+    auto prefix = [&](GR_PTR(unsigned) l, GR_PTR(unsigned) h, int c, unsigned long long total) {
+        return c < kBkBuckets ? ((unsigned long long)h[c] << 32) | l[c] : total;
+    };
+    unsigned long long qT = prefix(tl, th, tid * kBkPer, totT), qD = prefix(dl, dh, tid * kBkPer, totD);
 #pragma unroll
     for (int u = 0; u < kBkPer; u++) {
         const int c = tid * kBkPer + u;
-        tl[c] = (unsigned)pT; th[c] = (unsigned)(pT >> 32); dl[c] = (unsigned)pD; dh[c] = (unsigned)(pD >> 32);
-        const double T0 = (double)pT * iT, D0 = (double)pD * iD;
-        pT += mT[u]; pD += mD[u];
-        const double T1 = (double)pT * iT, D1 = (double)pD * iD;
+        const unsigned long long eT = prefix(tl, th, c + 1, totT), eD = prefix(dl, dh, c + 1, totD);
+        const double T0 = (double)qT * iT, D0 = (double)qD * iD, T1 = (double)eT * iT, D1 = (double)eD * iD;
+        const bool empty = eT == qT && eD == qD;
+        qT = eT; qD = eD;
         const double dn = power(D1, n);
         best = fmin(best, T1 - dn);
         // Inside the bucket every ratio tgt / drf is at least rho (its keys are at most kmax - c w; the first bucket has no
@@ -260,7 +281,7 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, int
         // covers the rounding of the masses to integers (one unit per id).
         const double khi = kmax - (invw > 0.0 ? (double)c / invw * (1.0 - 1e-12) : 0.0);
         const double rho = c == 0 ? 0.0 : exp(-khi) * rscale * (1.0 - 1e-9);
-        lb[u] = mT[u] + mD[u] == 0ull ? 1.0 : T0 + rho * (D1 - D0) - dn - slack;
+        lb[u] = empty ? 1.0 : T0 + rho * (D1 - D0) - dn - slack;
     }
     best = block_min(best, s_r);
     // ---- candidate buckets: those whose interior could hold a smaller psi
@@ -302,12 +323,9 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, int
         }
     }
     __syncthreads();
-    if (s_fallback) {
-        if (tid == 0) flag[0] = 1;
-        return;
-    }
+    const bool crowded = s_fallback != 0;
     // ---- each bucket into its own segment, ordered by (key descending, id ascending) by counting
-    if (s_nelem > 0) {
+    if (!crowded && s_nelem > 0) {
         constexpr int kOwn = kBkMaxCand / kBkThreads;
         int pos[kOwn];
 #pragma unroll
@@ -340,7 +358,7 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, int
         __syncthreads();
     }
     // ---- one warp per candidate bucket walks the prefixes
-    if (s_nelem > 0) {
+    if (!crowded && s_nelem > 0) {
         for (int c = lo + warp; c <= hi; c += kBkThreads / 32) {
             const int off = seg[c];
             if (off < 0) continue;
@@ -364,23 +382,33 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, int
         }
         best = block_min(best, s_r);
     }
-    if (tid == 0) {
-        flag[0] = 0;
+    if (crowded) todo |= 1 << ni;
+    else if (tid == 0) {
         if (hdr) { hdr->alpha_star = 1.0 + best; hdr->resid_total = -best; }
-        alpha_out[(size_t)b * out_stride + out_off] = (float)(1.0 + best);
+        alpha_out[(size_t)b * nl.count + ni] = (float)(1.0 + best);
+    }
+    if (ni + 1 < nl.count) {
+        __syncthreads();
+        for (int c = tid; c < kBkBuckets; c += kBkThreads) { cnt[c] = 0; seg[c] = -1; }
+        if (tid == 0) { s_nelem = 0; s_found = 0; s_fallback = 0; s_lo = kBkBuckets; s_hi = -1; }
+        __syncthreads();
+    }
+    }
+    if (tid == 0) {
+        flag[0] = todo;
         if (GR_CHECK_VALUE) {                       // (bounds-checked build: an access was out of range)
             if (hdr) hdr->status = GR_CHECK_FAILED;
             if (status_out) status_out[b] = GR_CHECK_FAILED;
-            alpha_out[(size_t)b * out_stride + out_off] = nanf("");
+            for (int j = 0; j < nl.count; j++) alpha_out[(size_t)b * nl.count + j] = nanf("");
         }
     }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kFsThreads)
-fullsort_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, int n, double temp_t, double temp_d,
+fullsort_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, const __grid_constant__ NList nl, double temp_t, double temp_d,
                       const char* __restrict__ ws, char* __restrict__ scratch, char* __restrict__ params, int pstride,
-                      int batch, float* __restrict__ alpha_out, int out_stride, int out_off)
+                      int batch, float* __restrict__ alpha_out)
 {
     __shared__ double s_a[kFsThreads / 32], s_b[kFsThreads / 32];
     __shared__ double s_carry[2];
@@ -489,6 +517,10 @@ fullsort_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, i
     __syncthreads();
     const double lse_t = mt + log(st0), lse_d = md + log(sd0);
     // prefix sums of tgt and drf along the order, psi_j = Tg_j - Dr_j^n, running minimum
+#pragma unroll 1
+    for (int ni = 0; ni < nl.count; ni++) {
+    if (((todo >> ni) & 1) == 0) continue;
+    const int n = nl.n[ni];
     if (tid == 0) { s_carry[0] = 0.0; s_carry[1] = 0.0; }
     __syncthreads();
     double best = 0.0;                              // psi of the empty prefix
@@ -538,16 +570,20 @@ fullsort_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, i
     if (tid == 0) {
         for (int w2 = 1; w2 < kFsThreads / 32; w2++) best = fmin(best, s_min[w2]);
         if (hdr) { hdr->alpha_star = 1.0 + best; hdr->resid_total = -best; }
-        alpha_out[(size_t)b * out_stride + out_off] = (float)(1.0 + best);
+        alpha_out[(size_t)b * nl.count + ni] = (float)(1.0 + best);
     }
     __syncthreads();
     }
+    }
 }
 
-void launch_fullsort(const void* q, const void* p, int dtype, int V, int n, double temp_t, double temp_d, int batch,
-                     const char* ws, char* scratch, char* params, int pstride, int force_sort, float* alpha_out,
-                     int out_stride, int out_off, int* status_out, cudaStream_t st)
+void launch_fullsort(const void* q, const void* p, int dtype, int V, const int* n_list, int n_count, double temp_t,
+                     double temp_d, int batch, const char* ws, char* scratch, char* params, int pstride, int force_sort, float* alpha_out,
+                     int* status_out, cudaStream_t st)
 {
+    NList nl;
+    nl.count = n_count;
+    for (int j = 0; j < n_count; j++) nl.n[j] = n_list[j];
     // function attributes belong to the device: set once per device (a failure shows up as a launch error)
     static bool configured[kMaxDevices] = {false};
     int dev = 0;
@@ -565,26 +601,18 @@ void launch_fullsort(const void* q, const void* p, int dtype, int V, int n, doub
     }
     const size_t sstride = (size_t)next_pow2(V) * 12;       // (room for V + 16 bucket numbers behind the flag: V > GR_MAX_SUPPORT)
     const int sort_grid = batch < 148 ? batch : 148;
-    if (dtype == GR_F32)
-        launch_pdl(bucket_alpha_kernel<float>, batch, kBkThreads, kBkSmemBytes, st, (const float*)q, (const float*)p, V, n, temp_t,
-                                                                            temp_d, ws, scratch, sstride, params, pstride,
-                                                                            force_sort, alpha_out, out_stride, out_off,
-                                                                            status_out);
-    else
+    if (dtype == GR_F32) {
+        launch_pdl(bucket_alpha_kernel<float>, batch, kBkThreads, kBkSmemBytes, st, (const float*)q, (const float*)p, V, nl,
+                   temp_t, temp_d, ws, scratch, sstride, params, pstride, force_sort, alpha_out, status_out);
+        launch_pdl(fullsort_alpha_kernel<float>, sort_grid, kFsThreads, kFsSmemBytes, st, (const float*)q, (const float*)p, V,
+                   nl, temp_t, temp_d, ws, scratch, params, pstride, batch, alpha_out);
+    } else {
         launch_pdl(bucket_alpha_kernel<__nv_bfloat16>, batch, kBkThreads, kBkSmemBytes, st, (const __nv_bfloat16*)q,
-                                                                                    (const __nv_bfloat16*)p, V, n, temp_t,
-                                                                                    temp_d, ws, scratch, sstride, params,
-                                                                                    pstride, force_sort, alpha_out, out_stride,
-                                                                                    out_off, status_out);
-    if (dtype == GR_F32)
-        launch_pdl(fullsort_alpha_kernel<float>, sort_grid, kFsThreads, kFsSmemBytes, st, (const float*)q, (const float*)p, V, n, temp_t,
-                                                                   temp_d, ws, scratch, params, pstride, batch, alpha_out,
-                                                                   out_stride, out_off);
-    else
+                   (const __nv_bfloat16*)p, V, nl, temp_t, temp_d, ws, scratch, sstride, params, pstride, force_sort,
+                   alpha_out, status_out);
         launch_pdl(fullsort_alpha_kernel<__nv_bfloat16>, sort_grid, kFsThreads, kFsSmemBytes, st, (const __nv_bfloat16*)q,
-                                                                           (const __nv_bfloat16*)p, V, n, temp_t,
-                                                                           temp_d, ws, scratch, params, pstride,
-                                                                           batch, alpha_out, out_stride, out_off);
+                   (const __nv_bfloat16*)p, V, nl, temp_t, temp_d, ws, scratch, params, pstride, batch, alpha_out);
+    }
 }
 
 }  // namespace gr
