@@ -82,6 +82,11 @@ __device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigne
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
 __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -246,7 +251,8 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
     if (cn > 1) cluster_barrier(); else __syncthreads();
 
     float g0 = -INFINITY;                  // running maximum of this thread's draft logits
-    unsigned long long chk = 0ull;         // plain sums (two packed): any NaN / inf makes them non-finite
+    unsigned long long chk = 0ull;         // sums of 0 * logit (two packed): zero until a NaN or an infinity makes them NaN,
+                                           // whatever the size of the finite ones (masks down to the type's lowest value)
     const float sc_t = A.sc_t;
     const unsigned long long sc2 = f_pack(sc_t, sc_t);
     float kmax = -INFINITY, kmin = INFINITY;                // range of the log-ratios draft / target (kFull)
@@ -288,7 +294,7 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
                     const float mn = fmaxf(cm, x);
                     cs = fmaf(cs, ex2((cm - mn) * sc_t), ex2((x - mn) * sc_t));
                     cm = mn;
-                    chk = add2(chk, f_pack(x, v));
+                    chk = fma2(f_pack(x, v), 0ull, chk);
                     g0 = fmaxf(g0, v);
                     if (kFull) ratio_range(f_pack(x, x), f_pack(v, v));
                     if (!kFull) push_candidate(sh, v, i, tau);
@@ -306,7 +312,7 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
                         for (int i = 0; i < VT::kPairs; i++) {
                             x[i] = VT::pair(qv[u], i);
                             vm = fmaxf(vm, fmaxf(f_lo(x[i]), f_hi(x[i])));
-                            chk = add2(chk, x[i]);
+                            chk = fma2(x[i], 0ull, chk);
                         }
                         const float mn = fmaxf(cm, vm);
                         // (a factor of exactly one where the maximum stands)
@@ -331,7 +337,7 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
                         for (int i = 0; i < VT::kPairs; i++) {
                             const unsigned long long x = VT::pair(pv[u], i);
                             vm = fmaxf(vm, fmaxf(f_lo(x), f_hi(x)));
-                            chk = add2(chk, x);
+                            chk = fma2(x, 0ull, chk);
                         }
                         g0 = fmaxf(g0, vm);
                         if (kFull) {
@@ -386,7 +392,7 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
     }
     // non-finite inputs
     {
-        const bool badl = !(fabsf(f_lo(chk)) <= 3.0e38f) || !(fabsf(f_hi(chk)) <= 3.0e38f);
+        const bool badl = !(f_lo(chk) == 0.f) || !(f_hi(chk) == 0.f);
         if (__any_sync(0xffffffffu, badl) && lane == 0) atomicOr(&sh.bad, 1);
     }
     // ---- candidates: a last threshold from the whole part, then composite keys of those that pass it

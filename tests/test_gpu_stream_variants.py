@@ -32,3 +32,33 @@ def test_support_and_log_sum_exp(V, batch):
         lse = torch.logsumexp(q.double() / 0.75, 1).cpu()
         assert float((lse - r.lse_target).abs().max()) < 1e-6, (dt, k)
         assert int((s.status > 1).sum()) == 0        # (1: a solve that did not converge, which is not this pass)
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("V,k", [(1500, 20), (40000, 50), (100, 0), (3001, 0), (50257, 0)])
+def test_masks_are_logits_and_only_nan_and_infinity_are_not(V, k, dt):
+    """Any finite value is a logit: ids masked with values down to the type's lowest, many at a time and in both rows, leave
+    the other ids' results as any other mask does.  One NaN or infinity in either row is reported."""
+    g = torch.Generator(device="cuda").manual_seed(V)
+    q = (2 * torch.randn(3, V, generator=g, device="cuda")).to(dt)
+    p = (q.float() + torch.randn(3, V, generator=g, device="cuda")).to(dt)
+    idx = torch.randperm(V, generator=g, device="cuda")[: V // 3]
+    want = None
+    for value in (-1.0e4, -1.0e30, -1.7e38, torch.finfo(dt).min):
+        qm, pm = q.clone(), p.clone()
+        qm[:, idx] = value
+        pm[:, idx] = value
+        s = G.solve(qm, pm, 3, k, 0.75, 0.75)
+        a, st = G.alpha_star(qm, pm, [3], k, 0.75, 0.75)
+        assert int(st.max()) == 0 and int((s.status == G.GR_BAD_LOGITS).sum()) == 0, value
+        got = (s.alpha_star.clone(), a[:, 0], G.read_rule(s).lse_target)
+        want = want or got
+        assert torch.equal(got[2], want[2]), value
+        assert all(float((x - y).abs().max()) < 1e-6 for x, y in zip(got[:2], want[:2])), (value, got, want)
+    for value in (float("nan"), float("inf"), float("-inf")):
+        for row in (q, p):
+            for at in (0, V // 2, V - 1):
+                bad = row.clone()
+                bad[1, at] = value
+                s = G.solve(bad if row is q else q, bad if row is p else p, 3, k, 0.75, 0.75)
+                assert [x == G.GR_BAD_LOGITS for x in s.status.tolist()] == [False, True, False], (value, at)
