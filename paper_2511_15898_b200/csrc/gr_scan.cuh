@@ -256,10 +256,14 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
     const float sc_t = A.sc_t;
     const unsigned long long sc2 = f_pack(sc_t, sc_t);
     float kmax = -INFINITY, kmin = INFINITY;                // range of the log-ratios draft / target (kFull)
+    // (with the rounding error of the target's product added back: ids masked by one huge value in both rows at one
+    // temperature get the key 0, and not a rounding error as large as the range of all the others; a key that overflows is
+    // left out, its id belongs to the first or the last bucket in any case)
     auto ratio_range = [&](unsigned long long x, unsigned long long v) {
-        const unsigned long long m = mul2(x, f_pack(-sc_t, -sc_t));
-        const float k0 = fmaf(f_lo(v), A.sc_d, f_lo(m)), k1 = fmaf(f_hi(v), A.sc_d, f_hi(m));
-        kmax = fmaxf(kmax, fmaxf(k0, k1)); kmin = fminf(kmin, fminf(k0, k1));
+        const unsigned long long down = f_pack(-sc_t, -sc_t), m = mul2(x, down);
+        const unsigned long long err = fma2(x, down, m ^ 0x8000000080000000ull);
+        const unsigned long long key = add2(fma2(v, f_pack(A.sc_d, A.sc_d), m), err);
+        kmax = fmaxf(kmax, fmaxf(f_lo(key), f_hi(key))); kmin = fminf(kmin, fminf(f_lo(key), f_hi(key)));
     };
     const int rounds = (nch + stride - 1) / stride;
     const int vec_end = head + ((V - head) / N) * N, tail = V - vec_end;

@@ -38,3 +38,24 @@ def test_alpha_star_of_whole_rows(V, dt):
     assert st.tolist() == [0] * 6
     for j, n in enumerate(ns):
         assert float((out[:, j].double() - _alpha(q, p, n, 0.75, 1.25)).abs().max()) < 1e-6, n
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("V", [50257, 152064])
+@pytest.mark.parametrize("value", [-1.0e9, -1.0e10, -1.0e30, -3.3e38])
+def test_masked_ids_do_not_send_the_row_to_the_sort(V, dt, value):
+    """Ids masked by one value in both rows at one temperature have the key 0: the range of the keys stays that of the other
+    ids, however large the value (its rounding error is not), and the bucket search separates the row.  The first word of the
+    row's scratch, behind the workspace's records, says what was left to the sort."""
+    g = torch.Generator(device="cuda").manual_seed(V)
+    q = (3 * torch.randn(2, V, generator=g, device="cuda")).to(dt)
+    p = (q.float() + torch.randn(2, V, generator=g, device="cuda")).to(dt)
+    q[:, V - 100:] = value
+    p[:, V - 100:] = value
+    q[:, 5] = value
+    p[:, 5] = value
+    s = G.solve(q, p, 8, 0, 1.0, 1.0)
+    words = s.workspace.view(torch.int32)
+    record, row = (32 + 128 * 12) // 4, 3 * (1 << (V - 1).bit_length())      # bytes / 4: one record, one row of the scratch
+    assert [int(words[2 * record + b * row]) for b in range(2)] == [0, 0]
+    assert float((s.alpha_star.double() - _alpha(q, p, 8, 1.0, 1.0)).abs().max()) < 1e-6
