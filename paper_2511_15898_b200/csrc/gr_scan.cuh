@@ -409,16 +409,22 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
         if (sh.cnt > SS::kCap) exact_select_slow<T>(sh, prow, V, head, nch, first, stride, nsel);
         M = min(sh.cnt, SS::kCap);
         constexpr int kPer = SS::kCap / SS::kThr;
-        const float tau = use_tau ? sh.tau : -INFINITY;
+        float vv[kPer], own = -INFINITY;
+#pragma unroll
+        for (int u = 0; u < kPer; u++) {
+            const int e = tid + u * SS::kThr;
+            vv[u] = e < M ? reinterpret_cast<const float*>(sh.keys)[e] : -INFINITY;
+            own = fmaxf(own, vv[u]);
+        }
+        // (a short row is in the list as a whole, and the threads' shares of the list are the groups: ranking 1500 elements
+        // among themselves took 60 us)
+        if (take_all && M > kRankAll) refine_tau(sh, own, nsel);
+        const float tau = sh.tau;
         unsigned long long kk[kPer];
 #pragma unroll
         for (int u = 0; u < kPer; u++) {
             const int e = tid + u * SS::kThr;
-            kk[u] = 0ull;
-            if (e < M) {
-                const float v = reinterpret_cast<const float*>(sh.keys)[e];
-                if (v >= tau) kk[u] = ckey(v, reinterpret_cast<const int*>(sh.keys)[SS::kCap + e]);
-            }
+            kk[u] = e < M && vv[u] >= tau ? ckey(vv[u], reinterpret_cast<const int*>(sh.keys)[SS::kCap + e]) : 0ull;
         }
         if (tid == 0) sh.kept = 0;
         __syncthreads();

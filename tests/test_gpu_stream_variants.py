@@ -62,3 +62,35 @@ def test_masks_are_logits_and_only_nan_and_infinity_are_not(V, k, dt):
                 bad[1, at] = value
                 s = G.solve(bad if row is q else q, bad if row is p else p, 3, k, 0.75, 0.75)
                 assert [x == G.GR_BAD_LOGITS for x in s.status.tolist()] == [False, True, False], (value, at)
+
+
+def _median_us(call):
+    for _ in range(3):
+        call()
+    ts = []
+    for _ in range(21):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        call()
+        b.record()
+        b.synchronize()
+        ts.append(a.elapsed_time(b) * 1e3)
+    return sorted(ts)[len(ts) // 2]
+
+
+@pytest.mark.parametrize("V", [129, 600, 1025, 2047, 2048])
+def test_rows_that_are_candidates_as_a_whole(V):
+    """Rows of up to 2048 ids go into the candidate list as a whole; the list is cut before it is ranked (many ties among
+    them), and a row of 2048 ids takes no longer than one of 2049, which has a threshold from the start."""
+    g = torch.Generator(device="cuda").manual_seed(V)
+    for k in (1, 8, 127, 128):
+        for levels in (3, 40, 100000):
+            p = torch.randint(0, levels, (5, V), generator=g, device="cuda").float() / 7 - 3
+            q = torch.randn(5, V, generator=g, device="cuda")
+            r = G.read_rule(G.solve(q, p, 1, k, 1.0, 1.0))
+            want = torch.sort(p, dim=1, descending=True, stable=True).indices[:, :k]
+            assert torch.equal(torch.sort(want, dim=1).values.int().cpu(), torch.sort(r.ids[:, :k], dim=1).values), (k, levels)
+    if V == 2048:
+        x = torch.randn(300, 2 * V, generator=g, device="cuda")
+        us = [_median_us(lambda a=x[:, :n].contiguous(): G.alpha_star(a, a, [2], 8, 1.0, 0.9)) for n in (V, V + 1)]
+        assert us[0] < 1.25 * us[1], us
