@@ -16,7 +16,6 @@ alpha_kernel(const char* __restrict__ ws, int V, int topk, double temp_t, double
     __shared__ int s_id[kMaxSupport];
     __shared__ double s_red[32];
     pdl_wait();
-    pdl_trigger();
     const int tid = threadIdx.x;
     const long long b = blockIdx.x;
     const WsView wv = view_ws(ws, b);

@@ -1501,7 +1501,6 @@ fast_solve_kernel(const char* __restrict__ ws, char* __restrict__ params, int ps
 {
     __shared__ int s_sel;
     pdl_wait();
-    pdl_trigger();
     GR_CHECK_FLAG_DECL;
     GR_CHECK_FLAG_INIT;
     const bool fused = fa.draft != nullptr;

@@ -128,7 +128,6 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
 {
     extern __shared__ __align__(16) unsigned char bk_smem[];
     pdl_wait();
-    pdl_trigger();
     GR_CHECK_FLAG_DECL;
     GR_CHECK_FLAG_INIT;
     double* const ckey_raw = reinterpret_cast<double*>(bk_smem);
@@ -414,7 +413,6 @@ fullsort_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, c
     __shared__ double s_carry[2];
     __shared__ double s_min[kFsThreads / 32];
     pdl_wait();
-    pdl_trigger();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // (normally no row is left to it: a grid of one wave looks)
 #pragma unroll 1

@@ -14,7 +14,6 @@ scan_kernel(const __grid_constant__ ScanArgs A, int cn)
 {
     __shared__ ScanSm sh;
     pdl_wait();
-    pdl_trigger();
     GR_CHECK_FLAG_DECL;
     GR_CHECK_FLAG_INIT;
     scan_row<T, kFull, kInFlight>(A, sh, (long long)(blockIdx.x / cn), (int)(blockIdx.x % cn), cn, GR_CHECK_FLAG);

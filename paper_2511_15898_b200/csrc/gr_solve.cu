@@ -719,7 +719,6 @@ solve_kernel(const char* __restrict__ ws, char* __restrict__ params, int pstride
 {
     __shared__ int s_list[kSolveThreads], s_count;
     pdl_wait();
-    pdl_trigger();
     if (!only_flagged) {
         solve_instance(blockIdx.x, ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol, max_iters, qstep, tau, Qt, 0,
                        alpha_out, status_out, fa);

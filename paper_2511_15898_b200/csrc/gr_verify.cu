@@ -20,7 +20,6 @@ verify_kernel(const char* __restrict__ params, const int* __restrict__ draft, co
 {
     __shared__ double s_scratch[kVerifyScratchBytes / 8];
     pdl_wait();
-    pdl_trigger();
     GR_CHECK_FLAG_DECL;
     GR_CHECK_FLAG_INIT;
     const long long b = blockIdx.x;
