@@ -155,7 +155,8 @@ __device__ __forceinline__ void push_candidate(SS& sh, float val, int id, float 
 template <typename T, class SS>
 __device__ __noinline__ void exact_select_slow(SS& sh, const T* prow, int V, int head, int nch, int first, int stride, int ksel)
 {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int kAhead = 8;                // loads in flight per thread
+    const int tid = threadIdx.x;
     if (tid == 0) { sh.prefix = 0ull; sh.need = ksel; }
     __syncthreads();
 #pragma unroll 1
@@ -166,15 +167,23 @@ __device__ __noinline__ void exact_select_slow(SS& sh, const T* prow, int V, int
         if (pass == 8 && tid == 0) sh.cnt = 0;
         __syncthreads();
         const unsigned long long prefix = sh.prefix;
-        for (int c = first + warp; c < nch; c += stride) {
-            const int e1 = chunk_end(c, head, nch, V);
-            for (int i = chunk_begin(c, head) + lane; i < e1; i += 32) {
-                const float v = load_logit<T>(prow, i);
-                const unsigned long long key = ckey(v, i);
-                if (pass == 8) {
-                    if (key >= prefix) push_candidate(sh, v, i, -INFINITY);
-                } else if (pass == 0 || (key >> (shift + 8)) == (prefix >> (shift + 8))) {
-                    atomicAdd(&sh.hist[(int)((key >> shift) & 255ull)], 1);
+        // (a round's chunks are neighbours; all threads take part, also where the row has fewer chunks than the CTA warps)
+        for (int c = first; c < nch; c += stride) {
+            const int e1 = chunk_end(min(c + SS::kThr / 32, nch) - 1, head, nch, V);
+            for (int i0 = chunk_begin(c, head) + tid; i0 < e1; i0 += kAhead * SS::kThr) {
+                float v[kAhead];
+#pragma unroll
+                for (int u = 0; u < kAhead; u++) v[u] = i0 + u * SS::kThr < e1 ? load_logit<T>(prow, i0 + u * SS::kThr) : 0.f;
+#pragma unroll
+                for (int u = 0; u < kAhead; u++) {
+                    const int i = i0 + u * SS::kThr;
+                    if (i >= e1) break;
+                    const unsigned long long key = ckey(v[u], i);
+                    if (pass == 8) {
+                        if (key >= prefix) push_candidate(sh, v[u], i, -INFINITY);
+                    } else if (pass == 0 || (key >> (shift + 8)) == (prefix >> (shift + 8))) {
+                        atomicAdd(&sh.hist[(int)((key >> shift) & 255ull)], 1);
+                    }
                 }
             }
         }
