@@ -24,7 +24,8 @@ namespace gr {
 
 constexpr int kMaxChunks = 2049;     // V <= 2^21
 constexpr int kMaxCluster = 8;
-constexpr int kRankAll = 128;        // candidates that are ranked as they are; more go through a last threshold first
+constexpr int kRankAll = 256;        // candidates that are ranked as they are; more go through a last threshold first (1 us;
+                                     // at 128 it cost more than it saved: 1000 bf16 rows of 16000, k = 128, 75 us for 69)
 
 // Arguments common to every row.
 struct ScanArgs {
@@ -408,10 +409,9 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
         const bool badl = !(f_lo(chk) == 0.f) || !(f_hi(chk) == 0.f);
         if (__any_sync(0xffffffffu, badl) && lane == 0) atomicOr(&sh.bad, 1);
     }
-    // ---- candidates: a last threshold from the whole part, then composite keys of those that pass it
+    // ---- candidates: a last threshold from the list itself, then composite keys of those that pass it
     __syncthreads();
     if (cn == 1) lse_terms(sh, nch, A.temp_t);
-    if (use_tau && sh.cnt > kRankAll) refine_tau(sh, g0, ksel);
     int M = 0, nsel = 0;
     if (!kFull) {
         nsel = ksel < V ? ksel : V;
@@ -425,9 +425,9 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
             vv[u] = e < M ? reinterpret_cast<const float*>(sh.keys)[e] : -INFINITY;
             own = fmaxf(own, vv[u]);
         }
-        // (a short row is in the list as a whole, and the threads' shares of the list are the groups: ranking 1500 elements
-        // among themselves took 60 us)
-        if (take_all && M > kRankAll) refine_tau(sh, own, nsel);
+        // (the threads' shares of the list are the groups: in a short row the threads' maxima are too few to tell anything, and
+        // ranking 1500 elements among themselves took 60 us)
+        if (M > kRankAll) refine_tau(sh, own, nsel);
         const float tau = sh.tau;
         unsigned long long kk[kPer];
 #pragma unroll

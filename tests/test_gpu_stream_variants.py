@@ -78,10 +78,11 @@ def _median_us(call):
     return sorted(ts)[len(ts) // 2]
 
 
-@pytest.mark.parametrize("V", [129, 600, 1025, 2047, 2048])
-def test_rows_that_are_candidates_as_a_whole(V):
-    """Rows of up to 2048 ids go into the candidate list as a whole; the list is cut before it is ranked (many ties among
-    them), and a row of 2048 ids takes no longer than one of 2049, which has a threshold from the start."""
+@pytest.mark.parametrize("V", [129, 600, 1025, 2047, 2048, 2100, 3500, 4100])
+def test_rows_with_long_candidate_lists(V):
+    """Rows of up to 2048 ids go into the candidate list as a whole, and rows of a few chunks have a threshold too low to
+    keep much out; the list is cut before it is ranked (many ties among them).  A row of 2048 ids takes no longer than one
+    of 2049, which has a threshold from the start."""
     g = torch.Generator(device="cuda").manual_seed(V)
     for k in (1, 8, 127, 128):
         for levels in (3, 40, 100000):
