@@ -5,7 +5,7 @@
 namespace gr {
 // The fast kernel covers supports up to 128 tokens with n <= 16; everything else, and any instance the fast
 // kernel could not finish, takes the robust kernel.
-int launch_solve_any(const char* ws, char* params, int pstride, int kcap, int V, int n, int topk, double temp_t,
+int launch_solve_any(char* ws, char* params, int pstride, int kcap, int V, int n, int topk, double temp_t,
                      double temp_d, double tol, int max_iters, double qstep, double tau, int batch, int force_robust,
                      float* alpha_out, int* status_out, FusedArgs fa, cudaStream_t st)
 {
@@ -95,7 +95,7 @@ static int solve_impl(const void* q_logits, const void* p_logits, int dtype, int
     if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return GR_E_LAUNCH; }
     if (scan_done && cudaEventRecord(scan_done, st) != cudaSuccess) { cudaGetLastError(); return GR_E_LAUNCH; }
     gr::NvtxRange r(fa.draft ? "gr:solve+draw" : "gr:solve");
-    int rc = gr::launch_solve_any((const char*)workspace, (char*)params, pstride, kcap, V, n, topk,
+    int rc = gr::launch_solve_any((char*)workspace, (char*)params, pstride, kcap, V, n, topk,
                                   (double)temp_target, (double)temp_draft, tol, max_iters, qstep, tau, batch,
                                   force_robust, alpha_star, status, fa, st);
     if (rc != GR_OK) return rc;

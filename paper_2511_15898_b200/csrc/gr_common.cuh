@@ -156,11 +156,12 @@ __host__ __device__ inline ParamView view_params(void* base, int kcap, int V = 1
 // Workspace of one instance (written by the scan kernel, read by the solve kernel).
 struct __align__(16) WsHeader {
     double lse_t;        // log sum exp of target logits / temp_target
-    double lse_d;        // (unused)
+    int flagged, taken;  // record 0 only: instances the fast kernel left to the general one, and how many of them that one
+                         // has begun (the streaming pass clears both)
     int count;           // entries that follow (the support, k of them)
     int bad;             // 1 when a non-finite logit was met
     int check;           // bounds-checked build: the streaming kernel skipped an out-of-range access on this row
-    int pad;
+    int flagged_id;      // record i: the i-th instance left to the general kernel
 };
 // then: int id[kMaxSupport]; float dl[kMaxSupport]; float tl[kMaxSupport];
 // Of a whole-vocabulary row the streaming pass keeps, where the support would be: the draft row's maximum and the range of
@@ -271,6 +272,7 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), int grid, int block, int sme
     return launch_pdl_cluster<P...>(1, kernel, grid, block, smem, st, static_cast<P>(args)...);
 }
 
+constexpr int kSms = 148;                     // SMs of the chip: size of the grids that look for work
 constexpr int kMaxDevices = 64;               // per-device caches of the host code (function attributes, streams)
 
 }  // namespace gr

@@ -4,7 +4,7 @@
 namespace gr {
 
 #define GR_FAST_ARGS                                                                                              \
-    const char *ws, char *params, int pstride, int kcap, int V, int n, int topk, double temp_t, double temp_d,   \
+    char *ws, char *params, int pstride, int kcap, int V, int n, int topk, double temp_t, double temp_d,   \
         double tol, int max_iters, double qstep, double tau, int batch, float *alpha_out, int *status_out,       \
         FusedArgs fa, cudaStream_t st
 namespace fast {

@@ -1494,7 +1494,7 @@ __device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, c
 
 template <class C>
 __global__ void __launch_bounds__(C::T, C::kCtas)
-fast_solve_kernel(const char* __restrict__ ws, char* __restrict__ params, int pstride, int kcap, int V, int n, int topk,
+fast_solve_kernel(char* __restrict__ ws, char* __restrict__ params, int pstride, int kcap, int V, int n, int topk,
                   double temp_t, double temp_d, double tol, int max_iters, double qstep, double tau, double sigma,
                   float* __restrict__ alpha_out, int* __restrict__ status_out, FusedArgs fa,
                   const __grid_constant__ typename CircleOf<C::kContour>::type circle)
@@ -1607,6 +1607,10 @@ fast_solve_kernel(const char* __restrict__ ws, char* __restrict__ params, int ps
     }
     if (status == GR_OK && skipped) status = GR_PARTIAL_RULE;
     write_rule_header(pv, pr, n, status, gnorm_total, iters_total, alpha_out, status_out, b, GR_CHECK_FLAG, wv.h->check);
+    if (status == kNeedFallback && tid == 0) {
+        const int i = atomicAdd(&reinterpret_cast<WsHeader*>(ws)->flagged, 1);
+        reinterpret_cast<WsHeader*>(ws + (size_t)i * ws_stride())->flagged_id = (int)b;
+    }
     if (fused && status != kNeedFallback) {
         __syncthreads();                       // the rule this CTA wrote is visible to its first warp
         fused_draw(fa, pv.h, b, n, smem_raw + C::oU, GR_CHECK_FLAG);
@@ -1614,7 +1618,7 @@ fast_solve_kernel(const char* __restrict__ ws, char* __restrict__ params, int ps
 }
 
 template <class C>
-int launch_fast_t(const char* ws, char* params, int pstride, int kcap, int V, int n, int topk, double temp_t,
+int launch_fast_t(char* ws, char* params, int pstride, int kcap, int V, int n, int topk, double temp_t,
                   double temp_d, double tol, int max_iters, double qstep, double tau, int batch, float* alpha_out,
                   int* status_out, FusedArgs fa, cudaStream_t st)
 {
@@ -1652,7 +1656,7 @@ int launch_fast_t(const char* ws, char* params, int pstride, int kcap, int V, in
 
 // One translation unit per series length instantiates its kernels (they compile in parallel).
 #define GR_FAST_ARGS                                                                                              \
-    const char *ws, char *params, int pstride, int kcap, int V, int n, int topk, double temp_t, double temp_d,   \
+    char *ws, char *params, int pstride, int kcap, int V, int n, int topk, double temp_t, double temp_d,   \
         double tol, int max_iters, double qstep, double tau, int batch, float *alpha_out, int *status_out,       \
         FusedArgs fa, cudaStream_t st
 #define GR_FAST_PASS ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol, max_iters, qstep, tau, batch, alpha_out, status_out, fa, st

@@ -598,7 +598,7 @@ void launch_fullsort(const void* q, const void* p, int dtype, int V, const int* 
         if (dev >= 0 && ok) configured[dev] = true;
     }
     const size_t sstride = (size_t)next_pow2(V) * 12;       // (room for V + 16 bucket numbers behind the flag: V > GR_MAX_SUPPORT)
-    const int sort_grid = batch < 148 ? batch : 148;
+    const int sort_grid = batch < kSms ? batch : kSms;
     if (dtype == GR_F32) {
         launch_pdl(bucket_alpha_kernel<float>, batch, kBkThreads, kBkSmemBytes, st, (const float*)q, (const float*)p, V, nl,
                    temp_t, temp_d, ws, scratch, sstride, params, pstride, force_sort, alpha_out, status_out);

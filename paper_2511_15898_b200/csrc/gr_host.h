@@ -17,13 +17,13 @@ struct NvtxRange {
 
 void launch_scan(const void* q, const void* p, int dtype, int V, int ksel, bool full_large, double temp_t,
                  double temp_d, int batch, char* ws, char* params, int pstride, int kcap, cudaStream_t st);
-int launch_solve(const char* ws, char* params, int pstride, int kcap, int V, int n, int topk, double temp_t,
+int launch_solve(char* ws, char* params, int pstride, int kcap, int V, int n, int topk, double temp_t,
                  double temp_d, double tol, int max_iters, double qstep, double tau, int batch, int only_flagged,
                  float* alpha_out, int* status_out, FusedArgs fa, cudaStream_t st);
-int launch_fast(const char* ws, char* params, int pstride, int kcap, int V, int n, int topk, double temp_t,
+int launch_fast(char* ws, char* params, int pstride, int kcap, int V, int n, int topk, double temp_t,
                 double temp_d, double tol, int max_iters, double qstep, double tau, int batch, float* alpha_out,
                 int* status_out, FusedArgs fa, cudaStream_t st);
-int launch_solve_any(const char* ws, char* params, int pstride, int kcap, int V, int n, int topk, double temp_t,
+int launch_solve_any(char* ws, char* params, int pstride, int kcap, int V, int n, int topk, double temp_t,
                      double temp_d, double tol, int max_iters, double qstep, double tau, int batch, int force_robust,
                      float* alpha_out, int* status_out, FusedArgs fa, cudaStream_t st);
 size_t fullsort_scratch_bytes(int V);

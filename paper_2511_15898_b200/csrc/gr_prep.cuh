@@ -8,8 +8,9 @@ namespace gr {
 
 constexpr int kNeedFallback = 100;   // internal status: the fast kernel asks the robust kernel to redo the instance
 
-// CTA-wide reductions; `scratch` needs one double per warp.  Every thread gets the result.
-static __device__ __noinline__ double block_reduce_max(double v, GR_PTR(double) scratch) {
+// CTA-wide reductions; `scratch` needs one double per warp.  Every thread gets the result.  (Out of line where they are used
+// once per instance; the general kernel's iteration takes the inline forms.)
+__device__ __forceinline__ double reduce_max(double v, GR_PTR(double) scratch) {
 #pragma unroll 1
     for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
     const int nw = blockDim.x >> 5;
@@ -21,7 +22,7 @@ static __device__ __noinline__ double block_reduce_max(double v, GR_PTR(double) 
     for (int i = 1; i < nw; i++) r = fmax(r, scratch[i]);
     return r;
 }
-static __device__ __noinline__ double block_reduce_sum(double v, GR_PTR(double) scratch) {
+__device__ __forceinline__ double reduce_sum(double v, GR_PTR(double) scratch) {
 #pragma unroll 1
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     const int nw = blockDim.x >> 5;
@@ -33,6 +34,8 @@ static __device__ __noinline__ double block_reduce_sum(double v, GR_PTR(double) 
     for (int i = 0; i < nw; i++) r += scratch[i];
     return r;
 }
+static __device__ __noinline__ double block_reduce_max(double v, GR_PTR(double) scratch) { return reduce_max(v, scratch); }
+static __device__ __noinline__ double block_reduce_sum(double v, GR_PTR(double) scratch) { return reduce_sum(v, scratch); }
 
 // shared-memory arrays of the preparation (KP entries each; psi and Dr: KP + 4)
 struct PrepSm {

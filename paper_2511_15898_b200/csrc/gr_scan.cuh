@@ -548,7 +548,7 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
     if (tid == 0) {
         WsHeader* wh = reinterpret_cast<WsHeader*>(wsb);
         wh->lse_t = sh.lse[0];
-        wh->lse_d = 0.0;
+        wh->flagged = 0; wh->taken = 0;
         wh->count = nsel;
         wh->bad = sh.bad;
         wh->check = check ? *check : 0;

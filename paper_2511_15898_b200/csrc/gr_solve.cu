@@ -28,7 +28,7 @@ constexpr double kTEnd = 25.0;      // integrand below exp(-kTEnd) at the upper 
 constexpr double kDrop = 1.0;       // the lower-tail compression starts this far below the fastest transition
 constexpr double kTail = 3.0;       // and the grid extends this far below that
 constexpr int kMaxNodes = 512;
-constexpr int kFlaggedGrid = 148;  // CTAs of the pass that looks for flagged instances: one per SM
+constexpr int kFlaggedGrid = 2 * kSms;  // CTAs of the pass over the flagged instances: what the SMs hold
 constexpr double kAlphaClamp = 80.0;
 constexpr double kStepClamp = 3.0;
 
@@ -95,8 +95,8 @@ __device__ int eval_system(const Sm& sm, int m, GR_PTR(const double) d, double h
     // weights and their range
     double wj = 0.0;
     if (tid < m) { wj = exp(sm.alpha[tid]); sm.w[tid] = wj; sm.g[tid] = 0.0; sm.g2[tid] = 0.0; }
-    double wmax = block_reduce_max(tid < m ? wj : 0.0, red);
-    double wmin = -block_reduce_max(tid < m ? -wj : -1.0e300, red);
+    double wmax = reduce_max(tid < m ? wj : 0.0, red);
+    double wmin = -reduce_max(tid < m ? -wj : -1.0e300, red);
     if (want_jac)
         for (int e = tid; e < m * (m + 1) / 2; e += kSolveThreads) sm.J[e] = 0.0;
     const double rate = slack ? 1.0 + wmin : wmin;
@@ -438,7 +438,7 @@ __device__ int solve_system(const Sm& sm, int m, GR_PTR(const double) d, GR_PTR(
     // starting point: the single-token balance  w/(1+w) * Pr[i in set(omega)] = rhs
     double a0 = 0.0;
     bool warm_used = false;
-    const double D = block_reduce_sum(tid < m ? d[tid] : 0.0, red);   // draft mass of the system
+    const double D = reduce_sum(tid < m ? d[tid] : 0.0, red);   // draft mass of the system
     if (tid < m) {
         if (slack) {
             // Pr[i drafted and every draft inside the system] = D^n - (D - d_i)^n
@@ -458,7 +458,7 @@ __device__ int solve_system(const Sm& sm, int m, GR_PTR(const double) d, GR_PTR(
         warm_used = !bad && moved;
     }
     if (!slack) {
-        double mean = block_reduce_sum(tid < m ? a0 : 0.0, red) / (double)m;
+        double mean = reduce_sum(tid < m ? a0 : 0.0, red) / (double)m;
         a0 -= mean;
     }
     if (tid < m) sm.alpha[tid] = fmin(fmax(a0, -kAlphaClamp), kAlphaClamp);
@@ -477,7 +477,7 @@ __device__ int solve_system(const Sm& sm, int m, GR_PTR(const double) d, GR_PTR(
         const bool comparable = coarse == (sm.scal[S_COARSE] != 0.0);
         __syncthreads();
         eval_system(sm, m, d, hmass, slack, true, coarse ? 2.0 * qstep : qstep);
-        rn = block_reduce_sum(tid < m ? fabs(sm.g[tid] - rhs[tid]) : 0.0, red);
+        rn = reduce_sum(tid < m ? fabs(sm.g[tid] - rhs[tid]) : 0.0, red);
         if (rn <= tol && !coarse) { status = GR_OK; it++; break; }
         const double rprev = sm.scal[S_RPREV];
         const double lam = sm.scal[S_LAM];
@@ -523,7 +523,7 @@ __device__ int solve_system(const Sm& sm, int m, GR_PTR(const double) d, GR_PTR(
             __syncthreads();
         }
         // (a component that is not a number counts as infinite: fmax would drop it)
-        double dm = block_reduce_max(tid < m ? (sm.delta[tid] == sm.delta[tid] ? fabs(sm.delta[tid]) : 1.0e300) : 0.0, red);
+        double dm = reduce_max(tid < m ? (sm.delta[tid] == sm.delta[tid] ? fabs(sm.delta[tid]) : 1.0e300) : 0.0, red);
         if (!(dm < 1.0e300)) dm = 1.0e300;
         // a full Newton step below 1e-11 in alpha: the weights cannot be improved at this quadrature accuracy
         if (!fail && dm < 1.0e-11) { status = GR_OK; it++; break; }
@@ -535,7 +535,7 @@ __device__ int solve_system(const Sm& sm, int m, GR_PTR(const double) d, GR_PTR(
         }
         __syncthreads();
         double mean = 0.0;
-        if (!slack) mean = block_reduce_sum(tid < m ? sm.delta[tid] : 0.0, red) / (double)m;
+        if (!slack) mean = reduce_sum(tid < m ? sm.delta[tid] : 0.0, red) / (double)m;
         if (tid < m) {
             sm.delta[tid] -= mean;
             double a = sm.alpha[tid] + sm.delta[tid];
@@ -546,7 +546,7 @@ __device__ int solve_system(const Sm& sm, int m, GR_PTR(const double) d, GR_PTR(
         // evaluated on the full grid leaves a residual of at most a small multiple of it (within 3.1 times, plus the
         // quadrature floor, on every benchmark shape).  Ten times below the tolerance: the step is taken and the
         // iteration stops without another evaluation; the reported norm is then the bound 3 s2.
-        const double s2 = block_reduce_sum(tid < m ? sm.g[tid] * sm.delta[tid] * sm.delta[tid] : 0.0, red);
+        const double s2 = reduce_sum(tid < m ? sm.g[tid] * sm.delta[tid] * sm.delta[tid] : 0.0, red);
         // (not after a factorisation that cancelled all but a few percent of a diagonal entry: see the fast kernel)
         if (!fail && !coarse && dm <= 1.0 && 10.0 * s2 < tol && sm.scal[S_PIVOT] > 0.02) {
             if (tid < m) sm.w[tid] = exp(sm.alpha[tid]);
@@ -562,8 +562,9 @@ __device__ int solve_system(const Sm& sm, int m, GR_PTR(const double) d, GR_PTR(
     return status;
 }
 
-// One instance, by the whole CTA.
-__device__ void solve_instance(long long b, const char* __restrict__ ws, char* __restrict__ params, int pstride, int kcap, int V, int n, int topk,
+// One instance, by the whole CTA.  Out of line, for the two kernels below: in a loop, or with two calls in one kernel, it
+// was inlined with up to twice the spills, 4 to 9 % of its time.
+__device__ __noinline__ void solve_instance(long long b, const char* __restrict__ ws, char* __restrict__ params, int pstride, int kcap, int V, int n, int topk,
              double temp_t, double temp_d, double tol, int max_iters, double qstep, double tau, int Qt, int only_flagged,
              float* __restrict__ alpha_out, int* __restrict__ status_out, FusedArgs fa)
 {
@@ -710,40 +711,43 @@ __device__ void solve_instance(long long b, const char* __restrict__ ws, char* _
     }
 }
 
-// only_flagged: the second pass after the fast kernel, which redoes the instances that one gave up (normally none).  A grid
-// of one wave looks them up, one instance per thread, and does those it finds one after the other.
+// Every instance of the batch, one per CTA.
 __global__ void __launch_bounds__(kSolveThreads)
-solve_kernel(const char* __restrict__ ws, char* __restrict__ params, int pstride, int kcap, int V, int n, int topk,
-             double temp_t, double temp_d, double tol, int max_iters, double qstep, double tau, int Qt, int only_flagged,
-             int batch, float* __restrict__ alpha_out, int* __restrict__ status_out, FusedArgs fa)
+solve_kernel(char* __restrict__ ws, char* __restrict__ params, int pstride, int kcap, int V, int n, int topk, double temp_t,
+             double temp_d, double tol, int max_iters, double qstep, double tau, int Qt, float* __restrict__ alpha_out,
+             int* __restrict__ status_out, FusedArgs fa)
 {
-    __shared__ int s_list[kSolveThreads], s_count;
     pdl_wait();
-    if (!only_flagged) {
-        solve_instance(blockIdx.x, ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol, max_iters, qstep, tau, Qt, 0,
-                       alpha_out, status_out, fa);
-        return;
-    }
-    for (long long b0 = blockIdx.x; b0 < batch; b0 += (long long)gridDim.x * kSolveThreads) {
+    solve_instance(blockIdx.x, ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol, max_iters, qstep, tau, Qt, 0,
+                   alpha_out, status_out, fa);
+}
+
+// The instances that the fast kernel gave up (normally none): a grid of what the SMs hold takes them from the list in the
+// workspace, the next one as soon as a place is free.
+__global__ void __launch_bounds__(kSolveThreads)
+solve_flagged_kernel(char* __restrict__ ws, char* __restrict__ params, int pstride, int kcap, int V, int n, int topk,
+                     double temp_t, double temp_d, double tol, int max_iters, double qstep, double tau, int Qt,
+                     float* __restrict__ alpha_out, int* __restrict__ status_out, FusedArgs fa)
+{
+    __shared__ int s_next;
+    pdl_wait();
+    WsHeader* const list = reinterpret_cast<WsHeader*>(ws);
+    const int flagged = list->flagged;
+    if ((int)blockIdx.x >= flagged) return;
+#pragma unroll 1
+    while (true) {
+        if (threadIdx.x == 0) s_next = atomicAdd(&list->taken, 1);
         __syncthreads();
-        if (threadIdx.x == 0) s_count = 0;
+        const int i = s_next;
+        if (i >= flagged) return;
+        const int b = reinterpret_cast<const WsHeader*>(ws + (size_t)i * ws_stride())->flagged_id;
+        solve_instance(b, ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol, max_iters, qstep, tau, Qt, 1, alpha_out,
+                       status_out, fa);
         __syncthreads();
-        const long long b = b0 + (long long)threadIdx.x * gridDim.x;
-        if (b < batch) {
-            const Header* h = reinterpret_cast<const Header*>(params + (size_t)b * pstride);
-            if (h->magic == kMagic && h->status == kNeedFallback) s_list[atomicAdd(&s_count, 1)] = (int)b;
-        }
-        __syncthreads();
-        const int count = s_count;
-        for (int i = 0; i < count; i++) {
-            solve_instance(s_list[i], ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol, max_iters, qstep, tau, Qt, 1,
-                           alpha_out, status_out, fa);
-            __syncthreads();
-        }
     }
 }
 
-int launch_solve(const char* ws, char* params, int pstride, int kcap, int V, int n, int topk, double temp_t,
+int launch_solve(char* ws, char* params, int pstride, int kcap, int V, int n, int topk, double temp_t,
                  double temp_d, double tol, int max_iters, double qstep, double tau, int batch, int only_flagged,
                  float* alpha_out, int* status_out, FusedArgs fa, cudaStream_t st)
 {
@@ -761,13 +765,14 @@ int launch_solve(const char* ws, char* params, int pstride, int kcap, int V, int
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return GR_E_LAUNCH; }
     if (!configured[dev]) {
-        if (cudaFuncSetAttribute(solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess)
+        if (cudaFuncSetAttribute(solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess ||
+            cudaFuncSetAttribute(solve_flagged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess)
             return GR_E_LAUNCH;
         configured[dev] = true;
     }
     const int grid = only_flagged && batch > kFlaggedGrid ? kFlaggedGrid : batch;
-    launch_pdl(solve_kernel, grid, kSolveThreads, smem, st, ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol,
-               max_iters, qstep, tau, Qt, only_flagged, batch, alpha_out, status_out, fa);
+    launch_pdl(only_flagged ? solve_flagged_kernel : solve_kernel, grid, kSolveThreads, smem, st, ws, params, pstride, kcap, V, n,
+               topk, temp_t, temp_d, tol, max_iters, qstep, tau, Qt, alpha_out, status_out, fa);
     return GR_OK;
 }
 

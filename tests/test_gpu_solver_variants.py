@@ -47,3 +47,37 @@ def test_slack_below_fp32():
     G.solve(other.q_logits, other.p_logits, 3, 64, 1.0, 1.0)
     again = G.read_rule(G.solve(q, p, n, topk, 0.7, 1.0))
     assert torch.equal(first.w, again.w) and torch.equal(first.iters, again.iters)
+
+
+def _median_us(call):
+    call()
+    ts = []
+    for _ in range(9):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        call()
+        b.record()
+        b.synchronize()
+        ts.append(a.elapsed_time(b) * 1e3)
+    return sorted(ts)[len(ts) // 2]
+
+
+def test_instances_left_to_the_general_kernel():
+    """With two iterations allowed half of a batch is left to the general kernel, more than its grid holds at a time: the
+    results do not depend on what else is in the batch, and the call takes less than two passes of the general kernel over
+    all rows (it takes the instances as places become free, two to an SM)."""
+    wl = W.config3(batch=1400, device="cuda", V=2500, n=8, topk=50, seed=31)
+    q, p, tt, td = wl.q_logits, wl.p_logits, 0.7, 1.0
+    opt = G.Options(max_iters=2)
+    s = G.solve(q, p, 8, 50, tt, td, opt)
+    r = G.read_rule(s)
+    left = int((r.status == G.GR_NOT_CONVERGED).sum())
+    assert 296 < left and set(r.status.tolist()) <= {G.GR_OK, G.GR_NOT_CONVERGED}
+    for lo in range(0, 1400, 350):
+        part = G.read_rule(G.solve(q[lo:lo + 350], p[lo:lo + 350], 8, 50, tt, td, opt))
+        assert torch.equal(part.w, r.w[lo:lo + 350]) and torch.equal(part.status, r.status[lo:lo + 350])
+    pair = G.solve_verify(q, p, wl.draft_tokens, wl.uniforms, 50, tt, td, opt)
+    assert torch.equal(pair[1].token, G.verify(s, wl.draft_tokens, wl.uniforms).token)
+    robust = G.Options(max_iters=2, force_robust=1)
+    mixed, alone = (_median_us(lambda o=o: G.solve(q, p, 8, 50, tt, td, o)) for o in (opt, robust))
+    assert mixed < 2.2 * alone, (mixed, alone)
