@@ -81,6 +81,9 @@ static __device__ __noinline__ double block_incl_scan(double v, GR_PTR(double) r
 // chunk per thread), then an exact fp64 pass over the one chunk selected (its residuals in shared memory, a run of
 // consecutive ids per thread).  Bound by the latency of three dependent reads; with one warp per instance the two
 // passes took 25 us.
+// Only an id of positive residual is ever returned.  A chunk's mass comes from fp32 sums: where all its ids are in H* or
+// masked, a rounding error of theirs can be left and select it; the nearest chunk that does hold some residual then stands
+// in for it (the next one up, at its first id; if there is none, the next one down, at its last).
 __device__ inline int resample_draw(const Header* h, const ParamView& pv, int k, double frac, const VerifyScratch& vs)
 {
     const int tid = threadIdx.x, bd = blockDim.x;
@@ -88,71 +91,88 @@ __device__ inline int resample_draw(const Header* h, const ParamView& pv, int k,
     const double rT = m_div(1.0, (double)h->temp_target), lse = h->lse_t;
     const void* row = h->q_row;
     // the total residual mass is known in closed form (1 - alpha*, or 1 when the target itself is sampled)
-    const double thr = frac * (k > 0 ? h->resid_total : 1.0);
-    if (tid == 0) { vs.dec[4] = 0x7fffffff; vs.dec[5] = -1; }
-    double run = 0.0;
-    int sel = 0x7fffffff;
+    double thr = frac * (k > 0 ? h->resid_total : 1.0);
+    int lo = 0, hi = nch, origin = -1;          // chunks looked at; the one that was selected in vain
 #pragma unroll 1
-    for (int c0 = 0; c0 < nch; c0 += bd) {
-        const int c = c0 + tid;
-        // flows of the support ids per chunk, as integers (2^-62 units: the sums do not depend on the order of the atomics)
-        GR_PTR(unsigned long long) sub = GR_PCAST(unsigned long long, vs.res);
-        sub[tid] = 0ull;
-        __syncthreads();
-        for (int j = tid; j < k; j += bd) {
-            const int at = vs.chunk[j] - c0;
-            if (at >= 0 && at < bd) atomicAdd(&sub[at], (unsigned long long)__double2ll_rn(vs.p[j] * 4611686018427387904.0));
+    while (true) {
+        if (tid == 0) { vs.dec[4] = 0x7fffffff; vs.dec[5] = -1; }
+        double run = 0.0;
+        int sel = 0x7fffffff;
+#pragma unroll 1
+        for (int c0 = 0; c0 < hi; c0 += bd) {
+            const int c = c0 + tid;
+            const bool in = c >= lo && c < hi;
+            // flows of the support ids per chunk, as integers (2^-62 units: the sums do not depend on the order of the atomics)
+            GR_PTR(unsigned long long) sub = GR_PCAST(unsigned long long, vs.res);
+            sub[tid] = 0ull;
+            __syncthreads();
+            for (int j = tid; j < k; j += bd) {
+                const int at = vs.chunk[j] - c0;
+                if (at >= 0 && at < bd) atomicAdd(&sub[at], (unsigned long long)__double2ll_rn(vs.p[j] * 4611686018427387904.0));
+            }
+            double R = 0.0;
+            if (in) {
+                const float2 ms = pv.chunk[c];
+                R = (double)ms.y * m_exp((double)ms.x * rT - lse);
+            }
+            __syncthreads();
+            if (in) R = fmax(R - (double)(long long)sub[tid] * (1.0 / 4611686018427387904.0), 0.0);
+            double tot;
+            const double inc = block_incl_scan(R, vs.red, &tot) + run;
+            if (R > 0.0 && inc > thr) atomicMin(&vs.dec[4], c);
+            if (R > 0.0) atomicMax(&vs.dec[5], c);
+            __syncthreads();
+            sel = vs.dec[4];
+            if (sel == c) vs.red[32] = inc - R;
+            run += tot;
+            if (sel != 0x7fffffff) break;
         }
-        double R = 0.0;
-        if (c < nch) {
-            const float2 ms = pv.chunk[c];
-            R = (double)ms.y * m_exp((double)ms.x * rT - lse);
-        }
         __syncthreads();
-        if (c < nch) R = fmax(R - (double)(long long)sub[tid] * (1.0 / 4611686018427387904.0), 0.0);
-        double tot;
-        const double inc = block_incl_scan(R, vs.red, &tot) + run;
-        if (c < nch && inc > thr) atomicMin(&vs.dec[4], c);
-        if (c < nch && R > 0.0) atomicMax(&vs.dec[5], c);
-        __syncthreads();
-        sel = vs.dec[4];
-        if (sel == c) vs.red[32] = inc - R;
-        run += tot;
-        if (sel != 0x7fffffff) break;
-    }
-    __syncthreads();
-    double want = 1.0e300;                      // (rounding left the threshold above the total: the last id of positive mass)
-    if (sel != 0x7fffffff) want = thr - vs.red[32];
-    else sel = vs.dec[5];
-    if (sel < 0) return -1;
-    // ---- exact pass over the chunk in id order
-    const int cb = chunk_begin(sel, head), len = chunk_end(sel, head, nch, V) - cb;
+        double want = 1.0e300;                      // (rounding left the threshold above the total: the last id of positive mass)
+        if (sel != 0x7fffffff) want = thr - vs.red[32];
+        else sel = vs.dec[5];
+        int found = 0x7fffffff, last = -1, cb = 0;
+        if (sel >= 0) {
+            // ---- exact pass over the chunk in id order
+            cb = chunk_begin(sel, head);
+            const int len = chunk_end(sel, head, nch, V) - cb;
 #pragma unroll 4
-    for (int e = tid; e < len; e += bd) vs.res[e] = exp_neg(lse - (double)load_logit_dyn(row, dtype, cb + e) * rT);
-    __syncthreads();
-    for (int j = tid; j < k; j += bd) if (vs.chunk[j] == sel) vs.res[vs.id[j] - cb] = pv.r[j];
-    if (tid == 0) { vs.dec[4] = 0x7fffffff; vs.dec[5] = -1; }
-    __syncthreads();
-    const int per = ((len + bd - 1) / bd) | 1;              // (odd: no bank conflicts)
-    const int e0 = min(tid * per, len), e1 = min(e0 + per, len);
-    double sum = 0.0;
-    int lastp = -1;
+            for (int e = tid; e < len; e += bd) vs.res[e] = exp_neg(lse - (double)load_logit_dyn(row, dtype, cb + e) * rT);
+            __syncthreads();
+            for (int j = tid; j < k; j += bd) if (vs.chunk[j] == sel) vs.res[vs.id[j] - cb] = pv.r[j];
+            if (tid == 0) { vs.dec[4] = 0x7fffffff; vs.dec[5] = -1; }
+            __syncthreads();
+            const int per = ((len + bd - 1) / bd) | 1;              // (odd: no bank conflicts)
+            const int e0 = min(tid * per, len), e1 = min(e0 + per, len);
+            double sum = 0.0;
+            int lastp = -1;
 #pragma unroll 1
-    for (int e = e0; e < e1; e++) { const double r = vs.res[e]; sum += r; if (r > 0.0) lastp = e; }
-    double tot;
-    const double inc = block_incl_scan(sum, vs.red, &tot);
-    double acc = inc - sum;
-    int hit = 0x7fffffff;
-    if (inc > want) {
+            for (int e = e0; e < e1; e++) { const double r = vs.res[e]; sum += r; if (r > 0.0) lastp = e; }
+            double tot;
+            const double inc = block_incl_scan(sum, vs.red, &tot);
+            double acc = inc - sum;
+            int hit = -1;
+            if (lastp >= 0 && inc > want) {
+                hit = lastp;                        // (the run's sum and its walk round differently)
 #pragma unroll 1
-        for (int e = e0; e < e1; e++) { acc += vs.res[e]; if (acc > want) { hit = e; break; } }
-        if (hit == 0x7fffffff && e1 > e0) hit = e1 - 1;     // (the run's sum and its walk round differently)
+                for (int e = e0; e < lastp; e++) { const double r = vs.res[e]; acc += r; if (r > 0.0 && acc > want) { hit = e; break; } }
+            }
+            if (hit >= 0) atomicMin(&vs.dec[4], hit);
+            if (lastp >= 0) atomicMax(&vs.dec[5], lastp);
+            __syncthreads();
+            found = vs.dec[4]; last = vs.dec[5];
+        }
+        if (found != 0x7fffffff) return cb + found;
+        if (last >= 0) return cb + last;
+        // nothing there: the chunks above the one selected, then those below
+        if (thr > 1.0e299) { if (sel < 0) return -1; hi = sel; }
+        else {
+            if (origin < 0) origin = sel < 0 ? 0 : sel;
+            lo = sel + 1; thr = 0.0;
+            if (sel < 0 || lo >= nch) { lo = 0; hi = origin; thr = 1.0e300; }
+        }
+        __syncthreads();
     }
-    if (hit != 0x7fffffff) atomicMin(&vs.dec[4], hit);
-    if (lastp >= 0) atomicMax(&vs.dec[5], lastp);
-    __syncthreads();
-    const int found = vs.dec[4], last = vs.dec[5];
-    return found != 0x7fffffff ? cb + found : (last >= 0 ? cb + last : -1);
 }
 
 // One lane's share of the slice pi(.|omega) (Eq. "cases", Eq. "approx-c", "normalized" in Algorithm 1): lane s < n
@@ -243,7 +263,7 @@ __device__ inline void verify_instance(const Header* h, const int* draft_row, co
         const int st = slice_instance(h, pv, vs.pos[lane], lane, sl);
         if (st == GR_OK) {
             const double cum = warp_incl_scan(sl.pi, lane);
-            const unsigned hit = __ballot_sync(0xffffffffu, sl.uniq && cum > u0);
+            const unsigned hit = __ballot_sync(0xffffffffu, sl.uniq && sl.pi > 0.0 && cum > u0);
             const unsigned posm = __ballot_sync(0xffffffffu, sl.uniq && sl.pi > 0.0);
             if (hit || !sl.inner) {
                 tk = __shfl_sync(0xffffffffu, tok, hit ? __ffs(hit) - 1 : 31 - __clz(posm));
