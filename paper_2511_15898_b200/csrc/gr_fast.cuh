@@ -41,12 +41,12 @@ constexpr double kFStepClamp = 3.0;
 constexpr double kFCoarse = 1.0e-2;        // above this residual the trapezoid step is doubled
 constexpr double kFPredictStep = 1.0;      // largest |delta alpha| after which the stop on a predicted residual is allowed
 constexpr double kFPredictSafety = 10.0;   // the prediction s2 must be this many times below the tolerance
-constexpr double kFRatioSafety = 3.0;      // the predicted residual rho * r must be this many times below the tolerance
+constexpr double kFRatioSafety = 3.0;      // the residual predicted by the last step's contraction must be this many times below the tolerance
 constexpr double kFTrustPivot = 0.02;      // smallest relative pivot at which a predicted stop is allowed
 constexpr double kFPredictBound = 3.0;     // reported norm after such a stop: kFPredictBound * s2
 constexpr double kFLowLeave = 3.0e-5;      // predicted residual at which the iteration goes over to fp64
 constexpr double kFLowFloor = 1.0e-4;      // below this residual a failure to improve is taken for fp32's noise
-constexpr double kFChordBase = 0.02;       // contraction assumed of a step with the Hessian of a point a distance 0 away
+constexpr double kFChordBase = 0.02;       // contraction assumed of a step by conjugate gradients (a third of what the stop allows for)
 constexpr int kFCgMax = 16;                // conjugate-gradient iterations before the factorisation takes over
 constexpr float kFCgTol = 2.0e-4f;         // and their relative residual
 constexpr float kFScaleJump = 0.5f;        // distance of the common scale from which its curve is inverted exactly
@@ -1459,25 +1459,32 @@ __device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, c
         delta = dl;
         alpha = fmin(fmax(alpha + dl, -kFAlphaClamp), kFAlphaClamp);
         // Stop on a predicted residual, without another evaluation, after a step from a point evaluated in fp64 on the
-        // full grid.  s2 = sum_i g_i delta_i^2 is what a full Newton step in alpha = log w leaves behind (each flow is a
-        // sum of terms exponential in alpha over positive normalisers; measured on every benchmark shape and at target
-        // temperatures down to 0.3, 2300 full-grid steps: next residual <= 8.5 s2 + the quadrature floor of ~3e-9, median
-        // 0.15 s2).  (i) By the step: 10 s2 below the tolerance.  (ii) With a reused Hessian a linear term comes on top: the
-        // distance to the point it was formed at, plus the accuracy it was formed with.  (iii) By the ratio: the last full
-        // step on this grid contracted the residual by rho < 0.1 and the next one is taken to contract no worse.
-        // None is trusted when the factorisation cancelled all but a few percent of some diagonal entry: with weights of
+        // full grid.  Measured against the oracle's residual at the weights returned, 9500 such stops at tolerances of 1e-8,
+        // 3e-7 and 1e-5: every benchmark shape, random rows of 16 to 128 tokens with 2 to 32 drafts, and rows picked for
+        // prefixes that are almost tight (weights on several scales), inner systems and outer blocks:
+        // (i) By the step.  Second order: s2 = sum_i g_i delta_i^2 (each flow is a sum of terms exponential in alpha over
+        // positive normalisers; never above 8.5 s2 + the quadrature floor of ~3e-9, median 0.15 s2).  First order, after
+        // conjugate gradients: what the half-precision Hessian leaves of the residual, up to 0.03 of it (0.01 in outer
+        // blocks), plus the distance to the point where a reused one was formed.
+        // (ii) By the ratio: the last full step on this grid contracted the residual by rho < 0.1, and the next one is taken
+        // to contract by no less than that and its own length (along a direction in which the flows hardly change s2 says
+        // nothing, and half the length of the step is what it leaves: steps of 0.2 to 0.9 left 0.1 to 0.4 of the residual).
+        // Neither is trusted when the factorisation cancelled all but a few percent of some diagonal entry, or, after
+        // conjugate gradients, when the common scale of the weights has a slope of that order: with weights of
         // 1e5 and more the fp32 system stops producing Newton steps, the residual stays where it is while the steps, and
-        // with them s2, shrink; every such case measured had a relative pivot below 4e-3, every other above 3e-2.
+        // with them s2, shrink.  (Relative pivots then lie below 4e-3, others above 3e-2.  An outer block has no common
+        // scale: it is the direction that the system leaves out.)
         const bool trusted = !fail && pivot > (float)kFTrustPivot;
         if (mode == kLow) {
             // the next point is close enough: fp64 from here on, with this factorisation
             if (kFPredictBound * s2 < kFLowLeave && dm + fabs(jump) <= 0.1) { mode = trusted ? kChord : kHigh; full_grid = true; dist = dm; }
         } else if (trusted && !coarse) {
-            const double lin = mode == kChord ? (kFChordBase + 2.0 * dist) * rn : 0.0;
+            const double lin = chol ? 0.0 : (kFChordBase + (mode == kChord ? 2.0 * dist : 0.0)) * rn;
+            const double next = fmax(rho, dm + fabs(jump));
             const bool by_step = dm + fabs(jump) <= kFPredictStep && kFPredictSafety * s2 + 3.0 * lin < tol;
-            const bool by_ratio = rho < 0.1 && dm <= kFStepClamp && kFRatioSafety * rho * rn < tol;
+            const bool by_ratio = rho < 0.1 && dm <= kFStepClamp && kFRatioSafety * next * rn < tol;
             if (by_step || by_ratio) {
-                rn = by_step ? kFPredictBound * s2 + lin : rho * rn;
+                rn = by_step ? kFPredictBound * s2 + lin : next * rn;
                 status = GR_OK; it++;
                 predicted = true;
                 break;

@@ -49,6 +49,46 @@ def test_slack_below_fp32():
     assert torch.equal(first.w, again.w) and torch.equal(first.iters, again.iters)
 
 
+def _nearly_tight_rows(V, n, k, scale, noise, count, pool, seed):
+    """The rows, out of `pool` random ones, whose chain psi comes closest to a second minimum without reaching it: half of
+    them by a prefix of H*, half by a prefix beyond it.  Their weights lie on several scales."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    q = scale * torch.randn(pool, V, generator=g, device="cuda")
+    p = q + noise * torch.randn(pool, V, generator=g, device="cuda")
+    top, idx = torch.topk(p.double(), k, dim=1)
+    t, d = torch.softmax(q.double(), 1).gather(1, idx), torch.softmax(top, 1)
+    o = torch.argsort(top - q.double().gather(1, idx), dim=1, descending=True)
+    zero = torch.zeros(pool, 1, device="cuda", dtype=torch.float64)
+    psi = torch.cat([zero, torch.cumsum(t.gather(1, o), 1) - torch.cumsum(d.gather(1, o), 1).clamp(max=1.0) ** n], 1)
+    least, at = psi.min(1, keepdim=True)
+    pos = torch.arange(k + 1, device="cuda")[None]
+    below = torch.flip(torch.cummin(torch.flip(psi, [1]), 1).values, [1])
+    below = torch.cat([below[:, 1:], zero + 9.0], 1)
+    away = torch.where(pos != at, psi - least, 9.0).min(1).values
+    picked = []
+    for gap in (torch.where((pos > at) & (psi > below), psi - below, 9.0), torch.where(pos < at, psi - least, 9.0)):
+        m = gap.min(1).values
+        picked.append(torch.argsort(torch.where((m < 3e-6) | (away < 3e-6), 9.0, m))[: count // 2])
+    sel = torch.cat(picked)
+    return q[sel].contiguous(), p[sel].contiguous()
+
+
+@pytest.mark.parametrize("V,n,k,scale,noise", [(40, 2, 16, 2, 1), (40, 16, 20, 3, 3), (129, 4, 100, 3, 2), (60, 32, 50, 3, 3)])
+@pytest.mark.parametrize("tol,quad_step", [(3.0e-7, 0.4), (1.0e-8, 0.25)])
+def test_stops_on_predicted_residuals(V, n, k, scale, noise, tol, quad_step):
+    """Where the weights lie on several scales a step can be long in directions that the flows hardly feel: the residual a
+    system stops at is still the one it reports, within the tolerance (one per system of the instance; the lower one with a quadrature step whose
+    own error is far below it)."""
+    q, p = _nearly_tight_rows(V, n, k, scale, noise, 256, 100000, 77 + V + n + k)
+    wl = W.Workload("nearly tight", V, n, k, 1.0, 1.0, q, p, torch.zeros(256, n, dtype=torch.int32, device="cuda"),
+                    torch.full((256, 2), 0.5, device="cuda"))
+    rep = P.certify(wl, G.Options(tol=tol, quad_step=quad_step))
+    print(rep.summary())
+    assert rep.n_status_ok == rep.n_inst and rep.n_struct_mismatch == 0
+    assert rep.n_underreported == 0 and rep.n_evaluated_off == 0, (rep.summary(), rep.details[:5])
+    assert rep.cert_solver_max <= 2.0 * tol + 1.0e-8, rep.summary()
+
+
 def _median_us(call):
     call()
     ts = []
