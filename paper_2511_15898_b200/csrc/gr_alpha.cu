@@ -80,7 +80,7 @@ alpha_kernel(const char* __restrict__ ws, int V, int topk, double temp_t, double
         for (int o = 16; o > 0; o >>= 1) best = fmin(best, __shfl_xor_sync(0xffffffffu, best, o));
         if (lane == 0) alpha_out[(size_t)b * nl.count + e] = (float)(1.0 + best);
     }
-    if (tid == 0) status_out[b] = GR_OK;
+    if (tid == 0) status_out[b] = wv.h->check ? GR_CHECK_FAILED : GR_OK;    // (never set but in the bounds-checked build)
 }
 
 void launch_alpha(const char* ws, int V, int topk, double temp_t, double temp_d, const int* n_list, int n_count,

@@ -207,26 +207,32 @@ int gr_read_slice(const void* params, const int* draft_tokens, int batch, int n,
 }
 
 #ifdef GR_CHECK
-// Bounds-checked build only: exercises the checked pointer itself.  A kernel reads and writes a 4-entry shared
-// array through it at indices -1 .. 4; out[0] = number of accesses that were skipped and flagged (expected 2),
-// out[1] = sum of what the in-range reads returned (expected 0+1+2+3), out[2] = the values the skipped reads gave.
+// Bounds-checked build only: exercises the checked pointer and the checked array.  A kernel reads and writes four entries in
+// shared memory through each, at indices -1 .. 4; out[0] = number of accesses that were skipped and flagged (expected 2),
+// out[1] = sum of what the in-range reads returned (expected 0+1+2+3), out[2] = the values the skipped reads gave, out[3] =
+// the sum of the entries afterwards; out[4 .. 7] the same of the array.
 namespace gr {
 __global__ void check_selftest_kernel(int* out)
 {
     __shared__ int arr[4];
+    __shared__ CkArray<int, 4> own;
     __shared__ int flag;
     if (threadIdx.x == 0) {
-        for (int i = 0; i < 4; i++) arr[i] = i;
-        int skipped = 0, sum = 0, ghost = 0;
+        for (int i = 0; i < 4; i++) { arr[i] = i; own[i] = i; }
+        int skipped = 0, sum = 0, ghost = 0, skipped2 = 0, sum2 = 0, ghost2 = 0;
         for (int i = -1; i <= 4; i++) {
             flag = 0;
             CkPtr<int> p(arr, 4, &flag);
             const int v = p[i];
             p[i] = v;                       // a skipped write must not land anywhere
             if (flag) { skipped++; ghost += v; } else sum += v;
+            GR_ARRAY_RESET(own);
+            const int w = own[i];
+            own[i] = w;
+            if (GR_ARRAY_BAD(own)) { skipped2++; ghost2 += w; } else sum2 += w;
         }
-        out[0] = skipped; out[1] = sum; out[2] = ghost;
-        out[3] = arr[0] + arr[1] + arr[2] + arr[3];
+        out[0] = skipped; out[1] = sum; out[2] = ghost; out[3] = arr[0] + arr[1] + arr[2] + arr[3];
+        out[4] = skipped2; out[5] = sum2; out[6] = ghost2; out[7] = own[0] + own[1] + own[2] + own[3];
     }
 }
 }  // namespace gr

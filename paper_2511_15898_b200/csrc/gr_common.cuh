@@ -12,7 +12,7 @@ namespace gr {
 
 // ---- Bounds-checked build.  Compiled with -DGR_CHECK (paper_2511_15898_b200.build.build_library(check=True), a
 // separate library file) every pointer into shared memory, into the workspace records and into the params block
-// carries its extent: an access outside it is SKIPPED (a read gives 0) and raises a per-CTA flag, which the kernel
+// carries its extent (and every array of a shared structure its own): an access outside it is SKIPPED (a read gives 0) and raises a per-CTA flag, which the kernel
 // turns into the instance's status GR_CHECK_FAILED.  It stands in for a memory checker on machines where none may
 // run; nothing traps or asserts.  Without the macro the same names are plain pointers and cost nothing.
 #ifdef GR_CHECK
@@ -38,6 +38,24 @@ struct CkPtr {
         return CkPtr<U>(reinterpret_cast<U*>(p), n * (long long)sizeof(T) / (long long)sizeof(U), bad);
     }
 };
+// An array that is a member of a shared structure (whose address the accesses do not pass around): it carries the report.
+template <class T, int N>
+struct CkArray {
+    T a[N];
+    int bad;
+    union { unsigned long long word[2]; } sink;
+    template <class U> __device__ U& as(long long i) {
+        if (i >= 0 && (i + 1) * (long long)sizeof(U) <= (long long)sizeof(a)) return reinterpret_cast<U*>(a)[i];
+        bad = 1;
+        sink.word[0] = sink.word[1] = 0ull;
+        return *reinterpret_cast<U*>(&sink);
+    }
+    __device__ T& operator[](long long i) { return as<T>(i); }
+};
+#define GR_ARRAY(T, name, count) ::gr::CkArray<T, (count)> name
+#define GR_ARRAY_AS(U, array, i) ((array).template as<U>(i))
+#define GR_ARRAY_RESET(array) ((void)((array).bad = 0))
+#define GR_ARRAY_BAD(array) ((array).bad)
 #define GR_PTR(T) ::gr::CkPtr<T>
 #define GR_MKPTR(T, ptr, count, flag) ::gr::CkPtr<T>((ptr), (count), (flag))
 #define GR_PCAST(T, ptr) ((ptr).template as<T>())
@@ -48,6 +66,10 @@ struct CkPtr {
 #else
 template <class T> using RawPtr = T*;       // (an alias, so that "GR_PTR(double) a, b;" declares two pointers)
 #define GR_PTR(T) ::gr::RawPtr<T>
+#define GR_ARRAY(T, name, count) T name[count]
+#define GR_ARRAY_AS(U, array, i) (reinterpret_cast<U*>(array)[i])
+#define GR_ARRAY_RESET(array) ((void)0)
+#define GR_ARRAY_BAD(array) (0)
 #define GR_MKPTR(T, ptr, count, flag) (ptr)
 #define GR_PCAST(T, ptr) (reinterpret_cast<T*>(ptr))
 #define GR_CHECK_FLAG_DECL

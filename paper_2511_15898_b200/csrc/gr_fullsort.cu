@@ -395,7 +395,7 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
     }
     if (tid == 0) {
         flag[0] = todo;
-        if (GR_CHECK_VALUE) {                       // (bounds-checked build: an access was out of range)
+        if (GR_CHECK_VALUE || wh->check) {          // (bounds-checked build: an access was out of range)
             if (hdr) hdr->status = GR_CHECK_FAILED;
             if (status_out) status_out[b] = GR_CHECK_FAILED;
             for (int j = 0; j < nl.count; j++) alpha_out[(size_t)b * nl.count + j] = nanf("");

@@ -41,16 +41,24 @@ struct ScanArgs {
 template <int NTHR, int CAP, int CH>
 struct __align__(16) ScanShared {
     static constexpr int kThr = NTHR, kCap = CAP, kCh = CH;
-    unsigned long long keys[CAP];    // candidates (value, id), then composite keys
-    float2 chunk[CH];
+    GR_ARRAY(unsigned long long, keys, CAP);    // candidates (value, id), then composite keys
+    GR_ARRAY(float2, chunk, CH);
     double lse[1], part[NTHR / 32], top;
     unsigned long long prefix;
-    unsigned int gkey[NTHR];
-    int hist[256];
+    GR_ARRAY(unsigned int, gkey, NTHR);
+    GR_ARRAY(int, hist, 256);
     int need, cnt, bad, kept;
     float tau;
-    // cluster-split rows (used in the leading CTA): what the others found
-    int part_cnt[kMaxCluster], part_bad[kMaxCluster];
+    // cluster-split rows (used in the leading CTA): what the others found; bit 1 of part_bad: one of their accesses was skipped
+    GR_ARRAY(int, part_cnt, kMaxCluster);
+    GR_ARRAY(int, part_bad, kMaxCluster);
+    // bounds-checked build: whether an access to one of the arrays was skipped
+    __device__ void reset_checks() {
+        GR_ARRAY_RESET(keys); GR_ARRAY_RESET(chunk); GR_ARRAY_RESET(gkey); GR_ARRAY_RESET(hist); GR_ARRAY_RESET(part_cnt); GR_ARRAY_RESET(part_bad);
+    }
+    __device__ int checks() {
+        return GR_ARRAY_BAD(keys) | GR_ARRAY_BAD(chunk) | GR_ARRAY_BAD(gkey) | GR_ARRAY_BAD(hist) | GR_ARRAY_BAD(part_cnt) | GR_ARRAY_BAD(part_bad);
+    }
 };
 
 template <typename T> struct VecTraits;
@@ -145,8 +153,8 @@ __device__ __forceinline__ void push_candidate(SS& sh, float val, int id, float 
     if (val >= tau) {
         const int slot = atomicAdd(&sh.cnt, 1);
         if (slot < SS::kCap) {
-            reinterpret_cast<float*>(sh.keys)[slot] = val;
-            reinterpret_cast<int*>(sh.keys)[SS::kCap + slot] = id;
+            GR_ARRAY_AS(float, sh.keys, slot) = val;
+            GR_ARRAY_AS(int, sh.keys, SS::kCap + slot) = id;
         }
     }
 }
@@ -256,7 +264,7 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
     const int first = cr * W, stride = cn * W;           // this CTA's chunks: first + warp, + stride, ...
     const bool take_all = !kFull && V <= SS::kCap;       // every element is a candidate
     const bool use_tau = !kFull && !take_all;
-    if (tid == 0) { sh.cnt = 0; sh.bad = 0; sh.tau = -INFINITY; }
+    if (tid == 0) { sh.cnt = 0; sh.bad = 0; sh.tau = -INFINITY; sh.reset_checks(); }
     if (kFull && tid < 3) sh.hist[tid] = 0;
     if (cn > 1) cluster_barrier(); else __syncthreads();
 
@@ -422,7 +430,7 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
 #pragma unroll
         for (int u = 0; u < kPer; u++) {
             const int e = tid + u * SS::kThr;
-            vv[u] = e < M ? reinterpret_cast<const float*>(sh.keys)[e] : -INFINITY;
+            vv[u] = e < M ? GR_ARRAY_AS(float, sh.keys, e) : -INFINITY;
             own = fmaxf(own, vv[u]);
         }
         // (the threads' shares of the list are the groups: in a short row the threads' maxima are too few to tell anything, and
@@ -433,7 +441,7 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
 #pragma unroll
         for (int u = 0; u < kPer; u++) {
             const int e = tid + u * SS::kThr;
-            kk[u] = e < M && vv[u] >= tau ? ckey(vv[u], reinterpret_cast<const int*>(sh.keys)[SS::kCap + e]) : 0ull;
+            kk[u] = e < M && vv[u] >= tau ? ckey(vv[u], GR_ARRAY_AS(int, sh.keys, SS::kCap + e)) : 0ull;
         }
         if (tid == 0) sh.kept = 0;
         __syncthreads();
@@ -456,22 +464,24 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
             for (int c = first + warp; c < nch; c += stride) {
                 if (lane == 0) {
                     const float2 t = sh.chunk[c];
+#ifdef GR_CHECK
+                    if (c >= SS::kCh) { *check = 1; continue; }
+#endif
                     st_cluster(lead_chunk + 8u * (unsigned)c, f_pack(t.x, t.y));
                 }
             }
         }
         const int keep = min(M, nsel);
         // (the leader's list is overwritten only after it has taken its own largest: a barrier on both sides)
-        if (tid == 0) { st_cluster(cluster_addr(&sh.part_cnt[cr], 0), (unsigned int)keep); st_cluster(cluster_addr(&sh.part_bad[cr], 0), (unsigned int)sh.bad); }
         unsigned long long own = 0ull;
         int own_rank = -1;
         // keep <= kMaxSupport <= kThr candidates survive in one CTA; a thread may hold several of the M, so survivors go
         // through the upper half of the key array
-        unsigned long long* stage = sh.keys + SS::kCap - kMaxSupport;
+        constexpr int stage = SS::kCap - kMaxSupport;
         const bool overlap = M > SS::kCap - kMaxSupport;
-        if (!overlap) rank_select(sh, M, keep, [&](int rank, unsigned long long key) { stage[rank] = key; });
+        if (!overlap) rank_select(sh, M, keep, [&](int rank, unsigned long long key) { sh.keys[stage + rank] = key; });
         __syncthreads();
-        if (!overlap && tid < keep) { own = stage[tid]; own_rank = tid; }
+        if (!overlap && tid < keep) { own = sh.keys[stage + tid]; own_rank = tid; }
         if (overlap) {
             // (a list this full comes from rows of ties only: one thread per key, ranks counted from global order)
             for (int e = tid; e < M; e += SS::kThr) {
@@ -483,7 +493,14 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
             __syncthreads();
             if (tid < keep) { own = sh.keys[sh.gkey[tid]]; own_rank = tid; }
         }
+#ifdef GR_CHECK
+        if (own_rank >= kMaxSupport || (cr + 1) * kMaxSupport > SS::kCap) { *check = 1; own_rank = -1; }
+#endif
         cluster_barrier();
+        if (tid == 0) {
+            st_cluster(cluster_addr(&sh.part_cnt[cr], 0), (unsigned int)keep);
+            st_cluster(cluster_addr(&sh.part_bad[cr], 0), (unsigned int)(sh.bad | ((sh.checks() | (check ? *check : 0)) ? 2 : 0)));
+        }
         if (own_rank >= 0) st_cluster(lead_keys + 8u * (unsigned)(cr * kMaxSupport + own_rank), own);
         cluster_barrier();
         if (cr > 0) return;
@@ -496,7 +513,10 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
         }
         if (tid == 0) {
             sh.kept = 0;
-            for (int i = 1; i < cn; i++) sh.bad |= sh.part_bad[i];
+            for (int i = 1; i < cn; i++) {
+                sh.bad |= sh.part_bad[i] & 1;
+                if (check && (sh.part_bad[i] & 2)) *check = 1;
+            }
         }
         __syncthreads();
 #pragma unroll
@@ -511,8 +531,10 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
         // (sh.hist is zero)
         const unsigned a = __reduce_max_sync(0xffffffffu, fkey(g0)), k1 = __reduce_max_sync(0xffffffffu, fkey(kmax));
         const unsigned k0 = __reduce_max_sync(0xffffffffu, fkey(-kmin));
-        unsigned* const top = reinterpret_cast<unsigned*>(sh.hist);
-        if (lane == 0) { atomicMax(&top[0], a); atomicMax(&top[1], k1); atomicMax(&top[2], k0); }
+        if (lane == 0) {
+            atomicMax(&GR_ARRAY_AS(unsigned, sh.hist, 0), a); atomicMax(&GR_ARRAY_AS(unsigned, sh.hist, 1), k1);
+            atomicMax(&GR_ARRAY_AS(unsigned, sh.hist, 2), k0);
+        }
     }
     // ---- row totals (the terms are in shared memory since a barrier at least)
     if (cn > 1) lse_terms(sh, nch, A.temp_t);
@@ -551,11 +573,11 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
         wh->flagged = 0; wh->taken = 0;
         wh->count = nsel;
         wh->bad = sh.bad;
-        wh->check = check ? *check : 0;
+        wh->check = sh.checks() | (check ? *check : 0);
         if (kFull) {
-            const unsigned* const top = reinterpret_cast<const unsigned*>(sh.hist);
             FullRow fr;
-            fr.pmax = fkey_inv(top[0]); fr.kmax = fkey_inv(top[1]); fr.kmin = -fkey_inv(top[2]); fr.qmax = (float)sh.top;
+            fr.pmax = fkey_inv(GR_ARRAY_AS(unsigned, sh.hist, 0)); fr.kmax = fkey_inv(GR_ARRAY_AS(unsigned, sh.hist, 1));
+            fr.kmin = -fkey_inv(GR_ARRAY_AS(unsigned, sh.hist, 2)); fr.qmax = (float)sh.top;
             *reinterpret_cast<FullRow*>(wsb + sizeof(WsHeader)) = fr;
         }
     }

@@ -26,12 +26,16 @@ from paper_2511_15898_b200 import workloads as W
 lib = G.load_library()
 out = {"cases": []}
 if checked:
-    buf = torch.zeros(4, dtype=torch.int32, device="cuda")
+    buf = torch.zeros(8, dtype=torch.int32, device="cuda")
     lib.gr_check_selftest.restype = ctypes.c_int
     lib.gr_check_selftest.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
     assert lib.gr_check_selftest(buf.data_ptr(), None) == 0
     torch.cuda.synchronize()
     out["selftest"] = buf.cpu().tolist()
+def ascending(wl):
+    wl.p_logits = wl.p_logits.sort(dim=1).values.contiguous()
+    wl.draft_tokens = torch.full_like(wl.draft_tokens, wl.V - 1)
+    return wl
 cases = [("config1", W.config1(batch=16, device="cuda"), None),
          ("config2 V=5000", W.config2(batch=8, device="cuda", V=5000), None),
          ("support 80, n=6", W.config3(batch=4, device="cuda", seed=3100, V=20000, n=6, topk=80), None),
@@ -44,6 +48,11 @@ cases = [("config1", W.config1(batch=16, device="cuda"), None),
          ("whole vocabulary V=50257 (bucket search)", W.config4(8, 0, 1.0, batch=2, device="cuda", seed=98), None),
          ("whole vocabulary V=5000 (sort)", W.config4(4, 0, 1.0, batch=2, device="cuda", V=5000, seed=97),
           G.Options(force_robust=1)),
+         # rows split over clusters of 8, 4 and 2 CTAs; a candidate list that overflows
+         ("cluster of 8, V=150771", W.config3(batch=2, device="cuda", seed=3104, V=150771, n=4, topk=100), None),
+         ("cluster of 4, V=70001", W.config3(batch=20, device="cuda", seed=3105, V=70001, n=3, topk=20), None),
+         ("cluster of 2, V=33001", W.config3(batch=40, device="cuda", seed=3106, V=33001, n=2, topk=8), None),
+         ("ascending V=33001", ascending(W.config3(batch=5, device="cuda", seed=3107, V=33001, n=2, topk=64)), None),
          ("bf16 V=9001", W.config5(batch=4, device="cuda", V=9001, rows_per_pass=4), None)]
 for name, wl, opt in cases:
     s = G.solve(wl.q_logits, wl.p_logits, wl.n, wl.topk, wl.temp_target, wl.temp_draft, opt)
@@ -71,9 +80,9 @@ def _run(checked: int):
 def test_checked_build_reports_nothing_and_agrees_with_the_regular_build():
     chk = _run(1)
     ref = _run(0)
-    # the checked pointer itself: two of six accesses (indices -1 and 4) skipped and flagged, reads there gave 0,
-    # the array is untouched
-    assert chk["selftest"] == [2, 6, 0, 6], chk["selftest"]
+    # the checked pointer and the checked array themselves: two of six accesses (indices -1 and 4) skipped and flagged,
+    # reads there gave 0, the entries are untouched
+    assert chk["selftest"] == [2, 6, 0, 6] * 2, chk["selftest"]
     GR_CHECK_FAILED = 7
     for a, b in zip(chk["cases"], ref["cases"]):
         assert a["name"] == b["name"]
