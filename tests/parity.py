@@ -87,6 +87,12 @@ def _host_inputs(wl: W.Workload):
             wl.uniforms.cpu().numpy())
 
 
+def oracle_temps(wl: W.Workload):
+    """The temperatures as the C interface takes them, rounded to fp32: at 0.7 the rounding (1.7e-8) is up to 2e-7 in the
+    target of a row whose logits spread over ten units."""
+    return float(np.float32(wl.temp_target)), float(np.float32(wl.temp_draft))
+
+
 def _sweep_uniforms(B: int, draws: int, rho: np.ndarray, seed: int) -> np.ndarray:
     """[B, draws, 2] float32: the first half uniform in the unit square; the second half with u0 placed inside the
     resample segment where there is one (so that the two-level residual CDF is exercised by every instance that has
@@ -116,7 +122,8 @@ def compare(wl: W.Workload, opt=None, oracle_tol: float = 1e-11, tie_gap: float 
     g_alpha = solved.alpha_star.cpu().numpy().astype(np.float64)
 
     tl, dl, toks, uni = _host_inputs(wl)
-    res = O.solve_verify_batch(tl, dl, wl.n, wl.topk, wl.temp_target, wl.temp_draft, toks, uni, tol=oracle_tol)
+    tt, td = oracle_temps(wl)
+    res = O.solve_verify_batch(tl, dl, wl.n, wl.topk, tt, td, toks, uni, tol=oracle_tol)
 
     # draws: the workload's own uniforms first, then the seeded sweep
     U = np.empty((B, draws, 2), dtype=np.float32)
@@ -136,7 +143,7 @@ def compare(wl: W.Workload, opt=None, oracle_tol: float = 1e-11, tie_gap: float 
         g_tok[:, q] = ver.token.cpu().numpy(); g_acc[:, q] = ver.accepted.cpu().numpy()
         if q == 0:
             g_st = ver.status.cpu().numpy()
-    o_tok, o_acc, margin = O.draw_sweep_batch(tl, dl, wl.n, wl.topk, wl.temp_target, wl.temp_draft, res, toks, U)
+    o_tok, o_acc, margin = O.draw_sweep_batch(tl, dl, wl.n, wl.topk, tt, td, res, toks, U)
     assert np.array_equal(o_tok[:, 0], res.token) and np.array_equal(o_acc[:, 0], res.accepted)
 
     alpha_err = float(np.max(np.abs(g_alpha - res.alpha_star))) if B else 0.0
@@ -235,6 +242,7 @@ def certify(wl: W.Workload, opt=None, tie_gap: float = 1e-6, chunk: int = 256) -
     rule = G.read_rule(solved)
     torch.cuda.synchronize()
     B = wl.batch
+    tt, td = oracle_temps(wl)
     g_ids = rule.ids.numpy(); g_blk = rule.block.numpy(); g_w = rule.w.numpy(); g_lse = rule.lse_target.numpy()
     near = 0; bad = 0; cert_max = 0.0; cert2_max = 0.0; lse_err = 0.0; alpha_err = 0.0; under = 0
     predicted = rule.gnorm_predicted.numpy(); n_pred = int(predicted.sum()); n_off = 0
@@ -242,7 +250,7 @@ def certify(wl: W.Workload, opt=None, tie_gap: float = 1e-6, chunk: int = 256) -
     for c0 in range(0, B, chunk):
         c1 = min(B, c0 + chunk)
         tl = W.logits_to_f64(wl.q_logits[c0:c1]); dl = W.logits_to_f64(wl.p_logits[c0:c1])
-        cert = O.certify_batch(tl, dl, wl.n, wl.topk, wl.temp_target, wl.temp_draft, g_w[c0:c1], lse=g_lse[c0:c1])
+        cert = O.certify_batch(tl, dl, wl.n, wl.topk, tt, td, g_w[c0:c1], lse=g_lse[c0:c1])
         for i in range(c1 - c0):
             b = c0 + i
             k = int(cert.k[i]); js = int(cert.jstar[i])

@@ -41,7 +41,14 @@ cases = [("config1", W.config1(batch=16, device="cuda"), None),
          ("support 80, n=6", W.config3(batch=4, device="cuda", seed=3100, V=20000, n=6, topk=80), None),
          ("support 128, n=16", W.config3(batch=3, device="cuda", seed=3101, V=20000, n=16, topk=128), None),
          ("ragged V=1031", W.config4(3, 6, 1.0, batch=5, device="cuda", V=1031, seed=77), None),
-         ("ragged V=4099 n=32 (robust kernel)", W.config4(32, 20, 1.0, batch=3, device="cuda", V=4099, seed=78), None),
+         ("ragged V=4099 n=32", W.config4(32, 20, 1.0, batch=3, device="cuda", V=4099, seed=78), None),
+         ("ragged V=4099 n=32 (general kernel)", W.config4(32, 20, 1.0, batch=3, device="cuda", V=4099, seed=78),
+          G.Options(force_robust=1)),
+         ("support 100, n=20", W.config3(batch=2, device="cuda", seed=3108, V=4099, n=20, topk=100), None),
+         ("support 100, n=20, tau=0.02 (general kernel)", W.config3(batch=2, device="cuda", seed=3108, V=4099, n=20, topk=100),
+          G.Options(force_robust=1, tau=0.02)),
+         ("left to the general kernel", W.config3(batch=20, device="cuda", seed=3109, V=4099, n=8, topk=50),
+          G.Options(max_iters=2)),
          ("headline shape, robust kernel", W.config3(batch=3, device="cuda", seed=3102), G.Options(force_robust=1)),
          ("headline shape, tau=0.05", W.config3(batch=4, device="cuda", seed=3103), G.Options(tau=0.05)),
          ("whole vocabulary V=5000", W.config4(4, 0, 1.0, batch=3, device="cuda", V=5000, seed=99), None),

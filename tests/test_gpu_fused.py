@@ -41,6 +41,8 @@ def _same_draws(ver, vf):
     lambda: W.config4(8, 20, 1.0, batch=128, device="cuda"),
     lambda: W.config4(16, 5, 2.0, batch=128, device="cuda"),
     lambda: W.config5(batch=24, device="cuda"),
+    lambda: W.config4(32, 20, 1.0, batch=96, device="cuda"),
+    lambda: W.config3(batch=24, device="cuda", seed=3111, V=9001, n=20, topk=100),
 ])
 def test_fused_call_emits_the_tokens_of_the_two_call_path(make):
     wl = make()
@@ -135,3 +137,27 @@ def test_fused_call_rejects_missing_pointers():
                            None, 0, wl.uniforms.data_ptr(), sv.params.data_ptr(), sv.workspace.data_ptr(),
                            sv.alpha_star.data_ptr(), 0, 0, sv.status.data_ptr(), 0)
     assert rc == -2
+
+
+def test_calls_in_a_captured_graph():
+    """The calls' dependent launches, captured and replayed on new inputs: the same bits as the calls themselves."""
+    a, b = W.config3(batch=40, device="cuda", seed=3112), W.config3(batch=40, device="cuda", seed=3113)
+    q, p, toks, uni = (x.clone() for x in (a.q_logits, a.p_logits, a.draft_tokens, a.uniforms))
+    s = G.solve(q, p, a.n, a.topk, a.temp_target, a.temp_draft)
+    v = G.verify(s, toks, uni)
+    sv, vf = G.solve_verify(q, p, toks, uni, a.topk, a.temp_target, a.temp_draft)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        G.solve(q, p, a.n, a.topk, a.temp_target, a.temp_draft, None, s)
+        G.verify(s, toks, uni, v)
+        G.solve_verify(q, p, toks, uni, a.topk, a.temp_target, a.temp_draft, None, (sv, vf))
+    for wl in (b, a):
+        for x, y in ((q, wl.q_logits), (p, wl.p_logits), (toks, wl.draft_tokens), (uni, wl.uniforms)):
+            x.copy_(y)
+        graph.replay()
+        torch.cuda.synchronize()
+        solved, ver, sv2, vf2 = _both(wl)
+        _same_draws(ver, v)
+        _same_draws(vf2, vf)
+        assert torch.equal(s.alpha_star, solved.alpha_star) and torch.equal(sv.alpha_star, sv2.alpha_star)

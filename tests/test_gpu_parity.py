@@ -133,11 +133,13 @@ def test_supports_of_65_to_128_tokens(n, topk):
     _check(P.compare(wl))
 
 
+@pytest.mark.parametrize("force_robust", [0, 1])
 @pytest.mark.parametrize("n,topk", [(32, 128), (24, 64), (17, 100)])
-def test_general_kernel_on_wide_supports_with_more_than_16_drafts(n, topk):
-    """n above 16 takes the general kernel whatever the support: up to sixteen tokens per group in its product tree."""
+def test_wide_supports_with_more_than_16_drafts(n, topk, force_robust):
+    """n above 16: the fast kernel's samples on a circle, and the general kernel (up to sixteen tokens per group in its
+    product tree), which takes over what the fast one flags."""
     wl = W.config3(batch=3, device="cuda", seed=4000 + n + topk, V=20000, n=n, topk=topk)
-    _check(P.compare(wl))
+    _check(P.compare(wl, G.Options(force_robust=force_robust)))
 
 
 def test_low_target_temperature_with_a_saturated_token():
@@ -156,10 +158,10 @@ def test_low_target_temperature_with_a_saturated_token():
     _check(P.compare(wl.rows(list(range(416, 440)))))      # includes the heaviest instance (428)
 
 
-def test_very_low_target_temperature_hands_instances_to_the_fp64_kernel():
-    """Target temperature 0.3 on the headline shape: acceptance ~0.9997, weights up to 1e7.  The fp32 Newton system
-    of the fast kernel runs out of accuracy on some instances; those are finished by the fp64 kernel from the point
-    the fast kernel reached.  Every instance must end converged, with the oracle's structure and a gradient norm
+def test_very_low_target_temperature():
+    """Target temperature 0.3 on the headline shape: acceptance ~0.9997, weights up to 1e7, where the fp32 Newton system
+    runs out of accuracy (an instance it cannot finish goes to the fp64 kernel from the point reached; that path is driven
+    in test_gpu_solver_variants.py).  Every instance must end converged, with the oracle's structure and a gradient norm
     within the tolerance at the GPU's weights."""
     base = W.config3(batch=192, device="cuda", seed=77)
     g = torch.Generator(device="cuda"); g.manual_seed(78)
@@ -364,14 +366,18 @@ def test_whole_vocabulary_alpha_star_rows_the_buckets_cannot_separate():
     assert np.abs(b - want).max() <= ALPHA_TOL, (b, want)
 
 
-def test_n32_with_a_dominant_draft_token_converges():
-    """n = 32: tokens holding a large share of the draft mass need the multiplied-out leave-one-out products
-    (the series division loses too many digits there); every instance must converge, and match the oracle."""
-    wl = W.config4(32, 20, 1.0, batch=96, device="cuda")
-    solved = G.solve(wl.q_logits, wl.p_logits, wl.n, wl.topk, wl.temp_target, wl.temp_draft)
+@pytest.mark.parametrize("force_robust", [0, 1])
+@pytest.mark.parametrize("n", [17, 32])
+def test_more_than_16_drafts_with_a_dominant_draft_token(n, force_robust):
+    """Tokens holding a large share of the draft mass: the general kernel needs the multiplied-out leave-one-out products
+    there (the series division loses too many digits), the fast one's samples on a circle divide by nothing small.  Every
+    instance must converge, and match the oracle."""
+    wl = W.config4(n, 20, 1.0, batch=96, device="cuda", seed=4043)
+    opt = G.Options(force_robust=force_robust)
+    solved = G.solve(wl.q_logits, wl.p_logits, wl.n, wl.topk, wl.temp_target, wl.temp_draft, opt)
     torch.cuda.synchronize()
     assert solved.status.cpu().tolist() == [G.GR_OK] * 96
     top = torch.softmax(torch.topk(wl.p_logits, 20, dim=1).values.double(), dim=1)[:, 0]
     assert float(top.max()) > 0.5          # the workload does contain dominant tokens
     idx = torch.argsort(top, descending=True)[:6].tolist()
-    _check(P.compare(wl.rows(idx)))
+    _check(P.compare(wl.rows(idx), opt))

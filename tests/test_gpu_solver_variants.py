@@ -41,7 +41,7 @@ def test_slack_below_fp32():
                     torch.full((16, 2), 0.5, device="cuda"))
     rep = P.certify(wl)
     print(rep.summary())
-    assert rep.alpha_err <= 1e-6 and rep.cert_solver_max <= 1.0e-6, rep.summary()
+    assert rep.alpha_err <= 1e-6 and rep.cert_solver_max <= 3.2e-7, rep.summary()
     first = G.read_rule(G.solve(q, p, n, topk, 0.7, 1.0))
     other = W.config3(batch=300, device="cuda", V=2000, n=3, topk=64)
     G.solve(other.q_logits, other.p_logits, 3, 64, 1.0, 1.0)

@@ -91,9 +91,10 @@ def test_truncated_config2_and_config4_cell():
     _check_tau(W.config4(8, 20, 1.0, batch=32, device="cuda"), 1e-2)
 
 
-def test_truncated_robust_kernel_and_32_drafts():
-    _check_tau(W.config4(32, 20, 1.0, batch=16, device="cuda"), 1e-2)
-    _check_tau(W.config3(batch=12, device="cuda", seed=3012), 1e-2, force_robust=1)
+@pytest.mark.parametrize("force_robust", [0, 1])
+def test_truncated_32_drafts_and_the_general_kernel(force_robust):
+    _check_tau(W.config4(32, 20, 1.0, batch=16, device="cuda"), 1e-2, force_robust=force_robust)
+    _check_tau(W.config3(batch=12, device="cuda", seed=3012), 1e-2, force_robust=force_robust)
 
 
 def test_truncated_wide_support():
