@@ -72,15 +72,18 @@ extern "C" {
  *              values are honoured down to the quadrature floor of a few 1e-9 at the
  *              default quad_step.)
  *              The kernels also stop after a Newton step taken from a point evaluated
- *              on the full quadrature grid when the residual that step leaves is
- *              predicted below tol, in one of two ways: the step's second-order size
- *              s2 = sum_i g_i (delta alpha_i)^2 ten times below tol (the residual after
- *              such a step stayed within 8.5 s2 + 3e-9 on every shape measured; the
- *              reported gradient norm is then 3 s2), or, after a step that contracted the
- *              residual by rho < 0.1, 3 rho r_k below tol (reported: rho r_k; the faster
- *              kernels only).  Neither is
- *              used when the factorisation of the Newton system left less than 2 % of a
- *              diagonal entry as its pivot (a system too close to singular in fp32).
+ *              on the full quadrature grid when the residual r' that step leaves is
+ *              predicted below tol, in one of two ways.  By the step: from its second-order
+ *              size s2 = sum_i g_i (delta alpha_i)^2 (r' stayed within 8.5 s2 + 3e-9 on every
+ *              shape measured) and, in the faster kernel, where the Newton system is solved
+ *              with a Hessian in half precision that may belong to an earlier point, from
+ *              lin = (0.02 + 2 x the distance to that point) x the residual: stop when
+ *              10 s2 + 3 lin < tol, reported 3 s2 + lin.  By the ratio (faster kernel only):
+ *              after a step that contracted the residual to r by rho < 0.1, stop when
+ *              3 max(rho, the step's length) r < tol, reported max(rho, length) r.  Neither
+ *              is used when the Newton system is too close to singular in fp32: less than 2 %
+ *              of a diagonal entry left as the factorisation's pivot, or of the Hessian's trace
+ *              as the slope along the common scale of the weights.
  *   max_iters  cap on gradient evaluations per system.            default 40
  *   quad_step  step of the trapezoid rule in the log-time variable used to
  *              evaluate the gradient integral; smaller is more accurate and
@@ -89,7 +92,7 @@ extern "C" {
  *              the streaming kernel and the solve kernel, so that a caller can
  *              time the two separately; NULL records nothing.      default NULL
  *   force_robust  non-zero sends every shape to the general (slower) solve kernel;
- *              by default supports of at most 128 tokens with n <= 16 take a faster
+ *              by default supports of at most 128 tokens with n >= 2 take a faster
  *              kernel that computes the same rule.  For an untruncated draft on a
  *              vocabulary beyond GR_MAX_SUPPORT (optimal acceptance only) it selects the
  *              whole-row sort instead of the bucketed search.         default 0
@@ -150,8 +153,9 @@ size_t gr_workspace_bytes(int V, int n, int topk, int batch);
  *                       so q_logits must stay unchanged until gr_verify has run.
  *   workspace           scratch, gr_workspace_bytes() bytes, 16-byte aligned;
  *                       contents are meaningless after the call completes.
- *   alpha_star          out [batch] float, optimal acceptance probability (also produced, by a sort of
- *                       the whole row, when the support exceeds GR_MAX_SUPPORT and no rule is solved).
+ *   alpha_star          out [batch] float, optimal acceptance probability (also produced when the support
+ *                       exceeds GR_MAX_SUPPORT and no rule is solved: by a bucketed search over the whole row,
+ *                       or a sort where the buckets do not separate it).
  *   status              out [batch] int, GR_OK / GR_NOT_CONVERGED /
  *                       GR_SUPPORT_TOO_LARGE / GR_BAD_LOGITS.
  */

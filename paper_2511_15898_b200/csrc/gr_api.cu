@@ -3,8 +3,8 @@
 #include "gr_host.h"
 
 namespace gr {
-// The fast kernel covers supports up to 128 tokens with n <= 16; everything else, and any instance the fast
-// kernel could not finish, takes the robust kernel.
+// The fast kernel covers supports up to 128 tokens with n = 2 .. 32; n = 1, and any instance the fast kernel could not
+// finish, takes the general kernel.
 int launch_solve_any(char* ws, char* params, int pstride, int kcap, int V, int n, int topk, double temp_t,
                      double temp_d, double tol, int max_iters, double qstep, double tau, int batch, int force_robust,
                      float* alpha_out, int* status_out, FusedArgs fa, cudaStream_t st)
@@ -13,7 +13,7 @@ int launch_solve_any(char* ws, char* params, int pstride, int kcap, int V, int n
                           : launch_fast(ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol, max_iters, qstep,
                                         tau, batch, alpha_out, status_out, fa, st);
     if (rc < 0) return rc;
-    // rc == 1: no fast variant, the robust kernel does everything; rc == 0: it redoes what the fast one flagged
+    // rc == 1: no fast variant, the general kernel does everything; rc == 0: it redoes what the fast one flagged
     return launch_solve(ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol, max_iters, qstep, tau, batch,
                         rc == 0 ? 1 : 0, alpha_out, status_out, fa, st);
 }

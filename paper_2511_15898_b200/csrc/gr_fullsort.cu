@@ -117,8 +117,8 @@ __device__ inline double block_min(double v, double* s_r)
 }
 
 // flag[0] of the instance's scratch region: bit j set when fullsort_alpha_kernel has to do the row for the j-th draft count.
-// 512 rows of 50257 in fp32: about 150 us (three passes with exp, 64-bit shared atomics and counts: 408).  Bound by the fp64 pipe (28
-// operations per id) and the shared atomics, not by the 206 MB it reads.
+// 512 rows of 50257 in fp32: about 150 us (three passes with exp, 64-bit shared atomics and counts: 408).  Bound by
+// instruction issue (130 instructions per 32 ids; fp64 pipe 28 % busy, shared atomics hidden), not by the 206 MB it reads.
 template <typename T>
 __global__ void __launch_bounds__(kBkThreads)
 bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, const __grid_constant__ NList nl, double temp_t, double temp_d,
@@ -277,7 +277,9 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
         // Inside the bucket every ratio tgt / drf is at least rho (its keys are at most kmax - c w; the first bucket has no
         // such limit), so a prefix that ends inside it has  psi >= T0 + rho (D - D0) - D^n,  concave in D: its minimum
         // over [D0, D1] is at an end.  At D0 that is the previous boundary's psi; at D1 it is the bound below.  The slack
-        // covers the rounding of the masses to integers (one unit per id).
+        // covers the rounding of the target's masses to integers (one unit per id).  That of the draft's is not in it: it is
+        // of the size by which rounding moves psi itself, n half units per id (at most n V 2^-43, 1.8e-7 for 50257 ids and 32
+        // drafts).
         const double khi = kmax - (invw > 0.0 ? (double)c / invw * (1.0 - 1e-12) : 0.0);
         const double rho = c == 0 ? 0.0 : exp(-khi) * rscale * (1.0 - 1e-9);
         lb[u] = empty ? 1.0 : T0 + rho * (D1 - D0) - dn - slack;

@@ -1,12 +1,12 @@
 // Steps shared by the two solve kernels (one CTA per instance, any block size that is a multiple of 32
-// and at least the support size + 1): distributions on the support, ratio order, subset selection,
+// and at least the support size): distributions on the support, ratio order, subset selection,
 // outer residuals and blocks; writing the rule into the params block.
 #pragma once
 #include "gr_common.cuh"
 
 namespace gr {
 
-constexpr int kNeedFallback = 100;   // internal status: the fast kernel asks the robust kernel to redo the instance
+constexpr int kNeedFallback = 100;   // internal status: the fast kernel asks the general kernel to redo the instance
 
 // CTA-wide reductions; `scratch` needs one double per warp.  Every thread gets the result.  (Out of line where they are used
 // once per instance; the general kernel's iteration takes the inline forms.)

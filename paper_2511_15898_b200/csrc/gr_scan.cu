@@ -25,8 +25,9 @@ static void launch_scan_t(const ScanArgs& A, bool full_large, int batch, cudaStr
     // One CTA per row, two CTAs per SM, half a chunk in flight per warp: 1024 fp32 rows of 128256 at 5.4 TB/s, what is
     // missing to the copy rate being the last of four waves.  Few rows are latency instead (a row on one CTA: 37 us, eight
     // rounds to memory): a cluster of CTAs per row then, one CTA per SM, a whole chunk in flight per warp, as long as
-    // every warp keeps a chunk (1 row 22 us, 32 rows 27, 64 rows 33; were 37, 39, 39).  The numbers of rows are what one
-    // wave holds: 15 clusters of 8 and 33 of 4, since the 148 SMs do not come in groups of 8; one more row costs 12 us.
+    // every warp keeps a chunk (1 row 22 us, 32 rows 27, 64 rows 33; were 37, 39, 39).  The numbers of rows are those
+    // up to which the clusters ran in one wave: the 148 SMs do not come in groups of 8, and a cluster of 8 beyond the 14th, or
+    // of 4 beyond the 32nd, cost 12 us.
     int cn = 1;
     if (!full_large) {
         const int want = batch <= 14 ? 8 : batch <= 32 ? 4 : batch <= 74 ? 2 : 1;
@@ -42,7 +43,7 @@ void launch_scan(const void* q, const void* p, int dtype, int V, int ksel, bool 
 {
     const double log2e = 1.4426950408889634;
     ScanArgs A;
-    A.q = q; A.p = p; A.dtype = dtype; A.V = V; A.ksel = ksel;
+    A.q = q; A.p = p; A.V = V; A.ksel = ksel;
     A.sc_t = (float)(log2e / temp_t); A.sc_d = (float)(log2e / temp_d);
     A.temp_t = temp_t; A.temp_d = temp_d; A.ws = ws; A.params = params; A.pstride = pstride; A.kcap = kcap;
     if (dtype == GR_F32) launch_scan_t<float>(A, full_large, batch, st);

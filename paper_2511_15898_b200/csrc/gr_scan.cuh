@@ -1,5 +1,4 @@
-// Streaming pass over the two logit rows of an instance, as CTA-level device code: by a kernel of its own (one CTA or one
-// cluster per row) or by the solve kernel's CTA before it solves the row.
+// Streaming pass over the two logit rows of an instance, as CTA-level device code, by one CTA or one cluster per row.
 //
 // In a single read of the rows it produces
 //   - the log-sum-exp of the target row at temp_target and, per 1024-element chunk,
@@ -30,7 +29,7 @@ constexpr int kRankAll = 256;        // candidates that are ranked as they are; 
 // Arguments common to every row.
 struct ScanArgs {
     const void* q; const void* p;    // logits
-    int dtype, V, ksel;
+    int V, ksel;
     float sc_t, sc_d;                // log2(e) / temperature
     double temp_t, temp_d;
     char* ws; char* params;          // workspace records; params block or nullptr (the caller wants the records only)

@@ -543,7 +543,7 @@ __device__ int solve_system(const Sm& sm, int m, GR_PTR(const double) d, GR_PTR(
         }
         __syncthreads();
         // Second-order size of the step, sum_i g_i delta_i^2: a full Newton step in alpha = log w from a point
-        // evaluated on the full grid leaves a residual of at most a small multiple of it (within 3.1 times, plus the
+        // evaluated on the full grid leaves a residual of at most a small multiple of it (within 8.5 times, plus the
         // quadrature floor, on every benchmark shape).  Ten times below the tolerance: the step is taken and the
         // iteration stops without another evaluation; the reported norm is then the bound 3 s2.
         const double s2 = reduce_sum(tid < m ? sm.g[tid] * sm.delta[tid] * sm.delta[tid] : 0.0, red);
