@@ -31,7 +31,9 @@ def test_support_and_log_sum_exp(V, batch):
         assert torch.equal(torch.sort(want, dim=1).values.int().cpu(), torch.sort(r.ids[:, :k], dim=1).values), (dt, k)
         lse = torch.logsumexp(q.double() / 0.75, 1).cpu()
         assert float((lse - r.lse_target).abs().max()) < 1e-6, (dt, k)
-        assert int((s.status > 1).sum()) == 0        # (1: a solve that did not converge, which is not this pass)
+        # (50 tokens and two drafts are a hard system in a few rows: one solve of 297 has been seen not to converge)
+        assert set(s.status.tolist()) <= {G.GR_OK, G.GR_NOT_CONVERGED}, (dt, k)
+        assert int((s.status != G.GR_OK).sum()) <= batch // 200, (dt, k)
 
 
 @pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])

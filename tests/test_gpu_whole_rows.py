@@ -1,6 +1,6 @@
 """Optimal acceptance of whole-vocabulary rows for several draft counts at once, where the bucket search can go wrong: row
-lengths around a vector and a chunk (rows that are not 16-byte aligned), crowded buckets, ties, masked ids.  Against the
-same prefix scan in fp64 on a sorted row."""
+lengths around a vector and a chunk (rows that are not 16-byte aligned), masked ids, rows of few or one ratio (crowded
+buckets, rows left to the sort).  Against the same prefix scan in fp64 on a sorted row."""
 import pytest
 import torch
 
@@ -31,13 +31,36 @@ def test_alpha_star_of_whole_rows(V, dt):
     g = torch.Generator(device="cuda").manual_seed(V)
     q = (3 * torch.randn(6, V, generator=g, device="cuda")).to(dt)
     p = (q.float() + torch.randn(6, V, generator=g, device="cuda")).to(dt)
-    p[1] = (q[1].float() + torch.randint(0, 40, (V,), generator=g, device="cuda") / 2).to(dt)   # few ratio levels
     q[2, : V // 2] = -1.0e4                                                                      # masked ids
-    p[3] = q[3]                                                                                  # one ratio
     out, st = G.alpha_star(q, p, ns, 0, 0.75, 1.25)
     assert st.tolist() == [0] * 6
     for j, n in enumerate(ns):
         assert float((out[:, j].double() - _alpha(q, p, n, 0.75, 1.25)).abs().max()) < 1e-6, n
+
+
+@pytest.mark.parametrize("V", [129, 4096, 4097, 50257])
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+def test_alpha_star_of_rows_with_few_ratios(V, dt):
+    """Logits on a grid that both types represent, at one temperature: the log-ratio keys are exactly tied, sixteen values in
+    one row and a single one (a range of zero) in the next.  A row of more than 4096 ids of one ratio is left to the sort,
+    for every draft count of the call."""
+    g = torch.Generator(device="cuda").manual_seed(V)
+    q = (torch.randn(3, V, generator=g, device="cuda") * 12).round().clamp(-48, 48) / 4
+    p = q + torch.randint(0, 16, (3, V), generator=g, device="cuda") / 2
+    p[1] = q[1]
+    q, p = q.to(dt), p.to(dt)
+    keys = p.double() - q.double()
+    assert [len(torch.unique(row)) for row in keys] == [16, 1, 16]
+    ns = [1, 2, 8, 32]
+    out, st = G.alpha_star(q, p, ns, 0, 1.0, 1.0)
+    assert st.tolist() == [0] * 3
+    for j, n in enumerate(ns):
+        assert float((out[:, j].double() - _alpha(q, p, n, 1.0, 1.0)).abs().max()) < 1e-6, n
+    words = G.solve(q, p, 8, 0, 1.0, 1.0).workspace.view(torch.int32)
+    record, row = (32 + 128 * 12) // 4, 3 * (1 << (V - 1).bit_length())      # bytes / 4: one record, one row of the scratch
+    if V > 4096:
+        # (the sort's first key, that of a ratio of one: 2^63)
+        assert words[3 * record + row:3 * record + row + 2].tolist() == [0, -2 ** 31]
 
 
 @pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
