@@ -496,7 +496,7 @@ def run_ours(args):
                    "batch1_call": float(np.median(lat)) if lat else None},
         "cpu_baseline": cpu,
         "e2e": e2e,
-        "gpu_launches": 4 * K,   # scan, fast solve, one wave that looks for flagged instances, verify
+        "gpu_launches": 4 * K,   # scan, fast solve, the pass over flagged instances, verify
         "clocks": clocks,
         "quality": {"accept_rate": acc_rate, "alpha_star_mean": float(solved.alpha_star.float().nanmean().item()),
                     "status_ok": int((status == 0).sum()), "status_not_converged": int((status == 1).sum()),
