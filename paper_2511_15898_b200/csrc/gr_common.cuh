@@ -245,6 +245,7 @@ __device__ inline unsigned long long ckey(float v, int id) {
 static __device__ __noinline__ double m_exp(double x) { return exp(x); }
 static __device__ __noinline__ double m_log(double x) { return log(x); }
 static __device__ __noinline__ double m_div(double a, double b) { return a / b; }
+static __device__ __noinline__ double2 m_div2(double a0, double a1, double b) { return make_double2(a0 / b, a1 / b); }
 
 // exp(-y) for y >= 0 (fp64): Cody and Waite's range reduction by a two-part ln 2 and a degree-13 Taylor polynomial on
 // |r| <= ln2/2 (truncation below 1e-17 relative), summed in pairs and fours (Estrin's scheme: a third of Horner's chain,

@@ -48,10 +48,12 @@ constexpr double kFLowLeave = 3.0e-5;      // predicted residual at which the it
 constexpr double kFLowFloor = 1.0e-4;      // below this residual a failure to improve is taken for fp32's noise
 constexpr double kFChordBase = 0.02;       // contraction assumed of a step by conjugate gradients (a third of what the stop allows for)
 constexpr int kFCgMax = 16;                // conjugate-gradient iterations before the factorisation takes over
-constexpr float kFCgTol = 2.0e-4f;         // and their relative residual
+constexpr float kFCgTol = 2.0e-4f;         // and their relative residual; in fp32 kFCgLow times the gradient norm, up to kFCgLoose
+constexpr float kFCgLow = 0.1f, kFCgLoose = 5.0e-3f;
 constexpr float kFScaleJump = 0.5f;        // distance of the common scale from which its curve is inverted exactly
 constexpr float kFSmallSlack = 1.0e-4f;     // share of the mass below which Tn - sum g is mostly rounding in fp32
 constexpr float kFLeastSlack = 1.0e-9f;     // and the least share aimed at (the quadrature's floor)
+constexpr float kFNone = 1.0e30f;          // no residual or ratio yet
 constexpr int kFSweeps = 5;                // fixed-point sweeps of the starting point
 
 // Compile-time geometry.  NT: series length (>= n), MP: padded support size, T: threads, JC: Hessian nodes staged
@@ -148,7 +150,8 @@ struct FSm {
         pi = GR_MKPTR(__half, reinterpret_cast<__half*>(sb + C::oU), C::MP * C::kNS, ck);
     }
 };
-enum { SC_FAIL = 0, SC_PIVOT = 1, SC_NP = 2, SC_OUT = 4 };
+// (what stays the same during a system is read from here: kept in registers it was spilled around every call)
+enum { SC_FAIL = 0, SC_PIVOT = 1, SC_NP = 2, SC_OUT = 4, SC_TOL = 8, SC_QSTEP = 9, SC_SIGMA = 10, SC_HS = 11, SC_TN = 12, SC_GNORM = 13, SC_ITERS = 14 };
 
 // The circle of the contour kernels: `np` conjugate pairs of points r e^(i theta), angles theta and n theta (mod 2 pi),
 // factor 2 n! / (N r^n) of the mean.
@@ -243,55 +246,62 @@ __device__ __forceinline__ uint32_t pack_half(float a, float b) {
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// ---- reductions over the token threads (the first kTW warps; the other copies' values are ignored); every thread
-// gets the result.  Two scratch areas in turn (`par`): one barrier each.  Out of line for the sake of code size.
-// (maximum of a, or its sum with `add`; sum of b)
-template <class C>
-__device__ __noinline__ double2 tok_max_sum_fn(double a, double b, bool add, int par, int* flag)
+// Sums (fp64 and fp32) and maxima (unsigned) over the token threads, every thread gets them: the first kTW warps hold the
+// tokens (the other copies hold the same values, and no barrier is needed where a warp holds them all).  Two scratch areas
+// in turn (`par`), one barrier for all values of a call: what an iteration needs is asked for together, since a call costs
+// about 400 cycles whatever it carries.
+template <class C, int ND, int NF, int NU>
+__device__ __forceinline__ void tok_reduce(const FSm<C>& sm, double* d, float* f, unsigned* u, int& par)
 {
-#pragma unroll 1
-    for (int o = 16; o > 0; o >>= 1) {
-        const double t = __shfl_xor_sync(0xffffffffu, a, o);
-        a = add ? a + t : fmax(a, t);
-        b += __shfl_xor_sync(0xffffffffu, b, o);
-    }
-    GR_PTR(double) r = GR_MKPTR(double, reinterpret_cast<double*>(smem_raw + C::oRed), 64, flag) + 32 * par;
-    const int w = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0 && w < C::kTW) { r[2 * w] = a; r[2 * w + 1] = b; }
-    __syncthreads();
-    a = r[0]; b = r[1];
+    static_assert(ND <= 2 && NF <= 4 && NU <= 4 && C::kTW <= 4, "a warp's slot is eight doubles");
+    __syncwarp();
 #pragma unroll
-    for (int i = 1; i < C::kTW; i++) { a = add ? a + r[2 * i] : fmax(a, r[2 * i]); b += r[2 * i + 1]; }
-    return make_double2(a, b);
-}
-template <class C>
-__device__ __forceinline__ void tok_max_sum(const FSm<C>& sm, double& a, double& b, int& par)
-{
-    const double2 t = tok_max_sum_fn<C>(a, b, false, par, sm.flag);
+    for (int k = 0; k < NU; k++) u[k] = __reduce_max_sync(0xffffffffu, u[k]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int k = 0; k < ND; k++) d[k] += __shfl_xor_sync(0xffffffffu, d[k], o);
+#pragma unroll
+        for (int k = 0; k < NF; k++) f[k] += __shfl_xor_sync(0xffffffffu, f[k], o);
+    }
+    if (C::kTW == 1) return;
+    GR_PTR(double) area = sm.red + 32 * par;
     par ^= 1;
-    a = t.x; b = t.y;
+    const int w = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0 && w < C::kTW) {
+        GR_PTR(double) r = area + 8 * w;
+        if (ND > 0) st_d2(r, make_double2(d[0], ND > 1 ? d[ND > 1 ? 1 : 0] : 0.0));
+        if (NF > 0) st_f4(GR_PCAST(float, r + 2), make_float4(f[0], NF > 1 ? f[NF > 1 ? 1 : 0] : 0.f, NF > 2 ? f[NF > 2 ? 2 : 0] : 0.f, NF > 3 ? f[NF > 3 ? 3 : 0] : 0.f));
+        if (NU > 0) st_f4(GR_PCAST(float, r + 4), make_float4(__uint_as_float(u[0]), __uint_as_float(u[NU > 1 ? 1 : 0]), __uint_as_float(u[NU > 2 ? 2 : 0]), __uint_as_float(u[NU > 3 ? 3 : 0])));
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < C::kTW; i++) {
+        GR_PTR(double) r = area + 8 * i;
+        if (ND > 0) {
+            const double2 t = ld_d2(r);
+            d[0] = i == 0 ? t.x : d[0] + t.x;
+            if (ND > 1) d[ND > 1 ? 1 : 0] = i == 0 ? t.y : d[ND > 1 ? 1 : 0] + t.y;
+        }
+        if (NF > 0) {
+            const float4 t = ld_f4(GR_PCAST(float, r + 2));
+            const float tv[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+            for (int k = 0; k < NF; k++) f[k] = i == 0 ? tv[k] : f[k] + tv[k];
+        }
+        if (NU > 0) {
+            const float4 t = ld_f4(GR_PCAST(float, r + 4));
+            const float tv[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+            for (int k = 0; k < NU; k++) u[k] = i == 0 ? __float_as_uint(tv[k]) : max(u[k], __float_as_uint(tv[k]));
+        }
+    }
 }
 template <class C>
 __device__ __forceinline__ double tok_sum(const FSm<C>& sm, double v, int& par)
 {
-    const double2 t = tok_max_sum_fn<C>(0.0, v, false, par, sm.flag);
-    par ^= 1;
-    return t.y;
-}
-// largest and smallest of the tokens' log-weights (fp32: they only place the quadrature grid)
-template <class C>
-__device__ __forceinline__ void tok_range(const FSm<C>& sm, float v, bool on, float& hi, float& lo, int& par)
-{
-    const unsigned a = __reduce_max_sync(0xffffffffu, on ? fkey(v) : 0u), b = __reduce_max_sync(0xffffffffu, on ? fkey(-v) : 0u);
-    GR_PTR(double) r = sm.red + 32 * par;
-    par ^= 1;
-    const int w = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0 && w < C::kTW) r[w] = __hiloint2double((int)a, (int)b);
-    __syncthreads();
-    unsigned ka = 0u, kb = 0u;
-#pragma unroll
-    for (int i = 0; i < C::kTW; i++) { const double t = r[i]; ka = max(ka, (unsigned)__double2hiint(t)); kb = max(kb, (unsigned)__double2loint(t)); }
-    hi = fkey_inv(ka); lo = -fkey_inv(kb);
+    tok_reduce<C, 1, 0, 0>(sm, &v, nullptr, nullptr, par);
+    return v;
 }
 
 // Accumulator fragments of the tiles a warp owns: row tiles a and b of its pair, column tiles cs, cs + kS, ...
@@ -340,19 +350,19 @@ __device__ __forceinline__ int quad_grid(float amax, float amin, int slack, floa
     return Q > kFMaxNodes ? kFMaxNodes : Q;
 }
 
-// Sum of (g, g2) over the copies of the token threads, in the same order everywhere.
+// Sum of (g, g2) over the copies of the token threads, in the same order everywhere.  (A barrier before the array is written
+// again is the caller's.)
 template <class C>
 __device__ __forceinline__ void sum_copies(const FSm<C>& sm, double& g, double& g2)
 {
     if (C::kNG > 1) {
         const int tid = threadIdx.x, i = tid % C::MP;
         GR_PTR(double) gs = GR_MKPTR(double, reinterpret_cast<double*>(sm.base + C::oSP), C::kSPBytes / 8, sm.flag);
-        gs[2 * tid] = g; gs[2 * tid + 1] = g2;
+        st_d2(gs + 2 * tid, make_double2(g, g2));
         __syncthreads();
         g = 0.0; g2 = 0.0;
 #pragma unroll
-        for (int k = 0; k < C::kNG; k++) { g += gs[2 * (k * C::MP + i)]; g2 += gs[2 * (k * C::MP + i) + 1]; }
-        __syncthreads();
+        for (int k = 0; k < C::kNG; k++) { const double2 t = ld_d2(gs + 2 * (k * C::MP + i)); g += t.x; g2 += t.y; }
     }
 }
 
@@ -746,14 +756,15 @@ __device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, doub
 
 // The fp64 evaluation, kept out of line (it is called once or twice per system, and its registers stay its own).
 template <class C>
-__device__ __noinline__ double2 eval_fp64(int m, int n, double hs, int slack, double qstep, float amax, float amin, double w_own,
-                                          double ds_own, int* flag)
+__device__ __noinline__ double2 eval_fp64(int m, int n, int slack, bool coarse, float amax, float amin, int* flag)
 {
     const FSm<C> sm(flag);
+    const int i = threadIdx.x % C::MP;
+    const double qstep = sm.scal[SC_QSTEP] * (coarse ? 2.0 : 1.0);
     Frags<C> none;
     double2 r;
-    if constexpr (C::kContour) eval_contour<C, double, false>(sm, m, slack, qstep, 1, amax, amin, w_own, 0.f, r.x, r.y, none);
-    else eval_system<C, double, false>(sm, m, n, hs, slack, qstep, 1, amax, amin, w_own, ds_own, 0.f, r.x, r.y, none);
+    if constexpr (C::kContour) eval_contour<C, double, false>(sm, m, slack, qstep, 1, amax, amin, sm.wd[i], 0.f, r.x, r.y, none);
+    else eval_system<C, double, false>(sm, m, n, sm.scal[SC_HS], slack, qstep, 1, amax, amin, sm.wd[i], i < m ? sm.dsd[i] : 0.0, 0.f, r.x, r.y, none);
     return r;
 }
 
@@ -992,22 +1003,81 @@ __device__ __forceinline__ float newton_rhs(double g, double g2, double r)
     return room > 1e-3f ? hii * (fabsf(arg) < 0.01f ? arg * fmaf(arg, fmaf(arg, 1.f / 3.f, -0.5f), 1.f) : __logf(1.f + arg)) : diff;
 }
 
+// Matrix-vector products with the half-precision matrices in sm.pi: thread t has row t / kNG and the (t % kNG)-th share of its
+// columns, so that the shares of a row meet in neighbouring lanes and not through shared memory.  The vector's shares are four
+// floats apart (their loads fall into different banks); three buffers behind what sum_copies uses.
+template <class C> __device__ __forceinline__ int vec_pos(int i) { return i + 4 * (i / (C::MP / C::kNG)); }
+template <class C>
+__device__ __forceinline__ GR_PTR(float) vec_buffer(const FSm<C>& sm, int which)
+{
+    constexpr int kLen = C::MP + 4 * C::kNG;
+    static_assert(C::T * 16 + 3 * kLen * 4 <= C::kSPBytes, "vector buffers");
+    return GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oSP + C::T * 16) + which * kLen, kLen, sm.flag);
+}
+template <class C>
+__device__ __forceinline__ float share_sum(float v)
+{
+    __syncwarp();
+#pragma unroll
+    for (int o = 1; o < C::kNG; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+template <class C>
+__device__ __forceinline__ void load_row(GR_PTR(const __half) mat, float* row)
+{
+    constexpr int kCol = C::MP / C::kNG;
+    GR_PTR(const __half) np = mat + (threadIdx.x / C::kNG) * C::kNS + (threadIdx.x % C::kNG) * kCol;
+#pragma unroll
+    for (int c = 0; c < kCol; c += 8) {
+        const uint4 v = ld_h8(np + c);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int z = 0; z < 4; z++) {
+            const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[z]));
+            row[c + 2 * z] = f.x; row[c + 2 * z + 1] = f.y;
+        }
+    }
+}
+template <class C>
+__device__ __forceinline__ float dot_row(const float* row, GR_PTR(const float) vec)
+{
+    constexpr int kCol = C::MP / C::kNG;
+    GR_PTR(const float) vp = vec + (threadIdx.x % C::kNG) * (kCol + 4);
+    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll
+    for (int c = 0; c < kCol; c += 4) {
+        const float4 v = ld_f4(vp + c);
+        a0 = fmaf(row[c], v.x, a0); a1 = fmaf(row[c + 1], v.y, a1); a2 = fmaf(row[c + 2], v.z, a2); a3 = fmaf(row[c + 3], v.w, a3);
+    }
+    return share_sum<C>((a0 + a1) + (a2 + a3));
+}
+template <class C>
+__device__ __forceinline__ float row_times(GR_PTR(const __half) mat, GR_PTR(const float) vec)
+{
+    float row[C::MP / C::kNG];
+    load_row<C>(mat, row);
+    return dot_row<C>(row, vec);
+}
+
 // fp32 evaluation at one point and what the Newton step needs from it, out of line (its registers, fragments included, stay
 // its own).  Default: the Hessian scaled to unit diagonal, I - N with N_il = H_il / sqrt(H_ii H_ll), N in half precision
 // (its error, 2^-11, is that of the contraction's operands) for cg_solve below; sm.dg receives 1 / sqrt(H_ii).
 // With `chol` a Cholesky factorisation instead, for systems conjugate gradients do not get through.  `given`: the gradient
 // and the diagonal part come from the caller, in fp64.
 template <class C>
-__device__ __noinline__ double2 eval_hessian(int m, int n, double hs, int slack, double qstep, int jstride, float amax, float amin,
-                                             double w_own, double ds_own, double rhs, bool given, bool chol, double2 gg, int* flag)
+__device__ __noinline__ double2 eval_hessian(int m, int n, int slack, bool coarse, float amax, float amin, bool given, bool chol,
+                                             double2 gg, int* flag)
 {
     const FSm<C> sm(flag);
     const int tid = threadIdx.x, i = tid % C::MP, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tig = lane & 3;
     Frags<C> fr;
     double g, g2;
+    const double qstep = sm.scal[SC_QSTEP] * (coarse ? 2.0 : 1.0);
+    const int jstride = coarse ? 1 : 2;
+    const double rhs = i < m ? sm.rhs[sm.ord[i]] : 0.0;
     const float zr = i < m ? (float)rhs : 1.f, zi = rsqrtf(zr);
-    if constexpr (C::kContour) eval_contour<C, float, true>(sm, m, slack, qstep, jstride, amax, amin, w_own, i < m ? zi : 0.f, g, g2, fr);
-    else eval_system<C, float, true>(sm, m, n, hs, slack, qstep, jstride, amax, amin, w_own, ds_own, i < m ? zi : 0.f, g, g2, fr);
+    if constexpr (C::kContour) eval_contour<C, float, true>(sm, m, slack, qstep, jstride, amax, amin, sm.wd[i], i < m ? zi : 0.f, g, g2, fr);
+    else eval_system<C, float, true>(sm, m, n, sm.scal[SC_HS], slack, qstep, jstride, amax, amin, sm.wd[i], i < m ? sm.dsd[i] : 0.0, i < m ? zi : 0.f, g, g2, fr);
     if (given) { g = gg.x; g2 = gg.y; }
     if (chol) {
         // an outer block's function is constant along (1,...,1): that direction is pinned with 1/m everywhere
@@ -1021,22 +1091,37 @@ __device__ __noinline__ double2 eval_hessian(int m, int n, double hs, int slack,
         factor<C>(sm, fr, m, add);
     } else {
         // (a diagonal that is not positive gives NaN, which the solve reports)
+        GR_PTR(float) vec = vec_buffer(sm, 0);
         if (tid < C::MP) {
             const float rd = i < m ? rsqrtf((float)(g - g2)) : 1.f;
             sm.dg[i] = rd;
             sm.wf[i] = zr * zi * rd;
+            vec[vec_pos<C>(i)] = i < m ? __fdividef(1.f, rd) : 0.f;
         }
         __syncthreads();
         const int ra = warp % C::kPr, rb = C::MP / 16 - 1 - ra, cs = warp / C::kPr;
         GR_PTR(__half) N = sm.pi;
-        // the lower triangle (and what the diagonal tiles hold beyond it) out of the fragments ...
+        // Both triangles out of the fragments' lower one: an entry and its mirror image.  (Storing one triangle and reading the
+        // other out of its columns afterwards took a barrier and twice the time.)
         auto put = [&](const float* v, int rt, int ni) {
             const int c0 = 8 * ni + 2 * tig, r0 = 16 * rt + gid;
             const float2 sc = ld_f2(sm.wf + c0);
             const float s0 = sm.wf[r0], s1 = sm.wf[r0 + 8];
-            GR_PTR(__half) q = N + r0 * C::kNS + c0;
-            st_h2(q, pack_half(v[0] * s0 * sc.x, v[1] * s0 * sc.y));
-            st_h2(q + 8 * C::kNS, pack_half(v[2] * s1 * sc.x, v[3] * s1 * sc.y));           // (eight rows further)
+            const float e[4] = {v[0] * s0 * sc.x, v[1] * s0 * sc.y, v[2] * s1 * sc.x, v[3] * s1 * sc.y};
+#pragma unroll
+            for (int z = 0; z < 2; z++) {
+                const int r = r0 + 8 * z;                       // (eight rows further)
+                const uint32_t h = pack_half(e[2 * z], e[2 * z + 1]);
+                if (ni < 2 * rt) st_h2(N + r * C::kNS + c0, h);
+                else {
+                    // a tile on the diagonal: what lies above belongs to the mirror images, the diagonal itself is zero
+                    if (c0 < r) N[r * C::kNS + c0] = __ushort_as_half((unsigned short)h);
+                    if (c0 + 1 < r) N[r * C::kNS + c0 + 1] = __ushort_as_half((unsigned short)(h >> 16));
+                    if (c0 == r || c0 + 1 == r) N[r * C::kNS + r] = __ushort_as_half((unsigned short)0);
+                }
+                if (c0 < r) N[c0 * C::kNS + r] = __ushort_as_half((unsigned short)h);
+                if (c0 + 1 < r) N[(c0 + 1) * C::kNS + r] = __ushort_as_half((unsigned short)(h >> 16));
+            }
         };
 #pragma unroll
         for (int s = 0; s < C::kNB; s++) {
@@ -1045,167 +1130,105 @@ __device__ __noinline__ double2 eval_hessian(int m, int n, double hs, int slack,
             if (ni <= 2 * rb + 1) put(fr.B[s], rb, ni);
         }
         __syncthreads();
-        // ... and every row's upper part out of its column (eight entries at a time; what other threads rewrite meanwhile in
-        // the lower triangle does not change)
-#pragma unroll 2
-        for (int c = tid / C::MP; c < C::MP / 8; c += C::kNG) {
-            GR_PTR(__half) own = N + i * C::kNS + 8 * c;
-            const uint4 o = ld_h8(own);
-            const uint32_t ov[4] = {o.x, o.y, o.z, o.w};
-            uint32_t nv[4];
-#pragma unroll
-            for (int z = 0; z < 4; z++) {
-                const int l = 8 * c + 2 * z;
-                const uint32_t t0 = __half_as_ushort(N[l * C::kNS + i]), t1 = __half_as_ushort(N[(l + 1) * C::kNS + i]);
-                const uint32_t e0 = l == i ? 0u : (l > i ? t0 : (ov[z] & 0xffffu));
-                const uint32_t e1 = l + 1 == i ? 0u : (l + 1 > i ? t1 : (ov[z] >> 16));
-                nv[z] = e0 | (e1 << 16);
-            }
-            st_h8(own, make_uint4(nv[0], nv[1], nv[2], nv[3]));
-        }
-        __syncthreads();
+        // row sums of |H| less the diagonal, for the diagonal that cg_solve sets
+        const float nrow = row_times<C>(N, vec);
+        if (tid % C::kNG == 0) sm.Ld[tid / C::kNG] = nrow;
     }
     double2 r; r.x = g; r.y = g2;
     return r;
 }
 
-// sums of up to three values over the token threads
-template <class C, int K>
-__device__ __forceinline__ void tok_sums(const FSm<C>& sm, float* v, int& par)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-        for (int k = 0; k < K; k++) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-    }
-    if (C::T == 32) return;
-    GR_PTR(float) r = GR_PCAST(float, sm.red + 32 * par);
-    par ^= 1;
-    if ((threadIdx.x & 31) == 0 && (threadIdx.x >> 5) < C::kTW)
-        st_f4(r + 4 * (threadIdx.x >> 5), make_float4(v[0], K > 1 ? v[K > 1 ? 1 : 0] : 0.f, K > 2 ? v[K > 2 ? 2 : 0] : 0.f, 0.f));
-    __syncthreads();
-#pragma unroll
-    for (int w = 0; w < C::kTW; w++) {
-        const float4 t = ld_f4(r + 4 * w);
-        const float tv[3] = {t.x, t.y, t.z};
-#pragma unroll
-        for (int k = 0; k < K; k++) v[k] = w == 0 ? tv[k] : v[k] + tv[k];
-    }
-}
-
-// Newton step by conjugate gradients on the scaled Hessian: this thread's component of the step, or NaN when the residual
-// did not fall by `rtol` in kFCgMax iterations.  Off the heavy-weight regime the scaled Hessian has all its eigenvalues
-// within 0.8 - 1.5 but one, so four or five iterations give four digits: 2 k cycles against 18 k for a 50 x 50
-// factorisation with its substitutions.  One thread per row, the row in registers; one reduction per iteration
-// (Chronopoulos and Gear's form).
+// Newton step by conjugate gradients on the scaled Hessian; the step of token i is left in sm.yv[i], NaN when the residual did
+// not fall by `rtol` in kFCgMax iterations.  Off the heavy-weight regime the scaled Hessian has all its eigenvalues
+// within 0.8 - 1.5 but one, so four or five iterations give four digits.
+// One thread per row (or share of a row), the row in registers; the pipelined form of the method (Ghysels and Vanroose), in which
+// the scalar products of an iteration do not wait for its matrix product: one barrier each, where Chronopoulos and Gear's form
+// with the shares summed through shared memory had three.  (50 tokens to 2e-4, one CTA alone: 3.76 k cycles, 3.87 k before; what it saves is barriers for the CTAs beside it.)
 // The one eigenvalue is the common scale of the weights, the direction (1,...,1): H 1 = s, s_i = g2_i / w_i the rate at
 // which token i takes mass from the slack, tiny when the acceptance is close to one.  s is known exactly, so the diagonal
-// is set from the row sums, s_i + sum_l |H_il| (whatever the rounding of the off-diagonal part, the matrix then has the
+// is set from the row sums (sm.Ld), s_i + sum_l |H_il| (whatever the rounding of the off-diagonal part, the matrix then has the
 // right action on that direction), and the direction itself is deflated: the iteration works on
 // (I - s 1^T / sum s) H, and the step gets `shift`, the caller's answer for the common scale, less s . y / sum s.
 // (kap = -1 / sum s, lin = sum rhs / sum s.)
 // An outer block (slack == 0) has s = 0: the matrix is singular along the direction, e e^T / (e . e) is added, e = sqrt(H_ii)
 // (kap = 1 / (e . e), lin = 0).
+// In: sm.yv right-hand side, sm.dl s, visible to all.
 template <class C>
-__device__ __noinline__ float cg_solve(int m, int slack, float rhs, float s_own, float kap, float lin, float shift, float rtol,
-                                       int* flag)
+__device__ __noinline__ void cg_solve(int m, int slack, float kap, float lin, float shift, float rtol, int* flag)
 {
-    constexpr int kCol = C::MP / C::kNG;                        // columns of this copy
+    constexpr int kCol = C::MP / C::kNG;                        // columns of this share
     const FSm<C> sm(flag);
-    const int tid = threadIdx.x, i = tid % C::MP, ng = tid / C::MP;
-    int par = 0;
-    const float sd = sm.dg[i];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, i = tid / C::kNG;
+    const bool on = i < m, lead = tid % C::kNG == 0;
+    const float sd = sm.dg[i], rhs = sm.yv[i];
     float row[kCol];
-    {
-        GR_PTR(const __half) np = sm.pi + i * C::kNS + ng * kCol;
-#pragma unroll
-        for (int c = 0; c < kCol; c += 8) {
-            const uint4 v = ld_h8(np + c);
-            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int z = 0; z < 4; z++) {
-                const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[z]));
-                row[c + 2 * z] = f.x; row[c + 2 * z + 1] = f.y;
-            }
-        }
-    }
-    const bool on = i < m;
-    GR_PTR(float) part = GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oSP), C::T, flag);
-    // N times the vector in `vec` (the caller has written its own entry)
-    auto times_n = [&](GR_PTR(float) vec) {
-        __syncthreads();
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll
-        for (int c = 0; c < kCol; c += 4) {
-            const float4 v = ld_f4(vec + ng * kCol + c);
-            a0 = fmaf(row[c], v.x, a0); a1 = fmaf(row[c + 1], v.y, a1); a2 = fmaf(row[c + 2], v.z, a2); a3 = fmaf(row[c + 3], v.w, a3);
-        }
-        float nv = (a0 + a1) + (a2 + a3);
-        if (C::kNG > 1) {
-            part[tid] = nv;
-            __syncthreads();
-            nv = 0.f;
-#pragma unroll
-            for (int k = 0; k < C::kNG; k++) nv += part[k * C::MP + i];
-        }
-        return nv;
-    };
+    load_row<C>(sm.pi, row);
     // diagonal from the row sums; v: the deflated (slack) or added (outer block) direction, kap its factor
-    const float sdi = on ? __fdividef(1.f, sd) : 0.f;
-    if (ng == 0) sm.yv[i] = sdi;
-    const float nrow = times_n(sm.yv);
-    const float si = on && slack ? s_own : 0.f;
-    const float diag = on ? sd * fmaf(si, sd, nrow) : 1.f;
-    const float v = slack ? si * sd : sdi;
-    float r = on ? rhs * sd : 0.f, x = 0.f, p = 0.f, s = 0.f;
-    r = fmaf(-lin, v, r);
-    float gam_old = 0.f, al_old = 0.f, goal = 0.f;
+    const float si = on && slack ? sm.dl[i] : 0.f;
+    const float diag = on ? sd * fmaf(si, sd, sm.Ld[i]) : 1.f;
+    const float v = slack ? si * sd : (on ? __fdividef(1.f, sd) : 0.f);
+    float r = on ? fmaf(-lin, v, rhs * sd) : 0.f, x = 0.f, p = 0.f, s = 0.f, z = 0.f, w = 0.f;
+    float gam_old = 1.f, al_old = 1.f, goal = 0.f, vp = 0.f, vx = 0.f;
     bool done = false;
+    // (the quadrature nodes' arrays, which only evaluations use, take the warps' sums: tok_reduce's may still be read)
+    static_assert(2 * C::kW * 16 <= 2 * kQC * 8, "warp sums");
+    GR_PTR(float) sums = GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oTq), 4 * kQC, flag);
 #pragma unroll 1
-    for (int it = 0; it <= kFCgMax; it++) {
-        GR_PTR(float) vec = (it & 1) ? sm.yv : sm.dl;            // two buffers in turn
-        if (ng == 0) vec[i] = r;
-        float w = fmaf(diag, r, -times_n(vec));
-        float d[3] = {r * r, r * w, v * r};
-        tok_sums<C, 3>(sm, d, par);
-        w = fmaf(v, kap * d[2], w);
-        d[1] = fmaf(d[2] * d[2], kap, d[1]);
+    for (int it = -1; it <= kFCgMax; it++) {
+        // products r.r, w.r, v.w, v.r (the first time v.r alone counts) over the rows, and w (r) for the matrix product
+        GR_PTR(float) vec = vec_buffer(sm, it & 1);
+        const float in = it < 0 ? r : w;
+        if (lead) vec[vec_pos<C>(i)] = in;
+        float d[4] = {r * r, w * r, v * w, v * r};
+        __syncwarp();
+#pragma unroll
+        for (int o = C::kNG; o < 32; o <<= 1) {
+#pragma unroll
+            for (int k = 0; k < 4; k++) d[k] += __shfl_xor_sync(0xffffffffu, d[k], o);
+        }
+        GR_PTR(float) part = sums + 4 * C::kW * (it & 1);
+        if (lane == 0) st_f4(part + 4 * warp, make_float4(d[0], d[1], d[2], d[3]));
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < C::kW; u++) {
+            const float4 t = ld_f4(part + 4 * u);
+            const float tv[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+            for (int k = 0; k < 4; k++) d[k] = u == 0 ? tv[k] : d[k] + tv[k];
+        }
+        const float q = fmaf(v, kap * (it < 0 ? d[3] : d[2]), fmaf(diag, in, -dot_row<C>(row, vec)));
+        if (it < 0) { w = q; continue; }
         const float gam = d[0];
         if (it == 0) goal = gam * rtol * rtol;
         if (gam <= goal) { done = true; break; }
         const float beta = it == 0 ? 0.f : __fdividef(gam, gam_old);
         const float al = __fdividef(gam, it == 0 ? d[1] : d[1] - beta * __fdividef(gam, al_old));
-        p = fmaf(beta, p, r); s = fmaf(beta, s, w);
-        x = fmaf(al, p, x); r = fmaf(-al, s, r);
+        z = fmaf(beta, z, q); s = fmaf(beta, s, w); p = fmaf(beta, p, r); vp = fmaf(beta, vp, d[3]);
+        x = fmaf(al, p, x); r = fmaf(-al, s, r); w = fmaf(-al, z, w); vx = fmaf(al, vp, vx);
         gam_old = gam; al_old = al;
     }
     float y = x * sd;
-    if (slack) {
-        float sy[1] = {si * y};
-        tok_sums<C, 1>(sm, sy, par);
-        y += shift + kap * sy[0];
-    }
-    __syncthreads();
+    if (slack) y += shift + kap * vx;
     // (not positive definite, NaN or slow: NaN)
-    return done ? y : __int_as_float(0x7fc00000);
+    if (lead) sm.yv[i] = done ? y : __int_as_float(0x7fc00000);
+    if (C::kNG > 1) __syncthreads();
 }
 
-// One system: m tokens at support positions ord[0 .. m) (draft mass ascending), draft mass above the block.
-struct System { int m, slack; double hmass; };
-
-// Starting point (log-weight of this thread's token): token i wins the share w_i / (slack + w_i + S_i) of the tuples that contain it, S_i = the
+// Starting point (log-weights, left in sm.yv): token i wins the share w_i / (slack + w_i + S_i) of the tuples that contain it, S_i = the
 // weight it is up against.  A competitor j, present with probability pi_ij = Pr[i and j drafted] / Pr[i drafted],
 // adds to S_i the weight e_j for which 1 / (A + e_j) = (1 - pi_ij) / A + pi_ij / (A + w_j), A = slack + w_i + S_i:
 // e_j = A pi_ij / (A / w_j + 1 - pi_ij).  For w_j << A this is the mean-field value pi_ij w_j; a huge w_j counts for
 // A pi_ij / (1 - pi_ij) only (token i simply loses the tuples that contain j).  fp32: it is a starting point.
+// Rows and shares of columns as in the matrix products above (one barrier a sweep; three before).
 template <class C>
-__device__ __noinline__ double start_point(int m, int slack, int n, double d_i, double rhs_i, double Tm,
-                                           int* flag)
+__device__ __noinline__ void start_point(int m, int slack, int n, double Tm, int* flag)
 {
+    constexpr int kCol = C::MP / C::kNG;
     const FSm<C> sm(flag);
-    const int tid = threadIdx.x, i = tid % C::MP, ng = tid / C::MP;
-    const bool on = i < m, lead = ng == 0;
-    int par = 0;
+    const int tid = threadIdx.x, i = tid / C::kNG, share = tid % C::kNG;
+    const bool on = i < m, lead = share == 0;
+    const int pos = on ? sm.ord[i] : 0;
+    const double rhs_i = on ? sm.rhs[pos] : 0.0, d_i = on ? sm.d[pos] : 0.0;
     // masses relative to the system's total: token avoided / a pair avoided, (1 - d_i / T)^n and (1 - (d_i + d_j) / T)^n
     const double iT = m_div(1.0, Tm);
     const float fn = (float)n, rel = (float)(d_i * iT);
@@ -1217,105 +1240,118 @@ __device__ __noinline__ double start_point(int m, int slack, int n, double d_i, 
     // a rarely drafted token: Pr[j drafted | i drafted] tends to 1 - (1 - d_j / T)^(n - 1)
     const bool rare = ci < 0.02f;
     const float pres = 1.f - (rel < 1.f ? __fdividef(col, 1.f - rel) : 0.f);
-    RSm<C, float> rf(sm);
-    GR_PTR(float) tab = rf.SP;
-    if (lead) { st_f4(tab + 4 * i, make_float4(rel, col, pres, 0.f)); sm.wf[i] = __fdividef(1.f, wi); }
+    // (the table behind the vectors)
+    GR_PTR(float) tab = GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oPP), 4 * C::MP, sm.flag);
+    static_assert(4 * C::MP * 4 <= C::kPPBytes + C::T * 16, "start table");
+    if (lead) { st_f4(tab + 4 * i, make_float4(rel, col, pres, 0.f)); vec_buffer(sm, 0)[vec_pos<C>(i)] = __fdividef(1.f, wi); }
     __syncthreads();
-    // (eight columns at a time: their chains overlap; columns beyond m hold 0)
-    GR_PTR(__half) prow = sm.pi + i * C::kNS;
-    const int nc = (m + 7) >> 3;
-    if ((i & ~31) < m) {
+    // (eight columns at a time: their chains overlap; columns beyond m hold 0.  A share of up to 32 columns stays in registers)
+    constexpr bool kRegs = kCol <= 32;
+    GR_PTR(__half) prow = sm.pi + i * C::kNS + share * kCol;
+    const int nc = min(kCol, (max(0, m - share * kCol) + 7) & ~7) >> 3;
+    float preg[kRegs ? kCol : 1];
+    auto presence = [&](int j) {
+        const float4 tj = ld_f4(tab + 4 * j);
+        const float both = ex2_approx(fn * __log2f(fmaxf(1.f - rel - tj.x, 0.f)));
+        const float pij = rare ? tj.z : (1.f - col - tj.y + both) * ic;
+        return (j == i || j >= m) ? 0.f : fminf(fmaxf(pij, 0.f), 1.f);
+    };
+    if constexpr (kRegs) {
+#pragma unroll
+        for (int c = 0; c < kCol; c++) preg[c] = 0.f;
+#pragma unroll
+        for (int c = 0; c < kCol; c += 8) {
+            if (c < 8 * nc) {
+#pragma unroll
+                for (int z = 0; z < 8; z++) preg[c + z] = presence(share * kCol + c + z);
+            }
+        }
+    } else if (on) {
 #pragma unroll 1
-        for (int c = ng; c < nc; c += C::kNG) {
+        for (int c = 0; c < nc; c++) {
             uint32_t pk[4];
 #pragma unroll
             for (int z = 0; z < 4; z++) {
-                float pv[2];
-#pragma unroll
-                for (int y = 0; y < 2; y++) {
-                    const int j = 8 * c + 2 * z + y;
-                    const float4 tj = ld_f4(tab + 4 * j);
-                    const float both = ex2_approx(fn * __log2f(fmaxf(1.f - rel - tj.x, 0.f)));
-                    const float pij = rare ? tj.z : (1.f - col - tj.y + both) * ic;
-                    pv[y] = (j == i || j >= m) ? 0.f : fminf(fmaxf(pij, 0.f), 1.f);
-                }
-                const __half2 h = __floats2half2_rn(pv[0], pv[1]);
+                const __half2 h = __floats2half2_rn(presence(share * kCol + 8 * c + 2 * z), presence(share * kCol + 8 * c + 2 * z + 1));
                 pk[z] = *reinterpret_cast<const uint32_t*>(&h);
             }
             st_h8(prow + 8 * c, make_uint4(pk[0], pk[1], pk[2], pk[3]));
         }
     }
-    __syncthreads();
+    // (a thread reads back what it wrote)
     float A = (slack ? 1.f : 0.f) + wi;
-    GR_PTR(float) part = GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oSP), C::T, sm.flag);
 #pragma unroll 1
     for (int sweep = 0; sweep < kFSweeps; sweep++) {
+        GR_PTR(const float) inv = vec_buffer(sm, sweep & 1) + share * (kCol + 4);
         float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        if ((i & ~31) < m) {
+        auto group = [&](int c, const float* pv) {
+            const float4 w0 = ld_f4(inv + 8 * c), w1 = ld_f4(inv + 8 * c + 4);
+            const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+#pragma unroll
+            for (int z = 0; z < 8; z++) acc[z >> 1] += __fdividef(pv[z], fmaf(A, wv[z], 1.f - pv[z]));
+        };
+        if constexpr (kRegs) {
+#pragma unroll
+            for (int c = 0; c < kCol / 8; c++) if (c < nc) group(c, preg + 8 * c);
+        } else if (on) {
 #pragma unroll 2
-            for (int c = ng; c < nc; c += C::kNG) {
+            for (int c = 0; c < nc; c++) {
                 const uint4 pk = ld_h8(prow + 8 * c);
-                const float4 w0 = ld_f4(sm.wf + 8 * c), w1 = ld_f4(sm.wf + 8 * c + 4);
                 const uint32_t u[4] = {pk.x, pk.y, pk.z, pk.w};
-                const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+                float pv[8];
 #pragma unroll
                 for (int z = 0; z < 4; z++) {
-                    const float2 pv = __half22float2(*reinterpret_cast<const __half2*>(&u[z]));
-                    acc[z] += __fdividef(pv.x, fmaf(A, wv[2 * z], 1.f - pv.x));
-                    acc[z] += __fdividef(pv.y, fmaf(A, wv[2 * z + 1], 1.f - pv.y));
+                    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&u[z]));
+                    pv[2 * z] = f.x; pv[2 * z + 1] = f.y;
                 }
+                group(c, pv);
             }
         }
-        float Si = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-        if (C::kNG > 1) {
-            part[tid] = Si;
-            __syncthreads();
-            Si = 0.f;
-#pragma unroll
-            for (int k = 0; k < C::kNG; k++) Si += part[k * C::MP + i];
-        }
-        Si *= A;
+        const float Si = share_sum<C>((acc[0] + acc[1]) + (acc[2] + acc[3])) * A;
         if (on) {
             wi = odds * (slack ? 1.f + Si : fmaxf(Si, 1e-30f));
             A = (slack ? 1.f : 0.f) + wi + Si;
         }
-        __syncthreads();
-        if (lead && on) sm.wf[i] = __fdividef(1.f, wi);
-        __syncthreads();
+        if (sweep + 1 < kFSweeps) {
+            if (lead) vec_buffer(sm, (sweep + 1) & 1)[vec_pos<C>(i)] = __fdividef(1.f, wi);
+            __syncthreads();
+        }
     }
-    double alpha = on ? (double)__logf(wi) : 0.0;
-    if (!slack) {
-        const double mean = tok_sum<C>(sm, on ? alpha : 0.0, par) / (double)m;
-        if (on) alpha -= mean;
-    }
-    return fmin(fmax(alpha, -kFAlphaClamp), kFAlphaClamp);
+    if (lead) sm.yv[i] = on ? __logf(wi) : 0.f;
+    __syncthreads();
 }
 
-// Newton iteration for one system.  Returns the status; w_out = exp(alpha) of this thread's token at the last accepted point.
+// Newton iteration for one system.  Returns the status; sm.wd receives exp(alpha) at the last accepted point, the scalars the
+// gradient norm and the number of evaluations.  Out of line, with what it does not change in shared memory: inlined into the
+// kernel it had 600 to 1000 bytes of spills, which did not fit the first-level cache beside the shared memory and cost
+// more than the evaluations' arithmetic (the same scalar code took three times as long as in the variant without them).
 template <class C>
-__device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, const typename CircleOf<C::kContour>::type& circle,
-                                           int n, double sigma, double tol, int max_iters,
-                                           double qstep, double* gnorm, int* iters, double* w_out)
+__device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, int max_iters,
+                                        const typename CircleOf<C::kContour>::type& circle, int* flag)
 {
+    const FSm<C> sm(flag);
     const int tid = threadIdx.x, i = tid % C::MP;
-    const int m = sy.m, slack = sy.slack;
     const bool on = i < m, lead = tid < C::MP;
     int par = 0;
+    float t0;                // the slack's share of the mass at the solution
+    bool dominant;           // one token has most of the mass
+    {
     const int pos = on ? sm.ord[i] : 0;
-    const double rhs_i = on ? sm.rhs[pos] : 0.0, d_i = on ? sm.d[pos] : 0.0, ds_i = d_i * sigma;
-    double dmax = d_i, Tm = d_i;
-    tok_max_sum<C>(sm, dmax, Tm, par);
-    Tm += sy.hmass;
-    // mass of the tuples the system serves, and the slack's share of it at the solution
+    const double d_i = on ? sm.d[pos] : 0.0, ds_i = d_i * sm.scal[SC_SIGMA];
+    double tot[2] = {d_i, on ? sm.rhs[pos] : 0.0};
+    tok_reduce<C, 2, 0, 0>(sm, tot, nullptr, nullptr, par);
+    const double Tm = tot[0] + hmass;
+    // mass of the tuples the system serves
     const double Tn = ipow(Tm, n);
-    const float t0 = slack ? (float)(Tn - tok_sum<C>(sm, rhs_i, par)) : 0.f;
-    const double hs = sy.hmass * sigma;
+    t0 = slack ? (float)(Tn - tot[1]) : 0.f;
+    dominant = !(sm.d[sm.ord[m - 1]] < 0.6 * Tm);       // (ascending draft mass: the last is the largest)
+    if (tid == 0) { sm.scal[SC_HS] = hmass * sm.scal[SC_SIGMA]; sm.scal[SC_TN] = Tn; }
 
-    double alpha = start_point<C>(m, slack, n, d_i, rhs_i, Tm, sm.flag);
+    start_point<C>(m, slack, n, Tm, sm.flag);
     // scaled draft masses (and at short series their powers) for the evaluations
     if constexpr (C::kContour) {
         const double iT = m_div(1.0, Tm);
-        contour_tables<C>(circle, m, d_i * iT, sy.hmass * iT, Tn, sm.flag);
+        contour_tables<C>(circle, m, d_i * iT, hmass * iT, Tn, sm.flag);
     } else if (lead) {
         sm.dsd[i] = ds_i;
         RSm<C, float> rs(sm);
@@ -1328,14 +1364,24 @@ __device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, c
         }
     }
 
-    double alpha_prev = alpha, delta = 0.0, g = 0.0, g2 = 0.0;
+    }
+    double alpha = on ? (double)sm.yv[i] : 0.0;
+    if (!slack) {
+        const double mean = tok_sum<C>(sm, alpha, par) / (double)m;
+        if (on) alpha -= mean;
+    }
+    alpha = fmin(fmax(alpha, -kFAlphaClamp), kFAlphaClamp);
+    double alpha_prev = alpha;
     int status = GR_NOT_CONVERGED, it = 0, stalls = 0, was_kind = -1;
-    double rn = 0.0, rprev = 1.0e300, lam = 1.0, dist = 0.0;
+    double rn = 0.0;
+    float rprev = kFNone, lam = 1.f, dist = 0.f;
+    float amax = 0.f, amin = 0.f;            // extreme log-weights
+    bool ranged = false;                     // they are known for this point
     // Three modes.  Low: gradient and Hessian in fp32, conjugate gradients.  Chord: fp64 gradient, the last Hessian.  High:
     // fp64 gradient, fp32 Hessian of the same point, with `chol` a Cholesky factorisation.  A single token that dominates a
     // long series (its terms would cancel in fp32) starts in the last mode.
     enum { kLow, kChord, kHigh };
-    int mode = (C::NT <= 8 || C::kContour || dmax < 0.6 * Tm) ? kLow : kHigh;
+    int mode = (C::NT <= 8 || C::kContour || !dominant) ? kLow : kHigh;
     bool full_grid = false, predicted = false, chol = false;
 #pragma unroll 1
     for (; it < max_iters; it++) {
@@ -1345,17 +1391,28 @@ __device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, c
         const int kind = 2 * mode + (coarse ? 1 : 0);
         const double w_i = !on ? 0.0 : (mode == kLow ? (double)__expf((float)alpha) : m_exp(alpha));
         if (lead) { sm.wd[i] = w_i; sm.wf[i] = (float)w_i; }
-        float amax, amin;
-        tok_range<C>(sm, (float)alpha, on, amax, amin, par);
-        const double qs = coarse ? 2.0 * qstep : qstep;
+        if (!ranged) {
+            unsigned ext[2] = {on ? fkey((float)alpha) : 0u, on ? fkey(-(float)alpha) : 0u};
+            tok_reduce<C, 0, 0, 2>(sm, nullptr, nullptr, ext, par);
+            amax = fkey_inv(ext[0]); amin = -fkey_inv(ext[1]);
+        }
+        ranged = false;
+        __syncthreads();
         double2 gg = make_double2(0.0, 0.0);
-        if (mode != kLow) gg = eval_fp64<C>(m, n, hs, slack, qs, amax, amin, w_i, ds_i, sm.flag);
+        if (mode != kLow) gg = eval_fp64<C>(m, n, slack, coarse, amax, amin, sm.flag);
+        if (mode == kHigh) __syncthreads();          // (sum_copies' array)
         if (mode != kChord)
-            gg = eval_hessian<C>(m, n, hs, slack, qs, coarse ? 1 : 2, amax, amin, w_i, ds_i, rhs_i, mode == kHigh, chol, gg, sm.flag);
-        g = gg.x; g2 = gg.y;
-        const double2 rg = tok_max_sum_fn<C>(on ? g : 0.0, on ? fabs(g - rhs_i) : 0.0, true, par, sm.flag);
-        par ^= 1;
-        rn = rg.y;
+            gg = eval_hessian<C>(m, n, slack, coarse, amax, amin, mode == kHigh, chol, gg, sm.flag);
+        const double g = gg.x, g2 = gg.y, rhs_i = on ? sm.rhs[sm.ord[i]] : 0.0, tol = sm.scal[SC_TOL];
+        // The residual, and what the step below needs of the tokens: right-hand side b of the Newton system, s_i = g2_i / w_i,
+        // and the sums of b, s and the Hessian's diagonal.
+        const float b = on ? newton_rhs(g, g2, rhs_i) : 0.f, s_i = on ? __fdividef((float)g2, (float)sm.wd[i]) : 0.f;
+        if (!chol && lead) { sm.yv[i] = b; sm.dl[i] = s_i; }
+        double rg[2] = {on ? g : 0.0, on ? fabs(g - rhs_i) : 0.0};
+        float sums[3] = {b, slack ? s_i : 0.f, on ? (float)(g - g2) : 0.f};
+        tok_reduce<C, 2, 3, 0>(sm, rg, sums, nullptr, par);
+        if (C::kTW == 1) __syncthreads();
+        rn = rg[1];
         // (residuals are only compared within one grid and one precision)
         const bool comparable = kind == was_kind && it > 0;
         was_kind = kind;
@@ -1372,10 +1429,10 @@ __device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, c
             high = !(rn <= 1.0e-3) || (comparable && !(rn < 0.3 * rprev));
         } else if (comparable && !(rn < rprev)) {
             if (mode == kLow && rn < kFLowFloor) high = true;          // at the noise of fp32
-            else if (lam > 1.0 / 64.0) {
+            else if (lam > 1.f / 64.f) {
                 // the last step did not reduce the gradient norm: retry it at half length
-                lam *= 0.5;
-                alpha = alpha_prev + lam * delta;
+                lam *= 0.5f;
+                alpha = alpha_prev + 0.5 * (alpha - alpha_prev);
                 continue;
             } else if (mode == kLow) {
                 high = true; alpha = alpha_prev;
@@ -1386,56 +1443,49 @@ __device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, c
                 if (chol && ++stalls >= 2) { alpha = alpha_prev; break; }
                 if (!chol) {
                     // (the last accepted point once more: this one has no factorisation)
-                    chol = true; alpha = alpha_prev; rprev = 1.0e300; lam = 1.0; was_kind = -1;
+                    chol = true; alpha = alpha_prev; rprev = kFNone; lam = 1.f; was_kind = -1;
                     continue;
                 }
             }
         }
-        if (high) { mode = kHigh; full_grid = true; rprev = 1.0e300; lam = 1.0; was_kind = -1; continue; }
+        if (high) { mode = kHigh; full_grid = true; rprev = kFNone; lam = 1.f; was_kind = -1; continue; }
         // contraction of the last full step (same grid and precision on both sides)
-        const double rho = (comparable && !coarse && lam == 1.0) ? rn / rprev : 1.0e300;
-        rprev = rn; lam = 1.0;
+        const float rho = (comparable && !coarse && lam == 1.f) ? __fdividef((float)rn, rprev) : kFNone;
+        rprev = (float)rn; lam = 1.f;
         alpha_prev = alpha;
         // Newton step
         double dl;
         bool fail = false;
         float pivot = 1.f;
-        double jump = 0.0;               // part of the step that is a common shift, not subject to the clamp
+        float jump = 0.f;                // part of the step that is a common shift, not subject to the clamp
         if (!chol) {
             // The common scale of the weights.  The slack's share g0 = T^n - sum g is, along that scale, a falling logistic
             // curve whose slope is sum s; where its target t0 is far below (acceptance close to one), the curve is inverted
             // exactly, as the tokens' own curves are in newton_rhs: a Newton step would move the scale by one at most.
-            const float b = on ? newton_rhs(g, g2, rhs_i) : 0.f, s_i = on ? __fdividef((float)g2, (float)w_i) : 0.f;
             float shift = 0.f;
-            float sums[3] = {b, slack ? s_i : 0.f, on ? (float)(g - g2) : 0.f};
-            tok_sums<C, 3>(sm, sums, par);
             const float lin = slack ? __fdividef(sums[0], sums[1]) : 0.f;
             if (slack) {
-                const float g0 = (float)(Tn - rg.x), slope = sums[1];
+                const double Tn = sm.scal[SC_TN];
+                const float g0 = (float)(Tn - rg[0]), slope = sums[1];
                 shift = lin;
                 pivot = __fdividef(slope, sums[2]);                 // of the order of the smallest relative pivot
                 float far = 0.f;
                 if (g0 < kFSmallSlack * (float)Tn) {
                     // too small a difference for fp32; the slope, a sum of positive terms, is the share itself there
                     far = __logf(__fdividef(fmaxf(slope, 1.0e-30f), fmaxf(t0, kFLeastSlack * (float)Tn)));
-                    if (mode == kLow || fabsf(far) > kFScaleJump) { shift = fminf(fmaxf(far, -16.f), 16.f); jump = (double)shift; }
+                    if (mode == kLow || fabsf(far) > kFScaleJump) { shift = fminf(fmaxf(far, -16.f), 16.f); jump = shift; }
                 } else if (t0 > 0.f && g0 > slope) {
                     // saturation level c0 from value and slope:  slope = g0 (1 - g0 / c0)
                     const float inv = __fdividef(g0 - slope, g0 * g0);                // 1 / c0
                     const float q = __fdividef(g0 * (1.f - t0 * inv), t0 * (1.f - g0 * inv));
                     far = q > 0.f ? __logf(q) : 0.f;
-                    if (far > kFScaleJump) { shift = fminf(far, 16.f); jump = (double)shift; }
+                    if (far > kFScaleJump) { shift = fminf(far, 16.f); jump = shift; }
                 }
             }
-            const float step = cg_solve<C>(m, slack, b, s_i, slack ? -__fdividef(1.f, sums[1]) : __fdividef(1.f, sums[2]), lin, shift, kFCgTol, sm.flag);
-
-            // (NaN for every thread or none: the iteration's scalars are common)
-            if (__syncthreads_or(!(step == step))) {
-                // badly conditioned: the same point again with an fp64 gradient and a factorisation
-                mode = kHigh; chol = true; full_grid = true; rprev = 1.0e300; was_kind = -1;
-                continue;
-            }
-            dl = (double)step;
+            // (far from the solution the step need not be solved to more than the model is worth)
+            const float rtol = mode == kLow ? fminf(fmaxf(kFCgLow * (float)rn, kFCgTol), kFCgLoose) : kFCgTol;
+            cg_solve<C>(m, slack, slack ? -__fdividef(1.f, sums[1]) : __fdividef(1.f, sums[2]), lin, shift, rtol, sm.flag);
+            dl = on ? (double)sm.yv[i] : 0.0;
         } else {
             backward_subst<C>(m, sm.flag);
             __syncthreads();
@@ -1444,19 +1494,29 @@ __device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, c
             dl = on ? (double)sm.dl[i] : 0.0;
             // proportional-fitting step  alpha += log(rhs / g)  (and the full grid from here on)
             if (fail) { full_grid = true; dl = on ? m_log(rhs_i / g) : 0.0; }
-            // (no usable step: the general kernel's)
-            if (__syncthreads_or(!(fabs(dl) < 1.0e300))) break;
         }
         if (!slack) {
             const double mean = tok_sum<C>(sm, dl, par) / (double)m;
             if (on) dl -= mean;
         }
-        double dm = on ? fabs(dl - jump) : 0.0, s2 = on ? g * dl * dl : 0.0;
-        tok_max_sum<C>(sm, dm, s2, par);
+        // largest component, s2 = sum g dl^2 (see below), the extremes of the weights after the step, and whether it is a number
+        double s2 = on ? g * dl * dl : 0.0;
+        const float an = (float)fmin(fmax(alpha + dl, -kFAlphaClamp), kFAlphaClamp);
+        unsigned ext[3] = {on ? __float_as_uint(fabsf((float)(dl - (double)jump))) : 0u, on ? fkey(an) : 0u, on ? fkey(-an) : 0u};
+        tok_reduce<C, 1, 0, 3>(sm, &s2, nullptr, ext, par);
+        const float dm = __uint_as_float(ext[0]), far = dm + fabsf(jump);
+        // (NaN for every thread or none)
+        if (!(s2 < 1.0e300) || !(dm < kFNone)) {
+            if (chol) break;                 // no usable step: the general kernel's
+            // badly conditioned: the same point again with an fp64 gradient and a factorisation
+            mode = kHigh; chol = true; full_grid = true; rprev = kFNone; was_kind = -1;
+            continue;
+        }
+        amax = fkey_inv(ext[1]); amin = -fkey_inv(ext[2]);
+        ranged = !(dm > (float)kFStepClamp);
         // a full Newton step below 1e-11 in alpha: the weights cannot be improved at this quadrature accuracy
-        if (!fail && mode != kLow && dm + fabs(jump) < 1.0e-11) { status = GR_OK; it++; break; }
-        if (dm > kFStepClamp && on) dl = jump + (dl - jump) * (kFStepClamp / dm);
-        delta = dl;
+        if (!fail && mode != kLow && far < 1.0e-11f) { status = GR_OK; it++; break; }
+        if (dm > (float)kFStepClamp && on) dl = jump + (dl - (double)jump) * (double)__fdividef((float)kFStepClamp, dm);
         alpha = fmin(fmax(alpha + dl, -kFAlphaClamp), kFAlphaClamp);
         // Stop on a predicted residual, without another evaluation, after a step from a point evaluated in fp64 on the
         // full grid.  Measured against the oracle's residual at the weights returned, 9500 such stops at tolerances of 1e-8,
@@ -1477,14 +1537,14 @@ __device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, c
         const bool trusted = !fail && pivot > (float)kFTrustPivot;
         if (mode == kLow) {
             // the next point is close enough: fp64 from here on, with this factorisation
-            if (kFPredictBound * s2 < kFLowLeave && dm + fabs(jump) <= 0.1) { mode = trusted ? kChord : kHigh; full_grid = true; dist = dm; }
+            if (kFPredictBound * s2 < kFLowLeave && far <= 0.1f) { mode = trusted ? kChord : kHigh; full_grid = true; dist = dm; }
         } else if (trusted && !coarse) {
-            const double lin = chol ? 0.0 : (kFChordBase + (mode == kChord ? 2.0 * dist : 0.0)) * rn;
-            const double next = fmax(rho, dm + fabs(jump));
-            const bool by_step = dm + fabs(jump) <= kFPredictStep && kFPredictSafety * s2 + 3.0 * lin < tol;
-            const bool by_ratio = rho < 0.1 && dm <= kFStepClamp && kFRatioSafety * next * rn < tol;
+            const float lin = chol ? 0.f : ((float)kFChordBase + (mode == kChord ? 2.f * dist : 0.f)) * (float)rn;
+            const float next = fmaxf(rho, far);
+            const bool by_step = far <= (float)kFPredictStep && kFPredictSafety * s2 + 3.0 * (double)lin < tol;
+            const bool by_ratio = rho < 0.1f && dm <= (float)kFStepClamp && kFRatioSafety * (double)next * rn < tol;
             if (by_step || by_ratio) {
-                rn = by_step ? kFPredictBound * s2 + lin : next * rn;
+                rn = by_step ? kFPredictBound * s2 + (double)lin : (double)next * rn;
                 status = GR_OK; it++;
                 predicted = true;
                 break;
@@ -1493,9 +1553,8 @@ __device__ __forceinline__ int fast_system(const FSm<C>& sm, const System& sy, c
         }
     }
     // (not converged here: the last accepted point, the general kernel's starting point)
-    *w_out = on ? m_exp(status == GR_OK ? alpha : alpha_prev) : 0.0;
-    *gnorm = rn;
-    *iters = it | (predicted ? kItersPredicted : 0);
+    if (lead) sm.wd[i] = on ? m_exp(status == GR_OK ? alpha : alpha_prev) : 0.0;
+    if (tid == 0) { sm.scal[SC_GNORM] = rn; sm.scal[SC_ITERS] = (double)(it | (predicted ? kItersPredicted : 0)); }
     return status;
 }
 
@@ -1511,7 +1570,7 @@ fast_solve_kernel(char* __restrict__ ws, char* __restrict__ params, int pstride,
     GR_CHECK_FLAG_DECL;
     GR_CHECK_FLAG_INIT;
     const bool fused = fa.draft != nullptr;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long b = blockIdx.x;
     char* pb = params + (size_t)b * pstride;
     ParamView pv = view_params(pb, kcap, V, GR_CHECK_FLAG);
@@ -1547,6 +1606,7 @@ fast_solve_kernel(char* __restrict__ ws, char* __restrict__ params, int pstride,
         truncation_sets(ps, sm.trunc, ps.itmp, k, jstar, n, tau);
         tol = 5.0 * tau;
     }
+    if (tid == 0) { sm.scal[SC_TOL] = tol; sm.scal[SC_QSTEP] = qstep; sm.scal[SC_SIGMA] = sigma; }
     // with the drafted tuple at hand only the system it selects is solved
     const int sel = fused ? selected_system(fa.draft + (size_t)b * n, n, k, jstar, ps.id, sm.blk, &s_sel) : -2;
     // the rule's arrays, except the weights of the systems solved below
@@ -1568,17 +1628,26 @@ fast_solve_kernel(char* __restrict__ ws, char* __restrict__ params, int pstride,
 #pragma unroll 1
     while (lo < k && status == GR_OK) {
         const bool inner = lo < jstar;
-        int hi;
         const int bk = sm.blk[lo];
-        if (inner) hi = jstar;
-        else { hi = lo + 1; while (hi < k && sm.blk[hi] == bk) hi++; }
+        int hi = jstar;
+        if (!inner) {
+            // the first position of another block
+            hi = k;
+            for (int j0 = lo + 1; j0 < k; j0 += 32) {
+                const unsigned other = __ballot_sync(0xffffffffu, j0 + lane < k && sm.blk[j0 + lane] != bk);
+                if (other) { hi = j0 + __ffs(other) - 1; break; }
+            }
+        }
         const bool wanted = sel == -2 || (inner ? sel < 0 : sel == bk);
-        if (tid < MP) sm.wf[tid] = tid < k ? (float)sm.d[tid] : 0.f;
-        __syncthreads();
-        // tokens of the system in ascending draft mass (positions break ties; fp32 is enough to order them)
-        const int pos = lo + tid;
-        const bool in = tid < MP && pos < hi && (!trunc || sm.trunc[pos] != 0);
-        const float dv = in ? sm.wf[pos] : 0.f;
+        // tokens of the system in ascending draft mass (fp32 is enough to order them; positions break ties, so that no two keys
+        // are equal; what is not in the truncation set has the key of none)
+        GR_PTR(unsigned long long) okey = GR_PCAST(unsigned long long, sm.wd);
+        unsigned long long mine = 0ull;
+        const bool in = tid < hi - lo && (!trunc || sm.trunc[lo + tid] != 0);
+        if (in) mine = ((unsigned long long)(0x7fffffffu - __float_as_uint((float)sm.d[lo + tid])) << 32) | (unsigned)(MP - tid);
+        if (tid < hi - lo) okey[tid] = mine;
+        const int m = __syncthreads_count(in);
+        if (in) sm.ord[count_above(okey, 0, hi - lo, mine)] = lo + tid;
         double hm = inner ? 0.0 : sm.Dr[lo];
         if (trunc && !inner) {
             // tuples counted: those inside (H* u T)^n, so the mass above the block is drf(H*) plus the T-part of the
@@ -1586,28 +1655,19 @@ fast_solve_kernel(char* __restrict__ ws, char* __restrict__ params, int pstride,
             hm = sm.Dr[jstar];
             for (int j = jstar; j < lo; j++) hm += sm.trunc[j] ? sm.d[j] : 0.0;
         }
-        if (in) {
-            int rank = 0;
-#pragma unroll 4
-            for (int j = lo; j < hi; j++) {
-                const float dj = sm.wf[j];
-                rank += ((!trunc || sm.trunc[j] != 0) && (dj < dv || (dj == dv && j < pos))) ? 1 : 0;
-            }
-            sm.ord[rank] = pos;
-        }
-        const int m = __syncthreads_count(in);
-        if (trunc && !inner && m == 1 && in) pv.w[pos] = 1.0;
+        __syncthreads();
+        const int only = trunc && !inner && m == 1 ? sm.ord[0] : -1;
+        if (only >= 0 && tid == 0) pv.w[only] = 1.0;
         const bool solve = inner ? m > 0 : m >= 2;
         // (a skipped inner system always leaves the rule partial)
         if (!wanted && (solve || inner)) skipped = true;
         if (solve && wanted) {
-            System sy;
-            sy.m = m; sy.slack = inner ? 1 : 0; sy.hmass = hm;
-            double gn, w; int it;
-            const int st = fast_system<C>(sm, sy, circle, n, sigma, tol, max_iters, qstep, &gn, &it, &w);
+            const int st = fast_system<C>(m, inner ? 1 : 0, n, hm, max_iters, circle, ck);
             if (st != GR_OK) status = kNeedFallback;
-            gnorm_total += gn; iters_total = add_iters(iters_total, it);
-            if (tid < m) pv.w[sm.ord[tid]] = w;
+            // (a thread reads back the weight it wrote)
+            if (tid < m) pv.w[sm.ord[tid]] = sm.wd[tid];
+            __syncthreads();
+            gnorm_total += sm.scal[SC_GNORM]; iters_total = add_iters(iters_total, (int)sm.scal[SC_ITERS]);
         }
         __syncthreads();
         lo = hi;
@@ -1636,9 +1696,11 @@ int launch_fast_t(char* ws, char* params, int pstride, int kcap, int V, int n, i
     if (!configured[dev]) {
         if (cudaFuncSetAttribute(fast_solve_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kBytes) != cudaSuccess)
             return GR_E_LAUNCH;
-        // the CTAs are small: ask for the largest shared-memory carve-out so that many of them fit on an SM
-        if (cudaFuncSetAttribute(fast_solve_kernel<C>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+        // as much shared memory as the CTAs that fit an SM use, and no more: the rest is the first-level cache, which the
+        // spills of the out-of-line calls live in
+        constexpr int kTotal = 228 * 1024, kUsed = C::kCtas * (C::kBytes + 1024 + 64);
+        constexpr int kPercent = kUsed >= kTotal ? 100 : (100 * kUsed + kTotal - 1) / kTotal;
+        if (cudaFuncSetAttribute(fast_solve_kernel<C>, cudaFuncAttributePreferredSharedMemoryCarveout, kPercent) != cudaSuccess)
             return GR_E_LAUNCH;
         configured[dev] = true;
     }
