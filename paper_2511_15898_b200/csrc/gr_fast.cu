@@ -9,13 +9,21 @@ namespace gr {
         FusedArgs fa, cudaStream_t st
 namespace fast {
 int launch_fast_n4_m32(GR_FAST_ARGS);
+int launch_fast_n4_m32w(GR_FAST_ARGS);
 int launch_fast_n4_m64(GR_FAST_ARGS);
+int launch_fast_n4_m64w(GR_FAST_ARGS);
 int launch_fast_n8_m32(GR_FAST_ARGS);
+int launch_fast_n8_m32w(GR_FAST_ARGS);
 int launch_fast_n8_m64(GR_FAST_ARGS);
+int launch_fast_n8_m64w(GR_FAST_ARGS);
 int launch_fast_n8_m128(GR_FAST_ARGS);
+int launch_fast_n8_m128w(GR_FAST_ARGS);
 int launch_fast_n16_m32(GR_FAST_ARGS);
+int launch_fast_n16_m32w(GR_FAST_ARGS);
 int launch_fast_n16_m64(GR_FAST_ARGS);
+int launch_fast_n16_m64w(GR_FAST_ARGS);
 int launch_fast_n16_m128(GR_FAST_ARGS);
+int launch_fast_n16_m128w(GR_FAST_ARGS);
 int launch_fast_c24_m32(GR_FAST_ARGS);
 int launch_fast_c24_m64(GR_FAST_ARGS);
 int launch_fast_c24_m128(GR_FAST_ARGS);
@@ -27,23 +35,28 @@ int launch_fast(GR_FAST_ARGS)
 {
     if (kcap <= 0 || kcap > 128 || n < 2) return 1;
 #define GR_FAST_PASS ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol, max_iters, qstep, tau, batch, alpha_out, status_out, fa, st
+    // Twice to four times the threads per instance, and registers without spills, where the batch leaves an SM with one
+    // instance (two of the narrow supports): an instance is a chain of dependent steps then, and 1 row of the headline shape
+    // takes 60 us for 74, 128 rows 62 for 81, 64 whole rows of 16 ids 70 for 77.  Beyond one wave the other variants' places
+    // count for more (1024 headline rows: 300 us in the wide variant, 163 in the other; 512 rows, n = 16, k = 20: 118 and 97).
+    const bool one = batch <= kSms, two = batch <= 2 * kSms;
     if (n > 16) {
         if (kcap <= 32) return fast::launch_fast_c24_m32(GR_FAST_PASS);
         if (kcap <= 64) return fast::launch_fast_c24_m64(GR_FAST_PASS);
         return fast::launch_fast_c24_m128(GR_FAST_PASS);
     }
     if (kcap <= 32) {
-        if (n <= 4) return fast::launch_fast_n4_m32(GR_FAST_PASS);
-        if (n <= 8) return fast::launch_fast_n8_m32(GR_FAST_PASS);
-        return fast::launch_fast_n16_m32(GR_FAST_PASS);
+        if (n <= 4) return two ? fast::launch_fast_n4_m32w(GR_FAST_PASS) : fast::launch_fast_n4_m32(GR_FAST_PASS);
+        if (n <= 8) return two ? fast::launch_fast_n8_m32w(GR_FAST_PASS) : fast::launch_fast_n8_m32(GR_FAST_PASS);
+        return two ? fast::launch_fast_n16_m32w(GR_FAST_PASS) : fast::launch_fast_n16_m32(GR_FAST_PASS);
     }
     if (kcap <= 64) {
-        if (n <= 4) return fast::launch_fast_n4_m64(GR_FAST_PASS);
-        if (n <= 8) return fast::launch_fast_n8_m64(GR_FAST_PASS);
-        return fast::launch_fast_n16_m64(GR_FAST_PASS);
+        if (n <= 4) return one ? fast::launch_fast_n4_m64w(GR_FAST_PASS) : fast::launch_fast_n4_m64(GR_FAST_PASS);
+        if (n <= 8) return one ? fast::launch_fast_n8_m64w(GR_FAST_PASS) : fast::launch_fast_n8_m64(GR_FAST_PASS);
+        return one ? fast::launch_fast_n16_m64w(GR_FAST_PASS) : fast::launch_fast_n16_m64(GR_FAST_PASS);
     }
-    if (n <= 8) return fast::launch_fast_n8_m128(GR_FAST_PASS);
-    return fast::launch_fast_n16_m128(GR_FAST_PASS);
+    if (n <= 8) return one ? fast::launch_fast_n8_m128w(GR_FAST_PASS) : fast::launch_fast_n8_m128(GR_FAST_PASS);
+    return one ? fast::launch_fast_n16_m128w(GR_FAST_PASS) : fast::launch_fast_n16_m128(GR_FAST_PASS);
 }
 
 }  // namespace gr

@@ -6,6 +6,7 @@ import torch
 
 import paper_2511_15898_b200 as G
 from paper_2511_15898_b200 import workloads as W
+from oracle import gr_oracle as O
 from paper_2511_15898_b200.build import build_library
 from tests import parity as P
 
@@ -27,6 +28,27 @@ def test_draft_counts_and_supports_at_the_edges(n, topk):
     assert rep.n_status_ok == rep.n_inst and rep.n_struct_mismatch == 0, (rep.summary(), rep.details[:5])
     assert rep.alpha_err <= 1e-6 and rep.cert_solver_max <= 3.2e-7, rep.summary()
     assert rep.n_underreported == 0 and rep.n_evaluated_off == 0, (rep.summary(), rep.details[:5])
+
+
+@pytest.mark.parametrize("n", [2, 4, 5, 8, 9, 16])
+@pytest.mark.parametrize("topk", [17, 32, 33, 64, 65, 128])
+def test_both_widths_of_a_variant(n, topk):
+    """The number of threads per instance depends on the batch: rows of a batch beyond two waves of SMs against the oracle, and
+    against the same rows in a batch of their own."""
+    wl = W.config3(batch=300, device="cuda", seed=700 + 40 * topk + n, V=2000, n=n, topk=topk)
+    large = G.read_rule(G.solve(wl.q_logits, wl.p_logits, n, topk, wl.temp_target, wl.temp_draft))
+    tt, td = P.oracle_temps(wl)
+    cert = O.certify_batch(W.logits_to_f64(wl.q_logits[:3]), W.logits_to_f64(wl.p_logits[:3]), n, topk, tt, td,
+                           large.w[:3].numpy(), lse=large.lse_target[:3].numpy())
+    assert set(large.status.tolist()) == {G.GR_OK} and float(cert.gnorm_lse.max()) <= 3.2e-7
+    assert abs(large.alpha_star[:3].numpy() - cert.alpha_star).max() <= 1e-6
+    small = G.read_rule(G.solve(wl.q_logits[:100], wl.p_logits[:100], n, topk, wl.temp_target, wl.temp_draft))
+    assert torch.equal(small.ids, large.ids[:100]) and torch.equal(small.flow, large.flow[:100])
+    # (each within 3e-7 of the target in L1: their emitted distributions are within the sum of the two)
+    uni, tok = wl.uniforms, wl.draft_tokens
+    a = G.verify(G.solve(wl.q_logits, wl.p_logits, n, topk, wl.temp_target, wl.temp_draft), tok, uni).token[:100]
+    b = G.verify(G.solve(wl.q_logits[:100], wl.p_logits[:100], n, topk, wl.temp_target, wl.temp_draft), tok[:100], uni[:100]).token
+    assert int((a != b).sum()) <= 1
 
 
 def test_slack_below_fp32():
