@@ -269,6 +269,27 @@ __device__ __forceinline__ double exp_neg(double y)
     return kf < -1000.0 ? 0.0 : __hiloint2double(__double2hiint(p) + (k << 20), __double2loint(p));
 }
 
+// Two fp32 numbers in one 64-bit register pair (sm_100's packed arithmetic: one instruction for both).
+__device__ __forceinline__ float f_lo(unsigned long long v) { return __uint_as_float((unsigned int)v); }
+__device__ __forceinline__ float f_hi(unsigned long long v) { return __uint_as_float((unsigned int)(v >> 32)); }
+__device__ __forceinline__ unsigned long long f_pack(float lo, float hi) {
+    return ((unsigned long long)__float_as_uint(hi) << 32) | __float_as_uint(lo);
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
 // Programmatic dependent launch.  Every kernel of a call is launched with launch_pdl and begins with this: its launch is
 // prepared while the predecessor runs, but it touches no memory until the predecessor has completed (which, by the same
 // rule, had waited for its own).  No kernel lets its successor's CTAs in early (griddepcontrol.launch_dependents): they

@@ -196,6 +196,24 @@ template <> struct Rx<float> {
     static __device__ __forceinline__ float lg(float x) { return __logf(x); }
 };
 
+// Two fp32 numbers (of two tokens or of two quadrature nodes) as one operand of the formulas below.
+struct F2 {
+    unsigned long long v;
+    __device__ __forceinline__ F2() {}
+    __device__ __forceinline__ explicit F2(unsigned long long x) : v(x) {}
+    __device__ __forceinline__ explicit F2(double c) : v(f_pack((float)c, (float)c)) {}
+    __device__ __forceinline__ explicit F2(float c) : v(f_pack(c, c)) {}
+    __device__ __forceinline__ explicit F2(int c) : F2((float)c) {}
+    __device__ __forceinline__ F2(float lo, float hi) : v(f_pack(lo, hi)) {}
+    __device__ __forceinline__ float lo() const { return f_lo(v); }
+    __device__ __forceinline__ float hi() const { return f_hi(v); }
+};
+using ::fma;
+__device__ __forceinline__ F2 fma(F2 a, F2 b, F2 c) { return F2(fma2(a.v, b.v, c.v)); }
+__device__ __forceinline__ F2 operator*(F2 a, F2 b) { return F2(mul2(a.v, b.v)); }
+__device__ __forceinline__ F2 operator+(F2 a, F2 b) { return F2(add2(a.v, b.v)); }
+__device__ __forceinline__ F2 operator-(F2 a, F2 b) { return fma(b, F2(-1.f), a); }
+
 // h[c], c = 1 .. N (N <= 8): coefficients of h(mu; x), from u = 1 - 2x and p = x (1 - x)
 // (closed forms of the Riccati recurrence below).
 template <int N, typename R>
@@ -542,24 +560,47 @@ __device__ __forceinline__ void eval_contour(const FSm<C>& sm, int m, int slack,
     sum_copies<C>(sm, g_out, g2_out);
 }
 
-// Gradient g and the Hessian's diagonal part g2 at the weights in shared memory (this thread's in w_own), in fp64; or in
-// fp32 with kJac, which adds the Hessian's contraction (fragments fr) from every jstride-th node: the off-diagonal entries
-// times z_i z_l, z = rhs^(-1/2) (z_own is this thread's), which keeps the fp16 operands of order one.
+// Node of the quadrature grid at s = s_hi - qstep q, lower tail compressed below s0: t and its weight.
+template <typename R>
+__device__ __forceinline__ R quad_node(float s_hi, float s0, R qstep, int q, R& e)
+{
+    const R s = (R)s_hi - qstep * (R)q;
+    e = Rx<R>::expneg(s - (R)s0);
+    return Rx<R>::expneg(e - s);
+}
+
+// Series S of d/dlambda log P -> product series P[0 .. n-1] of one node, handed to put(e, P[e]) (zeros at and beyond n).
+template <int NT, typename R, class F>
+__device__ __forceinline__ void product_series(const R* S, int n, F put)
+{
+    R P[NT + 1], acc[NT + 1];
+    P[0] = R(1);
+#pragma unroll
+    for (int c = 1; c <= NT; c++) acc[c] = R(0);
+#pragma unroll
+    for (int k = 0; k < NT - 1; k++) {
+#pragma unroll
+        for (int c = k + 1; c < NT; c++) acc[c] = fma(S[c - 1 - k], P[k], acc[c]);
+        P[k + 1] = acc[k + 1] * R(1.0 / (k + 1));
+    }
+#pragma unroll
+    for (int e = 0; e < NT; e++) put(e, P[e]);
+}
+
+// Gradient g and the Hessian's diagonal part g2 at the weights in shared memory (this thread's in w_own), in fp64.
 //   amax, amin  extreme log-weights;  hs = sigma * (draft mass above the block)
 // Every token thread (all copies) gets g and g2.
-template <class C, typename R, bool kJac>
-__device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, double hs, int slack, double qstep_d, int jstride,
-                                            float amax, float amin, double w_own, double ds_own, float z_own, double& g_out,
-                                            double& g2_out, Frags<C>& fr)
+template <class C>
+__device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, double hs, int slack, double qstep, float amax,
+                                            float amin, double w_own, double ds_own, double& g_out, double& g2_out)
 {
-    static_assert(!kJac || sizeof(R) == 4, "the contraction's operands are fp32");
     constexpr int NT = C::NT, T = C::T;
+    typedef double R;
     const RSm<C, R> rs(sm);
     const int tid = threadIdx.x, i = tid % C::MP, ng = tid / C::MP;
-    const R qstep = (R)qstep_d;
     float s_hi, s0;
-    const int Q = quad_grid(amax, amin, slack, (float)qstep_d, s_hi, s0);
-    const R wi = (R)w_own, dsi = (R)ds_own;
+    const int Q = quad_grid(amax, amin, slack, (float)qstep, s_hi, s0);
+    const R wi = w_own, dsi = ds_own;
     R dp[NT <= 8 ? NT + 1 : 1];
     if (NT <= 8) {
         dp[0] = R(1);
@@ -567,28 +608,19 @@ __device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, doub
         for (int c = 1; c <= (NT <= 8 ? NT : 0); c++) dp[c] = dp[c - 1] * dsi;
     }
     R g = R(0), g2 = R(0);
-    if (kJac) {
-#pragma unroll
-        for (int s = 0; s < C::kNA; s++) { fr.A[s][0] = fr.A[s][1] = fr.A[s][2] = fr.A[s][3] = 0.f; }
-#pragma unroll
-        for (int s = 0; s < C::kNB; s++) { fr.B[s][0] = fr.B[s][1] = fr.B[s][2] = fr.B[s][3] = 0.f; }
-    }
-    const bool live = kJac || (i & ~31) < m;       // (the contraction's operands are staged for every slot: zeros beyond m)
+    const bool live = (i & ~31) < m;
 #pragma unroll 1
     for (int q0 = 0; q0 < Q; q0 += kQC) {
         const int nq = min(kQC, Q - q0);
         // ---- S: this thread's share of the tokens at its node (16 or 32 node slots)
         const bool narrow = nq <= 16;
         const int q = tid & (narrow ? 15 : 31), G = T / (narrow ? 16 : 32), grp = tid / (narrow ? 16 : 32);
-        constexpr int kSS = sizeof(R) == 4 ? NT + 4 : NT + 2;      // row stride of the shares: conflict-free vector access
+        constexpr int kSS = NT + 2;                                // row stride of the shares: conflict-free vector access
         {
-            const R s = (R)s_hi - qstep * (R)(q0 + q);
-            const R e = Rx<R>::expneg(s - (R)s0);
-            const R t = Rx<R>::expneg(e - s);
+            R e;
+            const R t = quad_node<R>(s_hi, s0, qstep, q0 + q, e);
             if (tid < nq) {
-                const R c0 = qstep * (R(1) + e) * t * (slack ? Rx<R>::expneg(t) : R(1));
-                rs.tq[q] = t; rs.cq[q] = c0;
-                if (kJac) sm.kq[q] = sqrtf((float)((R)jstride * c0 * t));
+                rs.tq[q] = t; rs.cq[q] = qstep * (R(1) + e) * t * (slack ? Rx<R>::expneg(t) : R(1));
             }
             R S[NT];
 #pragma unroll
@@ -604,16 +636,9 @@ __device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, doub
                     if (NT <= 8) {
                         unit_series<NT - 1, R>(u, p, h);
                         R pe[8];                           // p ds^(c+1)
-                        if (sizeof(R) == 4) {
-                            const float4 e0 = ld_f4(sm.E + 8 * j), e1 = NT > 4 ? ld_f4(sm.E + 8 * j + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-                            const float ev[8] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
-#pragma unroll
-                            for (int c = 1; c < 8; c++) pe[c] = p * (R)ev[c];
-                        } else {
-                            const R d2 = d * d, d4 = d2 * d2, pd = p * d;
-                            pe[1] = p * d2; pe[2] = pd * d2; pe[3] = p * d4; pe[4] = pd * d4;
-                            pe[5] = pe[1] * d4; pe[6] = pe[2] * d4; pe[7] = pe[3] * d4;
-                        }
+                        const R d2 = d * d, d4 = d2 * d2, pd = p * d;
+                        pe[1] = p * d2; pe[2] = pd * d2; pe[3] = p * d4; pe[4] = pd * d4;
+                        pe[5] = pe[1] * d4; pe[6] = pe[2] * d4; pe[7] = pe[3] * d4;
 #pragma unroll
                         for (int c = 1; c < NT; c++) S[c] = fma(pe[c & 7], h[c], S[c]);
                     } else {
@@ -631,52 +656,34 @@ __device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, doub
             if (q < nq && (!narrow || (tid & 16) == 0)) {
                 GR_PTR(R) row = rs.SP + ((tid >> 5) * 32 + q) * kSS;
 #pragma unroll
-                for (int c = 0; c < NT; c += 16 / (int)sizeof(R)) st_vec(row + c, S + c);
+                for (int c = 0; c < NT; c += 2) st_vec(row + c, S + c);
             }
         }
         __syncthreads();
         // ---- P: one thread per node.  PP[j] = P[n - 1 - j], so that PP[c - 1] pairs with h[c] in [lambda^n] P h
         if (tid < nq) {
-            R S[NT], P[NT + 1], acc[NT + 1];
+            R S[NT];
 #pragma unroll
             for (int c = 0; c < NT; c++) S[c] = R(0);
 #pragma unroll 2
             for (int k = 0; k < C::kW; k++) {
                 GR_PTR(const R) row = rs.SP + (k * 32 + tid) * kSS;
 #pragma unroll
-                for (int c = 0; c < NT; c += 16 / (int)sizeof(R)) {
-                    R v[16 / sizeof(R)];
+                for (int c = 0; c < NT; c += 2) {
+                    R v[2];
                     ld_vec(row + c, v);
-#pragma unroll
-                    for (int z = 0; z < 16 / (int)sizeof(R); z++) S[c + z] += v[z];
+                    S[c] += v[0]; S[c + 1] += v[1];
                 }
             }
-            S[0] += (R)hs;
-            P[0] = R(1);
-#pragma unroll
-            for (int c = 1; c <= NT; c++) acc[c] = R(0);
-#pragma unroll
-            for (int k = 0; k < NT - 1; k++) {
-#pragma unroll
-                for (int c = k + 1; c < NT; c++) acc[c] = fma(S[c - 1 - k], P[k], acc[c]);
-                P[k + 1] = acc[k + 1] * R(1.0 / (k + 1));
-            }
+            S[0] += hs;
             GR_PTR(R) row = rs.PP + tid * C::kRow;
-#pragma unroll
-            for (int e = 0; e < NT; e++) {
-                // (entries at and beyond n are zero)
-                if (e < n) row[n - 1 - e] = P[e]; else row[e] = R(0);
-            }
+            product_series<NT, R>(S, n, [&](int e, R v) { if (e < n) row[n - 1 - e] = v; else row[e] = R(0); });
         }
         __syncthreads();
-        // ---- g: one thread per token; with kJac the operands of the contraction for every jstride-th node
-        const int span = kJac ? jstride * C::JC : nq;
-        const int step = kJac ? jstride : 1;
-#pragma unroll 1
-        for (int qa = 0; qa < nq; qa += span) {
-            const int qb = min(nq, qa + span);
-            const int nst = kJac ? (qb - qa + jstride - 1) / jstride : 0;
-            auto node = [&](int q2, bool stage, int slot) {
+        // ---- g: one thread per token
+        if (live) {
+#pragma unroll 2
+            for (int q2 = ng; q2 < nq; q2 += C::kNG) {
                 const R t = rs.tq[q2], c0 = rs.cq[q2];
                 const R x = Rx<R>::expneg(t * wi);
                 const R u = fma(R(-2), x, R(1)), p = fma(-x, x, x);
@@ -691,66 +698,215 @@ __device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, doub
                 R pr[NT];
                 R v0 = R(0), v1 = R(0);
 #pragma unroll
-                for (int c = 0; c < NT; c += 16 / (int)sizeof(R)) ld_vec(rs.PP + q2 * C::kRow + c, pr + c);
+                for (int c = 0; c < NT; c += 2) ld_vec(rs.PP + q2 * C::kRow + c, pr + c);
 #pragma unroll
                 for (int c = 0; c < NT; c += 2) { v0 = fma(pr[c], h[c + 1], v0); v1 = fma(pr[c + 1], h[c + 2], v1); }
-                const R ux = wi * x;
-                const R gi = c0 * ux * (v0 + v1);
+                const R gi = c0 * (wi * x) * (v0 + v1);
                 g += gi;
                 g2 = fma(gi * t, wi, g2);
-                if (stage) {
-                    // A = P h (series), paired as sum_kappa A[n - kappa] h_l[kappa], kappa = 1 .. n - 1; both sides carry the
-                    // square root of the node's weight and of the token's scale
-                    const float uz = sm.kq[q2] * (float)ux * z_own;
-                    // (pair z of the node's series indices: element (z & 3) of its MMA depth, half (z >> 2) of the fragment)
-                    const int o = (slot / C::kPack) * 8 * C::kTS + 2 * i;
-                    const int sub = slot % C::kPack;
-#pragma unroll
-                    for (int z = 0; z < NT / 2; z++) {
-                        float a[2];
-#pragma unroll
-                        for (int y = 0; y < 2; y++) {
-                            const int kap = 2 * z + y + 1;
-                            float v = 0.f;
-#pragma unroll
-                            for (int c = 1; c <= NT - kap; c++) v = fmaf((float)h[c], (float)pr[kap + c - 1], v);
-                            a[y] = v;
-                        }
-                        const int f = sub * (NT / 2) + z, at = o + (f & 3) * 2 * C::kTS + (f >> 2);
-                        sm.AS[at] = pack_half(uz * a[0], uz * a[1]);
-                        sm.HS[at] = pack_half(uz * (float)h[2 * z + 1], z == NT / 2 - 1 ? 0.f : uz * (float)h[2 * z + 2]);
-                    }
-                }
-            };
-            if (live) {
-                if (kJac) {
-#pragma unroll 2
-                    for (int z = ng; z < nst; z += C::kNG) node(qa + z * step, true, z);
-                    if (jstride == 2) {
-#pragma unroll 2
-                        for (int z = qa + 1 + 2 * ng; z < qb; z += 2 * C::kNG) node(z, false, 0);
-                    }
-                } else {
-#pragma unroll 2
-                    for (int z = ng; z < nq; z += C::kNG) node(z, false, 0);
-                }
-            }
-            if (kJac) {
-                // unused slots of the last MMA depth
-                if (C::kPack > 1 && nst % C::kPack != 0) {
-                    for (int e = nst * (NT / 2) + tid / C::MP; e < (nst + C::kPack - 1) / C::kPack * 8; e += C::kNG) {
-                        const int at = (e >> 3) * 8 * C::kTS + 2 * i + (e & 3) * 2 * C::kTS + ((e & 7) >> 2);
-                        sm.AS[at] = 0u; sm.HS[at] = 0u;
-                    }
-                }
-                __syncthreads();
-                hess_mma<C>(sm, fr, (nst + C::kPack - 1) / C::kPack);
-                __syncthreads();
             }
         }
-        if (!kJac) __syncthreads();
+        __syncthreads();
     }
-    g_out = (double)g; g2_out = (double)g2;
+    g_out = g; g2_out = g2;
+    sum_copies<C>(sm, g_out, g2_out);
+}
+
+// The same in fp32, and the Hessian's contraction (fragments fr) from every jstride-th node: the off-diagonal entries
+// times z_i z_l, z = rhs^(-1/2) (z_own is this thread's), which keeps the fp16 operands of order one.
+// Packed arithmetic: two tokens at a time where a node's series are summed, two nodes (of which both or neither give the
+// contraction operands: jstride apart) where a token walks them.  The kernel runs a few warps per scheduler and waits for
+// its own results; packed, a wait serves two.  (4096 rows of n = 16, k = 100: 1552 to 1480 us, 64 whole rows of
+// 16 ids 70 to 63, headline 163 to 159.)
+template <class C>
+__device__ __forceinline__ void eval_low(const FSm<C>& sm, int m, int n, float hs, int slack, float qstep, int jstride, float amax,
+                                         float amin, float wi, float dsi, float z_own, double& g_out, double& g2_out, Frags<C>& fr)
+{
+    constexpr int NT = C::NT, T = C::T, kRow2 = 2 * C::kRow;
+    static_assert(C::JC % 2 == 0, "whole pairs of nodes");
+    typedef float R;
+    const RSm<C, R> rs(sm);
+    const int tid = threadIdx.x, i = tid % C::MP, ng = tid / C::MP;
+    float s_hi, s0;
+    const int Q = quad_grid(amax, amin, slack, qstep, s_hi, s0);
+    F2 dp[NT <= 8 ? NT + 1 : 1];
+    if (NT <= 8) {
+        float pw = 1.f;
+#pragma unroll
+        for (int c = 1; c <= (NT <= 8 ? NT : 0); c++) { pw *= dsi; dp[c] = F2(pw); }
+    }
+    F2 g(0.f), g2(0.f);
+#pragma unroll
+    for (int s = 0; s < C::kNA; s++) { fr.A[s][0] = fr.A[s][1] = fr.A[s][2] = fr.A[s][3] = 0.f; }
+#pragma unroll
+    for (int s = 0; s < C::kNB; s++) { fr.B[s][0] = fr.B[s][1] = fr.B[s][2] = fr.B[s][3] = 0.f; }
+    // place of a node among the pairs: node 2 p + h of a coarse grid, nodes 4 p + {0, 2} and 4 p + {1, 3} of a full one
+    auto place = [&](int q) { return jstride == 1 ? q : (q & ~3) | ((q & 1) << 1) | ((q >> 1) & 1); };
+#pragma unroll 1
+    for (int q0 = 0; q0 < Q; q0 += kQC) {
+        const int nq = min(kQC, Q - q0), nqp = (nq + 3) & ~3;
+        // ---- S: this thread's share of the pairs of tokens at its node (16 or 32 node slots)
+        const bool narrow = nq <= 16;
+        const int q = tid & (narrow ? 15 : 31), G = T / (narrow ? 16 : 32), grp = tid / (narrow ? 16 : 32);
+        constexpr int kSS = NT + 4;                                // row stride of the shares: conflict-free vector access
+        {
+            R e;
+            const R t = quad_node<R>(s_hi, s0, qstep, q0 + q, e);
+            if (tid < nqp) {
+                // (places beyond the last node: weight zero)
+                const R c0 = tid < nq ? qstep * (R(1) + e) * t * (slack ? Rx<R>::expneg(t) : R(1)) : 0.f;
+                const int at = place(tid);
+                rs.tq[at] = tid < nq ? t : 0.f; rs.cq[at] = c0;
+                sm.kq[at] = sqrtf((float)jstride * c0 * t);
+            }
+            F2 S2[NT];
+#pragma unroll
+            for (int c = 0; c < NT; c++) S2[c] = F2(0.f);
+            if (q < nq) {
+                // (behind the last token draft masses and weights are zero)
+#pragma unroll 2
+                for (int j = grp; j < (m + 1) >> 1; j += G) {
+                    const float2 wv = ld_f2(rs.w + 2 * j), dv = ld_f2(rs.ds + 2 * j);
+                    const F2 x(Rx<R>::expneg(t * wv.x), Rx<R>::expneg(t * wv.y)), d(dv.x, dv.y);
+                    const F2 u = fma(F2(-2.f), x, F2(1.f)), p = fma(x * F2(-1.f), x, x);
+                    S2[0] = fma(x, d, S2[0]);
+                    F2 h[NT + 1];
+                    if (NT <= 8) {
+                        unit_series<NT - 1, F2>(u, p, h);
+                        GR_PTR(const float) ep = sm.E + 16 * j;       // ds^(c+1) of both
+#pragma unroll
+                        for (int c = 0; c < NT; c += 2) {
+                            const float4 ev = ld_f4(ep + 2 * c);
+                            if (c > 0) S2[c] = fma(p * F2(ev.x, ev.y), h[c], S2[c]);
+                            S2[c + 1] = fma(p * F2(ev.z, ev.w), h[c + 1], S2[c + 1]);
+                        }
+                    } else {
+                        const F2 pd = p * d;
+                        riccati_series<NT - 1, F2>(d, d * u, pd, h);
+#pragma unroll
+                        for (int c = 1; c < NT; c++) S2[c] = fma(pd, h[c], S2[c]);
+                    }
+                }
+            }
+            R S[NT];
+#pragma unroll
+            for (int c = 0; c < NT; c++) S[c] = S2[c].lo() + S2[c].hi();
+            if (narrow) {
+#pragma unroll
+                for (int c = 0; c < NT; c++) S[c] += __shfl_xor_sync(0xffffffffu, S[c], 16);
+            }
+            if (q < nq && (!narrow || (tid & 16) == 0)) {
+                GR_PTR(R) row = rs.SP + ((tid >> 5) * 32 + q) * kSS;
+#pragma unroll
+                for (int c = 0; c < NT; c += 4) st_vec(row + c, S + c);
+            }
+        }
+        __syncthreads();
+        // ---- P: one thread per node.  PP[j] = P[n - 1 - j], so that PP[c - 1] pairs with h[c] in [lambda^n] P h
+        if (tid < nqp) {
+            const int at = place(tid);
+            GR_PTR(R) row = rs.PP + (at >> 1) * kRow2 + (at & 1);
+            if (tid < nq) {
+                R S[NT];
+#pragma unroll
+                for (int c = 0; c < NT; c++) S[c] = R(0);
+#pragma unroll 2
+                for (int k = 0; k < C::kW; k++) {
+                    GR_PTR(const R) part = rs.SP + (k * 32 + tid) * kSS;
+#pragma unroll
+                    for (int c = 0; c < NT; c += 4) {
+                        R v[4];
+                        ld_vec(part + c, v);
+#pragma unroll
+                        for (int z = 0; z < 4; z++) S[c + z] += v[z];
+                    }
+                }
+                S[0] += hs;
+                product_series<NT, R>(S, n, [&](int e, R v) { if (e < n) row[2 * (n - 1 - e)] = v; else row[2 * e] = R(0); });
+            } else {
+#pragma unroll
+                for (int e = 0; e < NT; e++) row[2 * e] = R(0);
+            }
+        }
+        __syncthreads();
+        // ---- g: one thread per token; pairs of nodes, those that stage the operands of the contraction first
+        auto pair = [&](int at, bool stage, int slot) {
+            const float2 tv = ld_f2(rs.tq + 2 * at), cv = ld_f2(rs.cq + 2 * at);
+            const F2 x(Rx<R>::expneg(tv.x * wi), Rx<R>::expneg(tv.y * wi));
+            const F2 u = fma(F2(-2.f), x, F2(1.f)), p = fma(x * F2(-1.f), x, x);
+            F2 h[NT + 1];
+            if (NT <= 8) {
+                unit_series<NT, F2>(u, p, h);
+#pragma unroll
+                for (int c = 1; c <= NT; c++) h[c] = h[c] * dp[NT <= 8 ? c : 0];
+            } else {
+                const F2 ds2(dsi);
+                riccati_series<NT, F2>(ds2, ds2 * u, ds2 * p, h);
+            }
+            F2 pr[NT];
+            F2 v0(0.f), v1(0.f);
+#pragma unroll
+            for (int c = 0; c < NT; c += 2) {
+                const float4 v = ld_f4(rs.PP + at * kRow2 + 2 * c);
+                pr[c] = F2(v.x, v.y); pr[c + 1] = F2(v.z, v.w);
+            }
+#pragma unroll
+            for (int c = 0; c < NT; c += 2) { v0 = fma(pr[c], h[c + 1], v0); v1 = fma(pr[c + 1], h[c + 2], v1); }
+            const F2 ux = x * F2(wi);
+            const F2 gi = F2(cv.x, cv.y) * ux * (v0 + v1);
+            g = g + gi;
+            g2 = fma(gi * F2(tv.x, tv.y), F2(wi), g2);
+            if (stage) {
+                // A = P h (series), paired as sum_kappa A[n - kappa] h_l[kappa], kappa = 1 .. n - 1; both sides carry the
+                // square root of the node's weight and of the token's scale
+                const float2 kv = ld_f2(sm.kq + 2 * at);
+                const F2 uz = F2(kv.x, kv.y) * ux * F2(z_own);
+                // (pair z of a node's series indices: element (z & 3) of its MMA depth, half (z >> 2) of the fragment)
+                const int oa = (slot / C::kPack) * 8 * C::kTS + 2 * i, ob = ((slot + 1) / C::kPack) * 8 * C::kTS + 2 * i;
+                const int sa = (slot % C::kPack) * (NT / 2), sb = ((slot + 1) % C::kPack) * (NT / 2);
+#pragma unroll
+                for (int z = 0; z < NT / 2; z++) {
+                    F2 a[2];
+#pragma unroll
+                    for (int y = 0; y < 2; y++) {
+                        const int kap = 2 * z + y + 1;
+                        F2 v(0.f);
+#pragma unroll
+                        for (int c = 1; c <= NT - kap; c++) v = fma(h[c], pr[kap + c - 1], v);
+                        a[y] = uz * v;
+                    }
+                    const F2 h0 = uz * h[2 * z + 1], h1 = z == NT / 2 - 1 ? F2(0.f) : uz * h[2 * z + 2];
+                    const int fa = sa + z, fb = sb + z;
+                    const int ata = oa + (fa & 3) * 2 * C::kTS + (fa >> 2), atb = ob + (fb & 3) * 2 * C::kTS + (fb >> 2);
+                    sm.AS[ata] = pack_half(a[0].lo(), a[1].lo()); sm.HS[ata] = pack_half(h0.lo(), h1.lo());
+                    sm.AS[atb] = pack_half(a[0].hi(), a[1].hi()); sm.HS[atb] = pack_half(h0.hi(), h1.hi());
+                }
+            }
+        };
+        const int staged = ((nq + jstride - 1) / jstride + 1) >> 1;         // pairs of nodes that stage
+        if (jstride == 2 && (i & ~31) < m) {
+            // (the copies that have one pair less to stage begin)
+#pragma unroll 1
+            for (int z = C::kNG - 1 - ng; z < nqp >> 2; z += C::kNG) pair(2 * z + 1, false, 0);
+        }
+#pragma unroll 1
+        for (int pa = 0; pa < staged; pa += C::JC / 2) {
+            const int np = min(staged - pa, C::JC / 2), nst = 2 * np;
+#pragma unroll 1
+            for (int z = ng; z < np; z += C::kNG) pair((pa + z) * jstride, true, 2 * z);
+            // unused slots of the last MMA depth
+            if (C::kPack > 2 && nst % C::kPack != 0) {
+                for (int e = nst * (NT / 2) + tid / C::MP; e < (nst + C::kPack - 1) / C::kPack * 8; e += C::kNG) {
+                    const int at = (e >> 3) * 8 * C::kTS + 2 * i + (e & 3) * 2 * C::kTS + ((e & 7) >> 2);
+                    sm.AS[at] = 0u; sm.HS[at] = 0u;
+                }
+            }
+            __syncthreads();
+            hess_mma<C>(sm, fr, (nst + C::kPack - 1) / C::kPack);
+            __syncthreads();
+        }
+    }
+    g_out = (double)g.lo() + (double)g.hi(); g2_out = (double)g2.lo() + (double)g2.hi();
     sum_copies<C>(sm, g_out, g2_out);
 }
 
@@ -761,10 +917,9 @@ __device__ __noinline__ double2 eval_fp64(int m, int n, int slack, bool coarse, 
     const FSm<C> sm(flag);
     const int i = threadIdx.x % C::MP;
     const double qstep = sm.scal[SC_QSTEP] * (coarse ? 2.0 : 1.0);
-    Frags<C> none;
     double2 r;
-    if constexpr (C::kContour) eval_contour<C, double, false>(sm, m, slack, qstep, 1, amax, amin, sm.wd[i], 0.f, r.x, r.y, none);
-    else eval_system<C, double, false>(sm, m, n, sm.scal[SC_HS], slack, qstep, 1, amax, amin, sm.wd[i], i < m ? sm.dsd[i] : 0.0, 0.f, r.x, r.y, none);
+    if constexpr (C::kContour) { Frags<C> none; eval_contour<C, double, false>(sm, m, slack, qstep, 1, amax, amin, sm.wd[i], 0.f, r.x, r.y, none); }
+    else eval_system<C>(sm, m, n, sm.scal[SC_HS], slack, qstep, amax, amin, sm.wd[i], i < m ? sm.dsd[i] : 0.0, r.x, r.y);
     return r;
 }
 
@@ -1059,6 +1214,8 @@ __device__ __forceinline__ float row_times(GR_PTR(const __half) mat, GR_PTR(cons
     return dot_row<C>(row, vec);
 }
 
+template <class C> __device__ __forceinline__ float rs_ds(const FSm<C>& sm, int i) { return RSm<C, float>(sm).ds[i]; }
+
 // fp32 evaluation at one point and what the Newton step needs from it, out of line (its registers, fragments included, stay
 // its own).  Default: the Hessian scaled to unit diagonal, I - N with N_il = H_il / sqrt(H_ii H_ll), N in half precision
 // (its error, 2^-11, is that of the contraction's operands) for cg_solve below; sm.dg receives 1 / sqrt(H_ii).
@@ -1077,7 +1234,7 @@ __device__ __noinline__ double2 eval_hessian(int m, int n, int slack, bool coars
     const double rhs = i < m ? sm.rhs[sm.ord[i]] : 0.0;
     const float zr = i < m ? (float)rhs : 1.f, zi = rsqrtf(zr);
     if constexpr (C::kContour) eval_contour<C, float, true>(sm, m, slack, qstep, jstride, amax, amin, sm.wd[i], i < m ? zi : 0.f, g, g2, fr);
-    else eval_system<C, float, true>(sm, m, n, sm.scal[SC_HS], slack, qstep, jstride, amax, amin, sm.wd[i], i < m ? sm.dsd[i] : 0.0, i < m ? zi : 0.f, g, g2, fr);
+    else eval_low<C>(sm, m, n, (float)sm.scal[SC_HS], slack, (float)qstep, jstride, amax, amin, sm.wf[i], i < m ? rs_ds<C>(sm, i) : 0.f, i < m ? zi : 0.f, g, g2, fr);
     if (given) { g = gg.x; g2 = gg.y; }
     if (chol) {
         // an outer block's function is constant along (1,...,1): that direction is pinned with 1/m everywhere
@@ -1360,7 +1517,7 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
             float pw = (float)ds_i;
             const float f = pw;
 #pragma unroll
-            for (int c = 0; c < 8; c++) { sm.E[8 * i + c] = pw; pw *= f; }
+            for (int c = 0; c < 8; c++) { sm.E[16 * (i >> 1) + 2 * c + (i & 1)] = pw; pw *= f; }     // (two tokens side by side)
         }
     }
 
