@@ -54,7 +54,7 @@ constexpr float kFScaleJump = 0.5f;        // distance of the common scale from 
 constexpr float kFSmallSlack = 1.0e-4f;     // share of the mass below which Tn - sum g is mostly rounding in fp32
 constexpr float kFLeastSlack = 1.0e-9f;     // and the least share aimed at (the quadrature's floor)
 constexpr float kFNone = 1.0e30f;          // no residual or ratio yet
-constexpr int kFSweeps = 5;                // fixed-point sweeps of the starting point
+constexpr int kFSweeps = 3;                // fixed-point sweeps of the starting point (five took as many evaluations after them)
 
 // Compile-time geometry.  NT: series length (>= n), MP: padded support size, T: threads, JC: Hessian nodes staged
 // together, CTAS: CTAs per SM the registers are held to.
