@@ -12,8 +12,9 @@ __global__ void __launch_bounds__(kAlphaThreads)
 alpha_kernel(const char* __restrict__ ws, int V, int topk, double temp_t, double temp_d, NList nl,
              float* __restrict__ alpha_out, int* __restrict__ status_out)
 {
-    __shared__ double s_key[kMaxSupport], s_tg[kMaxSupport], s_d[kMaxSupport], s_Tg[kMaxSupport + 1], s_Dr[kMaxSupport + 1];
-    __shared__ int s_id[kMaxSupport];
+    __shared__ unsigned long long s_key[kMaxSupport];
+    __shared__ double s_tg[kMaxSupport], s_d[kMaxSupport], s_Tg[kMaxSupport + 1], s_Dr[kMaxSupport + 1];
+    __shared__ int s_id[kMaxSupport], s_at[kMaxSupport];
     __shared__ double s_red[32];
     pdl_wait();
     const int tid = threadIdx.x;
@@ -35,7 +36,8 @@ alpha_kernel(const char* __restrict__ ws, int V, int topk, double temp_t, double
         a_i = (double)wv.tl[tid] / temp_t;
         b_i = (double)wv.dl[tid] / temp_d;
     }
-    const double bmax = block_reduce_max(tid < k ? b_i : -1.0e300, GR_MKPTR(double, s_red, 32, nullptr));
+    // (the streaming pass leaves the support in descending order: the first entry is the largest)
+    const double bmax = (double)wv.dl[0] / temp_d;
     const double bsum = block_reduce_sum(tid < k ? exp(b_i - bmax) : 0.0, GR_MKPTR(double, s_red, 32, nullptr));
     const double lse_d = bmax + log(bsum);
     if (kfull == V) {
@@ -44,28 +46,21 @@ alpha_kernel(const char* __restrict__ ws, int V, int topk, double temp_t, double
         lse_t = amax + log(asum);
     }
     // ratio order: decreasing log-ratio, equal keys by smaller id (Sec. 5.1)
-    if (tid < k) { s_key[tid] = b_i - a_i; s_id[tid] = my_id; }
+    const unsigned long long key = order_key(b_i - a_i);
+    if (tid < k) { s_key[tid] = key; s_id[tid] = my_id; }
     __syncthreads();
+    const int rank = ratio_rank(GR_MKPTR(const unsigned long long, s_key, kMaxSupport, nullptr), GR_MKPTR(const int, s_id, kMaxSupport, nullptr),
+                                GR_MKPTR(int, s_at, kMaxSupport, nullptr), k, key, my_id);
     if (tid < k) {
-        const double ky = s_key[tid];
-        int rank = 0;
-        for (int j = 0; j < k; j++) {
-            const double kj = s_key[j];
-            rank += (kj > ky || (kj == ky && s_id[j] < my_id)) ? 1 : 0;
-        }
         s_tg[rank] = exp(a_i - lse_t);
         s_d[rank] = exp(b_i - lse_d);
     }
     __syncthreads();
-    if (tid == 0) {
-        double Tg = 0.0, Dr = 0.0;
-        s_Tg[0] = 0.0; s_Dr[0] = 0.0;
-        for (int j = 1; j <= k; j++) {
-            Tg += s_tg[j - 1]; Dr += s_d[j - 1];
-            if (j == k) { Dr = 1.0; if (kfull == V) Tg = 1.0; }   // both distributions are normalised
-            s_Tg[j] = Tg; s_Dr[j] = Dr;
-        }
-    }
+    prefix_sums(GR_MKPTR(const double, s_tg, kMaxSupport, nullptr), GR_MKPTR(double, s_Tg, kMaxSupport + 1, nullptr),
+                GR_MKPTR(const double, s_d, kMaxSupport, nullptr), GR_MKPTR(double, s_Dr, kMaxSupport + 1, nullptr), k);
+    // both distributions are normalised
+    if (tid == 0 && kfull == V) s_Tg[k] = 1.0;
+    if (tid == 32) s_Dr[k] = 1.0;
     __syncthreads();
     // one warp per draft count: min over the prefixes of Tg_j - Dr_j^n
     const int warp = tid >> 5, lane = tid & 31;
@@ -77,6 +72,7 @@ alpha_kernel(const char* __restrict__ ws, int V, int topk, double temp_t, double
             for (int m = n; m > 0; m >>= 1) { if (m & 1) pw *= sq; sq *= sq; }
             best = fmin(best, s_Tg[j] - pw);
         }
+#pragma unroll
         for (int o = 16; o > 0; o >>= 1) best = fmin(best, __shfl_xor_sync(0xffffffffu, best, o));
         if (lane == 0) alpha_out[(size_t)b * nl.count + e] = (float)(1.0 + best);
     }

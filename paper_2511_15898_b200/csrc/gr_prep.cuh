@@ -58,6 +58,50 @@ __device__ __forceinline__ int count_above(GR_PTR(const unsigned long long) keys
     return n0 + n1;
 }
 
+// Position of this thread's token in the ratio order: larger keys first, equal keys by smaller id.  keys and ids are visible to all;
+// `scratch` is overwritten.  Every thread of the CTA calls it (as many threads as tokens at least).
+__device__ __forceinline__ int ratio_rank(GR_PTR(const unsigned long long) keys, GR_PTR(const int) ids, GR_PTR(int) scratch, int k,
+                                          unsigned long long key, int my_id)
+{
+    const int tid = threadIdx.x;
+    const bool on = tid < k;
+    int rank = on ? count_above(keys, 0, k, key) : 0;
+    // equal keys have met at one rank: whoever does not find himself there has company
+    if (on) scratch[rank] = tid;
+    __syncthreads();
+    if (__syncthreads_or(on && scratch[rank] != tid)) {
+        if (on) {
+            int before = 0;
+            for (int j = 0; j < k; j++) before += (keys[j] == key && ids[j] < my_id) ? 1 : 0;
+            rank += before;
+        }
+    }
+    return rank;
+}
+// Prefix sums of two arrays (dst[j] = src[0] + ... + src[j - 1], dst[0] = 0), each summed in order, one after the other, by a thread of
+// its own (threads 0 and 32, which own what they wrote until the next barrier), eight loads ahead of the additions.
+__device__ __forceinline__ void prefix_sums(GR_PTR(const double) src0, GR_PTR(double) dst0, GR_PTR(const double) src1, GR_PTR(double) dst1, int k)
+{
+    if (threadIdx.x == 0 || threadIdx.x == 32) {
+        GR_PTR(const double) src = src0;
+        GR_PTR(double) dst = dst0;
+        if (threadIdx.x == 32) { src = src1; dst = dst1; }
+        double acc = 0.0;
+        dst[0] = 0.0;
+#pragma unroll 1
+        for (int j0 = 0; j0 < k; j0 += 8) {
+            double v[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++) v[u] = src[min(j0 + u, k - 1)];
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                acc += v[u];
+                if (j0 + u < k) dst[j0 + u + 1] = acc;
+            }
+        }
+    }
+}
+
 // shared-memory arrays of the preparation (KP entries each; psi and Dr: KP + 4)
 struct PrepSm {
     GR_PTR(double) d, tg, p, r, key, psi, Dr;
@@ -134,47 +178,18 @@ __device__ inline PrepResult prep_instance(const PrepSm& sm, const WsView& wv, H
     }
     // ---- ratio order: decreasing log-ratio key, equal keys by smaller id (Sec. 5.1)
     // (the reductions above made the keys visible)
-    {
-        GR_PTR(const unsigned long long) keys = GR_PCAST(const unsigned long long, sm.key);
-        int rank = on ? count_above(keys, 0, k, key) : 0;
-        // equal keys have met at one rank: whoever does not find himself there has company
-        if (on) sm.blk[rank] = tid;
-        __syncthreads();
-        if (__syncthreads_or(on && sm.blk[rank] != tid)) {
-            if (on) {
-                for (int j = 0; j < k; j++) rank += (keys[j] == key && sm.itmp[j] < my_id) ? 1 : 0;
-            }
-        }
-        if (on) {
-            sm.id[rank] = my_id;
-            sm.tg[rank] = tg_i;
-            sm.d[rank] = m_div(eb, bsum);
-        }
+    const int rank = ratio_rank(GR_PCAST(const unsigned long long, sm.key), sm.itmp, sm.blk, k, key, my_id);
+    if (on) {
+        sm.id[rank] = my_id;
+        sm.tg[rank] = tg_i;
+        sm.d[rank] = m_div(eb, bsum);
     }
     __syncthreads();
     // ---- prefix sums in order, psi along the chain, H* and alpha* (Eq. "subset-select")
-    // (each summed in order, one after the other, by a thread of its own, eight loads ahead of the additions; the block has two
-    // warps at least)
-    if (lane == 0 && warp < 2) {
-        GR_PTR(const double) src = sm.tg;
-        GR_PTR(double) dst = sm.psi;
-        if (warp == 1) { src = sm.d; dst = sm.Dr; }
-        double acc = 0.0;
-        dst[0] = 0.0;
-#pragma unroll 1
-        for (int j0 = 0; j0 < k; j0 += 8) {
-            double v[8];
-#pragma unroll
-            for (int u = 0; u < 8; u++) v[u] = src[min(j0 + u, k - 1)];
-#pragma unroll
-            for (int u = 0; u < 8; u++) {
-                acc += v[u];
-                if (j0 + u < k) dst[j0 + u + 1] = acc;
-            }
-        }
-        // both distributions are normalised
-        if (warp == 1 || kfull == V) dst[k] = 1.0;
-    }
+    prefix_sums(sm.tg, sm.psi, sm.d, sm.Dr, k);
+    // both distributions are normalised
+    if (tid == 0 && kfull == V) sm.psi[k] = 1.0;
+    if (tid == 32) sm.Dr[k] = 1.0;
     __syncthreads();
     // thread `pos` owns psi[pos + 1]
     double v = 1.0e300;
