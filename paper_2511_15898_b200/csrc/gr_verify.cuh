@@ -48,12 +48,12 @@ __device__ inline VerifyScratch verify_scratch(void* base, int* flag = nullptr) 
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll 1
+#pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 __device__ __forceinline__ double warp_incl_scan(double v, int lane) {
-#pragma unroll 1
+#pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         double t = __shfl_up_sync(0xffffffffu, v, o);
         if (lane >= o) v += t;
@@ -136,8 +136,21 @@ __device__ inline int resample_draw(const Header* h, const ParamView& pv, int k,
             // ---- exact pass over the chunk in id order
             cb = chunk_begin(sel, head);
             const int len = chunk_end(sel, head, nch, V) - cb;
-#pragma unroll 4
-            for (int e = tid; e < len; e += bd) vs.res[e] = exp_neg(lse - (double)load_logit_dyn(row, dtype, cb + e) * rT);
+            // (four loads in flight: they come from HBM)
+#pragma unroll 1
+            for (int e0 = tid; e0 < len; e0 += 4 * bd) {
+                float x[4];
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    const int e = min(e0 + u * bd, len - 1);
+                    x[u] = dtype == GR_BF16 ? __bfloat162float(((const __nv_bfloat16*)row)[cb + e]) : __ldg((const float*)row + cb + e);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    if (e0 + u * bd >= len) break;
+                    vs.res[e0 + u * bd] = exp_neg(lse - (double)x[u] * rT);
+                }
+            }
             __syncthreads();
             for (int j = tid; j < k; j += bd) if (vs.chunk[j] == sel) vs.res[vs.id[j] - cb] = pv.r[j];
             if (tid == 0) { vs.dec[4] = 0x7fffffff; vs.dec[5] = -1; }
@@ -146,7 +159,7 @@ __device__ inline int resample_draw(const Header* h, const ParamView& pv, int k,
             const int e0 = min(tid * per, len), e1 = min(e0 + per, len);
             double sum = 0.0;
             int lastp = -1;
-#pragma unroll 1
+#pragma unroll 4
             for (int e = e0; e < e1; e++) { const double r = vs.res[e]; sum += r; if (r > 0.0) lastp = e; }
             double tot;
             const double inc = block_incl_scan(sum, vs.red, &tot);
@@ -154,8 +167,8 @@ __device__ inline int resample_draw(const Header* h, const ParamView& pv, int k,
             int hit = -1;
             if (lastp >= 0 && inc > want) {
                 hit = lastp;                        // (the run's sum and its walk round differently)
-#pragma unroll 1
-                for (int e = e0; e < lastp; e++) { const double r = vs.res[e]; acc += r; if (r > 0.0 && acc > want) { hit = e; break; } }
+#pragma unroll 4
+                for (int e = e0; e < lastp; e++) { const double r = vs.res[e]; acc += r; if (hit == lastp && r > 0.0 && acc > want) hit = e; }
             }
             if (hit >= 0) atomicMin(&vs.dec[4], hit);
             if (lastp >= 0) atomicMax(&vs.dec[5], lastp);
