@@ -23,8 +23,7 @@ namespace gr {
 
 constexpr int kMaxChunks = 2049;     // V <= 2^21
 constexpr int kMaxCluster = 8;
-constexpr int kRankAll = 256;        // candidates that are ranked as they are; more go through a last threshold first (1 us;
-                                     // at 128 it cost more than it saved: 1000 bf16 rows of 16000, k = 128, 75 us for 69)
+constexpr int kRankAll = 128;        // listed vectors that are taken apart as they are; more go through a last threshold first
 
 // Arguments common to every row.
 struct ScanArgs {
@@ -36,11 +35,12 @@ struct ScanArgs {
     int pstride, kcap;
 };
 
-// Shared memory.  NTHR threads, CAP candidates, CH chunk entries.
-template <int NTHR, int CAP, int CH>
+// Shared memory.  NTHR threads, VCAP listed vectors, CAP candidates, CH chunk entries.
+template <int NTHR, int VCAP, int CAP, int CH>
 struct __align__(16) ScanShared {
-    static constexpr int kThr = NTHR, kCap = CAP, kCh = CH;
-    GR_ARRAY(unsigned long long, keys, CAP);    // candidates (value, id), then composite keys
+    static constexpr int kThr = NTHR, kList = VCAP, kCap = CAP, kCh = CH;
+    static_assert(20 * VCAP >= 8 * CAP && VCAP % 2 == 0, "the candidates take the list's place");
+    GR_ARRAY(unsigned long long, keys, 5 * VCAP / 2);   // listed 16-byte vectors, then their first ids; in their place later composite keys
     GR_ARRAY(float2, chunk, CH);
     double lse[1], part[NTHR / 32], top;
     unsigned long long prefix;
@@ -63,12 +63,42 @@ struct __align__(16) ScanShared {
 template <typename T> struct VecTraits;
 template <> struct VecTraits<float> {
     static constexpr int N = 4;
+    static constexpr unsigned long long kBad = 0x7fc000007fc00000ull, kNone = 0xff800000ff800000ull;        // elements that are -infinity
+    __device__ static float largest(const ulonglong2& v) { return fmaxf(fmaxf(f_lo(v.x), f_hi(v.x)), fmaxf(f_lo(v.y), f_hi(v.y))); }
+    // sums of 0 * logit: zero until a NaN or an infinity makes them NaN, whatever the size of the finite ones (masks down to
+    // the type's lowest value)
+    typedef unsigned long long Check;
+    __device__ static void check(Check& c, const ulonglong2& v) { c = fma2(v.x, 0ull, c); c = fma2(v.y, 0ull, c); }
+    __device__ static bool bad(Check c) { return !(f_lo(c) == 0.f) || !(f_hi(c) == 0.f); }
+    __device__ static ulonglong2 alone(float x) { ulonglong2 v; v.x = (kNone & ~0xffffffffull) | __float_as_uint(x); v.y = kNone; return v; }
+    __device__ static float element(const ulonglong2& v, int i) { const unsigned long long w = i < 2 ? v.x : v.y; return i & 1 ? f_hi(w) : f_lo(w); }
     // the two packed pairs of a 16-byte vector, i = 0, 1
     __device__ static unsigned long long pair(const ulonglong2& v, int i) { return i == 0 ? v.x : v.y; }
     static constexpr int kPairs = 2;
 };
 template <> struct VecTraits<__nv_bfloat16> {
     static constexpr int N = 8;
+    static constexpr unsigned int kBad = 0x7fc07fc0u;
+    static constexpr unsigned long long kNone = 0xff80ff80ff80ff80ull;
+    __device__ static __nv_bfloat162 two(unsigned int w) { return *reinterpret_cast<const __nv_bfloat162*>(&w); }
+    // (on the packed elements: a third of the instructions of unpacking them first)
+    __device__ static float largest(const ulonglong2& v) {
+        const __nv_bfloat162 m = __hmax2(__hmax2(two((unsigned int)v.x), two((unsigned int)(v.x >> 32))), __hmax2(two((unsigned int)v.y), two((unsigned int)(v.y >> 32))));
+        const unsigned int w = *reinterpret_cast<const unsigned int*>(&m);
+        return fmaxf(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+    }
+    typedef unsigned int Check;
+    __device__ static void check(Check& c, const ulonglong2& v) {
+        const unsigned int w[4] = {(unsigned int)v.x, (unsigned int)(v.x >> 32), (unsigned int)v.y, (unsigned int)(v.y >> 32)};
+#pragma unroll
+        for (int i = 0; i < 4; i++) asm("fma.rn.bf16x2 %0, %1, %2, %0;" : "+r"(c) : "r"(w[i]), "r"(0u));
+    }
+    __device__ static bool bad(Check c) { return !(__uint_as_float(c << 16) == 0.f) || !(__uint_as_float(c & 0xffff0000u) == 0.f); }
+    __device__ static ulonglong2 alone(float x) { ulonglong2 v; v.x = (kNone & ~0xffffull) | (__float_as_uint(x) >> 16); v.y = kNone; return v; }
+    __device__ static float element(const ulonglong2& v, int i) {
+        const unsigned long long w = i < 4 ? v.x : v.y;
+        return __uint_as_float((unsigned int)((w >> (16 * (i & 3))) & 0xffffull) << 16);
+    }
     __device__ static unsigned long long pair(const ulonglong2& v, int i) {
         const unsigned int w = (unsigned int)((i < 2 ? v.x : v.y) >> (32 * (i & 1)));
         return ((unsigned long long)(w & 0xffff0000u) << 32) | (unsigned long long)(w << 16);
@@ -127,19 +157,19 @@ __device__ __forceinline__ void refine_tau(SS& sh, float mx, int need)
     __syncthreads();
 }
 
+// A vector that holds a candidate goes into the list as it is (with the elements beside it: eight tests and appends of their
+// own were a third of the pass's instructions in bf16, where nearly every warp's vector of a wide support holds one).
 template <class SS>
-__device__ __forceinline__ void push_candidate(SS& sh, float val, int id, float tau) {
-    if (val >= tau) {
-        const int slot = atomicAdd(&sh.cnt, 1);
-        if (slot < SS::kCap) {
-            GR_ARRAY_AS(float, sh.keys, slot) = val;
-            GR_ARRAY_AS(int, sh.keys, SS::kCap + slot) = id;
-        }
+__device__ __forceinline__ void push_vector(SS& sh, const ulonglong2& v, int id) {
+    const int slot = atomicAdd(&sh.cnt, 1);
+    if (slot < SS::kList) {
+        GR_ARRAY_AS(ulonglong2, sh.keys, slot) = v;
+        GR_ARRAY_AS(int, sh.keys, 4 * SS::kList + slot) = id;
     }
 }
 
 // Exact selection of the ksel largest composite keys among this CTA's chunks by eight 8-bit radix passes over them (slow
-// path, taken only when the candidate list overflowed).
+// path, taken only when the candidate list overflowed); they are left in sh.keys, their number in sh.cnt.
 template <typename T, class SS>
 __device__ __noinline__ void exact_select_slow(SS& sh, const T* prow, int V, int head, int nch, int first, int stride, int ksel)
 {
@@ -168,7 +198,10 @@ __device__ __noinline__ void exact_select_slow(SS& sh, const T* prow, int V, int
                     if (i >= e1) break;
                     const unsigned long long key = ckey(v[u], i);
                     if (pass == 8) {
-                        if (key >= prefix) push_candidate(sh, v[u], i, -INFINITY);
+                        if (key >= prefix) {
+                            const int slot = atomicAdd(&sh.cnt, 1);
+                            if (slot < SS::kCap) sh.keys[slot] = key;
+                        }
                     } else if (pass == 0 || (key >> (shift + 8)) == (prefix >> (shift + 8))) {
                         atomicAdd(&sh.hist[(int)((key >> shift) & 255ull)], 1);
                     }
@@ -189,10 +222,23 @@ __device__ __noinline__ void exact_select_slow(SS& sh, const T* prow, int V, int
     }
 }
 
-// The nsel largest of the M composite keys in sh.keys, handed to `take(rank, key)`.
+// The nsel largest of the M composite keys in sh.keys, handed to `take(rank, key)`.  (Four threads to a key where there are
+// enough of them.)
 template <class SS, class F>
 __device__ __forceinline__ void rank_select(SS& sh, int M, int nsel, F take)
 {
+    if (4 * M <= SS::kThr) {
+        const int e = threadIdx.x >> 2, part = threadIdx.x & 3;
+        const unsigned long long me = e < M ? sh.keys[e] : ~0ull;
+        int rank = 0;
+#pragma unroll 4
+        for (int j = part; j < M; j += 4) rank += (sh.keys[j] > me) ? 1 : 0;
+        __syncwarp();
+        rank += __shfl_xor_sync(0xffffffffu, rank, 1);
+        rank += __shfl_xor_sync(0xffffffffu, rank, 2);
+        if (part == 0 && e < M && rank < nsel) take(rank, me);
+        return;
+    }
 #pragma unroll 1
     for (int e = threadIdx.x; e < M; e += SS::kThr) {
         const unsigned long long me = sh.keys[e];
@@ -248,8 +294,7 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
     if (cn > 1) cluster_barrier(); else __syncthreads();
 
     float g0 = -INFINITY;                  // running maximum of this thread's draft logits
-    unsigned long long chk = 0ull;         // sums of 0 * logit (two packed): zero until a NaN or an infinity makes them NaN,
-                                           // whatever the size of the finite ones (masks down to the type's lowest value)
+    typename VT::Check chk = 0;
     const float sc_t = A.sc_t;
     const unsigned long long sc2 = f_pack(sc_t, sc_t);
     float kmax = -INFINITY, kmin = INFINITY;                // range of the log-ratios draft / target (kFull)
@@ -263,6 +308,7 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
         kmax = fmaxf(kmax, fmaxf(f_lo(key), f_hi(key))); kmin = fminf(kmin, fminf(f_lo(key), f_hi(key)));
     };
     const int rounds = (nch + stride - 1) / stride;
+    float m0 = -INFINITY, s0 = 0.f, m1 = m0, s1 = s0, m2 = m0, s2 = s0, m3, s3;     // sums of the last four chunks
     const int vec_end = head + ((V - head) / N) * N, tail = V - vec_end;
 
 #pragma unroll 1
@@ -295,10 +341,10 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
                     const float mn = fmaxf(cm, x);
                     cs = fmaf(cs, ex2((cm - mn) * sc_t), ex2((x - mn) * sc_t));
                     cm = mn;
-                    chk = fma2(f_pack(x, v), 0ull, chk);
+                    chk = x - x == 0.f && v - v == 0.f ? chk : VT::kBad;
                     g0 = fmaxf(g0, v);
                     if (kFull) ratio_range(f_pack(x, x), f_pack(v, v));
-                    if (!kFull) push_candidate(sh, v, i, tau);
+                    if (!kFull && v >= tau) push_vector(sh, VT::alone(v), i);
                 };
                 if (nb == 0) {
                     if (c == 0 && lane < head) scalar(lane);
@@ -308,14 +354,10 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
                 for (int u = 0; u < U; u++) {
                     if (whole || base + u * 32 * N + N <= vec_end) {
                         unsigned long long x[VT::kPairs];
-                        float vm = -INFINITY;
 #pragma unroll
-                        for (int i = 0; i < VT::kPairs; i++) {
-                            x[i] = VT::pair(qv[u], i);
-                            vm = fmaxf(vm, fmaxf(f_lo(x[i]), f_hi(x[i])));
-                            chk = fma2(x[i], 0ull, chk);
-                        }
-                        const float mn = fmaxf(cm, vm);
+                        for (int i = 0; i < VT::kPairs; i++) x[i] = VT::pair(qv[u], i);
+                        VT::check(chk, qv[u]);
+                        const float mn = fmaxf(cm, VT::largest(qv[u]));
                         // (a factor of exactly one where the maximum stands)
                         const float keep = cm == mn ? 1.f : ex2((cm - mn) * sc_t);
                         const unsigned long long nm = f_pack(-mn, -mn);
@@ -333,26 +375,14 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
 #pragma unroll
                 for (int u = 0; u < U; u++) {
                     if (whole || base + u * 32 * N + N <= vec_end) {
-                        float vm = -INFINITY;
-#pragma unroll
-                        for (int i = 0; i < VT::kPairs; i++) {
-                            const unsigned long long x = VT::pair(pv[u], i);
-                            vm = fmaxf(vm, fmaxf(f_lo(x), f_hi(x)));
-                            chk = fma2(x, 0ull, chk);
-                        }
+                        const float vm = VT::largest(pv[u]);
+                        VT::check(chk, pv[u]);
                         g0 = fmaxf(g0, vm);
                         if (kFull) {
 #pragma unroll
                             for (int i = 0; i < VT::kPairs; i++) ratio_range(VT::pair(qv[u], i), VT::pair(pv[u], i));
                         }
-                        if (!kFull && vm >= tau) {
-#pragma unroll
-                            for (int i = 0; i < VT::kPairs; i++) {
-                                const unsigned long long x = VT::pair(pv[u], i);
-                                push_candidate(sh, f_lo(x), base + u * 32 * N + 2 * i, tau);
-                                push_candidate(sh, f_hi(x), base + u * 32 * N + 2 * i + 1, tau);
-                            }
-                        }
+                        if (!kFull && vm >= tau) push_vector(sh, pv[u], base + u * 32 * N);
                     }
                 }
             }
@@ -363,29 +393,40 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
                     const float t1 = *((volatile float*)&sh.tau);
 #pragma unroll
                     for (int u = 0; u < U; u++) {
-                        if (whole || base + u * 32 * N + N <= vec_end) {
-#pragma unroll
-                            for (int i = 0; i < VT::kPairs; i++) {
-                                const unsigned long long x = VT::pair(pv[u], i);
-                                if (fmaxf(f_lo(x), f_hi(x)) >= t1) {
-                                    push_candidate(sh, f_lo(x), base + u * 32 * N + 2 * i, t1);
-                                    push_candidate(sh, f_hi(x), base + u * 32 * N + 2 * i + 1, t1);
-                                }
-                            }
-                        }
+                        if ((whole || base + u * 32 * N + N <= vec_end) && VT::largest(pv[u]) >= t1) push_vector(sh, pv[u], base + u * 32 * N);
                     }
-                    if (c == 0 && lane < head) push_candidate(sh, load_logit<T>(prow, lane), lane, t1);
-                    if (c == nch - 1 && lane < tail) push_candidate(sh, load_logit<T>(prow, vec_end + lane), vec_end + lane, t1);
+                    auto scalar = [&](int i) {
+                        const float v = load_logit<T>(prow, i);
+                        if (v >= t1) push_vector(sh, VT::alone(v), i);
+                    };
+                    if (c == 0 && lane < head) scalar(lane);
+                    if (c == nch - 1 && lane < tail) scalar(vec_end + lane);
                 }
             }
         }
-        if (cvalid) {
+        // the chunk's lanes put together (a butterfly from 16 lanes down), four chunks at a time: two lanes that meet each go on
+        // with one of two chunks, so that four take six steps of a lane and not twenty
+        m3 = m2; s3 = s2; m2 = m1; s2 = s1; m1 = m0; s1 = s0; m0 = cm; s0 = cs;
+        if ((r & 3) == 3 || r == rounds - 1) {
+            auto meet = [&](float& ma, float& sa, float mb, float sb, int o) {
+                const bool up = (lane & o) != 0;
+                const float ms = up ? ma : mb, ss = up ? sa : sb;
+                ma = up ? mb : ma; sa = up ? sb : sa;
+                const float mo = __shfl_xor_sync(0xffffffffu, ms, o), so = __shfl_xor_sync(0xffffffffu, ss, o);
+                osm_merge(ma, sa, mo, so, sc_t);
+            };
+            __syncwarp();
+            float ma = m0, sa = s0, mb = m2, sb = s2;
+            meet(ma, sa, m1, s1, 16);
+            meet(mb, sb, m3, s3, 16);
+            meet(ma, sa, mb, sb, 8);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float mo = __shfl_xor_sync(0xffffffffu, cm, o), so = __shfl_xor_sync(0xffffffffu, cs, o);
-                osm_merge(cm, cs, mo, so, sc_t);
+            for (int o = 4; o > 0; o >>= 1) {
+                const float mo = __shfl_xor_sync(0xffffffffu, ma, o), so = __shfl_xor_sync(0xffffffffu, sa, o);
+                osm_merge(ma, sa, mo, so, sc_t);
             }
-            if (lane == 0) sh.chunk[c] = make_float2(cm, cs);
+            const int age = (lane >> 4) + ((lane >> 3) & 1) * 2, at = c - age * stride;
+            if ((lane & 7) == 0 && age <= (r & 3) && at >= 0 && at < nch) sh.chunk[at] = make_float2(ma, sa);
         }
         // a better threshold whenever the part read has grown fourfold (k = 50 of 512 groups: some 60 candidates in a first
         // part, 180 more per fourfold)
@@ -393,7 +434,7 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
     }
     // non-finite inputs
     {
-        const bool badl = !(f_lo(chk) == 0.f) || !(f_hi(chk) == 0.f);
+        const bool badl = VT::bad(chk);
         if (__any_sync(0xffffffffu, badl) && lane == 0) atomicOr(&sh.bad, 1);
     }
     // ---- candidates: a last threshold from the list itself, then composite keys of those that pass it
@@ -402,39 +443,50 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
     int M = 0, nsel = 0;
     if (!kFull) {
         nsel = ksel < V ? ksel : V;
-        if (sh.cnt > SS::kCap) exact_select_slow<T>(sh, prow, V, head, nch, first, stride, nsel);
-        M = min(sh.cnt, SS::kCap);
-        constexpr int kPer = SS::kCap / SS::kThr;
-        float vv[kPer], own = -INFINITY;
+        M = min(sh.cnt, SS::kList);
+        bool over = sh.cnt > SS::kList;
+        if (!over) {
+            constexpr int kPer = (SS::kList + SS::kThr - 1) / SS::kThr;
+            ulonglong2 vv[kPer];
+            int id[kPer];
+            float own = -INFINITY;
 #pragma unroll
-        for (int u = 0; u < kPer; u++) {
-            const int e = tid + u * SS::kThr;
-            vv[u] = e < M ? GR_ARRAY_AS(float, sh.keys, e) : -INFINITY;
-            own = fmaxf(own, vv[u]);
-        }
-        // (the threads' shares of the list are the groups: in a short row the threads' maxima are too few to tell anything, and
-        // ranking 1500 elements among themselves took 60 us)
-        if (M > kRankAll) refine_tau(sh, own, nsel);
-        const float tau = sh.tau;
-        unsigned long long kk[kPer];
+            for (int u = 0; u < kPer; u++) {
+                const int e = tid + u * SS::kThr;
+                vv[u].x = VT::kNone; vv[u].y = VT::kNone; id[u] = 0;
+                if (e < M) { vv[u] = GR_ARRAY_AS(ulonglong2, sh.keys, e); id[u] = GR_ARRAY_AS(int, sh.keys, 4 * SS::kList + e); }
+                own = fmaxf(own, VT::largest(vv[u]));
+            }
+            // (the threads' shares of the list are the groups: in a short row the threads' maxima are too few to tell anything, and
+            // ranking 1500 elements among themselves took 60 us)
+            if (M > kRankAll) refine_tau(sh, own, nsel);
+            const float tau = sh.tau;
+            if (tid == 0) sh.kept = 0;
+            __syncthreads();
+            if (own >= tau) {
 #pragma unroll
-        for (int u = 0; u < kPer; u++) {
-            const int e = tid + u * SS::kThr;
-            kk[u] = e < M && vv[u] >= tau ? ckey(vv[u], GR_ARRAY_AS(int, sh.keys, SS::kCap + e)) : 0ull;
-        }
-        if (tid == 0) sh.kept = 0;
-        __syncthreads();
+                for (int u = 0; u < kPer; u++) {
+                    if (VT::largest(vv[u]) >= tau) {
 #pragma unroll
-        for (int u = 0; u < kPer; u++) {
-            const bool on = kk[u] != 0ull;
-            const unsigned mk = __ballot_sync(0xffffffffu, on);
-            int at = 0;
-            if (mk != 0 && lane == 0) at = atomicAdd(&sh.kept, __popc(mk));
-            at = __shfl_sync(0xffffffffu, at, 0) + __popc(mk & ((1u << lane) - 1u));
-            if (on) sh.keys[at] = kk[u];
+                        for (int i = 0; i < N; i++) {
+                            const float v = VT::element(vv[u], i);
+                            if (v >= tau && v > -INFINITY) {
+                                const int slot = atomicAdd(&sh.kept, 1);
+                                if (slot < SS::kCap) sh.keys[slot] = ckey(v, id[u] + i);
+                            }
+                        }
+                    }
+                }
+            }
+            __syncthreads();
+            M = sh.kept;
+            over = M > SS::kCap;
         }
-        __syncthreads();
-        M = sh.kept;
+        if (over) {
+            __syncthreads();
+            exact_select_slow<T>(sh, prow, V, head, nch, first, stride, nsel);
+            M = min(sh.cnt, SS::kCap);
+        }
     }
     if (cn > 1) {
         // ---- the other CTAs' parts to the first one: chunk entries, status, and each one's own nsel largest keys

@@ -36,6 +36,22 @@ def test_support_and_log_sum_exp(V, batch):
         assert int((s.status != G.GR_OK).sum()) <= batch // 200, (dt, k)
 
 
+@pytest.mark.parametrize("V,batch", [(65535, 148), (65536, 148), (65537, 149), (50257, 296), (50257, 298), (300, 593), (2048, 741), (7001, 741)])
+def test_support_where_the_threads_per_row_change(V, batch):
+    test_support_and_log_sum_exp(V, batch)
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+def test_whole_rows_in_a_large_batch(dt):
+    """Whole-vocabulary rows by the CTAs of a large batch and by those of a small one: the same bits."""
+    g = torch.Generator(device="cuda").manual_seed(4)
+    q = (3 * torch.randn(300, 5003, generator=g, device="cuda")).to(dt)
+    p = (q.float() + torch.randn(300, 5003, generator=g, device="cuda")).to(dt)
+    large, st = G.alpha_star(q, p, [2, 8], 0, 0.75, 1.0)
+    small, _ = G.alpha_star(q[:37], p[:37], [2, 8], 0, 0.75, 1.0)
+    assert int(st.max()) == 0 and torch.equal(small, large[:37])
+
+
 @pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("V,k", [(1500, 20), (40000, 50), (100, 0), (3001, 0), (50257, 0)])
 def test_masks_are_logits_and_only_nan_and_infinity_are_not(V, k, dt):
