@@ -20,11 +20,13 @@ int launch_fast_n8_m128(GR_FAST_ARGS);
 int launch_fast_n8_m128w(GR_FAST_ARGS);
 int launch_fast_n16_m32(GR_FAST_ARGS);
 int launch_fast_n16_m32w(GR_FAST_ARGS);
+int launch_fast_n16_m32h(GR_FAST_ARGS);
 int launch_fast_n16_m64(GR_FAST_ARGS);
 int launch_fast_n16_m64w(GR_FAST_ARGS);
 int launch_fast_n16_m128(GR_FAST_ARGS);
 int launch_fast_n16_m128w(GR_FAST_ARGS);
 int launch_fast_c24_m32(GR_FAST_ARGS);
+int launch_fast_c24_m32w(GR_FAST_ARGS);
 int launch_fast_c24_m64(GR_FAST_ARGS);
 int launch_fast_c24_m128(GR_FAST_ARGS);
 }
@@ -41,14 +43,15 @@ int launch_fast(GR_FAST_ARGS)
     // count for more (1024 headline rows: 300 us in the wide variant, 163 in the other; 512 rows, n = 16, k = 20: 118 and 97).
     const bool one = batch <= kSms, two = batch <= 2 * kSms;
     if (n > 16) {
-        if (kcap <= 32) return fast::launch_fast_c24_m32(GR_FAST_PASS);
+        if (kcap <= 32) return two ? fast::launch_fast_c24_m32w(GR_FAST_PASS) : fast::launch_fast_c24_m32(GR_FAST_PASS);
         if (kcap <= 64) return fast::launch_fast_c24_m64(GR_FAST_PASS);
         return fast::launch_fast_c24_m128(GR_FAST_PASS);
     }
     if (kcap <= 32) {
         if (n <= 4) return two ? fast::launch_fast_n4_m32w(GR_FAST_PASS) : fast::launch_fast_n4_m32(GR_FAST_PASS);
         if (n <= 8) return two ? fast::launch_fast_n8_m32w(GR_FAST_PASS) : fast::launch_fast_n8_m32(GR_FAST_PASS);
-        return two ? fast::launch_fast_n16_m32w(GR_FAST_PASS) : fast::launch_fast_n16_m32(GR_FAST_PASS);
+        if (two) return fast::launch_fast_n16_m32w(GR_FAST_PASS);
+        return batch <= 4 * kSms ? fast::launch_fast_n16_m32h(GR_FAST_PASS) : fast::launch_fast_n16_m32(GR_FAST_PASS);
     }
     if (kcap <= 64) {
         if (n <= 4) return one ? fast::launch_fast_n4_m64w(GR_FAST_PASS) : fast::launch_fast_n4_m64(GR_FAST_PASS);

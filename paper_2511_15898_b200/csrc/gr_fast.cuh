@@ -54,7 +54,8 @@ constexpr float kFScaleJump = 0.5f;        // distance of the common scale from 
 constexpr float kFSmallSlack = 1.0e-4f;     // share of the mass below which Tn - sum g is mostly rounding in fp32
 constexpr float kFLeastSlack = 1.0e-9f;     // and the least share aimed at (the quadrature's floor)
 constexpr float kFNone = 1.0e30f;          // no residual or ratio yet
-constexpr int kFSweeps = 3;                // fixed-point sweeps of the starting point (five took as many evaluations after them)
+constexpr int kFSweeps = 3, kFSweepsCircle = 5;   // fixed-point sweeps of the starting point (with series five saved no evaluation; on
+                                           // the circle, where an evaluation costs several times as much, they may)
 
 // Compile-time geometry.  NT: series length (>= n), MP: padded support size, T: threads, JC: Hessian nodes staged
 // together, CTAS: CTAs per SM the registers are held to.
@@ -1437,8 +1438,9 @@ __device__ __noinline__ void start_point(int m, int slack, int n, double Tm, int
     }
     // (a thread reads back what it wrote)
     float A = (slack ? 1.f : 0.f) + wi;
+    constexpr int sweeps = C::kContour ? kFSweepsCircle : kFSweeps;
 #pragma unroll 1
-    for (int sweep = 0; sweep < kFSweeps; sweep++) {
+    for (int sweep = 0; sweep < sweeps; sweep++) {
         GR_PTR(const float) inv = vec_buffer(sm, sweep & 1) + share * (kCol + 4);
         float acc[4] = {0.f, 0.f, 0.f, 0.f};
         auto group = [&](int c, const float* pv) {
@@ -1469,7 +1471,7 @@ __device__ __noinline__ void start_point(int m, int slack, int n, double Tm, int
             wi = odds * (slack ? 1.f + Si : fmaxf(Si, 1e-30f));
             A = (slack ? 1.f : 0.f) + wi + Si;
         }
-        if (sweep + 1 < kFSweeps) {
+        if (sweep + 1 < sweeps) {
             if (lead) vec_buffer(sm, (sweep + 1) & 1)[vec_pos<C>(i)] = __fdividef(1.f, wi);
             __syncthreads();
         }

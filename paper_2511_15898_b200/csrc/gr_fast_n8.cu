@@ -5,6 +5,6 @@ namespace gr {
 namespace fast {
 GR_FAST_INSTANTIATE(n8_m32, 8, 32, 64, 8, 8)
 GR_FAST_INSTANTIATE(n8_m64, 8, 64, 128, 6, 4)
-GR_FAST_INSTANTIATE(n8_m128, 8, 128, 128, 4, 3)
+GR_FAST_INSTANTIATE(n8_m128, 8, 128, 256, 4, 2)
 }  // namespace fast
 }  // namespace gr
