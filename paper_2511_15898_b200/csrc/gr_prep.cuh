@@ -45,7 +45,7 @@ __device__ __forceinline__ unsigned long long order_key(double x) {
     return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
 }
 // How many of keys[lo .. hi) are above `key`.  Integers, strict comparisons and several loads ahead: 50 fp64 keys with the
-// tie rule in the comparison took 5.8 k cycles, a warp's ballots 5.4 k, this 0.6 k.
+// tie rule in the comparison took 5.8 k cycles, a warp's ballots 5.4 k, this with what surrounds it 1.3 k.
 __device__ __forceinline__ int count_above(GR_PTR(const unsigned long long) keys, int lo, int hi, unsigned long long key)
 {
     int n0 = 0, n1 = 0;
