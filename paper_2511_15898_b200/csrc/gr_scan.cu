@@ -6,6 +6,8 @@ namespace gr {
 
 constexpr int kScanThreads = 512;
 
+// (1280 listed vectors hold what random rows bring between two cuts of the list at any support up to 128, and 2048 candidates what
+// the last threshold leaves of it; with them four CTAs fit an SM.)
 template <int NTHR> using ScanSm = ScanShared<NTHR, 1280, 2048, kMaxChunks>;
 
 template <typename T, bool kFull, int kInFlight, int NTHR, int CTAS>

@@ -13,9 +13,10 @@
 //
 // Selection without a second pass: a threshold tau that is provably not above the ksel-th largest draft logit is derived
 // from running maxima of disjoint groups of elements (each of the ksel largest group maxima is a distinct element, so the
-// ksel-th largest of them bounds the answer from below), refined whenever the part read has grown fourfold; elements >= tau are
-// appended to a shared candidate list and the exact answer is taken from the list at the end.  If the list ever
-// overflows (adversarially ordered rows) an exact multi-pass radix selection over the row replaces it.
+// ksel-th largest of them bounds the answer from below), refined whenever the part read has grown fourfold; vectors with an
+// element >= tau are appended to a shared candidate list and the exact answer is taken from the list at the end.  Where the
+// list would not hold what is still to come, a refined threshold cuts it (keep_listed).  If it overflows all the same
+// (adversarially ordered rows) an exact multi-pass radix selection over the row replaces it.
 #pragma once
 #include "gr_common.cuh"
 
@@ -143,8 +144,9 @@ __device__ __forceinline__ void cluster_barrier() {
 
 // The `need`-th largest of the threads' running maxima (16 leading key bits, rounded down); never below the old threshold.
 // (512 threads: 16 counting barriers, 0.3 us; one warp searching 512 values in shared memory took three times that.)
+// Returns the length of the list, the same for every thread (nobody appends between the first of the barriers and the last).
 template <class SS>
-__device__ __forceinline__ void refine_tau(SS& sh, float mx, int need)
+__device__ __forceinline__ int refine_tau(SS& sh, float mx, int need)
 {
     const unsigned int key = fkey(mx);
     unsigned int res = 0;
@@ -153,8 +155,10 @@ __device__ __forceinline__ void refine_tau(SS& sh, float mx, int need)
         const unsigned int t = res | (1u << bit);
         if (__syncthreads_count(key >= t) >= need) res = t;
     }
+    const int listed = sh.cnt;
     if (threadIdx.x == 0) sh.tau = fmaxf(sh.tau, fkey_inv(res));
     __syncthreads();
+    return listed;
 }
 
 // A vector that holds a candidate goes into the list as it is (with the elements beside it: eight tests and appends of their
@@ -166,6 +170,31 @@ __device__ __forceinline__ void push_vector(SS& sh, const ulonglong2& v, int id)
         GR_ARRAY_AS(ulonglong2, sh.keys, slot) = v;
         GR_ARRAY_AS(int, sh.keys, 4 * SS::kList + slot) = id;
     }
+}
+
+// Cuts the list of `listed` vectors to those that hold an element >= tau, in place: a round's vectors are read before any of
+// them is written, and what is kept of them goes to places at or before their own.
+template <typename T, class SS>
+__device__ __forceinline__ void keep_listed(SS& sh, int listed)
+{
+    const float tau = sh.tau;
+    if (threadIdx.x == 0) sh.kept = 0;
+#pragma unroll 1
+    for (int e0 = 0; e0 < listed; e0 += SS::kThr) {
+        const int e = e0 + (int)threadIdx.x;
+        ulonglong2 v = VecTraits<T>::alone(-INFINITY);
+        int id = 0;
+        if (e < listed) { v = GR_ARRAY_AS(ulonglong2, sh.keys, e); id = GR_ARRAY_AS(int, sh.keys, 4 * SS::kList + e); }
+        __syncthreads();
+        if (e < listed && VecTraits<T>::largest(v) >= tau) {
+            const int slot = atomicAdd(&sh.kept, 1);
+            GR_ARRAY_AS(ulonglong2, sh.keys, slot) = v;
+            GR_ARRAY_AS(int, sh.keys, 4 * SS::kList + slot) = id;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) sh.cnt = sh.kept;
+    __syncthreads();
 }
 
 // Exact selection of the ksel largest composite keys among this CTA's chunks by eight 8-bit radix passes over them (slow
@@ -311,126 +340,139 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
     float m0 = -INFINITY, s0 = 0.f, m1 = m0, s1 = s0, m2 = m0, s2 = s0, m3, s3;     // sums of the last four chunks
     const int vec_end = head + ((V - head) / N) * N, tail = V - vec_end;
 
+    int r = 0, part = use_tau ? 1 : rounds;                 // rounds up to the next threshold
 #pragma unroll 1
-    for (int r = 0; r < rounds; r++) {
-        const int c = first + r * stride + warp;
-        const bool cvalid = c < nch;
-        const bool whole = cvalid && head + (c + 1) * kChunk <= vec_end;
-        // target: this lane's (max, sum exp2) of the chunk, vector by vector; the elements before the first and behind the
-        // last vector come first.  (The order of these fp32 sums is part of the results: it decides the last bit of the
-        // chunk masses, and with 10^5 ids a resampled token can hang on that.)
-        float cm = -INFINITY, cs = 0.f;
+    while (true) {
 #pragma unroll 1
-        for (int nb = 0; nb < NB; nb++) {
-            const int base = head + c * kChunk + (nb * U * 32 + lane) * N;
-            const bool sample = use_tau && r == 0 && nb == 0;
-            const float tau = sample ? INFINITY : (use_tau ? *((volatile float*)&sh.tau) : -INFINITY);
-            ulonglong2 qv[U], pv[U];
-            if (cvalid) {
-#pragma unroll
-                for (int u = 0; u < U; u++) {
-                    const int i0 = base + u * 32 * N;
-                    bool ok = whole || i0 + N <= vec_end;
-#ifdef GR_CHECK
-                    if (ok && (i0 < 0 || i0 + N > V || ((size_t)(qrow + i0) & 15) || ((size_t)(prow + i0) & 15))) { if (check) *check = 1; ok = false; }
-#endif
-                    if (ok) { qv[u] = ldg_stream(qrow + i0); pv[u] = ldg_stream(prow + i0); }
-                }
-                auto scalar = [&](int i) {
-                    const float x = load_logit<T>(qrow, i), v = load_logit<T>(prow, i);
-                    const float mn = fmaxf(cm, x);
-                    cs = fmaf(cs, ex2((cm - mn) * sc_t), ex2((x - mn) * sc_t));
-                    cm = mn;
-                    chk = x - x == 0.f && v - v == 0.f ? chk : VT::kBad;
-                    g0 = fmaxf(g0, v);
-                    if (kFull) ratio_range(f_pack(x, x), f_pack(v, v));
-                    if (!kFull && v >= tau) push_vector(sh, VT::alone(v), i);
-                };
-                if (nb == 0) {
-                    if (c == 0 && lane < head) scalar(lane);
-                    if (c == nch - 1 && lane < tail) scalar(vec_end + lane);
-                }
-#pragma unroll
-                for (int u = 0; u < U; u++) {
-                    if (whole || base + u * 32 * N + N <= vec_end) {
-                        unsigned long long x[VT::kPairs];
-#pragma unroll
-                        for (int i = 0; i < VT::kPairs; i++) x[i] = VT::pair(qv[u], i);
-                        VT::check(chk, qv[u]);
-                        const float mn = fmaxf(cm, VT::largest(qv[u]));
-                        // (a factor of exactly one where the maximum stands)
-                        const float keep = cm == mn ? 1.f : ex2((cm - mn) * sc_t);
-                        const unsigned long long nm = f_pack(-mn, -mn);
-#pragma unroll
-                        for (int i = 0; i < VT::kPairs; i++) {
-                            const unsigned long long y = mul2(add2(x[i], nm), sc2);
-                            const float e0 = ex2(f_lo(y)), e1 = ex2(f_hi(y));
-                            cs = i == 0 ? fmaf(cs, keep, e0) : cs + e0;
-                            cs += e1;
-                        }
-                        cm = mn;
-                    }
-                }
-                // draft
-#pragma unroll
-                for (int u = 0; u < U; u++) {
-                    if (whole || base + u * 32 * N + N <= vec_end) {
-                        const float vm = VT::largest(pv[u]);
-                        VT::check(chk, pv[u]);
-                        g0 = fmaxf(g0, vm);
-                        if (kFull) {
-#pragma unroll
-                            for (int i = 0; i < VT::kPairs; i++) ratio_range(VT::pair(qv[u], i), VT::pair(pv[u], i));
-                        }
-                        if (!kFull && vm >= tau) push_vector(sh, pv[u], base + u * 32 * N);
-                    }
-                }
-            }
-            if (sample) {
-                // the first batch had no threshold: it gives one, and its draft logits, still in registers, are tested now
-                refine_tau(sh, g0, ksel);
+        for (; r < min(part, rounds); r++) {
+            const int c = first + r * stride + warp;
+            const bool cvalid = c < nch;
+            const bool whole = cvalid && head + (c + 1) * kChunk <= vec_end;
+            // target: this lane's (max, sum exp2) of the chunk, vector by vector; the elements before the first and behind the
+            // last vector come first.  (The order of these fp32 sums is part of the results: it decides the last bit of the
+            // chunk masses, and with 10^5 ids a resampled token can hang on that.)
+            float cm = -INFINITY, cs = 0.f;
+#pragma unroll 1
+            for (int nb = 0; nb < NB; nb++) {
+                const int base = head + c * kChunk + (nb * U * 32 + lane) * N;
+                const bool sample = use_tau && r == 0 && nb == 0;
+                const float tau = sample ? INFINITY : (use_tau ? *((volatile float*)&sh.tau) : -INFINITY);
+                ulonglong2 qv[U], pv[U];
                 if (cvalid) {
-                    const float t1 = *((volatile float*)&sh.tau);
 #pragma unroll
                     for (int u = 0; u < U; u++) {
-                        if ((whole || base + u * 32 * N + N <= vec_end) && VT::largest(pv[u]) >= t1) push_vector(sh, pv[u], base + u * 32 * N);
+                        const int i0 = base + u * 32 * N;
+                        bool ok = whole || i0 + N <= vec_end;
+#ifdef GR_CHECK
+                        if (ok && (i0 < 0 || i0 + N > V || ((size_t)(qrow + i0) & 15) || ((size_t)(prow + i0) & 15))) { if (check) *check = 1; ok = false; }
+#endif
+                        if (ok) { qv[u] = ldg_stream(qrow + i0); pv[u] = ldg_stream(prow + i0); }
                     }
                     auto scalar = [&](int i) {
-                        const float v = load_logit<T>(prow, i);
-                        if (v >= t1) push_vector(sh, VT::alone(v), i);
+                        const float x = load_logit<T>(qrow, i), v = load_logit<T>(prow, i);
+                        const float mn = fmaxf(cm, x);
+                        cs = fmaf(cs, ex2((cm - mn) * sc_t), ex2((x - mn) * sc_t));
+                        cm = mn;
+                        chk = x - x == 0.f && v - v == 0.f ? chk : VT::kBad;
+                        g0 = fmaxf(g0, v);
+                        if (kFull) ratio_range(f_pack(x, x), f_pack(v, v));
+                        if (!kFull && v >= tau) push_vector(sh, VT::alone(v), i);
                     };
-                    if (c == 0 && lane < head) scalar(lane);
-                    if (c == nch - 1 && lane < tail) scalar(vec_end + lane);
+                    if (nb == 0) {
+                        if (c == 0 && lane < head) scalar(lane);
+                        if (c == nch - 1 && lane < tail) scalar(vec_end + lane);
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; u++) {
+                        if (whole || base + u * 32 * N + N <= vec_end) {
+                            unsigned long long x[VT::kPairs];
+#pragma unroll
+                            for (int i = 0; i < VT::kPairs; i++) x[i] = VT::pair(qv[u], i);
+                            VT::check(chk, qv[u]);
+                            const float mn = fmaxf(cm, VT::largest(qv[u]));
+                            // (a factor of exactly one where the maximum stands)
+                            const float keep = cm == mn ? 1.f : ex2((cm - mn) * sc_t);
+                            const unsigned long long nm = f_pack(-mn, -mn);
+#pragma unroll
+                            for (int i = 0; i < VT::kPairs; i++) {
+                                const unsigned long long y = mul2(add2(x[i], nm), sc2);
+                                const float e0 = ex2(f_lo(y)), e1 = ex2(f_hi(y));
+                                cs = i == 0 ? fmaf(cs, keep, e0) : cs + e0;
+                                cs += e1;
+                            }
+                            cm = mn;
+                        }
+                    }
+                    // draft
+#pragma unroll
+                    for (int u = 0; u < U; u++) {
+                        if (whole || base + u * 32 * N + N <= vec_end) {
+                            const float vm = VT::largest(pv[u]);
+                            VT::check(chk, pv[u]);
+                            g0 = fmaxf(g0, vm);
+                            if (kFull) {
+#pragma unroll
+                                for (int i = 0; i < VT::kPairs; i++) ratio_range(VT::pair(qv[u], i), VT::pair(pv[u], i));
+                            }
+                            if (!kFull && vm >= tau) push_vector(sh, pv[u], base + u * 32 * N);
+                        }
+                    }
+                }
+                if (sample) {
+                    // the first batch had no threshold: it gives one, and its draft logits, still in registers, are tested now
+                    refine_tau(sh, g0, ksel);
+                    if (cvalid) {
+                        const float t1 = *((volatile float*)&sh.tau);
+#pragma unroll
+                        for (int u = 0; u < U; u++) {
+                            if ((whole || base + u * 32 * N + N <= vec_end) && VT::largest(pv[u]) >= t1) push_vector(sh, pv[u], base + u * 32 * N);
+                        }
+                        auto scalar = [&](int i) {
+                            const float v = load_logit<T>(prow, i);
+                            if (v >= t1) push_vector(sh, VT::alone(v), i);
+                        };
+                        if (c == 0 && lane < head) scalar(lane);
+                        if (c == nch - 1 && lane < tail) scalar(vec_end + lane);
+                    }
                 }
             }
-        }
-        // the chunk's lanes put together (a butterfly from 16 lanes down), four chunks at a time: two lanes that meet each go on
-        // with one of two chunks, so that four take six steps of a lane and not twenty
-        m3 = m2; s3 = s2; m2 = m1; s2 = s1; m1 = m0; s1 = s0; m0 = cm; s0 = cs;
-        if ((r & 3) == 3 || r == rounds - 1) {
-            auto meet = [&](float& ma, float& sa, float mb, float sb, int o) {
-                const bool up = (lane & o) != 0;
-                const float ms = up ? ma : mb, ss = up ? sa : sb;
-                ma = up ? mb : ma; sa = up ? sb : sa;
-                const float mo = __shfl_xor_sync(0xffffffffu, ms, o), so = __shfl_xor_sync(0xffffffffu, ss, o);
-                osm_merge(ma, sa, mo, so, sc_t);
-            };
-            __syncwarp();
-            float ma = m0, sa = s0, mb = m2, sb = s2;
-            meet(ma, sa, m1, s1, 16);
-            meet(mb, sb, m3, s3, 16);
-            meet(ma, sa, mb, sb, 8);
+            // the chunk's lanes put together (a butterfly from 16 lanes down), four chunks at a time: two lanes that meet each go on
+            // with one of two chunks, so that four take six steps of a lane and not twenty
+            m3 = m2; s3 = s2; m2 = m1; s2 = s1; m1 = m0; s1 = s0; m0 = cm; s0 = cs;
+            if ((r & 3) == 3 || r == rounds - 1) {
+                auto meet = [&](float& ma, float& sa, float mb, float sb, int o) {
+                    const bool up = (lane & o) != 0;
+                    const float ms = up ? ma : mb, ss = up ? sa : sb;
+                    ma = up ? mb : ma; sa = up ? sb : sa;
+                    const float mo = __shfl_xor_sync(0xffffffffu, ms, o), so = __shfl_xor_sync(0xffffffffu, ss, o);
+                    osm_merge(ma, sa, mo, so, sc_t);
+                };
+                __syncwarp();
+                float ma = m0, sa = s0, mb = m2, sb = s2;
+                meet(ma, sa, m1, s1, 16);
+                meet(mb, sb, m3, s3, 16);
+                meet(ma, sa, mb, sb, 8);
 #pragma unroll
-            for (int o = 4; o > 0; o >>= 1) {
-                const float mo = __shfl_xor_sync(0xffffffffu, ma, o), so = __shfl_xor_sync(0xffffffffu, sa, o);
-                osm_merge(ma, sa, mo, so, sc_t);
+                for (int o = 4; o > 0; o >>= 1) {
+                    const float mo = __shfl_xor_sync(0xffffffffu, ma, o), so = __shfl_xor_sync(0xffffffffu, sa, o);
+                    osm_merge(ma, sa, mo, so, sc_t);
+                }
+                const int age = (lane >> 4) + ((lane >> 3) & 1) * 2, at = c - age * stride;
+                if ((lane & 7) == 0 && age <= (r & 3) && at >= 0 && at < nch) sh.chunk[at] = make_float2(ma, sa);
             }
-            const int age = (lane >> 4) + ((lane >> 3) & 1) * 2, at = c - age * stride;
-            if ((lane & 7) == 0 && age <= (r & 3) && at >= 0 && at < nch) sh.chunk[at] = make_float2(ma, sa);
         }
-        // a better threshold whenever the part read has grown fourfold (k = 50 of 512 groups: some 60 candidates in a first
-        // part, 180 more per fourfold)
-        if (use_tau && r + 1 < rounds && (r & (r + 1)) == 0 && ((r + 1) & 0x55555555)) refine_tau(sh, g0, ksel);
+        if (r >= rounds) break;
+        // A better threshold whenever the part read has grown fourfold.  With N groups (threads) about A = N ln(1 / (1 - k / N)) of
+        // the elements read so far reach a fresh threshold (k = 50: 53 at 512 threads, 56 at 256; k = 100: 111, 127; k = 128: 147,
+        // 177), so A elements come with the first part and 3 A more per fourfold.  Where the list does not hold what is expected
+        // until the next threshold, and a quarter more (A <= k + k^2 / N), it is cut by this one: it then fits random rows of any
+        // length at any support.  (Uncut, k = 128 at 256 threads lists 1370 vectors of 128256 fp32 logits, and most rows took the
+        // exact selection: 1024 rows, acceptance alone, 1450 us; now 215, and 209 at k = 100, where nothing is cut.  A call or the
+        // cut inside the loop over the rounds cost calls that need no cut 1 to 2 %.)
+        const int listed = refine_tau(sh, g0, ksel);
+        const int more = (ksel + ksel * ksel / SS::kThr) * min(3 * r, rounds - r);           // times r
+        if (listed <= SS::kList && 5 * more > 4 * (SS::kList - listed) * r) keep_listed<T>(sh, listed);
+        part *= 4;
     }
     // non-finite inputs
     {

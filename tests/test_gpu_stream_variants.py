@@ -113,3 +113,20 @@ def test_rows_with_long_candidate_lists(V):
         x = torch.randn(300, 2 * V, generator=g, device="cuda")
         us = [_median_us(lambda a=x[:, :n].contiguous(): G.alpha_star(a, a, [2], 8, 1.0, 0.9)) for n in (V, V + 1)]
         assert us[0] < 1.25 * us[1], us
+
+
+@pytest.mark.parametrize("V,batch,dt", [(128256, 300, torch.float32), (152064, 560, torch.float32), (152064, 600, torch.bfloat16),
+                                        (524289, 148, torch.float32), (524289, 300, torch.float32)])
+def test_wide_supports_of_long_rows_fit_the_list(V, batch, dt):
+    """Random rows do not fill the candidate list, whatever the support, the vocabulary and the threads per row: a support of
+    112 to 128 tokens takes about what one of 64 does (1.1 times as long; the exact selection that an overfull list leads to
+    takes three times as long and more), and it is the right one."""
+    g = torch.Generator(device="cuda").manual_seed(V + batch)
+    q = (3 * torch.randn(batch, V, generator=g, device="cuda")).to(dt)
+    p = (q.float() + torch.randn(batch, V, generator=g, device="cuda")).to(dt)
+    us = {k: _median_us(lambda: G.alpha_star(q, p, [8], k, 0.7, 1.0)) for k in (64, 112, 120, 128)}
+    assert max(us.values()) < 1.5 * us[64], us
+    rows = slice(batch - 8, batch)
+    ids = G.read_rule(G.solve(q, p, 2, 128, 0.7, 1.0)).ids[rows, :128]
+    want = torch.sort(p[rows], dim=1, descending=True, stable=True).indices[:, :128]
+    assert torch.equal(torch.sort(want, dim=1).values.int().cpu(), torch.sort(ids, dim=1).values)
