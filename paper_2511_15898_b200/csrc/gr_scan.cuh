@@ -25,6 +25,7 @@ namespace gr {
 constexpr int kMaxChunks = 2049;     // V <= 2^21
 constexpr int kMaxCluster = 8;
 constexpr int kRankAll = 128;        // listed vectors that are taken apart as they are; more go through a last threshold first
+constexpr int kRankKeys = 256;       // and elements of them where no threshold has been met yet (rows that are listed whole)
 
 // Arguments common to every row.
 struct ScanArgs {
@@ -502,6 +503,19 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
             // (the threads' shares of the list are the groups: in a short row the threads' maxima are too few to tell anything, and
             // ranking 1500 elements among themselves took 60 us)
             if (M > kRankAll) refine_tau(sh, own, nsel);
+            else if (sh.tau == -INFINITY && M * N > kRankKeys) {
+                // Up to 1024 elements in few vectors, all of them candidates: halves of a vector are the groups, quarters up to
+                // 64 vectors, so that there are as many as a support has tokens.  (400 rows, k = 8: 1000 bf16 logits 115 -> 31 us,
+                // 600 64 -> 31, 500 fp32 ones 51 -> 31.)
+                static_assert(2 * kRankAll <= SS::kThr && 2 * (kRankKeys / 4) >= kMaxSupport && 4 * (kRankKeys / 8) >= kMaxSupport, "groups");
+                const int lg = M > kRankAll / 2 ? 1 : 2, e = tid >> lg, n0 = (tid & ((1 << lg) - 1)) * (N >> lg);
+                float most = -INFINITY;
+                if (e < M) {
+                    const ulonglong2 v = GR_ARRAY_AS(ulonglong2, sh.keys, e);
+                    for (int i = 0; i < N >> lg; i++) most = fmaxf(most, VT::element(v, n0 + i));
+                }
+                refine_tau(sh, most, nsel);
+            }
             const float tau = sh.tau;
             if (tid == 0) sh.kept = 0;
             __syncthreads();

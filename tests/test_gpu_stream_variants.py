@@ -130,3 +130,21 @@ def test_wide_supports_of_long_rows_fit_the_list(V, batch, dt):
     ids = G.read_rule(G.solve(q, p, 2, 128, 0.7, 1.0)).ids[rows, :128]
     want = torch.sort(p[rows], dim=1, descending=True, stable=True).indices[:, :128]
     assert torch.equal(torch.sort(want, dim=1).values.int().cpu(), torch.sort(ids, dim=1).values)
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+def test_short_rows_are_cut_before_they_are_ranked(dt):
+    """Rows of up to about 1000 ids are listed whole in few vectors: the list is cut by parts of a vector (many ties among the
+    elements, odd lengths), and the row takes no longer than one of 1100, whose list is cut by vectors."""
+    g = torch.Generator(device="cuda").manual_seed(12)
+    for V in (129, 256, 257, 263, 300, 511, 515, 519, 600, 1000, 1023, 1024, 1031):
+        for k in (1, 8, 64, 65, 127, 128):
+            for levels in (3, 40, 100000):
+                p = (torch.randint(0, levels, (5, V), generator=g, device="cuda").float() / 7 - 3).to(dt)
+                q = torch.randn(5, V, generator=g, device="cuda").to(dt)
+                r = G.read_rule(G.solve(q, p, 1, k, 1.0, 1.0))
+                want = torch.sort(p, dim=1, descending=True, stable=True).indices[:, :k]
+                assert torch.equal(torch.sort(want, dim=1).values.int().cpu(), torch.sort(r.ids[:, :k], dim=1).values), (V, k, levels)
+    x = torch.randn(400, 1100, generator=g, device="cuda").to(dt)
+    us = {n: _median_us(lambda a=x[:, :n].contiguous(): G.alpha_star(a, a, [2], 8, 1.0, 0.9)) for n in (500, 600, 1000, 1100)}
+    assert max(us.values()) < 1.25 * us[1100], us
