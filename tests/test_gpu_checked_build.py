@@ -60,7 +60,22 @@ cases = [("config1", W.config1(batch=16, device="cuda"), None),
          ("cluster of 4, V=70001", W.config3(batch=20, device="cuda", seed=3105, V=70001, n=3, topk=20), None),
          ("cluster of 2, V=33001", W.config3(batch=40, device="cuda", seed=3106, V=33001, n=2, topk=8), None),
          ("ascending V=33001", ascending(W.config3(batch=5, device="cuda", seed=3107, V=33001, n=2, topk=64)), None),
-         ("bf16 V=9001", W.config5(batch=4, device="cuda", V=9001, rows_per_pass=4), None)]
+         ("bf16 V=9001", W.config5(batch=4, device="cuda", V=9001, rows_per_pass=4), None),
+         # the streaming pass by 256 threads per row, by pairs of CTAs, with a list that is cut on the way, on short rows
+         ("256 threads, V=4099", W.config3(batch=300, device="cuda", seed=3120, V=4099, n=2, topk=8), None),
+         ("pairs, V=65541", W.config3(batch=76, device="cuda", seed=3121, V=65541, n=2, topk=8), None),
+         ("list cut, V=120001", W.config3(batch=300, device="cuda", seed=3122, V=120001, n=2, topk=128), None),
+         ("list cut in pairs, V=600001", W.config3(batch=76, device="cuda", seed=3123, V=600001, n=2, topk=128), None),
+         ("short row V=501", W.config3(batch=5, device="cuda", seed=3124, V=501, n=3, topk=20), None),
+         ("short bf16 row V=1003", W.config5(batch=300, device="cuda", seed=5120, V=1003, n=3, topk=100), None)]
+# the solve kernel's variants, by series length, support and batch (few rows: more threads per instance)
+for n, topk, batches in ((4, 20, (3, 300)), (4, 50, (3, 150)), (8, 20, (3, 300)), (8, 50, (150,)), (8, 100, (3, 150)),
+                         (16, 20, (3, 300, 600)), (16, 50, (3, 150)), (16, 100, (3, 150)), (32, 20, (300,)), (20, 50, (3,))):
+    for batch in batches:
+        cases.append(("variant n=%%d k=%%d, %%d rows" %% (n, topk, batch),
+                      W.config3(batch=batch, device="cuda", seed=6000 + 10 * n + topk + batch, V=2501, n=n, topk=topk), None))
+cases.append(("bf16 variant n=16 k=100, 300 rows", W.config5(batch=300, device="cuda", seed=5121, V=2501), None))
+cases.append(("tau=0.02, n=8 k=20, 300 rows", W.config3(batch=300, device="cuda", seed=6500, V=2501, n=8, topk=20), G.Options(tau=0.02)))
 for name, wl, opt in cases:
     s = G.solve(wl.q_logits, wl.p_logits, wl.n, wl.topk, wl.temp_target, wl.temp_draft, opt)
     v = G.verify(s, wl.draft_tokens, wl.uniforms)

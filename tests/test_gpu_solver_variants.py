@@ -30,6 +30,33 @@ def test_draft_counts_and_supports_at_the_edges(n, topk):
     assert rep.n_underreported == 0 and rep.n_evaluated_off == 0, (rep.summary(), rep.details[:5])
 
 
+def _certified(wl, rule, rows):
+    """The rows' gradient norms at the weights of `rule` and their optimal acceptances, by the oracle."""
+    tt, td = P.oracle_temps(wl)
+    cert = O.certify_batch(W.logits_to_f64(wl.q_logits[rows]), W.logits_to_f64(wl.p_logits[rows]), wl.n, wl.topk, tt, td,
+                           rule.w[rows].numpy(), lse=rule.lse_target[rows].numpy())
+    assert set(rule.status.tolist()) == {G.GR_OK} and float(rule.gnorm.max()) <= 3.2e-7
+    assert float(cert.gnorm_lse.max()) <= 3.2e-7
+    assert abs(rule.alpha_star[rows].numpy() - cert.alpha_star).max() <= 1e-6
+
+
+@pytest.mark.parametrize("n,topk,batch", [(n, k, b) for n in (2, 4, 5, 8, 9, 16, 17, 32) for k in (17, 32)
+                                          for b in ((296, 297, 592, 593) if 8 < n <= 16 else (296, 297))]
+                         + [(n, k, b) for n in (2, 4, 5, 8, 9, 16) for k in (33, 64, 65, 128) for b in (148, 149)])
+def test_rows_of_both_sides_of_a_change_of_variant(n, topk, batch):
+    """The number of threads per instance depends on the batch: first, last and other rows of batches at each change, and the
+    whole batch's draws by the fused call and by the two calls (from one law each within 3e-7 of the target: a fused call solves
+    a system from the same logits in the same way, so the tokens are the same)."""
+    wl = W.config3(batch=batch, device="cuda", seed=300 + 40 * topk + n, V=2000, n=n, topk=topk)
+    args = (wl.q_logits, wl.p_logits, n, topk, wl.temp_target, wl.temp_draft)
+    solved = G.solve(*args)
+    rows = [0, 1, batch // 2, batch - 2, batch - 1]
+    _certified(wl, G.read_rule(solved), rows)
+    two = G.verify(solved, wl.draft_tokens, wl.uniforms)
+    one = G.solve_verify(wl.q_logits, wl.p_logits, wl.draft_tokens, wl.uniforms, topk, wl.temp_target, wl.temp_draft)[1]
+    assert torch.equal(two.token, one.token) and torch.equal(two.accepted, one.accepted) and torch.equal(two.status, one.status)
+
+
 @pytest.mark.parametrize("n", [2, 4, 5, 8, 9, 16])
 @pytest.mark.parametrize("topk", [17, 32, 33, 64, 65, 128])
 def test_both_widths_of_a_variant(n, topk):

@@ -102,6 +102,12 @@ def test_truncated_wide_support():
     assert tr > 0
 
 
+@pytest.mark.parametrize("n,topk,batch", [(4, 20, 300), (8, 50, 150), (16, 20, 600)])
+def test_truncated_in_larger_batches(n, topk, batch):
+    """Batches that take the variants with fewer threads per instance."""
+    _check_tau(W.config3(batch=batch, device="cuda", seed=3014 + n, V=2000, n=n, topk=topk), 2e-2, draws=2)
+
+
 def test_vanishing_tau_reproduces_the_exact_rule():
     wl = W.config3(batch=24, device="cuda", seed=3013)
     exact = G.read_rule(G.solve(wl.q_logits, wl.p_logits, wl.n, wl.topk, wl.temp_target, wl.temp_draft))
