@@ -54,11 +54,8 @@ constexpr float kFScaleJump = 0.5f;        // distance of the common scale from 
 constexpr float kFSmallSlack = 1.0e-4f;     // share of the mass below which Tn - sum g is mostly rounding in fp32
 constexpr float kFLeastSlack = 1.0e-9f;     // and the least share aimed at (the quadrature's floor)
 constexpr float kFNone = 1.0e30f;          // no residual or ratio yet
-// Fixed-point sweeps of the starting point.  Up to 64 tokens three instead of five take 0.02 to 0.26 evaluations more (n = 8,
-// 1024 rows: k = 50 3.995 to 4.080, k = 20 3.04 to 3.30) and mostly more time (159 to 166 us, 66 to 68; n = 4, k = 8, 256 rows 32
-// to 36; n = 4, k = 20 alone 58 to 56).  Up to 128 tokens a sweep costs more and the last two save no evaluation (n = 8, k = 128:
-// 4.005 with five, 4.009 with three, 381 and 365 us; n = 16, k = 100: 2.05 with either, 376 and 365).
-constexpr int kFSweeps = 5, kFSweepsWide = 3;
+constexpr int kFSweeps = 3, kFSweepsCircle = 5;   // fixed-point sweeps of the starting point (with series five saved no evaluation; on
+                                           // the circle, where an evaluation costs several times as much, they may)
 
 // Compile-time geometry.  NT: series length (>= n), MP: padded support size, T: threads, JC: Hessian nodes staged
 // together, CTAS: CTAs per SM the registers are held to.
@@ -1441,7 +1438,7 @@ __device__ __noinline__ void start_point(int m, int slack, int n, double Tm, int
     }
     // (a thread reads back what it wrote)
     float A = (slack ? 1.f : 0.f) + wi;
-    constexpr int sweeps = C::MP > 64 && !C::kContour ? kFSweepsWide : kFSweeps;
+    constexpr int sweeps = C::kContour ? kFSweepsCircle : kFSweeps;
 #pragma unroll 1
     for (int sweep = 0; sweep < sweeps; sweep++) {
         GR_PTR(const float) inv = vec_buffer(sm, sweep & 1) + share * (kCol + 4);
