@@ -54,8 +54,6 @@ constexpr float kFScaleJump = 0.5f;        // distance of the common scale from 
 constexpr float kFSmallSlack = 1.0e-4f;     // share of the mass below which Tn - sum g is mostly rounding in fp32
 constexpr float kFLeastSlack = 1.0e-9f;     // and the least share aimed at (the quadrature's floor)
 constexpr float kFNone = 1.0e30f;          // no residual or ratio yet
-constexpr int kFSweeps = 3, kFSweepsCircle = 5;   // fixed-point sweeps of the starting point (with series five saved no evaluation; on
-                                           // the circle, where an evaluation costs several times as much, they may)
 
 // Compile-time geometry.  NT: series length (>= n), MP: padded support size, T: threads, JC: Hessian nodes staged
 // together, CTAS: CTAs per SM the registers are held to.
@@ -63,6 +61,13 @@ template <int NT_, int MP_, int T_, int JC_, int CTAS_>
 struct Cfg {
     static constexpr int NT = NT_, MP = MP_, T = T_, JC = JC_, kCtas = CTAS_;
     static constexpr bool kContour = NT > 16;     // samples on a circle instead of series (NT: largest number of them)
+    // Fixed-point sweeps of the starting point: five where an evaluation weighs more than the sweeps, three elsewhere.  Three take 0.02
+    // to 0.26 evaluations an instance more up to 64 tokens (n = 8, 1024 rows: k = 50 3.995 to 4.080, k = 20 3.04 to 3.30).  Whole calls, us,
+    // three / five: a batch that leaves an SM with one or two instances 128 headline rows 88.2 / 85.1, 64 whole rows of 16 ids 86 / 78 (three
+    // draws of rows), one row 64.2 / 63.7 (three); series of 16, n = 16, k = 20, 512 rows 133.1 / 129.6, 1777 rows of k = 5 238.2 / 231.1, n = 12,
+    // k = 20 114.8 / 117.2; full SMs with shorter series 1024 headline rows 329.7 / 337.2 (two draws), n = 4, 1024 rows: k = 8 83.6 / 91.4, k = 20
+    // 102.7 / 107.2, k = 50 172.9 / 177.7.  Up to 128 tokens the last two save no evaluation (n = 8, k = 128, solve 365 / 381; n = 16, k = 100 365 / 376).
+    static constexpr int kSweeps = kContour || (MP <= 64 && (NT == 16 || kCtas <= 2)) ? 5 : 3;
     static constexpr int kNG = T / MP;            // copies of the token threads (they share the nodes out among them)
     static constexpr int kW = T / 32, kTW = MP / 32;
     static constexpr int kRow = NT + 4;           // row stride of the product series (16-byte aligned rows in fp32 and fp64)
@@ -1438,7 +1443,7 @@ __device__ __noinline__ void start_point(int m, int slack, int n, double Tm, int
     }
     // (a thread reads back what it wrote)
     float A = (slack ? 1.f : 0.f) + wi;
-    constexpr int sweeps = C::kContour ? kFSweepsCircle : kFSweeps;
+    constexpr int sweeps = C::kSweeps;
 #pragma unroll 1
     for (int sweep = 0; sweep < sweeps; sweep++) {
         GR_PTR(const float) inv = vec_buffer(sm, sweep & 1) + share * (kCol + 4);
