@@ -46,9 +46,10 @@ constexpr double kFTrustPivot = 0.02;      // smallest relative pivot at which a
 constexpr double kFPredictBound = 3.0;     // reported norm after such a stop: kFPredictBound * s2
 constexpr double kFLowLeave = 3.0e-5;      // predicted residual at which the iteration goes over to fp64
 constexpr double kFLowFloor = 1.0e-4;      // below this residual a failure to improve is taken for fp32's noise
-constexpr double kFChordBase = 0.02;       // contraction assumed of a step by conjugate gradients (a third of what the stop allows for)
+constexpr double kFChordBase = 0.02;       // contraction assumed of a step by conjugate gradients (a third of what the stop allows for; 0.008 seen)
 constexpr int kFCgMax = 16;                // conjugate-gradient iterations before the factorisation takes over
-constexpr float kFCgTol = 2.0e-4f;         // and their relative residual; in fp32 kFCgLow times the gradient norm, up to kFCgLoose
+constexpr float kFCgTol = 2.0e-4f;         // and their relative residual; in fp32 kFCgLow times the gradient norm, up to kFCgLoose (at
+                                           // 2e-4 throughout no instance of 16 shapes takes an evaluation less; 1 to 3 % more time at 128 tokens)
 constexpr float kFCgLow = 0.1f, kFCgLoose = 5.0e-3f;
 constexpr float kFScaleJump = 0.5f;        // distance of the common scale from which its curve is inverted exactly
 constexpr float kFSmallSlack = 1.0e-4f;     // share of the mass below which Tn - sum g is mostly rounding in fp32
@@ -1307,6 +1308,8 @@ __device__ __noinline__ double2 eval_hessian(int m, int n, int slack, bool coars
 // One thread per row (or share of a row), the row in registers; the pipelined form of the method (Ghysels and Vanroose), in which
 // the scalar products of an iteration do not wait for its matrix product: one barrier each, where Chronopoulos and Gear's form
 // with the shares summed through shared memory had three.  (50 tokens to 2e-4, one CTA alone: 3.76 k cycles, 3.87 k before; what it saves is barriers for the CTAs beside it.)
+// The step's product with s, which goes into the common scale, is summed once at the end: carried along by the recurrences it drifts
+// with them, and saves nothing (64 whole rows of 16 ids 94 us a call with the recurrence, 89 with the sum; 256 rows of n = 4, k = 8 58.0, 56.9).
 // The one eigenvalue is the common scale of the weights, the direction (1,...,1): H 1 = s, s_i = g2_i / w_i the rate at
 // which token i takes mass from the slack, tiny when the acceptance is close to one.  s is known exactly, so the diagonal
 // is set from the row sums (sm.Ld), s_i + sum_l |H_il| (whatever the rounding of the off-diagonal part, the matrix then has the
@@ -1331,47 +1334,60 @@ __device__ __noinline__ void cg_solve(int m, int slack, float kap, float lin, fl
     const float diag = on ? sd * fmaf(si, sd, sm.Ld[i]) : 1.f;
     const float v = slack ? si * sd : (on ? __fdividef(1.f, sd) : 0.f);
     float r = on ? fmaf(-lin, v, rhs * sd) : 0.f, x = 0.f, p = 0.f, s = 0.f, z = 0.f, w = 0.f;
-    float gam_old = 1.f, al_old = 1.f, goal = 0.f, vp = 0.f, vx = 0.f;
+    float gam_old = 1.f, al_old = 1.f, goal = 0.f;
+    int it;
     bool done = false;
     // (the quadrature nodes' arrays, which only evaluations use, take the warps' sums: tok_reduce's may still be read)
     static_assert(2 * C::kW * 16 <= 2 * kQC * 8, "warp sums");
     GR_PTR(float) sums = GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oTq), 4 * kQC, flag);
 #pragma unroll 1
-    for (int it = -1; it <= kFCgMax; it++) {
-        // products r.r, w.r, v.w, v.r (the first time v.r alone counts) over the rows, and w (r) for the matrix product
+    for (it = -1; it <= kFCgMax; it++) {
+        // products r.r, w.r, v.w (the first time only v.r) over the rows, and w (r) for the matrix product
         GR_PTR(float) vec = vec_buffer(sm, it & 1);
         const float in = it < 0 ? r : w;
         if (lead) vec[vec_pos<C>(i)] = in;
-        float d[4] = {r * r, w * r, v * w, v * r};
+        float d[3] = {r * r, w * r, v * in};
         __syncwarp();
 #pragma unroll
         for (int o = C::kNG; o < 32; o <<= 1) {
 #pragma unroll
-            for (int k = 0; k < 4; k++) d[k] += __shfl_xor_sync(0xffffffffu, d[k], o);
+            for (int k = 0; k < 3; k++) d[k] += __shfl_xor_sync(0xffffffffu, d[k], o);
         }
         GR_PTR(float) part = sums + 4 * C::kW * (it & 1);
-        if (lane == 0) st_f4(part + 4 * warp, make_float4(d[0], d[1], d[2], d[3]));
+        if (lane == 0) st_f4(part + 4 * warp, make_float4(d[0], d[1], d[2], 0.f));
         __syncthreads();
 #pragma unroll
         for (int u = 0; u < C::kW; u++) {
             const float4 t = ld_f4(part + 4 * u);
-            const float tv[4] = {t.x, t.y, t.z, t.w};
+            const float tv[3] = {t.x, t.y, t.z};
 #pragma unroll
-            for (int k = 0; k < 4; k++) d[k] = u == 0 ? tv[k] : d[k] + tv[k];
+            for (int k = 0; k < 3; k++) d[k] = u == 0 ? tv[k] : d[k] + tv[k];
         }
-        const float q = fmaf(v, kap * (it < 0 ? d[3] : d[2]), fmaf(diag, in, -dot_row<C>(row, vec)));
+        const float q = fmaf(v, kap * d[2], fmaf(diag, in, -dot_row<C>(row, vec)));
         if (it < 0) { w = q; continue; }
         const float gam = d[0];
         if (it == 0) goal = gam * rtol * rtol;
         if (gam <= goal) { done = true; break; }
         const float beta = it == 0 ? 0.f : __fdividef(gam, gam_old);
         const float al = __fdividef(gam, it == 0 ? d[1] : d[1] - beta * __fdividef(gam, al_old));
-        z = fmaf(beta, z, q); s = fmaf(beta, s, w); p = fmaf(beta, p, r); vp = fmaf(beta, vp, d[3]);
-        x = fmaf(al, p, x); r = fmaf(-al, s, r); w = fmaf(-al, z, w); vx = fmaf(al, vp, vx);
+        z = fmaf(beta, z, q); s = fmaf(beta, s, w); p = fmaf(beta, p, r);
+        x = fmaf(al, p, x); r = fmaf(-al, s, r); w = fmaf(-al, z, w);
         gam_old = gam; al_old = al;
     }
     float y = x * sd;
-    if (slack) y += shift + kap * vx;
+    if (slack) {
+        // the step's product with the direction, from the step itself: it decides where the common scale ends
+        float t = v * x;
+#pragma unroll
+        for (int o = C::kNG; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        GR_PTR(float) part = sums + 4 * C::kW * ((it + 1) & 1);
+        if (lane == 0) part[warp] = t;
+        __syncthreads();
+        float vx = 0.f;
+#pragma unroll
+        for (int u = 0; u < C::kW; u++) vx += part[u];
+        y += shift + kap * vx;
+    }
     // (not positive definite, NaN or slow: NaN)
     if (lead) sm.yv[i] = done ? y : __int_as_float(0x7fc00000);
     if (C::kNG > 1) __syncthreads();
@@ -1683,16 +1699,16 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
         if (dm > (float)kFStepClamp && on) dl = jump + (dl - (double)jump) * (double)__fdividef((float)kFStepClamp, dm);
         alpha = fmin(fmax(alpha + dl, -kFAlphaClamp), kFAlphaClamp);
         // Stop on a predicted residual, without another evaluation, after a step from a point evaluated in fp64 on the
-        // full grid.  Measured against the oracle's residual at the weights returned, 9500 such stops at tolerances of 1e-8,
-        // 3e-7 and 1e-5: every benchmark shape, random rows of 16 to 128 tokens with 2 to 32 drafts, and rows picked for
-        // prefixes that are almost tight (weights on several scales), inner systems and outer blocks:
+        // full grid.  Measured with this iteration against the oracle's residual at the weights returned, 7000 such stops at tolerances
+        // of 1e-8, 3e-7 and 1e-5: every benchmark shape, random rows of 16 to 128 tokens with 2 to 32 drafts, whole and truncated, and
+        // rows picked for prefixes that are almost tight (weights on several scales), 6231 in inner systems, 767 in outer blocks:
         // (i) By the step.  Second order: s2 = sum_i g_i delta_i^2 (each flow is a sum of terms exponential in alpha over
-        // positive normalisers; never above 8.5 s2 + the quadrature floor of ~3e-9, median 0.15 s2).  First order, after
-        // conjugate gradients: what the half-precision Hessian leaves of the residual, up to 0.03 of it (0.01 in outer
-        // blocks), plus the distance to the point where a reused one was formed.
+        // positive normalisers).  First order, after conjugate gradients: what the half-precision Hessian leaves of the residual,
+        // plus the distance to the point where a reused one was formed.  Left were never more than 8.5 s2 + 0.008 of the residual
+        // + the quadrature floor of ~3e-9, and never more than half of what is held against the tolerance.
         // (ii) By the ratio: the last full step on this grid contracted the residual by rho < 0.1, and the next one is taken
         // to contract by no less than that and its own length (along a direction in which the flows hardly change s2 says
-        // nothing, and half the length of the step is what it leaves: steps of 0.2 to 0.9 left 0.1 to 0.4 of the residual).
+        // nothing, and the length of the step times the residual is what it leaves: 0.63 of that in the worst of 23 such stops).
         // Neither is trusted when the factorisation cancelled all but a few percent of some diagonal entry, or, after
         // conjugate gradients, when the common scale of the weights has a slope of that order: with weights of
         // 1e5 and more the fp32 system stops producing Newton steps, the residual stays where it is while the steps, and
@@ -1734,7 +1750,7 @@ fast_solve_kernel(char* __restrict__ ws, char* __restrict__ params, int pstride,
     GR_CHECK_FLAG_DECL;
     GR_CHECK_FLAG_INIT;
     const bool fused = fa.draft != nullptr;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31;
     const long long b = blockIdx.x;
     char* pb = params + (size_t)b * pstride;
     ParamView pv = view_params(pb, kcap, V, GR_CHECK_FLAG);
