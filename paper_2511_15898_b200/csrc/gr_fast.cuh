@@ -1554,6 +1554,7 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
     double alpha_prev = alpha;
     int status = GR_NOT_CONVERGED, it = 0, stalls = 0, was_kind = -1;
     double rn = 0.0;
+    // (what steers the iteration only is fp32: it is compared with margins of three and more, and in fp64 cost 1 % at series of 16)
     float rprev = kFNone, lam = 1.f, dist = 0.f;
     float amax = 0.f, amin = 0.f;            // extreme log-weights
     bool ranged = false;                     // they are known for this point

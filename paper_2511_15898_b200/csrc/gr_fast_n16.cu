@@ -1,7 +1,7 @@
 // Fast solve kernels for series length 16 (draft counts up to 16).  Threads and CTAs per SM: supports of up to 128 tokens ran
 // 7 % faster on two CTAs of 256 threads than on three of 128 (4096 rows, k = 100: 1480 to 1378 us).  Up to 32 tokens four CTAs
-// of 128 threads are faster while they hold the batch (512 rows, k = 20: 95 to 91 us), six of 64 beyond (1777 rows, k = 8: 392
-// to 354 for the whole call).  At 64 tokens, where two CTAs of 256 for four of 128 lost a third at series length 8, the narrow ones stay.
+// of 128 threads are no slower while they hold the batch (512 rows, k = 20: 155 us a call for 160, fused 156 for 156), six of 64
+// faster beyond (1777 rows, k = 8: 267 us a call for 310).  At 64 tokens, where two CTAs of 256 for four of 128 lost a third at series length 8, the narrow ones stay.
 #include "gr_fast.cuh"
 
 namespace gr {

@@ -117,7 +117,7 @@ __device__ inline double block_min(double v, double* s_r)
 }
 
 // flag[0] of the instance's scratch region: bit j set when fullsort_alpha_kernel has to do the row for the j-th draft count.
-// 512 rows of 50257 in fp32: about 150 us (three passes with exp, 64-bit shared atomics and counts: 408).  Bound by
+// 512 rows of 50257 in fp32: 168 us (three passes with exp, 64-bit shared atomics and counts: 408).  Bound by
 // instruction issue (130 instructions per 32 ids; fp64 pipe 28 % busy, shared atomics hidden), not by the 206 MB it reads.
 template <typename T>
 __global__ void __launch_bounds__(kBkThreads)

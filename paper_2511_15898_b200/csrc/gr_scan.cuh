@@ -144,7 +144,7 @@ __device__ __forceinline__ void cluster_barrier() {
 }
 
 // The `need`-th largest of the threads' running maxima (16 leading key bits, rounded down); never below the old threshold.
-// (512 threads: 16 counting barriers, 0.3 us; one warp searching 512 values in shared memory took three times that.)
+// (16 counting barriers, 0.3 us at 512 threads; one warp searching 512 values in shared memory took three times that.)
 // Returns the length of the list, the same for every thread (nobody appends between the first of the barriers and the last).
 template <class SS>
 __device__ __forceinline__ int refine_tau(SS& sh, float mx, int need)
