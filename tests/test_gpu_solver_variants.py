@@ -83,7 +83,7 @@ def test_both_widths_of_a_variant(n, topk):
                                        (lambda: W.config3(batch=1024, device="cuda", V=9001, n=12, topk=50), 4.05)])
 def test_evaluations_per_instance(make, most):
     """Where an evaluation weighs more than the sweeps of the starting point there are enough of those for four evaluations (three
-    at k = 20) in nearly every instance: 4.00, 3.04 and 4.00 on such rows; with two sweeps less 4.07, 3.30 and 4.10."""
+    at k = 20) in nearly every instance: 4.01, 3.04 and 4.00 on these rows; with two sweeps less 4.07, 3.31 and 4.10."""
     wl = make()
     r = G.read_rule(G.solve(wl.q_logits, wl.p_logits, wl.n, wl.topk, wl.temp_target, wl.temp_draft))
     assert float((r.iters & 0xffff).double().mean()) <= most
