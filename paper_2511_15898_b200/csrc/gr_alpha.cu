@@ -50,7 +50,7 @@ alpha_kernel(const char* __restrict__ ws, int V, int topk, double temp_t, double
     if (tid < k) { s_key[tid] = key; s_id[tid] = my_id; }
     __syncthreads();
     const int rank = ratio_rank(GR_MKPTR(const unsigned long long, s_key, kMaxSupport, nullptr), GR_MKPTR(const int, s_id, kMaxSupport, nullptr),
-                                GR_MKPTR(int, s_at, kMaxSupport, nullptr), k, key, my_id);
+                                GR_MKPTR(int, s_at, kMaxSupport, nullptr), 0, tid < k ? k : 0, key, my_id);
     if (tid < k) {
         s_tg[rank] = exp(a_i - lse_t);
         s_d[rank] = exp(b_i - lse_d);

@@ -58,21 +58,21 @@ __device__ __forceinline__ int count_above(GR_PTR(const unsigned long long) keys
     return n0 + n1;
 }
 
-// Position of this thread's token in the ratio order: larger keys first, equal keys by smaller id.  keys and ids are visible to all;
-// `scratch` is overwritten.  Every thread of the CTA calls it (as many threads as tokens at least).
-__device__ __forceinline__ int ratio_rank(GR_PTR(const unsigned long long) keys, GR_PTR(const int) ids, GR_PTR(int) scratch, int k,
+// Position of this thread's token among those of [lo, hi): larger keys first, equal keys by smaller id.  keys and ids are visible to all;
+// `scratch` is overwritten.  Every thread of the CTA calls it (as many threads as tokens at least; lo == hi: no token), a group's threads with one range.
+__device__ __forceinline__ int ratio_rank(GR_PTR(const unsigned long long) keys, GR_PTR(const int) ids, GR_PTR(int) scratch, int lo, int hi,
                                           unsigned long long key, int my_id)
 {
     const int tid = threadIdx.x;
-    const bool on = tid < k;
-    int rank = on ? count_above(keys, 0, k, key) : 0;
+    const bool on = lo < hi;
+    int rank = on ? lo + count_above(keys, lo, hi, key) : 0;
     // equal keys have met at one rank: whoever does not find himself there has company
     if (on) scratch[rank] = tid;
     __syncthreads();
     if (__syncthreads_or(on && scratch[rank] != tid)) {
         if (on) {
             int before = 0;
-            for (int j = 0; j < k; j++) before += (keys[j] == key && ids[j] < my_id) ? 1 : 0;
+            for (int j = lo; j < hi; j++) before += (keys[j] == key && ids[j] < my_id) ? 1 : 0;
             rank += before;
         }
     }
@@ -178,7 +178,7 @@ __device__ inline PrepResult prep_instance(const PrepSm& sm, const WsView& wv, H
     }
     // ---- ratio order: decreasing log-ratio key, equal keys by smaller id (Sec. 5.1)
     // (the reductions above made the keys visible)
-    const int rank = ratio_rank(GR_PCAST(const unsigned long long, sm.key), sm.itmp, sm.blk, k, key, my_id);
+    const int rank = ratio_rank(GR_PCAST(const unsigned long long, sm.key), sm.itmp, sm.blk, 0, on ? k : 0, key, my_id);
     if (on) {
         sm.id[rank] = my_id;
         sm.tg[rank] = tg_i;
@@ -265,48 +265,52 @@ __device__ inline PrepResult prep_instance(const PrepSm& sm, const WsView& wv, H
 //   inner:  T in H*,       gamma_T   = drf(H*)^n - drf(T)^n      <= tau,
 //   outer:  T in V \ H*,   epsilon_T = 1 - (drf(H*) + drf(T))^n  <= tau,
 // i.e. tokens in decreasing drf (equal drf: smaller id first) until the bound holds.  in_T[pos] = 1 / 0 for the
-// k support positions (ratio order); scratch: k ints.  Every thread of the CTA calls it (blockDim.x >= k).
+// k support positions (ratio order); scratch: k ints.  sm.key and sm.psi are overwritten.  Every thread of the CTA calls it (blockDim.x >= k,
+// two warps at least).  The bounds of both groups' prefixes fall with their length (sums and powers of numbers that grow are monotone in floating
+// point too), so a token is in the set if and only if the bound of those before it does not hold yet: one token per thread, and only the sums are a chain.
+// (One thread walking both groups, a power per token, took 23 k cycles of 50 tokens and n = 8: 512 rows of 128256, tau = 1e-3, solve 180 us, so 171.)
 __device__ inline void truncation_sets(const PrepSm& sm, GR_PTR(int) in_T, GR_PTR(int) scratch, int k, int jstar, int n,
                                        double tau)
 {
     const int tid = threadIdx.x;
-    if (tid < k) {
-        // rank inside the own group (H* or the outer support) by (drf descending, id ascending)
-        const bool inner = tid < jstar;
-        const int lo = inner ? 0 : jstar, hi = inner ? jstar : k;
-        const double dv = sm.d[tid];
-        const int iv = sm.id[tid];
-        int rank = 0;
+    // rank inside the own group (H* or the outer support) by (drf descending, id ascending)
+    const bool on = tid < k, inner = tid < jstar;
+    const int lo = inner ? 0 : jstar, hi = inner ? jstar : k;
+    const double dv = on ? sm.d[tid] : 0.0;
+    GR_PTR(unsigned long long) keys = GR_PCAST(unsigned long long, sm.key);
+    if (on) keys[tid] = order_key(dv);
+    __syncthreads();
+    const int rank = ratio_rank(keys, sm.id, scratch, lo, on ? hi : lo, order_key(dv), on ? sm.id[tid] : 0);
+    __syncthreads();
+    if (on) { scratch[rank] = tid; sm.key[rank] = dv; }
+    __syncthreads();
+    // sums before a token, in order: a thread for each group (the outer one's begin with the mass of H*), eight loads ahead of the additions
+    if (tid == 0 || tid == 32) {
+        const int b0 = tid == 0 ? 0 : jstar, b1 = tid == 0 ? jstar : k;
+        double acc = tid == 0 ? 0.0 : sm.Dr[jstar];
 #pragma unroll 1
-        for (int j = lo; j < hi; j++) {
-            const double dj = sm.d[j];
-            rank += (dj > dv || (dj == dv && sm.id[j] < iv)) ? 1 : 0;
+        for (int j0 = b0; j0 < b1; j0 += 8) {
+            double v[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++) v[u] = sm.key[min(j0 + u, b1 - 1)];
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                if (j0 + u < b1) sm.psi[j0 + u] = acc;
+                acc += v[u];
+            }
         }
-        scratch[lo + rank] = tid;          // position of the group's rank-th token
-        in_T[tid] = 0;
     }
     __syncthreads();
-    if (tid == 0) {
-        double D = 0.0;
+    if (on) {
+        auto powi = [](double x, int e) {
+            double r = 1.0;
 #pragma unroll 1
-        for (int j = 0; j < jstar; j++) D += sm.d[j];
-        auto powi = [](double x, int e) { double r = 1.0; while (e > 0) { if (e & 1) r *= x; x *= x; e >>= 1; } return r; };
-        const double Dn = powi(D, n);
-        double c = 0.0, gam = Dn;
-#pragma unroll 1
-        for (int q = 0; q < jstar && gam > tau; q++) {
-            const int pos = scratch[q];
-            c += sm.d[pos]; in_T[pos] = 1;
-            gam = Dn - powi(c, n);
-        }
-        c = D;
-        double eps = 1.0 - Dn;
-#pragma unroll 1
-        for (int q = jstar; q < k && eps > tau; q++) {
-            const int pos = scratch[q];
-            c += sm.d[pos]; in_T[pos] = 1;
-            eps = 1.0 - powi(c, n);
-        }
+            for (; e > 0; e >>= 1) { if (e & 1) r *= x; x *= x; }
+            return r;
+        };
+        // (this thread's rank in the order of masses, whichever token it is)
+        const double before = powi(sm.psi[tid], n), all = powi(sm.Dr[jstar], n);
+        in_T[scratch[tid]] = (inner ? all - before : 1.0 - before) > tau ? 1 : 0;
     }
     __syncthreads();
 }
