@@ -85,9 +85,11 @@ extern "C" {
  *              of a diagonal entry left as the factorisation's pivot, or of the Hessian's trace
  *              as the slope along the common scale of the weights.
  *   max_iters  cap on gradient evaluations per system.            default 40
- *   quad_step  step of the trapezoid rule in the log-time variable used to
- *              evaluate the gradient integral; smaller is more accurate and
- *              slower (error roughly exp(-pi^2/quad_step)).        default 0.4
+ *   quad_step  accuracy of the rule by which the gradient integral is evaluated, as the step of
+ *              a trapezoid rule in the log-time variable; smaller is more accurate and
+ *              slower (error roughly exp(-pi^2/quad_step)).  From 0.4 up the faster kernel
+ *              takes rules with fewer nodes and a relative error of 2e-10, below that of
+ *              the step 0.4, where the weights of an instance allow it.      default 0.4
  *   scan_done_event  optional cudaEvent_t (as void*) recorded on `stream` between
  *              the streaming kernel and the solve kernel, so that a caller can
  *              time the two separately; NULL records nothing.      default NULL

@@ -27,6 +27,7 @@
 #pragma once
 #include "gr_prep.cuh"
 #include "gr_verify.cuh"
+#include "gr_quad.cuh"
 
 namespace gr {
 namespace fast {
@@ -364,15 +365,99 @@ __device__ __forceinline__ void hess_mma(const FSm<C>& sm, Frags<C>& fr, int kst
     }
 }
 
-// Quadrature grid in the log-time variable for log-weights in [amin, amax]: number of nodes, upper end, start of the
-// lower-tail compression.  (Where the grid lies does not matter to its accuracy: fp32.)
-__device__ __forceinline__ int quad_grid(float amax, float amin, int slack, float qstep, float& s_hi, float& s0)
+// Extent of a point's weights: the extreme log-weights, and the largest over the smallest total W of a tuple's weights (slack +
+// sum over its distinct tokens), infinite where the caller's quadrature step asks for more than the tables hold.
+struct Extent { float amax, amin, ratio; };
+__device__ __forceinline__ Extent extent_of(float amax, float amin, float wsum, int n, int slack, double qstep)
 {
-    const float wmax = Rx<float>::ex(amax), wmin = Rx<float>::ex(amin);
-    s_hi = Rx<float>::lg((float)kFTEnd / (slack ? 1.f + wmin : wmin));
-    s0 = -Rx<float>::lg((slack ? 1.f : 0.f) + wmax) - (float)kFDrop;
-    const int Q = (int)ceilf((s_hi - (s0 - (float)kFTail)) / qstep) + 1;
-    return Q > kFMaxNodes ? kFMaxNodes : Q;
+    Extent e;
+    e.amax = amax; e.amin = amin;
+    const float s = slack ? 1.f : 0.f;
+    // (rounded up: exponentials of fp32 log-weights are good to 1e-5)
+    e.ratio = qstep >= kTableStep ? 1.0001f * (s + fminf(wsum, (float)n * Rx<float>::ex(amax))) / (s + Rx<float>::ex(amin)) : INFINITY;
+    return e;
+}
+
+// Quadrature nodes for one evaluation, of R's accuracy.  Where 1 / W is wanted for W in a known interval, the fewest nodes are those of the
+// best exponential sum on it (gr_quad.cuh): 4 to 16 where the trapezoid rule in the log-time variable, with its lower tail
+// compressed below s0, takes 20 to 30 for the same accuracy.  The trapezoid rule serves the rest: wider intervals and steps below kTableStep.
+// (Where a grid lies does not matter to its accuracy: fp32.)
+template <typename R>
+struct Grid {
+    int Q;
+    bool table;
+    R unit;                         // table: 1 / smallest W; else the step
+    int at;                         // table: first entry
+    float s_hi, s0;
+    __device__ __forceinline__ Grid(const Extent& e, int slack, R qstep)
+    {
+        const float wmin = Rx<float>::ex(e.amin), s = slack ? 1.f : 0.f;
+        const int level = quad_level<R>(e.ratio);
+        table = level < QuadTable<R>::kLevels;
+        if (table) {
+            Q = 2 * (level + 1); at = level * (level + 1);
+            unit = (R)__fdividef(1.00005f, s + wmin);              // (any number not below 1 / lo)
+            s_hi = s0 = 0.f;
+        } else {
+            s_hi = Rx<float>::lg((float)kFTEnd / (s + wmin));
+            s0 = -Rx<float>::lg(s + Rx<float>::ex(e.amax)) - (float)kFDrop;
+            Q = min((int)ceilf((s_hi - (s0 - (float)kFTail)) / (float)qstep) + 1, kFMaxNodes);
+            unit = qstep; at = 0;
+        }
+    }
+    // node q (any q; beyond the last one of a table: the last) and its weight, e^(-t slack) included
+    __device__ __forceinline__ void node(int q, int slack, R& t, R& c) const
+    {
+        if (table) {
+            R tc, cc;
+            QuadTable<R>::load(at + min(q, Q - 1), tc, cc);
+            t = tc * unit; c = cc * unit;
+        } else {
+            const R s = (R)s_hi - unit * (R)q, e = Rx<R>::expneg(s - (R)s0);
+            t = Rx<R>::expneg(e - s);
+            c = unit * (R(1) + e) * t;
+        }
+        if (slack) c *= Rx<R>::expneg(t);
+    }
+};
+// Node slots of an evaluation's first phase (a power of two; the threads beyond one set share out the tokens).
+__device__ __forceinline__ int slot_bits(int nq) { return nq <= 8 ? 3 : nq <= 16 ? 4 : 5; }
+// Sums over the shares that a warp holds of the same nodes (32 >> bits lanes each), left in `row`: lanes that meet each go on with half
+// of the series, so two steps take 3/4 of NT shuffles.
+template <int N, typename R, class P>
+__device__ __forceinline__ void st_row(const P& row, const R* v)
+{
+    constexpr int kVec = 16 / (int)sizeof(R);
+#pragma unroll
+    for (int c = 0; c < N; c += N % kVec ? 1 : kVec) { if constexpr (N % kVec) row[c] = v[c]; else st_vec(row + c, v + c); }
+}
+template <int NT, typename R, class P>
+__device__ __forceinline__ void put_shares(R* S, int bits, bool on, const P& row)
+{
+    const int lane = threadIdx.x & 31;
+    if (bits == 5) {
+        if (on) st_row<NT>(row, S);
+        return;
+    }
+    __syncwarp();
+    auto meet = [&](int half, int o) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int c = 0; c < NT / 2; c++) {
+            if (c < half) {
+                const R send = up ? S[c] : S[c + half], keep = up ? S[c + half] : S[c];
+                S[c] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        }
+    };
+    meet(NT / 2, 16);
+    const int c0 = lane & 16 ? NT / 2 : 0;
+    if (bits == 3) {
+        meet(NT / 4, 8);
+        if (on) st_row<NT / 4>(row + c0 + (lane & 8 ? NT / 4 : 0), S);
+    } else if (on) {
+        st_row<NT / 2>(row + c0, S);
+    }
 }
 
 // Sum of (g, g2) over the copies of the token threads, in the same order everywhere.  (A barrier before the array is written
@@ -449,17 +534,17 @@ __device__ __forceinline__ double recip(double x) { return __drcp_rn(x); }
 // the token's mass.  Errors against 96 points and fp64 throughout, n = 17 to 32, largest mass 0.12 to 0.6: flows 1e-11 in
 // fp64, 1e-7 in fp32; scaled Hessian 2e-5 from 11-bit operands.
 template <class C, typename R, bool kJac>
-__device__ __forceinline__ void eval_contour(const FSm<C>& sm, int m, int slack, double qstep_d, int jstride, float amax,
-                                             float amin, double w_own, float z_own, double& g_out, double& g2_out, Frags<C>& fr)
+__device__ __forceinline__ void eval_contour(const FSm<C>& sm, int m, int slack, double qstep_d, int jstride, const Extent& ext,
+                                             double w_own, float z_own, double& g_out, double& g2_out, Frags<C>& fr)
 {
     constexpr int T = C::T;
     const CSm<C, R> cs(sm);
     GR_PTR(double) cw = GR_MKPTR(double, reinterpret_cast<double*>(sm.base + C::oCd), 2 * C::NT, sm.flag);
     const int tid = threadIdx.x, i = tid % C::MP, ng = tid / C::MP;
     const int np = (int)sm.scal[SC_NP];
-    const R qstep = (R)qstep_d, wi = (R)w_own;
-    float s_hi, s0;
-    const int Q = quad_grid(amax, amin, slack, (float)qstep_d, s_hi, s0);
+    const R wi = (R)w_own;
+    const Grid<R> grid(ext, slack, (R)qstep_d);
+    const int Q = grid.Q;
     R g = R(0), g2 = R(0);
     if (kJac) {
 #pragma unroll
@@ -471,22 +556,22 @@ __device__ __forceinline__ void eval_contour(const FSm<C>& sm, int m, int slack,
 #pragma unroll 1
     for (int q0 = 0; q0 < Q; q0 += kQC) {
         const int nq = min(kQC, Q - q0);
-        const int slots = nq <= 16 ? 16 : 32;
-        const int q = tid & (slots - 1), G = T / slots, grp = tid / slots;
         // ---- x of every token at this thread's node
-        const R s = (R)s_hi - qstep * (R)(q0 + q);
-        const R e = Rx<R>::expneg(s - (R)s0);
-        const R t = Rx<R>::expneg(e - s);
-        if (tid < nq) {
-            const R c0 = qstep * (R(1) + e) * t * (slack ? Rx<R>::expneg(t) : R(1));
-            cs.tq[q] = t; cs.cq[q] = c0;
-            if (kJac) sm.kq[q] = sqrtf((float)((R)jstride * c0 * t));
-        }
+        // (threads are dealt to nodes evenly: 5 nodes of 24 points are one round of 128 threads)
+        const int grp = tid / nq, q = tid - grp * nq, G = T / nq;
+        if (grp < G) {
+            R t, c0;
+            grid.node(q0 + q, slack, t, c0);
+            if (grp == 0) {
+                cs.tq[q] = t; cs.cq[q] = c0;
+                if (kJac) sm.kq[q] = sqrtf((float)((R)jstride * c0 * t));
+            }
 #pragma unroll 2
-        for (int j = grp; j < m; j += G) cs.X[j * C::kXS + q] = Rx<R>::expneg(t * cs.w[j]);
+            for (int j = grp; j < m; j += G) cs.X[j * C::kXS + q] = Rx<R>::expneg(t * cs.w[j]);
+        }
         __syncthreads();
         // ---- product of the factors, one thread per (node, point)
-        if (q < nq) {
+        if (grp < G) {
 #pragma unroll 1
             for (int p = grp; p < np; p += G) {
                 R a = (R)cw[2 * p], b = (R)cw[2 * p + 1];
@@ -510,15 +595,15 @@ __device__ __forceinline__ void eval_contour(const FSm<C>& sm, int m, int slack,
             }
         }
         __syncthreads();
-        // ---- g: one thread per token; with kJac the operands of the contraction for every jstride-th node
-        const int span = kJac ? jstride * C::JC : nq;
+        // ---- g: one thread per token, its copies share out the points; with kJac the operands of the contraction for every jstride-th node
+        const int span = kJac ? jstride * C::JC : nq, pw = np / C::kNG;
 #pragma unroll 1
         for (int qa = 0; qa < nq; qa += span) {
             const int qb = min(nq, qa + span);
             const int nst = kJac ? (qb - qa + jstride - 1) / jstride : 0;
             if (live) {
 #pragma unroll 1
-                for (int q2 = qa + ng; q2 < qb; q2 += C::kNG) {
+                for (int q2 = qa; q2 < qb; q2++) {
                     const R t2 = cs.tq[q2], c0 = cs.cq[q2];
                     const R x = i < m ? cs.X[i * C::kXS + q2] : R(0);
                     const R ux = wi * x;
@@ -527,7 +612,7 @@ __device__ __forceinline__ void eval_contour(const FSm<C>& sm, int m, int slack,
                     const int f0 = stage ? (q2 - qa) / jstride * np : 0;
                     R v0 = R(0), v1 = R(0);
 #pragma unroll 4
-                    for (int p = 0; p < np; p++) {
+                    for (int p = ng * pw; p < (ng + 1) * pw; p++) {
                         R er, ei, pr, pi;
                         ld_c(cs.E + 2 * (p * C::MP + i), er, ei);
                         ld_c(cs.P + 2 * (p * kQC + q2), pr, pi);
@@ -567,15 +652,6 @@ __device__ __forceinline__ void eval_contour(const FSm<C>& sm, int m, int slack,
     sum_copies<C>(sm, g_out, g2_out);
 }
 
-// Node of the quadrature grid at s = s_hi - qstep q, lower tail compressed below s0: t and its weight.
-template <typename R>
-__device__ __forceinline__ R quad_node(float s_hi, float s0, R qstep, int q, R& e)
-{
-    const R s = (R)s_hi - qstep * (R)q;
-    e = Rx<R>::expneg(s - (R)s0);
-    return Rx<R>::expneg(e - s);
-}
-
 // Series S of d/dlambda log P -> product series P[0 .. n-1] of one node, handed to put(e, P[e]) (zeros at and beyond n).
 template <int NT, typename R, class F>
 __device__ __forceinline__ void product_series(const R* S, int n, F put)
@@ -595,18 +671,18 @@ __device__ __forceinline__ void product_series(const R* S, int n, F put)
 }
 
 // Gradient g and the Hessian's diagonal part g2 at the weights in shared memory (this thread's in w_own), in fp64.
-//   amax, amin  extreme log-weights;  hs = sigma * (draft mass above the block)
+//   ext  extent of the weights;  hs = sigma * (draft mass above the block)
 // Every token thread (all copies) gets g and g2.
 template <class C>
-__device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, double hs, int slack, double qstep, float amax,
-                                            float amin, double w_own, double ds_own, double& g_out, double& g2_out)
+__device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, double hs, int slack, double qstep, const Extent& ext,
+                                            double w_own, double ds_own, double& g_out, double& g2_out)
 {
     constexpr int NT = C::NT, T = C::T;
     typedef double R;
     const RSm<C, R> rs(sm);
     const int tid = threadIdx.x, i = tid % C::MP, ng = tid / C::MP;
-    float s_hi, s0;
-    const int Q = quad_grid(amax, amin, slack, (float)qstep, s_hi, s0);
+    const Grid<R> grid(ext, slack, qstep);
+    const int Q = grid.Q;
     const R wi = w_own, dsi = ds_own;
     R dp[NT <= 8 ? NT + 1 : 1];
     if (NT <= 8) {
@@ -619,16 +695,13 @@ __device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, doub
 #pragma unroll 1
     for (int q0 = 0; q0 < Q; q0 += kQC) {
         const int nq = min(kQC, Q - q0);
-        // ---- S: this thread's share of the tokens at its node (16 or 32 node slots)
-        const bool narrow = nq <= 16;
-        const int q = tid & (narrow ? 15 : 31), G = T / (narrow ? 16 : 32), grp = tid / (narrow ? 16 : 32);
+        // ---- S: this thread's share of the tokens at its node
+        const int bits = slot_bits(nq), q = tid & ((1 << bits) - 1), G = T >> bits, grp = tid >> bits;
         constexpr int kSS = NT + 2;                                // row stride of the shares: conflict-free vector access
         {
-            R e;
-            const R t = quad_node<R>(s_hi, s0, qstep, q0 + q, e);
-            if (tid < nq) {
-                rs.tq[q] = t; rs.cq[q] = qstep * (R(1) + e) * t * (slack ? Rx<R>::expneg(t) : R(1));
-            }
+            R t, c0;
+            grid.node(q0 + q, slack, t, c0);
+            if (tid < nq) { rs.tq[q] = t; rs.cq[q] = c0; }
             R S[NT];
 #pragma unroll
             for (int c = 0; c < NT; c++) S[c] = R(0);
@@ -656,15 +729,7 @@ __device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, doub
                     }
                 }
             }
-            if (narrow) {
-#pragma unroll
-                for (int c = 0; c < NT; c++) S[c] += __shfl_xor_sync(0xffffffffu, S[c], 16);
-            }
-            if (q < nq && (!narrow || (tid & 16) == 0)) {
-                GR_PTR(R) row = rs.SP + ((tid >> 5) * 32 + q) * kSS;
-#pragma unroll
-                for (int c = 0; c < NT; c += 2) st_vec(row + c, S + c);
-            }
+            put_shares<NT, R>(S, bits, q < nq, rs.SP + ((tid >> 5) * 32 + q) * kSS);
         }
         __syncthreads();
         // ---- P: one thread per node.  PP[j] = P[n - 1 - j], so that PP[c - 1] pairs with h[c] in [lambda^n] P h
@@ -726,16 +791,16 @@ __device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, doub
 // its own results; packed, a wait serves two.  (4096 rows of n = 16, k = 100: 1552 to 1480 us, 64 whole rows of
 // 16 ids 70 to 63, headline 163 to 159.)
 template <class C>
-__device__ __forceinline__ void eval_low(const FSm<C>& sm, int m, int n, float hs, int slack, float qstep, int jstride, float amax,
-                                         float amin, float wi, float dsi, float z_own, double& g_out, double& g2_out, Frags<C>& fr)
+__device__ __forceinline__ void eval_low(const FSm<C>& sm, int m, int n, float hs, int slack, float qstep, int jstride, const Extent& ext,
+                                         float wi, float dsi, float z_own, double& g_out, double& g2_out, Frags<C>& fr)
 {
     constexpr int NT = C::NT, T = C::T, kRow2 = 2 * C::kRow;
     static_assert(C::JC % 2 == 0, "whole pairs of nodes");
     typedef float R;
     const RSm<C, R> rs(sm);
     const int tid = threadIdx.x, i = tid % C::MP, ng = tid / C::MP;
-    float s_hi, s0;
-    const int Q = quad_grid(amax, amin, slack, qstep, s_hi, s0);
+    const Grid<R> grid(ext, slack, qstep);
+    const int Q = grid.Q;
     F2 dp[NT <= 8 ? NT + 1 : 1];
     if (NT <= 8) {
         float pw = 1.f;
@@ -752,17 +817,16 @@ __device__ __forceinline__ void eval_low(const FSm<C>& sm, int m, int n, float h
 #pragma unroll 1
     for (int q0 = 0; q0 < Q; q0 += kQC) {
         const int nq = min(kQC, Q - q0), nqp = (nq + 3) & ~3;
-        // ---- S: this thread's share of the pairs of tokens at its node (16 or 32 node slots)
-        const bool narrow = nq <= 16;
-        const int q = tid & (narrow ? 15 : 31), G = T / (narrow ? 16 : 32), grp = tid / (narrow ? 16 : 32);
+        // ---- S: this thread's share of the pairs of tokens at its node
+        const int bits = slot_bits(nq), q = tid & ((1 << bits) - 1), G = T >> bits, grp = tid >> bits;
         constexpr int kSS = NT + 4;                                // row stride of the shares: conflict-free vector access
         {
-            R e;
-            const R t = quad_node<R>(s_hi, s0, qstep, q0 + q, e);
+            R t, c0;
+            grid.node(q0 + q, slack, t, c0);
             if (tid < nqp) {
                 // (places beyond the last node: weight zero)
-                const R c0 = tid < nq ? qstep * (R(1) + e) * t * (slack ? Rx<R>::expneg(t) : R(1)) : 0.f;
                 const int at = place(tid);
+                c0 = tid < nq ? c0 : 0.f;
                 rs.tq[at] = tid < nq ? t : 0.f; rs.cq[at] = c0;
                 sm.kq[at] = sqrtf((float)jstride * c0 * t);
             }
@@ -798,15 +862,7 @@ __device__ __forceinline__ void eval_low(const FSm<C>& sm, int m, int n, float h
             R S[NT];
 #pragma unroll
             for (int c = 0; c < NT; c++) S[c] = S2[c].lo() + S2[c].hi();
-            if (narrow) {
-#pragma unroll
-                for (int c = 0; c < NT; c++) S[c] += __shfl_xor_sync(0xffffffffu, S[c], 16);
-            }
-            if (q < nq && (!narrow || (tid & 16) == 0)) {
-                GR_PTR(R) row = rs.SP + ((tid >> 5) * 32 + q) * kSS;
-#pragma unroll
-                for (int c = 0; c < NT; c += 4) st_vec(row + c, S + c);
-            }
+            put_shares<NT, R>(S, bits, q < nq, rs.SP + ((tid >> 5) * 32 + q) * kSS);
         }
         __syncthreads();
         // ---- P: one thread per node.  PP[j] = P[n - 1 - j], so that PP[c - 1] pairs with h[c] in [lambda^n] P h
@@ -919,14 +975,14 @@ __device__ __forceinline__ void eval_low(const FSm<C>& sm, int m, int n, float h
 
 // The fp64 evaluation, kept out of line (it is called once or twice per system, and its registers stay its own).
 template <class C>
-__device__ __noinline__ double2 eval_fp64(int m, int n, int slack, bool coarse, float amax, float amin, int* flag)
+__device__ __noinline__ double2 eval_fp64(int m, int n, int slack, bool coarse, Extent ext, int* flag)
 {
     const FSm<C> sm(flag);
     const int i = threadIdx.x % C::MP;
     const double qstep = sm.scal[SC_QSTEP] * (coarse ? 2.0 : 1.0);
     double2 r;
-    if constexpr (C::kContour) { Frags<C> none; eval_contour<C, double, false>(sm, m, slack, qstep, 1, amax, amin, sm.wd[i], 0.f, r.x, r.y, none); }
-    else eval_system<C>(sm, m, n, sm.scal[SC_HS], slack, qstep, amax, amin, sm.wd[i], i < m ? sm.dsd[i] : 0.0, r.x, r.y);
+    if constexpr (C::kContour) { Frags<C> none; eval_contour<C, double, false>(sm, m, slack, qstep, 1, ext, sm.wd[i], 0.f, r.x, r.y, none); }
+    else eval_system<C>(sm, m, n, sm.scal[SC_HS], slack, qstep, ext, sm.wd[i], i < m ? sm.dsd[i] : 0.0, r.x, r.y);
     return r;
 }
 
@@ -1229,7 +1285,7 @@ template <class C> __device__ __forceinline__ float rs_ds(const FSm<C>& sm, int 
 // With `chol` a Cholesky factorisation instead, for systems conjugate gradients do not get through.  `given`: the gradient
 // and the diagonal part come from the caller, in fp64.
 template <class C>
-__device__ __noinline__ double2 eval_hessian(int m, int n, int slack, bool coarse, float amax, float amin, bool given, bool chol,
+__device__ __noinline__ double2 eval_hessian(int m, int n, int slack, bool coarse, Extent ext, bool given, bool chol,
                                              double2 gg, int* flag)
 {
     const FSm<C> sm(flag);
@@ -1237,11 +1293,12 @@ __device__ __noinline__ double2 eval_hessian(int m, int n, int slack, bool coars
     Frags<C> fr;
     double g, g2;
     const double qstep = sm.scal[SC_QSTEP] * (coarse ? 2.0 : 1.0);
-    const int jstride = coarse ? 1 : 2;
+    // (a table's nodes all serve the Hessian, of the full trapezoid grid every other one)
+    const int jstride = coarse || quad_level<float>(ext.ratio) < QuadTable<float>::kLevels ? 1 : 2;
     const double rhs = i < m ? sm.rhs[sm.ord[i]] : 0.0;
     const float zr = i < m ? (float)rhs : 1.f, zi = rsqrtf(zr);
-    if constexpr (C::kContour) eval_contour<C, float, true>(sm, m, slack, qstep, jstride, amax, amin, sm.wd[i], i < m ? zi : 0.f, g, g2, fr);
-    else eval_low<C>(sm, m, n, (float)sm.scal[SC_HS], slack, (float)qstep, jstride, amax, amin, sm.wf[i], i < m ? rs_ds<C>(sm, i) : 0.f, i < m ? zi : 0.f, g, g2, fr);
+    if constexpr (C::kContour) eval_contour<C, float, true>(sm, m, slack, qstep, jstride, ext, sm.wd[i], i < m ? zi : 0.f, g, g2, fr);
+    else eval_low<C>(sm, m, n, (float)sm.scal[SC_HS], slack, (float)qstep, jstride, ext, sm.wf[i], i < m ? rs_ds<C>(sm, i) : 0.f, i < m ? zi : 0.f, g, g2, fr);
     if (given) { g = gg.x; g2 = gg.y; }
     if (chol) {
         // an outer block's function is constant along (1,...,1): that direction is pinned with 1/m everywhere
@@ -1556,7 +1613,7 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
     double rn = 0.0;
     // (what steers the iteration only is fp32: it is compared with margins of three and more, and in fp64 cost 1 % at series of 16)
     float rprev = kFNone, lam = 1.f, dist = 0.f;
-    float amax = 0.f, amin = 0.f;            // extreme log-weights
+    Extent ext{0.f, 0.f, 0.f};               // of the weights
     bool ranged = false;                     // they are known for this point
     // Three modes.  Low: gradient and Hessian in fp32, conjugate gradients.  Chord: fp64 gradient, the last Hessian.  High:
     // fp64 gradient, fp32 Hessian of the same point, with `chol` a Cholesky factorisation.  A single token that dominates a
@@ -1566,24 +1623,25 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
     bool full_grid = false, predicted = false, chol = false;
 #pragma unroll 1
     for (; it < max_iters; it++) {
-        // far from the solution the trapezoid step is doubled (quadrature error ~4e-6, far below the gradient norm
-        // there): half the nodes, every one of them a Hessian node.  Convergence is only declared on the full grid.
-        const bool coarse = rprev > kFCoarse && !full_grid && mode != kChord;
-        const int kind = 2 * mode + (coarse ? 1 : 0);
         const double w_i = !on ? 0.0 : (mode == kLow ? (double)__expf((float)alpha) : m_exp(alpha));
         if (lead) { sm.wd[i] = w_i; sm.wf[i] = (float)w_i; }
         if (!ranged) {
-            unsigned ext[2] = {on ? fkey((float)alpha) : 0u, on ? fkey(-(float)alpha) : 0u};
-            tok_reduce<C, 0, 0, 2>(sm, nullptr, nullptr, ext, par);
-            amax = fkey_inv(ext[0]); amin = -fkey_inv(ext[1]);
+            unsigned top[2] = {on ? fkey((float)alpha) : 0u, on ? fkey(-(float)alpha) : 0u};
+            float wsum = on ? Rx<float>::ex((float)alpha) : 0.f;
+            tok_reduce<C, 0, 1, 2>(sm, nullptr, &wsum, top, par);
+            ext = extent_of(fkey_inv(top[0]), -fkey_inv(top[1]), wsum, n, slack, sm.scal[SC_QSTEP]);
         }
         ranged = false;
+        // On the trapezoid rule the step is doubled far from the solution (quadrature error ~1e-4, far below the gradient norm
+        // there): half the nodes, every one of them a Hessian node.  Convergence is only declared on the full grid.
+        const bool coarse = rprev > kFCoarse && !full_grid && mode != kChord && !(ext.ratio <= kTableReach);
+        const int kind = 2 * mode + (coarse ? 1 : 0);
         __syncthreads();
         double2 gg = make_double2(0.0, 0.0);
-        if (mode != kLow) gg = eval_fp64<C>(m, n, slack, coarse, amax, amin, sm.flag);
+        if (mode != kLow) gg = eval_fp64<C>(m, n, slack, coarse, ext, sm.flag);
         if (mode == kHigh) __syncthreads();          // (sum_copies' array)
         if (mode != kChord)
-            gg = eval_hessian<C>(m, n, slack, coarse, amax, amin, mode == kHigh, chol, gg, sm.flag);
+            gg = eval_hessian<C>(m, n, slack, coarse, ext, mode == kHigh, chol, gg, sm.flag);
         const double g = gg.x, g2 = gg.y, rhs_i = on ? sm.rhs[sm.ord[i]] : 0.0, tol = sm.scal[SC_TOL];
         // The residual, and what the step below needs of the tokens: right-hand side b of the Newton system, s_i = g2_i / w_i,
         // and the sums of b, s and the Hessian's diagonal.
@@ -1683,9 +1741,10 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
         // largest component, s2 = sum g dl^2 (see below), the extremes of the weights after the step, and whether it is a number
         double s2 = on ? g * dl * dl : 0.0;
         const float an = (float)fmin(fmax(alpha + dl, -kFAlphaClamp), kFAlphaClamp);
-        unsigned ext[3] = {on ? __float_as_uint(fabsf((float)(dl - (double)jump))) : 0u, on ? fkey(an) : 0u, on ? fkey(-an) : 0u};
-        tok_reduce<C, 1, 0, 3>(sm, &s2, nullptr, ext, par);
-        const float dm = __uint_as_float(ext[0]), far = dm + fabsf(jump);
+        unsigned top[3] = {on ? __float_as_uint(fabsf((float)(dl - (double)jump))) : 0u, on ? fkey(an) : 0u, on ? fkey(-an) : 0u};
+        float wsum = on ? Rx<float>::ex(an) : 0.f;
+        tok_reduce<C, 1, 1, 3>(sm, &s2, &wsum, top, par);
+        const float dm = __uint_as_float(top[0]), far = dm + fabsf(jump);
         // (NaN for every thread or none)
         if (!(s2 < 1.0e300) || !(dm < kFNone)) {
             if (chol) break;                 // no usable step: the general kernel's
@@ -1693,7 +1752,7 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
             mode = kHigh; chol = true; full_grid = true; rprev = kFNone; was_kind = -1;
             continue;
         }
-        amax = fkey_inv(ext[1]); amin = -fkey_inv(ext[2]);
+        ext = extent_of(fkey_inv(top[1]), -fkey_inv(top[2]), wsum, n, slack, sm.scal[SC_QSTEP]);
         ranged = !(dm > (float)kFStepClamp);
         // a full Newton step below 1e-11 in alpha: the weights cannot be improved at this quadrature accuracy
         if (!fail && mode != kLow && far < 1.0e-11f) { status = GR_OK; it++; break; }
@@ -1747,6 +1806,7 @@ fast_solve_kernel(char* __restrict__ ws, char* __restrict__ params, int pstride,
                   const __grid_constant__ typename CircleOf<C::kContour>::type circle)
 {
     __shared__ int s_sel;
+    warm_tables();
     pdl_wait();
     GR_CHECK_FLAG_DECL;
     GR_CHECK_FLAG_INIT;

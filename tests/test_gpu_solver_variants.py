@@ -181,3 +181,26 @@ def test_instances_left_to_the_general_kernel():
     robust = G.Options(max_iters=2, force_robust=1)
     mixed, alone = (_median_us(lambda o=o: G.solve(q, p, 8, 50, tt, td, o)) for o in (opt, robust))
     assert mixed < 2.2 * alone, (mixed, alone)
+
+
+@pytest.mark.parametrize("n,k", [(2, 16), (4, 40), (8, 50), (16, 20), (16, 100), (20, 24), (32, 64)])
+@pytest.mark.parametrize("quad_step", [0.4, 0.39])
+def test_quadrature_rules_over_the_extents_of_the_weights(n, k, quad_step):
+    """The number of quadrature nodes follows the extent of the tuples' weights: rows from nearly equal distributions (weights over
+    many orders of magnitude) to unrelated ones (all weights small), by the tabulated sums (the default step) and by the trapezoid rule
+    (a smaller step).  Both rules' errors are below 1e-9 of a flow, far below the tolerance the norm is held to."""
+    g = torch.Generator(device="cuda").manual_seed(4100 + 40 * n + k)
+    noise = torch.tensor([0.02, 0.1, 0.3, 0.6, 1.0, 1.5, 2.5, 4.0], device="cuda").repeat(12)[:, None]
+    q = 2.0 * torch.randn(96, 150, generator=g, device="cuda")
+    p = q + noise * torch.randn(96, 150, generator=g, device="cuda")
+    wl = W.Workload("extents", 150, n, k, 1.0, 1.0, q, p, torch.zeros(96, n, dtype=torch.int32, device="cuda"),
+                    torch.full((96, 2), 0.5, device="cuda"))
+    rep = P.certify(wl, G.Options(quad_step=quad_step))
+    r = G.read_rule(G.solve(q, p, n, k, 1.0, 1.0, G.Options(quad_step=quad_step)))
+    extents = [float((1 + w[b == -1].max()) / (1 + w[b == -1].min())) for w, b in zip(r.w, r.block) if (b == -1).any()]
+    print(rep.summary(), min(extents), max(extents))
+    # (what the rows are for: 8 nodes and fewer, and 14 and more)
+    assert max(extents) > 29 and min(extents) < 6
+    assert rep.n_status_ok == rep.n_inst and rep.n_struct_mismatch == 0, (rep.summary(), rep.details[:5])
+    assert rep.alpha_err <= 1e-6 and rep.cert_solver_max <= 3.2e-7, rep.summary()
+    assert rep.n_underreported == 0 and rep.n_evaluated_off == 0, (rep.summary(), rep.details[:5])
