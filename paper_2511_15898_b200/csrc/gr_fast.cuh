@@ -36,7 +36,6 @@ constexpr double kFTEnd = 25.0;       // quadrature range constants, identical t
 constexpr double kFDrop = 1.0;
 constexpr double kFTail = 3.0;
 constexpr int kFMaxNodes = 128;
-constexpr int kQC = 32;               // quadrature nodes handled together
 constexpr double kFAlphaClamp = 80.0;
 constexpr double kFStepClamp = 3.0;
 constexpr double kFCoarse = 1.0e-2;        // above this residual the trapezoid step is doubled
@@ -58,10 +57,10 @@ constexpr float kFLeastSlack = 1.0e-9f;     // and the least share aimed at (the
 constexpr float kFNone = 1.0e30f;          // no residual or ratio yet
 
 // Compile-time geometry.  NT: series length (>= n), MP: padded support size, T: threads, JC: Hessian nodes staged
-// together, CTAS: CTAs per SM the registers are held to.
-template <int NT_, int MP_, int T_, int JC_, int CTAS_>
+// together, CTAS: CTAs per SM the registers are held to, QC: quadrature nodes handled together.
+template <int NT_, int MP_, int T_, int JC_, int CTAS_, int QC_ = 32>
 struct Cfg {
-    static constexpr int NT = NT_, MP = MP_, T = T_, JC = JC_, kCtas = CTAS_;
+    static constexpr int NT = NT_, MP = MP_, T = T_, JC = JC_, kCtas = CTAS_, kQC = QC_;
     static constexpr bool kContour = NT > 16;     // samples on a circle instead of series (NT: largest number of them)
     // Fixed-point sweeps of the starting point: five where an evaluation weighs more than the sweeps, three elsewhere.  Three take 0.02
     // to 0.26 evaluations an instance more up to 64 tokens (n = 8, 1024 rows: k = 50 3.995 to 4.080, k = 20 3.04 to 3.30).  Whole calls, us,
@@ -90,7 +89,8 @@ struct Cfg {
     static constexpr int kXS = kQC + 1;
     static constexpr int kPPBytes = kContour ? NT * kQC * 16 : kQC * kRow * 8;
     static constexpr int kSPMin = T * 16 > MP * 16 ? T * 16 : MP * 16;
-    static constexpr int kSPBytes = !kContour ? T * (NT + 2) * 8 : (MP * kXS * 8 > kSPMin ? MP * kXS * 8 : kSPMin);
+    static constexpr int kSPShares = kW * kQC * (NT + 2) * 8, kSPVec = T * 16 + 12 * (MP + 4 * kNG);
+    static constexpr int kSPBytes = !kContour ? (kSPShares > kSPVec ? kSPShares : kSPVec) : (MP * kXS * 8 > kSPMin ? MP * kXS * 8 : kSPMin);
     static constexpr int oPP = oKq + kQC * 4, oSP = oPP + kPPBytes, oSQ = oPP + NT * kQC * 8;
     static constexpr int oEd = oSP + kSPBytes, oEs = oEd + (kContour ? NT * MP * 16 : 0);
     static constexpr int oCd = oEs + (kContour ? NT * MP * 8 : 0);
@@ -153,7 +153,7 @@ struct FSm {
         trunc = GR_MKPTR(int, reinterpret_cast<int*>(sb + C::oTr), C::MP, ck);
         AS = GR_MKPTR(uint32_t, reinterpret_cast<uint32_t*>(sb + C::oU), C::kStage / 4, ck);
         HS = GR_MKPTR(uint32_t, reinterpret_cast<uint32_t*>(sb + C::oU + (C::kOps - 1) * C::kStage), C::kStage / 4, ck);
-        kq = GR_MKPTR(float, reinterpret_cast<float*>(sb + C::oKq), kQC, ck);
+        kq = GR_MKPTR(float, reinterpret_cast<float*>(sb + C::oKq), C::kQC, ck);
         Lp = GR_MKPTR(float, reinterpret_cast<float*>(sb + C::oU), C::kLFloats, ck);
         pi = GR_MKPTR(__half, reinterpret_cast<__half*>(sb + C::oU), C::MP * C::kNS, ck);
     }
@@ -174,8 +174,8 @@ template <class C, typename R>
 struct RSm {
     GR_PTR(R) tq, cq, PP, SP, w, ds;
     __device__ explicit RSm(const FSm<C>& sm) {
-        tq = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oTq), kQC, sm.flag);
-        cq = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oCq), kQC, sm.flag);
+        tq = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oTq), C::kQC, sm.flag);
+        cq = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oCq), C::kQC, sm.flag);
         PP = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oPP), C::kPPBytes / (int)sizeof(R), sm.flag);
         SP = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oSP), C::kSPBytes / (int)sizeof(R), sm.flag);
         const int ow = sizeof(R) == 4 ? C::oWf : C::oWd, od = sizeof(R) == 4 ? C::oDsf : C::oDsd;
@@ -483,13 +483,13 @@ struct CSm {
     GR_PTR(float) sq;
     __device__ explicit CSm(const FSm<C>& sm) {
         constexpr int k = (int)sizeof(R);
-        tq = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oTq), kQC, sm.flag);
-        cq = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oCq), kQC, sm.flag);
+        tq = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oTq), C::kQC, sm.flag);
+        cq = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oCq), C::kQC, sm.flag);
         X = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oSP), C::MP * C::kXS, sm.flag);
-        P = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oPP), 2 * C::NT * kQC, sm.flag);
+        P = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + C::oPP), 2 * C::NT * C::kQC, sm.flag);
         E = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + (k == 4 ? C::oEs : C::oEd)), 2 * C::NT * C::MP, sm.flag);
         w = GR_MKPTR(R, reinterpret_cast<R*>(sm.base + (k == 4 ? C::oWf : C::oWd)), C::MP, sm.flag);
-        sq = GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oSQ), 2 * C::NT * kQC, sm.flag);
+        sq = GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oSQ), 2 * C::NT * C::kQC, sm.flag);
     }
 };
 template <class P> __device__ __forceinline__ void ld_c(const P& p, float& a, float& b) { const float2 v = ld_f2(p); a = v.x; b = v.y; }
@@ -554,8 +554,8 @@ __device__ __forceinline__ void eval_contour(const FSm<C>& sm, int m, int slack,
     }
     const bool live = kJac || (i & ~31) < m;
 #pragma unroll 1
-    for (int q0 = 0; q0 < Q; q0 += kQC) {
-        const int nq = min(kQC, Q - q0);
+    for (int q0 = 0; q0 < Q; q0 += C::kQC) {
+        const int nq = min(C::kQC, Q - q0);
         // ---- x of every token at this thread's node
         // (threads are dealt to nodes evenly: 5 nodes of 24 points are one round of 128 threads)
         const int grp = tid / nq, q = tid - grp * nq, G = T / nq;
@@ -585,12 +585,12 @@ __device__ __forceinline__ void eval_contour(const FSm<C>& sm, int m, int slack,
                     b = fma(a, fy, b * fx);
                     a = a2;
                 }
-                st_c(cs.P + 2 * (p * kQC + q), a, b);
+                st_c(cs.P + 2 * (p * C::kQC + q), a, b);
                 if (kJac) {
                     // square root, either branch: only products of two of them are used
                     const float af = (float)a, bf = (float)b, mag = sqrtf(fmaf(af, af, bf * bf));
                     const float u = sqrtf(0.5f * (mag + fabsf(af))), v = u > 0.f ? __fdividef(0.5f * bf, u) : 0.f;
-                    st_c(cs.sq + 2 * (p * kQC + q), af >= 0.f ? u : fabsf(v), af >= 0.f ? v : copysignf(u, bf));
+                    st_c(cs.sq + 2 * (p * C::kQC + q), af >= 0.f ? u : fabsf(v), af >= 0.f ? v : copysignf(u, bf));
                 }
             }
         }
@@ -615,7 +615,7 @@ __device__ __forceinline__ void eval_contour(const FSm<C>& sm, int m, int slack,
                     for (int p = ng * pw; p < (ng + 1) * pw; p++) {
                         R er, ei, pr, pi;
                         ld_c(cs.E + 2 * (p * C::MP + i), er, ei);
-                        ld_c(cs.P + 2 * (p * kQC + q2), pr, pi);
+                        ld_c(cs.P + 2 * (p * C::kQC + q2), pr, pi);
                         const R fx = fma(x, er, R(1)), fy = x * ei;
                         const R inv = recip(fma(fx, fx, fy * fy));
                         // h = E conj(f) / |f|^2
@@ -624,7 +624,7 @@ __device__ __forceinline__ void eval_contour(const FSm<C>& sm, int m, int slack,
                         v0 = fma(pr, hr, v0); v1 = fma(-pi, hi, v1);
                         if (kJac && stage) {
                             float sr, si;
-                            ld_c(cs.sq + 2 * (p * kQC + q2), sr, si);
+                            ld_c(cs.sq + 2 * (p * C::kQC + q2), sr, si);
                             const float a = uz * (float)hr, b = uz * (float)hi;
                             const int f = f0 + p;
                             sm.AS[((f >> 3) * 4 + (f & 3)) * 2 * C::kTS + 2 * i + ((f >> 2) & 1)] =
@@ -693,8 +693,8 @@ __device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, doub
     R g = R(0), g2 = R(0);
     const bool live = (i & ~31) < m;
 #pragma unroll 1
-    for (int q0 = 0; q0 < Q; q0 += kQC) {
-        const int nq = min(kQC, Q - q0);
+    for (int q0 = 0; q0 < Q; q0 += C::kQC) {
+        const int nq = min(C::kQC, Q - q0);
         // ---- S: this thread's share of the tokens at its node
         const int bits = slot_bits(nq), q = tid & ((1 << bits) - 1), G = T >> bits, grp = tid >> bits;
         constexpr int kSS = NT + 2;                                // row stride of the shares: conflict-free vector access
@@ -729,7 +729,7 @@ __device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, doub
                     }
                 }
             }
-            put_shares<NT, R>(S, bits, q < nq, rs.SP + ((tid >> 5) * 32 + q) * kSS);
+            put_shares<NT, R>(S, bits, q < nq, rs.SP + ((tid >> 5) * C::kQC + q) * kSS);
         }
         __syncthreads();
         // ---- P: one thread per node.  PP[j] = P[n - 1 - j], so that PP[c - 1] pairs with h[c] in [lambda^n] P h
@@ -739,7 +739,7 @@ __device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, doub
             for (int c = 0; c < NT; c++) S[c] = R(0);
 #pragma unroll 2
             for (int k = 0; k < C::kW; k++) {
-                GR_PTR(const R) row = rs.SP + (k * 32 + tid) * kSS;
+                GR_PTR(const R) row = rs.SP + (k * C::kQC + tid) * kSS;
 #pragma unroll
                 for (int c = 0; c < NT; c += 2) {
                     R v[2];
@@ -815,8 +815,8 @@ __device__ __forceinline__ void eval_low(const FSm<C>& sm, int m, int n, float h
     // place of a node among the pairs: node 2 p + h of a coarse grid, nodes 4 p + {0, 2} and 4 p + {1, 3} of a full one
     auto place = [&](int q) { return jstride == 1 ? q : (q & ~3) | ((q & 1) << 1) | ((q >> 1) & 1); };
 #pragma unroll 1
-    for (int q0 = 0; q0 < Q; q0 += kQC) {
-        const int nq = min(kQC, Q - q0), nqp = (nq + 3) & ~3;
+    for (int q0 = 0; q0 < Q; q0 += C::kQC) {
+        const int nq = min(C::kQC, Q - q0), nqp = (nq + 3) & ~3;
         // ---- S: this thread's share of the pairs of tokens at its node
         const int bits = slot_bits(nq), q = tid & ((1 << bits) - 1), G = T >> bits, grp = tid >> bits;
         constexpr int kSS = NT + 4;                                // row stride of the shares: conflict-free vector access
@@ -862,7 +862,7 @@ __device__ __forceinline__ void eval_low(const FSm<C>& sm, int m, int n, float h
             R S[NT];
 #pragma unroll
             for (int c = 0; c < NT; c++) S[c] = S2[c].lo() + S2[c].hi();
-            put_shares<NT, R>(S, bits, q < nq, rs.SP + ((tid >> 5) * 32 + q) * kSS);
+            put_shares<NT, R>(S, bits, q < nq, rs.SP + ((tid >> 5) * C::kQC + q) * kSS);
         }
         __syncthreads();
         // ---- P: one thread per node.  PP[j] = P[n - 1 - j], so that PP[c - 1] pairs with h[c] in [lambda^n] P h
@@ -875,7 +875,7 @@ __device__ __forceinline__ void eval_low(const FSm<C>& sm, int m, int n, float h
                 for (int c = 0; c < NT; c++) S[c] = R(0);
 #pragma unroll 2
                 for (int k = 0; k < C::kW; k++) {
-                    GR_PTR(const R) part = rs.SP + (k * 32 + tid) * kSS;
+                    GR_PTR(const R) part = rs.SP + (k * C::kQC + tid) * kSS;
 #pragma unroll
                     for (int c = 0; c < NT; c += 4) {
                         R v[4];
@@ -1395,8 +1395,8 @@ __device__ __noinline__ void cg_solve(int m, int slack, float kap, float lin, fl
     int it;
     bool done = false;
     // (the quadrature nodes' arrays, which only evaluations use, take the warps' sums: tok_reduce's may still be read)
-    static_assert(2 * C::kW * 16 <= 2 * kQC * 8, "warp sums");
-    GR_PTR(float) sums = GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oTq), 4 * kQC, flag);
+    static_assert(2 * C::kW * 16 <= 2 * C::kQC * 8, "warp sums");
+    GR_PTR(float) sums = GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oTq), 4 * C::kQC, flag);
 #pragma unroll 1
     for (it = -1; it <= kFCgMax; it++) {
         // products r.r, w.r, v.w (the first time only v.r) over the rows, and w (r) for the matrix product
@@ -1970,8 +1970,8 @@ int launch_fast_t(char* ws, char* params, int pstride, int kcap, int V, int n, i
         double tol, int max_iters, double qstep, double tau, int batch, float *alpha_out, int *status_out,       \
         FusedArgs fa, cudaStream_t st
 #define GR_FAST_PASS ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol, max_iters, qstep, tau, batch, alpha_out, status_out, fa, st
-#define GR_FAST_INSTANTIATE(NAME, NT, MP, T, JC, CTAS)                                                            \
-    int launch_fast_##NAME(GR_FAST_ARGS) { return launch_fast_t<Cfg<NT, MP, T, JC, CTAS>>(GR_FAST_PASS); }
+#define GR_FAST_INSTANTIATE(NAME, ...)                                                                            \
+    int launch_fast_##NAME(GR_FAST_ARGS) { return launch_fast_t<Cfg<__VA_ARGS__>>(GR_FAST_PASS); }
 
 }  // namespace fast
 }  // namespace gr

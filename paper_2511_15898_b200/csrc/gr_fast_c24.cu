@@ -7,7 +7,7 @@ namespace gr {
 namespace fast {
 GR_FAST_INSTANTIATE(c24_m32, 24, 32, 128, 3, 4)
 GR_FAST_INSTANTIATE(c24_m32w, 24, 32, 128, 8, 2)
-GR_FAST_INSTANTIATE(c24_m64, 24, 64, 256, 4, 2)
-GR_FAST_INSTANTIATE(c24_m128, 24, 128, 256, 2, 1)
+GR_FAST_INSTANTIATE(c24_m64, 24, 64, 256, 4, 2, 16)
+GR_FAST_INSTANTIATE(c24_m128, 24, 128, 256, 4, 1, 16)
 }  // namespace fast
 }  // namespace gr
