@@ -1224,7 +1224,7 @@ __device__ __forceinline__ float newton_rhs(double g, double g2, double r)
 // Matrix-vector products with the half-precision matrices in sm.pi: thread t has row t / kNG and the (t % kNG)-th share of its
 // columns, so that the shares of a row meet in neighbouring lanes and not through shared memory.  The vector's shares are four
 // floats apart (their loads fall into different banks); three buffers behind what sum_copies uses.
-template <class C> __device__ __forceinline__ int vec_pos(int i) { return i + 4 * (i / (C::MP / C::kNG)); }
+template <class C, int kNG = C::kNG> __device__ __forceinline__ int vec_pos(int i) { return i + 4 * (i / (C::MP / kNG)); }
 template <class C>
 __device__ __forceinline__ GR_PTR(float) vec_buffer(const FSm<C>& sm, int which)
 {
@@ -1232,19 +1232,19 @@ __device__ __forceinline__ GR_PTR(float) vec_buffer(const FSm<C>& sm, int which)
     static_assert(C::T * 16 + 3 * kLen * 4 <= C::kSPBytes, "vector buffers");
     return GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oSP + C::T * 16) + which * kLen, kLen, sm.flag);
 }
-template <class C>
+template <int kNG>
 __device__ __forceinline__ float share_sum(float v)
 {
     __syncwarp();
 #pragma unroll
-    for (int o = 1; o < C::kNG; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int o = 1; o < kNG; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-template <class C>
+template <class C, int kNG>
 __device__ __forceinline__ void load_row(GR_PTR(const __half) mat, float* row)
 {
-    constexpr int kCol = C::MP / C::kNG;
-    GR_PTR(const __half) np = mat + (threadIdx.x / C::kNG) * C::kNS + (threadIdx.x % C::kNG) * kCol;
+    constexpr int kCol = C::MP / kNG;
+    GR_PTR(const __half) np = mat + (threadIdx.x / kNG) * C::kNS + (threadIdx.x % kNG) * kCol;
 #pragma unroll
     for (int c = 0; c < kCol; c += 8) {
         const uint4 v = ld_h8(np + c);
@@ -1256,25 +1256,25 @@ __device__ __forceinline__ void load_row(GR_PTR(const __half) mat, float* row)
         }
     }
 }
-template <class C>
+template <class C, int kNG>
 __device__ __forceinline__ float dot_row(const float* row, GR_PTR(const float) vec)
 {
-    constexpr int kCol = C::MP / C::kNG;
-    GR_PTR(const float) vp = vec + (threadIdx.x % C::kNG) * (kCol + 4);
+    constexpr int kCol = C::MP / kNG;
+    GR_PTR(const float) vp = vec + (threadIdx.x % kNG) * (kCol + 4);
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
     for (int c = 0; c < kCol; c += 4) {
         const float4 v = ld_f4(vp + c);
         a0 = fmaf(row[c], v.x, a0); a1 = fmaf(row[c + 1], v.y, a1); a2 = fmaf(row[c + 2], v.z, a2); a3 = fmaf(row[c + 3], v.w, a3);
     }
-    return share_sum<C>((a0 + a1) + (a2 + a3));
+    return share_sum<kNG>((a0 + a1) + (a2 + a3));
 }
 template <class C>
 __device__ __forceinline__ float row_times(GR_PTR(const __half) mat, GR_PTR(const float) vec)
 {
     float row[C::MP / C::kNG];
-    load_row<C>(mat, row);
-    return dot_row<C>(row, vec);
+    load_row<C, C::kNG>(mat, row);
+    return dot_row<C, C::kNG>(row, vec);
 }
 
 template <class C> __device__ __forceinline__ float rs_ds(const FSm<C>& sm, int i) { return RSm<C, float>(sm).ds[i]; }
@@ -1364,7 +1364,7 @@ __device__ __noinline__ double2 eval_hessian(int m, int n, int slack, bool coars
 // within 0.8 - 1.5 but one, so four or five iterations give four digits.
 // One thread per row (or share of a row), the row in registers; the pipelined form of the method (Ghysels and Vanroose), in which
 // the scalar products of an iteration do not wait for its matrix product: one barrier each, where Chronopoulos and Gear's form
-// with the shares summed through shared memory had three.  (50 tokens to 2e-4, one CTA alone: 3.76 k cycles, 3.87 k before; what it saves is barriers for the CTAs beside it.)
+// with the shares summed through shared memory had three.  (50 tokens to 2e-4, one CTA alone: 3.7 k cycles.)
 // The step's product with s, which goes into the common scale, is summed once at the end: carried along by the recurrences it drifts
 // with them, and saves nothing (64 whole rows of 16 ids 94 us a call with the recurrence, 89 with the sum; 256 rows of n = 4, k = 8 58.0, 56.9).
 // The one eigenvalue is the common scale of the weights, the direction (1,...,1): H 1 = s, s_i = g2_i / w_i the rate at
@@ -1375,79 +1375,104 @@ __device__ __noinline__ double2 eval_hessian(int m, int n, int slack, bool coars
 // (kap = -1 / sum s, lin = sum rhs / sum s.)
 // An outer block (slack == 0) has s = 0: the matrix is singular along the direction, e e^T / (e . e) is added, e = sqrt(H_ii)
 // (kap = 1 / (e . e), lin = 0).
+// Up to 32 tokens one warp does it all, a row per lane: its sums need no barrier and no shared memory, and an iteration takes half the
+// time (64 whole rows of 16 ids, a call: 70.7 -> 67.7 us; 256 rows of n = 4, k = 8: 55.4 -> 54.0).
 // In: sm.yv right-hand side, sm.dl s, visible to all.
 template <class C>
 __device__ __noinline__ void cg_solve(int m, int slack, float kap, float lin, float shift, float rtol, int* flag)
 {
-    constexpr int kCol = C::MP / C::kNG;                        // columns of this share
+    constexpr bool kOne = C::MP == 32;                          // one warp
+    constexpr int kNG = kOne ? 1 : C::kNG, kW = kOne ? 1 : C::kW, kCol = C::MP / kNG;       // copies, warps, columns of a share
     const FSm<C> sm(flag);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, i = tid / C::kNG;
-    const bool on = i < m, lead = tid % C::kNG == 0;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, i = tid / kNG;
+    if (kOne && warp > 0) { __syncthreads(); return; }
+    const bool on = i < m, lead = tid % kNG == 0;
     const float sd = sm.dg[i], rhs = sm.yv[i];
     float row[kCol];
-    load_row<C>(sm.pi, row);
+    load_row<C, kNG>(sm.pi, row);
     // diagonal from the row sums; v: the deflated (slack) or added (outer block) direction, kap its factor
     const float si = on && slack ? sm.dl[i] : 0.f;
     const float diag = on ? sd * fmaf(si, sd, sm.Ld[i]) : 1.f;
     const float v = slack ? si * sd : (on ? __fdividef(1.f, sd) : 0.f);
     float r = on ? fmaf(-lin, v, rhs * sd) : 0.f, x = 0.f, p = 0.f, s = 0.f, z = 0.f, w = 0.f;
-    float gam_old = 1.f, al_old = 1.f, goal = 0.f;
+    // (1 / r.r of the last iteration and that times 1 / al: formed behind it, off the chain)
+    float inv = 0.f, inva = 0.f, goal = 0.f;
     int it;
     bool done = false;
     // (the quadrature nodes' arrays, which only evaluations use, take the warps' sums: tok_reduce's may still be read)
     static_assert(2 * C::kW * 16 <= 2 * C::kQC * 8, "warp sums");
     GR_PTR(float) sums = GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oTq), 4 * C::kQC, flag);
+    // Sums over the rows.  The lanes that share a row hold the same numbers: each takes one of the three.
+    auto row_sums = [&](float* d, GR_PTR(float) part) {
+        __syncwarp();
+        if constexpr (kNG >= 4) {
+            float a = (lane & 3) == 0 ? d[0] : (lane & 3) == 1 ? d[1] : d[2];
+#pragma unroll
+            for (int o = kNG; o < 32; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (lane < 3) part[4 * warp + lane] = a;
+        } else if constexpr (kNG == 2) {
+            float a = lane & 1 ? d[1] : d[0], b = d[2];
+#pragma unroll
+            for (int o = kNG; o < 32; o <<= 1) { a += __shfl_xor_sync(0xffffffffu, a, o); b += __shfl_xor_sync(0xffffffffu, b, o); }
+            if (lane < 2) part[4 * warp + lane] = a;
+            if (lane == 0) part[4 * warp + 2] = b;
+        } else {
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+#pragma unroll
+                for (int k = 0; k < 3; k++) d[k] += __shfl_xor_sync(0xffffffffu, d[k], o);
+            }
+            if (!kOne && lane == 0) st_f4(part + 4 * warp, make_float4(d[0], d[1], d[2], 0.f));
+        }
+    };
 #pragma unroll 1
     for (it = -1; it <= kFCgMax; it++) {
         // products r.r, w.r, v.w (the first time only v.r) over the rows, and w (r) for the matrix product
         GR_PTR(float) vec = vec_buffer(sm, it & 1);
         const float in = it < 0 ? r : w;
-        if (lead) vec[vec_pos<C>(i)] = in;
+        if (lead) vec[vec_pos<C, kNG>(i)] = in;
         float d[3] = {r * r, w * r, v * in};
-        __syncwarp();
-#pragma unroll
-        for (int o = C::kNG; o < 32; o <<= 1) {
-#pragma unroll
-            for (int k = 0; k < 3; k++) d[k] += __shfl_xor_sync(0xffffffffu, d[k], o);
-        }
         GR_PTR(float) part = sums + 4 * C::kW * (it & 1);
-        if (lane == 0) st_f4(part + 4 * warp, make_float4(d[0], d[1], d[2], 0.f));
-        __syncthreads();
+        row_sums(d, part);
+        if constexpr (!kOne) {
+            __syncthreads();
 #pragma unroll
-        for (int u = 0; u < C::kW; u++) {
-            const float4 t = ld_f4(part + 4 * u);
-            const float tv[3] = {t.x, t.y, t.z};
+            for (int u = 0; u < kW; u++) {
+                const float4 t = ld_f4(part + 4 * u);
+                const float tv[3] = {t.x, t.y, t.z};
 #pragma unroll
-            for (int k = 0; k < 3; k++) d[k] = u == 0 ? tv[k] : d[k] + tv[k];
+                for (int k = 0; k < 3; k++) d[k] = u == 0 ? tv[k] : d[k] + tv[k];
+            }
         }
-        const float q = fmaf(v, kap * d[2], fmaf(diag, in, -dot_row<C>(row, vec)));
+        const float q = fmaf(v, kap * d[2], fmaf(diag, in, -dot_row<C, kNG>(row, vec)));
         if (it < 0) { w = q; continue; }
         const float gam = d[0];
         if (it == 0) goal = gam * rtol * rtol;
         if (gam <= goal) { done = true; break; }
-        const float beta = it == 0 ? 0.f : __fdividef(gam, gam_old);
-        const float al = __fdividef(gam, it == 0 ? d[1] : d[1] - beta * __fdividef(gam, al_old));
+        const float beta = gam * inv, den = fmaf(-beta * gam, inva, d[1]), al = __fdividef(gam, den);
         z = fmaf(beta, z, q); s = fmaf(beta, s, w); p = fmaf(beta, p, r);
         x = fmaf(al, p, x); r = fmaf(-al, s, r); w = fmaf(-al, z, w);
-        gam_old = gam; al_old = al;
+        inv = __fdividef(1.f, gam); inva = den * inv;
     }
     float y = x * sd;
     if (slack) {
         // the step's product with the direction, from the step itself: it decides where the common scale ends
         float t = v * x;
 #pragma unroll
-        for (int o = C::kNG; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        GR_PTR(float) part = sums + 4 * C::kW * ((it + 1) & 1);
-        if (lane == 0) part[warp] = t;
-        __syncthreads();
-        float vx = 0.f;
+        for (int o = kNG; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if constexpr (!kOne) {
+            GR_PTR(float) part = sums + 4 * C::kW * ((it + 1) & 1);
+            if (lane == 0) part[warp] = t;
+            __syncthreads();
+            t = 0.f;
 #pragma unroll
-        for (int u = 0; u < C::kW; u++) vx += part[u];
-        y += shift + kap * vx;
+            for (int u = 0; u < kW; u++) t += part[u];
+        }
+        y += shift + kap * t;
     }
     // (not positive definite, NaN or slow: NaN)
     if (lead) sm.yv[i] = done ? y : __int_as_float(0x7fc00000);
-    if (C::kNG > 1) __syncthreads();
+    if (kOne || C::kNG > 1) __syncthreads();
 }
 
 // Starting point (log-weights, left in sm.yv): token i wins the share w_i / (slack + w_i + S_i) of the tuples that contain it, S_i = the
@@ -1544,7 +1569,7 @@ __device__ __noinline__ void start_point(int m, int slack, int n, double Tm, int
                 group(c, pv);
             }
         }
-        const float Si = share_sum<C>((acc[0] + acc[1]) + (acc[2] + acc[3])) * A;
+        const float Si = share_sum<C::kNG>((acc[0] + acc[1]) + (acc[2] + acc[3])) * A;
         if (on) {
             wi = odds * (slack ? 1.f + Si : fmaxf(Si, 1e-30f));
             A = (slack ? 1.f : 0.f) + wi + Si;
