@@ -290,6 +290,16 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
 }
+// Brings `bytes` from p on into the first-level cache, a line per thread (as many threads as lines at least); nothing waits for it.
+__device__ __forceinline__ void touch_lines(const void* p, int bytes)
+{
+    const int at = 128 * (int)threadIdx.x;
+    if (at < bytes) {
+        unsigned v;
+        asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"((const char*)p + at));
+        (void)v;
+    }
+}
 // Programmatic dependent launch.  Every kernel of a call is launched with launch_pdl and begins with this: its launch is
 // prepared while the predecessor runs, but it touches no memory until the predecessor has completed (which, by the same
 // rule, had waited for its own).  No kernel lets its successor's CTAs in early (griddepcontrol.launch_dependents): they

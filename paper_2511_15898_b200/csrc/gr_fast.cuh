@@ -1841,6 +1841,8 @@ fast_solve_kernel(char* __restrict__ ws, char* __restrict__ params, int pstride,
     char* pb = params + (size_t)b * pstride;
     ParamView pv = view_params(pb, kcap, V, GR_CHECK_FLAG);
     const WsView wv = view_ws(ws, b, GR_CHECK_FLAG);
+    // (the record's lines on their way while its header is looked at)
+    touch_lines(wv.h, ws_stride());
     if (kcap == 0 || wv.h->bad != 0 || wv.h->count <= 0) {
         if (tid == 0) write_no_rule(pv.h, n, wv.h->bad != 0, alpha_out, status_out, b);
         if (fused) {
@@ -1904,6 +1906,8 @@ fast_solve_kernel(char* __restrict__ ws, char* __restrict__ params, int pstride,
                 if (other) { hi = j0 + __ffs(other) - 1; break; }
             }
         }
+        // (a block of one token: its weight says nothing)
+        if (!inner && hi - lo == 1 && !trunc) { lo = hi; continue; }
         const bool wanted = sel == -2 || (inner ? sel < 0 : sel == bk);
         // tokens of the system in ascending draft mass (fp32 is enough to order them; positions break ties, so that no two keys
         // are equal; what is not in the truncation set has the key of none)
