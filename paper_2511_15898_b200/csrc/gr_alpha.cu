@@ -12,7 +12,7 @@ __global__ void __launch_bounds__(kAlphaThreads)
 alpha_kernel(const char* __restrict__ ws, int V, int topk, double temp_t, double temp_d, NList nl,
              float* __restrict__ alpha_out, int* __restrict__ status_out)
 {
-    __shared__ unsigned long long s_key[kMaxSupport];
+    __shared__ __align__(16) unsigned long long s_key[kMaxSupport];
     __shared__ double s_tg[kMaxSupport], s_d[kMaxSupport], s_Tg[kMaxSupport + 1], s_Dr[kMaxSupport + 1];
     __shared__ int s_id[kMaxSupport], s_at[kMaxSupport];
     __shared__ double s_red[32];
@@ -46,10 +46,10 @@ alpha_kernel(const char* __restrict__ ws, int V, int topk, double temp_t, double
         lse_t = amax + log(asum);
     }
     // ratio order: decreasing log-ratio, equal keys by smaller id (Sec. 5.1)
-    const unsigned long long key = order_key(b_i - a_i);
-    if (tid < k) { s_key[tid] = key; s_id[tid] = my_id; }
+    const unsigned long long key = tid < k ? order_key(b_i - a_i) : 0ull;
+    if (tid < ((k + 3) & ~3)) { s_key[tid] = key; s_id[tid] = my_id; }
     __syncthreads();
-    const int rank = ratio_rank(GR_MKPTR(const unsigned long long, s_key, kMaxSupport, nullptr), GR_MKPTR(const int, s_id, kMaxSupport, nullptr),
+    const int rank = ratio_rank<true>(GR_MKPTR(const unsigned long long, s_key, kMaxSupport, nullptr), GR_MKPTR(const int, s_id, kMaxSupport, nullptr),
                                 GR_MKPTR(int, s_at, kMaxSupport, nullptr), 0, tid < k ? k : 0, key, my_id);
     if (tid < k) {
         s_tg[rank] = exp(a_i - lse_t);

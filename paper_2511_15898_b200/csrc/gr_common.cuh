@@ -85,6 +85,8 @@ template <class P> __device__ inline float4 ld_f4(const P& p) { return make_floa
 template <class P> __device__ inline float2 ld_f2(const P& p) { return make_float2(p[0], p[1]); }
 template <class P> __device__ inline double2 ld_d2(const P& p) { return make_double2(p[0], p[1]); }
 template <class P> __device__ inline uint2 ld_u2(const P& p) { return make_uint2(p[0], p[1]); }
+template <class P> __device__ inline uint4 ld_u4(const P& p) { return make_uint4(p[0], p[1], p[2], p[3]); }
+template <class P> __device__ inline ulonglong2 ld_ull2(const P& p) { return make_ulonglong2(p[0], p[1]); }
 template <class P> __device__ inline void st_f4(const P& p, float4 v) { p[0] = v.x; p[1] = v.y; p[2] = v.z; p[3] = v.w; }
 template <class P> __device__ inline void st_f2(const P& p, float2 v) { p[0] = v.x; p[1] = v.y; }
 template <class P> __device__ inline void st_d2(const P& p, double2 v) { p[0] = v.x; p[1] = v.y; }
@@ -102,6 +104,8 @@ __device__ __forceinline__ float4 ld_f4(const float* p) { return *reinterpret_ca
 __device__ __forceinline__ float2 ld_f2(const float* p) { return *reinterpret_cast<const float2*>(p); }
 __device__ __forceinline__ double2 ld_d2(const double* p) { return *reinterpret_cast<const double2*>(p); }
 __device__ __forceinline__ uint2 ld_u2(const uint32_t* p) { return *reinterpret_cast<const uint2*>(p); }
+__device__ __forceinline__ uint4 ld_u4(const uint32_t* p) { return *reinterpret_cast<const uint4*>(p); }
+__device__ __forceinline__ ulonglong2 ld_ull2(const unsigned long long* p) { return *reinterpret_cast<const ulonglong2*>(p); }
 __device__ __forceinline__ void st_f4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
 __device__ __forceinline__ void st_f2(float* p, float2 v) { *reinterpret_cast<float2*>(p) = v; }
 __device__ __forceinline__ void st_d2(double* p, double2 v) { *reinterpret_cast<double2*>(p) = v; }

@@ -281,19 +281,21 @@ __device__ __forceinline__ void tok_reduce(const FSm<C>& sm, double* d, float* f
 {
     static_assert(ND <= 2 && NF <= 4 && NU <= 4 && C::kTW <= 4, "a warp's slot is eight doubles");
     __syncwarp();
+    const int w = threadIdx.x >> 5;
+    if (C::kTW == 1 || w < C::kTW) {
 #pragma unroll
-    for (int k = 0; k < NU; k++) u[k] = __reduce_max_sync(0xffffffffu, u[k]);
+        for (int k = 0; k < NU; k++) u[k] = __reduce_max_sync(0xffffffffu, u[k]);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+        for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
-        for (int k = 0; k < ND; k++) d[k] += __shfl_xor_sync(0xffffffffu, d[k], o);
+            for (int k = 0; k < ND; k++) d[k] += __shfl_xor_sync(0xffffffffu, d[k], o);
 #pragma unroll
-        for (int k = 0; k < NF; k++) f[k] += __shfl_xor_sync(0xffffffffu, f[k], o);
+            for (int k = 0; k < NF; k++) f[k] += __shfl_xor_sync(0xffffffffu, f[k], o);
+        }
     }
     if (C::kTW == 1) return;
     GR_PTR(double) area = sm.red + 32 * par;
     par ^= 1;
-    const int w = threadIdx.x >> 5;
     if ((threadIdx.x & 31) == 0 && w < C::kTW) {
         GR_PTR(double) r = area + 8 * w;
         if (ND > 0) st_d2(r, make_double2(d[0], ND > 1 ? d[ND > 1 ? 1 : 0] : 0.0));
@@ -1627,10 +1629,12 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
     }
 
     }
-    double alpha = on ? (double)sm.yv[i] : 0.0;
+    // (the tokens' own numbers: the warps of their copies leave them out, where a reduction hands them the results)
+    const bool act = on && (C::kTW == 1 || lead);
+    double alpha = act ? (double)sm.yv[i] : 0.0;
     if (!slack) {
         const double mean = tok_sum<C>(sm, alpha, par) / (double)m;
-        if (on) alpha -= mean;
+        if (act) alpha -= mean;
     }
     alpha = fmin(fmax(alpha, -kFAlphaClamp), kFAlphaClamp);
     double alpha_prev = alpha;
@@ -1648,11 +1652,11 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
     bool full_grid = false, predicted = false, chol = false;
 #pragma unroll 1
     for (; it < max_iters; it++) {
-        const double w_i = !on ? 0.0 : (mode == kLow ? (double)__expf((float)alpha) : m_exp(alpha));
+        const double w_i = !act ? 0.0 : (mode == kLow ? (double)__expf((float)alpha) : m_exp(alpha));
         if (lead) { sm.wd[i] = w_i; sm.wf[i] = (float)w_i; }
         if (!ranged) {
-            unsigned top[2] = {on ? fkey((float)alpha) : 0u, on ? fkey(-(float)alpha) : 0u};
-            float wsum = on ? Rx<float>::ex((float)alpha) : 0.f;
+            unsigned top[2] = {act ? fkey((float)alpha) : 0u, act ? fkey(-(float)alpha) : 0u};
+            float wsum = act ? Rx<float>::ex((float)alpha) : 0.f;
             tok_reduce<C, 0, 1, 2>(sm, nullptr, &wsum, top, par);
             ext = extent_of(fkey_inv(top[0]), -fkey_inv(top[1]), wsum, n, slack, sm.scal[SC_QSTEP]);
         }
@@ -1667,13 +1671,13 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
         if (mode == kHigh) __syncthreads();          // (sum_copies' array)
         if (mode != kChord)
             gg = eval_hessian<C>(m, n, slack, coarse, ext, mode == kHigh, chol, gg, sm.flag);
-        const double g = gg.x, g2 = gg.y, rhs_i = on ? sm.rhs[sm.ord[i]] : 0.0, tol = sm.scal[SC_TOL];
+        const double g = gg.x, g2 = gg.y, rhs_i = act ? sm.rhs[sm.ord[i]] : 0.0, tol = sm.scal[SC_TOL];
         // The residual, and what the step below needs of the tokens: right-hand side b of the Newton system, s_i = g2_i / w_i,
         // and the sums of b, s and the Hessian's diagonal.
-        const float b = on ? newton_rhs(g, g2, rhs_i) : 0.f, s_i = on ? __fdividef((float)g2, (float)sm.wd[i]) : 0.f;
+        const float b = act ? newton_rhs(g, g2, rhs_i) : 0.f, s_i = act ? __fdividef((float)g2, (float)sm.wd[i]) : 0.f;
         if (!chol && lead) { sm.yv[i] = b; sm.dl[i] = s_i; }
-        double rg[2] = {on ? g : 0.0, on ? fabs(g - rhs_i) : 0.0};
-        float sums[3] = {b, slack ? s_i : 0.f, on ? (float)(g - g2) : 0.f};
+        double rg[2] = {act ? g : 0.0, act ? fabs(g - rhs_i) : 0.0};
+        float sums[3] = {b, slack ? s_i : 0.f, act ? (float)(g - g2) : 0.f};
         tok_reduce<C, 2, 3, 0>(sm, rg, sums, nullptr, par);
         if (C::kTW == 1) __syncthreads();
         rn = rg[1];
@@ -1749,25 +1753,25 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
             // (far from the solution the step need not be solved to more than the model is worth)
             const float rtol = mode == kLow ? fminf(fmaxf(kFCgLow * (float)rn, kFCgTol), kFCgLoose) : kFCgTol;
             cg_solve<C>(m, slack, slack ? -__fdividef(1.f, sums[1]) : __fdividef(1.f, sums[2]), lin, shift, rtol, sm.flag);
-            dl = on ? (double)sm.yv[i] : 0.0;
+            dl = act ? (double)sm.yv[i] : 0.0;
         } else {
             backward_subst<C>(m, sm.flag);
             __syncthreads();
             fail = sm.scal[SC_FAIL] != 0.0;
             pivot = (float)sm.scal[SC_PIVOT];
-            dl = on ? (double)sm.dl[i] : 0.0;
+            dl = act ? (double)sm.dl[i] : 0.0;
             // proportional-fitting step  alpha += log(rhs / g)  (and the full grid from here on)
-            if (fail) { full_grid = true; dl = on ? m_log(rhs_i / g) : 0.0; }
+            if (fail) { full_grid = true; dl = act ? m_log(rhs_i / g) : 0.0; }
         }
         if (!slack) {
             const double mean = tok_sum<C>(sm, dl, par) / (double)m;
-            if (on) dl -= mean;
+            if (act) dl -= mean;
         }
         // largest component, s2 = sum g dl^2 (see below), the extremes of the weights after the step, and whether it is a number
-        double s2 = on ? g * dl * dl : 0.0;
+        double s2 = act ? g * dl * dl : 0.0;
         const float an = (float)fmin(fmax(alpha + dl, -kFAlphaClamp), kFAlphaClamp);
-        unsigned top[3] = {on ? __float_as_uint(fabsf((float)(dl - (double)jump))) : 0u, on ? fkey(an) : 0u, on ? fkey(-an) : 0u};
-        float wsum = on ? Rx<float>::ex(an) : 0.f;
+        unsigned top[3] = {act ? __float_as_uint(fabsf((float)(dl - (double)jump))) : 0u, act ? fkey(an) : 0u, act ? fkey(-an) : 0u};
+        float wsum = act ? Rx<float>::ex(an) : 0.f;
         tok_reduce<C, 1, 1, 3>(sm, &s2, &wsum, top, par);
         const float dm = __uint_as_float(top[0]), far = dm + fabsf(jump);
         // (NaN for every thread or none)
@@ -1781,7 +1785,7 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
         ranged = !(dm > (float)kFStepClamp);
         // a full Newton step below 1e-11 in alpha: the weights cannot be improved at this quadrature accuracy
         if (!fail && mode != kLow && far < 1.0e-11f) { status = GR_OK; it++; break; }
-        if (dm > (float)kFStepClamp && on) dl = jump + (dl - (double)jump) * (double)__fdividef((float)kFStepClamp, dm);
+        if (dm > (float)kFStepClamp && act) dl = jump + (dl - (double)jump) * (double)__fdividef((float)kFStepClamp, dm);
         alpha = fmin(fmax(alpha + dl, -kFAlphaClamp), kFAlphaClamp);
         // Stop on a predicted residual, without another evaluation, after a step from a point evaluated in fp64 on the
         // full grid.  Measured with this iteration against the oracle's residual at the weights returned, 7000 such stops at tolerances
@@ -1818,7 +1822,7 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
         }
     }
     // (not converged here: the last accepted point, the general kernel's starting point)
-    if (lead) sm.wd[i] = on ? m_exp(status == GR_OK ? alpha : alpha_prev) : 0.0;
+    if (lead) sm.wd[i] = act ? m_exp(status == GR_OK ? alpha : alpha_prev) : 0.0;
     if (tid == 0) { sm.scal[SC_GNORM] = rn; sm.scal[SC_ITERS] = (double)(it | (predicted ? kItersPredicted : 0)); }
     return status;
 }
@@ -1909,15 +1913,23 @@ fast_solve_kernel(char* __restrict__ ws, char* __restrict__ params, int pstride,
         // (a block of one token: its weight says nothing)
         if (!inner && hi - lo == 1 && !trunc) { lo = hi; continue; }
         const bool wanted = sel == -2 || (inner ? sel < 0 : sel == bk);
-        // tokens of the system in ascending draft mass (fp32 is enough to order them; positions break ties, so that no two keys
-        // are equal; what is not in the truncation set has the key of none)
-        GR_PTR(unsigned long long) okey = GR_PCAST(unsigned long long, sm.wd);
-        unsigned long long mine = 0ull;
+        // tokens of the system in ascending draft mass (16 bits of it are enough to order them; positions break ties, so that no two keys
+        // are equal; what is not in the truncation set, or behind the last token, has the key of none)
+        GR_PTR(unsigned) okey = GR_PCAST(unsigned, sm.wd);
+        unsigned mine = 0u;
         const bool in = tid < hi - lo && (!trunc || sm.trunc[lo + tid] != 0);
-        if (in) mine = ((unsigned long long)(0x7fffffffu - __float_as_uint((float)sm.d[lo + tid])) << 32) | (unsigned)(MP - tid);
-        if (tid < hi - lo) okey[tid] = mine;
+        if (in) mine = ((0x7fffffffu - __float_as_uint((float)sm.d[lo + tid])) & ~127u) | (unsigned)(127 - tid);
+        if (tid < ((hi - lo + 3) & ~3)) okey[tid] = mine;
         const int m = __syncthreads_count(in);
-        if (in) sm.ord[count_above(okey, 0, hi - lo, mine)] = lo + tid;
+        if (in) {
+            int above = 0;
+#pragma unroll 4
+            for (int j = 0; j < hi - lo; j += 4) {
+                const uint4 o = ld_u4(okey + j);
+                above += (o.x > mine ? 1 : 0) + (o.y > mine ? 1 : 0) + (o.z > mine ? 1 : 0) + (o.w > mine ? 1 : 0);
+            }
+            sm.ord[above] = lo + tid;
+        }
         double hm = inner ? 0.0 : sm.Dr[lo];
         if (trunc && !inner) {
             // tuples counted: those inside (H* u T)^n, so the mass above the block is drf(H*) plus the T-part of the

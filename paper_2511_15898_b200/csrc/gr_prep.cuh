@@ -58,14 +58,29 @@ __device__ __forceinline__ int count_above(GR_PTR(const unsigned long long) keys
     return n0 + n1;
 }
 
+// The same over keys[0 .. k), 16-byte aligned, with zeros (no key) up to the next multiple of four.
+__device__ __forceinline__ int count_above_all(GR_PTR(const unsigned long long) keys, int k, unsigned long long key)
+{
+    int n0 = 0, n1 = 0;
+#pragma unroll 4
+    for (int j = 0; j < k; j += 4) {
+        const ulonglong2 a = ld_ull2(keys + j), b = ld_ull2(keys + j + 2);
+        n0 += (a.x > key ? 1 : 0) + (b.x > key ? 1 : 0);
+        n1 += (a.y > key ? 1 : 0) + (b.y > key ? 1 : 0);
+    }
+    return n0 + n1;
+}
+
 // Position of this thread's token among those of [lo, hi): larger keys first, equal keys by smaller id.  keys and ids are visible to all;
 // `scratch` is overwritten.  Every thread of the CTA calls it (as many threads as tokens at least; lo == hi: no token), a group's threads with one range.
+// kAll: one range from 0 on, padded for count_above_all.
+template <bool kAll>
 __device__ __forceinline__ int ratio_rank(GR_PTR(const unsigned long long) keys, GR_PTR(const int) ids, GR_PTR(int) scratch, int lo, int hi,
                                           unsigned long long key, int my_id)
 {
     const int tid = threadIdx.x;
     const bool on = lo < hi;
-    int rank = on ? lo + count_above(keys, lo, hi, key) : 0;
+    int rank = !on ? 0 : kAll ? count_above_all(keys, hi, key) : lo + count_above(keys, lo, hi, key);
     // equal keys have met at one rank: whoever does not find himself there has company
     if (on) scratch[rank] = tid;
     __syncthreads();
@@ -158,8 +173,9 @@ __device__ inline PrepResult prep_instance(const PrepSm& sm, const WsView& wv, H
         // (the streaming pass leaves the support in descending order: the first entry is the largest)
         b_i = b2.x; bmax = b2.y;
         key = order_key(b_i - a_i);
-        GR_PCAST(unsigned long long, sm.key)[tid] = key; sm.itmp[tid] = my_id;
+        sm.itmp[tid] = my_id;
     }
+    if (tid < ((k + 3) & ~3)) GR_PCAST(unsigned long long, sm.key)[tid] = key;
     const double eb = on ? m_exp(b_i - bmax) : 0.0;
     const double bsum = block_reduce_sum(eb, sm.red);
     double tg_i;
@@ -178,7 +194,7 @@ __device__ inline PrepResult prep_instance(const PrepSm& sm, const WsView& wv, H
     }
     // ---- ratio order: decreasing log-ratio key, equal keys by smaller id (Sec. 5.1)
     // (the reductions above made the keys visible)
-    const int rank = ratio_rank(GR_PCAST(const unsigned long long, sm.key), sm.itmp, sm.blk, 0, on ? k : 0, key, my_id);
+    const int rank = ratio_rank<true>(GR_PCAST(const unsigned long long, sm.key), sm.itmp, sm.blk, 0, on ? k : 0, key, my_id);
     if (on) {
         sm.id[rank] = my_id;
         sm.tg[rank] = tg_i;
@@ -280,7 +296,7 @@ __device__ inline void truncation_sets(const PrepSm& sm, GR_PTR(int) in_T, GR_PT
     GR_PTR(unsigned long long) keys = GR_PCAST(unsigned long long, sm.key);
     if (on) keys[tid] = order_key(dv);
     __syncthreads();
-    const int rank = ratio_rank(keys, sm.id, scratch, lo, on ? hi : lo, order_key(dv), on ? sm.id[tid] : 0);
+    const int rank = ratio_rank<false>(keys, sm.id, scratch, lo, on ? hi : lo, order_key(dv), on ? sm.id[tid] : 0);
     __syncthreads();
     if (on) { scratch[rank] = tid; sm.key[rank] = dv; }
     __syncthreads();
