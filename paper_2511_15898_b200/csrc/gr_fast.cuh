@@ -1494,7 +1494,7 @@ __device__ __noinline__ void start_point(int m, int slack, int n, double Tm, int
     const double rhs_i = on ? sm.rhs[pos] : 0.0, d_i = on ? sm.d[pos] : 0.0;
     // masses relative to the system's total: token avoided / a pair avoided, (1 - d_i / T)^n and (1 - (d_i + d_j) / T)^n
     const double iT = m_div(1.0, Tm);
-    const float fn = (float)n, rel = (float)(d_i * iT);
+    const float rel = (float)(d_i * iT);
     const double col_d = on ? ipow(fmax(1.0 - d_i * iT, 0.0), n) : 0.0;
     const float col = (float)col_d, ci = on ? (float)(1.0 - col_d) : 1.f, ic = __fdividef(1.f, ci);   // ci: Pr[token i drafted]
     const float rho = on ? fminf((float)(rhs_i * ipow(iT, n)) * ic, 0.999f) : 0.5f;
@@ -1503,42 +1503,61 @@ __device__ __noinline__ void start_point(int m, int slack, int n, double Tm, int
     // a rarely drafted token: Pr[j drafted | i drafted] tends to 1 - (1 - d_j / T)^(n - 1)
     const bool rare = ci < 0.02f;
     const float pres = 1.f - (rel < 1.f ? __fdividef(col, 1.f - rel) : 0.f);
-    // (the table behind the vectors)
-    GR_PTR(float) tab = GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oPP), 4 * C::MP, sm.flag);
-    static_assert(4 * C::MP * 4 <= C::kPPBytes + C::T * 16, "start table");
-    if (lead) { st_f4(tab + 4 * i, make_float4(rel, col, pres, 0.f)); vec_buffer(sm, 0)[vec_pos<C>(i)] = __fdividef(1.f, wi); }
+    // (the table behind the vectors: masses, probabilities of being avoided, presences of a rare token's competitors.  Behind the last token:
+    // avoided for certain, and an inverse weight that leaves nothing)
+    GR_PTR(float) tab = GR_MKPTR(float, reinterpret_cast<float*>(sm.base + C::oPP), 3 * C::MP, sm.flag);
+    static_assert(3 * C::MP * 4 <= C::kPPBytes + C::T * 16, "start table");
+    // (bounds within which the product of two denominators below neither overflows nor vanishes)
+    auto inverse = [&](float w) { return on ? fminf(fmaxf(__fdividef(1.f, w), 1e-18f), 1e15f) : 1e15f; };
+    if (lead) { tab[i] = rel; tab[C::MP + i] = on ? col : 1.f; tab[2 * C::MP + i] = on ? pres : 0.f; vec_buffer(sm, 0)[vec_pos<C>(i)] = inverse(wi); }
     __syncthreads();
-    // (eight columns at a time: their chains overlap; columns beyond m hold 0.  A share of up to 32 columns stays in registers)
+    // (eight columns at a time: their chains overlap, pairs of them in packed arithmetic.  A share of up to 32 columns stays in registers)
     constexpr bool kRegs = kCol <= 32;
+    const int nc = (min(kCol, max(0, m - share * kCol)) + 7) >> 3;
     GR_PTR(__half) prow = sm.pi + i * C::kNS + share * kCol;
-    const int nc = min(kCol, (max(0, m - share * kCol) + 7) & ~7) >> 3;
-    float preg[kRegs ? kCol : 1];
-    auto presence = [&](int j) {
-        const float4 tj = ld_f4(tab + 4 * j);
-        const float both = ex2_approx(fn * __log2f(fmaxf(1.f - rel - tj.x, 0.f)));
-        const float pij = rare ? tj.z : (1.f - col - tj.y + both) * ic;
-        return (j == i || j >= m) ? 0.f : fminf(fmaxf(pij, 0.f), 1.f);
+    F2 preg[kRegs ? kCol / 2 : 1];
+    const F2 avoid(1.f - rel), nrel(-1.f);
+    const float own = (1.f - col) * ic;
+    auto presence = [&](int c, F2* o) {
+        GR_PTR(const float) tp = tab + share * kCol + 8 * c;
+        F2 x[4], b[4];
+#pragma unroll
+        for (int z = 0; z < 8; z += 4) {
+            const float4 v = ld_f4(tp + z);
+            x[z / 2] = fma(F2(v.x, v.y), nrel, avoid); x[z / 2 + 1] = fma(F2(v.z, v.w), nrel, avoid);
+        }
+        // both avoided: x^n
+#pragma unroll
+        for (int z = 0; z < 4; z++) b[z] = F2(1.f);
+#pragma unroll 1
+        for (int e = n; e > 0; e >>= 1) {
+#pragma unroll
+            for (int z = 0; z < 4; z++) { if (e & 1) b[z] = b[z] * x[z]; x[z] = x[z] * x[z]; }
+        }
+#pragma unroll
+        for (int z = 0; z < 8; z += 4) {
+            const float4 v = ld_f4(tp + C::MP + z), r = ld_f4(tp + 2 * C::MP + z);
+            const F2 d0 = b[z / 2] - F2(v.x, v.y), d1 = b[z / 2 + 1] - F2(v.z, v.w);
+            const float p[4] = {__saturatef(fmaf(d0.lo(), ic, own)), __saturatef(fmaf(d0.hi(), ic, own)),
+                                __saturatef(fmaf(d1.lo(), ic, own)), __saturatef(fmaf(d1.hi(), ic, own))};
+            const float q[4] = {r.x, r.y, r.z, r.w};
+            float u[4];
+#pragma unroll
+            for (int y = 0; y < 4; y++) u[y] = share * kCol + 8 * c + z + y == i ? 0.f : rare ? q[y] : p[y];
+            o[z / 2] = F2(u[0], u[1]); o[z / 2 + 1] = F2(u[2], u[3]);
+        }
     };
     if constexpr (kRegs) {
 #pragma unroll
-        for (int c = 0; c < kCol; c++) preg[c] = 0.f;
+        for (int c = 0; c < kCol / 2; c++) preg[c] = F2(0.f);
 #pragma unroll
-        for (int c = 0; c < kCol; c += 8) {
-            if (c < 8 * nc) {
-#pragma unroll
-                for (int z = 0; z < 8; z++) preg[c + z] = presence(share * kCol + c + z);
-            }
-        }
+        for (int c = 0; c < kCol / 8; c++) if (c < nc) presence(c, preg + 4 * c);
     } else if (on) {
 #pragma unroll 1
         for (int c = 0; c < nc; c++) {
-            uint32_t pk[4];
-#pragma unroll
-            for (int z = 0; z < 4; z++) {
-                const __half2 h = __floats2half2_rn(presence(share * kCol + 8 * c + 2 * z), presence(share * kCol + 8 * c + 2 * z + 1));
-                pk[z] = *reinterpret_cast<const uint32_t*>(&h);
-            }
-            st_h8(prow + 8 * c, make_uint4(pk[0], pk[1], pk[2], pk[3]));
+            F2 o[4];
+            presence(c, o);
+            st_h8(prow + 8 * c, make_uint4(pack_half(o[0].lo(), o[0].hi()), pack_half(o[1].lo(), o[1].hi()), pack_half(o[2].lo(), o[2].hi()), pack_half(o[3].lo(), o[3].hi())));
         }
     }
     // (a thread reads back what it wrote)
@@ -1546,38 +1565,43 @@ __device__ __noinline__ void start_point(int m, int slack, int n, double Tm, int
     constexpr int sweeps = C::kSweeps;
 #pragma unroll 1
     for (int sweep = 0; sweep < sweeps; sweep++) {
+        // e_j / A = p / (1 / w_j + (1 - p) / A), two competitors to a reciprocal
         GR_PTR(const float) inv = vec_buffer(sm, sweep & 1) + share * (kCol + 4);
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        auto group = [&](int c, const float* pv) {
+        const F2 invA(fminf(__fdividef(1.f, A), 1e15f));
+        float acc[2] = {0.f, 0.f};
+        auto group = [&](int c, const F2* pv) {
             const float4 w0 = ld_f4(inv + 8 * c), w1 = ld_f4(inv + 8 * c + 4);
-            const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+            const F2 wv[4] = {F2(w0.x, w0.y), F2(w0.z, w0.w), F2(w1.x, w1.y), F2(w1.z, w1.w)};
 #pragma unroll
-            for (int z = 0; z < 8; z++) acc[z >> 1] += __fdividef(pv[z], fmaf(A, wv[z], 1.f - pv[z]));
+            for (int z = 0; z < 4; z++) {
+                const F2 b = fma(F2(1.f) - pv[z], invA, wv[z]);
+                acc[z & 1] = fmaf(fmaf(pv[z].lo(), b.hi(), pv[z].hi() * b.lo()), __fdividef(1.f, b.lo() * b.hi()), acc[z & 1]);
+            }
         };
         if constexpr (kRegs) {
 #pragma unroll
-            for (int c = 0; c < kCol / 8; c++) if (c < nc) group(c, preg + 8 * c);
+            for (int c = 0; c < kCol / 8; c++) if (c < nc) group(c, preg + 4 * c);
         } else if (on) {
 #pragma unroll 2
             for (int c = 0; c < nc; c++) {
                 const uint4 pk = ld_h8(prow + 8 * c);
                 const uint32_t u[4] = {pk.x, pk.y, pk.z, pk.w};
-                float pv[8];
+                F2 pv[4];
 #pragma unroll
                 for (int z = 0; z < 4; z++) {
                     const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&u[z]));
-                    pv[2 * z] = f.x; pv[2 * z + 1] = f.y;
+                    pv[z] = F2(f.x, f.y);
                 }
                 group(c, pv);
             }
         }
-        const float Si = share_sum<C::kNG>((acc[0] + acc[1]) + (acc[2] + acc[3])) * A;
+        const float Si = share_sum<C::kNG>(acc[0] + acc[1]);
         if (on) {
             wi = odds * (slack ? 1.f + Si : fmaxf(Si, 1e-30f));
             A = (slack ? 1.f : 0.f) + wi + Si;
         }
         if (sweep + 1 < sweeps) {
-            if (lead) vec_buffer(sm, (sweep + 1) & 1)[vec_pos<C>(i)] = __fdividef(1.f, wi);
+            if (lead) vec_buffer(sm, (sweep + 1) & 1)[vec_pos<C>(i)] = inverse(wi);
             __syncthreads();
         }
     }
