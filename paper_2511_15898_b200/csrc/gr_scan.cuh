@@ -359,11 +359,14 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
                 const bool sample = use_tau && r == 0 && nb == 0;
                 const float tau = sample ? INFINITY : (use_tau ? *((volatile float*)&sh.tau) : -INFINITY);
                 ulonglong2 qv[U], pv[U];
-                if (cvalid) {
+                // One batch; `all`: every vector of it lies within the row, as in all chunks but the last (the tests of each vector, at its load and at
+                // each use, were a third of the instructions).
+                auto batch = [&](auto all) {
+                    auto in = [&](int i0) { return decltype(all)::value || i0 + N <= vec_end; };
 #pragma unroll
                     for (int u = 0; u < U; u++) {
                         const int i0 = base + u * 32 * N;
-                        bool ok = whole || i0 + N <= vec_end;
+                        bool ok = in(i0);
 #ifdef GR_CHECK
                         if (ok && (i0 < 0 || i0 + N > V || ((size_t)(qrow + i0) & 15) || ((size_t)(prow + i0) & 15))) { if (check) *check = 1; ok = false; }
 #endif
@@ -385,14 +388,14 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
                     }
 #pragma unroll
                     for (int u = 0; u < U; u++) {
-                        if (whole || base + u * 32 * N + N <= vec_end) {
+                        if (in(base + u * 32 * N)) {
                             unsigned long long x[VT::kPairs];
 #pragma unroll
                             for (int i = 0; i < VT::kPairs; i++) x[i] = VT::pair(qv[u], i);
                             VT::check(chk, qv[u]);
                             const float mn = fmaxf(cm, VT::largest(qv[u]));
-                            // (a factor of exactly one where the maximum stands)
-                            const float keep = cm == mn ? 1.f : ex2((cm - mn) * sc_t);
+                            // (exactly one where the maximum stands)
+                            const float keep = ex2((cm - mn) * sc_t);
                             const unsigned long long nm = f_pack(-mn, -mn);
 #pragma unroll
                             for (int i = 0; i < VT::kPairs; i++) {
@@ -407,7 +410,7 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
                     // draft
 #pragma unroll
                     for (int u = 0; u < U; u++) {
-                        if (whole || base + u * 32 * N + N <= vec_end) {
+                        if (in(base + u * 32 * N)) {
                             const float vm = VT::largest(pv[u]);
                             VT::check(chk, pv[u]);
                             g0 = fmaxf(g0, vm);
@@ -418,7 +421,9 @@ __device__ __forceinline__ void scan_row(const ScanArgs& A, SS& sh, long long b,
                             if (!kFull && vm >= tau) push_vector(sh, pv[u], base + u * 32 * N);
                         }
                     }
-                }
+                };
+                if (whole) batch(std::true_type());
+                else if (cvalid) batch(std::false_type());
                 if (sample) {
                     // the first batch had no threshold: it gives one, and its draft logits, still in registers, are tested now
                     refine_tau(sh, g0, ksel);
