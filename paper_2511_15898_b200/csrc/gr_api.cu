@@ -95,16 +95,21 @@ static int solve_impl(const void* q_logits, const void* p_logits, int dtype, int
     if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return GR_E_LAUNCH; }
     if (scan_done && cudaEventRecord(scan_done, st) != cudaSuccess) { cudaGetLastError(); return GR_E_LAUNCH; }
     gr::NvtxRange r(fa.draft ? "gr:solve+draw" : "gr:solve");
-    int rc = gr::launch_solve_any((char*)workspace, (char*)params, pstride, kcap, V, n, topk,
-                                  (double)temp_target, (double)temp_draft, tol, max_iters, qstep, tau, batch,
-                                  force_robust, alpha_star, status, fa, st);
-    if (rc != GR_OK) return rc;
+    // (a whole row's header without a rule is written on the way to its optimal acceptance, unless it is to be drawn from here)
+    const bool header_later = full_large && !fa.draft;
+    if (!header_later) {
+        const int rc = gr::launch_solve_any((char*)workspace, (char*)params, pstride, kcap, V, n, topk,
+                                            (double)temp_target, (double)temp_draft, tol, max_iters, qstep, tau, batch,
+                                            force_robust, alpha_star, status, fa, st);
+        if (rc != GR_OK) return rc;
+    }
     if (full_large) {
         // no rule is solved for this shape, but the optimal acceptance still is (bucketed search for the minimum of
         // psi, or with force_robust a sort of the whole row and a prefix scan)
         char* scratch = (char*)workspace + (size_t)gr::ws_stride() * (size_t)batch;
         gr::launch_fullsort(q_logits, p_logits, dtype, V, &n, 1, (double)temp_target, (double)temp_draft, batch,
-                            (const char*)workspace, scratch, (char*)params, pstride, force_robust, alpha_star, nullptr, st);
+                            (const char*)workspace, scratch, (char*)params, pstride, force_robust, alpha_star, nullptr,
+                            header_later ? status : nullptr, st);
     }
     if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return GR_E_LAUNCH; }
     return GR_OK;
@@ -157,7 +162,7 @@ int gr_alpha_star(const void* q_logits, const void* p_logits, int dtype, int V, 
                         (char*)workspace, nullptr, 0, kcap, st);
         char* scratch = (char*)workspace + (size_t)gr::ws_stride() * (size_t)batch;
         gr::launch_fullsort(q_logits, p_logits, dtype, V, n_list, n_count, (double)temp_target, (double)temp_draft, batch,
-                            (const char*)workspace, scratch, nullptr, 0, 0, alpha_star, status, st);
+                            (const char*)workspace, scratch, nullptr, 0, 0, alpha_star, status, nullptr, st);
         if (cudaPeekAtLastError() != cudaSuccess) { cudaGetLastError(); return GR_E_LAUNCH; }
         return GR_OK;
     }

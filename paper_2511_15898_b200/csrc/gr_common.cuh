@@ -88,6 +88,7 @@ template <class P> __device__ inline uint2 ld_u2(const P& p) { return make_uint2
 template <class P> __device__ inline uint4 ld_u4(const P& p) { return make_uint4(p[0], p[1], p[2], p[3]); }
 template <class P> __device__ inline ulonglong2 ld_ull2(const P& p) { return make_ulonglong2(p[0], p[1]); }
 template <class P> __device__ inline void st_f4(const P& p, float4 v) { p[0] = v.x; p[1] = v.y; p[2] = v.z; p[3] = v.w; }
+template <class P> __device__ inline void st_u4(const P& p, uint4 v) { p[0] = v.x; p[1] = v.y; p[2] = v.z; p[3] = v.w; }
 template <class P> __device__ inline void st_f2(const P& p, float2 v) { p[0] = v.x; p[1] = v.y; }
 template <class P> __device__ inline void st_d2(const P& p, double2 v) { p[0] = v.x; p[1] = v.y; }
 template <class P> __device__ inline uint4 ld_h8(const P& p) {
@@ -107,6 +108,7 @@ __device__ __forceinline__ uint2 ld_u2(const uint32_t* p) { return *reinterpret_
 __device__ __forceinline__ uint4 ld_u4(const uint32_t* p) { return *reinterpret_cast<const uint4*>(p); }
 __device__ __forceinline__ ulonglong2 ld_ull2(const unsigned long long* p) { return *reinterpret_cast<const ulonglong2*>(p); }
 __device__ __forceinline__ void st_f4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ void st_u4(uint32_t* p, uint4 v) { *reinterpret_cast<uint4*>(p) = v; }
 __device__ __forceinline__ void st_f2(float* p, float2 v) { *reinterpret_cast<float2*>(p) = v; }
 __device__ __forceinline__ void st_d2(double* p, double2 v) { *reinterpret_cast<double2*>(p) = v; }
 __device__ __forceinline__ uint4 ld_h8(const __half* p) { return *reinterpret_cast<const uint4*>(p); }

@@ -13,7 +13,7 @@
 // pairs of the row in global scratch with a bitonic network, then scans tgt and drf along the order.
 // The network's passes with a compare distance below the tile size (4096 pairs, 48 KB) run on tiles staged in
 // shared memory: 15 trips through global memory for a 65536-entry row instead of 136.
-#include "gr_common.cuh"
+#include "gr_prep.cuh"
 
 namespace gr {
 
@@ -38,26 +38,26 @@ constexpr int kBkThreads = 1024;
 constexpr int kBkBuckets = 4096;
 constexpr int kBkPer = kBkBuckets / kBkThreads;   // buckets per thread in the scan over buckets
 constexpr int kBkMaxCand = 4096;                  // elements of candidate buckets held in shared memory
-constexpr int kBkTab = 32, kBkCopies = 16;        // 2^(42 + j / 32), a copy for every lane of a half-warp
+constexpr int kBkFew = 128;                       // up to so many are taken without ordering them
+constexpr int kBkTab = 128, kBkCopies = 16;       // 2^(42 + j / 128), a copy for every lane of a half-warp
 constexpr int kBkSmemBytes = kBkBuckets * (4 * 4 + 4 + 4) + kBkMaxCand * (8 + 4 + 4 + 4 + 4) + kBkTab * kBkCopies * 8;
 
-// exp(-y) in units of 2^-42, rounded to an integer (masses are summed as integers: exact, order-free).  y >= 0.
-// 2^(k/32) from a table times a degree-5 Taylor polynomial on |r| <= ln2/64 (2e-15 relative, a hundredth of the unit):
-// ten fp64 operations, where exp and llrint took about forty.
+// exp(-y) in units of 2^-42, rounded to an integer (masses are summed as integers: exact, order-free).  y >= 0 (but for its last bit).
+// 2^(k/128) from a table times a degree-4 Taylor polynomial on |r| <= ln2/256 (1.2e-15 relative, a hundredth of the unit; degree 5 and 32
+// entries took two operations more), scaled and rounded by one multiplication and addition: nine fp64 operations.
 __device__ __forceinline__ unsigned long long mass_fixed(double y, GR_PTR(const double) tab)
 {
-    const double magic = 6755399441055744.0;                                   // 1.5 * 2^52
+    constexpr double ln2 = 0.6931471805599453, magic = 6755399441055744.0;         // 1.5 * 2^52
     y = __hiloint2double(min(__double2hiint(y), 0x40468000), __double2loint(y));   // (at 45 and beyond it rounds to nothing)
-    const double m = fma(y, -46.16624130844682, magic);                        // 32 / ln 2
+    const double m = fma(y, -kBkTab / ln2, magic);
     const int k = __double2loint(m);
-    const double r = fma(magic - m, 0.021660849392498290, -y);                 // ln 2 / 32
-    double p = fma(r, 8.333333333333333e-03, 4.1666666666666664e-02);
-    p = fma(r, p, 1.6666666666666666e-01);
+    const double r = fma(magic - m, ln2 / kBkTab, -y);
+    double p = fma(r, 4.1666666666666664e-02, 1.6666666666666666e-01);
     p = fma(r, p, 0.5);
     p = fma(r, p, 1.0);
     p = fma(r, p, 1.0);
-    const double v = p * tab[(k & (kBkTab - 1)) * kBkCopies];                  // (tab: this lane's copy)
-    const double u = __hiloint2double(__double2hiint(v) + (k & ~(kBkTab - 1)) * 32768, __double2loint(v)) + 4503599627370496.0;   // 2^52
+    const double s = tab[(k & (kBkTab - 1)) * kBkCopies];                      // (tab: this lane's copy)
+    const double u = fma(p, __hiloint2double(__double2hiint(s) + (k & ~(kBkTab - 1)) * ((1 << 20) / kBkTab), __double2loint(s)), 4503599627370496.0);   // 2^52
     return (unsigned long long)__double_as_longlong(u) - 0x4330000000000000ull;
 }
 
@@ -80,28 +80,30 @@ __device__ __forceinline__ double power(double x, int n)
     return r;
 }
 
-// Exclusive prefix over the CTA of one 64-bit integer per thread; *total gets the sum.  s_w: a slot per warp (32 of them).
-__device__ inline unsigned long long block_exscan_u64(unsigned long long v, unsigned long long* s_w,
-                                                      unsigned long long* total)
+// Exclusive prefixes over the CTA of two 64-bit integers per thread, in place; total gets the sums.  s_w: two slots per warp (32 of them).
+__device__ inline void block_exscan_u64(unsigned long long* v, unsigned long long* s_w, unsigned long long* total)
 {
     static_assert(kBkThreads == 1024, "one slot per lane");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    auto warp_scan = [&](unsigned long long x) {
+    auto warp_scan = [&](unsigned long long* x) {
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long t = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += t;
+            const unsigned long long t0 = __shfl_up_sync(0xffffffffu, x[0], o), t1 = __shfl_up_sync(0xffffffffu, x[1], o);
+            if (lane >= o) { x[0] += t0; x[1] += t1; }
         }
-        return x;
     };
-    const unsigned long long inc = warp_scan(v);
+    unsigned long long inc[2] = {v[0], v[1]};
+    warp_scan(inc);
+    if (lane == 31) { s_w[2 * warp] = inc[0]; s_w[2 * warp + 1] = inc[1]; }
     __syncthreads();
-    if (lane == 31) s_w[warp] = inc;
-    __syncthreads();
-    const unsigned long long all = warp_scan(s_w[lane]);
-    const unsigned long long off = __shfl_sync(0xffffffffu, all, (warp + 31) & 31);
-    *total = __shfl_sync(0xffffffffu, all, 31);
-    return (warp > 0 ? off : 0ull) + inc - v;
+    unsigned long long all[2] = {s_w[2 * lane], s_w[2 * lane + 1]};
+    warp_scan(all);
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+        const unsigned long long off = __shfl_sync(0xffffffffu, all[k], (warp + 31) & 31);
+        total[k] = __shfl_sync(0xffffffffu, all[k], 31);
+        v[k] = (warp > 0 ? off : 0ull) + inc[k] - v[k];
+    }
 }
 // Minimum over the CTA, for every thread (s_r: a slot per warp; a barrier before its next use is the caller's).
 __device__ inline double block_min(double v, double* s_r)
@@ -117,14 +119,16 @@ __device__ inline double block_min(double v, double* s_r)
 }
 
 // flag[0] of the instance's scratch region: bit j set when fullsort_alpha_kernel has to do the row for the j-th draft count.
-// 512 rows of 50257 in fp32: 168 us (three passes with exp, 64-bit shared atomics and counts: 408).  Bound by
-// instruction issue (130 instructions per 32 ids; fp64 pipe 28 % busy, shared atomics hidden), not by the 206 MB it reads.
+// With a params block and `rule_status` it also writes the header of a row without a rule (nl.n[0] drafts).
+// 512 rows of 50257 in fp32: the call 195 us, 220 before (bucket numbers and masses out of scaled logits formed first, a polynomial of degree 5, every thread
+// its own quotients and exponentials, candidates ordered in three rounds).  A row takes 71 k cycles, one to an SM: 46 k its masses (instruction
+// issue: 113 instructions per 32 ids in all, fp64 25 of them), 4 k sums, 5 k bounds, 6 k numbers read back, 6 k candidates; the 206 MB it reads are a fifth of the time.
 template <typename T>
 __global__ void __launch_bounds__(kBkThreads)
-bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, const __grid_constant__ NList nl, double temp_t, double temp_d,
+bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, const __grid_constant__ NList nl, double rt, double rd,
                     const char* __restrict__ ws, char* __restrict__ scratch, size_t scratch_stride,
                     char* __restrict__ params, int pstride, int force_sort, float* __restrict__ alpha_out,
-                    int* __restrict__ status_out)
+                    int* __restrict__ status_out, int* __restrict__ rule_status)
 {
     extern __shared__ __align__(16) unsigned char bk_smem[];
     pdl_wait();
@@ -146,8 +150,8 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
     GR_PTR(int) sid = GR_MKPTR(int, i_raw + 2 * kBkBuckets + kBkMaxCand, kBkMaxCand, GR_CHECK_FLAG);         // ids in order,
     GR_PTR(int) lid = GR_MKPTR(int, i_raw + 2 * kBkBuckets + 2 * kBkMaxCand, kBkMaxCand, GR_CHECK_FLAG);     // ids and
     GR_PTR(int) lbk = GR_MKPTR(int, i_raw + 2 * kBkBuckets + 3 * kBkMaxCand, kBkMaxCand, GR_CHECK_FLAG);     // buckets as found
-    __shared__ double s_r[kBkThreads / 32];
-    __shared__ unsigned long long s_w[kBkThreads / 32];
+    __shared__ double s_r[kBkThreads / 32], s_c[6], s_up[32], s_at[32];      // s_c: bucket width, scales; s_at[warp] s_up[lane]: bounds on the ratios
+    __shared__ unsigned long long s_w[2 * kBkThreads / 32];
     __shared__ int s_nelem, s_found, s_fallback, s_lo, s_hi;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long b = blockIdx.x;
@@ -158,6 +162,7 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
     char* const scr = scratch + (size_t)b * scratch_stride;
     int* flag = reinterpret_cast<int*>(scr);
     if (tid == 0 && status_out) status_out[b] = wh->bad != 0 ? GR_BAD_LOGITS : GR_OK;
+    if (tid == 0 && rule_status) write_no_rule(hdr, nl.n[0], wh->bad != 0, alpha_out, rule_status, b);
     if (wh->bad != 0 || force_sort) {
         if (tid == 0) {
             flag[0] = (1 << nl.count) - 1;          // (a bad row returns at once there too)
@@ -169,20 +174,29 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
     const T* qrow = q + (size_t)b * V;
     const T* prow = p + (size_t)b * V;
     const FullRow fr = *reinterpret_cast<const FullRow*>(rec + sizeof(WsHeader));
-    // (scaled logits as products with the reciprocal temperatures: one rounding away from the quotients the sort
+    // (scaled logits as products with the reciprocal temperatures rt and rd: one rounding away from the quotients the sort
     // uses, which moves alpha* by ~1e-16; every pass here forms them the same way)
-    const double rt = 1.0 / temp_t, rd = 1.0 / temp_d;
     const double mt = (double)fr.qmax * rt, md = (double)fr.pmax * rd;
-    // bucket of a key d - a: floor((kmax - key) * invw), clamped: a non-decreasing function of kmax - key in floating
-    // point, so every element of a lower bucket comes before every element of a higher one in the ratio order.  (kmax
+    // bucket of a key d - a: floor((kmax - key) * invw), clamped, formed from the logits at once (two operations; rounding moves an id whose
+    // key is 1e-13 of a bucket's width from its border, which changes no mass by more, and the bound below allows for it).  (kmax
     // and kmin are fp32 values: a key may lie outside.)
     const double ln2 = 0.6931471805599453;
     const double kmax = (double)fr.kmax * ln2, span = kmax - (double)fr.kmin * ln2;
-    const double invw = span > 0.0 ? (double)kBkBuckets / (span * (1.0 + 1e-9)) : 0.0;
-    for (int c = tid; c < kBkBuckets; c += kBkThreads) { tl[c] = 0u; th[c] = 0u; dl[c] = 0u; dh[c] = 0u; cnt[c] = 0; seg[c] = -1; }
-    for (int e = tid; e < kBkTab * kBkCopies; e += kBkThreads) tab_all[e] = exp2(42.0 + (double)(e / kBkCopies) / kBkTab);
+    // (what every thread needs the same is formed by one: a quotient by 1024 threads keeps the fp64 units busy for 700 cycles)
+    if (tid == 0) s_c[0] = span > 0.0 ? (double)kBkBuckets / (span * (1.0 + 1e-9)) : 0.0;
+    // (masses and counts lie behind one another)
+    static_assert(5 * kBkBuckets % (4 * kBkThreads) == 0 && kBkBuckets == 4 * kBkThreads && kBkTab <= kBkThreads, "a vector per thread");
+#pragma unroll
+    for (int u = 0; u < 5 * kBkBuckets / (4 * kBkThreads); u++) reinterpret_cast<uint4*>(w_raw)[tid + u * kBkThreads] = make_uint4(0u, 0u, 0u, 0u);
+    reinterpret_cast<int4*>(i_raw + kBkBuckets)[tid] = make_int4(-1, -1, -1, -1);
+    if (tid < kBkTab) {
+        const double v = exp2(42.0 + (double)tid / kBkTab);
+#pragma unroll
+        for (int c = 0; c < kBkCopies; c++) tab_all[tid * kBkCopies + ((c + tid) & (kBkCopies - 1))] = v;
+    }
     if (tid == 0) { s_nelem = 0; s_found = 0; s_fallback = 0; s_lo = kBkBuckets; s_hi = -1; }
     __syncthreads();
+    const double invw = s_c[0];
     // ---- the row: bucket masses (integers: the sums do not depend on the order of the atomics), bucket numbers to scratch
     // (number of id i at code[i + shift], so that a vector of logits has its numbers in one aligned store)
     constexpr int N = 16 / (int)sizeof(T);
@@ -190,12 +204,13 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
     unsigned short* const code_raw = reinterpret_cast<unsigned short*>(scr + 16);
     GR_PTR(unsigned short) code = GR_MKPTR(unsigned short, code_raw, V + 16, GR_CHECK_FLAG);
     auto key_of = [&](float x, float v) { return (double)v * rd - (double)x * rt; };
+    const double ca = rt * invw, cd = -rd * invw, c0 = kmax * invw;
     auto element = [&](float x, float v) {
-        const double a = (double)x * rt, d = (double)v * rd;
-        const double t = __dadd_rd((kmax - (d - a)) * invw, 6755399441055744.0);
+        const double a = (double)x, d = (double)v;
+        const double t = __dadd_rd(fma(a, ca, fma(d, cd, c0)), 6755399441055744.0);
         const int c = min(max(__double2loint(t), 0), kBkBuckets - 1);
-        add_mass(tl, th, c, mass_fixed(mt - a, tab));
-        add_mass(dl, dh, c, mass_fixed(md - d, tab));
+        add_mass(tl, th, c, mass_fixed(fma(-a, rt, mt), tab));
+        add_mass(dl, dh, c, mass_fixed(fma(-d, rd, md), tab));
         return c;
     };
     const int nvec = (V - head) / N, tail0 = head + nvec * N;
@@ -204,11 +219,11 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
     const uint4* const qv = reinterpret_cast<const uint4*>(qrow + head);
     const uint4* const pv = reinterpret_cast<const uint4*>(prow + head);
     uint4 xq = make_uint4(0u, 0u, 0u, 0u), xp = xq;
-    if (tid < nvec) { xq = __ldcs(qv + tid); xp = __ldcs(pv + tid); }
+    if (tid < nvec) { xq = __ldg(qv + tid); xp = __ldg(pv + tid); }
 #pragma unroll 1
     for (int e = tid; e < nvec; e += kBkThreads) {
         const uint4 cq = xq, cp = xp;
-        if (e + kBkThreads < nvec) { xq = __ldcs(qv + e + kBkThreads); xp = __ldcs(pv + e + kBkThreads); }
+        if (e + kBkThreads < nvec) { xq = __ldg(qv + e + kBkThreads); xp = __ldg(pv + e + kBkThreads); }
         const unsigned wq[4] = {cq.x, cq.y, cq.z, cq.w}, wp[4] = {cp.x, cp.y, cp.z, cp.w};
         unsigned out[N / 2];
 #pragma unroll
@@ -233,56 +248,80 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
     }
     __syncthreads();
     // ---- prefixes over the buckets, psi at every boundary, lower bound inside every bucket
-    unsigned long long mT[kBkPer], mD[kBkPer], sT = 0, sD = 0;
-#pragma unroll
-    for (int u = 0; u < kBkPer; u++) {
-        const int c = tid * kBkPer + u;
-        mT[u] = ((unsigned long long)th[c] << 32) | tl[c]; mD[u] = ((unsigned long long)dh[c] << 32) | dl[c];
-        sT += mT[u]; sD += mD[u];
-    }
+    // (a thread's four buckets lie in one vector of each table)
+    static_assert(kBkPer == 4, "a vector per thread");
+    auto join = [](unsigned l, unsigned h) { return ((unsigned long long)h << 32) | l; };
     unsigned long long totT, totD;
     {
-        unsigned long long t = block_exscan_u64(sT, s_w, &totT), d = block_exscan_u64(sD, s_w, &totD);
-#pragma unroll
-        for (int u = 0; u < kBkPer; u++) {
-            const int c = tid * kBkPer + u;
-            tl[c] = (unsigned)t; th[c] = (unsigned)(t >> 32); dl[c] = (unsigned)d; dh[c] = (unsigned)(d >> 32);
-            t += mT[u]; d += mD[u];
-        }
+        const uint4 tv = ld_u4(tl + 4 * tid), tw = ld_u4(th + 4 * tid), dv = ld_u4(dl + 4 * tid), dw = ld_u4(dh + 4 * tid);
+        const unsigned long long mT[4] = {join(tv.x, tw.x), join(tv.y, tw.y), join(tv.z, tw.z), join(tv.w, tw.w)};
+        const unsigned long long mD[4] = {join(dv.x, dw.x), join(dv.y, dw.y), join(dv.z, dw.z), join(dv.w, dw.w)};
+        unsigned long long s[2] = {(mT[0] + mT[1]) + (mT[2] + mT[3]), (mD[0] + mD[1]) + (mD[2] + mD[3])}, tot[2];
+        block_exscan_u64(s, s_w, tot);
+        totT = tot[0]; totD = tot[1];
+        auto put = [&](GR_PTR(unsigned) l, GR_PTR(unsigned) h, unsigned long long x, const unsigned long long* m) {
+            const unsigned long long y = x + m[0], z = y + m[1], w = z + m[2];
+            st_u4(l + 4 * tid, make_uint4((unsigned)x, (unsigned)y, (unsigned)z, (unsigned)w));
+            st_u4(h + 4 * tid, make_uint4((unsigned)(x >> 32), (unsigned)(y >> 32), (unsigned)(z >> 32), (unsigned)(w >> 32)));
+        };
+        put(tl, th, s[0], mT);
+        put(dl, dh, s[1], mD);
     }
-    const double iT = 1.0 / (double)totT, iD = 1.0 / (double)totD;
-    // tgt_i / drf_i = exp(-key_i) * rscale
-    const double rscale = exp(md - mt) * ((double)totD / (double)totT);
-    const double slack = (double)(V + 1) * iT + 1e-14;
+    // tgt_i / drf_i = exp(-key_i) * rscale.  Every ratio of bucket c is at least rho: its keys are at most kmax - c w (rho of a thread's first bucket
+    // as a product of two numbers, of the others one from the other; where the factors are far from overflowing).
+    const double wide = invw > 0.0 ? (1.0 - 1e-12) / invw : 0.0;
+    if (warp == 0) s_up[lane] = exp((double)(lane * kBkPer) * fmin(wide, 1.0));
+    else if (warp == 1) s_at[lane] = exp((double)(32 * lane * kBkPer) * wide - kmax);
+    else if (tid == 64) { s_c[1] = 1.0 / (double)totT; s_c[4] = (double)(V + 1) * s_c[1] + 1e-14; }
+    else if (tid == 96) s_c[2] = 1.0 / (double)totD;
+    else if (tid == 128) s_c[3] = exp(md - mt) * ((double)totD / (double)totT) * (1.0 - 1e-9);
+    else if (tid == 160) s_c[5] = exp(fmin(wide, 1.0));
     __syncthreads();
+    const double iT = s_c[1], iD = s_c[2], rscale = s_c[3], slack = s_c[4], grow = s_c[5];
+    const double rho_first = wide <= 1.0 ? s_at[warp] * s_up[lane] * rscale : exp((double)(tid * kBkPer) * wide - kmax) * rscale;
     int todo = 0;                                           // draft counts left to the sort
 #pragma unroll 1
     for (int ni = 0; ni < nl.count; ni++) {
     const int n = nl.n[ni];
     double lb[kBkPer], best = 0.0;                          // psi of the empty prefix
     // (the masses are read back as prefixes: holding them in registers across this loop spilled, 10 % of the kernel)
-    auto prefix = [&](GR_PTR(unsigned) l, GR_PTR(unsigned) h, int c, unsigned long long total) {
-        return c < kBkBuckets ? ((unsigned long long)h[c] << 32) | l[c] : total;
-    };
-    unsigned long long qT = prefix(tl, th, tid * kBkPer, totT), qD = prefix(dl, dh, tid * kBkPer, totD);
+    unsigned long long pT[kBkPer + 1], pD[kBkPer + 1];
+    {
+        const uint4 tv = ld_u4(tl + 4 * tid), tw = ld_u4(th + 4 * tid), dv = ld_u4(dl + 4 * tid), dw = ld_u4(dh + 4 * tid);
+        const bool last = tid == kBkThreads - 1;
+        pT[0] = join(tv.x, tw.x); pT[1] = join(tv.y, tw.y); pT[2] = join(tv.z, tw.z); pT[3] = join(tv.w, tw.w);
+        pD[0] = join(dv.x, dw.x); pD[1] = join(dv.y, dw.y); pD[2] = join(dv.z, dw.z); pD[3] = join(dv.w, dw.w);
+        pT[4] = last ? totT : join(tl[last ? 0 : 4 * tid + 4], th[last ? 0 : 4 * tid + 4]);
+        pD[4] = last ? totD : join(dl[last ? 0 : 4 * tid + 4], dh[last ? 0 : 4 * tid + 4]);
+    }
+    double rho_next = rho_first, T0 = (double)pT[0] * iT, D0 = (double)pD[0] * iD;
+    double D1[kBkPer], dn[kBkPer];
+    {
+        double x[kBkPer];
+#pragma unroll
+        for (int u = 0; u < kBkPer; u++) { x[u] = D1[u] = (double)pD[u + 1] * iD; dn[u] = 1.0; }
+#pragma unroll 1
+        for (int e = n; e > 0; e >>= 1) {
+#pragma unroll
+            for (int u = 0; u < kBkPer; u++) { if (e & 1) dn[u] *= x[u]; x[u] *= x[u]; }
+        }
+    }
 #pragma unroll
     for (int u = 0; u < kBkPer; u++) {
         const int c = tid * kBkPer + u;
-        const unsigned long long eT = prefix(tl, th, c + 1, totT), eD = prefix(dl, dh, c + 1, totD);
-        const double T0 = (double)qT * iT, D0 = (double)qD * iD, T1 = (double)eT * iT, D1 = (double)eD * iD;
-        const bool empty = eT == qT && eD == qD;
-        qT = eT; qD = eD;
-        const double dn = power(D1, n);
-        best = fmin(best, T1 - dn);
+        const double T1 = (double)pT[u + 1] * iT;
+        const bool empty = pT[u + 1] == pT[u] && pD[u + 1] == pD[u];
+        best = fmin(best, T1 - dn[u]);
         // Inside the bucket every ratio tgt / drf is at least rho (its keys are at most kmax - c w; the first bucket has no
         // such limit), so a prefix that ends inside it has  psi >= T0 + rho (D - D0) - D^n,  concave in D: its minimum
         // over [D0, D1] is at an end.  At D0 that is the previous boundary's psi; at D1 it is the bound below.  The slack
         // covers the rounding of the target's masses to integers (one unit per id).  That of the draft's is not in it: it is
         // of the size by which rounding moves psi itself, n half units per id (at most n V 2^-43, 1.8e-7 for 50257 ids and 32
         // drafts).
-        const double khi = kmax - (invw > 0.0 ? (double)c / invw * (1.0 - 1e-12) : 0.0);
-        const double rho = c == 0 ? 0.0 : exp(-khi) * rscale * (1.0 - 1e-9);
-        lb[u] = empty ? 1.0 : T0 + rho * (D1 - D0) - dn - slack;
+        const double rho = c == 0 ? 0.0 : rho_next;
+        rho_next = wide <= 1.0 ? rho_next * grow : exp((double)(c + 1) * wide - kmax) * rscale;
+        lb[u] = empty ? 1.0 : T0 + rho * (D1[u] - D0) - dn[u] - slack;
+        T0 = T1; D0 = D1[u];
     }
     best = block_min(best, s_r);
     // ---- candidate buckets: those whose interior could hold a smaller psi
@@ -296,10 +335,15 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
     // ---- their elements, found by the bucket numbers
     if (hi >= lo) {
         const int ncode = V + shift;
-#pragma unroll 2
+        // (numbers less the first candidate's, two at a time: below `cap` is a candidate's range)
+        const unsigned cap = (unsigned)(hi - lo + 1) * 0x10001u, down = ((unsigned)(-lo) & 0xffffu) * 0x10001u;
+#pragma unroll 4
         for (int e = tid; e < (ncode + 7) / 8; e += kBkThreads) {
             const uint4 w = *reinterpret_cast<const uint4*>(code_raw + 8 * e);     // (16-byte aligned; within the region)
             const unsigned ww[4] = {w.x, w.y, w.z, w.w};
+            const unsigned least = __vminu2(__vminu2(__viaddmin_u16x2(w.x, down, cap), __viaddmin_u16x2(w.y, down, cap)),
+                                                 __vminu2(__viaddmin_u16x2(w.z, down, cap), __viaddmin_u16x2(w.w, down, cap)));
+            if (least == cap) continue;
 #pragma unroll
             for (int z = 0; z < 8; z++) {
                 const int c = (int)((ww[z / 2] >> (16 * (z & 1))) & 0xffffu), i = 8 * e + z - shift;
@@ -313,75 +357,107 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
     }
     __syncthreads();
     const int found = s_found;
-#pragma unroll
-    for (int u = 0; u < kBkPer; u++) {
-        const int c = tid * kBkPer + u;
-        if (seg[c] >= 0) {
-            const int L = cnt[c];
-            if (found > kBkMaxCand) s_fallback = 1;
-            else if (L >= 2) { seg[c] = atomicAdd(&s_nelem, L); cnt[c] = 0; }
-            else seg[c] = -1;
-        }
-    }
-    __syncthreads();
-    const bool crowded = s_fallback != 0;
-    // ---- each bucket into its own segment, ordered by (key descending, id ascending) by counting
-    if (!crowded && s_nelem > 0) {
-        constexpr int kOwn = kBkMaxCand / kBkThreads;
-        int pos[kOwn];
-#pragma unroll
-        for (int u = 0; u < kOwn; u++) {
-            const int e = tid + u * kBkThreads;
-            pos[u] = -1;
-            if (e < found) {
+    // ---- A few elements (nearly every row: 32 on average of N(0, 3) logits): each one's prefix is summed by a warp, over the elements
+    // of its bucket that come before it.  (Segments, ranks and walk, below, are three more rounds to memory: 10 k cycles of 77 k.)
+    bool crowded = false;
+    if (found <= kBkFew) {
+        if (found > 0) {
+            GR_PTR(unsigned long long) mt_f = GR_PCAST(unsigned long long, cid), md_f = GR_PCAST(unsigned long long, sid);
+            if (tid < found) {
+                const int i = lid[tid];
+                const float x = load_logit<T>(qrow, i), v = load_logit<T>(prow, i);
+                ckey[tid] = key_of(x, v);
+                mt_f[tid] = mass_fixed(fma(-(double)x, rt, mt), tab); md_f[tid] = mass_fixed(fma(-(double)v, rd, md), tab);
+            }
+            __syncthreads();
+            for (int e = warp; e < found; e += kBkThreads / 32) {
                 const int c = lbk[e], i = lid[e];
-                if (seg[c] >= 0) {
-                    pos[u] = seg[c] + atomicAdd(&cnt[c], 1);
-                    ckey[pos[u]] = key_of(load_logit<T>(qrow, i), load_logit<T>(prow, i)); cid[pos[u]] = i;
-                }
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < kOwn; u++) {
-            if (pos[u] >= 0) {
-                const int c = lbk[tid + u * kBkThreads], off = seg[c], L = cnt[c];
-                const double ke = ckey[pos[u]];
-                const int ie = cid[pos[u]];
-                int rank = 0;
-                for (int j = off; j < off + L; j++) {
+                const double ke = ckey[e];
+                unsigned long long cT = 0, cD = 0;
+                for (int j = lane; j < found; j += 32) {
                     const double kj = ckey[j];
-                    rank += (kj > ke || (kj == ke && cid[j] < ie)) ? 1 : 0;
+                    if (lbk[j] == c && (kj > ke || (kj == ke && lid[j] <= i))) { cT += mt_f[j]; cD += md_f[j]; }
                 }
-                sid[off + rank] = ie;
+                __syncwarp();
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) { cT += __shfl_xor_sync(0xffffffffu, cT, o); cD += __shfl_xor_sync(0xffffffffu, cD, o); }
+                cT += join(tl[c], th[c]); cD += join(dl[c], dh[c]);
+                best = fmin(best, (double)cT * iT - power((double)cD * iD, n));
+            }
+            // (block_min's slots have been read by all)
+            best = block_min(best, s_r);
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < kBkPer; u++) {
+            const int c = tid * kBkPer + u;
+            if (seg[c] >= 0) {
+                const int L = cnt[c];
+                if (found > kBkMaxCand) s_fallback = 1;
+                else if (L >= 2) { seg[c] = atomicAdd(&s_nelem, L); cnt[c] = 0; }
+                else seg[c] = -1;
             }
         }
         __syncthreads();
-    }
-    // ---- one warp per candidate bucket walks the prefixes
-    if (!crowded && s_nelem > 0) {
-        for (int c = lo + warp; c <= hi; c += kBkThreads / 32) {
-            const int off = seg[c];
-            if (off < 0) continue;
-            const int L = cnt[c];
-            unsigned long long cT = ((unsigned long long)th[c] << 32) | tl[c], cD = ((unsigned long long)dh[c] << 32) | dl[c];
-            for (int base = 0; base < L; base += 32) {
-                unsigned long long tf = 0, df = 0;
-                if (base + lane < L) {
-                    const int id = sid[off + base + lane];
-                    tf = mass_fixed(mt - (double)load_logit<T>(qrow, id) * rt, tab);
-                    df = mass_fixed(md - (double)load_logit<T>(prow, id) * rd, tab);
+        crowded = s_fallback != 0;
+        // ---- each bucket into its own segment, ordered by (key descending, id ascending) by counting
+        if (!crowded && s_nelem > 0) {
+            constexpr int kOwn = kBkMaxCand / kBkThreads;
+            int pos[kOwn];
+#pragma unroll
+            for (int u = 0; u < kOwn; u++) {
+                const int e = tid + u * kBkThreads;
+                pos[u] = -1;
+                if (e < found) {
+                    const int c = lbk[e], i = lid[e];
+                    if (seg[c] >= 0) {
+                        pos[u] = seg[c] + atomicAdd(&cnt[c], 1);
+                        ckey[pos[u]] = key_of(load_logit<T>(qrow, i), load_logit<T>(prow, i)); cid[pos[u]] = i;
+                    }
                 }
-                for (int o = 1; o < 32; o <<= 1) {
-                    const unsigned long long t2 = __shfl_up_sync(0xffffffffu, tf, o), d2 = __shfl_up_sync(0xffffffffu, df, o);
-                    if (lane >= o) { tf += t2; df += d2; }
-                }
-                if (base + lane < L)
-                    best = fmin(best, (double)(cT + tf) * iT - power((double)(cD + df) * iD, n));
-                cT += __shfl_sync(0xffffffffu, tf, 31); cD += __shfl_sync(0xffffffffu, df, 31);
             }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < kOwn; u++) {
+                if (pos[u] >= 0) {
+                    const int c = lbk[tid + u * kBkThreads], off = seg[c], L = cnt[c];
+                    const double ke = ckey[pos[u]];
+                    const int ie = cid[pos[u]];
+                    int rank = 0;
+                    for (int j = off; j < off + L; j++) {
+                        const double kj = ckey[j];
+                        rank += (kj > ke || (kj == ke && cid[j] < ie)) ? 1 : 0;
+                    }
+                    sid[off + rank] = ie;
+                }
+            }
+            __syncthreads();
         }
-        best = block_min(best, s_r);
+        // ---- one warp per candidate bucket walks the prefixes
+        if (!crowded && s_nelem > 0) {
+            for (int c = lo + warp; c <= hi; c += kBkThreads / 32) {
+                const int off = seg[c];
+                if (off < 0) continue;
+                const int L = cnt[c];
+                unsigned long long cT = ((unsigned long long)th[c] << 32) | tl[c], cD = ((unsigned long long)dh[c] << 32) | dl[c];
+                for (int base = 0; base < L; base += 32) {
+                    unsigned long long tf = 0, df = 0;
+                    if (base + lane < L) {
+                        const int id = sid[off + base + lane];
+                        tf = mass_fixed(fma(-(double)load_logit<T>(qrow, id), rt, mt), tab);
+                        df = mass_fixed(fma(-(double)load_logit<T>(prow, id), rd, md), tab);
+                    }
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const unsigned long long t2 = __shfl_up_sync(0xffffffffu, tf, o), d2 = __shfl_up_sync(0xffffffffu, df, o);
+                        if (lane >= o) { tf += t2; df += d2; }
+                    }
+                    if (base + lane < L)
+                        best = fmin(best, (double)(cT + tf) * iT - power((double)(cD + df) * iD, n));
+                    cT += __shfl_sync(0xffffffffu, tf, 31); cD += __shfl_sync(0xffffffffu, df, 31);
+                }
+            }
+            best = block_min(best, s_r);
+        }
     }
     if (crowded) todo |= 1 << ni;
     else if (tid == 0) {
@@ -400,6 +476,7 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
         if (GR_CHECK_VALUE || wh->check) {          // (bounds-checked build: an access was out of range)
             if (hdr) hdr->status = GR_CHECK_FAILED;
             if (status_out) status_out[b] = GR_CHECK_FAILED;
+            if (rule_status) rule_status[b] = GR_CHECK_FAILED;
             for (int j = 0; j < nl.count; j++) alpha_out[(size_t)b * nl.count + j] = nanf("");
         }
     }
@@ -416,7 +493,13 @@ fullsort_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, c
     __shared__ double s_min[kFsThreads / 32];
     pdl_wait();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // (normally no row is left to it: a grid of one wave looks)
+    // (normally no row is left to it: a grid of one wave looks, all its rows' flags at once)
+    {
+        int any = 0;
+        for (long long b = blockIdx.x + (long long)tid * gridDim.x; b < batch; b += (long long)kFsThreads * gridDim.x)
+            any |= *reinterpret_cast<const int*>(scratch + (size_t)b * next_pow2(V) * 12);
+        if (!__syncthreads_or(any)) return;
+    }
 #pragma unroll 1
     for (long long b = blockIdx.x; b < batch; b += gridDim.x) {
     const WsHeader* wh = reinterpret_cast<const WsHeader*>(ws + (size_t)b * ws_stride());
@@ -579,7 +662,7 @@ fullsort_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, c
 
 void launch_fullsort(const void* q, const void* p, int dtype, int V, const int* n_list, int n_count, double temp_t,
                      double temp_d, int batch, const char* ws, char* scratch, char* params, int pstride, int force_sort, float* alpha_out,
-                     int* status_out, cudaStream_t st)
+                     int* status_out, int* rule_status, cudaStream_t st)
 {
     NList nl;
     nl.count = n_count;
@@ -603,13 +686,13 @@ void launch_fullsort(const void* q, const void* p, int dtype, int V, const int* 
     const int sort_grid = batch < kSms ? batch : kSms;
     if (dtype == GR_F32) {
         launch_pdl(bucket_alpha_kernel<float>, batch, kBkThreads, kBkSmemBytes, st, (const float*)q, (const float*)p, V, nl,
-                   temp_t, temp_d, ws, scratch, sstride, params, pstride, force_sort, alpha_out, status_out);
+                   1.0 / temp_t, 1.0 / temp_d, ws, scratch, sstride, params, pstride, force_sort, alpha_out, status_out, rule_status);
         launch_pdl(fullsort_alpha_kernel<float>, sort_grid, kFsThreads, kFsSmemBytes, st, (const float*)q, (const float*)p, V,
                    nl, temp_t, temp_d, ws, scratch, params, pstride, batch, alpha_out);
     } else {
         launch_pdl(bucket_alpha_kernel<__nv_bfloat16>, batch, kBkThreads, kBkSmemBytes, st, (const __nv_bfloat16*)q,
-                   (const __nv_bfloat16*)p, V, nl, temp_t, temp_d, ws, scratch, sstride, params, pstride, force_sort,
-                   alpha_out, status_out);
+                   (const __nv_bfloat16*)p, V, nl, 1.0 / temp_t, 1.0 / temp_d, ws, scratch, sstride, params, pstride, force_sort,
+                   alpha_out, status_out, rule_status);
         launch_pdl(fullsort_alpha_kernel<__nv_bfloat16>, sort_grid, kFsThreads, kFsSmemBytes, st, (const __nv_bfloat16*)q,
                    (const __nv_bfloat16*)p, V, nl, temp_t, temp_d, ws, scratch, params, pstride, batch, alpha_out);
     }

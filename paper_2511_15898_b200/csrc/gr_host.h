@@ -29,7 +29,7 @@ int launch_solve_any(char* ws, char* params, int pstride, int kcap, int V, int n
 size_t fullsort_scratch_bytes(int V);
 void launch_fullsort(const void* q, const void* p, int dtype, int V, const int* n_list, int n_count, double temp_t,
                      double temp_d, int batch, const char* ws, char* scratch, char* params, int pstride, int force_sort,
-                     float* alpha_out, int* status_out, cudaStream_t st);
+                     float* alpha_out, int* status_out, int* rule_status, cudaStream_t st);
 void launch_alpha(const char* ws, int V, int topk, double temp_t, double temp_d, const int* n_list, int n_count,
                   int batch, float* alpha_out, int* status_out, cudaStream_t st);
 void launch_verify(const char* params, const int* draft, const float* uni, int batch, int* out_token,

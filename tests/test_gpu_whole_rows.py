@@ -82,3 +82,27 @@ def test_masked_ids_do_not_send_the_row_to_the_sort(V, dt, value):
     record, row = (32 + 128 * 12) // 4, 3 * (1 << (V - 1).bit_length())      # bytes / 4: one record, one row of the scratch
     assert [int(words[2 * record + b * row]) for b in range(2)] == [0, 0]
     assert float((s.alpha_star.double() - _alpha(q, p, 8, 1.0, 1.0)).abs().max()) < 1e-6
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("ids", [1, 20, 64, 127, 128, 129, 1365, 2049])
+def test_candidates_at_the_edges_of_their_paths(ids, dt):
+    """Forty ratios, far enough apart for buckets of their own, of `ids` ids each: one or a few of them are candidates, taken without
+    an order up to 128, in order up to 4096 and left to the sort beyond."""
+    g = torch.Generator(device="cuda").manual_seed(ids)
+    V = 40 * ids + 129
+    q = (torch.randn(4, V, generator=g, device="cuda") * 8).round().clamp(-32, 32) / 4
+    p = q + (torch.arange(V, device="cuda") % 40) / 4
+    q, p = q.to(dt), p.to(dt)
+    ns = [1, 2, 8, 32]
+    out, st = G.alpha_star(q, p, ns, 0, 1.0, 1.0)
+    assert st.tolist() == [0] * 4
+    for j, n in enumerate(ns):
+        assert float((out[:, j].double() - _alpha(q, p, n, 1.0, 1.0)).abs().max()) < 1e-6, n
+    s = G.solve(q, p, 8, 0, 1.0, 1.0)
+    assert s.status.tolist() == [G.GR_SUPPORT_TOO_LARGE] * 4 and torch.equal(s.alpha_star, out[:, 2])
+    bad = q.clone()
+    bad[1, 7] = float("nan")
+    s = G.solve(bad, p, 8, 0, 1.0, 1.0)
+    assert s.status.tolist() == [G.GR_SUPPORT_TOO_LARGE, G.GR_BAD_LOGITS] + [G.GR_SUPPORT_TOO_LARGE] * 2
+    assert bool(torch.isnan(s.alpha_star[1])) and torch.equal(s.alpha_star[2:], out[2:, 2])
