@@ -509,12 +509,19 @@ __device__ __noinline__ void contour_tables(const Circle& ci, int m, double rel,
     const CSm<C, float> cf(sm);
     GR_PTR(double) cw = GR_MKPTR(double, reinterpret_cast<double*>(sm.base + C::oCd), 2 * C::NT, flag);
     const int tid = threadIdx.x, i = tid % C::MP;
-    for (int p = tid / C::MP; p < ci.np; p += C::kNG) {
+    // (points p and np - 1 - p lie on either side of the imaginary axis, angles theta and pi - theta: one sine and cosine for both, and the reciprocal
+    // of the exponential.  np is a multiple of four.)
+    for (int p = tid / C::MP; p < ci.np / 2; p += C::kNG) {
         double sn = 0.0, cs = 1.0, e = 1.0;
         if (i < m) { sincos(ci.r * ci.st[p] * rel, &sn, &cs); e = m_exp(ci.r * ci.ct[p] * rel); }
-        const double re = e * cs - 1.0, im = e * sn;
-        st_d2(cd.E + 2 * (p * C::MP + i), make_double2(re, im));
-        st_f2(cf.E + 2 * (p * C::MP + i), make_float2((float)re, (float)im));
+#pragma unroll
+        for (int z = 0; z < 2; z++) {
+            const int at = z == 0 ? p : ci.np - 1 - p;
+            const double re = e * cs - 1.0, im = e * sn;
+            st_d2(cd.E + 2 * (at * C::MP + i), make_double2(re, im));
+            st_f2(cf.E + 2 * (at * C::MP + i), make_float2((float)re, (float)im));
+            if (z == 0) e = __drcp_rn(e);
+        }
     }
     if (tid < ci.np) {
         double sn, cs;
