@@ -44,14 +44,15 @@ constexpr double kFPredictSafety = 10.0;   // the prediction s2 must be this man
 constexpr double kFRatioSafety = 3.0;      // the residual predicted by the last step's contraction must be this many times below the tolerance
 constexpr double kFTrustPivot = 0.02;      // smallest relative pivot at which a predicted stop is allowed
 constexpr double kFPredictBound = 3.0;     // reported norm after such a stop: kFPredictBound * s2
-constexpr double kFLowLeave = 3.0e-5;      // predicted residual at which the iteration goes over to fp64
+constexpr double kFLowLeave = 3.0e-3;      // bound on the next residual (kFPredictBound * s2; it is mostly a fiftieth of that) at which the iteration goes over to fp64
 constexpr double kFLowFloor = 1.0e-4;      // below this residual a failure to improve is taken for fp32's noise
 constexpr double kFChordBase = 0.02;       // contraction assumed of a step by conjugate gradients (a third of what the stop allows for; 0.008 seen)
 constexpr int kFCgMax = 16;                // conjugate-gradient iterations before the factorisation takes over
 constexpr float kFCgTol = 2.0e-4f;         // and their relative residual; in fp32 kFCgLow times the gradient norm, up to kFCgLoose (at
                                            // 2e-4 throughout no instance of 16 shapes takes an evaluation less; 1 to 3 % more time at 128 tokens)
 constexpr float kFCgLow = 0.1f, kFCgLoose = 5.0e-3f;
-constexpr float kFScaleJump = 0.5f;        // distance of the common scale from which its curve is inverted exactly
+constexpr float kFScaleJump = 0.02f, kFScaleJumpLow = 1.0e-3f, kFScaleJumpFar = 0.5f;    // distance of the common scale from which its curve is inverted exactly, in fp64 and in fp32
+                                           // evaluations (a difference of logarithms: good to 1e-7, which has to be far below the distance, and near the solution below the tolerance)
 constexpr float kFSmallSlack = 1.0e-4f;     // share of the mass below which Tn - sum g is mostly rounding in fp32
 constexpr float kFLeastSlack = 1.0e-9f;     // and the least share aimed at (the quadrature's floor)
 constexpr float kFNone = 1.0e30f;          // no residual or ratio yet
@@ -62,13 +63,11 @@ template <int NT_, int MP_, int T_, int JC_, int CTAS_, int QC_ = 32>
 struct Cfg {
     static constexpr int NT = NT_, MP = MP_, T = T_, JC = JC_, kCtas = CTAS_, kQC = QC_;
     static constexpr bool kContour = NT > 16;     // samples on a circle instead of series (NT: largest number of them)
-    // Fixed-point sweeps of the starting point: five where an evaluation weighs more than the sweeps, three elsewhere.  Three take 0.02
-    // to 0.26 evaluations an instance more up to 64 tokens (n = 8, 1024 rows: k = 50 3.995 to 4.080, k = 20 3.04 to 3.30).  Whole calls, us,
-    // three / five: a batch that leaves an SM with one or two instances 128 headline rows 88.2 / 85.1, 64 whole rows of 16 ids 86 / 78 (three
-    // draws of rows), one row 64.2 / 63.7 (three); series of 16, n = 16, k = 20, 512 rows 133.1 / 129.6, 1777 rows of k = 5 238.2 / 231.1, n = 12,
-    // k = 20 114.8 / 117.2; full SMs with shorter series 1024 headline rows 329.7 / 337.2 (two draws), n = 4, 1024 rows: k = 8 83.6 / 91.4, k = 20
-    // 102.7 / 107.2, k = 50 172.9 / 177.7.  Up to 128 tokens the last two save no evaluation (n = 8, k = 128, solve 365 / 381; n = 16, k = 100 365 / 376).
-    static constexpr int kSweeps = kContour || (MP <= 64 && (NT == 16 || kCtas <= 2)) ? 5 : 3;
+    // Fixed-point sweeps of the starting point: five where an evaluation weighs more than the sweeps, three elsewhere.  Whole calls, us, three / five sweeps:
+    // one headline row 50.8 / 48.7, 256 rows of n = 4, k = 8 52.0 / 51.5, 64 whole rows of 16 ids 60.8 / 59.1 (evaluations 3.96 / 3.81), 512 rows of n = 32,
+    // k = 20 107.1 / 102.8 (2.74 / 2.31); full SMs 1024 headline rows 280.6 / 283.0 (3.04 / 3.01), 600 rows of n = 12, k = 50 138.4 / 139.2, on the circle
+    // with 50 tokens 119.3 / 124.6; up to 128 tokens, 4096 rows of n = 16, k = 100 1431 / 1460, 600 of n = 8 223.5 / 221.9.
+    static constexpr int kSweeps = kContour ? (MP <= 32 ? 5 : 3) : MP <= 64 && (NT == 16 || kCtas <= 2) ? 5 : 3;
     static constexpr int kNG = T / MP;            // copies of the token threads (they share the nodes out among them)
     static constexpr int kW = T / 32, kTW = MP / 32;
     static constexpr int kRow = NT + 4;           // row stride of the product series (16-byte aligned rows in fp32 and fp64)
@@ -1778,7 +1777,8 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
                     const float inv = __fdividef(g0 - slope, g0 * g0);                // 1 / c0
                     const float q = __fdividef(g0 * (1.f - t0 * inv), t0 * (1.f - g0 * inv));
                     far = q > 0.f ? __logf(q) : 0.f;
-                    if (far > kFScaleJump) { shift = fminf(far, 16.f); jump = shift; }
+                    // (under a cap of one or two evaluations there is none left to confirm a short jump by: only a long one, which no Newton step replaces)
+                    if (fabsf(far) > (max_iters < 3 ? kFScaleJumpFar : mode == kLow ? kFScaleJumpLow : kFScaleJump)) { shift = fminf(fmaxf(far, -16.f), 16.f); jump = shift; }
                 }
             }
             // (far from the solution the step need not be solved to more than the model is worth)
@@ -1837,7 +1837,7 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
         const bool trusted = !fail && pivot > (float)kFTrustPivot;
         if (mode == kLow) {
             // the next point is close enough: fp64 from here on, with this factorisation
-            if (kFPredictBound * s2 < kFLowLeave && far <= 0.1f) { mode = trusted ? kChord : kHigh; full_grid = true; dist = dm; }
+            if (kFPredictBound * s2 < kFLowLeave && far <= 0.1f) { mode = trusted ? kChord : kHigh; full_grid = true; dist = far; }
         } else if (trusted && !coarse) {
             const float lin = chol ? 0.f : ((float)kFChordBase + (mode == kChord ? 2.f * dist : 0.f)) * (float)rn;
             const float next = fmaxf(rho, far);
