@@ -244,10 +244,11 @@ __device__ __forceinline__ void riccati_series(R ds, R du, R dp, R* h)
     const R m2 = R(-2) * dp;
 #pragma unroll
     for (int c = 1; c < N; c++) {
+        // (the term with the newest coefficient last: the others do not wait for it)
         R a = R(0);
+        if (c % 2 == 0) a = (R(0.5) * h[c / 2]) * h[c / 2];
 #pragma unroll
-        for (int k = 1; 2 * k < c; k++) a = fma(h[k], h[c - k], a);
-        if (c % 2 == 0) a = fma(R(0.5) * h[c / 2], h[c / 2], a);
+        for (int k = (c - 1) / 2; k >= 1; k--) a = c % 2 != 0 && k == (c - 1) / 2 ? h[k] * h[c - k] : fma(h[k], h[c - k], a);
         h[c + 1] = fma(m2, a, du * h[c]) * R(1.0 / (c + 1));
     }
 }
