@@ -51,8 +51,9 @@ constexpr int kFCgMax = 16;                // conjugate-gradient iterations befo
 constexpr float kFCgTol = 2.0e-4f;         // and their relative residual; in fp32 kFCgLow times the gradient norm, up to kFCgLoose (at
                                            // 2e-4 throughout no instance of 16 shapes takes an evaluation less; 1 to 3 % more time at 128 tokens)
 constexpr float kFCgLow = 0.1f, kFCgLoose = 5.0e-3f;
-constexpr float kFScaleJump = 0.02f, kFScaleJumpLow = 1.0e-3f, kFScaleJumpFar = 0.5f;    // distance of the common scale from which its curve is inverted exactly, in fp64 and in fp32
+constexpr float kFScaleJump = 0.02f, kFScaleJumpLow = 1.0e-3f;    // distance of the common scale from which its curve is inverted exactly, in fp64 and in fp32
                                            // evaluations (a difference of logarithms: good to 1e-7, which has to be far below the distance, and near the solution below the tolerance)
+constexpr float kFScaleJumpFar = 0.5f;     // the same where it is known roughly, or never confirmed
 constexpr float kFSmallSlack = 1.0e-4f;     // share of the mass below which Tn - sum g is mostly rounding in fp32
 constexpr float kFLeastSlack = 1.0e-9f;     // and the least share aimed at (the quadrature's floor)
 constexpr float kFNone = 1.0e30f;          // no residual or ratio yet
@@ -66,8 +67,8 @@ struct Cfg {
     // Fixed-point sweeps of the starting point: five where an evaluation weighs more than the sweeps, three elsewhere.  Whole calls, us, three / five sweeps:
     // one headline row 50.8 / 48.7, 256 rows of n = 4, k = 8 52.0 / 51.5, 64 whole rows of 16 ids 60.8 / 59.1 (evaluations 3.96 / 3.81), 512 rows of n = 32,
     // k = 20 107.1 / 102.8 (2.74 / 2.31); full SMs 1024 headline rows 280.6 / 283.0 (3.04 / 3.01), 600 rows of n = 12, k = 50 138.4 / 139.2, on the circle
-    // with 50 tokens 119.3 / 124.6; up to 128 tokens, 4096 rows of n = 16, k = 100 1431 / 1460, 600 of n = 8 223.5 / 221.9.
-    static constexpr int kSweeps = kContour ? (MP <= 32 ? 5 : 3) : MP <= 64 && (NT == 16 || kCtas <= 2) ? 5 : 3;
+    // with 50 tokens 119.3 / 124.6, with 100 194.5 / 190.8; up to 128 tokens, 4096 rows of n = 16, k = 100 1431 / 1460, 600 of n = 8 223.5 / 221.9.
+    static constexpr int kSweeps = kContour ? (MP == 64 ? 3 : 5) : MP <= 64 && (NT == 16 || kCtas <= 2) ? 5 : 3;
     static constexpr int kNG = T / MP;            // copies of the token threads (they share the nodes out among them)
     static constexpr int kW = T / 32, kTW = MP / 32;
     static constexpr int kRow = NT + 4;           // row stride of the product series (16-byte aligned rows in fp32 and fp64)
@@ -1770,16 +1771,18 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
                 pivot = __fdividef(slope, sums[2]);                 // of the order of the smallest relative pivot
                 float far = 0.f;
                 if (g0 < kFSmallSlack * (float)Tn) {
-                    // too small a difference for fp32; the slope, a sum of positive terms, is the share itself there
+                    // too small a difference for fp32; the slope, a sum of positive terms, is the share itself there, roughly: in fp64 it is for long jumps
+                    // only (from 0.02 on the steps kept away from the solution: 1024 headline rows at a target temperature of 0.2 2620 us for 380)
                     far = __logf(__fdividef(fmaxf(slope, 1.0e-30f), fmaxf(t0, kFLeastSlack * (float)Tn)));
-                    if (mode == kLow || fabsf(far) > kFScaleJump) { shift = fminf(fmaxf(far, -16.f), 16.f); jump = shift; }
+                    if (mode == kLow || fabsf(far) > kFScaleJumpFar) { shift = fminf(fmaxf(far, -16.f), 16.f); jump = shift; }
                 } else if (t0 > 0.f && g0 > slope) {
                     // saturation level c0 from value and slope:  slope = g0 (1 - g0 / c0)
                     const float inv = __fdividef(g0 - slope, g0 * g0);                // 1 / c0
                     const float q = __fdividef(g0 * (1.f - t0 * inv), t0 * (1.f - g0 * inv));
                     far = q > 0.f ? __logf(q) : 0.f;
                     // (under a cap of one or two evaluations there is none left to confirm a short jump by: only a long one, which no Newton step replaces)
-                    if (fabsf(far) > (max_iters < 3 ? kFScaleJumpFar : mode == kLow ? kFScaleJumpLow : kFScaleJump)) { shift = fminf(fmaxf(far, -16.f), 16.f); jump = shift; }
+                    const float least = max_iters < 3 ? kFScaleJumpFar : mode == kLow ? kFScaleJumpLow : kFScaleJump;
+                    if (fabsf(far) > least) { shift = fminf(fmaxf(far, -16.f), 16.f); jump = shift; }
                 }
             }
             // (far from the solution the step need not be solved to more than the model is worth)
