@@ -204,3 +204,13 @@ def test_quadrature_rules_over_the_extents_of_the_weights(n, k, quad_step):
     assert rep.n_status_ok == rep.n_inst and rep.n_struct_mismatch == 0, (rep.summary(), rep.details[:5])
     assert rep.alpha_err <= 1e-6 and rep.cert_solver_max <= 3.2e-7, rep.summary()
     assert rep.n_underreported == 0 and rep.n_evaluated_off == 0, (rep.summary(), rep.details[:5])
+
+
+@pytest.mark.parametrize("n,topk,temp,batch,most", [(8, 50, 0.2, 1024, 16), (8, 50, 0.3, 512, 12), (4, 50, 0.3, 512, 12), (8, 128, 0.3, 512, 18)])
+def test_low_target_temperatures_stay_with_the_fast_kernel(n, topk, temp, batch, most):
+    """Acceptances close to one, slacks far below what fp32 resolves: no instance takes more evaluations than a few beyond 14, 9, 9 and 15 on
+    these rows (17 to 22 and the general kernel when fp64 evaluations took short jumps of a roughly known common scale)."""
+    wl = W.config3(batch=batch, device="cuda", V=20000, n=n, topk=topk, seed=3)
+    r = G.read_rule(G.solve(wl.q_logits, wl.p_logits, n, topk, temp, 1.0))
+    assert set(r.status.tolist()) == {G.GR_OK}
+    assert int((r.iters & 0xffff).max()) <= most
