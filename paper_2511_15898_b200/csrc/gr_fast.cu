@@ -39,8 +39,8 @@ int launch_fast(GR_FAST_ARGS)
 #define GR_FAST_PASS ws, params, pstride, kcap, V, n, topk, temp_t, temp_d, tol, max_iters, qstep, tau, batch, alpha_out, status_out, fa, st
     // Twice to four times the threads per instance, and registers without spills, where the batch leaves an SM with one
     // instance (two of the narrow supports): an instance is a chain of dependent steps then, and 1 row of the headline shape
-    // takes 81 us a call for 90, 128 rows 102 for 111, 64 whole rows of 16 ids 72 for 78.  Beyond one wave the other variants' places
-    // count for more (1024 headline rows: 484 us a call in the wide variant, 354 in the other; 512 rows, n = 16, k = 20, 155 and 143).
+    // takes 50.5 us a call for 59.0, 128 rows 75 for 83, 64 whole rows of 16 ids 58 for 67.  Beyond one wave the other variants' places
+    // count for more (1024 rows of 9001, n = 8, k = 50: 253 us a call in the wide variant, 138 in the other; 512 rows, n = 16, k = 20, 92 and 71).
     const bool one = batch <= kSms, two = batch <= 2 * kSms;
     if (n > 16) {
         if (kcap <= 32) return two ? fast::launch_fast_c24_m32w(GR_FAST_PASS) : fast::launch_fast_c24_m32(GR_FAST_PASS);
