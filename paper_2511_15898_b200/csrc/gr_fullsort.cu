@@ -42,7 +42,7 @@ constexpr int kBkFew = 128;                       // up to so many are taken wit
 constexpr int kBkTab = 128, kBkCopies = 16;       // 2^(42 + j / 128), a copy for every lane of a half-warp
 constexpr int kBkSmemBytes = kBkBuckets * (4 * 4 + 4 + 4) + kBkMaxCand * (8 + 4 + 4 + 4 + 4) + kBkTab * kBkCopies * 8;
 
-// exp(-y) in units of 2^-42, rounded to an integer (masses are summed as integers: exact, order-free).  y >= 0 (but for its last bit).
+// exp(-y) in units of 2^-42, rounded to an integer (masses are summed as integers: exact, order-free).  y >= 0, up to infinity.
 // 2^(k/128) from a table times a degree-4 Taylor polynomial on |r| <= ln2/256 (1.2e-15 relative, a hundredth of the unit; degree 5 and 32
 // entries took two operations more), scaled and rounded by one multiplication and addition: nine fp64 operations.
 __device__ __forceinline__ unsigned long long mass_fixed(double y, GR_PTR(const double) tab)
@@ -174,9 +174,13 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
     const T* qrow = q + (size_t)b * V;
     const T* prow = p + (size_t)b * V;
     const FullRow fr = *reinterpret_cast<const FullRow*>(rec + sizeof(WsHeader));
-    // (scaled logits as products with the reciprocal temperatures rt and rd: one rounding away from the quotients the sort
-    // uses, which moves alpha* by ~1e-16; every pass here forms them the same way)
-    const double mt = (double)fr.qmax * rt, md = (double)fr.pmax * rd;
+    // Exponents: a logit's distance from its row's maximum, times the reciprocal temperature (a rounding or two from the quotients the sort
+    // uses, which moves alpha* by ~1e-16).  The subtraction comes first: zero for the maximum and never negative, however large the logits are.
+    // (One operation less as m - a rt with m rounded, but what m loses, 2^-53 of it, is then every exponent's error: from logits of 1e17
+    // on the maximum itself had no mass.)
+    const double qm = (double)fr.qmax, pm = (double)fr.pmax, mt = qm * rt, md = pm * rd;
+    auto exp_t = [&](float x) { return (qm - (double)x) * rt; };
+    auto exp_d = [&](float v) { return (pm - (double)v) * rd; };
     // bucket of a key d - a: floor((kmax - key) * invw), clamped, formed from the logits at once (two operations; rounding moves an id whose
     // key is 1e-13 of a bucket's width from its border, which changes no mass by more, and the bound below allows for it).  (kmax
     // and kmin are fp32 values: a key may lie outside.)
@@ -209,8 +213,8 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
         const double a = (double)x, d = (double)v;
         const double t = __dadd_rd(fma(a, ca, fma(d, cd, c0)), 6755399441055744.0);
         const int c = min(max(__double2loint(t), 0), kBkBuckets - 1);
-        add_mass(tl, th, c, mass_fixed(fma(-a, rt, mt), tab));
-        add_mass(dl, dh, c, mass_fixed(fma(-d, rd, md), tab));
+        add_mass(tl, th, c, mass_fixed(exp_t(x), tab));
+        add_mass(dl, dh, c, mass_fixed(exp_d(v), tab));
         return c;
     };
     const int nvec = (V - head) / N, tail0 = head + nvec * N;
@@ -367,7 +371,7 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
                 const int i = lid[tid];
                 const float x = load_logit<T>(qrow, i), v = load_logit<T>(prow, i);
                 ckey[tid] = key_of(x, v);
-                mt_f[tid] = mass_fixed(fma(-(double)x, rt, mt), tab); md_f[tid] = mass_fixed(fma(-(double)v, rd, md), tab);
+                mt_f[tid] = mass_fixed(exp_t(x), tab); md_f[tid] = mass_fixed(exp_d(v), tab);
             }
             __syncthreads();
             for (int e = warp; e < found; e += kBkThreads / 32) {
@@ -444,8 +448,8 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
                     unsigned long long tf = 0, df = 0;
                     if (base + lane < L) {
                         const int id = sid[off + base + lane];
-                        tf = mass_fixed(fma(-(double)load_logit<T>(qrow, id), rt, mt), tab);
-                        df = mass_fixed(fma(-(double)load_logit<T>(prow, id), rd, md), tab);
+                        tf = mass_fixed(exp_t(load_logit<T>(qrow, id)), tab);
+                        df = mass_fixed(exp_d(load_logit<T>(prow, id)), tab);
                     }
                     for (int o = 1; o < 32; o <<= 1) {
                         const unsigned long long t2 = __shfl_up_sync(0xffffffffu, tf, o), d2 = __shfl_up_sync(0xffffffffu, df, o);

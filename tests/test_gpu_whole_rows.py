@@ -106,3 +106,40 @@ def test_candidates_at_the_edges_of_their_paths(ids, dt):
     s = G.solve(bad, p, 8, 0, 1.0, 1.0)
     assert s.status.tolist() == [G.GR_SUPPORT_TOO_LARGE, G.GR_BAD_LOGITS] + [G.GR_SUPPORT_TOO_LARGE] * 2
     assert bool(torch.isnan(s.alpha_star[1])) and torch.equal(s.alpha_star[2:], out[2:, 2])
+
+
+def _alpha_of_large(q, p, n, tt, td):
+    """The same where logits are so large that a difference of scaled logits keeps nothing of the smaller one: the ratio order by the
+    logits' distances from their row's maximum."""
+    q, p = ((x.double() - x.double().max(1, keepdim=True).values) / t for x, t in ((q, tt), (p, td)))
+    return _alpha(q, p, n, 1.0, 1.0)
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("V", [2000, 50257])
+@pytest.mark.parametrize("where", ["target", "draft", "both", "two ids"])
+def test_any_finite_value_is_a_logit(V, dt, where):
+    """One logit of up to 1e30: its distribution is a point, whatever the temperature's reciprocal rounds to."""
+    g = torch.Generator(device="cuda").manual_seed(V)
+    values = [1.0e6, 1.0e10, 1.0e17, 1.0e18, 1.0e20, 1.0e25, 1.0e28, 1.0e30]
+    q = (3 * torch.randn(len(values), V, generator=g, device="cuda")).to(dt)
+    p = (q.float() + torch.randn(len(values), V, generator=g, device="cuda")).to(dt)
+    v = torch.tensor(values, dtype=torch.float64, device="cuda").to(dt)
+    # (the target's point on the draft's likeliest id: an acceptance well away from one)
+    at = p.argmax(1)
+    rows = torch.arange(len(values), device="cuda")
+    if where != "draft":
+        q[rows, at] = v
+    if where in ("draft", "both"):
+        p[rows, at] = v
+    if where == "two ids":
+        p[rows, (at + 1) % V] = v
+    ns = [1, 2, 8, 32]
+    for tt, td in [(0.6, 0.7), (0.7, 1.0), (0.75, 1.25), (0.8, 0.75), (1.25, 0.6), (1.0, 1.0)]:
+        out, st = G.alpha_star(q, p, ns, 0, tt, td)
+        assert st.tolist() == [0] * len(values)
+        s = G.solve(q, p, 8, 0, tt, td)
+        assert torch.equal(s.alpha_star, out[:, 2])
+        for j, n in enumerate(ns):
+            err = (out[:, j].double() - _alpha_of_large(q, p, n, tt, td)).abs()
+            assert float(err.max()) < 1e-6, (tt, td, n, err.tolist())
