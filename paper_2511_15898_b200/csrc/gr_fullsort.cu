@@ -178,16 +178,20 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
     // uses, which moves alpha* by ~1e-16).  The subtraction comes first: zero for the maximum and never negative, however large the logits are.
     // (One operation less as m - a rt with m rounded, but what m loses, 2^-53 of it, is then every exponent's error: from logits of 1e17
     // on the maximum itself had no mass.)
-    const double qm = (double)fr.qmax, pm = (double)fr.pmax, mt = qm * rt, md = pm * rd;
-    auto exp_t = [&](float x) { return (qm - (double)x) * rt; };
-    auto exp_d = [&](float v) { return (pm - (double)v) * rd; };
-    // bucket of a key d - a: floor((kmax - key) * invw), clamped, formed from the logits at once (two operations; rounding moves an id whose
-    // key is 1e-13 of a bucket's width from its border, which changes no mass by more, and the bound below allows for it).  (kmax
-    // and kmin are fp32 values: a key may lie outside.)
+    const double qm = (double)fr.qmax, pm = (double)fr.pmax;
+    auto exp_t = [&](float x) { return __dmul_rn(qm - (double)x, rt); };
+    auto exp_d = [&](float v) { return __dmul_rn(pm - (double)v, rd); };
+    // The keys here are the log-ratios draft / target less those of the rows' maxima, exp_t - exp_d: nothing of them is lost to what a row's
+    // logits have in common.  Bucket of a key: floor((kmax - key) * invw), clamped, one fused operation on the key and so a non-increasing function of
+    // it in floating point too.  The streaming pass's kmax and kmin are fp32 values, and keys that overflow fp32 are not among
+    // them: a key may lie outside (in the first or the last bucket; the bounds below hold for any kmax and width), and without a usable range there
+    // is one bucket.
     const double ln2 = 0.6931471805599453;
-    const double kmax = (double)fr.kmax * ln2, span = kmax - (double)fr.kmin * ln2;
+    const double span = ((double)fr.kmax - (double)fr.kmin) * ln2;
+    const bool ranged = span > 0.0 && span < INFINITY;
+    const double kmax = ranged ? (double)fr.kmax * ln2 - (pm * rd - qm * rt) : 0.0;
     // (what every thread needs the same is formed by one: a quotient by 1024 threads keeps the fp64 units busy for 700 cycles)
-    if (tid == 0) s_c[0] = span > 0.0 ? (double)kBkBuckets / (span * (1.0 + 1e-9)) : 0.0;
+    if (tid == 0) s_c[0] = ranged ? (double)kBkBuckets / (span * (1.0 + 1e-9)) : 0.0;
     // (masses and counts lie behind one another)
     static_assert(5 * kBkBuckets % (4 * kBkThreads) == 0 && kBkBuckets == 4 * kBkThreads && kBkTab <= kBkThreads, "a vector per thread");
 #pragma unroll
@@ -207,14 +211,16 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
     const int head = row_head(q, b, V, (int)sizeof(T)), shift = (N - head % N) % N;
     unsigned short* const code_raw = reinterpret_cast<unsigned short*>(scr + 16);
     GR_PTR(unsigned short) code = GR_MKPTR(unsigned short, code_raw, V + 16, GR_CHECK_FLAG);
-    auto key_of = [&](float x, float v) { return (double)v * rd - (double)x * rt; };
-    const double ca = rt * invw, cd = -rd * invw, c0 = kmax * invw;
+    auto key_of = [&](float x, float v) { return exp_t(x) - exp_d(v); };
+    const double c0 = kmax * invw;
     auto element = [&](float x, float v) {
-        const double a = (double)x, d = (double)v;
-        const double t = __dadd_rd(fma(a, ca, fma(d, cd, c0)), 6755399441055744.0);
-        const int c = min(max(__double2loint(t), 0), kBkBuckets - 1);
-        add_mass(tl, th, c, mass_fixed(exp_t(x), tab));
-        add_mass(dl, dh, c, mass_fixed(exp_d(v), tab));
+        const double yt = exp_t(x), yd = exp_d(v), t = fma(yt - yd, -invw, c0);
+        // (clamped by the leading word, to [0, 4096): the trailing one of a number that the magic constant does not hold says nothing)
+        static_assert(kBkBuckets == 4096, "0x40affffe: the last numbers below it");
+        const double u = __hiloint2double(min(max(__double2hiint(t), 0), 0x40affffe), __double2loint(t));
+        const int c = __double2loint(__dadd_rd(u, 6755399441055744.0));
+        add_mass(tl, th, c, mass_fixed(yt, tab));
+        add_mass(dl, dh, c, mass_fixed(yd, tab));
         return c;
     };
     const int nvec = (V - head) / N, tail0 = head + nvec * N;
@@ -272,13 +278,16 @@ bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, con
         put(dl, dh, s[1], mD);
     }
     // tgt_i / drf_i = exp(-key_i) * rscale.  Every ratio of bucket c is at least rho: its keys are at most kmax - c w (rho of a thread's first bucket
-    // as a product of two numbers, of the others one from the other; where the factors are far from overflowing).
+    // as a product of two numbers, of the others one from the other; where the factors are far from overflowing).  The number of an id is rounded: its
+    // key lies at most 2^-53 |kmax| above  kmax - c w (1 - 2^-53).  The 1e-12 taken off the width and the 1e-9 off rho cover that for kmax up to 1e7;
+    // beyond, rho is zero unless c w is nearly kmax, which the 1e-12 covers.  (The draft's likeliest id has a key of at least zero: a kmax below, by fp32
+    // rounding, leaves every id with draft mass in the first bucket.)
     const double wide = invw > 0.0 ? (1.0 - 1e-12) / invw : 0.0;
     if (warp == 0) s_up[lane] = exp((double)(lane * kBkPer) * fmin(wide, 1.0));
     else if (warp == 1) s_at[lane] = exp((double)(32 * lane * kBkPer) * wide - kmax);
     else if (tid == 64) { s_c[1] = 1.0 / (double)totT; s_c[4] = (double)(V + 1) * s_c[1] + 1e-14; }
     else if (tid == 96) s_c[2] = 1.0 / (double)totD;
-    else if (tid == 128) s_c[3] = exp(md - mt) * ((double)totD / (double)totT) * (1.0 - 1e-9);
+    else if (tid == 128) s_c[3] = (double)totD / (double)totT * (1.0 - 1e-9);
     else if (tid == 160) s_c[5] = exp(fmin(wide, 1.0));
     __syncthreads();
     const double iT = s_c[1], iD = s_c[2], rscale = s_c[3], slack = s_c[4], grow = s_c[5];

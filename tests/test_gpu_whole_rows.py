@@ -119,9 +119,9 @@ def _alpha_of_large(q, p, n, tt, td):
 @pytest.mark.parametrize("V", [2000, 50257])
 @pytest.mark.parametrize("where", ["target", "draft", "both", "two ids"])
 def test_any_finite_value_is_a_logit(V, dt, where):
-    """One logit of up to 1e30: its distribution is a point, whatever the temperature's reciprocal rounds to."""
+    """One logit of up to the type's largest value: its distribution is a point, whatever the temperature's reciprocal rounds to."""
     g = torch.Generator(device="cuda").manual_seed(V)
-    values = [1.0e6, 1.0e10, 1.0e17, 1.0e18, 1.0e20, 1.0e25, 1.0e28, 1.0e30]
+    values = [1.0e6, 1.0e10, 1.0e17, 1.0e18, 1.0e20, 1.0e30, 0.99 * torch.finfo(dt).max, torch.finfo(dt).max]
     q = (3 * torch.randn(len(values), V, generator=g, device="cuda")).to(dt)
     p = (q.float() + torch.randn(len(values), V, generator=g, device="cuda")).to(dt)
     v = torch.tensor(values, dtype=torch.float64, device="cuda").to(dt)
@@ -141,5 +141,46 @@ def test_any_finite_value_is_a_logit(V, dt, where):
         s = G.solve(q, p, 8, 0, tt, td)
         assert torch.equal(s.alpha_star, out[:, 2])
         for j, n in enumerate(ns):
+            err = (out[:, j].double() - _alpha_of_large(q, p, n, tt, td)).abs()
+            assert float(err.max()) < 1e-6, (tt, td, n, err.tolist())
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("V", [2000, 50257])
+@pytest.mark.parametrize("masked", ["target", "draft"])
+@pytest.mark.parametrize("value", [-1.0e4, -1.0e18, -1.0e30, None])
+def test_ids_masked_in_one_row_only(V, dt, masked, value):
+    """Ids that one of the distributions excludes, by a value of up to the type's lowest, come first (no target mass) or last (no draft mass)
+    in the ratio order: their log-ratio is far outside the other ids' range, or overflows fp32."""
+    value = torch.finfo(dt).min if value is None else value
+    for seed, (tt, td) in enumerate([(1.0, 1.0), (0.7, 1.0), (0.75, 1.25), (1.25, 0.6)]):
+        g = torch.Generator(device="cuda").manual_seed(100 * V + seed)
+        q = (3 * torch.randn(6, V, generator=g, device="cuda")).to(dt)
+        p = (q.float() + torch.randn(6, V, generator=g, device="cuda")).to(dt)
+        gone = torch.rand(6, V, generator=g, device="cuda") < torch.tensor([0.5, 0.5, 0.1, 0.01, 0.9, 0.001], device="cuda")[:, None]
+        (q if masked == "target" else p)[gone] = value
+        ns = [1, 2, 8, 32]
+        out, st = G.alpha_star(q, p, ns, 0, tt, td)
+        assert st.tolist() == [0] * 6
+        sort = G.solve(q, p, 8, 0, tt, td, G.Options(force_robust=1)).alpha_star
+        assert float((out[:, 2] - sort).abs().max()) < 1e-6
+        for j, n in enumerate(ns):
+            err = (out[:, j].double() - _alpha_of_large(q, p, n, tt, td)).abs()
+            assert float(err.max()) < 1e-6, (tt, td, n, err.tolist())
+
+
+@pytest.mark.parametrize("V", [2000, 50257])
+@pytest.mark.parametrize("offset", [30.0, 1.0e3, 1.0e5, -1.0e6, 3.0e7, 1.0e9])
+def test_common_offsets_and_narrow_ranges(V, offset):
+    """Distributions are those of the logits without a common offset.  Rounded to fp32 beside it, the range of the ratios spans a few or
+    many of fp32's steps, down to 0.001."""
+    g = torch.Generator(device="cuda").manual_seed(V)
+    q = 3 * torch.randn(4, V, generator=g, device="cuda")
+    p = q + torch.tensor([1.0, 1.0e-3, 1.0, 0.1], device="cuda")[:, None] * torch.randn(4, V, generator=g, device="cuda")
+    q, p = q + offset, p + torch.tensor([0.0, 0.0, 1.0, -1.0], device="cuda")[:, None] * offset
+    for tt, td in [(1.0, 1.0), (0.7, 0.7), (0.75, 1.25)]:
+        out, st = G.alpha_star(q, p, [2, 8, 32], 0, tt, td)
+        assert st.tolist() == [0] * 4
+        for j, n in enumerate([2, 8, 32]):
             err = (out[:, j].double() - _alpha_of_large(q, p, n, tt, td)).abs()
             assert float(err.max()) < 1e-6, (tt, td, n, err.tolist())
