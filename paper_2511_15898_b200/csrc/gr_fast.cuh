@@ -1948,12 +1948,12 @@ fast_solve_kernel(char* __restrict__ ws, char* __restrict__ params, int pstride,
         // (a block of one token: its weight says nothing)
         if (!inner && hi - lo == 1 && !trunc) { lo = hi; continue; }
         const bool wanted = sel == -2 || (inner ? sel < 0 : sel == bk);
-        // tokens of the system in ascending draft mass (16 bits of it are enough to order them; positions break ties, so that no two keys
-        // are equal; what is not in the truncation set, or behind the last token, has the key of none)
+        // tokens of the system in ascending draft mass (fp32 is enough to order them), equal masses by position: a key of an earlier position
+        // counts as larger where it is equal.  What is not in the truncation set, or behind the last token, has the key of none, far below all others.
         GR_PTR(unsigned) okey = GR_PCAST(unsigned, sm.wd);
         unsigned mine = 0u;
         const bool in = tid < hi - lo && (!trunc || sm.trunc[lo + tid] != 0);
-        if (in) mine = ((0x7fffffffu - __float_as_uint((float)sm.d[lo + tid])) & ~127u) | (unsigned)(127 - tid);
+        if (in) mine = 0x7fffffffu - __float_as_uint((float)sm.d[lo + tid]);
         if (tid < ((hi - lo + 3) & ~3)) okey[tid] = mine;
         const int m = __syncthreads_count(in);
         if (in) {
@@ -1961,7 +1961,8 @@ fast_solve_kernel(char* __restrict__ ws, char* __restrict__ params, int pstride,
 #pragma unroll 4
             for (int j = 0; j < hi - lo; j += 4) {
                 const uint4 o = ld_u4(okey + j);
-                above += (o.x > mine ? 1 : 0) + (o.y > mine ? 1 : 0) + (o.z > mine ? 1 : 0) + (o.w > mine ? 1 : 0);
+                above += (o.x + (j < tid ? 1u : 0u) > mine ? 1 : 0) + (o.y + (j + 1 < tid ? 1u : 0u) > mine ? 1 : 0) +
+                         (o.z + (j + 2 < tid ? 1u : 0u) > mine ? 1 : 0) + (o.w + (j + 3 < tid ? 1u : 0u) > mine ? 1 : 0);
             }
             sm.ord[above] = lo + tid;
         }
