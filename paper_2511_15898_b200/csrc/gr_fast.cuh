@@ -56,6 +56,7 @@ constexpr float kFScaleJump = 0.02f, kFScaleJumpLow = 1.0e-3f;    // distance of
 constexpr float kFScaleJumpFar = 0.5f;     // the same where it is known roughly, or never confirmed
 constexpr float kFSmallSlack = 1.0e-4f;     // share of the mass below which Tn - sum g is mostly rounding in fp32
 constexpr float kFLeastSlack = 1.0e-9f;     // and the least share aimed at (the quadrature's floor)
+constexpr double kFLowEnds = 1.0e-4;       // tolerance from which on an fp32 evaluation may end the iteration
 constexpr float kFNone = 1.0e30f;          // no residual or ratio yet
 
 // Compile-time geometry.  NT: series length (>= n), MP: padded support size, T: threads, JC: Hessian nodes staged
@@ -370,14 +371,19 @@ __device__ __forceinline__ void hess_mma(const FSm<C>& sm, Frags<C>& fr, int kst
 
 // Extent of a point's weights: the extreme log-weights, and the largest over the smallest total W of a tuple's weights (slack +
 // sum over its distinct tokens), infinite where the caller's quadrature step asks for more than the tables hold.
-struct Extent { float amax, amin, ratio; };
-__device__ __forceinline__ Extent extent_of(float amax, float amin, float wsum, int n, int slack, double qstep)
+// Beside it which sum an fp32 evaluation takes: its nodes (0: the trapezoid rule) and first entry.
+struct Extent { float amax, amin, ratio; int nodes, at; };
+__device__ __forceinline__ Extent extent_of(float amax, float amin, float wsum, int n, int slack, double qstep, double tol)
 {
     Extent e;
     e.amax = amax; e.amin = amin;
     const float s = slack ? 1.f : 0.f;
     // (rounded up: exponentials of fp32 log-weights are good to 1e-5)
     e.ratio = qstep >= kTableStep ? 1.0001f * (s + fminf(wsum, (float)n * Rx<float>::ex(amax))) / (s + Rx<float>::ex(amin)) : INFINITY;
+    const bool fine = tol >= kFLowEnds;
+    const int level = fine ? quad_level<double>(e.ratio) : quad_level<float>(e.ratio);
+    e.nodes = level < (fine ? kLevels64 : kLevels32) ? 2 * (level + 1) : 0;
+    e.at = level * (level + 1) + (fine ? kFine : 0);
     return e;
 }
 
@@ -395,10 +401,11 @@ struct Grid {
     __device__ __forceinline__ Grid(const Extent& e, int slack, R qstep)
     {
         const float wmin = Rx<float>::ex(e.amin), s = slack ? 1.f : 0.f;
-        const int level = quad_level<R>(e.ratio);
-        table = level < QuadTable<R>::kLevels;
+        int level = 0;
+        if (sizeof(R) == 8) { level = quad_level<double>(e.ratio); table = level < kLevels64; }
+        else table = e.nodes > 0;
         if (table) {
-            Q = 2 * (level + 1); at = level * (level + 1);
+            Q = sizeof(R) == 8 ? 2 * (level + 1) : e.nodes; at = sizeof(R) == 8 ? level * (level + 1) : e.at;
             unit = (R)__fdividef(1.00005f, s + wmin);              // (any number not below 1 / lo)
             s_hi = s0 = 0.f;
         } else {
@@ -1304,7 +1311,7 @@ __device__ __noinline__ double2 eval_hessian(int m, int n, int slack, bool coars
     double g, g2;
     const double qstep = sm.scal[SC_QSTEP] * (coarse ? 2.0 : 1.0);
     // (a table's nodes all serve the Hessian, of the full trapezoid grid every other one)
-    const int jstride = coarse || quad_level<float>(ext.ratio) < QuadTable<float>::kLevels ? 1 : 2;
+    const int jstride = coarse || ext.nodes > 0 ? 1 : 2;
     const double rhs = i < m ? sm.rhs[sm.ord[i]] : 0.0;
     const float zr = i < m ? (float)rhs : 1.f, zi = rsqrtf(zr);
     if constexpr (C::kContour) eval_contour<C, float, true>(sm, m, slack, qstep, jstride, ext, sm.wd[i], i < m ? zi : 0.f, g, g2, fr);
@@ -1674,7 +1681,7 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
     double rn = 0.0;
     // (what steers the iteration only is fp32: it is compared with margins of three and more, and in fp64 cost 1 % at series of 16)
     float rprev = kFNone, lam = 1.f, dist = 0.f;
-    Extent ext{0.f, 0.f, 0.f};               // of the weights
+    Extent ext{0.f, 0.f, 0.f, 0, 0};         // of the weights
     bool ranged = false;                     // they are known for this point
     // Three modes.  Low: gradient and Hessian in fp32, conjugate gradients.  Chord: fp64 gradient, the last Hessian.  High:
     // fp64 gradient, fp32 Hessian of the same point, with `chol` a Cholesky factorisation.  A single token that dominates a
@@ -1690,12 +1697,12 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
             unsigned top[2] = {act ? fkey((float)alpha) : 0u, act ? fkey(-(float)alpha) : 0u};
             float wsum = act ? Rx<float>::ex((float)alpha) : 0.f;
             tok_reduce<C, 0, 1, 2>(sm, nullptr, &wsum, top, par);
-            ext = extent_of(fkey_inv(top[0]), -fkey_inv(top[1]), wsum, n, slack, sm.scal[SC_QSTEP]);
+            ext = extent_of(fkey_inv(top[0]), -fkey_inv(top[1]), wsum, n, slack, sm.scal[SC_QSTEP], sm.scal[SC_TOL]);
         }
         ranged = false;
         // On the trapezoid rule the step is doubled far from the solution (quadrature error ~1e-4, far below the gradient norm
         // there): half the nodes, every one of them a Hessian node.  Convergence is only declared on the full grid.
-        const bool coarse = rprev > kFCoarse && !full_grid && mode != kChord && !(ext.ratio <= kTableReach);
+        const bool coarse = rprev > kFCoarse && !full_grid && mode != kChord && ext.nodes == 0;
         const int kind = 2 * mode + (coarse ? 1 : 0);
         __syncthreads();
         double2 gg = make_double2(0.0, 0.0);
@@ -1716,10 +1723,10 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
         // (residuals are only compared within one grid and one precision)
         const bool comparable = kind == was_kind && it > 0;
         was_kind = kind;
-        // Stop on an evaluated residual.  (An fp32 evaluation on the full grid is good to ~1e-6: enough to see a tolerance
-        // of 1e-4 and more met.  Between half the tolerance and the tolerance one more step, which costs a tenth of an
+        // Stop on an evaluated residual.  (An fp32 evaluation by the fine sums or on the full grid is good to ~1e-6, where a dominant token's terms
+        // cancel to 4e-5: enough to see a tolerance of 1e-4 and more met.  Between half the tolerance and the tolerance one more step, which costs a tenth of an
         // evaluation, leaves a residual far below it, unless steps have stopped helping.)
-        if (rn <= tol && !coarse && (mode != kLow || tol >= 1.0e-4) && (rn <= 0.5 * tol || (comparable && rn > 0.5 * rprev))) {
+        if (rn <= tol && !coarse && (mode != kLow || tol >= kFLowEnds) && (rn <= 0.5 * tol || (comparable && rn > 0.5 * rprev))) {
             status = GR_OK; it++;
             break;
         }
@@ -1816,7 +1823,7 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
             mode = kHigh; chol = true; full_grid = true; rprev = kFNone; was_kind = -1;
             continue;
         }
-        ext = extent_of(fkey_inv(top[1]), -fkey_inv(top[2]), wsum, n, slack, sm.scal[SC_QSTEP]);
+        ext = extent_of(fkey_inv(top[1]), -fkey_inv(top[2]), wsum, n, slack, sm.scal[SC_QSTEP], sm.scal[SC_TOL]);
         ranged = !(dm > (float)kFStepClamp);
         // a full Newton step below 1e-11 in alpha: the weights cannot be improved at this quadrature accuracy
         if (!fail && mode != kLow && far < 1.0e-11f) { status = GR_OK; it++; break; }
