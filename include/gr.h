@@ -80,7 +80,9 @@ extern "C" {
  *              lin = (0.02 + 2 x the distance to that point) x the residual: stop when
  *              10 s2 + 3 lin < tol, reported 3 s2 + lin.  By the ratio (faster kernel only):
  *              after a step that contracted the residual to r by rho < 0.1, stop when
- *              3 max(rho, the step's length) r < tol, reported max(rho, length) r.  Neither
+ *              3 c r < tol, reported c r, with c the largest of rho, the step's length and (with such a
+ *              Hessian) 0.02 + 2 x the distance.  On 22 kinds of rows at tolerances of 1e-8, 3e-7 and 1e-5 a stop
+ *              left at most 0.42 of what it reported, beyond the floor of 3e-9.  Neither
  *              is used when the Newton system is too close to singular in fp32: less than 2 %
  *              of a diagonal entry left as the factorisation's pivot, or of the Hessian's trace
  *              as the slope along the common scale of the weights.

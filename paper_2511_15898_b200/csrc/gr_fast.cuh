@@ -22,8 +22,8 @@
 //     lambda, so [lambda^n] is a mean over a few points of |lambda| = 0.8 n (conjugate pairs, 16 to 24 of them), exact to
 //     1e-11 and free of the cancellation that a dominant token brings into the division e / f as series;
 //   - the iteration runs in fp32 as long as the residual is far above fp32's noise; the last evaluations, the only ones
-//     that can end it, are fp64 on the full quadrature grid and reuse the last factorisation (a Newton step with a
-//     Hessian from a point 1e-4 away contracts as well as one with a fresh one).
+//     that can end it at a tolerance below 1e-4, are fp64 and reuse the last Hessian (a Newton step with a Hessian from a point at a
+//     distance of d in alpha leaves 0.02 + d of the residual at most: 0.004 away, the median, as little as one with a fresh one).
 #pragma once
 #include "gr_prep.cuh"
 #include "gr_verify.cuh"
@@ -1830,16 +1830,20 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
         if (dm > (float)kFStepClamp && act) dl = jump + (dl - (double)jump) * (double)__fdividef((float)kFStepClamp, dm);
         alpha = fmin(fmax(alpha + dl, -kFAlphaClamp), kFAlphaClamp);
         // Stop on a predicted residual, without another evaluation, after a step from a point evaluated in fp64 on the
-        // full grid.  Measured with this iteration against the oracle's residual at the weights returned, 7000 such stops at tolerances
-        // of 1e-8, 3e-7 and 1e-5: every benchmark shape, random rows of 16 to 128 tokens with 2 to 32 drafts, whole and truncated, and
-        // rows picked for prefixes that are almost tight (weights on several scales), 6231 in inner systems, 767 in outer blocks:
-        // (i) By the step.  Second order: s2 = sum_i g_i delta_i^2 (each flow is a sum of terms exponential in alpha over
-        // positive normalisers).  First order, after conjugate gradients: what the half-precision Hessian leaves of the residual,
-        // plus the distance to the point where a reused one was formed.  Left were never more than 8.5 s2 + 0.008 of the residual
-        // + the quadrature floor of ~3e-9, and never more than half of what is held against the tolerance.
-        // (ii) By the ratio: the last full step on this grid contracted the residual by rho < 0.1, and the next one is taken
-        // to contract by no less than that and its own length (along a direction in which the flows hardly change s2 says
-        // nothing, and the length of the step times the residual is what it leaves: 0.63 of that in the worst of 23 such stops).
+        // full grid.  Measured with this iteration against the oracle's residual at the weights returned, 7633 such stops at tolerances
+        // of 1e-8 (quadrature steps 0.25 and 0.4), 3e-7 and 1e-5 on 22 kinds of rows: every benchmark shape, random rows of 16 to 128 tokens with 2 to 32 drafts,
+        // whole and truncated, and rows picked for prefixes that are almost tight (weights on several scales); 842 in outer blocks.  6498 were an
+        // instance's only system and are held one by one against what they left, less the floor of 3e-9:
+        // (i) By the step (6484).  Second order: s2 = sum_i g_i delta_i^2 (each flow is a sum of terms exponential in alpha over
+        // positive normalisers).  First order, after conjugate gradients: what the half-precision Hessian leaves of the residual (403 stops
+        // after a fresh one: 0.0125 of it at most), plus the distance to the point where a reused one was formed (6073 stops, distances of 0.004 in the
+        // median, 0.028 in one of ten, 0.11 at most: 0.45 lin at most).  Left were never more than 13 % of 10 s2 + 3 lin, 38 % of the norm reported
+        // and 10 % of the tolerance; lin is the larger term in all but 25.
+        // (ii) By the ratio (14): the last full step on this grid contracted the residual by rho < 0.1, and the next one is taken
+        // to contract by no less than that, its own length (along a direction in which the flows hardly change s2 says
+        // nothing, and the length of the step times the residual is what it leaves) and the Hessian's share of (i).  0.42 of it was left at most.
+        // (Without the last, 541 stops were of this form, by contractions that the next step, with the same Hessian, did not repeat: up
+        // to 5 times the norm reported was left, and 0.77 of a tolerance of 1e-8.)
         // Neither is trusted when the factorisation cancelled all but a few percent of some diagonal entry, or, after
         // conjugate gradients, when the common scale of the weights has a slope of that order: with weights of
         // 1e5 and more the fp32 system stops producing Newton steps, the residual stays where it is while the steps, and
@@ -1850,8 +1854,9 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
             // the next point is close enough: fp64 from here on, with this factorisation
             if (kFPredictBound * s2 < kFLowLeave && far <= 0.1f) { mode = trusted ? kChord : kHigh; full_grid = true; dist = far; }
         } else if (trusted && !coarse) {
-            const float lin = chol ? 0.f : ((float)kFChordBase + (mode == kChord ? 2.f * dist : 0.f)) * (float)rn;
-            const float next = fmaxf(rho, far);
+            // (what a step by conjugate gradients leaves of the residual, at least)
+            const float base = chol ? 0.f : (float)kFChordBase + (mode == kChord ? 2.f * dist : 0.f);
+            const float lin = base * (float)rn, next = fmaxf(fmaxf(rho, far), base);
             const bool by_step = far <= (float)kFPredictStep && kFPredictSafety * s2 + 3.0 * (double)lin < tol;
             const bool by_ratio = rho < 0.1f && dm <= (float)kFStepClamp && kFRatioSafety * (double)next * rn < tol;
             if (by_step || by_ratio) {

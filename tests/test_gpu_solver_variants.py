@@ -228,3 +228,17 @@ def test_norms_of_fp32_evaluations_that_end_the_iteration(make):
     tt, td = P.oracle_temps(wl)
     c = O.certify_batch(W.logits_to_f64(wl.q_logits), W.logits_to_f64(wl.p_logits), wl.n, wl.topk, tt, td, r.w.numpy(), lse=r.lse_target.numpy())
     assert float(abs(c.gnorm_lse - r.gnorm.numpy()).max()) <= 4 * 2.0 ** -24
+
+
+@pytest.mark.parametrize("V,n,k,scale,noise", [(40, 2, 16, 2, 1), (40, 16, 20, 3, 3), (60, 32, 50, 3, 3), (60, 8, 40, 3, 1)])
+@pytest.mark.parametrize("tol,quad_step,floor", [(3.0e-7, 0.4, 5.0e-9), (1.0e-8, 0.25, 1.0e-9)])
+def test_predicted_norms_are_bounds(V, n, k, scale, noise, tol, quad_step, floor):
+    """A norm predicted from the last step is no smaller than the oracle's at the weights returned, but for the floor of the evaluation (3e-9 at the
+    default quadrature step, 2e-10 seen at 0.25): also after a step whose predecessor happened to contract far better than its Hessian can."""
+    q, p = _nearly_tight_rows(V, n, k, scale, noise, 256, 60000, 5 + V + n + k)
+    r = G.read_rule(G.solve(q, p, n, k, 1.0, 1.0, G.Options(tol=tol, quad_step=quad_step)))
+    assert set(r.status.tolist()) == {G.GR_OK}
+    c = O.certify_batch(W.logits_to_f64(q), W.logits_to_f64(p), n, k, 1.0, 1.0, r.w.numpy(), lse=r.lse_target.numpy())
+    predicted = r.gnorm_predicted.numpy().astype(bool)
+    assert predicted.any()
+    assert float((c.gnorm_lse - r.gnorm.numpy())[predicted].max()) <= floor
