@@ -24,6 +24,7 @@ int launch_fast_n16_m32h(GR_FAST_ARGS);
 int launch_fast_n16_m64(GR_FAST_ARGS);
 int launch_fast_n16_m64w(GR_FAST_ARGS);
 int launch_fast_n16_m128(GR_FAST_ARGS);
+int launch_fast_n16_m128h(GR_FAST_ARGS);
 int launch_fast_n16_m128w(GR_FAST_ARGS);
 int launch_fast_c24_m32(GR_FAST_ARGS);
 int launch_fast_c24_m32w(GR_FAST_ARGS);
@@ -40,7 +41,7 @@ int launch_fast(GR_FAST_ARGS)
     // Twice to four times the threads per instance, and registers without spills, where the batch leaves an SM with one
     // instance (two of the narrow supports): an instance is a chain of dependent steps then, and 1 row of the headline shape
     // takes 50.5 us a call for 59.0, 128 rows 75 for 83, 64 whole rows of 16 ids 58 for 67.  Beyond one wave the other variants' places
-    // count for more (1024 rows of 9001, n = 8, k = 50: 253 us a call in the wide variant, 138 in the other; 512 rows, n = 16, k = 20, 92 and 71).
+    // count for more (series of 16 and up to 128 tokens: from two waves on, gr_fast_n16.cu; 1024 rows of 9001, n = 8, k = 50: 253 us a call in the wide variant, 138 in the other; 512 rows, n = 16, k = 20, 92 and 71).
     const bool one = batch <= kSms, two = batch <= 2 * kSms;
     if (n > 16) {
         if (kcap <= 32) return two ? fast::launch_fast_c24_m32w(GR_FAST_PASS) : fast::launch_fast_c24_m32(GR_FAST_PASS);
@@ -59,7 +60,8 @@ int launch_fast(GR_FAST_ARGS)
         return one ? fast::launch_fast_n16_m64w(GR_FAST_PASS) : fast::launch_fast_n16_m64(GR_FAST_PASS);
     }
     if (n <= 8) return one ? fast::launch_fast_n8_m128w(GR_FAST_PASS) : fast::launch_fast_n8_m128(GR_FAST_PASS);
-    return one ? fast::launch_fast_n16_m128w(GR_FAST_PASS) : fast::launch_fast_n16_m128(GR_FAST_PASS);
+    if (one) return fast::launch_fast_n16_m128w(GR_FAST_PASS);
+    return two ? fast::launch_fast_n16_m128h(GR_FAST_PASS) : fast::launch_fast_n16_m128(GR_FAST_PASS);
 }
 
 }  // namespace gr
