@@ -66,10 +66,12 @@ struct Cfg {
     static constexpr int NT = NT_, MP = MP_, T = T_, JC = JC_, kCtas = CTAS_, kQC = QC_;
     static constexpr bool kContour = NT > 16;     // samples on a circle instead of series (NT: largest number of them)
     // Fixed-point sweeps of the starting point: five where an evaluation weighs more than the sweeps, three elsewhere.  Whole calls, us, three / five sweeps:
-    // one headline row 50.8 / 48.7, 256 rows of n = 4, k = 8 52.0 / 51.5, 64 whole rows of 16 ids 60.8 / 59.1 (evaluations 3.96 / 3.81), 512 rows of n = 32,
-    // k = 20 107.1 / 102.8 (2.74 / 2.31); full SMs 1024 headline rows 280.6 / 283.0 (3.04 / 3.01), 600 rows of n = 12, k = 50 138.4 / 139.2, on the circle
-    // with 50 tokens 119.3 / 124.6, with 100 194.5 / 190.8; up to 128 tokens, 4096 rows of n = 16, k = 100 1431 / 1460, 600 of n = 8 223.5 / 221.9.
-    static constexpr int kSweeps = kContour ? (MP == 64 ? 3 : 5) : MP <= 64 && (NT == 16 || kCtas <= 2) ? 5 : 3;
+    // one headline row 50.8 / 48.7, 256 rows of n = 4, k = 8 52.0 / 51.5, 64 whole rows of 16 ids 60.8 / 59.1 (evaluations 3.96 / 3.81); full SMs 1024
+    // headline rows 280.6 / 283.0 (3.04 / 3.01), 600 rows of n = 12, k = 50 138.4 / 139.2; up to 128 tokens, 4096 rows of n = 16, k = 100 1431 / 1460, 600 of n = 8
+    // 223.5 / 221.9.  On the circle 512 rows of n = 32, k = 20 107.1 / 102.8 (2.74 / 2.31); solve calls up to 64 tokens, 700 rows of n = 17, k = 50 195.8 / 188.4, of
+    // n = 20, k = 40 182.9 / 173.6, of n = 32, k = 50 218.5 / 205.5, 256 rows of these 84.7 / 89.9, 78.3 / 75.9, 97.2 / 95.9 (evaluations 2.98 / 2.69, 2.94 / 2.42,
+    // 2.97 / 2.55); up to 128 tokens 700 rows of n = 24, k = 128 480 / 492, 64 of n = 20, k = 100 131 / 112 (one evaluation more in the slowest instance).
+    static constexpr int kSweeps = kContour || (MP <= 64 && (NT == 16 || kCtas <= 2)) ? 5 : 3;
     static constexpr int kNG = T / MP;            // copies of the token threads (they share the nodes out among them)
     static constexpr int kW = T / 32, kTW = MP / 32;
     static constexpr int kRow = NT + 4;           // row stride of the product series (16-byte aligned rows in fp32 and fp64)
