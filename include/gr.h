@@ -89,9 +89,11 @@ extern "C" {
  *   max_iters  cap on gradient evaluations per system.            default 40
  *   quad_step  accuracy of the rule by which the gradient integral is evaluated, as the step of
  *              a trapezoid rule in the log-time variable; smaller is more accurate and
- *              slower (error roughly exp(-pi^2/quad_step)).  From 0.4 up the faster kernel
- *              takes rules with fewer nodes and a relative error of 2e-10, below that of
- *              the step 0.4, where the weights of an instance allow it.      default 0.4
+ *              slower (largest relative error of a tuple's term at 0.25 2e-13, 0.3 3e-13, 0.35
+ *              2e-11, 0.39 3e-10, 0.4 6e-10, 0.5 7e-8, 0.8 9e-5).  From 0.4 up the faster kernel
+ *              takes rules with fewer nodes and a relative error of 2e-10 where the weights of an
+ *              instance allow it, whatever the step: a larger one saves it nothing then.  (Evaluations
+ *              that cannot end the iteration are fp32 by rules of 5e-7.)      default 0.4
  *   scan_done_event  optional cudaEvent_t (as void*) recorded on `stream` between
  *              the streaming kernel and the solve kernel, so that a caller can
  *              time the two separately; NULL records nothing.      default NULL
