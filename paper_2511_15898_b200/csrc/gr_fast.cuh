@@ -162,7 +162,7 @@ struct FSm {
     }
 };
 // (what stays the same during a system is read from here: kept in registers it was spilled around every call)
-enum { SC_FAIL = 0, SC_PIVOT = 1, SC_NP = 2, SC_OUT = 4, SC_TOL = 8, SC_QSTEP = 9, SC_SIGMA = 10, SC_HS = 11, SC_TN = 12, SC_GNORM = 13, SC_ITERS = 14 };
+enum { SC_FAIL = 0, SC_PIVOT = 1, SC_NP = 2, SC_RANGE = 3, SC_OUT = 4, SC_TOL = 8, SC_QSTEP = 9, SC_SIGMA = 10, SC_HS = 11, SC_TN = 12, SC_GNORM = 13, SC_ITERS = 14, SC_RATIO = 15 };
 
 // The circle of the contour kernels: `np` conjugate pairs of points r e^(i theta), angles theta and n theta (mod 2 pi),
 // factor 2 n! / (N r^n) of the mean.
@@ -373,20 +373,30 @@ __device__ __forceinline__ void hess_mma(const FSm<C>& sm, Frags<C>& fr, int kst
 
 // Extent of a point's weights: the extreme log-weights, and the largest over the smallest total W of a tuple's weights (slack +
 // sum over its distinct tokens), infinite where the caller's quadrature step asks for more than the tables hold.
-// Beside it which sum an fp32 evaluation takes: its nodes (0: the trapezoid rule) and first entry.
+// Beside it which sum an fp32 evaluation takes: its nodes (0: the trapezoid rule) and first entry.  In shared memory, written by one thread (a
+// barrier before it is read is the caller's): five registers of every thread across the evaluations were spilled around them, and every thread looked for the
+// level (512 rows of n = 16, k = 20 86.1 -> 84.4 us a solve call, 1024 headline rows 270.6 -> 269.1, 4096 of n = 16, k = 100 1387 -> 1378; on the circle 700 of n = 24, k = 64
+// 209.5 -> 212.4).
 struct Extent { float amax, amin, ratio; int nodes, at; };
-__device__ __forceinline__ Extent extent_of(float amax, float amin, float wsum, int n, int slack, double qstep, double tol)
+template <class C>
+__device__ __forceinline__ void put_extent(const FSm<C>& sm, float amax, float amin, float wsum, int n, int slack)
 {
-    Extent e;
-    e.amax = amax; e.amin = amin;
     const float s = slack ? 1.f : 0.f;
     // (rounded up: exponentials of fp32 log-weights are good to 1e-5)
-    e.ratio = qstep >= kTableStep ? 1.0001f * (s + fminf(wsum, (float)n * Rx<float>::ex(amax))) / (s + Rx<float>::ex(amin)) : INFINITY;
-    const bool fine = tol >= kFLowEnds;
-    const int level = fine ? quad_level<double>(e.ratio) : quad_level<float>(e.ratio);
-    e.nodes = level < (fine ? kLevels64 : kLevels32) ? 2 * (level + 1) : 0;
-    e.at = level * (level + 1) + (fine ? kFine : 0);
-    return e;
+    const float ratio = sm.scal[SC_QSTEP] >= kTableStep ? 1.0001f * (s + fminf(wsum, (float)n * Rx<float>::ex(amax))) / (s + Rx<float>::ex(amin)) : INFINITY;
+    const bool fine = sm.scal[SC_TOL] >= kFLowEnds;
+    const int level = fine ? quad_level<double>(ratio) : quad_level<float>(ratio);
+    const int nodes = level < (fine ? kLevels64 : kLevels32) ? 2 * (level + 1) : 0;
+    GR_PTR(float) e = GR_PCAST(float, sm.scal);
+    e[2 * SC_RANGE] = amax; e[2 * SC_RANGE + 1] = amin; e[2 * SC_RATIO] = ratio;
+    e[2 * SC_RATIO + 1] = __int_as_float(nodes | (level * (level + 1) + (fine ? kFine : 0)) << 8);
+}
+template <class C>
+__device__ __forceinline__ Extent get_extent(const FSm<C>& sm)
+{
+    GR_PTR(const float) e = GR_PCAST(const float, sm.scal);
+    const int low = __float_as_int(e[2 * SC_RATIO + 1]);
+    return Extent{e[2 * SC_RANGE], e[2 * SC_RANGE + 1], e[2 * SC_RATIO], low & 255, low >> 8};
 }
 
 // Quadrature nodes for one evaluation, of R's accuracy.  Where 1 / W is wanted for W in a known interval, the fewest nodes are those of the
@@ -553,7 +563,7 @@ __device__ __forceinline__ double recip(double x) { return __drcp_rn(x); }
 // the token's mass.  Errors against 96 points and fp64 throughout, n = 17 to 32, largest mass 0.12 to 0.6: flows 1e-11 in
 // fp64, 1e-7 in fp32; scaled Hessian 2e-5 from 11-bit operands.
 template <class C, typename R, bool kJac>
-__device__ __forceinline__ void eval_contour(const FSm<C>& sm, int m, int slack, double qstep_d, int jstride, const Extent& ext,
+__device__ __forceinline__ void eval_contour(const FSm<C>& sm, int m, int slack, double qstep_d, int jstride,
                                              double w_own, float z_own, double& g_out, double& g2_out, Frags<C>& fr)
 {
     constexpr int T = C::T;
@@ -562,7 +572,7 @@ __device__ __forceinline__ void eval_contour(const FSm<C>& sm, int m, int slack,
     const int tid = threadIdx.x, i = tid % C::MP, ng = tid / C::MP;
     const int np = (int)sm.scal[SC_NP];
     const R wi = (R)w_own;
-    const Grid<R> grid(ext, slack, (R)qstep_d);
+    const Grid<R> grid(get_extent(sm), slack, (R)qstep_d);
     const int Q = grid.Q;
     R g = R(0), g2 = R(0);
     if (kJac) {
@@ -690,17 +700,17 @@ __device__ __forceinline__ void product_series(const R* S, int n, F put)
 }
 
 // Gradient g and the Hessian's diagonal part g2 at the weights in shared memory (this thread's in w_own), in fp64.
-//   ext  extent of the weights;  hs = sigma * (draft mass above the block)
+//   hs = sigma * (draft mass above the block)
 // Every token thread (all copies) gets g and g2.
 template <class C>
-__device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, double hs, int slack, double qstep, const Extent& ext,
+__device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, double hs, int slack, double qstep,
                                             double w_own, double ds_own, double& g_out, double& g2_out)
 {
     constexpr int NT = C::NT, T = C::T;
     typedef double R;
     const RSm<C, R> rs(sm);
     const int tid = threadIdx.x, i = tid % C::MP, ng = tid / C::MP;
-    const Grid<R> grid(ext, slack, qstep);
+    const Grid<R> grid(get_extent(sm), slack, qstep);
     const int Q = grid.Q;
     const R wi = w_own, dsi = ds_own;
     R dp[NT <= 8 ? NT + 1 : 1];
@@ -810,7 +820,7 @@ __device__ __forceinline__ void eval_system(const FSm<C>& sm, int m, int n, doub
 // its own results; packed, a wait serves two.  (4096 rows of n = 16, k = 100: 1552 to 1480 us, 64 whole rows of
 // 16 ids 70 to 63, headline 163 to 159.)
 template <class C>
-__device__ __forceinline__ void eval_low(const FSm<C>& sm, int m, int n, float hs, int slack, float qstep, int jstride, const Extent& ext,
+__device__ __forceinline__ void eval_low(const FSm<C>& sm, int m, int n, float hs, int slack, float qstep, int jstride,
                                          float wi, float dsi, float z_own, double& g_out, double& g2_out, Frags<C>& fr)
 {
     constexpr int NT = C::NT, T = C::T, kRow2 = 2 * C::kRow;
@@ -818,7 +828,7 @@ __device__ __forceinline__ void eval_low(const FSm<C>& sm, int m, int n, float h
     typedef float R;
     const RSm<C, R> rs(sm);
     const int tid = threadIdx.x, i = tid % C::MP, ng = tid / C::MP;
-    const Grid<R> grid(ext, slack, qstep);
+    const Grid<R> grid(get_extent(sm), slack, qstep);
     const int Q = grid.Q;
     F2 dp[NT <= 8 ? NT + 1 : 1];
     if (NT <= 8) {
@@ -994,14 +1004,14 @@ __device__ __forceinline__ void eval_low(const FSm<C>& sm, int m, int n, float h
 
 // The fp64 evaluation, kept out of line (it is called once or twice per system, and its registers stay its own).
 template <class C>
-__device__ __noinline__ double2 eval_fp64(int m, int n, int slack, bool coarse, Extent ext, int* flag)
+__device__ __noinline__ double2 eval_fp64(int m, int n, int slack, bool coarse, int* flag)
 {
     const FSm<C> sm(flag);
     const int i = threadIdx.x % C::MP;
     const double qstep = sm.scal[SC_QSTEP] * (coarse ? 2.0 : 1.0);
     double2 r;
-    if constexpr (C::kContour) { Frags<C> none; eval_contour<C, double, false>(sm, m, slack, qstep, 1, ext, sm.wd[i], 0.f, r.x, r.y, none); }
-    else eval_system<C>(sm, m, n, sm.scal[SC_HS], slack, qstep, ext, sm.wd[i], i < m ? sm.dsd[i] : 0.0, r.x, r.y);
+    if constexpr (C::kContour) { Frags<C> none; eval_contour<C, double, false>(sm, m, slack, qstep, 1, sm.wd[i], 0.f, r.x, r.y, none); }
+    else eval_system<C>(sm, m, n, sm.scal[SC_HS], slack, qstep, sm.wd[i], i < m ? sm.dsd[i] : 0.0, r.x, r.y);
     return r;
 }
 
@@ -1304,7 +1314,7 @@ template <class C> __device__ __forceinline__ float rs_ds(const FSm<C>& sm, int 
 // With `chol` a Cholesky factorisation instead, for systems conjugate gradients do not get through.  `given`: the gradient
 // and the diagonal part come from the caller, in fp64.
 template <class C>
-__device__ __noinline__ double2 eval_hessian(int m, int n, int slack, bool coarse, Extent ext, bool given, bool chol,
+__device__ __noinline__ double2 eval_hessian(int m, int n, int slack, bool coarse, bool given, bool chol,
                                              double2 gg, int* flag)
 {
     const FSm<C> sm(flag);
@@ -1313,11 +1323,11 @@ __device__ __noinline__ double2 eval_hessian(int m, int n, int slack, bool coars
     double g, g2;
     const double qstep = sm.scal[SC_QSTEP] * (coarse ? 2.0 : 1.0);
     // (a table's nodes all serve the Hessian, of the full trapezoid grid every other one)
-    const int jstride = coarse || ext.nodes > 0 ? 1 : 2;
+    const int jstride = coarse || get_extent(sm).nodes > 0 ? 1 : 2;
     const double rhs = i < m ? sm.rhs[sm.ord[i]] : 0.0;
     const float zr = i < m ? (float)rhs : 1.f, zi = rsqrtf(zr);
-    if constexpr (C::kContour) eval_contour<C, float, true>(sm, m, slack, qstep, jstride, ext, sm.wd[i], i < m ? zi : 0.f, g, g2, fr);
-    else eval_low<C>(sm, m, n, (float)sm.scal[SC_HS], slack, (float)qstep, jstride, ext, sm.wf[i], i < m ? rs_ds<C>(sm, i) : 0.f, i < m ? zi : 0.f, g, g2, fr);
+    if constexpr (C::kContour) eval_contour<C, float, true>(sm, m, slack, qstep, jstride, sm.wd[i], i < m ? zi : 0.f, g, g2, fr);
+    else eval_low<C>(sm, m, n, (float)sm.scal[SC_HS], slack, (float)qstep, jstride, sm.wf[i], i < m ? rs_ds<C>(sm, i) : 0.f, i < m ? zi : 0.f, g, g2, fr);
     if (given) { g = gg.x; g2 = gg.y; }
     if (chol) {
         // an outer block's function is constant along (1,...,1): that direction is pinned with 1/m everywhere
@@ -1683,8 +1693,7 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
     double rn = 0.0;
     // (what steers the iteration only is fp32: it is compared with margins of three and more, and in fp64 cost 1 % at series of 16)
     float rprev = kFNone, lam = 1.f, dist = 0.f;
-    Extent ext{0.f, 0.f, 0.f, 0, 0};         // of the weights
-    bool ranged = false;                     // they are known for this point
+    bool ranged = false;                     // the extent of the weights is known for this point
     // Three modes.  Low: gradient and Hessian in fp32, conjugate gradients.  Chord: fp64 gradient, the last Hessian.  High:
     // fp64 gradient, fp32 Hessian of the same point, with `chol` a Cholesky factorisation.  A single token that dominates a
     // long series (its terms would cancel in fp32) starts in the last mode.
@@ -1699,19 +1708,19 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
             unsigned top[2] = {act ? fkey((float)alpha) : 0u, act ? fkey(-(float)alpha) : 0u};
             float wsum = act ? Rx<float>::ex((float)alpha) : 0.f;
             tok_reduce<C, 0, 1, 2>(sm, nullptr, &wsum, top, par);
-            ext = extent_of(fkey_inv(top[0]), -fkey_inv(top[1]), wsum, n, slack, sm.scal[SC_QSTEP], sm.scal[SC_TOL]);
+            if (tid == 0) put_extent(sm, fkey_inv(top[0]), -fkey_inv(top[1]), wsum, n, slack);
         }
         ranged = false;
+        __syncthreads();
         // On the trapezoid rule the step is doubled far from the solution (quadrature error ~1e-4, far below the gradient norm
         // there): half the nodes, every one of them a Hessian node.  Convergence is only declared on the full grid.
-        const bool coarse = rprev > kFCoarse && !full_grid && mode != kChord && ext.nodes == 0;
+        const bool coarse = rprev > kFCoarse && !full_grid && mode != kChord && get_extent(sm).nodes == 0;
         const int kind = 2 * mode + (coarse ? 1 : 0);
-        __syncthreads();
         double2 gg = make_double2(0.0, 0.0);
-        if (mode != kLow) gg = eval_fp64<C>(m, n, slack, coarse, ext, sm.flag);
+        if (mode != kLow) gg = eval_fp64<C>(m, n, slack, coarse, sm.flag);
         if (mode == kHigh) __syncthreads();          // (sum_copies' array)
         if (mode != kChord)
-            gg = eval_hessian<C>(m, n, slack, coarse, ext, mode == kHigh, chol, gg, sm.flag);
+            gg = eval_hessian<C>(m, n, slack, coarse, mode == kHigh, chol, gg, sm.flag);
         const double g = gg.x, g2 = gg.y, rhs_i = act ? sm.rhs[sm.ord[i]] : 0.0, tol = sm.scal[SC_TOL];
         // The residual, and what the step below needs of the tokens: right-hand side b of the Newton system, s_i = g2_i / w_i,
         // and the sums of b, s and the Hessian's diagonal.
@@ -1826,7 +1835,7 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
             mode = kHigh; chol = true; full_grid = true; rprev = kFNone; was_kind = -1;
             continue;
         }
-        ext = extent_of(fkey_inv(top[1]), -fkey_inv(top[2]), wsum, n, slack, sm.scal[SC_QSTEP], sm.scal[SC_TOL]);
+        if (tid == 0) put_extent(sm, fkey_inv(top[1]), -fkey_inv(top[2]), wsum, n, slack);
         ranged = !(dm > (float)kFStepClamp);
         // a full Newton step below 1e-11 in alpha: the weights cannot be improved at this quadrature accuracy
         if (!fail && mode != kLow && far < 1.0e-11f) { status = GR_OK; it++; break; }
