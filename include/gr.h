@@ -80,9 +80,9 @@ extern "C" {
  *              lin = (0.02 + 2 x the distance to that point) x the residual: stop when
  *              10 s2 + 3 lin < tol, reported 3 s2 + lin.  By the ratio (faster kernel only):
  *              after a step that contracted the residual to r by rho < 0.1, stop when
- *              3 c r < tol, reported c r, with c the largest of rho, the step's length and (with such a
- *              Hessian) 0.02 + 2 x the distance.  On 22 kinds of rows at tolerances of 1e-8, 3e-7 and 1e-5 a stop
- *              left at most 0.42 of what it reported, beyond the floor of 3e-9.  Neither
+ *              3 c r < tol and 1.5 h r < tol, with c the larger of rho and the step's length and h (with such a
+ *              Hessian) 0.02 + 2 x the distance, reported max(c, h) r.  On 28 kinds of rows at tolerances of 1e-8,
+ *              3e-7 and 1e-5 a stop left at most 0.44 of what it reported, beyond the floor of 3e-9.  Neither
  *              is used when the Newton system is too close to singular in fp32: less than 2 %
  *              of a diagonal entry left as the factorisation's pivot, or of the Hessian's trace
  *              as the slope along the common scale of the weights.

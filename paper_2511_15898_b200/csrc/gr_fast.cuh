@@ -42,6 +42,7 @@ constexpr double kFCoarse = 1.0e-2;        // above this residual the trapezoid 
 constexpr double kFPredictStep = 1.0;      // largest |delta alpha| after which the stop on a predicted residual is allowed
 constexpr double kFPredictSafety = 10.0;   // the prediction s2 must be this many times below the tolerance
 constexpr double kFRatioSafety = 3.0;      // the residual predicted by the last step's contraction must be this many times below the tolerance
+constexpr double kFBaseSafety = 1.5;       // and what the Hessian leaves of it this many times
 constexpr double kFTrustPivot = 0.02;      // smallest relative pivot at which a predicted stop is allowed
 constexpr double kFPredictBound = 3.0;     // reported norm after such a stop: kFPredictBound * s2
 constexpr double kFLowLeave = 3.0e-3;      // bound on the next residual (kFPredictBound * s2; it is mostly a fiftieth of that) at which the iteration goes over to fp64
@@ -1842,20 +1843,21 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
         if (dm > (float)kFStepClamp && act) dl = jump + (dl - (double)jump) * (double)__fdividef((float)kFStepClamp, dm);
         alpha = fmin(fmax(alpha + dl, -kFAlphaClamp), kFAlphaClamp);
         // Stop on a predicted residual, without another evaluation, after a step from a point evaluated in fp64 on the
-        // full grid.  Measured with this iteration against the oracle's residual at the weights returned, 7633 such stops at tolerances
-        // of 1e-8 (quadrature steps 0.25 and 0.4), 3e-7 and 1e-5 on 22 kinds of rows: every benchmark shape, random rows of 16 to 128 tokens with 2 to 32 drafts,
-        // whole and truncated, and rows picked for prefixes that are almost tight (weights on several scales); 842 in outer blocks.  6498 were an
-        // instance's only system and are held one by one against what they left, less the floor of 3e-9:
-        // (i) By the step (6484).  Second order: s2 = sum_i g_i delta_i^2 (each flow is a sum of terms exponential in alpha over
-        // positive normalisers).  First order, after conjugate gradients: what the half-precision Hessian leaves of the residual (403 stops
-        // after a fresh one: 0.0125 of it at most), plus the distance to the point where a reused one was formed (6073 stops, distances of 0.004 in the
-        // median, 0.028 in one of ten, 0.11 at most: 0.45 lin at most).  Left were never more than 13 % of 10 s2 + 3 lin, 38 % of the norm reported
+        // full grid.  Measured with this iteration against the oracle's residual at the weights returned, 14191 such stops at tolerances
+        // of 1e-8 (quadrature steps 0.25 and 0.4), 3e-7 and 1e-5 on 28 kinds of rows: every benchmark shape, random rows of 16 to 128 tokens with 2 to 32 drafts,
+        // whole and truncated, rows picked for prefixes that are almost tight (weights on several scales), and long series with a dominant token; 916 in outer blocks.  12960
+        // were an instance's only system and are held one by one against what they left, less the floor of 3e-9:
+        // (i) By the step (12261).  Second order: s2 = sum_i g_i delta_i^2 (each flow is a sum of terms exponential in alpha over
+        // positive normalisers).  First order, after conjugate gradients: what the half-precision Hessian leaves of the residual (1202 stops
+        // after a fresh one: 0.007 of it at most, 0.0125 on other draws of the same kinds), plus the distance to the point where a reused one was formed (11051 stops, distances of 0.004 in
+        // the median, 0.03 in one of ten, 0.11 at most: 0.45 lin at most).  Left were never more than 13 % of 10 s2 + 3 lin, 38 % of the norm reported
         // and 10 % of the tolerance; lin is the larger term in all but 25.
-        // (ii) By the ratio (14): the last full step on this grid contracted the residual by rho < 0.1, and the next one is taken
+        // (ii) By the ratio (699): the last full step on this grid contracted the residual by rho < 0.1, and the next one is taken
         // to contract by no less than that, its own length (along a direction in which the flows hardly change s2 says
-        // nothing, and the length of the step times the residual is what it leaves) and the Hessian's share of (i).  0.42 of it was left at most.
-        // (Without the last, 541 stops were of this form, by contractions that the next step, with the same Hessian, did not repeat: up
-        // to 5 times the norm reported was left, and 0.77 of a tolerance of 1e-8.)
+        // nothing, and the length of the step times the residual is what it leaves) and the Hessian's share of (i), which already is twice what was seen and is held
+        // with half the margin.  0.44 of the norm reported was left at most, 0.19 of the tolerance.
+        // (Without the last, by contractions that the next step, with the same Hessian, did not repeat, up to 5 times the norm reported was left, and 0.77 of a
+        // tolerance of 1e-8.  Held with a margin of three it costs up to 6 % of the instances of a dominant token an evaluation, with 1.5 half of those.)
         // Neither is trusted when the factorisation cancelled all but a few percent of some diagonal entry, or, after
         // conjugate gradients, when the common scale of the weights has a slope of that order: with weights of
         // 1e5 and more the fp32 system stops producing Newton steps, the residual stays where it is while the steps, and
@@ -1870,7 +1872,7 @@ __device__ __noinline__ int fast_system(int m, int slack, int n, double hmass, i
             const float base = chol ? 0.f : (float)kFChordBase + (mode == kChord ? 2.f * dist : 0.f);
             const float lin = base * (float)rn, next = fmaxf(fmaxf(rho, far), base);
             const bool by_step = far <= (float)kFPredictStep && kFPredictSafety * s2 + 3.0 * (double)lin < tol;
-            const bool by_ratio = rho < 0.1f && dm <= (float)kFStepClamp && kFRatioSafety * (double)next * rn < tol;
+            const bool by_ratio = rho < 0.1f && dm <= (float)kFStepClamp && kFRatioSafety * (double)fmaxf(rho, far) * rn < tol && kFBaseSafety * (double)lin < tol;
             if (by_step || by_ratio) {
                 rn = by_step ? kFPredictBound * s2 + (double)lin : (double)next * rn;
                 status = GR_OK; it++;
