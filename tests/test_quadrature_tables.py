@@ -28,3 +28,17 @@ def test_sums_reproduce_the_reciprocal(name, bits, bound):
         x = np.exp(np.linspace(0.0, np.log(limit), 20001))
         err = np.abs(1.0 - x * (np.exp(-np.outer(x, t)) @ c)).max()
         assert err <= bound, (level, limit, err)
+
+
+@pytest.mark.parametrize("name,bits,terms,eps", [("double", "64", 2, 2e-10), ("double", "64", 4, 2e-10), ("float", "32", 4, 5e-7), ("float", "32", 6, 5e-7)])
+def test_generator_makes_the_tables(name, bits, terms, eps):
+    """The generator's sums and the tables': both stop within 1e-3 of the wanted error, which falls with the fifth power of log R and faster, so
+    that limits, nodes and coefficients agree to a few 1e-4."""
+    pytest.importorskip("mpmath")
+    from paper_2511_15898_b200.quadrature import best_sum
+    entries, limits = _tables(name, bits)
+    level = terms // 2 - 1
+    R, t, c = best_sum(terms, eps)
+    t0, c0 = entries[level * (level + 1):(level + 1) * (level + 2)].T
+    assert abs(np.log(R) / np.log(limits[level]) - 1) < 3e-4
+    assert np.allclose(t, t0, rtol=3e-4, atol=0) and np.allclose(c, c0, rtol=3e-4, atol=0)
