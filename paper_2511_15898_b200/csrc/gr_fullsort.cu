@@ -120,8 +120,8 @@ __device__ inline double block_min(double v, double* s_r)
 
 // flag[0] of the instance's scratch region: bit j set when fullsort_alpha_kernel has to do the row for the j-th draft count.
 // With a params block and `rule_status` it also writes the header of a row without a rule (nl.n[0] drafts).
-// 512 rows of 50257 in fp32: the call 195 us, 220 before (bucket numbers and masses out of scaled logits formed first, a polynomial of degree 5, every thread
-// its own quotients and exponentials, candidates ordered in three rounds).  A row takes 71 k cycles, one to an SM: 46 k its masses (instruction
+// 512 rows of 50257 in fp32: the call 202 us, 222 before (bucket numbers and masses out of scaled logits formed first, a polynomial of degree 5, every thread
+// its own quotients and exponentials, candidates ordered in three rounds); 201 with exponents out of products rounded first, which fail for logits of 1e17 and more.  A row takes 71 k cycles, one to an SM: 46 k its masses (instruction
 // issue: 113 instructions per 32 ids in all, fp64 25 of them), 4 k sums, 5 k bounds, 6 k numbers read back, 6 k candidates; the 206 MB it reads are a fifth of the time.
 template <typename T>
 __global__ void __launch_bounds__(kBkThreads)
