@@ -122,7 +122,7 @@ __device__ inline double block_min(double v, double* s_r)
 // With a params block and `rule_status` it also writes the header of a row without a rule (nl.n[0] drafts).
 // 512 rows of 50257 in fp32: the call 202 us, 222 before (bucket numbers and masses out of scaled logits formed first, a polynomial of degree 5, every thread
 // its own quotients and exponentials, candidates ordered in three rounds); 201 with exponents out of products rounded first, which fail for logits of 1e17 and more.  A row takes 71 k cycles, one to an SM: 46 k its masses (instruction
-// issue: 113 instructions per 32 ids in all, fp64 25 of them), 4 k sums, 5 k bounds, 6 k numbers read back, 6 k candidates; the 206 MB it reads are a fifth of the time.
+// issue: 116 instructions per 32 ids in all, fp64 25 of them), 4 k sums, 5 k bounds, 6 k numbers read back, 6 k candidates; the 206 MB it reads are a fifth of the time.
 template <typename T>
 __global__ void __launch_bounds__(kBkThreads)
 bucket_alpha_kernel(const T* __restrict__ q, const T* __restrict__ p, int V, const __grid_constant__ NList nl, double rt, double rd,
