@@ -42,8 +42,7 @@ def _certified(wl, rule, rows):
 
 @pytest.mark.parametrize("n,topk,batch", [(n, k, b) for n in (2, 4, 5, 8, 9, 16, 17, 32) for k in (17, 32)
                                           for b in ((296, 297, 592, 593) if 8 < n <= 16 else (296, 297))]
-                         + [(n, k, b) for n in (2, 4, 5, 8, 9, 16) for k in (33, 64, 65, 128) for b in (148, 149)]
-                         + [(n, k, b) for n in (9, 16) for k in (65, 128) for b in (296, 297)])
+                         + [(n, k, b) for n in (2, 4, 5, 8, 9, 16) for k in (33, 64, 65, 128) for b in (148, 149)])
 def test_rows_of_both_sides_of_a_change_of_variant(n, topk, batch):
     """The number of threads per instance depends on the batch: first, last and other rows of batches at each change, and the
     whole batch's draws by the fused call and by the two calls (from one law each within 3e-7 of the target: a fused call solves
@@ -56,6 +55,12 @@ def test_rows_of_both_sides_of_a_change_of_variant(n, topk, batch):
     two = G.verify(solved, wl.draft_tokens, wl.uniforms)
     one = G.solve_verify(wl.q_logits, wl.p_logits, wl.draft_tokens, wl.uniforms, topk, wl.temp_target, wl.temp_draft)[1]
     assert torch.equal(two.token, one.token) and torch.equal(two.accepted, one.accepted) and torch.equal(two.status, one.status)
+
+
+@pytest.mark.parametrize("n,topk,batch", [(n, k, b) for n in (9, 16) for k in (65, 128) for b in (296, 297)])
+def test_rows_of_both_sides_of_two_waves_of_wide_supports(n, topk, batch):
+    """Series of 16 and supports of up to 128 tokens change their number of threads at two instances to an SM as well."""
+    test_rows_of_both_sides_of_a_change_of_variant(n, topk, batch)
 
 
 @pytest.mark.parametrize("n", [2, 4, 5, 8, 9, 16])
